@@ -10,6 +10,7 @@
 #include <new>
 
 #include "common.cuh"
+#include "forward.cuh"
 #include "tc_gemm.cuh"
 
 using namespace mtad;
@@ -18,6 +19,7 @@ using namespace mtad;
 // per tensor-memory accumulator, the pieces being added in fp32 (relative error about 4e-7 instead of 4e-6 at K = 8192)
 static const int kQkvSegCap = 8;
 static const int kCtas = 148;   // SMs the tensor-core GEMM spreads over
+static const bool kOneLaunchForward = false;
 
 // Host-side tensor maps of one model's weight matrices.
 struct WeightMaps {                      // index 0, 1, 2: tiles of 128, 256, 512 rows (1, 2, 4 halves)
@@ -43,6 +45,9 @@ struct ForwardPlan {
     bool split_kv = false;             // K and V have a launch of their own, fed by sc.xkv with kv_terms terms
     int kv_terms = 0;
     bool maps = false;                 // tensor maps encoded (false: decomposition only, for the extent audit)
+    bool one_launch = false;           // the whole forward is one launch (fw), g stays empty
+    FwArgs fw{};
+    double fw_bytes = 0.0;
 };
 
 struct mtad_ctx {
@@ -50,6 +55,9 @@ struct mtad_ctx {
     char* ws_base = nullptr;
     std::map<uint64_t, ForwardPlan> plans;   // by (model, sequences, rows per sequence, LM-head mode)
     WeightMaps tmaps, amaps;
+    FwLayer *fw_target = nullptr, *fw_aux = nullptr;   // device tables of the one-launch forward (in the workspace)
+    CUtensorMap fw_lm[2];                              // its LM-head maps: target, auxiliary model
+    bool fw_ok[2] = {false, false};
     bool use_tc = false, use_pdl = false;
     size_t tc_ws_floats = 0, tc_counter_n = 0, xf_elems = 0;
     ModelView target, aux;
@@ -216,8 +224,10 @@ size_t carve(mtad_ctx* c, const mtad_model_desc* t, const mtad_model_desc* a, in
     sc.xf = k.take<__nv_bfloat16>((size_t)2 * TC_X_ROWS * F, "xf");
     sc.xkv = k.take<__nv_bfloat16>((size_t)2 * TC_X_ROWS * d, "xkv");
     const size_t dt = (d + TC_TILE_N - 1) / TC_TILE_N;
-    sc.sumsq_a = k.take<float>(dt * TC_X_ROWS, "sumsq_a");
-    sc.sumsq_b = k.take<float>(dt * TC_X_ROWS, "sumsq_b");
+    // (the one-launch forward leaves a part per block that owns features)
+    const size_t sq_parts = std::max(dt, mx([](const mtad_model_desc* m) { return fw_parts_max(*m, kCtas, false); }));
+    sc.sumsq_a = k.take<float>(sq_parts * TC_X_ROWS, "sumsq_a");
+    sc.sumsq_b = k.take<float>(sq_parts * TC_X_ROWS, "sumsq_b");
     size_t ws_tiles = 0, max_tiles = 0, lm_tiles = 0;
     auto shape_ws = [&](const mtad_model_desc* m) {
         const int qdm = m->n_q_heads * m->head_dim, kvm = m->n_kv_heads * m->head_dim;
@@ -242,7 +252,12 @@ size_t carve(mtad_ctx* c, const mtad_model_desc* t, const mtad_model_desc* a, in
     if (a) shape_ws(a);
     sc.tc_ws = k.take<float>(ws_tiles * rpad * TC_TILE_N, "tc_ws");
     sc.tc_counters = k.take<int32_t>(max_tiles, "tc_counters");
-    sc.lm_part = k.take<float4>(Tc * lm_tiles, "lm_part");
+    sc.lm_part = k.take<float4>(Tc * std::max(lm_tiles, mx([](const mtad_model_desc* m) { return fw_parts_max(*m, kCtas, true); })),
+                                "lm_part");
+    sc.fw_sync_words = (int)mx([&](const mtad_model_desc* m) { return fw_sync_words(m->layers, max_batch, m->n_kv_heads); });
+    sc.fw_sync = k.take<int32_t>(sc.fw_sync_words, "fw_sync");
+    FwLayer* fw_t = k.take<FwLayer>(t->layers, "fw_target");
+    FwLayer* fw_a = a ? k.take<FwLayer>(a->layers, "fw_aux") : nullptr;
     sc.node_z = k.take<float>(T, "node_z");
     sc.draft_part = a ? k.take<DraftPart>((size_t)max_batch * MTAD_MAX_BEAM * MTAD_DRAFT_CHUNKS, "draft_part") : nullptr;
     sc.warp_part = k.take<WarpPart>(T * MTAD_DRAFT_CHUNKS, "warp_part");
@@ -264,6 +279,7 @@ size_t carve(mtad_ctx* c, const mtad_model_desc* t, const mtad_model_desc* a, in
     if (c) {
         c->ds = ds;
         c->st = st; c->rm = rm; c->sc = sc;
+        c->fw_target = fw_t; c->fw_aux = fw_a;
         c->tc_ws_floats = ws_tiles * rpad * TC_TILE_N;
         c->tc_counter_n = max_tiles;
         c->xf_elems = (size_t)2 * TC_X_ROWS * F;
@@ -381,6 +397,63 @@ bool build_weight_maps(const ModelView& m, WeightMaps& w) {
     }
     w.ok = ok;
     return ok;
+}
+
+// The layer table of the one-launch forward, encoded for the tile geometry of this model and copied to the workspace.
+bool build_forward_table(const ModelView& m, FwLayer* dev, CUtensorMap* lm) {
+    const mtad_model_desc& d = m.d;
+    if (d.head_dim != 64 && d.head_dim != 128) return false;
+    FwPhase ph[6];
+    fw_geometry(ph, d, kCtas);
+    const int qd = d.n_q_heads * d.head_dim, hp = d.head_dim / 2;
+    std::vector<FwLayer> tab(d.layers);
+    for (int l = 0; l < d.layers; ++l) {
+        FwLayer& t = tab[l];
+        if (tc_make_pair_map(&t.wq, m.w(l, 1), d.n_q_heads, hp, d.d_model, ph[FW_QKV].h) ||
+            tc_make_pair_map(&t.wk, m.w(l, 2), d.n_kv_heads, hp, d.d_model, ph[FW_QKV].h) ||
+            tc_make_pair_map(&t.wv, m.w(l, 3), d.n_kv_heads, hp, d.d_model, ph[FW_QKV].h) ||
+            tc_make_map(&t.wo, m.w(l, 4), d.d_model, qd, ph[FW_O].h) ||
+            tc_make_map(&t.gate, m.w(l, 6), d.d_ffn, d.d_model, ph[FW_GATEUP].h) ||
+            tc_make_map(&t.up, m.w(l, 7), d.d_ffn, d.d_model, ph[FW_GATEUP].h) ||
+            tc_make_map(&t.down, m.w(l, 8), d.d_model, d.d_ffn, ph[FW_DOWN].h))
+            return false;
+        t.gain_ffn = m.w(l, 5);
+        t.gain_next = l + 1 < d.layers ? m.w(l + 1, 0) : static_cast<const __nv_bfloat16*>(d.final_norm);
+    }
+    if (tc_make_map(lm, d.lm_head, d.vocab, d.d_model, ph[FW_LM].h)) return false;
+    return cudaMemcpy(dev, tab.data(), sizeof(FwLayer) * tab.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+}
+
+// The one-launch plan of a call of B x R rows: everything that the calls of this shape share.  `with_maps` as build_plan.
+bool build_forward_plan(ForwardPlan& fp, const Scratch& sc, const RowMeta& rm, const ModelView& m, const FwLayer* table,
+                        const CUtensorMap* lm, int B, int R, bool lm_plain, bool with_maps) {
+    const mtad_model_desc& d = m.d;
+    FwArgs& a = fp.fw;
+    if (!fw_plan(a, d, B, R, kCtas)) return false;
+    const int qd = d.n_q_heads * d.head_dim;
+    if (with_maps) {
+        if (!m.kv_map_ok || tc_make_map(&a.xd, sc.xd, 2 * TC_X_ROWS, d.d_model, a.cols) ||
+            tc_make_map(&a.xa, sc.xa, 2 * TC_X_ROWS, qd, a.cols) || tc_make_map(&a.xf, sc.xf, 2 * TC_X_ROWS, d.d_ffn, a.cols))
+            return false;
+        a.lm = *lm;
+        a.kv = m.kv_map;
+    }
+    a.layers = table;
+    a.lm_plain = lm_plain ? 1 : 0;
+    a.max_batch = m.max_batch; a.cap = d.kv_capacity;
+    a.parts0 = 1; a.inv_dim = 1.f / (float)d.d_model; a.eps = d.rms_eps;
+    a.sync = sc.fw_sync; a.acnt = sc.fw_sync + 5 * d.layers + 1;
+    a.sumsq_a = sc.sumsq_a; a.sumsq_b = sc.sumsq_b; a.hidden = sc.hidden;
+    a.x_d = sc.xd; a.x_a = sc.xa; a.x_f = sc.xf; a.q_hi = sc.q_hi; a.q_lo = sc.q_lo;
+    a.cache = static_cast<__nv_bfloat16*>(d.kv_cache);
+    a.rope = sc.rope; a.rm = rm; a.part = sc.attn_part;
+    a.lm_part = sc.lm_part; a.logits = sc.logits; a.node_z = sc.node_z;
+    const double kvd = (double)d.n_kv_heads * d.head_dim;
+    fp.fw_bytes = 2.0 * d.layers * ((double)d.d_model * (2.0 * qd + 2.0 * kvd + 3.0 * d.d_ffn)) + 2.0 * d.vocab * d.d_model;
+    fp.lm_tiles128 = a.ph[FW_LM].n_tiles;
+    fp.one_launch = true;
+    fp.maps = with_maps;
+    return true;
 }
 
 bool mma_attention(const ModelView& m) {
@@ -563,10 +636,23 @@ int forward_rows_tc(mtad_ctx* ctx, const ModelView& m, const WeightMaps& wm, int
     auto it = ctx->plans.find(key);
     if (it == ctx->plans.end()) {
         ForwardPlan fp;
-        if (int rc = build_plan(fp, sc, ctx->rm, m, &wm, B, R, lm_plain, true, &m == &ctx->target)) return rc;
+        const bool aux = &m == &ctx->aux;
+        if (!(ctx->fw_ok[aux] && build_forward_plan(fp, sc, ctx->rm, m, aux ? ctx->fw_aux : ctx->fw_target, &ctx->fw_lm[aux], B, R,
+                                                    lm_plain, true))) {
+            fp = ForwardPlan();
+            if (int rc = build_plan(fp, sc, ctx->rm, m, &wm, B, R, lm_plain, true, !aux)) return rc;
+        }
         it = ctx->plans.emplace(key, std::move(fp)).first;
     }
     ForwardPlan& fp = it->second;
+    if (fp.one_launch) {
+        fp.fw.status = status; fp.fw.uniforms = uniforms;
+        fp.fw.wait_limit = ctx->wait_limit; fp.fw.debug_no_operands = ctx->debug_no_operands;
+        fp.fw.pieces = (int)((total + FW_KEYS - 1) / FW_KEYS);
+        RUN(MTAD_K_GEMM, fp.fw_bytes, 1, launch_forward(fp.fw, s));
+        if (!lm_plain) RUN(MTAD_K_LMRED, 0, 2, launch_lm_merge(m, ctx->rm, sc, B, R, fp.lm_tiles128, uniforms, status, s));
+        return MTAD_OK;
+    }
     auto launch = [&](size_t i) -> int {
         GemmDesc& gd = fp.g[i];
         TcGemmParams& p = gd.p;
@@ -734,6 +820,10 @@ int mtad_create(const mtad_model_desc* target, const mtad_model_desc* aux, int m
         if (e == cudaSuccess) e = cudaMemset(ctx->ws_base + r.off + r.count * r.elem, 0xC5, kCanaryBytes);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) { delete ctx; return MTAD_E_CUDA; }
+    if (ctx->use_tc && kOneLaunchForward) {
+        ctx->fw_ok[0] = ctx->target.kv_map_ok && build_forward_table(ctx->target, ctx->fw_target, &ctx->fw_lm[0]);
+        ctx->fw_ok[1] = aux && ctx->amaps.ok && ctx->aux.kv_map_ok && build_forward_table(ctx->aux, ctx->fw_aux, &ctx->fw_lm[1]);
+    }
     *out = ctx;
     return MTAD_OK;
 }
@@ -1058,6 +1148,31 @@ void audit_forward(Audit& au, const mtad_ctx& c, const ModelView& m, int B, int 
     au.ws("xd", idx_xrow(T - 1, terms, terms - 1, d.d_model, d.d_model - 1) + 1);
     au.ws("sumsq_a", T);
     ForwardPlan fp;
+    if (kOneLaunchForward && build_forward_plan(fp, c.sc, c.rm, m, nullptr, nullptr, B, R, lm_plain, false)) {
+        // the one-launch forward: what its epilogues and its attention index
+        const FwArgs& a = fp.fw;
+        const long long cap = d.kv_capacity, total = std::min<long long>(len_ub, cap) + R;
+        const long long slot_max = std::min<long long>(len_ub + R - 1, cap - 1), pieces = (total + FW_KEYS - 1) / FW_KEYS;
+        for (const FwPhase* f : {&a.ph[FW_O], &a.ph[FW_DOWN]})
+            for (const char* n : {"sumsq_a", "sumsq_b"}) au.ws(n, (size_t)(f->n_tiles - 1) * TC_X_ROWS + T);
+        au.ws("hidden", (size_t)(T - 1) * d.d_model + d.d_model);
+        au.ws("q_hi", (size_t)T * qd);
+        au.ws("q_lo", (size_t)T * qd);
+        au.ws("xa", idx_xrow(T - 1, terms, terms - 1, qd, qd - 1) + 1);
+        au.ws("xf", idx_xrow(T - 1, terms, terms - 1, d.d_ffn, d.d_ffn - 1) + 1);
+        au.ws("attn_part", (size_t)T * Hq * pieces * (hd + 2));
+        au.ws("fw_sync", fw_sync_words(d.layers, m.max_batch, Hkv));
+        au.ws(&m == &c.target ? "fw_target" : "fw_aux", d.layers);
+        if (lm_plain) au.ws("logits", (size_t)T * d.vocab);
+        else au.ws("lm_part", idx_lm_part(T - 1, a.ph[FW_LM].n_tiles, a.ph[FW_LM].n_tiles - 1) + 1);
+        au.ext(cache_name, idx_cache(d.layers - 1, m.max_batch, m.max_batch - 1, 1, Hkv, Hkv - 1, cap, slot_max, hd) + hd,
+               (size_t)d.layers * m.max_batch * 2 * Hkv * cap * hd);
+        au.ext("operand rows of a box", a.cols, 2 * TC_X_ROWS);
+        au.ext("kv_map_planes", (size_t)((d.layers - 1) * m.max_batch + (m.max_batch - 1)) * 2 * Hkv + 2 * Hkv,
+               (size_t)d.layers * m.max_batch * 2 * Hkv);
+        return;
+    }
+    fp = ForwardPlan();
     build_plan(fp, c.sc, c.rm, m, nullptr, B, R, lm_plain, false, &m == &c.target);
     if (fp.split_kv) au.ws("xkv", idx_xrow(T - 1, fp.kv_terms, fp.kv_terms - 1, d.d_model, d.d_model - 1) + 1);
     const long long cap = d.kv_capacity;

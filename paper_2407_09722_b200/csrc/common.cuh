@@ -132,6 +132,8 @@ struct Scratch {
     float4* lm_part;     // [T][tiles(V)]
     float* node_z;       // [T]
     DraftPart* draft_part;   // [max_batch][MTAD_MAX_BEAM][MTAD_DRAFT_CHUNKS], only with an auxiliary model
+    int32_t* fw_sync;        // one-launch forward: phase counters and the attention's arrival counters
+    int fw_sync_words;
     WarpPart* warp_part;     // [T][MTAD_DRAFT_CHUNKS]
     WarpRow* warp_row;       // [T]
 };
@@ -199,6 +201,21 @@ __device__ __forceinline__ void store_terms(float y, __nv_bfloat16* x, size_t K,
     const __nv_bfloat16 l = __float2bfloat16_rn(r);
     x[K] = l;
     if (terms == 3) x[2 * K] = __float2bfloat16_rn(r - __bfloat162float(l));
+}
+
+// The same for four neighbouring elements: one 8-byte store per term.
+__device__ __forceinline__ void store_terms4(float4 v, __nv_bfloat16* x, size_t K, int terms) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        if (j >= terms) break;
+        const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+        uint2 w;
+        w.x = *reinterpret_cast<const uint32_t*>(&a);
+        w.y = *reinterpret_cast<const uint32_t*>(&b);
+        *reinterpret_cast<uint2*>(x + (size_t)j * K) = w;
+        v.x -= __bfloat162float(a.x); v.y -= __bfloat162float(a.y);
+        v.z -= __bfloat162float(b.x); v.w -= __bfloat162float(b.y);
+    }
 }
 
 // One embedding row -> the fp32 hidden row and (tensor-core path) its bf16 operand terms times the first norm's gain;

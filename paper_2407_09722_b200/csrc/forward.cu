@@ -1,0 +1,907 @@
+// The decoder forward of a few draft rows as one cooperative launch: one block per SM walks every layer's phases
+//   QKV (+ rotary, KV append)  |  attention  |  O (+ residual)  |  gate / up (+ SwiGLU)  |  down (+ residual)
+// and the LM head, with a grid barrier between phases.
+//
+// What bounds it: the weights (and K / V) pass once through every SM's copy ring, so the floor is HBM bandwidth.  As a
+// chain of launches this work lost 7..8 us at every projection - drain, split-K exchange, epilogue, the launch boundary,
+// and a copy ring that starts empty.  Here the weight producer does not know phases: as the last k-blocks of a projection
+// leave the ring, the first ones of the next (or the committed K / V tiles of the attention) take their place, so HBM
+// stays busy across the barrier for as long as the ring is deep.  Two more things keep the boundary short: every block
+// owns whole output features (the features are cut into one or two units per SM, not into 128-row tiles), so no partial
+// sum leaves an SM; and only the call's terms x rows operand rows are multiplied (16 columns for five rows).
+//
+// Contraction.  Weights are the 128-row MMA operand A, the operand rows (two or three bf16 terms per activation, see
+// store_terms) operand B.  Where a block owns at most 32 (64) features, a step brings S = 4 (2) k-blocks, whose weights
+// lie side by side in A and whose operand rows lie side by side in B: of the S x S blocks of the product the diagonal
+// ones are the k-blocks' contributions, summed by the epilogue.  One MMA of 128 x 64 costs what one of 128 x 16 does, so
+// this is S times fewer MMAs (an MMA takes 65 cycles whatever N <= 128 is: 28 rows a step would cap an SM at 27 GB/s).
+//
+// Attention: keys as the M dimension.  The (sequence, KV head, 128-key tile) items are dealt out evenly, in order.
+//   S^T = K Q^T   A = K tile as it lies in the cache, B = query rows (bf16 hi rows, then lo rows)
+//   P = exp2(S - m), a thread per key, written to shared memory as bf16 hi and lo
+//   O^T += V^T P  A = V tile (MN-major), B = P; a thread per head dimension adds it to its registers
+// Pieces of a (sequence, KV head) held by several blocks meet in global memory; the block that arrives last merges them.
+//
+// Warps: 0 weight and K / V producer (TMA), 1 operand-row producer (TMA; waits for the phase before), 2 MMA issuer,
+// 3 tensor memory, 4..11 epilogue; in the attention 4..7 softmax (a lane per key) and 8..11 output (a lane per dimension).
+// Every wait is bounded; a block that gives up raises MTAD_ST_TIMEOUT for every sequence of the call and leaves, and the
+// others run into their own limits at the grid barrier.
+#include <math_constants.h>
+
+#include <algorithm>
+
+#include "forward.cuh"
+#include "tc_device.cuh"
+
+namespace mtad {
+using namespace tcdev;
+
+namespace {
+
+constexpr int FW_THREADS = 32 * 12;
+constexpr int FW_EPI_WARP0 = 4;
+constexpr int FW_EPI = 256;
+constexpr int FW_UNION = 32 * 1024;       // epilogue tile Y, or the attention's query and probability tiles
+constexpr int FW_MAX_SLOTS = 6;
+constexpr int FW_TM_D = 128;              // attention: tensor-memory columns 0 / 64 scores, 128 / 192 outputs
+
+struct FwTail {
+    float rstd[64];
+    float smx[2][16][4];                  // row maxima of the four softmax warps
+    float sf[2][16];                      // rescale factor of the running output, per tile buffer
+    float sl[2][4][16];                   // row sums of the softmax warps
+    float sm[2][16];                      // row reference values
+    int pref[MTAD_MAX_BATCH + 1];         // flattened attention tiles before sequence b
+    uint64_t full[FW_MAX_SLOTS], empty[FW_MAX_SLOTS];
+    uint64_t tfull[2], tempty[2], sfull[2], pfull[2], ofull[2], oempty[2], qfull[2];
+    uint32_t tmem_ptr;
+    int abort_flag[2];
+    int last[2];
+};
+
+__device__ __forceinline__ bool grid_wait(const int* c, int want, volatile int* abort_flag) {
+    const uint32_t limit = (uint32_t)abort_flag[1];
+    for (uint32_t it = 0; it < limit; ++it) {
+        int v;
+        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(c) : "memory");
+        if (v >= want) return true;
+        if ((it & 31u) == 31u && *abort_flag) return false;
+    }
+    *abort_flag = 1;
+    return false;
+}
+__device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async;" ::: "memory"); }
+// barrier and consensus of `n` threads
+__device__ __forceinline__ bool all_of(int id, int n, bool ok) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.red.and.pred q, %2, %3, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"(ok ? 1u : 0u), "r"(id), "r"(n)
+        : "memory");
+    return r != 0;
+}
+__device__ __forceinline__ void bar_n(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z,
+                                            uint64_t hint) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+        " [%0], [%1, {%3, %4, %5}], [%2], %6;" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z), "l"(hint)
+        : "memory");
+}
+// MN-major, 128-byte swizzle: a k row (one key) is 64 elements = 128 bytes, 8 keys are 1024 bytes, the next 64 elements
+// of the M dimension lie 128 keys further
+__device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr) {
+    return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)((FW_KEYS * 128) >> 4) << 16) | (64ull << 32) | (1ull << 46) |
+           (2ull << 61);
+}
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
+    const int n = valid ? 16 : 0;                      // src-size 0: the 16 bytes are zero-filled
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+}
+
+// The attention items of a call: sequences in order, KV heads in order, 128-key tiles in order; block c takes
+// [c * per, (c + 1) * per).
+struct AttnItem {
+    int bi, g, tile, nt;                  // nt: tiles of the sequence
+    int f0;                               // first item of the (sequence, KV head)
+};
+__device__ __forceinline__ AttnItem attn_item(const int* pref, int Hkv, int x) {
+    AttnItem it;
+    int b = 0;
+    while (x >= pref[b + 1]) ++b;
+    const int nt = (pref[b + 1] - pref[b]) / Hkv, y = x - pref[b];
+    it.bi = b;
+    it.nt = nt;
+    it.g = y / nt;
+    it.tile = y - it.g * nt;
+    it.f0 = x - it.tile;
+    return it;
+}
+
+static_assert(1024 + FW_MAX_SLOTS * FW_SLOT + FW_UNION + sizeof(FwTail) <= 227 * 1024, "shared memory of the forward");
+
+template <int HD, int NQP>
+__global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_constant__ FwArgs a) {
+    constexpr int NCH = HD / 64;                       // 64-element chunks of a head row
+    constexpr int NQ2 = 2 * NQP;                       // query rows as hi and lo parts
+    constexpr uint32_t KV_BYTES = FW_KEYS * HD * 2;
+    constexpr int Q_BYTES = NQ2 * HD * 2;              // one query tile
+    constexpr int P_BYTES = NQ2 * FW_KEYS * 2;         // one probability tile
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    const int NS = a.slots;
+    uint8_t* uni = smem + (size_t)NS * FW_SLOT;
+    FwTail& s = *reinterpret_cast<FwTail*>(uni + FW_UNION);
+    float* Y = reinterpret_cast<float*>(uni);
+    uint8_t* Qs = uni;                                 // [2][Q_BYTES]
+    uint8_t* Ps = uni + 2 * Q_BYTES;                   // [2][P_BYTES]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int cta = (int)blockIdx.x, n_cta = a.n_cta;
+    const int T = a.T, cols = a.cols, terms = a.terms;
+    const int n_phases = 5 * a.n_layers + 1;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < NS; ++i) {
+            mbar_init(smem_u32(&s.full[i]), 1);
+            mbar_init(smem_u32(&s.empty[i]), 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(smem_u32(&s.tfull[i]), 1);
+            mbar_init(smem_u32(&s.tempty[i]), 8);
+            mbar_init(smem_u32(&s.sfull[i]), 1);
+            mbar_init(smem_u32(&s.pfull[i]), 4);
+            mbar_init(smem_u32(&s.ofull[i]), 1);
+            mbar_init(smem_u32(&s.oempty[i]), 4);
+            mbar_init(smem_u32(&s.qfull[i]), 4);
+        }
+        s.abort_flag[0] = 0;
+        s.abort_flag[1] = (int)(a.wait_limit ? a.wait_limit : WAIT_LIMIT);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        int run = 0;
+        for (int b = 0; b < a.B; ++b) {
+            s.pref[b] = run;
+            const int nk = min(__ldcg(a.rm.kv_base + b) + __ldcg(a.rm.n_spec + b), a.pieces * FW_KEYS);
+            if (__ldcg(a.rm.n_rows + b) > 0) run += (nk + FW_KEYS - 1) / FW_KEYS * a.Hkv;
+        }
+        s.pref[a.B] = run;
+    }
+    if (warp == 3) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s.tmem_ptr)), "r"(512)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = s.tmem_ptr;
+    volatile int* abort_flag = s.abort_flag;
+    const int a_tot = s.pref[a.B];
+    const int a_per = (a_tot + n_cta - 1) / n_cta;
+    const int a_lo = min(cta * a_per, a_tot), a_hi = min(a_lo + a_per, a_tot), a_n = a_hi - a_lo;
+    auto slot_ptr = [&](int pos) { return smem_u32(smem + (size_t)(pos % NS) * FW_SLOT); };
+    auto full_bar = [&](int pos) { return smem_u32(&s.full[pos % NS]); };
+    auto empty_bar = [&](int pos) { return smem_u32(&s.empty[pos % NS]); };
+    auto ring_par = [&](int pos) { return (uint32_t)(pos / NS) & 1u; };
+    // kind of phase p and its layer
+    auto kind_of = [&](int p) { return p == n_phases - 1 ? (int)FW_LM : p % 5; };
+
+    if (warp == 0) {
+        // ---------------- weight and K / V producer: walks all phases; only the K / V tiles that hold this call's own
+        // rows wait for the phase that writes them
+        if (lane == 0) {
+            int pos = 0;
+            bool ok = true;
+            for (int p = 0; p < n_phases && ok; ++p) {
+                const int kind = kind_of(p), layer = p / 5;
+                const FwLayer* L = a.layers + layer;
+                if (kind == FW_ATTN) {
+                    bool waited = false;
+                    for (int x = a_lo; x < a_hi && ok; ++x) {
+                        const AttnItem it = attn_item(s.pref, a.Hkv, x);
+                        const int seq = __ldcg(a.rm.call_seq + it.bi);
+                        const int plane = ((layer * a.max_batch + seq) * 2) * a.Hkv + it.g;
+                        if (!waited && (it.tile + 1) * FW_KEYS > __ldcg(a.rm.kv_base + it.bi)) {
+                            ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
+                            proxy_fence();
+                            waited = true;
+                        }
+                        for (int kv = 0; kv < 2 && ok; ++kv, ++pos) {
+                            ok = mbar_wait(empty_bar(pos), ring_par(pos) ^ 1u, abort_flag);
+                            if (!ok) break;
+                            const uint32_t bar = full_bar(pos), dst = slot_ptr(pos);
+                            mbar_expect_tx(bar, KV_BYTES);
+#pragma unroll
+                            for (int c = 0; c < NCH; ++c)
+#pragma unroll
+                                for (int k = 0; k < FW_KEYS / 64; ++k)
+                                    tma_load_3d(dst + c * (FW_KEYS * 128) + k * 8192, &a.kv, bar, c * 64,
+                                                it.tile * FW_KEYS + k * 64, plane + kv * a.Hkv, HINT_STREAM);
+                        }
+                    }
+                    continue;
+                }
+                if (kind == FW_QKV && layer + 1 < a.n_layers) {
+                    const CUtensorMap* nm = &L[1].wq;
+#pragma unroll
+                    for (int i = 0; i < 7; ++i)
+                        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(nm + i)) : "memory");
+                }
+                const FwPhase& f = a.ph[kind];
+                const int nsub = f.S * f.kp;
+                const uint32_t sub_stride = f.S > 1 ? (uint32_t)(TC_TILE_N / f.S) * 128u : (uint32_t)f.a_bytes;
+                for (int tile = cta; tile < f.n_tiles && ok; tile += n_cta) {
+                    const int unit0 = tile * f.upt, nu = min(f.upt, f.n_units - unit0);
+                    const uint32_t bytes = (uint32_t)(nsub * (nu * f.box_bytes + cols * 128));
+                    for (int step = 0; step < f.steps; ++step, ++pos) {
+                        ok = mbar_wait(empty_bar(pos), ring_par(pos) ^ 1u, abort_flag);
+                        if (!ok) break;
+                        const uint32_t bar = full_bar(pos), base = slot_ptr(pos);
+                        mbar_expect_tx(bar, bytes);
+                        for (int sb = 0; sb < nsub; ++sb) {
+                            const int kx = (step * nsub + sb) * TC_TILE_K;
+                            uint32_t dst = base + sb * sub_stride;
+                            for (int uu = 0; uu < nu; ++uu, dst += f.slots * 128) {
+                                const int unit = unit0 + uu;
+                                if (kind == FW_QKV) {
+                                    const int hg = unit / f.u, j0 = (unit - hg * f.u) * f.h;
+                                    const CUtensorMap* m = hg < a.Hq ? &L->wq : (hg < a.Hq + a.Hkv ? &L->wk : &L->wv);
+                                    const int hl = hg < a.Hq ? hg : (hg < a.Hq + a.Hkv ? hg - a.Hq : hg - a.Hq - a.Hkv);
+                                    tma_load_3d(dst, m, bar, kx, j0, 2 * hl, HINT_STREAM);
+                                } else if (kind == FW_GATEUP) {
+                                    tma_load_2d(dst, &L->gate, bar, kx, unit * f.h, HINT_STREAM);
+                                    tma_load_2d(dst + (f.slots >> 1) * 128, &L->up, bar, kx, unit * f.h, HINT_STREAM);
+                                } else {
+                                    const CUtensorMap* m = kind == FW_O ? &L->wo : (kind == FW_DOWN ? &L->down : &a.lm);
+                                    tma_load_2d(dst, m, bar, kx, unit * f.h, HINT_STREAM);
+                                }
+                            }
+                        }
+                    }
+                }
+            }
+            if (!ok)       // give the copies in flight a bounded chance to land before the block exits
+                for (int j = max(0, pos - NS); j < pos; ++j)
+                    for (uint32_t it = 0; it < (1u << 12) && !mbar_test(full_bar(j), ring_par(j)); ++it) __nanosleep(64);
+        }
+    } else if (warp == 1) {
+        // ---------------- operand-row producer: the rows of a phase exist once every block has finished the one before
+        if (lane == 0) {
+            int pos = 0;
+            bool ok = true;
+            for (int p = 0; p < n_phases && ok; ++p) {
+                const int kind = kind_of(p);
+                if (kind == FW_ATTN) { pos += 2 * a_n; continue; }
+                const FwPhase& f = a.ph[kind];
+                const int nsub = f.S * f.kp;
+                const CUtensorMap* m = kind == FW_O ? &a.xa : (kind == FW_DOWN ? &a.xf : &a.xd);
+                if (p > 0) {
+                    ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
+                    proxy_fence();
+                }
+                for (int tile = cta; tile < f.n_tiles && ok; tile += n_cta)
+                    for (int step = 0; step < f.steps; ++step, ++pos) {
+                        ok = mbar_wait(empty_bar(pos), ring_par(pos) ^ 1u, abort_flag);
+                        if (!ok) break;
+                        const uint32_t bar = full_bar(pos), base = slot_ptr(pos) + f.b_off;
+                        if (!a.debug_no_operands)
+                            for (int sb = 0; sb < nsub; ++sb)
+                                tma_load_2d(base + sb * cols * 128, m, bar, (step * nsub + sb) * TC_TILE_K, 0, HINT_KEEP);
+                    }
+            }
+        }
+    } else if (warp == 2) {
+        // ---------------- MMA issuer
+        if (lane == 0) {
+            constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (8u << 24);      // bf16 x bf16 -> fp32, M = 128
+            int pos = 0, tcount = 0, at = 0, as = 0;   // ring position, projection tiles, attention tiles, segments so far
+            bool ok = true;
+            for (int p = 0; p < n_phases && ok; ++p) {
+                const int kind = kind_of(p);
+                if (kind == FW_ATTN) {
+                    constexpr uint32_t idesc_s = IDESC | ((uint32_t)(NQ2 >> 3) << 17);
+                    constexpr uint32_t idesc_o = IDESC | (1u << 15) | ((uint32_t)(NQ2 >> 3) << 17);
+                    // scores of the block's tile i
+                    auto scores = [&](int i) -> bool {
+                        const AttnItem it = attn_item(s.pref, a.Hkv, a_lo + i);
+                        const bool fresh = i == 0 || it.tile == 0;
+                        if (fresh && i > 0) ++as;
+                        if (fresh && !mbar_wait(smem_u32(&s.qfull[as & 1]), (uint32_t)(as >> 1) & 1u, abort_flag)) return false;
+                        const int kpos = pos + 2 * i, b = (at + i) & 1;
+                        if (!mbar_wait(full_bar(kpos), ring_par(kpos), abort_flag)) return false;
+                        tc_fence_after();
+                        const uint32_t ka = slot_ptr(kpos), qa = smem_u32(Qs + (as & 1) * Q_BYTES);
+#pragma unroll
+                        for (int ks = 0; ks < HD / 16; ++ks)
+                            tc_mma(tmem + b * 64, smem_desc(ka + (ks >> 2) * (FW_KEYS * 128) + (ks & 3) * 32),
+                                   smem_desc(qa + (ks >> 2) * (NQ2 * 128) + (ks & 3) * 32), idesc_s, ks > 0 ? 1u : 0u);
+                        tc_commit(smem_u32(&s.sfull[b]));
+                        tc_commit(empty_bar(kpos));
+                        return true;
+                    };
+                    if (a_n > 0) ok = scores(0);
+                    for (int i = 0; i < a_n && ok; ++i) {
+                        if (i + 1 < a_n) ok = scores(i + 1);
+                        if (!ok) break;
+                        const int vpos = pos + 2 * i + 1, b = (at + i) & 1;
+                        const uint32_t par = (uint32_t)((at + i) >> 1) & 1u;
+                        ok = mbar_wait(smem_u32(&s.pfull[b]), par, abort_flag) && mbar_wait(full_bar(vpos), ring_par(vpos), abort_flag) &&
+                             mbar_wait(smem_u32(&s.oempty[b]), par ^ 1u, abort_flag);
+                        if (!ok) break;
+                        tc_fence_after();
+                        const uint32_t va = slot_ptr(vpos), pa = smem_u32(Ps + b * P_BYTES);
+#pragma unroll
+                        for (int ks = 0; ks < FW_KEYS / 16; ++ks)
+                            tc_mma(tmem + FW_TM_D + b * 64, smem_desc_mn(va + ks * 2048),
+                                   smem_desc(pa + (ks >> 2) * (NQ2 * 128) + (ks & 3) * 32), idesc_o, ks > 0 ? 1u : 0u);
+                        tc_commit(smem_u32(&s.ofull[b]));
+                        tc_commit(empty_bar(vpos));
+                    }
+                    if (a_n > 0) ++as;
+                    at += a_n;
+                    pos += 2 * a_n;
+                    continue;
+                }
+                const FwPhase& f = a.ph[kind];
+                const int mh = (f.rows + TC_TILE_N - 1) / TC_TILE_N;
+                const uint32_t idesc = IDESC | ((uint32_t)((f.S * cols) >> 3) << 17);
+                for (int tile = cta; tile < f.n_tiles && ok; tile += n_cta, ++tcount) {
+                    const int buf = tcount & 1;
+                    ok = mbar_wait(smem_u32(&s.tempty[buf]), ((uint32_t)(tcount >> 1) & 1u) ^ 1u, abort_flag);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t d = tmem + buf * 256;
+                    for (int step = 0; step < f.steps; ++step, ++pos) {
+                        ok = mbar_wait(full_bar(pos), ring_par(pos), abort_flag);
+                        if (!ok) break;
+                        tc_fence_after();
+                        const uint32_t base = slot_ptr(pos), bb = base + f.b_off;
+                        for (int sb = 0; sb < f.kp; ++sb)
+                            for (int m = 0; m < mh; ++m)
+#pragma unroll
+                                for (int k4 = 0; k4 < TC_TILE_K / 16; ++k4)
+                                    tc_mma(d + m * cols, smem_desc(base + sb * f.a_bytes + m * (TC_TILE_N * 128) + k4 * 32),
+                                           smem_desc(bb + sb * cols * 128 + k4 * 32), idesc, (step > 0 || sb > 0 || k4 > 0) ? 1u : 0u);
+                        tc_commit(empty_bar(pos));
+                    }
+                    if (ok) tc_commit(smem_u32(&s.tfull[buf]));
+                }
+            }
+        }
+    } else if (warp >= FW_EPI_WARP0) {
+        // ---------------- epilogue warps
+        const int e = threadIdx.x - 32 * FW_EPI_WARP0;   // 0..255
+        const int w = warp - FW_EPI_WARP0;                // 0..7
+        const int quad = warp & 3, half = w >> 2;         // TMEM lane quadrant; which of the quadrant's two warps
+        const uint32_t t_lane = tmem + ((uint32_t)(quad * 32) << 16);
+        int tcount = 0, at = 0, as = 0, pos = 0;
+        bool ok = true;
+        for (int p = 0; p < n_phases && ok; ++p) {
+            const int kind = kind_of(p), layer = p / 5;
+            if (kind == FW_ATTN) {
+                if (e == 0) ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
+                ok = all_of(1, FW_EPI, ok);
+                if (!ok) break;
+                const int G = a.Hq / a.Hkv, kl = quad * 32 + lane;    // this thread's key of a tile, or its head dimension
+                float m[NQP], l[NQP], acc[NQP];
+                for (int x = a_lo; x < a_hi; ++x) {
+                    const AttnItem it = attn_item(s.pref, a.Hkv, x);
+                    const int nrows = __ldcg(a.rm.n_rows + it.bi), L = __ldcg(a.rm.kv_base + it.bi);
+                    const int nkeys = min(L + __ldcg(a.rm.n_spec + it.bi), a.pieces * FW_KEYS);
+                    const int n_q = min(G * nrows, NQP);
+                    const int t0 = it.bi * a.R, h0 = it.g * G;        // query row i: row t0 + i % nrows, head h0 + i / nrows
+                    const bool fresh = x == a_lo || it.tile == 0;
+                    const int b = at & 1;
+                    const uint32_t par = (uint32_t)(at >> 1) & 1u;
+                    if (fresh) {
+#pragma unroll
+                        for (int r = 0; r < NQP; ++r) { m[r] = -CUDART_INF_F; l[r] = 0.f; acc[r] = 0.f; }
+                    }
+                    if (half == 0) {
+                        // -------- softmax: a lane per key
+                        if (fresh) {
+                            uint8_t* q = Qs + (as & 1) * Q_BYTES;
+                            for (int i = kl; i < NQ2 * (HD / 8); i += 128) {
+                                const int row = i / (HD / 8), c = i % (HD / 8), r = row & (NQP - 1);
+                                const bool valid = r < n_q;
+                                const int rr = valid ? r : 0;
+                                const __nv_bfloat16* src = (row >= NQP ? a.q_lo : a.q_hi) +
+                                    ((size_t)(t0 + rr % nrows) * a.Hq + h0 + rr / nrows) * HD + c * 8;
+                                cp_async16(smem_u32(q + (c >> 3) * (NQ2 * 128) + row * 128 + (((c & 7) ^ (row & 7)) << 4)), src, valid);
+                            }
+                            asm volatile("cp.async.wait_all;" ::: "memory");
+                            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(smem_u32(&s.qfull[as & 1]));
+                        }
+                        if (ok) ok = mbar_wait(smem_u32(&s.sfull[b]), par, abort_flag);
+                        __syncwarp();
+                        tc_fence_after();
+                        float v[NQP];
+                        {
+                            float c[NQ2];
+                            if (NQ2 == 16) tc_ld16(t_lane + b * 64, c);
+                            else { tc_ld16(t_lane + b * 64, c); tc_ld16(t_lane + b * 64 + 16, c + 16); }
+#pragma unroll
+                            for (int r = 0; r < NQP; ++r) v[r] = c[r] + c[NQP + r];
+                        }
+                        const int j = it.tile * FW_KEYS + kl;
+                        if ((it.tile + 1) * FW_KEYS > L) {
+                            // the tile reaches into the draft rows: ancestors and self only, nothing past the last key
+                            const int sr = j - L;
+#pragma unroll
+                            for (int r = 0; r < NQP; ++r) {
+                                bool vis = j < nkeys && r < n_q;
+                                if (vis && sr >= 0)
+                                    vis = (a.rm.mask[(size_t)(t0 + r % nrows) * MTAD_MASK_WORDS + (sr >> 5)] >> (sr & 31)) & 1u;
+                                if (!vis) v[r] = -CUDART_INF_F;
+                            }
+                        }
+                        float wm[NQP];
+#pragma unroll
+                        for (int r = 0; r < NQP; ++r) wm[r] = v[r];
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                            for (int r = 0; r < NQP; ++r) wm[r] = fmaxf(wm[r], __shfl_xor_sync(0xffffffffu, wm[r], o));
+#pragma unroll
+                        for (int r = 0; r < NQP; ++r)
+                            if (lane == r) s.smx[b][r][quad] = wm[r];
+                        // the buffers P and sf of this tile are free once the output warps are done with the tile before the last
+                        if (ok) ok = mbar_wait(smem_u32(&s.oempty[b]), par ^ 1u, abort_flag);
+                        ok = all_of(2, 128, ok);
+                        uint8_t* pt = Ps + b * P_BYTES + (kl >> 6) * (NQ2 * 128) + (kl & 7) * 2;
+                        const int pc = (kl & 63) >> 3;
+#pragma unroll
+                        for (int r = 0; r < NQP; ++r) {
+                            const float4 q4 = *reinterpret_cast<const float4*>(s.smx[b][r]);
+                            const float mn = fmaxf(m[r], fmaxf(fmaxf(q4.x, q4.y), fmaxf(q4.z, q4.w)));
+                            const float f = mn == -CUDART_INF_F ? 1.f : exp2f(m[r] - mn);
+                            const float pv = mn == -CUDART_INF_F ? 0.f : exp2f(v[r] - mn);      // exp2(-inf) = 0
+                            m[r] = mn;
+                            l[r] = l[r] * f + pv;
+                            if (kl == r) s.sf[b][r] = f;
+                            const __nv_bfloat16 hi = __float2bfloat16_rn(pv);
+                            *reinterpret_cast<__nv_bfloat16*>(pt + r * 128 + ((pc ^ (r & 7)) << 4)) = hi;
+                            *reinterpret_cast<__nv_bfloat16*>(pt + (NQP + r) * 128 + ((pc ^ (r & 7)) << 4)) =
+                                __float2bfloat16_rn(pv - __bfloat162float(hi));
+                        }
+                        if ((it.tile + 1) * FW_KEYS > nkeys) {
+                            // rows of V past the last key: their probabilities are 0, but 0 x (stale value) must not make a NaN
+                            const int vpos = pos + 2 * (x - a_lo) + 1;
+                            if (ok) ok = mbar_wait(full_bar(vpos), ring_par(vpos), abort_flag);
+                            if (ok && j >= nkeys) {
+                                uint8_t* vs = smem + (size_t)(vpos % NS) * FW_SLOT + kl * 128;
+#pragma unroll
+                                for (int c = 0; c < NCH * 8; ++c)
+                                    *reinterpret_cast<uint4*>(vs + (c >> 3) * (FW_KEYS * 128) + (c & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
+                            }
+                        }
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&s.pfull[b]));
+                    } else {
+                        // -------- output: a lane per head dimension
+                        if (ok) ok = mbar_wait(smem_u32(&s.ofull[b]), par, abort_flag);
+                        __syncwarp();
+                        tc_fence_after();
+                        float c[NQ2];
+                        if (NQ2 == 16) tc_ld16(t_lane + FW_TM_D + b * 64, c);
+                        else { tc_ld16(t_lane + FW_TM_D + b * 64, c); tc_ld16(t_lane + FW_TM_D + b * 64 + 16, c + 16); }
+#pragma unroll
+                        for (int r = 0; r < NQP; ++r) acc[r] = acc[r] * s.sf[b][r] + (c[r] + c[NQP + r]);
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&s.oempty[b]));
+                    }
+                    ++at;
+                    if (x + 1 == a_hi || it.tile + 1 == it.nt) {
+                        // -------- end of a segment: the row sums meet, then the rows leave (final, or as a piece)
+                        const int sb = as & 1;
+                        if (half == 0) {
+#pragma unroll
+                            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                                for (int r = 0; r < NQP; ++r) l[r] += __shfl_xor_sync(0xffffffffu, l[r], o);
+#pragma unroll
+                            for (int r = 0; r < NQP; ++r) {
+                                if (lane == r) s.sl[sb][quad][r] = l[r];
+                                if (kl == r) s.sm[sb][r] = m[r];
+                            }
+                        }
+                        ok = all_of(1, FW_EPI, ok);
+                        const int first = it.f0 / a_per, n_piece = (it.f0 + it.nt - 1) / a_per - first + 1, piece = cta - first;
+                        if (half == 1 && ok) {
+#pragma unroll
+                            for (int r = 0; r < NQP; ++r) {
+                                if (r >= n_q || (HD < 128 && kl >= HD)) continue;
+                                const int t = t0 + r % nrows, h = h0 + r / nrows;
+                                const float ls = (s.sl[sb][0][r] + s.sl[sb][1][r]) + (s.sl[sb][2][r] + s.sl[sb][3][r]);
+                                if (n_piece == 1) {
+                                    store_terms(acc[r] / ls, a.x_a + (size_t)t * terms * a.Hq * HD + (size_t)h * HD + kl,
+                                                (size_t)a.Hq * HD, terms);
+                                } else {
+                                    const size_t o = ((size_t)t * a.Hq + h) * a.pieces + piece;
+                                    a.part[o * HD + kl] = acc[r];
+                                    if (kl == 0)
+                                        reinterpret_cast<float2*>(a.part + (size_t)T * a.Hq * a.pieces * HD)[o] = make_float2(s.sm[sb][r], ls);
+                                }
+                            }
+                        }
+                        ++as;
+                    }
+                }
+                pos += 2 * a_n;
+                // pieces shared with other blocks (at most the first and the last segment): the last to arrive merges
+                if (a_n > 0) {
+                    const AttnItem i0 = attn_item(s.pref, a.Hkv, a_lo), i1 = attn_item(s.pref, a.Hkv, a_hi - 1);
+                    const bool two = i1.f0 != i0.f0;
+                    ok = all_of(1, FW_EPI, ok);
+                    if (!ok) break;
+                    if (e < 2) {
+                        const AttnItem it = e == 0 ? i0 : i1;
+                        const int n_piece = (it.f0 + it.nt - 1) / a_per - it.f0 / a_per + 1;
+                        int last = 0;
+                        if (n_piece > 1 && (e == 0 || two)) {
+                            __threadfence();
+                            last = atomicAdd(a.acnt + it.bi * a.Hkv + it.g, 1) + 1 == n_piece;
+                            __threadfence();
+                        }
+                        s.last[e] = last;
+                    }
+                    bar_n(1, FW_EPI);
+                    for (int q = 0; q < 2; ++q) {
+                        if (!s.last[q]) continue;
+                        const AttnItem it = q == 0 ? i0 : i1;
+                        const int nrows = __ldcg(a.rm.n_rows + it.bi), n_q = min(G * nrows, NQP);
+                        const int n_piece = (it.f0 + it.nt - 1) / a_per - it.f0 / a_per + 1;
+                        for (int i = e; i < n_q * (HD / 4); i += FW_EPI) {
+                            const int r = i / (HD / 4), c4 = i % (HD / 4);
+                            const int t = it.bi * a.R + r % nrows, h = it.g * G + r / nrows;
+                            const size_t o = ((size_t)t * a.Hq + h) * a.pieces;
+                            const float2* ml = reinterpret_cast<const float2*>(a.part + (size_t)T * a.Hq * a.pieces * HD) + o;
+                            const float4* po = reinterpret_cast<const float4*>(a.part + o * HD) + c4;
+                            float M = -CUDART_INF_F;
+                            for (int k = 0; k < n_piece; ++k) M = fmaxf(M, __ldcg(ml + k).x);
+                            float4 o4 = make_float4(0.f, 0.f, 0.f, 0.f);
+                            float ls = 0.f;
+                            for (int k = 0; k < n_piece; ++k) {          // piece order: deterministic
+                                const float2 v = __ldcg(ml + k);
+                                const float4 y = __ldcg(po + (size_t)k * (HD / 4));
+                                const float wg = v.x == -CUDART_INF_F ? 0.f : exp2f(v.x - M);
+                                ls += wg * v.y;
+                                o4.x += wg * y.x; o4.y += wg * y.y; o4.z += wg * y.z; o4.w += wg * y.w;
+                            }
+                            const float f = 1.f / ls;
+                            store_terms4(make_float4(o4.x * f, o4.y * f, o4.z * f, o4.w * f),
+                                         a.x_a + (size_t)t * terms * a.Hq * HD + (size_t)h * HD + c4 * 4, (size_t)a.Hq * HD, terms);
+                        }
+                        if (e == 0) a.acnt[it.bi * a.Hkv + it.g] = 0;     // ready for the next layer
+                    }
+                }
+            } else {
+                const FwPhase& f = a.ph[kind];
+                const FwLayer* L = a.layers + layer;
+                const int mine = cta < f.n_tiles ? (f.n_tiles - 1 - cta) / n_cta + 1 : 0;
+                const int ys = (f.S > 1 ? TC_TILE_N : f.rows) + 4;     // row stride of Y
+                const int nf = f.upt * f.h;                            // features (pairs) of a tile
+                if (mine > 0 && (kind == FW_QKV || kind == FW_GATEUP || kind == FW_LM)) {
+                    // scale of the deferred RMSNorm: the rows' sums of squares come from every block
+                    if (p > 0) {
+                        if (e == 0) ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
+                        ok = all_of(1, FW_EPI, ok);
+                        if (!ok) break;
+                    }
+                    const float* sq = kind == FW_GATEUP ? a.sumsq_b : a.sumsq_a;
+                    const int parts = kind == FW_GATEUP ? a.ph[FW_O].n_tiles : (p == 0 ? a.parts0 : a.ph[FW_DOWN].n_tiles);
+                    for (int r = w; r < T; r += 8) {
+                        float v = 0.f;
+                        for (int q = lane; q < parts; q += 32) v += __ldcg(sq + (size_t)q * TC_X_ROWS + r);
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                        if (lane == 0) s.rstd[r] = rsqrtf(v * a.inv_dim + a.eps);
+                    }
+                }
+                pos += mine * f.steps;
+                for (int tile = cta; tile < f.n_tiles; tile += n_cta, ++tcount) {
+                    const int buf = tcount & 1, unit0 = tile * f.upt;
+                    // what the first items of this thread need besides the accumulator, requested ahead of it
+                    float pre[4] = {0.f, 0.f, 0.f, 0.f};
+                    float u8[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) u8[i] = 0.5f;
+                    if (kind == FW_O || kind == FW_DOWN) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const int n = unit0 * f.h + lane + 32 * i;
+                            if (w < T && lane + 32 * i < nf && n < a.d) pre[i] = __ldcg(a.hidden + (size_t)w * a.d + n);
+                        }
+                    } else if (kind == FW_LM && !a.lm_plain) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const int n = unit0 * f.h + lane + 32 * i;
+                            if (w < T && lane + 32 * i < nf && n < a.V) u8[i] = a.uniforms[(size_t)(w / a.R) * a.V + n];
+                        }
+                    }
+                    ok = mbar_wait(smem_u32(&s.tfull[buf]), (uint32_t)(tcount >> 1) & 1u, abort_flag);
+                    __syncwarp();
+                    tc_fence_after();
+                    {   // accumulators -> Y[row][slot], the terms of a row added up
+                        const uint32_t t_acc = t_lane + buf * 256;
+                        const int mh = f.S > 1 ? 1 : (f.rows + TC_TILE_N - 1) / TC_TILE_N;
+                        const int slice = f.S == 4 ? quad : (f.S == 2 ? quad >> 1 : 0);
+                        const int per = terms == 3 ? 5 : 8, ng = (T + per - 1) / per;
+                        for (int i = half; i < mh * ng; i += 2) {
+                            const int mm = i / ng, rb = (i - mm * ng) * per, slot = mm * TC_TILE_N + quad * 32 + lane;
+                            float v[16];
+                            tc_ld16(t_acc + (mm + slice) * cols + rb * terms, v);
+                            if (slot < ys - 4) {
+                                if (terms == 3) {
+#pragma unroll
+                                    for (int j = 0; j < 5; ++j)
+                                        if (rb + j < T) Y[(rb + j) * ys + slot] = v[3 * j] + (v[3 * j + 1] + v[3 * j + 2]);
+                                } else {
+#pragma unroll
+                                    for (int j = 0; j < 8; ++j)
+                                        if (rb + j < T) Y[(rb + j) * ys + slot] = v[2 * j] + v[2 * j + 1];
+                                }
+                            }
+                        }
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&s.tempty[buf]));
+                    ok = all_of(1, FW_EPI, ok);
+                    if (!ok) break;
+                    // value of (row, slot): the S slices of the step lie side by side
+                    const int sst = TC_TILE_N / f.S;
+                    auto yv = [&](int t, int slot) -> float {
+                        const float* y = Y + t * ys + slot;
+                        float v = y[0];
+                        if (f.S == 4) v = (v + y[sst]) + (y[2 * sst] + y[3 * sst]);
+                        else if (f.S == 2) v += y[sst];
+                        return v;
+                    };
+                    if (kind == FW_QKV) {
+                        const int hp = HD / 2;
+                        const float scale = rsqrtf((float)HD);
+                        for (int i = e; i < T * nf; i += FW_EPI) {
+                            const int t = i / nf, jl = i - t * nf, uu = jl / f.h, j = jl - uu * f.h, unit = unit0 + uu;
+                            if (unit >= f.n_units) continue;
+                            const int hg = unit / f.u, jj = (unit - hg * f.u) * f.h + j;
+                            if (jj >= hp) continue;
+                            const int sl = a.rm.slot[t];
+                            const float2 cs = *reinterpret_cast<const float2*>(a.rope + ((size_t)t * hp + jj) * 2);
+                            const float rs = s.rstd[t];
+                            const float va = yv(t, uu * f.slots + j) * rs, vb = yv(t, uu * f.slots + f.h + j) * rs;
+                            if (sl < 0) continue;                         // inactive row: no query, no cache slot
+                            const float ra = va * cs.x - vb * cs.y, rb = vb * cs.x + va * cs.y;
+                            if (hg < a.Hq) {
+                                // attention operands: q * log2(e) / sqrt(hd) as bf16 hi + lo (softmax runs on exp2)
+                                const size_t o = ((size_t)t * a.Hq + hg) * HD + jj;
+                                split_store(ra * scale * 1.4426950408889634f, a.q_hi + o, a.q_lo + o);
+                                split_store(rb * scale * 1.4426950408889634f, a.q_hi + o + hp, a.q_lo + o + hp);
+                            } else {
+                                const int sq = a.rm.seq[t], kv = hg >= a.Hq + a.Hkv ? 1 : 0;
+                                if (sl >= a.cap || (unsigned)sq >= (unsigned)a.max_batch) continue;   // never past the cache
+                                __nv_bfloat16* c = a.cache + idx_cache(layer, a.max_batch, sq, kv, a.Hkv, hg - a.Hq - kv * a.Hkv, a.cap, sl, HD);
+                                c[jj] = __float2bfloat16_rn(kv ? va : ra);
+                                c[jj + hp] = __float2bfloat16_rn(kv ? vb : rb);
+                            }
+                        }
+                    } else if (kind == FW_GATEUP) {
+                        for (int i = e; i < T * nf; i += FW_EPI) {
+                            const int t = i / nf, jl = i - t * nf, uu = jl / f.h, j = jl - uu * f.h, n = (unit0 + uu) * f.h + j;
+                            if (n >= a.F) continue;
+                            const float rs = s.rstd[t];
+                            const float g = yv(t, uu * f.slots + j) * rs, up = yv(t, uu * f.slots + (f.slots >> 1) + j) * rs;
+                            store_terms(g / (1.f + expf(-g)) * up, a.x_f + (size_t)t * terms * a.F + n, a.F, terms);
+                        }
+                    } else if (kind == FW_LM && a.lm_plain) {
+                        for (int i = e; i < T * nf; i += FW_EPI) {
+                            const int t = i / nf, jl = i - t * nf, uu = jl / f.h, n = unit0 * f.h + jl;
+                            if (n < a.V) a.logits[(size_t)t * a.V + n] = yv(t, uu * f.slots + jl - uu * f.h) * s.rstd[t];
+                        }
+                    } else if (kind == FW_LM) {
+                        // a warp per row: maximum, sum of exponentials, arg-max of the perturbed logits over the tile
+                        for (int t = w; t < T; t += 8) {
+                            float z[8], m = -CUDART_INF_F, bv = -CUDART_INF_F, sum = 0.f;
+                            int bi = 0x7fffffff;
+                            const float rs = s.rstd[t];
+                            if (t != w)
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) {
+                                    const int n = unit0 * f.h + lane + 32 * i;
+                                    u8[i] = (lane + 32 * i < nf && n < a.V) ? a.uniforms[(size_t)(t / a.R) * a.V + n] : 0.5f;
+                                }
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                const int jl = lane + 32 * i, n = unit0 * f.h + jl, uu = jl / f.h;
+                                const bool in = jl < nf && n < a.V;
+                                z[i] = in ? yv(t, uu * f.slots + jl - uu * f.h) * rs : -CUDART_INF_F;
+                                m = fmaxf(m, z[i]);
+                                const float pz = in ? z[i] - logf(-logf(u8[i])) : -CUDART_INF_F;
+                                if (in && (pz > bv || (pz == bv && n < bi))) { bv = pz; bi = n; }
+                            }
+#pragma unroll
+                            for (int o = 16; o > 0; o >>= 1) {
+                                m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+                                const float v2 = __shfl_xor_sync(0xffffffffu, bv, o);
+                                const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
+                                if (v2 > bv || (v2 == bv && i2 < bi)) { bv = v2; bi = i2; }
+                            }
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) sum += z[i] == -CUDART_INF_F ? 0.f : expf(z[i] - m);
+#pragma unroll
+                            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                            if (lane == 0) a.lm_part[idx_lm_part(t, f.n_tiles, tile)] = make_float4(m, sum, bv, __int_as_float(bi));
+                        }
+                        // logit of each node's token under its parent row, where it falls into this tile
+                        for (int t = e; t < T; t += FW_EPI) {
+                            const int pr = a.rm.prow[t];
+                            if (pr < 0 || pr >= T) continue;
+                            const int tk = a.rm.tok[t] - unit0 * f.h, uu = tk / f.h;
+                            if (tk >= 0 && tk < nf) a.node_z[t] = yv(pr, uu * f.slots + tk - uu * f.h) * s.rstd[pr];
+                        }
+                    } else {
+                        // residual: a warp per row; emits the next operand rows and the row's share of its sum of squares
+                        const __nv_bfloat16* gain = kind == FW_O ? L->gain_ffn : L->gain_next;
+                        float* sq = kind == FW_O ? a.sumsq_b : a.sumsq_a;
+                        for (int t = w; t < T; t += 8) {
+                            float ss = 0.f;
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const int jl = lane + 32 * i, uu = jl / f.h, n = unit0 * f.h + jl;
+                                if (jl >= nf || n >= a.d) continue;
+                                float* hp = a.hidden + (size_t)t * a.d + n;
+                                const float y = yv(t, uu * f.slots + jl - uu * f.h) + (t == w ? pre[i] : __ldcg(hp));
+                                *hp = y;
+                                store_terms(y * __bfloat162float(gain[n]), a.x_d + (size_t)t * terms * a.d + n, a.d, terms);
+                                ss += y * y;
+                            }
+#pragma unroll
+                            for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+                            if (lane == 0) sq[(size_t)tile * TC_X_ROWS + t] = ss;
+                        }
+                    }
+                    if (tile + n_cta < f.n_tiles) bar_n(1, FW_EPI);       // Y is rewritten by the next tile
+                }
+                if (!ok) break;
+            }
+            if (kind != FW_LM) {
+                // phase barrier: this block's rows are visible to the other blocks' loads and TMA copies
+                proxy_fence();
+                bar_n(1, FW_EPI);
+                if (e == 0) {
+                    __threadfence();
+                    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(a.sync + p) : "memory");
+                }
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 3) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    }
+    if (threadIdx.x == 0 && *abort_flag && a.status)
+        for (int b = 0; b < a.B; ++b) atomicOr(a.status + b, MTAD_ST_TIMEOUT);
+}
+
+int up_div(int x, int y) { return (x + y - 1) / y; }
+int up8(int x) { return (x + 7) / 8 * 8; }
+
+}  // namespace
+
+void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta) {
+    auto rows = [&](FwPhase& f, int N, int per_cta) {
+        f.h = std::min(128, std::max(8, up_div(N, n_cta * per_cta)));
+        f.slots = up8(f.h);
+        f.n_units = up_div(N, f.h);
+        f.u = 1;
+        f.box_bytes = f.h * 128;
+    };
+    const int qd = d.n_q_heads * d.head_dim;
+    rows(ph[FW_O], d.d_model, 1);
+    rows(ph[FW_DOWN], d.d_model, 1);
+    rows(ph[FW_LM], d.vocab, 2);
+    rows(ph[FW_GATEUP], d.d_ffn, 2);
+    ph[FW_O].k_blocks = up_div(qd, TC_TILE_K);
+    ph[FW_DOWN].k_blocks = up_div(d.d_ffn, TC_TILE_K);
+    ph[FW_LM].k_blocks = ph[FW_GATEUP].k_blocks = ph[FW_QKV].k_blocks = up_div(d.d_model, TC_TILE_K);
+    ph[FW_GATEUP].slots *= 2;
+    ph[FW_GATEUP].box_bytes *= 2;
+    // QKV: a head's rotary pairs in u units of h; the cut whose busiest block streams the fewest rows
+    const int hp = d.head_dim / 2, heads = d.n_q_heads + 2 * d.n_kv_heads;
+    FwPhase& q = ph[FW_QKV];
+    long long best = -1;
+    for (int h = std::min(hp, 8); h <= hp; ++h) {
+        const int u = up_div(hp, h), upt = up_div(heads * u, n_cta);
+        const long long rows_max = (long long)upt * 2 * h;
+        if (upt * up8(2 * h) > 256 && upt > 1) continue;
+        const long long cost = rows_max * 64 + upt;            // fewer boxes among equals
+        if (best < 0 || cost < best) { best = cost; q.h = h; q.u = u; }
+    }
+    if (best < 0) { q.h = hp; q.u = 1; }
+    q.n_units = heads * q.u;
+    q.slots = up8(2 * q.h);
+    q.box_bytes = 2 * q.h * 128;
+}
+
+bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
+    const int T = B * R, G = d.n_q_heads / d.n_kv_heads;
+    if (d.head_dim != 64 && d.head_dim != 128) return false;
+    if (T > FW_MAX_ROWS || G * R > FW_MAX_QROWS || B > MTAD_MAX_BATCH) return false;
+    if (d.d_model >= 8192 && T > 32) return false;          // the accurate K / V projection has launches of its own
+    fw_geometry(a.ph, d, n_cta);
+    a.T = T; a.B = B; a.R = R; a.terms = tc_terms(T);
+    a.cols = (a.terms * T + 15) / 16 * 16;
+    a.n_cta = n_cta; a.n_layers = d.layers;
+    a.d = d.d_model; a.F = d.d_ffn; a.V = d.vocab; a.Hq = d.n_q_heads; a.Hkv = d.n_kv_heads; a.hd = d.head_dim;
+    a.slots = FW_MAX_SLOTS;
+    const int bb = a.cols * 128;                            // operand rows of one k-block
+    for (int k = 0; k < 6; ++k) {
+        if (k == FW_ATTN) continue;
+        FwPhase& f = a.ph[k];
+        bool found = false;
+        for (f.upt = up_div(f.n_units, n_cta); f.upt >= 1; --f.upt) {
+            f.rows = f.upt * f.slots;
+            const int mh = up_div(f.rows, TC_TILE_N);
+            if (f.rows > 256 || mh * a.cols > 256) continue;
+            f.S = 1; f.kp = 1; f.a_bytes = f.rows * 128;
+            if (f.rows <= 32 && 4 * bb <= 16384 && f.k_blocks >= 4) f.S = 4;
+            else if (f.rows <= 64 && 2 * bb <= 16384 && f.k_blocks >= 2) f.S = 2;
+            if (f.S > 1) {
+                f.b_off = TC_TILE_N * 128;
+            } else {
+                if (f.a_bytes + bb > FW_SLOT) continue;
+                f.kp = std::min(std::min(4, FW_SLOT / (f.a_bytes + bb)), f.k_blocks);
+                f.b_off = f.kp * f.a_bytes;
+            }
+            // the epilogue tile must fit its area
+            if ((size_t)T * ((f.S > 1 ? TC_TILE_N : f.rows) + 4) * 4 > FW_UNION) continue;
+            found = true;
+            break;
+        }
+        if (!found) return false;
+        f.n_tiles = up_div(f.n_units, f.upt);
+        f.steps = up_div(f.k_blocks, f.S * f.kp);
+        if ((k == FW_O || k == FW_DOWN) && (f.upt * f.h > 128 || f.n_tiles > n_cta)) return false;
+        if (k == FW_LM && f.upt * f.h > 256) return false;
+    }
+    return true;
+}
+
+size_t fw_parts_max(const mtad_model_desc& d, int n_cta, bool lm) {
+    FwPhase ph[6];
+    fw_geometry(ph, d, n_cta);
+    return (size_t)ph[lm ? FW_LM : FW_O].n_units;
+}
+
+cudaError_t launch_forward(const FwArgs& a, cudaStream_t st) {
+    const size_t smem = 1024 + (size_t)a.slots * FW_SLOT + FW_UNION + sizeof(FwTail);
+    auto go = [&](auto kernel) -> cudaError_t {
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (e != cudaSuccess) return e;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(a.n_cta);
+        cfg.blockDim = dim3(FW_THREADS);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeCooperative;         // the blocks wait on one another: all of them resident, or an error
+        at[0].val.cooperative = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, kernel, a);
+    };
+    const bool few = (a.Hq / a.Hkv) * a.R <= 8;
+    if (a.hd == 128) return few ? go(forward_kernel<128, 8>) : go(forward_kernel<128, 16>);
+    return few ? go(forward_kernel<64, 8>) : go(forward_kernel<64, 16>);
+}
+
+}  // namespace mtad

@@ -70,8 +70,10 @@ cudaError_t launch_seq_set(const SeqState& s, int seq, int kv_len, int root, int
 
 __global__ void prepare_kernel(const __nv_bfloat16* __restrict__ embed, int d, int vocab, int hd, RopeInv rinv,
                                long long kv_capacity, SeqState s, RowMeta rm, float* __restrict__ hidden,
-                               float* __restrict__ rope, PrepareArgs a, uint32_t* status) {
+                               float* __restrict__ rope, PrepareArgs a, uint32_t* status, int32_t* __restrict__ sync,
+                               int sync_words) {
     const int t = blockIdx.x, bi = t / a.R, r = t % a.R;
+    for (int i = t * blockDim.x + threadIdx.x; i < sync_words; i += gridDim.x * blockDim.x) sync[i] = 0;
     const int seq = a.seqs.v[bi];
     const int L = s.kv_len[seq];
     const int N = a.R - 1;
@@ -160,7 +162,7 @@ cudaError_t launch_prepare(const ModelView& m, const SeqState& s, const RowMeta&
     prepare_kernel<<<a.B * a.R, 128, 0, st>>>(static_cast<const __nv_bfloat16*>(m.d.embed), m.d.d_model, m.d.vocab,
                                               m.d.head_dim, rope_inv((double)m.d.rope_base, m.d.head_dim),
                                               (long long)m.d.kv_capacity, s, rm,
-                                              sc.hidden, sc.rope, a, status);
+                                              sc.hidden, sc.rope, a, status, sc.fw_sync, sc.fw_sync_words);
     return cudaGetLastError();
 }
 

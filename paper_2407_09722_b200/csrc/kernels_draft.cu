@@ -55,12 +55,13 @@ __global__ void draft_prepare_kernel(const __nv_bfloat16* __restrict__ embed, in
                                      float* __restrict__ hidden, float* __restrict__ rope, SeqList seqs, int R, int step,
                                      int beam, const __nv_bfloat16* __restrict__ gain0, __nv_bfloat16* x, int terms,
                                      float* sumsq_out, __nv_bfloat16* __restrict__ cache, int layers, int max_batch,
-                                     int Hkv) {
+                                     int Hkv, int32_t* __restrict__ sync, int sync_words) {
     const int t = blockIdx.x, bi = t / R, r = t % R;
     const int seq = seqs.v[bi];
     __shared__ int sh_tok, sh_pos, sh_ok, sh_hole;
     pdl_wait();               // the sequence and draft state, and every buffer written here, belong to earlier kernels
     pdl_trigger();
+    for (int i = t * blockDim.x + threadIdx.x; i < sync_words; i += gridDim.x * blockDim.x) sync[i] = 0;
     if (threadIdx.x == 0) {
         const int L = step == 0 ? s.aux_len[seq] : ds.base_len[seq];
         const int P = step == 0 ? s.aux_npend[seq] : ds.npend[seq];
@@ -161,7 +162,7 @@ cudaError_t launch_draft_prepare(const ModelView& m, const SeqState& s, const Dr
                       tc ? m.w(0, 0) : (const __nv_bfloat16*)nullptr, tc ? sc.xd : (__nv_bfloat16*)nullptr,
                       tc_terms(B * R), sc.sumsq_a,
                       warped ? static_cast<__nv_bfloat16*>(m.d.kv_cache) : (__nv_bfloat16*)nullptr, m.d.layers, m.max_batch,
-                      m.d.n_kv_heads);
+                      m.d.n_kv_heads, sc.fw_sync, sc.fw_sync_words);
 }
 
 // ---------------------------------------------------------------------------------------------------------------

@@ -469,6 +469,19 @@ int tc_make_kv_map(CUtensorMap* out, const void* cache, int hd, long long cap, l
     return r == CUDA_SUCCESS ? 0 : -1;
 }
 
+int tc_make_pair_map(CUtensorMap* out, const void* base, int heads, int hp, int K, int h) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn || h < 1 || h > 256) return -1;
+    const cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)hp, (cuuint64_t)2 * heads};
+    const cuuint64_t strides[2] = {(cuuint64_t)K * 2, (cuuint64_t)hp * K * 2};
+    const cuuint32_t box[3] = {(cuuint32_t)TC_TILE_K, (cuuint32_t)h, 2};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    const CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? 0 : -1;
+}
+
 int tc_boxes(int acc_cols) {
     for (int n = 1; n <= 3; ++n)
         if (acc_cols % n == 0 && acc_cols / n <= 256 && (acc_cols / n) % 16 == 0) return n;

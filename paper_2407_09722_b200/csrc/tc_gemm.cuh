@@ -36,7 +36,7 @@ struct TcGemmParams {
     int n_rows_total;      // weight rows, for skipping a half that lies beyond them
     int n_tiles128;        // ceil(N / 128): row stride of lm_part
     int stages;            // smem ring depth
-    unsigned int wait_limit;     // iterations a bounded wait may poll (0: the default, 2^22)
+    unsigned int wait_limit;     // iterations a bounded wait may poll (0: the default, WAIT_LIMIT)
     int debug_no_operands;       // test hook: the operand-row producer issues no copies, so the waits on them run out
     unsigned long long* trace;   // MTAD_TRACE builds: [CTA][8] global-timer stamps of this launch, else null
     int csize;             // cluster kernel: CTAs that share a tile's k-range (1..8)
@@ -102,6 +102,10 @@ int tc_make_map(CUtensorMap* out, const void* base, long long rows, long long co
 // KV cache [planes][cap][hd] bf16 as a 3-D map (hd, cap, planes) with boxes of 64 elements x 64 positions, 128-byte
 // swizzle (hd = 64 or 128).
 int tc_make_kv_map(CUtensorMap* out, const void* cache, int hd, long long cap, long long planes);
+
+// A [heads * 2 * hp, K] matrix as (K, hp, 2 * heads) with boxes of 64 elements x h rows x both halves of a head: h rotary
+// pairs, first the rows j0 .. j0 + h - 1 of the head's first half, then their partners.
+int tc_make_pair_map(CUtensorMap* out, const void* base, int heads, int hp, int K, int h);
 
 // Fills the decomposition fields of p (and p.terms, p.per_sm for T rows) for a problem of n_tiles x k_blocks on
 // `sms` SMs with per_sm CTAs each (0: tc_ctas_per_sm(T)).
