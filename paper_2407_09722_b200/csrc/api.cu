@@ -19,7 +19,7 @@ using namespace mtad;
 // per tensor-memory accumulator, the pieces being added in fp32 (relative error about 4e-7 instead of 4e-6 at K = 8192)
 static const int kQkvSegCap = 8;
 static const int kCtas = 148;   // SMs the tensor-core GEMM spreads over
-static const bool kOneLaunchForward = false;
+static const bool kOneLaunchForward = true;
 
 // Host-side tensor maps of one model's weight matrices.
 struct WeightMaps {                      // index 0, 1, 2: tiles of 128, 256, 512 rows (1, 2, 4 halves)

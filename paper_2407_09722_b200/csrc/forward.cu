@@ -323,7 +323,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     };
                     if (a_n > 0) ok = scores(0);
                     for (int i = 0; i < a_n && ok; ++i) {
-                        if (i + 1 < a_n) ok = scores(i + 1);
+                        // the next scores go ahead of this tile's output, except across segments: the next segment's query
+                        // rows are loaded once this segment has ended
+                        const bool more = i + 1 < a_n, ahead = more && attn_item(s.pref, a.Hkv, a_lo + i + 1).tile != 0;
+                        if (ahead) ok = scores(i + 1);
                         if (!ok) break;
                         const int vpos = pos + 2 * i + 1, b = (at + i) & 1;
                         const uint32_t par = (uint32_t)((at + i) >> 1) & 1u;
@@ -338,6 +341,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                                    smem_desc(pa + (ks >> 2) * (NQ2 * 128) + (ks & 3) * 32), idesc_o, ks > 0 ? 1u : 0u);
                         tc_commit(smem_u32(&s.ofull[b]));
                         tc_commit(empty_bar(vpos));
+                        if (more && !ahead) ok = scores(i + 1);
                     }
                     if (a_n > 0) ++as;
                     at += a_n;
