@@ -56,7 +56,7 @@ struct mtad_ctx {
     std::map<uint64_t, ForwardPlan> plans;   // by (model, sequences, rows per sequence, LM-head mode)
     WeightMaps tmaps, amaps;
     FwLayer *fw_target = nullptr, *fw_aux = nullptr;   // device tables of the one-launch forward (in the workspace)
-    CUtensorMap fw_lm[2];                              // its LM-head maps: target, auxiliary model
+    CUtensorMap fw_lm[2][FW_CLASSES];                  // its LM-head maps: target, auxiliary model
     bool fw_ok[2] = {false, false};
     bool use_tc = false, use_pdl = false;
     size_t tc_ws_floats = 0, tc_counter_n = 0, xf_elems = 0;
@@ -407,20 +407,25 @@ bool build_forward_table(const ModelView& m, FwLayer* dev, CUtensorMap* lm) {
     fw_geometry(ph, d, kCtas);
     const int qd = d.n_q_heads * d.head_dim, hp = d.head_dim / 2;
     std::vector<FwLayer> tab(d.layers);
-    for (int l = 0; l < d.layers; ++l) {
-        FwLayer& t = tab[l];
-        if (tc_make_pair_map(&t.wq, m.w(l, 1), d.n_q_heads, hp, d.d_model, ph[FW_QKV].h) ||
-            tc_make_pair_map(&t.wk, m.w(l, 2), d.n_kv_heads, hp, d.d_model, ph[FW_QKV].h) ||
-            tc_make_pair_map(&t.wv, m.w(l, 3), d.n_kv_heads, hp, d.d_model, ph[FW_QKV].h) ||
-            tc_make_map(&t.wo, m.w(l, 4), d.d_model, qd, ph[FW_O].h) ||
-            tc_make_map(&t.gate, m.w(l, 6), d.d_ffn, d.d_model, ph[FW_GATEUP].h) ||
-            tc_make_map(&t.up, m.w(l, 7), d.d_ffn, d.d_model, ph[FW_GATEUP].h) ||
-            tc_make_map(&t.down, m.w(l, 8), d.d_model, d.d_ffn, ph[FW_DOWN].h))
-            return false;
-        t.gain_ffn = m.w(l, 5);
-        t.gain_next = l + 1 < d.layers ? m.w(l + 1, 0) : static_cast<const __nv_bfloat16*>(d.final_norm);
+    for (int c = 0; c < FW_CLASSES; ++c) {
+        for (int l = 0; l < d.layers; ++l) {
+            CUtensorMap* w = tab[l].w[c];
+            const FwPhase &q = ph[FW_QKV], &o = ph[FW_O], &g = ph[FW_GATEUP], &dn = ph[FW_DOWN];
+            if (tc_make_pair_map(w, m.w(l, 1), d.n_q_heads, hp, d.d_model, q.h, q.kbc[c]) ||
+                tc_make_pair_map(w + 1, m.w(l, 2), d.n_kv_heads, hp, d.d_model, q.h, q.kbc[c]) ||
+                tc_make_pair_map(w + 2, m.w(l, 3), d.n_kv_heads, hp, d.d_model, q.h, q.kbc[c]) ||
+                tc_make_kb_map(w + 3, m.w(l, 4), d.d_model, qd, o.h, o.kbc[c]) ||
+                tc_make_kb_map(w + 4, m.w(l, 6), d.d_ffn, d.d_model, g.h, g.kbc[c]) ||
+                tc_make_kb_map(w + 5, m.w(l, 7), d.d_ffn, d.d_model, g.h, g.kbc[c]) ||
+                tc_make_kb_map(w + 6, m.w(l, 8), d.d_model, d.d_ffn, dn.h, dn.kbc[c]))
+                return false;
+        }
+        if (tc_make_kb_map(lm + c, d.lm_head, d.vocab, d.d_model, ph[FW_LM].h, ph[FW_LM].kbc[c])) return false;
     }
-    if (tc_make_map(lm, d.lm_head, d.vocab, d.d_model, ph[FW_LM].h)) return false;
+    for (int l = 0; l < d.layers; ++l) {
+        tab[l].gain_ffn = m.w(l, 5);
+        tab[l].gain_next = l + 1 < d.layers ? m.w(l + 1, 0) : static_cast<const __nv_bfloat16*>(d.final_norm);
+    }
     return cudaMemcpy(dev, tab.data(), sizeof(FwLayer) * tab.size(), cudaMemcpyHostToDevice) == cudaSuccess;
 }
 
@@ -432,10 +437,13 @@ bool build_forward_plan(ForwardPlan& fp, const Scratch& sc, const RowMeta& rm, c
     if (!fw_plan(a, d, B, R, kCtas)) return false;
     const int qd = d.n_q_heads * d.head_dim;
     if (with_maps) {
-        if (!m.kv_map_ok || tc_make_map(&a.xd, sc.xd, 2 * TC_X_ROWS, d.d_model, a.cols) ||
-            tc_make_map(&a.xa, sc.xa, 2 * TC_X_ROWS, qd, a.cols) || tc_make_map(&a.xf, sc.xf, 2 * TC_X_ROWS, d.d_ffn, a.cols))
-            return false;
-        a.lm = *lm;
+        if (!m.kv_map_ok) return false;
+        for (int k = 0; k < 6; ++k) {
+            if (k == FW_ATTN) continue;
+            const __nv_bfloat16* x = k == FW_O ? sc.xa : (k == FW_DOWN ? sc.xf : sc.xd);
+            if (tc_make_kb_map(&a.x[k], x, 2 * TC_X_ROWS, a.ph[k].K, a.cols, a.ph[k].kb)) return false;
+        }
+        a.lm = lm[a.cls];
         a.kv = m.kv_map;
     }
     a.layers = table;
@@ -637,7 +645,7 @@ int forward_rows_tc(mtad_ctx* ctx, const ModelView& m, const WeightMaps& wm, int
     if (it == ctx->plans.end()) {
         ForwardPlan fp;
         const bool aux = &m == &ctx->aux;
-        if (!(ctx->fw_ok[aux] && build_forward_plan(fp, sc, ctx->rm, m, aux ? ctx->fw_aux : ctx->fw_target, &ctx->fw_lm[aux], B, R,
+        if (!(ctx->fw_ok[aux] && build_forward_plan(fp, sc, ctx->rm, m, aux ? ctx->fw_aux : ctx->fw_target, ctx->fw_lm[aux], B, R,
                                                     lm_plain, true))) {
             fp = ForwardPlan();
             if (int rc = build_plan(fp, sc, ctx->rm, m, &wm, B, R, lm_plain, true, !aux)) return rc;
@@ -821,8 +829,8 @@ int mtad_create(const mtad_model_desc* target, const mtad_model_desc* aux, int m
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) { delete ctx; return MTAD_E_CUDA; }
     if (ctx->use_tc && kOneLaunchForward) {
-        ctx->fw_ok[0] = ctx->target.kv_map_ok && build_forward_table(ctx->target, ctx->fw_target, &ctx->fw_lm[0]);
-        ctx->fw_ok[1] = aux && ctx->amaps.ok && ctx->aux.kv_map_ok && build_forward_table(ctx->aux, ctx->fw_aux, &ctx->fw_lm[1]);
+        ctx->fw_ok[0] = ctx->target.kv_map_ok && build_forward_table(ctx->target, ctx->fw_target, ctx->fw_lm[0]);
+        ctx->fw_ok[1] = aux && ctx->amaps.ok && ctx->aux.kv_map_ok && build_forward_table(ctx->aux, ctx->fw_aux, ctx->fw_lm[1]);
     }
     *out = ctx;
     return MTAD_OK;

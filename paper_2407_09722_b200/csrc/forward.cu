@@ -7,14 +7,14 @@
 // and a copy ring that starts empty.  Here the weight producer does not know phases: as the last k-blocks of a projection
 // leave the ring, the first ones of the next (or the committed K / V tiles of the attention) take their place, so HBM
 // stays busy across the barrier for as long as the ring is deep.  Two more things keep the boundary short: every block
-// owns whole output features (the features are cut into one or two units per SM, not into 128-row tiles), so no partial
-// sum leaves an SM; and only the call's terms x rows operand rows are multiplied (16 columns for five rows).
+// owns whole output features (the features are cut into one tile per SM, not into 128-row tiles), so no partial sum leaves
+// an SM; and only the call's terms x rows operand rows are multiplied (16 columns for five rows).
 //
 // Contraction.  Weights are the 128-row MMA operand A, the operand rows (two or three bf16 terms per activation, see
-// store_terms) operand B.  Where a block owns at most 32 (64) features, a step brings S = 4 (2) k-blocks, whose weights
-// lie side by side in A and whose operand rows lie side by side in B: of the S x S blocks of the product the diagonal
-// ones are the k-blocks' contributions, summed by the epilogue.  One MMA of 128 x 64 costs what one of 128 x 16 does, so
-// this is S times fewer MMAs (an MMA takes 65 cycles whatever N <= 128 is: 28 rows a step would cap an SM at 27 GB/s).
+// store_terms) operand B.  Where a block owns at most 64 features, the MMA takes S k-blocks at once: their weights lie
+// side by side in A, their operand rows side by side in B, and of the S x S blocks of the product the diagonal ones are
+// the k-blocks' contributions, summed by the epilogue.  One MMA of 128 x 64 costs what one of 128 x 16 does, so this is S
+// times fewer MMAs (an MMA takes 65 cycles whatever N <= 128 is: 32 rows at a time would cap an SM at 30 GB/s).
 //
 // Attention: keys as the M dimension.  The (sequence, KV head, 128-key tile) items are dealt out evenly, in order.
 //   S^T = K Q^T   A = K tile as it lies in the cache, B = query rows (bf16 hi rows, then lo rows)
@@ -42,7 +42,8 @@ constexpr int FW_THREADS = 32 * 12;
 constexpr int FW_EPI_WARP0 = 4;
 constexpr int FW_EPI = 256;
 constexpr int FW_UNION = 32 * 1024;       // epilogue tile Y, or the attention's query and probability tiles
-constexpr int FW_MAX_SLOTS = 6;
+constexpr int NS = FW_SLOTS;
+constexpr int FW_ACC = 240;               // accumulator columns of a tile, of 256 (the drain reads up to 15 columns further)
 constexpr int FW_TM_D = 128;              // attention: tensor-memory columns 0 / 64 scores, 128 / 192 outputs
 
 struct FwTail {
@@ -52,7 +53,7 @@ struct FwTail {
     float sl[2][4][16];                   // row sums of the softmax warps
     float sm[2][16];                      // row reference values
     int pref[MTAD_MAX_BATCH + 1];         // flattened attention tiles before sequence b
-    uint64_t full[FW_MAX_SLOTS], empty[FW_MAX_SLOTS];
+    uint64_t full[NS], empty[NS];
     uint64_t tfull[2], tempty[2], sfull[2], pfull[2], ofull[2], oempty[2], qfull[2];
     uint32_t tmem_ptr;
     int abort_flag[2];
@@ -83,6 +84,14 @@ __device__ __forceinline__ bool all_of(int id, int n, bool ok) {
 }
 __device__ __forceinline__ void bar_n(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z, int u,
+                                            uint64_t hint) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+        " [%0], [%1, {%3, %4, %5, %6}], [%2], %7;" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(u), "l"(hint)
+        : "memory");
+}
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z,
                                             uint64_t hint) {
     asm volatile(
@@ -121,7 +130,7 @@ __device__ __forceinline__ AttnItem attn_item(const int* pref, int Hkv, int x) {
     return it;
 }
 
-static_assert(1024 + FW_MAX_SLOTS * FW_SLOT + FW_UNION + sizeof(FwTail) <= 227 * 1024, "shared memory of the forward");
+static_assert(1024 + NS * FW_SLOT + FW_UNION + sizeof(FwTail) <= 227 * 1024, "shared memory of the forward");
 
 template <int HD, int NQP>
 __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_constant__ FwArgs a) {
@@ -132,7 +141,6 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     constexpr int P_BYTES = NQ2 * FW_KEYS * 2;         // one probability tile
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    const int NS = a.slots;
     uint8_t* uni = smem + (size_t)NS * FW_SLOT;
     FwTail& s = *reinterpret_cast<FwTail*>(uni + FW_UNION);
     float* Y = reinterpret_cast<float*>(uni);
@@ -224,40 +232,42 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     continue;
                 }
                 if (kind == FW_QKV && layer + 1 < a.n_layers) {
-                    const CUtensorMap* nm = &L[1].wq;
+                    const CUtensorMap* nm = L[1].w[a.cls];
 #pragma unroll
                     for (int i = 0; i < 7; ++i)
                         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(nm + i)) : "memory");
                 }
                 const FwPhase& f = a.ph[kind];
-                const int nsub = f.S * f.kp;
-                const uint32_t sub_stride = f.S > 1 ? (uint32_t)(TC_TILE_N / f.S) * 128u : (uint32_t)f.a_bytes;
+                const CUtensorMap* w = L->w[a.cls];
+                const uint32_t bytes = (uint32_t)(f.nbox * f.box_bytes + f.kb * cols * 128);
                 for (int tile = cta; tile < f.n_tiles && ok; tile += n_cta) {
-                    const int unit0 = tile * f.upt, nu = min(f.upt, f.n_units - unit0);
-                    const uint32_t bytes = (uint32_t)(nsub * (nu * f.box_bytes + cols * 128));
+                    // the tile's first box: map, row coordinate (QKV: pair and half-head coordinates)
+                    const CUtensorMap* m = w;
+                    int row = tile * f.nbox * f.h, half = 0;
+                    if (kind == FW_QKV) {
+                        const int hg = tile / f.u;
+                        row = (tile - hg * f.u) * f.h;
+                        half = 2 * (hg < a.Hq ? hg : (hg < a.Hq + a.Hkv ? hg - a.Hq : hg - a.Hq - a.Hkv));
+                        m = w + (hg < a.Hq ? 0 : (hg < a.Hq + a.Hkv ? 1 : 2));
+                    } else if (kind == FW_GATEUP) {
+                        m = w + 4;
+                        row = tile * f.h;
+                    } else {
+                        m = kind == FW_O ? w + 3 : (kind == FW_DOWN ? w + 6 : &a.lm);
+                    }
                     for (int step = 0; step < f.steps; ++step, ++pos) {
                         ok = mbar_wait(empty_bar(pos), ring_par(pos) ^ 1u, abort_flag);
                         if (!ok) break;
                         const uint32_t bar = full_bar(pos), base = slot_ptr(pos);
+                        const int kx = f.flat ? step * TC_TILE_K : 0, kz = f.flat ? 0 : step * f.kb;
                         mbar_expect_tx(bar, bytes);
-                        for (int sb = 0; sb < nsub; ++sb) {
-                            const int kx = (step * nsub + sb) * TC_TILE_K;
-                            uint32_t dst = base + sb * sub_stride;
-                            for (int uu = 0; uu < nu; ++uu, dst += f.slots * 128) {
-                                const int unit = unit0 + uu;
-                                if (kind == FW_QKV) {
-                                    const int hg = unit / f.u, j0 = (unit - hg * f.u) * f.h;
-                                    const CUtensorMap* m = hg < a.Hq ? &L->wq : (hg < a.Hq + a.Hkv ? &L->wk : &L->wv);
-                                    const int hl = hg < a.Hq ? hg : (hg < a.Hq + a.Hkv ? hg - a.Hq : hg - a.Hq - a.Hkv);
-                                    tma_load_3d(dst, m, bar, kx, j0, 2 * hl, HINT_STREAM);
-                                } else if (kind == FW_GATEUP) {
-                                    tma_load_2d(dst, &L->gate, bar, kx, unit * f.h, HINT_STREAM);
-                                    tma_load_2d(dst + (f.slots >> 1) * 128, &L->up, bar, kx, unit * f.h, HINT_STREAM);
-                                } else {
-                                    const CUtensorMap* m = kind == FW_O ? &L->wo : (kind == FW_DOWN ? &L->down : &a.lm);
-                                    tma_load_2d(dst, m, bar, kx, unit * f.h, HINT_STREAM);
-                                }
-                            }
+                        if (kind == FW_QKV) {
+                            tma_load_4d(base, m, bar, kx, row, half, kz, HINT_STREAM);
+                        } else {
+                            tma_load_3d(base, m, bar, kx, row, kz, HINT_STREAM);
+                            if (f.nbox == 2)
+                                tma_load_3d(base + f.box_bytes, kind == FW_GATEUP ? m + 1 : m, bar, kx,
+                                            kind == FW_GATEUP ? row : row + f.h, kz, HINT_STREAM);
                         }
                     }
                 }
@@ -275,8 +285,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 const int kind = kind_of(p);
                 if (kind == FW_ATTN) { pos += 2 * a_n; continue; }
                 const FwPhase& f = a.ph[kind];
-                const int nsub = f.S * f.kp;
-                const CUtensorMap* m = kind == FW_O ? &a.xa : (kind == FW_DOWN ? &a.xf : &a.xd);
+                const CUtensorMap* m = &a.x[kind];
                 if (p > 0) {
                     ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
                     proxy_fence();
@@ -287,8 +296,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         if (!ok) break;
                         const uint32_t bar = full_bar(pos), base = slot_ptr(pos) + f.b_off;
                         if (!a.debug_no_operands)
-                            for (int sb = 0; sb < nsub; ++sb)
-                                tma_load_2d(base + sb * cols * 128, m, bar, (step * nsub + sb) * TC_TILE_K, 0, HINT_KEEP);
+                            tma_load_3d(base, m, bar, f.flat ? step * TC_TILE_K : 0, 0, f.flat ? 0 : step * f.kb, HINT_KEEP);
                     }
             }
         }
@@ -349,7 +357,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     continue;
                 }
                 const FwPhase& f = a.ph[kind];
-                const int mh = (f.rows + TC_TILE_N - 1) / TC_TILE_N;
+                const int groups = f.kb / f.S, sc = f.S * cols;      // MMAs along k, accumulator columns of a box
                 const uint32_t idesc = IDESC | ((uint32_t)((f.S * cols) >> 3) << 17);
                 for (int tile = cta; tile < f.n_tiles && ok; tile += n_cta, ++tcount) {
                     const int buf = tcount & 1;
@@ -362,12 +370,12 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         if (!ok) break;
                         tc_fence_after();
                         const uint32_t base = slot_ptr(pos), bb = base + f.b_off;
-                        for (int sb = 0; sb < f.kp; ++sb)
-                            for (int m = 0; m < mh; ++m)
+                        for (int gr = 0; gr < groups; ++gr)
+                            for (int q = 0; q < f.nbox; ++q)
 #pragma unroll
                                 for (int k4 = 0; k4 < TC_TILE_K / 16; ++k4)
-                                    tc_mma(d + m * cols, smem_desc(base + sb * f.a_bytes + m * (TC_TILE_N * 128) + k4 * 32),
-                                           smem_desc(bb + sb * cols * 128 + k4 * 32), idesc, (step > 0 || sb > 0 || k4 > 0) ? 1u : 0u);
+                                    tc_mma(d + q * sc, smem_desc(base + q * f.box_bytes + gr * f.S * f.hr * 128 + k4 * 32),
+                                           smem_desc(bb + gr * sc * 128 + k4 * 32), idesc, (step > 0 || gr > 0 || k4 > 0) ? 1u : 0u);
                         tc_commit(empty_bar(pos));
                     }
                     if (ok) tc_commit(smem_u32(&s.tfull[buf]));
@@ -590,8 +598,11 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 const FwPhase& f = a.ph[kind];
                 const FwLayer* L = a.layers + layer;
                 const int mine = cta < f.n_tiles ? (f.n_tiles - 1 - cta) / n_cta + 1 : 0;
-                const int ys = (f.S > 1 ? TC_TILE_N : f.rows) + 4;     // row stride of Y
-                const int nf = f.upt * f.h;                            // features (pairs) of a tile
+                const int yb = f.S * f.hr;                             // columns of Y that a box takes
+                const int ys = f.nbox * yb + 4;                        // row stride of Y
+                const int nf = kind == FW_LM ? f.nbox * f.h : f.h;     // features (pairs) of a tile
+                // rows that Y holds at a time, in whole drain groups
+                const int per = terms == 3 ? 5 : 8, blk = min((T + per - 1) / per, FW_UNION / (per * ys * 4)) * per;
                 if (mine > 0 && (kind == FW_QKV || kind == FW_GATEUP || kind == FW_LM)) {
                     // scale of the deferred RMSNorm: the rows' sums of squares come from every block
                     if (p > 0) {
@@ -611,7 +622,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 }
                 pos += mine * f.steps;
                 for (int tile = cta; tile < f.n_tiles; tile += n_cta, ++tcount) {
-                    const int buf = tcount & 1, unit0 = tile * f.upt;
+                    const int buf = tcount & 1, f0 = tile * nf;            // first feature (O, down, gate / up, LM head)
                     // what the first items of this thread need besides the accumulator, requested ahead of it
                     float pre[4] = {0.f, 0.f, 0.f, 0.f};
                     float u8[8];
@@ -620,67 +631,73 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     if (kind == FW_O || kind == FW_DOWN) {
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            const int n = unit0 * f.h + lane + 32 * i;
+                            const int n = f0 + lane + 32 * i;
                             if (w < T && lane + 32 * i < nf && n < a.d) pre[i] = __ldcg(a.hidden + (size_t)w * a.d + n);
                         }
                     } else if (kind == FW_LM && !a.lm_plain) {
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
-                            const int n = unit0 * f.h + lane + 32 * i;
+                            const int n = f0 + lane + 32 * i;
                             if (w < T && lane + 32 * i < nf && n < a.V) u8[i] = a.uniforms[(size_t)(w / a.R) * a.V + n];
                         }
                     }
                     ok = mbar_wait(smem_u32(&s.tfull[buf]), (uint32_t)(tcount >> 1) & 1u, abort_flag);
                     __syncwarp();
                     tc_fence_after();
-                    {   // accumulators -> Y[row][slot], the terms of a row added up
+                    for (int r0 = 0; r0 < T; r0 += blk) {
+                    const int r1 = min(T, r0 + blk);
+                    {   // accumulators -> Y[row][box][lane], the terms of a row added up; a lane's slice of the S k-blocks that
+                        // the MMA takes side by side is lane / hr, and a warp's 32 lanes may lie in several slices
                         const uint32_t t_acc = t_lane + buf * 256;
-                        const int mh = f.S > 1 ? 1 : (f.rows + TC_TILE_N - 1) / TC_TILE_N;
-                        const int slice = f.S == 4 ? quad : (f.S == 2 ? quad >> 1 : 0);
-                        const int per = terms == 3 ? 5 : 8, ng = (T + per - 1) / per;
-                        for (int i = half; i < mh * ng; i += 2) {
-                            const int mm = i / ng, rb = (i - mm * ng) * per, slot = mm * TC_TILE_N + quad * 32 + lane;
-                            float v[16];
-                            tc_ld16(t_acc + (mm + slice) * cols + rb * terms, v);
-                            if (slot < ys - 4) {
-                                if (terms == 3) {
+                        const int ng = (r1 - r0 + per - 1) / per, tl = quad * 32 + lane, my = tl / f.hr;
+                        const int s0 = f.S > 1 ? quad * 32 / f.hr : 0, s1 = f.S > 1 ? min(f.S - 1, (quad * 32 + 31) / f.hr) : 0;
+                        for (int i = half; i < f.nbox * ng; i += 2) {
+                            const int q = i / ng, rb = r0 + (i - q * ng) * per;
+                            for (int sl = s0; sl <= s1; ++sl) {
+                                float v[16];
+                                tc_ld16(t_acc + (q * f.S + sl) * cols + rb * terms, v);
+                                if (my == sl && tl < yb) {
+                                    float* y = Y + (rb - r0) * ys + q * yb + tl;
+                                    if (terms == 3) {
 #pragma unroll
-                                    for (int j = 0; j < 5; ++j)
-                                        if (rb + j < T) Y[(rb + j) * ys + slot] = v[3 * j] + (v[3 * j + 1] + v[3 * j + 2]);
-                                } else {
+                                        for (int j = 0; j < 5; ++j)
+                                            if (rb + j < r1) y[j * ys] = v[3 * j] + (v[3 * j + 1] + v[3 * j + 2]);
+                                    } else {
 #pragma unroll
-                                    for (int j = 0; j < 8; ++j)
-                                        if (rb + j < T) Y[(rb + j) * ys + slot] = v[2 * j] + v[2 * j + 1];
+                                        for (int j = 0; j < 8; ++j)
+                                            if (rb + j < r1) y[j * ys] = v[2 * j] + v[2 * j + 1];
+                                    }
                                 }
+                                __syncwarp();
                             }
                         }
                     }
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&s.tempty[buf]));
+                    if (r1 == T) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&s.tempty[buf]));
+                    }
                     ok = all_of(1, FW_EPI, ok);
                     if (!ok) break;
-                    // value of (row, slot): the S slices of the step lie side by side
-                    const int sst = TC_TILE_N / f.S;
-                    auto yv = [&](int t, int slot) -> float {
-                        const float* y = Y + t * ys + slot;
+                    // value of (row, box, weight row): the S slices lie side by side
+                    auto yv = [&](int t, int q, int row) -> float {
+                        const float* y = Y + (t - r0) * ys + q * yb + row;
                         float v = y[0];
-                        if (f.S == 4) v = (v + y[sst]) + (y[2 * sst] + y[3 * sst]);
-                        else if (f.S == 2) v += y[sst];
+                        for (int sl = 1; sl < f.S; ++sl) v += y[sl * f.hr];
                         return v;
                     };
+                    const int nr = r1 - r0;
                     if (kind == FW_QKV) {
                         const int hp = HD / 2;
                         const float scale = rsqrtf((float)HD);
-                        for (int i = e; i < T * nf; i += FW_EPI) {
-                            const int t = i / nf, jl = i - t * nf, uu = jl / f.h, j = jl - uu * f.h, unit = unit0 + uu;
-                            if (unit >= f.n_units) continue;
-                            const int hg = unit / f.u, jj = (unit - hg * f.u) * f.h + j;
+                        const int hg = tile / f.u, j0 = (tile - hg * f.u) * f.h;
+                        for (int i = e; i < nr * nf; i += FW_EPI) {
+                            const int t = r0 + i / nf, j = i % nf, jj = j0 + j;
                             if (jj >= hp) continue;
                             const int sl = a.rm.slot[t];
                             const float2 cs = *reinterpret_cast<const float2*>(a.rope + ((size_t)t * hp + jj) * 2);
                             const float rs = s.rstd[t];
-                            const float va = yv(t, uu * f.slots + j) * rs, vb = yv(t, uu * f.slots + f.h + j) * rs;
+                            const float va = yv(t, 0, j) * rs, vb = yv(t, 0, f.h + j) * rs;
                             if (sl < 0) continue;                         // inactive row: no query, no cache slot
                             const float ra = va * cs.x - vb * cs.y, rb = vb * cs.x + va * cs.y;
                             if (hg < a.Hq) {
@@ -697,35 +714,35 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             }
                         }
                     } else if (kind == FW_GATEUP) {
-                        for (int i = e; i < T * nf; i += FW_EPI) {
-                            const int t = i / nf, jl = i - t * nf, uu = jl / f.h, j = jl - uu * f.h, n = (unit0 + uu) * f.h + j;
+                        for (int i = e; i < nr * nf; i += FW_EPI) {
+                            const int t = r0 + i / nf, j = i % nf, n = f0 + j;
                             if (n >= a.F) continue;
                             const float rs = s.rstd[t];
-                            const float g = yv(t, uu * f.slots + j) * rs, up = yv(t, uu * f.slots + (f.slots >> 1) + j) * rs;
+                            const float g = yv(t, 0, j) * rs, up = yv(t, 1, j) * rs;
                             store_terms(g / (1.f + expf(-g)) * up, a.x_f + (size_t)t * terms * a.F + n, a.F, terms);
                         }
                     } else if (kind == FW_LM && a.lm_plain) {
-                        for (int i = e; i < T * nf; i += FW_EPI) {
-                            const int t = i / nf, jl = i - t * nf, uu = jl / f.h, n = unit0 * f.h + jl;
-                            if (n < a.V) a.logits[(size_t)t * a.V + n] = yv(t, uu * f.slots + jl - uu * f.h) * s.rstd[t];
+                        for (int i = e; i < nr * nf; i += FW_EPI) {
+                            const int t = r0 + i / nf, jl = i % nf, q = jl / f.h, n = f0 + jl;
+                            if (n < a.V) a.logits[(size_t)t * a.V + n] = yv(t, q, jl - q * f.h) * s.rstd[t];
                         }
                     } else if (kind == FW_LM) {
                         // a warp per row: maximum, sum of exponentials, arg-max of the perturbed logits over the tile
-                        for (int t = w; t < T; t += 8) {
+                        for (int t = r0 + w; t < r1; t += 8) {
                             float z[8], m = -CUDART_INF_F, bv = -CUDART_INF_F, sum = 0.f;
                             int bi = 0x7fffffff;
                             const float rs = s.rstd[t];
                             if (t != w)
 #pragma unroll
                                 for (int i = 0; i < 8; ++i) {
-                                    const int n = unit0 * f.h + lane + 32 * i;
+                                    const int n = f0 + lane + 32 * i;
                                     u8[i] = (lane + 32 * i < nf && n < a.V) ? a.uniforms[(size_t)(t / a.R) * a.V + n] : 0.5f;
                                 }
 #pragma unroll
                             for (int i = 0; i < 8; ++i) {
-                                const int jl = lane + 32 * i, n = unit0 * f.h + jl, uu = jl / f.h;
+                                const int jl = lane + 32 * i, n = f0 + jl, q = jl >= f.h ? 1 : 0;
                                 const bool in = jl < nf && n < a.V;
-                                z[i] = in ? yv(t, uu * f.slots + jl - uu * f.h) * rs : -CUDART_INF_F;
+                                z[i] = in ? yv(t, q, jl - q * f.h) * rs : -CUDART_INF_F;
                                 m = fmaxf(m, z[i]);
                                 const float pz = in ? z[i] - logf(-logf(u8[i])) : -CUDART_INF_F;
                                 if (in && (pz > bv || (pz == bv && n < bi))) { bv = pz; bi = n; }
@@ -746,22 +763,22 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         // logit of each node's token under its parent row, where it falls into this tile
                         for (int t = e; t < T; t += FW_EPI) {
                             const int pr = a.rm.prow[t];
-                            if (pr < 0 || pr >= T) continue;
-                            const int tk = a.rm.tok[t] - unit0 * f.h, uu = tk / f.h;
-                            if (tk >= 0 && tk < nf) a.node_z[t] = yv(pr, uu * f.slots + tk - uu * f.h) * s.rstd[pr];
+                            if (pr < r0 || pr >= r1) continue;
+                            const int tk = a.rm.tok[t] - f0, q = tk >= f.h ? 1 : 0;
+                            if (tk >= 0 && tk < nf) a.node_z[t] = yv(pr, q, tk - q * f.h) * s.rstd[pr];
                         }
                     } else {
                         // residual: a warp per row; emits the next operand rows and the row's share of its sum of squares
                         const __nv_bfloat16* gain = kind == FW_O ? L->gain_ffn : L->gain_next;
                         float* sq = kind == FW_O ? a.sumsq_b : a.sumsq_a;
-                        for (int t = w; t < T; t += 8) {
+                        for (int t = r0 + w; t < r1; t += 8) {
                             float ss = 0.f;
 #pragma unroll
                             for (int i = 0; i < 4; ++i) {
-                                const int jl = lane + 32 * i, uu = jl / f.h, n = unit0 * f.h + jl;
+                                const int jl = lane + 32 * i, n = f0 + jl;
                                 if (jl >= nf || n >= a.d) continue;
                                 float* hp = a.hidden + (size_t)t * a.d + n;
-                                const float y = yv(t, uu * f.slots + jl - uu * f.h) + (t == w ? pre[i] : __ldcg(hp));
+                                const float y = yv(t, 0, jl) + (t == w ? pre[i] : __ldcg(hp));
                                 *hp = y;
                                 store_terms(y * __bfloat162float(gain[n]), a.x_d + (size_t)t * terms * a.d + n, a.d, terms);
                                 ss += y * y;
@@ -771,7 +788,9 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             if (lane == 0) sq[(size_t)tile * TC_X_ROWS + t] = ss;
                         }
                     }
-                    if (tile + n_cta < f.n_tiles) bar_n(1, FW_EPI);       // Y is rewritten by the next tile
+                    if (r1 < T || tile + n_cta < f.n_tiles) bar_n(1, FW_EPI);       // Y is rewritten by the next rows or tile
+                    }
+                    if (!ok) break;
                 }
                 if (!ok) break;
             }
@@ -802,80 +821,72 @@ int up8(int x) { return (x + 7) / 8 * 8; }
 }  // namespace
 
 void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta) {
-    auto rows = [&](FwPhase& f, int N, int per_cta) {
-        f.h = std::min(128, std::max(8, up_div(N, n_cta * per_cta)));
-        f.slots = up8(f.h);
-        f.n_units = up_div(N, f.h);
+    const int qd = d.n_q_heads * d.head_dim, hp = d.head_dim / 2, heads = d.n_q_heads + 2 * d.n_kv_heads;
+    // rows of a matrix: one tile per SM, in whole groups of eight rows (swizzle atoms)
+    auto rows = [&](FwPhase& f, int N, int nbox, int cut) {
+        f.nbox = nbox;
+        f.h = f.hr = std::min(128, std::max(8, up8(up_div(N, n_cta * cut))));
+        f.n_tiles = up_div(N, f.h * cut);
         f.u = 1;
-        f.box_bytes = f.h * 128;
     };
-    const int qd = d.n_q_heads * d.head_dim;
-    rows(ph[FW_O], d.d_model, 1);
-    rows(ph[FW_DOWN], d.d_model, 1);
-    rows(ph[FW_LM], d.vocab, 2);
-    rows(ph[FW_GATEUP], d.d_ffn, 2);
-    ph[FW_O].k_blocks = up_div(qd, TC_TILE_K);
-    ph[FW_DOWN].k_blocks = up_div(d.d_ffn, TC_TILE_K);
-    ph[FW_LM].k_blocks = ph[FW_GATEUP].k_blocks = ph[FW_QKV].k_blocks = up_div(d.d_model, TC_TILE_K);
-    ph[FW_GATEUP].slots *= 2;
-    ph[FW_GATEUP].box_bytes *= 2;
-    // QKV: a head's rotary pairs in u units of h; the cut whose busiest block streams the fewest rows
-    const int hp = d.head_dim / 2, heads = d.n_q_heads + 2 * d.n_kv_heads;
+    rows(ph[FW_O], d.d_model, 1, 1);
+    rows(ph[FW_DOWN], d.d_model, 1, 1);
+    rows(ph[FW_GATEUP], d.d_ffn, 2, 1);
+    const int lm_boxes = up_div(d.vocab, n_cta) > 64 ? 2 : 1;
+    rows(ph[FW_LM], d.vocab, lm_boxes, lm_boxes);
+    // QKV: the rotary pairs of a head in u tiles, as many as the SMs allow
     FwPhase& q = ph[FW_QKV];
-    long long best = -1;
-    for (int h = std::min(hp, 8); h <= hp; ++h) {
-        const int u = up_div(hp, h), upt = up_div(heads * u, n_cta);
-        const long long rows_max = (long long)upt * 2 * h;
-        if (upt * up8(2 * h) > 256 && upt > 1) continue;
-        const long long cost = rows_max * 64 + upt;            // fewer boxes among equals
-        if (best < 0 || cost < best) { best = cost; q.h = h; q.u = u; }
+    q.u = std::max(1, std::min(n_cta / heads, hp / 4));
+    q.h = up_div(up_div(hp, q.u), 4) * 4;
+    q.u = up_div(hp, q.h);
+    q.hr = 2 * q.h;
+    q.nbox = 1;
+    q.n_tiles = heads * q.u;
+    ph[FW_O].K = qd;
+    ph[FW_DOWN].K = d.d_ffn;
+    ph[FW_LM].K = ph[FW_GATEUP].K = q.K = d.d_model;
+    static const int class_cols[FW_CLASSES] = {16, 32, 64, FW_MAX_COLS};
+    for (int k = 0; k < 6; ++k) {
+        if (k == FW_ATTN) continue;
+        FwPhase& f = ph[k];
+        f.k_blocks = up_div(f.K, TC_TILE_K);
+        for (int c = 0; c < FW_CLASSES; ++c) {
+            int kb = FW_SLOT / ((f.nbox * f.hr + class_cols[c]) * 128);
+            kb = std::min(std::min(kb, f.k_blocks), 16);
+            // a multiple of the k-blocks that the MMA can take side by side
+            const int S = std::min(TC_TILE_N / f.hr, FW_ACC / (class_cols[c] * f.nbox));
+            if (S > 1 && kb > S) kb -= kb % S;
+            f.kbc[c] = (f.K % TC_TILE_K || kb < 1) ? 1 : kb;
+        }
     }
-    if (best < 0) { q.h = hp; q.u = 1; }
-    q.n_units = heads * q.u;
-    q.slots = up8(2 * q.h);
-    q.box_bytes = 2 * q.h * 128;
 }
 
 bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
     const int T = B * R, G = d.n_q_heads / d.n_kv_heads;
     if (d.head_dim != 64 && d.head_dim != 128) return false;
-    if (T > FW_MAX_ROWS || G * R > FW_MAX_QROWS || B > MTAD_MAX_BATCH) return false;
+    if (T > 64 || G * R > FW_MAX_QROWS || B > MTAD_MAX_BATCH) return false;
     if (d.d_model >= 8192 && T > 32) return false;          // the accurate K / V projection has launches of its own
     fw_geometry(a.ph, d, n_cta);
     a.T = T; a.B = B; a.R = R; a.terms = tc_terms(T);
     a.cols = (a.terms * T + 15) / 16 * 16;
+    if (a.cols > FW_MAX_COLS) return false;
+    a.cls = a.cols <= 16 ? 0 : (a.cols <= 32 ? 1 : (a.cols <= 64 ? 2 : 3));
     a.n_cta = n_cta; a.n_layers = d.layers;
     a.d = d.d_model; a.F = d.d_ffn; a.V = d.vocab; a.Hq = d.n_q_heads; a.Hkv = d.n_kv_heads; a.hd = d.head_dim;
-    a.slots = FW_MAX_SLOTS;
-    const int bb = a.cols * 128;                            // operand rows of one k-block
     for (int k = 0; k < 6; ++k) {
         if (k == FW_ATTN) continue;
         FwPhase& f = a.ph[k];
-        bool found = false;
-        for (f.upt = up_div(f.n_units, n_cta); f.upt >= 1; --f.upt) {
-            f.rows = f.upt * f.slots;
-            const int mh = up_div(f.rows, TC_TILE_N);
-            if (f.rows > 256 || mh * a.cols > 256) continue;
-            f.S = 1; f.kp = 1; f.a_bytes = f.rows * 128;
-            if (f.rows <= 32 && 4 * bb <= 16384 && f.k_blocks >= 4) f.S = 4;
-            else if (f.rows <= 64 && 2 * bb <= 16384 && f.k_blocks >= 2) f.S = 2;
-            if (f.S > 1) {
-                f.b_off = TC_TILE_N * 128;
-            } else {
-                if (f.a_bytes + bb > FW_SLOT) continue;
-                f.kp = std::min(std::min(4, FW_SLOT / (f.a_bytes + bb)), f.k_blocks);
-                f.b_off = f.kp * f.a_bytes;
-            }
-            // the epilogue tile must fit its area
-            if ((size_t)T * ((f.S > 1 ? TC_TILE_N : f.rows) + 4) * 4 > FW_UNION) continue;
-            found = true;
-            break;
-        }
-        if (!found) return false;
-        f.n_tiles = up_div(f.n_units, f.upt);
-        f.steps = up_div(f.k_blocks, f.S * f.kp);
-        if ((k == FW_O || k == FW_DOWN) && (f.upt * f.h > 128 || f.n_tiles > n_cta)) return false;
-        if (k == FW_LM && f.upt * f.h > 256) return false;
+        f.kb = f.kbc[a.cls];
+        f.flat = tc_kb_flat(f.K, f.kb) ? 1 : 0;
+        f.S = 1;
+        for (int S = 2; S <= f.kb; ++S)
+            if (f.kb % S == 0 && S * f.hr <= TC_TILE_N && S * a.cols * f.nbox <= FW_ACC) f.S = S;
+        f.steps = up_div(f.k_blocks, f.kb);
+        f.box_bytes = f.hr * 128 * f.kb;
+        f.b_off = f.nbox * f.box_bytes;
+        if (f.b_off + f.kb * a.cols * 128 > FW_SLOT || f.nbox * f.S * a.cols > FW_ACC) return false;
+        if ((k == FW_O || k == FW_DOWN) && f.n_tiles > n_cta) return false;
+        if (FW_UNION / (8 * (f.nbox * f.S * f.hr + 4) * 4) < 1) return false;
     }
     return true;
 }
@@ -883,11 +894,11 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
 size_t fw_parts_max(const mtad_model_desc& d, int n_cta, bool lm) {
     FwPhase ph[6];
     fw_geometry(ph, d, n_cta);
-    return (size_t)ph[lm ? FW_LM : FW_O].n_units;
+    return (size_t)ph[lm ? FW_LM : FW_O].n_tiles;
 }
 
 cudaError_t launch_forward(const FwArgs& a, cudaStream_t st) {
-    const size_t smem = 1024 + (size_t)a.slots * FW_SLOT + FW_UNION + sizeof(FwTail);
+    const size_t smem = 1024 + (size_t)NS * FW_SLOT + FW_UNION + sizeof(FwTail);
     auto go = [&](auto kernel) -> cudaError_t {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e != cudaSuccess) return e;

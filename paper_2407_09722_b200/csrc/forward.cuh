@@ -5,36 +5,39 @@
 
 namespace mtad {
 
-constexpr int FW_SLOT = 32 * 1024;        // bytes of one ring slot: one step of a projection, or 128 keys of K or V
+constexpr int FW_SLOT = 48 * 1024;        // bytes of one ring slot: one step of a projection, or 128 keys of K or V
+constexpr int FW_SLOTS = 4;
 constexpr int FW_KEYS = 128;              // keys of an attention tile
-constexpr int FW_MAX_ROWS = 60;           // rows of a call
+constexpr int FW_MAX_COLS = 112;          // operand rows (terms x rows) of a call
 constexpr int FW_MAX_QROWS = 16;          // query rows of one KV head and sequence
 
-// Tile geometry of one projection.  A unit is what one box (two for gate / up) of the weight map brings: h feature rows
-// (QKV: h rotary pairs of a head; gate / up: h gate rows and the h matching up rows), in `slots` rows of shared memory.
-// h depends on the matrix and the SM count alone, so the weight maps are encoded once per model; how many units make a
-// tile, how many k-blocks a step and whether the step's k-blocks lie side by side in the MMA's M dimension (S > 1)
-// depends on the call's row count.
+// Tile geometry of one projection.  A step brings nbox boxes of hr weight rows x kb k-blocks (one copy each) and one box of
+// operand rows.  nbox = 1: the rows of h features (QKV: of h rotary pairs of a head, hr = 2 h); nbox = 2: h gate rows and
+// the h matching up rows, or 2 h rows of the LM head.  h depends on the matrix and the SM count alone; kb is the most that
+// a ring slot holds for the call's operand rows, in FW_CLASSES steps, so that the weight maps are encoded once per model.
+// Big boxes matter twice: a thread issues a copy about every quarter of a microsecond whatever its size, and rows of 256
+// bytes and more pass at 70 GB/s per SM where rows of 128 bytes pass at 43.
+constexpr int FW_CLASSES = 4;             // operand rows up to 16, 32, 64, 112
 struct FwPhase {
-    int h, slots, n_units, u;             // u: units per head (QKV)
-    int upt, n_tiles, rows;               // units per tile, tiles, shared-memory rows of a tile's weights
-    int S, kp, steps;                     // k-blocks side by side, k-blocks one after the other in a step, steps of a tile
-    int a_bytes, b_off;                   // weights of one k-block, offset of the operand rows in the slot
-    int box_bytes;                        // bytes that one unit brings per k-block
-    int k_blocks;
+    int h, hr, nbox, n_tiles, u;          // u: tiles per head (QKV)
+    int kbc[FW_CLASSES];                  // kb by class
+    int kb, flat, S, steps;               // k-blocks of a box, its map's view, k-blocks side by side in the MMA, steps of a tile
+    int box_bytes, b_off;                 // bytes of one weight box, offset of the operand rows in the slot
+    int k_blocks, K;
 };
 enum { FW_QKV = 0, FW_ATTN = 1, FW_O = 2, FW_GATEUP = 3, FW_DOWN = 4, FW_LM = 5 };
 
 struct alignas(64) FwLayer {              // device table, one entry per layer
-    CUtensorMap wq, wk, wv, wo, gate, up, down;
+    CUtensorMap w[FW_CLASSES][7];         // wq, wk, wv, wo, gate, up, down
     const __nv_bfloat16 *gain_ffn, *gain_next;
 };
 
 struct FwArgs {
-    CUtensorMap xd, xa, xf, lm, kv;
+    CUtensorMap x[6], lm, kv;             // operand rows by kind
+    int cls;
     FwPhase ph[6];                        // by kind; the entry of the attention is unused
     const FwLayer* layers;
-    int n_layers, n_cta, slots;           // slots: ring depth
+    int n_layers, n_cta;
     int T, terms, cols, B, R, d, F, V, Hq, Hkv, hd, max_batch, lm_plain;
     int pieces;                           // stride of the attention partials: pieces per (row, head)
     int parts0;                           // statistics of the prepared rows: parts of sumsq_a
@@ -54,9 +57,9 @@ struct FwArgs {
     int debug_no_operands;
 };
 
-// Host side.  fw_geometry fills h, slots, n_units, u of every projection; fw_plan the rest for a call of B x R rows and
-// returns false where the one-launch forward does not apply.  fw_parts_max: units of the LM head (lm) or of O / down,
-// i.e. the most partial results that a row of a call has.
+// Host side.  fw_geometry fills what the matrices alone decide; fw_plan the rest for a call of B x R rows and returns
+// false where the one-launch forward does not apply.  fw_parts_max: tiles of the LM head (lm) or of O / down, i.e. the
+// partial results that a row of a call has.
 void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta);
 bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta);
 size_t fw_parts_max(const mtad_model_desc& d, int n_cta, bool lm);

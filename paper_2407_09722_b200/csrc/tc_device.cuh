@@ -9,11 +9,10 @@
 namespace mtad {
 namespace tcdev {
 
-// A wait gives up after this many polls.  A poll is an mbarrier.try_wait, which parks the thread until the phase completes
-// or about WAIT_PARK_NS have passed: a parked warp takes no issue slots from the warps that work, and no hand-over waits for
-// the rest of a sleep.  The limit is about a quarter of a second.
-constexpr uint32_t WAIT_LIMIT = 1u << 18;
-constexpr uint32_t WAIT_PARK_NS = 1000;
+// A wait gives up after this many polls (some tenths of a second).  A poll is an mbarrier.try_wait, which may park the
+// thread for a while: a parked warp takes no issue slots from the warps that work, and no hand-over waits for the rest of
+// a sleep.
+constexpr uint32_t WAIT_LIMIT = 1u << 20;
 constexpr int MAX_STAGES = 12;
 constexpr int EPI_THREADS = 128;
 constexpr int EPI_ROWS = 8;                       // draft rows finished per epilogue pass
@@ -58,15 +57,16 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
 __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
-        : "r"(bar), "r"(parity), "r"(WAIT_PARK_NS)
+        : "r"(bar), "r"(parity)
         : "memory");
     return ok != 0;
 }
 // Bounded wait.  Returns false when the limit ran out here or another role already gave up.  abort_flag[0] is the
 // CTA's give-up flag, abort_flag[1] the iteration limit of every wait of this launch.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    if (mbar_try(bar, parity)) return true;
     const uint32_t limit = (uint32_t)abort_flag[1];
     for (uint32_t it = 0; it < limit; ++it) {
         if (mbar_try(bar, parity)) return true;

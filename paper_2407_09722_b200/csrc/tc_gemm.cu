@@ -469,14 +469,32 @@ int tc_make_kv_map(CUtensorMap* out, const void* cache, int hd, long long cap, l
     return r == CUDA_SUCCESS ? 0 : -1;
 }
 
-int tc_make_pair_map(CUtensorMap* out, const void* base, int heads, int hp, int K, int h) {
+int tc_make_kb_map(CUtensorMap* out, const void* base, long long rows, int K, int box_rows, int kb) {
     EncodeTiledFn fn = encode_fn();
-    if (!fn || h < 1 || h > 256) return -1;
-    const cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)hp, (cuuint64_t)2 * heads};
-    const cuuint64_t strides[2] = {(cuuint64_t)K * 2, (cuuint64_t)hp * K * 2};
-    const cuuint32_t box[3] = {(cuuint32_t)TC_TILE_K, (cuuint32_t)h, 2};
+    if (!fn || box_rows < 1 || box_rows > 256 || kb < 1 || kb > 256) return -1;
+    const bool flat = tc_kb_flat(K, kb);
+    if (flat && kb != 1) return -1;
+    const cuuint64_t dims[3] = {(cuuint64_t)(flat ? K : TC_TILE_K), (cuuint64_t)rows, (cuuint64_t)(flat ? 1 : K / TC_TILE_K)};
+    const cuuint64_t strides[2] = {(cuuint64_t)K * 2, (cuuint64_t)TC_TILE_K * 2};
+    const cuuint32_t box[3] = {(cuuint32_t)TC_TILE_K, (cuuint32_t)box_rows, (cuuint32_t)kb};
     const cuuint32_t estr[3] = {1, 1, 1};
     const CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? 0 : -1;
+}
+
+int tc_make_pair_map(CUtensorMap* out, const void* base, int heads, int hp, int K, int h, int kb) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn || h < 1 || h > 256 || kb < 1 || kb > 256) return -1;
+    const bool flat = tc_kb_flat(K, kb);
+    if (flat && kb != 1) return -1;
+    const cuuint64_t dims[4] = {(cuuint64_t)(flat ? K : TC_TILE_K), (cuuint64_t)hp, (cuuint64_t)2 * heads,
+                                (cuuint64_t)(flat ? 1 : K / TC_TILE_K)};
+    const cuuint64_t strides[3] = {(cuuint64_t)K * 2, (cuuint64_t)hp * K * 2, (cuuint64_t)TC_TILE_K * 2};
+    const cuuint32_t box[4] = {(cuuint32_t)TC_TILE_K, (cuuint32_t)h, 2, (cuuint32_t)kb};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    const CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? 0 : -1;

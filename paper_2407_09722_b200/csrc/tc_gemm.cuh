@@ -103,9 +103,13 @@ int tc_make_map(CUtensorMap* out, const void* base, long long rows, long long co
 // swizzle (hd = 64 or 128).
 int tc_make_kv_map(CUtensorMap* out, const void* cache, int hd, long long cap, long long planes);
 
-// A [heads * 2 * hp, K] matrix as (K, hp, 2 * heads) with boxes of 64 elements x h rows x both halves of a head: h rotary
-// pairs, first the rows j0 .. j0 + h - 1 of the head's first half, then their partners.
-int tc_make_pair_map(CUtensorMap* out, const void* base, int heads, int hp, int K, int h);
+// Maps whose boxes bring `kb` k-blocks of the same rows in one copy, laid out [k-block][row][64 elements], and whose rows
+// are runs of kb * 128 bytes in memory.  The matrix is seen as (64, rows, K / 64); where K is no multiple of 64, or with
+// kb = 1, as (K, rows, 1) instead, so that the last k-block ends with the row.  tc_make_pair_map: a [heads * 2 * hp, K] matrix
+// with boxes of h rotary pairs, [k-block][half][h rows].
+inline bool tc_kb_flat(int K, int kb) { return kb == 1 || K % TC_TILE_K != 0; }
+int tc_make_kb_map(CUtensorMap* out, const void* base, long long rows, int K, int box_rows, int kb);
+int tc_make_pair_map(CUtensorMap* out, const void* base, int heads, int hp, int K, int h, int kb);
 
 // Fills the decomposition fields of p (and p.terms, p.per_sm for T rows) for a problem of n_tiles x k_blocks on
 // `sms` SMs with per_sm CTAs each (0: tc_ctas_per_sm(T)).
