@@ -82,6 +82,11 @@ __device__ __forceinline__ bool all_of(int id, int n, bool ok) {
         : "memory");
     return r != 0;
 }
+// one lane of the warp waits
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, bool ok, int lane) {
+    if (lane == 0 && ok) ok = mbar_wait(bar, parity, abort_flag);
+    return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+}
 __device__ __forceinline__ void bar_n(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z, int u,
@@ -428,8 +433,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             __syncwarp();
                             if (lane == 0) mbar_arrive(smem_u32(&s.qfull[as & 1]));
                         }
-                        if (ok) ok = mbar_wait(smem_u32(&s.sfull[b]), par, abort_flag);
-                        __syncwarp();
+                        ok = warp_wait(smem_u32(&s.sfull[b]), par, abort_flag, ok, lane);
                         tc_fence_after();
                         float v[NQP];
                         {
@@ -462,7 +466,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         for (int r = 0; r < NQP; ++r)
                             if (lane == r) s.smx[b][r][quad] = wm[r];
                         // the buffers P and sf of this tile are free once the output warps are done with the tile before the last
-                        if (ok) ok = mbar_wait(smem_u32(&s.oempty[b]), par ^ 1u, abort_flag);
+                        ok = warp_wait(smem_u32(&s.oempty[b]), par ^ 1u, abort_flag, ok, lane);
                         ok = all_of(2, 128, ok);
                         uint8_t* pt = Ps + b * P_BYTES + (kl >> 6) * (NQ2 * 128) + (kl & 7) * 2;
                         const int pc = (kl & 63) >> 3;
@@ -483,7 +487,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         if ((it.tile + 1) * FW_KEYS > nkeys) {
                             // rows of V past the last key: their probabilities are 0, but 0 x (stale value) must not make a NaN
                             const int vpos = pos + 2 * (x - a_lo) + 1;
-                            if (ok) ok = mbar_wait(full_bar(vpos), ring_par(vpos), abort_flag);
+                            ok = warp_wait(full_bar(vpos), ring_par(vpos), abort_flag, ok, lane);
                             if (ok && j >= nkeys) {
                                 uint8_t* vs = smem + (size_t)(vpos % NS) * FW_SLOT + kl * 128;
 #pragma unroll
@@ -497,8 +501,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         if (lane == 0) mbar_arrive(smem_u32(&s.pfull[b]));
                     } else {
                         // -------- output: a lane per head dimension
-                        if (ok) ok = mbar_wait(smem_u32(&s.ofull[b]), par, abort_flag);
-                        __syncwarp();
+                        ok = warp_wait(smem_u32(&s.ofull[b]), par, abort_flag, ok, lane);
                         tc_fence_after();
                         float c[NQ2];
                         if (NQ2 == 16) tc_ld16(t_lane + FW_TM_D + b * 64, c);
@@ -558,9 +561,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         const int n_piece = (it.f0 + it.nt - 1) / a_per - it.f0 / a_per + 1;
                         int last = 0;
                         if (n_piece > 1 && (e == 0 || two)) {
-                            __threadfence();
-                            last = atomicAdd(a.acnt + it.bi * a.Hkv + it.g, 1) + 1 == n_piece;
-                            __threadfence();
+                            int old;
+                            asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;"
+                                         : "=r"(old) : "l"(a.acnt + it.bi * a.Hkv + it.g) : "memory");
+                            last = old + 1 == n_piece;
                         }
                         s.last[e] = last;
                     }
@@ -576,16 +580,30 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             const size_t o = ((size_t)t * a.Hq + h) * a.pieces;
                             const float2* ml = reinterpret_cast<const float2*>(a.part + (size_t)T * a.Hq * a.pieces * HD) + o;
                             const float4* po = reinterpret_cast<const float4*>(a.part + o * HD) + c4;
-                            float M = -CUDART_INF_F;
-                            for (int k = 0; k < n_piece; ++k) M = fmaxf(M, __ldcg(ml + k).x);
+                            // pieces in order (deterministic), four at a time: their loads are in flight together
+                            float M = -CUDART_INF_F, ls = 0.f;
                             float4 o4 = make_float4(0.f, 0.f, 0.f, 0.f);
-                            float ls = 0.f;
-                            for (int k = 0; k < n_piece; ++k) {          // piece order: deterministic
-                                const float2 v = __ldcg(ml + k);
-                                const float4 y = __ldcg(po + (size_t)k * (HD / 4));
-                                const float wg = v.x == -CUDART_INF_F ? 0.f : exp2f(v.x - M);
-                                ls += wg * v.y;
-                                o4.x += wg * y.x; o4.y += wg * y.y; o4.z += wg * y.z; o4.w += wg * y.w;
+                            for (int k0 = 0; k0 < n_piece; k0 += 4) {
+                                float2 v[4];
+                                float4 y[4];
+#pragma unroll
+                                for (int k = 0; k < 4; ++k) {
+                                    const int kk = min(k0 + k, n_piece - 1);
+                                    v[k] = __ldcg(ml + kk);
+                                    y[k] = __ldcg(po + (size_t)kk * (HD / 4));
+                                    if (k0 + k >= n_piece) v[k].x = -CUDART_INF_F;
+                                }
+                                const float mn = fmaxf(M, fmaxf(fmaxf(v[0].x, v[1].x), fmaxf(v[2].x, v[3].x)));
+                                const float fo = mn == -CUDART_INF_F ? 1.f : exp2f(M - mn);
+                                ls *= fo;
+                                o4.x *= fo; o4.y *= fo; o4.z *= fo; o4.w *= fo;
+                                M = mn;
+#pragma unroll
+                                for (int k = 0; k < 4; ++k) {
+                                    const float wg = v[k].x == -CUDART_INF_F ? 0.f : exp2f(v[k].x - mn);
+                                    ls += wg * v[k].y;
+                                    o4.x += wg * y[k].x; o4.y += wg * y[k].y; o4.z += wg * y[k].z; o4.w += wg * y[k].w;
+                                }
                             }
                             const float f = 1.f / ls;
                             store_terms4(make_float4(o4.x * f, o4.y * f, o4.z * f, o4.w * f),
@@ -625,7 +643,9 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     const int buf = tcount & 1, f0 = tile * nf;            // first feature (O, down, gate / up, LM head)
                     // what the first items of this thread need besides the accumulator, requested ahead of it
                     float pre[4] = {0.f, 0.f, 0.f, 0.f};
-                    float u8[8];
+                    float u8[8], gn[4] = {0.f, 0.f, 0.f, 0.f};
+                    float2 cs2[2] = {};
+                    int sl2[2] = {-1, -1}, sq2[2] = {};
 #pragma unroll
                     for (int i = 0; i < 8; ++i) u8[i] = 0.5f;
                     if (kind == FW_O || kind == FW_DOWN) {
@@ -633,6 +653,18 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         for (int i = 0; i < 4; ++i) {
                             const int n = f0 + lane + 32 * i;
                             if (w < T && lane + 32 * i < nf && n < a.d) pre[i] = __ldcg(a.hidden + (size_t)w * a.d + n);
+                            if (lane + 32 * i < nf && n < a.d) gn[i] = __bfloat162float((kind == FW_O ? L->gain_ffn : L->gain_next)[n]);
+                        }
+                    } else if (kind == FW_QKV) {
+                        const int j0 = (tile % f.u) * f.h;
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            const int i = e + q * FW_EPI, t = i / nf, jj = j0 + i % nf;
+                            if (t < T && jj < HD / 2) {
+                                cs2[q] = *reinterpret_cast<const float2*>(a.rope + ((size_t)t * (HD / 2) + jj) * 2);
+                                sl2[q] = a.rm.slot[t];
+                                sq2[q] = a.rm.seq[t];
+                            }
                         }
                     } else if (kind == FW_LM && !a.lm_plain) {
 #pragma unroll
@@ -641,8 +673,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             if (w < T && lane + 32 * i < nf && n < a.V) u8[i] = a.uniforms[(size_t)(w / a.R) * a.V + n];
                         }
                     }
-                    ok = mbar_wait(smem_u32(&s.tfull[buf]), (uint32_t)(tcount >> 1) & 1u, abort_flag);
-                    __syncwarp();
+                    // (one thread polls: 256 of them would take the shared-memory pipe away from the copies' barriers)
+                    if (e == 0) ok = mbar_wait(smem_u32(&s.tfull[buf]), (uint32_t)(tcount >> 1) & 1u, abort_flag);
+                    ok = all_of(1, FW_EPI, ok);
+                    if (!ok) break;
                     tc_fence_after();
                     for (int r0 = 0; r0 < T; r0 += blk) {
                     const int r1 = min(T, r0 + blk);
@@ -694,8 +728,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         for (int i = e; i < nr * nf; i += FW_EPI) {
                             const int t = r0 + i / nf, j = i % nf, jj = j0 + j;
                             if (jj >= hp) continue;
-                            const int sl = a.rm.slot[t];
-                            const float2 cs = *reinterpret_cast<const float2*>(a.rope + ((size_t)t * hp + jj) * 2);
+                            const int ahead = r0 == 0 ? i / FW_EPI : 2;
+                            const int sl = ahead == 0 ? sl2[0] : (ahead == 1 ? sl2[1] : a.rm.slot[t]);
+                            const float2 cs = ahead == 0 ? cs2[0] : (ahead == 1 ? cs2[1] :
+                                              *reinterpret_cast<const float2*>(a.rope + ((size_t)t * hp + jj) * 2));
                             const float rs = s.rstd[t];
                             const float va = yv(t, 0, j) * rs, vb = yv(t, 0, f.h + j) * rs;
                             if (sl < 0) continue;                         // inactive row: no query, no cache slot
@@ -706,7 +742,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                                 split_store(ra * scale * 1.4426950408889634f, a.q_hi + o, a.q_lo + o);
                                 split_store(rb * scale * 1.4426950408889634f, a.q_hi + o + hp, a.q_lo + o + hp);
                             } else {
-                                const int sq = a.rm.seq[t], kv = hg >= a.Hq + a.Hkv ? 1 : 0;
+                                const int sq = ahead == 0 ? sq2[0] : (ahead == 1 ? sq2[1] : a.rm.seq[t]), kv = hg >= a.Hq + a.Hkv ? 1 : 0;
                                 if (sl >= a.cap || (unsigned)sq >= (unsigned)a.max_batch) continue;   // never past the cache
                                 __nv_bfloat16* c = a.cache + idx_cache(layer, a.max_batch, sq, kv, a.Hkv, hg - a.Hq - kv * a.Hkv, a.cap, sl, HD);
                                 c[jj] = __float2bfloat16_rn(kv ? va : ra);
@@ -769,7 +805,6 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         }
                     } else {
                         // residual: a warp per row; emits the next operand rows and the row's share of its sum of squares
-                        const __nv_bfloat16* gain = kind == FW_O ? L->gain_ffn : L->gain_next;
                         float* sq = kind == FW_O ? a.sumsq_b : a.sumsq_a;
                         for (int t = r0 + w; t < r1; t += 8) {
                             float ss = 0.f;
@@ -780,7 +815,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                                 float* hp = a.hidden + (size_t)t * a.d + n;
                                 const float y = yv(t, 0, jl) + (t == w ? pre[i] : __ldcg(hp));
                                 *hp = y;
-                                store_terms(y * __bfloat162float(gain[n]), a.x_d + (size_t)t * terms * a.d + n, a.d, terms);
+                                store_terms(y * gn[i], a.x_d + (size_t)t * terms * a.d + n, a.d, terms);
                                 ss += y * y;
                             }
 #pragma unroll
@@ -795,11 +830,9 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 if (!ok) break;
             }
             if (kind != FW_LM) {
-                // phase barrier: this block's rows are visible to the other blocks' loads and TMA copies
-                proxy_fence();
+                // phase barrier: the release covers the whole group's stores (the readers' proxy fence follows their acquire)
                 bar_n(1, FW_EPI);
                 if (e == 0) {
-                    __threadfence();
                     asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(a.sync + p) : "memory");
                 }
             }
