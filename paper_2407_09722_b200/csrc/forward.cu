@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     float* Y = reinterpret_cast<float*>(uni);
     uint8_t* Qs = uni;                                 // [2][Q_BYTES]
     uint8_t* Ps = uni + 2 * Q_BYTES;                   // [2][P_BYTES]
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int cta = (int)blockIdx.x, n_cta = a.n_cta;
     const int T = a.T, cols = a.cols, terms = a.terms;
     const int n_phases = 5 * a.n_layers + 1;
@@ -306,8 +306,9 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
             }
         }
     } else if (warp == 2) {
-        // ---------------- MMA issuer
-        if (lane == 0) {
+        // ---------------- MMA issuer (the whole warp runs the loop, see tc_mma_one)
+        {
+            const uint32_t one = elect_one();
             constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (8u << 24);      // bf16 x bf16 -> fp32, M = 128
             int pos = 0, tcount = 0, at = 0, as = 0;   // ring position, projection tiles, attention tiles, segments so far
             bool ok = true;
@@ -321,17 +322,17 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         const AttnItem it = attn_item(s.pref, a.Hkv, a_lo + i);
                         const bool fresh = i == 0 || it.tile == 0;
                         if (fresh && i > 0) ++as;
-                        if (fresh && !mbar_wait(smem_u32(&s.qfull[as & 1]), (uint32_t)(as >> 1) & 1u, abort_flag)) return false;
+                        if (fresh && !mbar_wait_warp(smem_u32(&s.qfull[as & 1]), (uint32_t)(as >> 1) & 1u, abort_flag)) return false;
                         const int kpos = pos + 2 * i, b = (at + i) & 1;
-                        if (!mbar_wait(full_bar(kpos), ring_par(kpos), abort_flag)) return false;
+                        if (!mbar_wait_warp(full_bar(kpos), ring_par(kpos), abort_flag)) return false;
                         tc_fence_after();
                         const uint32_t ka = slot_ptr(kpos), qa = smem_u32(Qs + (as & 1) * Q_BYTES);
 #pragma unroll
                         for (int ks = 0; ks < HD / 16; ++ks)
-                            tc_mma(tmem + b * 64, smem_desc(ka + (ks >> 2) * (FW_KEYS * 128) + (ks & 3) * 32),
+                            tc_mma_one(one, tmem + b * 64, smem_desc(ka + (ks >> 2) * (FW_KEYS * 128) + (ks & 3) * 32),
                                    smem_desc(qa + (ks >> 2) * (NQ2 * 128) + (ks & 3) * 32), idesc_s, ks > 0 ? 1u : 0u);
-                        tc_commit(smem_u32(&s.sfull[b]));
-                        tc_commit(empty_bar(kpos));
+                        tc_commit_one(one, smem_u32(&s.sfull[b]));
+                        tc_commit_one(one, empty_bar(kpos));
                         return true;
                     };
                     if (a_n > 0) ok = scores(0);
@@ -343,17 +344,17 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         if (!ok) break;
                         const int vpos = pos + 2 * i + 1, b = (at + i) & 1;
                         const uint32_t par = (uint32_t)((at + i) >> 1) & 1u;
-                        ok = mbar_wait(smem_u32(&s.pfull[b]), par, abort_flag) && mbar_wait(full_bar(vpos), ring_par(vpos), abort_flag) &&
-                             mbar_wait(smem_u32(&s.oempty[b]), par ^ 1u, abort_flag);
+                        ok = mbar_wait_warp(smem_u32(&s.pfull[b]), par, abort_flag) && mbar_wait_warp(full_bar(vpos), ring_par(vpos), abort_flag) &&
+                             mbar_wait_warp(smem_u32(&s.oempty[b]), par ^ 1u, abort_flag);
                         if (!ok) break;
                         tc_fence_after();
                         const uint32_t va = slot_ptr(vpos), pa = smem_u32(Ps + b * P_BYTES);
 #pragma unroll
                         for (int ks = 0; ks < FW_KEYS / 16; ++ks)
-                            tc_mma(tmem + FW_TM_D + b * 64, smem_desc_mn(va + ks * 2048),
+                            tc_mma_one(one, tmem + FW_TM_D + b * 64, smem_desc_mn(va + ks * 2048),
                                    smem_desc(pa + (ks >> 2) * (NQ2 * 128) + (ks & 3) * 32), idesc_o, ks > 0 ? 1u : 0u);
-                        tc_commit(smem_u32(&s.ofull[b]));
-                        tc_commit(empty_bar(vpos));
+                        tc_commit_one(one, smem_u32(&s.ofull[b]));
+                        tc_commit_one(one, empty_bar(vpos));
                         if (more && !ahead) ok = scores(i + 1);
                     }
                     if (a_n > 0) ++as;
@@ -366,24 +367,25 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 const uint32_t idesc = IDESC | ((uint32_t)((f.S * cols) >> 3) << 17);
                 for (int tile = cta; tile < f.n_tiles && ok; tile += n_cta, ++tcount) {
                     const int buf = tcount & 1;
-                    ok = mbar_wait(smem_u32(&s.tempty[buf]), ((uint32_t)(tcount >> 1) & 1u) ^ 1u, abort_flag);
+                    ok = mbar_wait_warp(smem_u32(&s.tempty[buf]), ((uint32_t)(tcount >> 1) & 1u) ^ 1u, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t d = tmem + buf * 256;
                     for (int step = 0; step < f.steps; ++step, ++pos) {
-                        ok = mbar_wait(full_bar(pos), ring_par(pos), abort_flag);
+                        ok = mbar_wait_warp(full_bar(pos), ring_par(pos), abort_flag);
                         if (!ok) break;
                         tc_fence_after();
-                        const uint32_t base = slot_ptr(pos), bb = base + f.b_off;
-                        for (int gr = 0; gr < groups; ++gr)
+                        const uint32_t base = slot_ptr(pos);
+                        uint64_t ad = smem_desc(base), bd = smem_desc(base + f.b_off);      // (addresses in 16-byte units)
+                        for (int gr = 0; gr < groups; ++gr, ad += f.S * f.hr * 8, bd += sc * 8)
                             for (int q = 0; q < f.nbox; ++q)
 #pragma unroll
                                 for (int k4 = 0; k4 < TC_TILE_K / 16; ++k4)
-                                    tc_mma(d + q * sc, smem_desc(base + q * f.box_bytes + gr * f.S * f.hr * 128 + k4 * 32),
-                                           smem_desc(bb + gr * sc * 128 + k4 * 32), idesc, (step > 0 || gr > 0 || k4 > 0) ? 1u : 0u);
-                        tc_commit(empty_bar(pos));
+                                    tc_mma_one(one, d + q * sc, ad + (uint32_t)(q * f.box_bytes / 16 + k4 * 2), bd + k4 * 2, idesc,
+                                               (step > 0 || gr > 0 || k4 > 0) ? 1u : 0u);
+                        tc_commit_one(one, empty_bar(pos));
                     }
-                    if (ok) tc_commit(smem_u32(&s.tfull[buf]));
+                    if (ok) tc_commit_one(one, smem_u32(&s.tfull[buf]));
                 }
             }
         }

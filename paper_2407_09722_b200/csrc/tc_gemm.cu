@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) tc_gemm_kernel(const __grid_con
     const int stage_bytes = a_bytes + acc_cols * 128;
     const int stages = p0.stages, nbuf = p0.nbuf, T = p0.T;
     const Smem s = carve(smem_base, stages, stage_bytes);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&ch.maps[0].a0)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&ch.maps[0].x)) : "memory");
@@ -161,7 +161,8 @@ __global__ void __launch_bounds__(TC_THREADS, 2) tc_gemm_kernel(const __grid_con
     } else if (warp < 2 + MAX_HALVES) {
         // ---------------- MMA issuers: warp 2 + h owns the 128-row half h of every stage and its accumulator --------
         const int h = warp - 2;
-        if (lane == 0 && h < mh) {
+        if (h < mh) {       // (the whole warp runs the loop, see tc_mma_one)
+            const uint32_t one = elect_one();
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(bbox_rows >> 3) << 17) |
                                    ((uint32_t)(TC_TILE_N >> 4) << 24);
             int g = 0, seg = 0;                        // running unit and segment counters
@@ -179,16 +180,16 @@ __global__ void __launch_bounds__(TC_THREADS, 2) tc_gemm_kernel(const __grid_con
                     const int len = min(min(KB - kb0, n_units - i), cap);
                     const int buf = seg % nbuf;
                     const uint32_t aph = (uint32_t)(seg / nbuf) & 1u;
-                    ok = mbar_wait(smem_u32(&s.tempty[buf]), aph ^ 1u, abort_flag);
+                    ok = mbar_wait_warp(smem_u32(&s.tempty[buf]), aph ^ 1u, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t d_tmem = tmem_base + (uint32_t)(buf * mh * acc_cols);
                     for (int k = 0; k < len && ok; ++k, ++i, ++g) {
                         const int st = g % stages;
                         const uint32_t sph = (uint32_t)(g / stages) & 1u;
-                        ok = mbar_wait(smem_u32(&s.full[st]), sph, abort_flag);
+                        ok = mbar_wait_warp(smem_u32(&s.full[st]), sph, abort_flag);
                         if (!ok) break;
-                        if (g == 0 && h == 0) trace_stamp(p0.trace, 2);
+                        if (g == 0 && h == 0 && lane == 0) trace_stamp(p0.trace, 2);
                         tc_fence_after();
                         const uint32_t a_addr = smem_u32(s.ring + (size_t)st * stage_bytes);
                         const uint32_t b_addr = a_addr + a_bytes;
@@ -197,13 +198,13 @@ __global__ void __launch_bounds__(TC_THREADS, 2) tc_gemm_kernel(const __grid_con
                             const uint32_t acc = (k > 0 || k4 > 0) ? 1u : 0u;
                             const uint64_t ad = smem_desc(a_addr + h * TC_TILE_N * 128 + k4 * 32);
                             for (int b = 0; b < n_bbox; ++b)
-                                tc_mma(d_tmem + (uint32_t)(h * acc_cols + b * bbox_rows), ad,
+                                tc_mma_one(one, d_tmem + (uint32_t)(h * acc_cols + b * bbox_rows), ad,
                                        smem_desc(b_addr + b * bbox_rows * 128 + k4 * 32), idesc, acc);
                         }
-                        tc_commit(smem_u32(&s.empty[st]));      // frees the smem stage once these MMAs have read it
+                        tc_commit_one(one, smem_u32(&s.empty[st]));      // frees the smem stage once these MMAs have read it
                     }
-                    if (ok) tc_commit(smem_u32(&s.tfull[buf]));  // accumulator of this segment complete
-                    if (h == 0 && i == n_units) trace_stamp(p0.trace, 3);
+                    if (ok) tc_commit_one(one, smem_u32(&s.tfull[buf]));  // accumulator of this segment complete
+                    if (h == 0 && i == n_units && lane == 0) trace_stamp(p0.trace, 3);
                     ++seg;
                 }
             }

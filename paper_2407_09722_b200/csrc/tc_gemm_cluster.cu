@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(CL_THREADS, 2) tc_gemm_cluster_kernel(const __
     const int stages = p.stages;
     const int csize = p.csize, rpr = p.rpr;
     const ClSmem s = cl_carve(smem_base, stages, stage_bytes, cl_recv_floats(T, rpr, csize) * (int)sizeof(float));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int rank = (int)cluster_ctarank();
     const int tile = (int)blockIdx.x / csize;
     const int kb0 = (int)(((long long)rank * p.k_blocks) / csize);
@@ -171,26 +171,27 @@ __global__ void __launch_bounds__(CL_THREADS, 2) tc_gemm_cluster_kernel(const __
         }
     } else if (warp == 2) {
         // ---------------- MMA issuer
-        if (lane == 0) {
+        {   // (the whole warp runs the loop, see tc_mma_one)
+            const uint32_t one = elect_one();
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(acc_cols >> 3) << 17) |
                                    ((uint32_t)(TC_TILE_N >> 4) << 24);
             bool ok = true;
             for (int i = 0; i < n_kb && ok; ++i) {
                 const int st = i % stages;
-                ok = mbar_wait(smem_u32(&s.full[st]), (uint32_t)(i / stages) & 1u, abort_flag);
+                ok = mbar_wait_warp(smem_u32(&s.full[st]), (uint32_t)(i / stages) & 1u, abort_flag);
                 if (!ok) break;
-                if (i == 0) trace_stamp(p.trace, 2);
+                if (i == 0 && lane == 0) trace_stamp(p.trace, 2);
                 tc_fence_after();
                 const uint32_t a_addr = smem_u32(s.ring + (size_t)st * stage_bytes);
                 const uint32_t b_addr = a_addr + a_bytes;
 #pragma unroll
                 for (int k4 = 0; k4 < TC_TILE_K / 16; ++k4)
-                    tc_mma(tmem_base, smem_desc(a_addr + k4 * 32), smem_desc(b_addr + k4 * 32), idesc,
+                    tc_mma_one(one, tmem_base, smem_desc(a_addr + k4 * 32), smem_desc(b_addr + k4 * 32), idesc,
                            (i > 0 || k4 > 0) ? 1u : 0u);
-                tc_commit(smem_u32(&s.empty[st]));
+                tc_commit_one(one, smem_u32(&s.empty[st]));
             }
-            if (ok) tc_commit(smem_u32(s.tfull));
-            trace_stamp(p.trace, 3);
+            if (ok) tc_commit_one(one, smem_u32(s.tfull));
+            if (lane == 0) trace_stamp(p.trace, 3);
         }
     } else {
         // ---------------- epilogue

@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(BG_THREADS, 1) tc_gemm_cluster_big_kernel(cons
     const int stages = p.stages;
     const int csize = p.csize, rpr = p.rpr;
     const BgSmem s = bg_carve(smem_base, p.ring_bytes);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int rank = (int)cluster_ctarank();
     const int tile = p.tile_base + (int)blockIdx.x / csize;
     const int kb0 = (int)(((long long)rank * p.k_blocks) / csize);
@@ -193,27 +193,28 @@ __global__ void __launch_bounds__(BG_THREADS, 1) tc_gemm_cluster_big_kernel(cons
     } else if (warp < BG_EPI_WARP0) {
         // ---------------- MMA issuers: warp 2 + h owns the 128-feature half h of every stage and its accumulator
         const int h = warp - 2;
-        if (lane == 0 && h < mh) {
+        if (h < mh) {       // (the whole warp runs the loop, see tc_mma_one)
+            const uint32_t one = elect_one();
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(acc_cols >> 3) << 17) |
                                    ((uint32_t)(TC_TILE_N >> 4) << 24);
             const uint32_t d_tmem = tmem_base + (uint32_t)(h * acc_cols);
             bool ok = true;
             for (int i = 0; i < n_kb && ok; ++i) {
                 const int st = i % stages;
-                ok = mbar_wait(smem_u32(&s.full[st]), (uint32_t)(i / stages) & 1u, abort_flag);
+                ok = mbar_wait_warp(smem_u32(&s.full[st]), (uint32_t)(i / stages) & 1u, abort_flag);
                 if (!ok) break;
-                if (i == 0 && h == 0) trace_stamp(p.trace, 2);
+                if (i == 0 && h == 0 && lane == 0) trace_stamp(p.trace, 2);
                 tc_fence_after();
                 const uint32_t a_addr = smem_u32(s.ring + (size_t)st * stage_bytes) + h * TC_TILE_N * 128;
                 const uint32_t b_addr = smem_u32(s.ring + (size_t)st * stage_bytes) + a_bytes;
 #pragma unroll
                 for (int k4 = 0; k4 < TC_TILE_K / 16; ++k4)
-                    tc_mma(d_tmem, smem_desc(a_addr + k4 * 32), smem_desc(b_addr + k4 * 32), idesc,
+                    tc_mma_one(one, d_tmem, smem_desc(a_addr + k4 * 32), smem_desc(b_addr + k4 * 32), idesc,
                            (i > 0 || k4 > 0) ? 1u : 0u);
-                tc_commit(smem_u32(&s.empty[st]));
+                tc_commit_one(one, smem_u32(&s.empty[st]));
             }
-            if (ok) tc_commit(smem_u32(s.tfull));
-            if (h == 0) trace_stamp(p.trace, 3);
+            if (ok) tc_commit_one(one, smem_u32(s.tfull));
+            if (h == 0 && lane == 0) trace_stamp(p.trace, 3);
         }
     } else {
         // ---------------- epilogue: two groups of 128 threads
