@@ -22,8 +22,8 @@
 //   O^T += V^T P  A = V tile (MN-major), B = P; a thread per head dimension adds it to its registers
 // Pieces of a (sequence, KV head) held by several blocks meet in global memory; the block that arrives last merges them.
 //
-// Warps: 0 weight and K / V producer (TMA), 1 operand-row producer (TMA; waits for the phase before), 2 MMA issuer,
-// 3 tensor memory, 4..11 epilogue; in the attention 4..7 softmax (a lane per key) and 8..11 output (a lane per dimension).
+// Warps: 0 weight and K / V producer (TMA), 1 operand-row producer (TMA; waits for the phase before), 2 and 3 MMA issuers
+// (3 owns the tensor memory), 4..11 epilogue; in the attention 4..7 softmax (a lane per key) and 8..11 output (a lane per dimension).
 // Every wait is bounded; a block that gives up raises MTAD_ST_TIMEOUT for every sequence of the call and leaves, and the
 // others run into their own limits at the grid barrier.
 #include <math_constants.h>
@@ -45,20 +45,6 @@ constexpr int FW_UNION = 32 * 1024;       // epilogue tile Y, or the attention's
 constexpr int NS = FW_SLOTS;
 constexpr int FW_ACC = 240;               // accumulator columns of a tile, of 256 (the drain reads up to 15 columns further)
 constexpr int FW_TM_D = 128;              // attention: tensor-memory columns 0 / 64 scores, 128 / 192 outputs
-
-struct FwTail {
-    float rstd[64];
-    float smx[2][16][4];                  // row maxima of the four softmax warps
-    float sf[2][16];                      // rescale factor of the running output, per tile buffer
-    float sl[2][4][16];                   // row sums of the softmax warps
-    float sm[2][16];                      // row reference values
-    int pref[MTAD_MAX_BATCH + 1];         // flattened attention tiles before sequence b
-    uint64_t full[NS], empty[NS];
-    uint64_t tfull[2], tempty[2], sfull[2], pfull[2], ofull[2], oempty[2], qfull[2];
-    uint32_t tmem_ptr;
-    int abort_flag[2];
-    int last[2];
-};
 
 __device__ __forceinline__ bool grid_wait(const int* c, int want, volatile int* abort_flag) {
     const uint32_t limit = (uint32_t)abort_flag[1];
@@ -116,26 +102,321 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool v
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
 }
 
+// What a call's sequence looks like to the attention
+struct SeqMeta {
+    int nrows, L, nkeys, seq;
+};
+
 // The attention items of a call: sequences in order, KV heads in order, 128-key tiles in order; block c takes
 // [c * per, (c + 1) * per).
-struct AttnItem {
+struct AttnPos {
     int bi, g, tile, nt;                  // nt: tiles of the sequence
     int f0;                               // first item of the (sequence, KV head)
 };
-__device__ __forceinline__ AttnItem attn_item(const int* pref, int Hkv, int x) {
-    AttnItem it;
-    int b = 0;
-    while (x >= pref[b + 1]) ++b;
-    const int nt = (pref[b + 1] - pref[b]) / Hkv, y = x - pref[b];
-    it.bi = b;
-    it.nt = nt;
-    it.g = y / nt;
-    it.tile = y - it.g * nt;
-    it.f0 = x - it.tile;
+__device__ __forceinline__ int attn_tiles(const SeqMeta& m) { return m.nrows > 0 ? (m.nkeys + FW_KEYS - 1) / FW_KEYS : 0; }
+__device__ __forceinline__ AttnPos attn_find(const SeqMeta* meta, int B, int Hkv, int x) {
+    AttnPos it{};
+    int base = 0;
+    for (int b = 0; b < B; ++b) {
+        const int nt = attn_tiles(meta[b]);
+        if (x < base + nt * Hkv) {
+            it.bi = b;
+            it.nt = nt;
+            it.g = (x - base) / nt;
+            it.tile = x - base - it.g * nt;
+            it.f0 = x - it.tile;
+            break;
+        }
+        base += nt * Hkv;
+    }
     return it;
 }
+__device__ __forceinline__ void attn_next(AttnPos& it, const SeqMeta* meta, int B, int Hkv) {
+    if (++it.tile < it.nt) return;
+    it.f0 += it.nt;
+    it.tile = 0;
+    if (++it.g < Hkv) return;
+    it.g = 0;
+    do ++it.bi; while (it.bi < B && attn_tiles(meta[it.bi]) == 0);
+    if (it.bi < B) it.nt = attn_tiles(meta[it.bi]);
+}
 
-static_assert(1024 + NS * FW_SLOT + FW_UNION + sizeof(FwTail) <= 227 * 1024, "shared memory of the forward");
+struct FwTail {
+    SeqMeta meta[MTAD_MAX_BATCH];
+    float rstd[64];
+    float smx[2][16][4];                  // row maxima of the four softmax warps
+    float sf[2][16];                      // rescale factor of the running output, per tile buffer
+    float sl[2][4][16];                   // row sums of the softmax warps
+    float sm[2][16];                      // row reference values
+    uint64_t full[NS], empty[NS];
+    uint64_t tfull[2], tempty[2], sfull[2], pfull[2], ofull[2], oempty[2], qfull[2];
+    uint32_t tmem_ptr;
+    int abort_flag[2];
+    int last[2];
+};
+static_assert(NS * FW_SLOT + FW_UNION + sizeof(FwTail) <= 227 * 1024, "shared memory of the forward");
+
+// The epilogue group's part of one projection: row statistics, then per tile the accumulators -> Y in shared memory ->
+// the fused epilogue.  KIND is a template parameter so that the phase's geometry is read straight from the launch
+// parameters; index arithmetic and global loads stand ahead of the wait for the accumulator, because everything after it
+// is a chain of latencies between the last weight and the next phase's first.
+template <int KIND, int HD>
+__device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, int p, int layer, int& tcount, int e,
+                                          uint32_t tmem_lane, int cta) {
+    const FwPhase& f = a.ph[KIND];
+    if (cta >= f.n_tiles) return true;
+    volatile int* abort_flag = s.abort_flag;
+    const int lane = e & 31, w = e >> 5, quad = w & 3, half = w >> 2;
+    const int T = a.T, terms = a.terms, cols = a.cols, n_cta = a.n_cta;
+    const int hr = f.hr, S = f.S, nbox = f.nbox;
+    const int yb = S * hr, ys = nbox * yb + 4;             // columns of Y that a box takes, row stride of Y
+    const int nf = KIND == FW_LM ? nbox * f.h : f.h;       // features (pairs) of a tile
+    const int per = terms == 3 ? 5 : 8, blk = f.blk;       // rows of a drain load, rows that Y holds at a time
+    // a lane's slice of the S k-blocks that the MMA takes side by side is tl / hr; a warp's lanes may lie in several
+    const int tl = quad * 32 + lane, my = tl / hr;
+    const int s0 = S > 1 ? quad * 32 / hr : 0, s1 = S > 1 ? min(S - 1, (quad * 32 + 31) / hr) : 0;
+    const int it0 = e / nf, ij0 = e - it0 * nf, dt = FW_EPI / nf, dj = FW_EPI - dt * nf;    // this thread's items (row, feature)
+    bool ok = true;
+    if (KIND == FW_QKV || KIND == FW_GATEUP || KIND == FW_LM) {
+        // scale of the deferred RMSNorm: the rows' sums of squares come from every block
+        if (p > 0) {
+            if (e == 0) ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
+            ok = all_of(1, FW_EPI, ok);
+            if (!ok) return false;
+        }
+        const float* sq = KIND == FW_GATEUP ? a.sumsq_b : a.sumsq_a;
+        const int parts = KIND == FW_GATEUP ? a.ph[FW_O].n_tiles : (p == 0 ? a.parts0 : a.ph[FW_DOWN].n_tiles);
+        for (int r = w; r < T; r += 8) {
+            float v = 0.f;
+            for (int q = lane; q < parts; q += 32) v += __ldcg(sq + (size_t)q * TC_X_ROWS + r);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0) s.rstd[r] = rsqrtf(v * a.inv_dim + a.eps);
+        }
+    }
+    const FwLayer* L = a.layers + layer;
+    for (int tile = cta; tile < f.n_tiles; tile += n_cta, ++tcount) {
+        const int buf = tcount & 1, f0 = tile * nf;        // f0: first feature (O, down, gate / up, LM head)
+        // ---- what the first items need besides the accumulator
+        // QKV
+        const int hg = KIND == FW_QKV ? tile / f.u : 0, j0 = KIND == FW_QKV ? (tile - hg * f.u) * f.h : 0;
+        constexpr int NI = 4;                              // items per thread whose loads are in flight together
+        int sl4[NI], sq4[NI];
+        float2 cs4[NI];
+        auto qkv_load = [&](int t, int j) {
+#pragma unroll
+            for (int q = 0; q < NI; ++q) {
+                sl4[q] = -1;
+                if (t < T && j0 + j < HD / 2) {
+                    cs4[q] = *reinterpret_cast<const float2*>(a.rope + ((size_t)t * (HD / 2) + j0 + j) * 2);
+                    sl4[q] = a.rm.slot[t];
+                    sq4[q] = a.rm.seq[t];
+                }
+                t += dt; j += dj;
+                if (j >= nf) { j -= nf; ++t; }
+            }
+        };
+        // O, down: the residual rows w, w + 8, ... of the first 32 features
+        float hid[NI], gain0 = 0.f;
+        const __nv_bfloat16* gain = KIND == FW_O ? L->gain_ffn : L->gain_next;
+        auto res_load = [&](int t, int n, bool in) {
+#pragma unroll
+            for (int q = 0; q < NI; ++q)
+                hid[q] = (in && t + 8 * q < T) ? __ldcg(a.hidden + (size_t)(t + 8 * q) * a.d + n) : 0.f;
+        };
+        float u8[8];
+        auto lm_load = [&](int t) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int jl = lane + 32 * i, n = f0 + jl;
+                u8[i] = (t < T && jl < nf && n < a.V) ? a.uniforms[(size_t)(t / a.R) * a.V + n] : 0.5f;
+            }
+        };
+        if (KIND == FW_QKV) qkv_load(it0, ij0);
+        if (KIND == FW_O || KIND == FW_DOWN) {
+            const bool in = lane < nf && f0 + lane < a.d;
+            if (in) gain0 = __bfloat162float(gain[f0 + lane]);
+            res_load(w, f0 + lane, in);
+        }
+        if (KIND == FW_LM && !a.lm_plain) lm_load(w);
+        // (one thread polls: 256 of them would take the shared-memory pipe away from the copies' barriers)
+        if (e == 0) ok = mbar_wait(smem_u32(&s.tfull[buf]), (uint32_t)(tcount >> 1) & 1u, abort_flag);
+        ok = all_of(1, FW_EPI, ok);
+        if (!ok) return false;
+        tc_fence_after();
+        const uint32_t t_acc = tmem_lane + buf * 256;
+        for (int r0 = 0; r0 < T; r0 += blk) {
+            const int r1 = min(T, r0 + blk), nr = r1 - r0;
+            // ---- accumulators -> Y[row][box][lane], the terms of a row added up
+            int b = 0, rb = r0 + (nbox == 1 ? half * per : 0);
+            if (nbox == 2) b = half;                       // the two warps of a quadrant share out the boxes, or the row groups
+            for (; rb < r1; rb += nbox == 1 ? 2 * per : per)
+                for (int sl = s0; sl <= s1; ++sl) {
+                    float v[16];
+                    tc_ld16(t_acc + (b * S + sl) * cols + rb * terms, v);
+                    if (f.dual) {
+                        float v2[16];
+                        tc_ld16(t_acc + (S + sl) * cols + rb * terms, v2);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) v[j] += v2[j];
+                    }
+                    if (my == sl && tl < yb) {
+                        float* y = Y + (rb - r0) * ys + b * yb + tl;
+                        if (terms == 3) {
+#pragma unroll
+                            for (int j = 0; j < 5; ++j)
+                                if (rb + j < r1) y[j * ys] = v[3 * j] + (v[3 * j + 1] + v[3 * j + 2]);
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 8; ++j)
+                                if (rb + j < r1) y[j * ys] = v[2 * j] + v[2 * j + 1];
+                        }
+                    }
+                    __syncwarp();
+                }
+            if (r1 == T) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&s.tempty[buf]));
+            }
+            bar_n(1, FW_EPI);
+            // value of (row of the block, box, weight row): the S slices lie side by side
+            auto yv = [&](int t, int q, int row) -> float {
+                const float* y = Y + t * ys + q * yb + row;
+                float v = y[0];
+#pragma unroll 4
+                for (int sl = 1; sl < S; ++sl) v += y[sl * hr];
+                return v;
+            };
+            if (KIND == FW_QKV) {
+                constexpr int hp = HD / 2;
+                const float scale = rsqrtf((float)HD);
+                int t = it0, j = ij0;
+                for (int i = e; i < nr * nf; i += NI * FW_EPI) {
+                    if (r0 > 0 || i != e) qkv_load(r0 + t, j);
+#pragma unroll
+                    for (int q = 0; q < NI; ++q) {
+                        const int jj = j0 + j;
+                        if (t < nr && jj < hp && sl4[q] >= 0) {           // (no slot: an inactive row has no query and no keys)
+                            const float rs = s.rstd[r0 + t];
+                            const float va = yv(t, 0, j) * rs, vb = yv(t, 0, f.h + j) * rs;
+                            const float2 cs = cs4[q];
+                            const float ra = va * cs.x - vb * cs.y, rb2 = vb * cs.x + va * cs.y;
+                            if (hg < a.Hq) {
+                                // attention operands: q * log2(e) / sqrt(hd) as bf16 hi + lo (softmax runs on exp2)
+                                const size_t o = ((size_t)(r0 + t) * a.Hq + hg) * HD + jj;
+                                split_store(ra * scale * 1.4426950408889634f, a.q_hi + o, a.q_lo + o);
+                                split_store(rb2 * scale * 1.4426950408889634f, a.q_hi + o + hp, a.q_lo + o + hp);
+                            } else if (sl4[q] < a.cap && (unsigned)sq4[q] < (unsigned)a.max_batch) {   // never past the cache
+                                const int kv = hg >= a.Hq + a.Hkv ? 1 : 0;
+                                __nv_bfloat16* c = a.cache + idx_cache(layer, a.max_batch, sq4[q], kv, a.Hkv, hg - a.Hq - kv * a.Hkv,
+                                                                       a.cap, sl4[q], HD);
+                                c[jj] = __float2bfloat16_rn(kv ? va : ra);
+                                c[jj + hp] = __float2bfloat16_rn(kv ? vb : rb2);
+                            }
+                        }
+                        t += dt; j += dj;
+                        if (j >= nf) { j -= nf; ++t; }
+                    }
+                }
+            } else if (KIND == FW_GATEUP) {
+                int t = it0, j = ij0;
+                for (int i = e; i < nr * nf; i += 2 * FW_EPI) {
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const int n = f0 + j;
+                        if (t < nr && n < a.F) {
+                            const float rs = s.rstd[r0 + t];
+                            const float g = yv(t, 0, j) * rs, up = yv(t, 1, j) * rs;
+                            store_terms(g / (1.f + expf(-g)) * up, a.x_f + (size_t)(r0 + t) * terms * a.F + n, a.F, terms);
+                        }
+                        t += dt; j += dj;
+                        if (j >= nf) { j -= nf; ++t; }
+                    }
+                }
+            } else if (KIND == FW_LM) {
+                if (a.lm_plain) {
+                    int t = it0, j = ij0;
+                    for (int i = e; i < nr * nf; i += FW_EPI) {
+                        const int q = j >= f.h ? 1 : 0, n = f0 + j;
+                        if (n < a.V) a.logits[(size_t)(r0 + t) * a.V + n] = yv(t, q, j - q * f.h) * s.rstd[r0 + t];
+                        t += dt; j += dj;
+                        if (j >= nf) { j -= nf; ++t; }
+                    }
+                } else {
+                    // a warp per row: maximum, sum of exponentials, arg-max of the perturbed logits over the tile
+                    for (int t = r0 + w; t < r1; t += 8) {
+                        float z[8], m = -CUDART_INF_F, bv = -CUDART_INF_F, sum = 0.f;
+                        int bi = 0x7fffffff;
+                        const float rs = s.rstd[t];
+                        if (t != w) lm_load(t);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const int jl = lane + 32 * i, n = f0 + jl, q = jl >= f.h ? 1 : 0;
+                            const bool in = jl < nf && n < a.V;
+                            z[i] = in ? yv(t - r0, q, jl - q * f.h) * rs : -CUDART_INF_F;
+                            m = fmaxf(m, z[i]);
+                            const float pz = in ? z[i] - logf(-logf(u8[i])) : -CUDART_INF_F;
+                            if (in && (pz > bv || (pz == bv && n < bi))) { bv = pz; bi = n; }
+                        }
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) {
+                            m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+                            const float v2 = __shfl_xor_sync(0xffffffffu, bv, o);
+                            const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
+                            if (v2 > bv || (v2 == bv && i2 < bi)) { bv = v2; bi = i2; }
+                        }
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) sum += z[i] == -CUDART_INF_F ? 0.f : expf(z[i] - m);
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                        if (lane == 0) a.lm_part[idx_lm_part(t, f.n_tiles, tile)] = make_float4(m, sum, bv, __int_as_float(bi));
+                    }
+                    // logit of each node's token under its parent row, where it falls into this tile
+                    for (int t = e; t < T; t += FW_EPI) {
+                        const int pr = a.rm.prow[t];
+                        if (pr < r0 || pr >= r1) continue;
+                        const int tk = a.rm.tok[t] - f0, q = tk >= f.h ? 1 : 0;
+                        if (tk >= 0 && tk < nf) a.node_z[t] = yv(pr - r0, q, tk - q * f.h) * s.rstd[pr];
+                    }
+                }
+            } else {
+                // residual: a warp per row, four rows at a time; emits the next operand rows and the rows' share of their sums
+                // of squares
+                float* sq = KIND == FW_O ? a.sumsq_b : a.sumsq_a;
+                for (int t = r0 + w; t < r1; t += 8 * NI) {
+                    float ss[NI] = {};
+                    for (int jl = lane; jl < nf; jl += 32) {
+                        const int n = f0 + jl;
+                        const bool in = n < a.d;
+                        const bool first = t == w && jl == lane;
+                        if (!first) res_load(t, n, in);
+                        const float g = jl == lane ? gain0 : (in ? __bfloat162float(gain[n]) : 0.f);
+#pragma unroll
+                        for (int q = 0; q < NI; ++q) {
+                            const int tt = t + 8 * q;
+                            if (in && tt < r1) {
+                                const float y = yv(tt - r0, 0, jl) + hid[q];
+                                a.hidden[(size_t)tt * a.d + n] = y;
+                                store_terms(y * g, a.x_d + (size_t)tt * terms * a.d + n, a.d, terms);
+                                ss[q] += y * y;
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                        for (int q = 0; q < NI; ++q) ss[q] += __shfl_xor_sync(0xffffffffu, ss[q], o);
+#pragma unroll
+                    for (int q = 0; q < NI; ++q)
+                        if (lane == q && t + 8 * q < r1) sq[(size_t)tile * TC_X_ROWS + t + 8 * q] = ss[q];
+                }
+            }
+            if (r1 < T || tile + n_cta < f.n_tiles) bar_n(1, FW_EPI);       // Y is rewritten by the next rows or tile
+        }
+    }
+    return true;
+}
 
 template <int HD, int NQP>
 __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_constant__ FwArgs a) {
@@ -144,8 +425,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     constexpr uint32_t KV_BYTES = FW_KEYS * HD * 2;
     constexpr int Q_BYTES = NQ2 * HD * 2;              // one query tile
     constexpr int P_BYTES = NQ2 * FW_KEYS * 2;         // one probability tile
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* uni = smem + (size_t)NS * FW_SLOT;
     FwTail& s = *reinterpret_cast<FwTail*>(uni + FW_UNION);
     float* Y = reinterpret_cast<float*>(uni);
@@ -155,13 +435,21 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     const int cta = (int)blockIdx.x, n_cta = a.n_cta;
     const int T = a.T, cols = a.cols, terms = a.terms;
     const int n_phases = 5 * a.n_layers + 1;
+    for (int b = threadIdx.x; b < a.B; b += FW_THREADS) {
+        SeqMeta m;
+        m.nrows = __ldcg(a.rm.n_rows + b);
+        m.L = __ldcg(a.rm.kv_base + b);
+        m.nkeys = min(m.L + __ldcg(a.rm.n_spec + b), a.pieces * FW_KEYS);
+        m.seq = __ldcg(a.rm.call_seq + b);
+        s.meta[b] = m;
+    }
     if (threadIdx.x == 0) {
         for (int i = 0; i < NS; ++i) {
             mbar_init(smem_u32(&s.full[i]), 1);
-            mbar_init(smem_u32(&s.empty[i]), 1);
+            mbar_init(smem_u32(&s.empty[i]), 2);       // both MMA warps
         }
         for (int i = 0; i < 2; ++i) {
-            mbar_init(smem_u32(&s.tfull[i]), 1);
+            mbar_init(smem_u32(&s.tfull[i]), 2);
             mbar_init(smem_u32(&s.tempty[i]), 8);
             mbar_init(smem_u32(&s.sfull[i]), 1);
             mbar_init(smem_u32(&s.pfull[i]), 4);
@@ -173,13 +461,6 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         s.abort_flag[1] = (int)(a.wait_limit ? a.wait_limit : WAIT_LIMIT);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        int run = 0;
-        for (int b = 0; b < a.B; ++b) {
-            s.pref[b] = run;
-            const int nk = min(__ldcg(a.rm.kv_base + b) + __ldcg(a.rm.n_spec + b), a.pieces * FW_KEYS);
-            if (__ldcg(a.rm.n_rows + b) > 0) run += (nk + FW_KEYS - 1) / FW_KEYS * a.Hkv;
-        }
-        s.pref[a.B] = run;
     }
     if (warp == 3) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s.tmem_ptr)), "r"(512)
@@ -191,14 +472,16 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     tc_fence_after();
     const uint32_t tmem = s.tmem_ptr;
     volatile int* abort_flag = s.abort_flag;
-    const int a_tot = s.pref[a.B];
-    const int a_per = (a_tot + n_cta - 1) / n_cta;
-    const int a_lo = min(cta * a_per, a_tot), a_hi = min(a_lo + a_per, a_tot), a_n = a_hi - a_lo;
-    auto slot_ptr = [&](int pos) { return smem_u32(smem + (size_t)(pos % NS) * FW_SLOT); };
+    int a_tot = 0;
+    for (int b = 0; b < a.B; ++b) a_tot += attn_tiles(s.meta[b]) * a.Hkv;
+    const int a_per = max(1, (a_tot + n_cta - 1) / n_cta);
+    const int a_lo = min(cta * a_per, a_tot), a_n = min(a_lo + a_per, a_tot) - a_lo;
+    const AttnPos a_first = attn_find(s.meta, a.B, a.Hkv, a_lo);
+    auto slot_ptr = [&](int pos) { return smem_u32(smem) + (uint32_t)(pos % NS) * FW_SLOT; };
     auto full_bar = [&](int pos) { return smem_u32(&s.full[pos % NS]); };
     auto empty_bar = [&](int pos) { return smem_u32(&s.empty[pos % NS]); };
     auto ring_par = [&](int pos) { return (uint32_t)(pos / NS) & 1u; };
-    // kind of phase p and its layer
+    // kind of phase p
     auto kind_of = [&](int p) { return p == n_phases - 1 ? (int)FW_LM : p % 5; };
 
     if (warp == 0) {
@@ -212,11 +495,11 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 const FwLayer* L = a.layers + layer;
                 if (kind == FW_ATTN) {
                     bool waited = false;
-                    for (int x = a_lo; x < a_hi && ok; ++x) {
-                        const AttnItem it = attn_item(s.pref, a.Hkv, x);
-                        const int seq = __ldcg(a.rm.call_seq + it.bi);
-                        const int plane = ((layer * a.max_batch + seq) * 2) * a.Hkv + it.g;
-                        if (!waited && (it.tile + 1) * FW_KEYS > __ldcg(a.rm.kv_base + it.bi)) {
+                    AttnPos it = a_first;
+                    for (int i = 0; i < a_n && ok; ++i, attn_next(it, s.meta, a.B, a.Hkv)) {
+                        const SeqMeta sm = s.meta[it.bi];
+                        const int plane = ((layer * a.max_batch + sm.seq) * 2) * a.Hkv + it.g;
+                        if (!waited && (it.tile + 1) * FW_KEYS > sm.L) {
                             ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
                             proxy_fence();
                             waited = true;
@@ -305,113 +588,130 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     }
             }
         }
-    } else if (warp == 2) {
-        // ---------------- MMA issuer (the whole warp runs the loop, see tc_mma_one)
-        {
-            const uint32_t one = elect_one();
-            constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (8u << 24);      // bf16 x bf16 -> fp32, M = 128
-            int pos = 0, tcount = 0, at = 0, as = 0;   // ring position, projection tiles, attention tiles, segments so far
-            bool ok = true;
-            for (int p = 0; p < n_phases && ok; ++p) {
-                const int kind = kind_of(p);
-                if (kind == FW_ATTN) {
+    } else if (warp < FW_EPI_WARP0) {
+        // ---------------- MMA issuers, warps 2 and 3 (the whole warp runs the loop, see tc_mma_one).  In a projection they
+        // share out the boxes, or (one box, room for two accumulators) the MMAs along k; in the attention warp 2 forms the
+        // scores and warp 3 the outputs.  Every slot of the ring is released by both, or twice by the one that used it.
+        constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (8u << 24);      // bf16 x bf16 -> fp32, M = 128
+        const uint32_t one = elect_one();
+        const int me = warp - 2;
+        int pos = 0, tcount = 0, at = 0, as = 0;       // ring position, projection tiles, attention tiles, segments so far
+        bool ok = true;
+        for (int p = 0; p < n_phases && ok; ++p) {
+            const int kind = kind_of(p);
+            if (kind == FW_ATTN) {
+                if (me == 0) {
                     constexpr uint32_t idesc_s = IDESC | ((uint32_t)(NQ2 >> 3) << 17);
-                    constexpr uint32_t idesc_o = IDESC | (1u << 15) | ((uint32_t)(NQ2 >> 3) << 17);
-                    // scores of the block's tile i
-                    auto scores = [&](int i) -> bool {
-                        const AttnItem it = attn_item(s.pref, a.Hkv, a_lo + i);
+                    AttnPos it = a_first;
+                    for (int i = 0; i < a_n; ++i, attn_next(it, s.meta, a.B, a.Hkv)) {
                         const bool fresh = i == 0 || it.tile == 0;
                         if (fresh && i > 0) ++as;
-                        if (fresh && !mbar_wait_warp(smem_u32(&s.qfull[as & 1]), (uint32_t)(as >> 1) & 1u, abort_flag)) return false;
                         const int kpos = pos + 2 * i, b = (at + i) & 1;
-                        if (!mbar_wait_warp(full_bar(kpos), ring_par(kpos), abort_flag)) return false;
+                        // query rows of the segment, the K tile, and the score buffer (read by the softmax two tiles ago)
+                        ok = (!fresh || mbar_wait_warp(smem_u32(&s.qfull[as & 1]), (uint32_t)(as >> 1) & 1u, abort_flag)) &&
+                             mbar_wait_warp(full_bar(kpos), ring_par(kpos), abort_flag) &&
+                             mbar_wait_warp(smem_u32(&s.pfull[b]), ((uint32_t)((at + i) >> 1) & 1u) ^ 1u, abort_flag);
+                        if (!ok) break;
                         tc_fence_after();
-                        const uint32_t ka = slot_ptr(kpos), qa = smem_u32(Qs + (as & 1) * Q_BYTES);
+                        const uint64_t ka = smem_desc(slot_ptr(kpos)), qa = smem_desc(smem_u32(Qs) + (as & 1) * Q_BYTES);
 #pragma unroll
                         for (int ks = 0; ks < HD / 16; ++ks)
-                            tc_mma_one(one, tmem + b * 64, smem_desc(ka + (ks >> 2) * (FW_KEYS * 128) + (ks & 3) * 32),
-                                   smem_desc(qa + (ks >> 2) * (NQ2 * 128) + (ks & 3) * 32), idesc_s, ks > 0 ? 1u : 0u);
+                            tc_mma_one(one, tmem + b * 64, ka + (ks >> 2) * (FW_KEYS * 8) + (ks & 3) * 2,
+                                       qa + (ks >> 2) * (NQ2 * 8) + (ks & 3) * 2, idesc_s, ks > 0 ? 1u : 0u);
                         tc_commit_one(one, smem_u32(&s.sfull[b]));
                         tc_commit_one(one, empty_bar(kpos));
-                        return true;
-                    };
-                    if (a_n > 0) ok = scores(0);
-                    for (int i = 0; i < a_n && ok; ++i) {
-                        // the next scores go ahead of this tile's output, except across segments: the next segment's query
-                        // rows are loaded once this segment has ended
-                        const bool more = i + 1 < a_n, ahead = more && attn_item(s.pref, a.Hkv, a_lo + i + 1).tile != 0;
-                        if (ahead) ok = scores(i + 1);
-                        if (!ok) break;
+                        tc_commit_one(one, empty_bar(kpos));
+                    }
+                    if (a_n > 0) ++as;
+                } else {
+                    constexpr uint32_t idesc_o = IDESC | (1u << 15) | ((uint32_t)(NQ2 >> 3) << 17);
+                    for (int i = 0; i < a_n; ++i) {
                         const int vpos = pos + 2 * i + 1, b = (at + i) & 1;
                         const uint32_t par = (uint32_t)((at + i) >> 1) & 1u;
-                        ok = mbar_wait_warp(smem_u32(&s.pfull[b]), par, abort_flag) && mbar_wait_warp(full_bar(vpos), ring_par(vpos), abort_flag) &&
+                        ok = mbar_wait_warp(smem_u32(&s.pfull[b]), par, abort_flag) &&
+                             mbar_wait_warp(full_bar(vpos), ring_par(vpos), abort_flag) &&
                              mbar_wait_warp(smem_u32(&s.oempty[b]), par ^ 1u, abort_flag);
                         if (!ok) break;
                         tc_fence_after();
-                        const uint32_t va = slot_ptr(vpos), pa = smem_u32(Ps + b * P_BYTES);
+                        const uint64_t va = smem_desc_mn(slot_ptr(vpos)), pa = smem_desc(smem_u32(Ps) + b * P_BYTES);
 #pragma unroll
                         for (int ks = 0; ks < FW_KEYS / 16; ++ks)
-                            tc_mma_one(one, tmem + FW_TM_D + b * 64, smem_desc_mn(va + ks * 2048),
-                                   smem_desc(pa + (ks >> 2) * (NQ2 * 128) + (ks & 3) * 32), idesc_o, ks > 0 ? 1u : 0u);
+                            tc_mma_one(one, tmem + FW_TM_D + b * 64, va + ks * 128, pa + (ks >> 2) * (NQ2 * 8) + (ks & 3) * 2,
+                                       idesc_o, ks > 0 ? 1u : 0u);
                         tc_commit_one(one, smem_u32(&s.ofull[b]));
                         tc_commit_one(one, empty_bar(vpos));
-                        if (more && !ahead) ok = scores(i + 1);
+                        tc_commit_one(one, empty_bar(vpos));
                     }
-                    if (a_n > 0) ++as;
-                    at += a_n;
-                    pos += 2 * a_n;
-                    continue;
                 }
-                const FwPhase& f = a.ph[kind];
-                const int groups = f.kb / f.S, sc = f.S * cols;      // MMAs along k, accumulator columns of a box
-                const uint32_t idesc = IDESC | ((uint32_t)((f.S * cols) >> 3) << 17);
-                for (int tile = cta; tile < f.n_tiles && ok; tile += n_cta, ++tcount) {
-                    const int buf = tcount & 1;
-                    ok = mbar_wait_warp(smem_u32(&s.tempty[buf]), ((uint32_t)(tcount >> 1) & 1u) ^ 1u, abort_flag);
+                at += a_n;
+                pos += 2 * a_n;
+                continue;
+            }
+            const FwPhase& f = a.ph[kind];
+            const int groups = f.kb / f.S, sc = f.S * cols, nbox = f.nbox;      // MMAs along k, accumulator columns of a box
+            const bool dual = f.dual != 0;
+            const uint32_t idesc = IDESC | ((uint32_t)(sc >> 3) << 17);
+            const uint32_t a_step = f.S * f.hr * 8, b_step = sc * 8;            // 16-byte units
+            for (int tile = cta; tile < f.n_tiles && ok; tile += n_cta, ++tcount) {
+                const int buf = tcount & 1;
+                ok = mbar_wait_warp(smem_u32(&s.tempty[buf]), ((uint32_t)(tcount >> 1) & 1u) ^ 1u, abort_flag);
+                if (!ok) break;
+                tc_fence_after();
+                const bool mine = me == 0 || nbox == 2 || dual;
+                const uint32_t d = tmem + buf * 256 + me * sc;
+                uint32_t acc = 0;
+                int turn = 0;                              // dual: MMAs along k alternate between the warps
+                for (int step = 0; step < f.steps; ++step, ++pos) {
+                    ok = mbar_wait_warp(full_bar(pos), ring_par(pos), abort_flag);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t d = tmem + buf * 256;
-                    for (int step = 0; step < f.steps; ++step, ++pos) {
-                        ok = mbar_wait_warp(full_bar(pos), ring_par(pos), abort_flag);
-                        if (!ok) break;
-                        tc_fence_after();
+                    if (mine) {
                         const uint32_t base = slot_ptr(pos);
-                        uint64_t ad = smem_desc(base), bd = smem_desc(base + f.b_off);      // (addresses in 16-byte units)
-                        for (int gr = 0; gr < groups; ++gr, ad += f.S * f.hr * 8, bd += sc * 8)
-                            for (int q = 0; q < f.nbox; ++q)
+                        uint64_t ad = smem_desc(base), bd = smem_desc(base + f.b_off);
+                        if (nbox == 2) ad += (uint32_t)(me * f.box_bytes) >> 4;
+                        for (int gr = 0; gr < groups; ++gr, ad += a_step, bd += b_step) {
+                            if (dual) {
+                                turn ^= 1;
+                                if (turn == me) continue;
+                            }
 #pragma unroll
-                                for (int k4 = 0; k4 < TC_TILE_K / 16; ++k4)
-                                    tc_mma_one(one, d + q * sc, ad + (uint32_t)(q * f.box_bytes / 16 + k4 * 2), bd + k4 * 2, idesc,
-                                               (step > 0 || gr > 0 || k4 > 0) ? 1u : 0u);
-                        tc_commit_one(one, empty_bar(pos));
+                            for (int k4 = 0; k4 < TC_TILE_K / 16; ++k4) {
+                                tc_mma_one(one, d, ad + k4 * 2, bd + k4 * 2, idesc, acc);
+                                acc = 1u;
+                            }
+                        }
                     }
-                    if (ok) tc_commit_one(one, smem_u32(&s.tfull[buf]));
+                    tc_commit_one(one, empty_bar(pos));
                 }
+                if (ok) tc_commit_one(one, smem_u32(&s.tfull[buf]));
             }
         }
-    } else if (warp >= FW_EPI_WARP0) {
+    } else {
         // ---------------- epilogue warps
         const int e = threadIdx.x - 32 * FW_EPI_WARP0;   // 0..255
-        const int w = warp - FW_EPI_WARP0;                // 0..7
-        const int quad = warp & 3, half = w >> 2;         // TMEM lane quadrant; which of the quadrant's two warps
+        const int quad = warp & 3, half = (warp - FW_EPI_WARP0) >> 2;     // TMEM lane quadrant; which of its two warps
         const uint32_t t_lane = tmem + ((uint32_t)(quad * 32) << 16);
         int tcount = 0, at = 0, as = 0, pos = 0;
         bool ok = true;
+        auto steps_of = [&](const FwPhase& f) { return cta < f.n_tiles ? ((f.n_tiles - 1 - cta) / n_cta + 1) * f.steps : 0; };
+        const int ring_other = steps_of(a.ph[FW_O]) + steps_of(a.ph[FW_GATEUP]) + steps_of(a.ph[FW_DOWN]);
+        const int ring_qkv = steps_of(a.ph[FW_QKV]);
         for (int p = 0; p < n_phases && ok; ++p) {
             const int kind = kind_of(p), layer = p / 5;
             if (kind == FW_ATTN) {
                 if (e == 0) ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
                 ok = all_of(1, FW_EPI, ok);
                 if (!ok) break;
+                pos += ring_qkv;
                 const int G = a.Hq / a.Hkv, kl = quad * 32 + lane;    // this thread's key of a tile, or its head dimension
                 float m[NQP], l[NQP], acc[NQP];
-                for (int x = a_lo; x < a_hi; ++x) {
-                    const AttnItem it = attn_item(s.pref, a.Hkv, x);
-                    const int nrows = __ldcg(a.rm.n_rows + it.bi), L = __ldcg(a.rm.kv_base + it.bi);
-                    const int nkeys = min(L + __ldcg(a.rm.n_spec + it.bi), a.pieces * FW_KEYS);
+                AttnPos it = a_first;
+                for (int i = 0; i < a_n; ++i) {
+                    const SeqMeta sm = s.meta[it.bi];
+                    const int nrows = sm.nrows, L = sm.L, nkeys = sm.nkeys;
                     const int n_q = min(G * nrows, NQP);
-                    const int t0 = it.bi * a.R, h0 = it.g * G;        // query row i: row t0 + i % nrows, head h0 + i / nrows
-                    const bool fresh = x == a_lo || it.tile == 0;
+                    const int t0 = it.bi * a.R, h0 = it.g * G;        // query row r: row t0 + r % nrows, head h0 + r / nrows
+                    const bool fresh = i == 0 || it.tile == 0;
                     const int b = at & 1;
                     const uint32_t par = (uint32_t)(at >> 1) & 1u;
                     if (fresh) {
@@ -422,18 +722,35 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         // -------- softmax: a lane per key
                         if (fresh) {
                             uint8_t* q = Qs + (as & 1) * Q_BYTES;
-                            for (int i = kl; i < NQ2 * (HD / 8); i += 128) {
-                                const int row = i / (HD / 8), c = i % (HD / 8), r = row & (NQP - 1);
+#pragma unroll
+                            for (int x = 0; x < NQ2 * (HD / 8) / 128; ++x) {
+                                const int idx = kl + x * 128, row = idx / (HD / 8), c = idx % (HD / 8), r = row & (NQP - 1);
                                 const bool valid = r < n_q;
-                                const int rr = valid ? r : 0;
+                                const int rr = valid ? r : 0, hq = G == 1 ? 0 : rr / nrows;
                                 const __nv_bfloat16* src = (row >= NQP ? a.q_lo : a.q_hi) +
-                                    ((size_t)(t0 + rr % nrows) * a.Hq + h0 + rr / nrows) * HD + c * 8;
+                                    ((size_t)(t0 + rr - hq * nrows) * a.Hq + h0 + hq) * HD + c * 8;
                                 cp_async16(smem_u32(q + (c >> 3) * (NQ2 * 128) + row * 128 + (((c & 7) ^ (row & 7)) << 4)), src, valid);
                             }
                             asm volatile("cp.async.wait_all;" ::: "memory");
                             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                             __syncwarp();
                             if (lane == 0) mbar_arrive(smem_u32(&s.qfull[as & 1]));
+                        }
+                        const int j = it.tile * FW_KEYS + kl;
+                        // which query rows see this thread's key: all of a committed one; of a draft row those that have it
+                        // among their ancestors and themselves; none past the last key
+                        uint32_t vis = 0xffffffffu;
+                        if ((it.tile + 1) * FW_KEYS > L) {
+                            const int sr = j - L;
+                            vis = j < nkeys ? 0xffffffffu : 0u;
+                            if (sr >= 0 && vis) {
+                                vis = 0;
+#pragma unroll
+                                for (int r = 0; r < NQP; ++r) {
+                                    const int rr = r < n_q ? (G == 1 ? r : r % nrows) : 0;
+                                    vis |= ((a.rm.mask[(size_t)(t0 + rr) * MTAD_MASK_WORDS + (sr >> 5)] >> (sr & 31)) & 1u) << r;
+                                }
+                            }
                         }
                         ok = warp_wait(smem_u32(&s.sfull[b]), par, abort_flag, ok, lane);
                         tc_fence_after();
@@ -443,19 +760,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             if (NQ2 == 16) tc_ld16(t_lane + b * 64, c);
                             else { tc_ld16(t_lane + b * 64, c); tc_ld16(t_lane + b * 64 + 16, c + 16); }
 #pragma unroll
-                            for (int r = 0; r < NQP; ++r) v[r] = c[r] + c[NQP + r];
-                        }
-                        const int j = it.tile * FW_KEYS + kl;
-                        if ((it.tile + 1) * FW_KEYS > L) {
-                            // the tile reaches into the draft rows: ancestors and self only, nothing past the last key
-                            const int sr = j - L;
-#pragma unroll
-                            for (int r = 0; r < NQP; ++r) {
-                                bool vis = j < nkeys && r < n_q;
-                                if (vis && sr >= 0)
-                                    vis = (a.rm.mask[(size_t)(t0 + r % nrows) * MTAD_MASK_WORDS + (sr >> 5)] >> (sr & 31)) & 1u;
-                                if (!vis) v[r] = -CUDART_INF_F;
-                            }
+                            for (int r = 0; r < NQP; ++r) v[r] = ((vis >> r) & 1u) ? c[r] + c[NQP + r] : -CUDART_INF_F;
                         }
                         float wm[NQP];
 #pragma unroll
@@ -476,8 +781,9 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         for (int r = 0; r < NQP; ++r) {
                             const float4 q4 = *reinterpret_cast<const float4*>(s.smx[b][r]);
                             const float mn = fmaxf(m[r], fmaxf(fmaxf(q4.x, q4.y), fmaxf(q4.z, q4.w)));
-                            const float f = mn == -CUDART_INF_F ? 1.f : exp2f(m[r] - mn);
-                            const float pv = mn == -CUDART_INF_F ? 0.f : exp2f(v[r] - mn);      // exp2(-inf) = 0
+                            const float mz = mn == -CUDART_INF_F ? 0.f : mn;
+                            const float f = exp2f(m[r] - mz);                                   // exp2(-inf) = 0
+                            const float pv = exp2f(v[r] - mz);
                             m[r] = mn;
                             l[r] = l[r] * f + pv;
                             if (kl == r) s.sf[b][r] = f;
@@ -488,7 +794,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         }
                         if ((it.tile + 1) * FW_KEYS > nkeys) {
                             // rows of V past the last key: their probabilities are 0, but 0 x (stale value) must not make a NaN
-                            const int vpos = pos + 2 * (x - a_lo) + 1;
+                            const int vpos = pos + 2 * i + 1;
                             ok = warp_wait(full_bar(vpos), ring_par(vpos), abort_flag, ok, lane);
                             if (ok && j >= nkeys) {
                                 uint8_t* vs = smem + (size_t)(vpos % NS) * FW_SLOT + kl * 128;
@@ -515,7 +821,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         if (lane == 0) mbar_arrive(smem_u32(&s.oempty[b]));
                     }
                     ++at;
-                    if (x + 1 == a_hi || it.tile + 1 == it.nt) {
+                    if (i + 1 == a_n || it.tile + 1 == it.nt) {
                         // -------- end of a segment: the row sums meet, then the rows leave (final, or as a piece)
                         const int sb = as & 1;
                         if (half == 0) {
@@ -529,13 +835,13 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                                 if (kl == r) s.sm[sb][r] = m[r];
                             }
                         }
-                        ok = all_of(1, FW_EPI, ok);
                         const int first = it.f0 / a_per, n_piece = (it.f0 + it.nt - 1) / a_per - first + 1, piece = cta - first;
-                        if (half == 1 && ok) {
+                        ok = all_of(1, FW_EPI, ok);
+                        if (half == 1 && ok && (HD == 128 || kl < HD)) {
 #pragma unroll
                             for (int r = 0; r < NQP; ++r) {
-                                if (r >= n_q || (HD < 128 && kl >= HD)) continue;
-                                const int t = t0 + r % nrows, h = h0 + r / nrows;
+                                if (r >= n_q) continue;
+                                const int hq = G == 1 ? 0 : r / nrows, t = t0 + r - hq * nrows, h = h0 + hq;
                                 const float ls = (s.sl[sb][0][r] + s.sl[sb][1][r]) + (s.sl[sb][2][r] + s.sl[sb][3][r]);
                                 if (n_piece == 1) {
                                     store_terms(acc[r] / ls, a.x_a + (size_t)t * terms * a.Hq * HD + (size_t)h * HD + kl,
@@ -550,288 +856,87 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         }
                         ++as;
                     }
+                    if (i + 1 < a_n) attn_next(it, s.meta, a.B, a.Hkv);
                 }
-                pos += 2 * a_n;
+                pos += 2 * a_n + ring_other;
                 // pieces shared with other blocks (at most the first and the last segment): the last to arrive merges
                 if (a_n > 0) {
-                    const AttnItem i0 = attn_item(s.pref, a.Hkv, a_lo), i1 = attn_item(s.pref, a.Hkv, a_hi - 1);
-                    const bool two = i1.f0 != i0.f0;
                     ok = all_of(1, FW_EPI, ok);
                     if (!ok) break;
                     if (e < 2) {
-                        const AttnItem it = e == 0 ? i0 : i1;
-                        const int n_piece = (it.f0 + it.nt - 1) / a_per - it.f0 / a_per + 1;
+                        const AttnPos q = e == 0 ? a_first : it;
+                        const int n_piece = (q.f0 + q.nt - 1) / a_per - q.f0 / a_per + 1;
                         int last = 0;
-                        if (n_piece > 1 && (e == 0 || two)) {
+                        if (n_piece > 1 && (e == 0 || it.f0 != a_first.f0)) {
                             int old;
                             asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;"
-                                         : "=r"(old) : "l"(a.acnt + it.bi * a.Hkv + it.g) : "memory");
+                                         : "=r"(old) : "l"(a.acnt + q.bi * a.Hkv + q.g) : "memory");
                             last = old + 1 == n_piece;
                         }
                         s.last[e] = last;
                     }
                     bar_n(1, FW_EPI);
-                    for (int q = 0; q < 2; ++q) {
-                        if (!s.last[q]) continue;
-                        const AttnItem it = q == 0 ? i0 : i1;
-                        const int nrows = __ldcg(a.rm.n_rows + it.bi), n_q = min(G * nrows, NQP);
-                        const int n_piece = (it.f0 + it.nt - 1) / a_per - it.f0 / a_per + 1;
+                    for (int x = 0; x < 2; ++x) {
+                        if (!s.last[x]) continue;
+                        const AttnPos q = x == 0 ? a_first : it;
+                        const int nrows = s.meta[q.bi].nrows, n_q = min(G * nrows, NQP);
+                        const int n_piece = (q.f0 + q.nt - 1) / a_per - q.f0 / a_per + 1;
                         for (int i = e; i < n_q * (HD / 4); i += FW_EPI) {
                             const int r = i / (HD / 4), c4 = i % (HD / 4);
-                            const int t = it.bi * a.R + r % nrows, h = it.g * G + r / nrows;
+                            const int hq = G == 1 ? 0 : r / nrows, t = q.bi * a.R + r - hq * nrows, h = q.g * G + hq;
                             const size_t o = ((size_t)t * a.Hq + h) * a.pieces;
                             const float2* ml = reinterpret_cast<const float2*>(a.part + (size_t)T * a.Hq * a.pieces * HD) + o;
                             const float4* po = reinterpret_cast<const float4*>(a.part + o * HD) + c4;
-                            // pieces in order (deterministic), four at a time: their loads are in flight together
+                            // pieces in order (deterministic), six at a time: their loads are in flight together
+                            constexpr int NP = 6;
                             float M = -CUDART_INF_F, ls = 0.f;
                             float4 o4 = make_float4(0.f, 0.f, 0.f, 0.f);
-                            for (int k0 = 0; k0 < n_piece; k0 += 4) {
-                                float2 v[4];
-                                float4 y[4];
+                            for (int k0 = 0; k0 < n_piece; k0 += NP) {
+                                float2 v[NP];
+                                float4 y[NP];
 #pragma unroll
-                                for (int k = 0; k < 4; ++k) {
+                                for (int k = 0; k < NP; ++k) {
                                     const int kk = min(k0 + k, n_piece - 1);
                                     v[k] = __ldcg(ml + kk);
                                     y[k] = __ldcg(po + (size_t)kk * (HD / 4));
                                     if (k0 + k >= n_piece) v[k].x = -CUDART_INF_F;
                                 }
-                                const float mn = fmaxf(M, fmaxf(fmaxf(v[0].x, v[1].x), fmaxf(v[2].x, v[3].x)));
-                                const float fo = mn == -CUDART_INF_F ? 1.f : exp2f(M - mn);
+                                float mn = M;
+#pragma unroll
+                                for (int k = 0; k < NP; ++k) mn = fmaxf(mn, v[k].x);
+                                const float mz = mn == -CUDART_INF_F ? 0.f : mn;
+                                const float fo = exp2f(M - mz);
                                 ls *= fo;
                                 o4.x *= fo; o4.y *= fo; o4.z *= fo; o4.w *= fo;
                                 M = mn;
 #pragma unroll
-                                for (int k = 0; k < 4; ++k) {
-                                    const float wg = v[k].x == -CUDART_INF_F ? 0.f : exp2f(v[k].x - mn);
-                                    ls += wg * v[k].y;
-                                    o4.x += wg * y[k].x; o4.y += wg * y[k].y; o4.z += wg * y[k].z; o4.w += wg * y[k].w;
+                                for (int k = 0; k < NP; ++k) {
+                                    const float wg = exp2f(v[k].x - mz);
+                                    if (wg != 0.f) {
+                                        ls += wg * v[k].y;
+                                        o4.x += wg * y[k].x; o4.y += wg * y[k].y; o4.z += wg * y[k].z; o4.w += wg * y[k].w;
+                                    }
                                 }
                             }
                             const float f = 1.f / ls;
                             store_terms4(make_float4(o4.x * f, o4.y * f, o4.z * f, o4.w * f),
                                          a.x_a + (size_t)t * terms * a.Hq * HD + (size_t)h * HD + c4 * 4, (size_t)a.Hq * HD, terms);
                         }
-                        if (e == 0) a.acnt[it.bi * a.Hkv + it.g] = 0;     // ready for the next layer
+                        if (e == 0) a.acnt[q.bi * a.Hkv + q.g] = 0;       // ready for the next layer
                     }
                 }
+            } else if (kind == FW_QKV) {
+                ok = epi_phase<FW_QKV, HD>(a, s, Y, p, layer, tcount, e, t_lane, cta);
+            } else if (kind == FW_O) {
+                ok = epi_phase<FW_O, HD>(a, s, Y, p, layer, tcount, e, t_lane, cta);
+            } else if (kind == FW_GATEUP) {
+                ok = epi_phase<FW_GATEUP, HD>(a, s, Y, p, layer, tcount, e, t_lane, cta);
+            } else if (kind == FW_DOWN) {
+                ok = epi_phase<FW_DOWN, HD>(a, s, Y, p, layer, tcount, e, t_lane, cta);
             } else {
-                const FwPhase& f = a.ph[kind];
-                const FwLayer* L = a.layers + layer;
-                const int mine = cta < f.n_tiles ? (f.n_tiles - 1 - cta) / n_cta + 1 : 0;
-                const int yb = f.S * f.hr;                             // columns of Y that a box takes
-                const int ys = f.nbox * yb + 4;                        // row stride of Y
-                const int nf = kind == FW_LM ? f.nbox * f.h : f.h;     // features (pairs) of a tile
-                // rows that Y holds at a time, in whole drain groups
-                const int per = terms == 3 ? 5 : 8, blk = min((T + per - 1) / per, FW_UNION / (per * ys * 4)) * per;
-                if (mine > 0 && (kind == FW_QKV || kind == FW_GATEUP || kind == FW_LM)) {
-                    // scale of the deferred RMSNorm: the rows' sums of squares come from every block
-                    if (p > 0) {
-                        if (e == 0) ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
-                        ok = all_of(1, FW_EPI, ok);
-                        if (!ok) break;
-                    }
-                    const float* sq = kind == FW_GATEUP ? a.sumsq_b : a.sumsq_a;
-                    const int parts = kind == FW_GATEUP ? a.ph[FW_O].n_tiles : (p == 0 ? a.parts0 : a.ph[FW_DOWN].n_tiles);
-                    for (int r = w; r < T; r += 8) {
-                        float v = 0.f;
-                        for (int q = lane; q < parts; q += 32) v += __ldcg(sq + (size_t)q * TC_X_ROWS + r);
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                        if (lane == 0) s.rstd[r] = rsqrtf(v * a.inv_dim + a.eps);
-                    }
-                }
-                pos += mine * f.steps;
-                for (int tile = cta; tile < f.n_tiles; tile += n_cta, ++tcount) {
-                    const int buf = tcount & 1, f0 = tile * nf;            // first feature (O, down, gate / up, LM head)
-                    // what the first items of this thread need besides the accumulator, requested ahead of it
-                    float pre[4] = {0.f, 0.f, 0.f, 0.f};
-                    float u8[8], gn[4] = {0.f, 0.f, 0.f, 0.f};
-                    float2 cs2[2] = {};
-                    int sl2[2] = {-1, -1}, sq2[2] = {};
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) u8[i] = 0.5f;
-                    if (kind == FW_O || kind == FW_DOWN) {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const int n = f0 + lane + 32 * i;
-                            if (w < T && lane + 32 * i < nf && n < a.d) pre[i] = __ldcg(a.hidden + (size_t)w * a.d + n);
-                            if (lane + 32 * i < nf && n < a.d) gn[i] = __bfloat162float((kind == FW_O ? L->gain_ffn : L->gain_next)[n]);
-                        }
-                    } else if (kind == FW_QKV) {
-                        const int j0 = (tile % f.u) * f.h;
-#pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            const int i = e + q * FW_EPI, t = i / nf, jj = j0 + i % nf;
-                            if (t < T && jj < HD / 2) {
-                                cs2[q] = *reinterpret_cast<const float2*>(a.rope + ((size_t)t * (HD / 2) + jj) * 2);
-                                sl2[q] = a.rm.slot[t];
-                                sq2[q] = a.rm.seq[t];
-                            }
-                        }
-                    } else if (kind == FW_LM && !a.lm_plain) {
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const int n = f0 + lane + 32 * i;
-                            if (w < T && lane + 32 * i < nf && n < a.V) u8[i] = a.uniforms[(size_t)(w / a.R) * a.V + n];
-                        }
-                    }
-                    // (one thread polls: 256 of them would take the shared-memory pipe away from the copies' barriers)
-                    if (e == 0) ok = mbar_wait(smem_u32(&s.tfull[buf]), (uint32_t)(tcount >> 1) & 1u, abort_flag);
-                    ok = all_of(1, FW_EPI, ok);
-                    if (!ok) break;
-                    tc_fence_after();
-                    for (int r0 = 0; r0 < T; r0 += blk) {
-                    const int r1 = min(T, r0 + blk);
-                    {   // accumulators -> Y[row][box][lane], the terms of a row added up; a lane's slice of the S k-blocks that
-                        // the MMA takes side by side is lane / hr, and a warp's 32 lanes may lie in several slices
-                        const uint32_t t_acc = t_lane + buf * 256;
-                        const int ng = (r1 - r0 + per - 1) / per, tl = quad * 32 + lane, my = tl / f.hr;
-                        const int s0 = f.S > 1 ? quad * 32 / f.hr : 0, s1 = f.S > 1 ? min(f.S - 1, (quad * 32 + 31) / f.hr) : 0;
-                        for (int i = half; i < f.nbox * ng; i += 2) {
-                            const int q = i / ng, rb = r0 + (i - q * ng) * per;
-                            for (int sl = s0; sl <= s1; ++sl) {
-                                float v[16];
-                                tc_ld16(t_acc + (q * f.S + sl) * cols + rb * terms, v);
-                                if (my == sl && tl < yb) {
-                                    float* y = Y + (rb - r0) * ys + q * yb + tl;
-                                    if (terms == 3) {
-#pragma unroll
-                                        for (int j = 0; j < 5; ++j)
-                                            if (rb + j < r1) y[j * ys] = v[3 * j] + (v[3 * j + 1] + v[3 * j + 2]);
-                                    } else {
-#pragma unroll
-                                        for (int j = 0; j < 8; ++j)
-                                            if (rb + j < r1) y[j * ys] = v[2 * j] + v[2 * j + 1];
-                                    }
-                                }
-                                __syncwarp();
-                            }
-                        }
-                    }
-                    if (r1 == T) {
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&s.tempty[buf]));
-                    }
-                    ok = all_of(1, FW_EPI, ok);
-                    if (!ok) break;
-                    // value of (row, box, weight row): the S slices lie side by side
-                    auto yv = [&](int t, int q, int row) -> float {
-                        const float* y = Y + (t - r0) * ys + q * yb + row;
-                        float v = y[0];
-                        for (int sl = 1; sl < f.S; ++sl) v += y[sl * f.hr];
-                        return v;
-                    };
-                    const int nr = r1 - r0;
-                    if (kind == FW_QKV) {
-                        const int hp = HD / 2;
-                        const float scale = rsqrtf((float)HD);
-                        const int hg = tile / f.u, j0 = (tile - hg * f.u) * f.h;
-                        for (int i = e; i < nr * nf; i += FW_EPI) {
-                            const int t = r0 + i / nf, j = i % nf, jj = j0 + j;
-                            if (jj >= hp) continue;
-                            const int ahead = r0 == 0 ? i / FW_EPI : 2;
-                            const int sl = ahead == 0 ? sl2[0] : (ahead == 1 ? sl2[1] : a.rm.slot[t]);
-                            const float2 cs = ahead == 0 ? cs2[0] : (ahead == 1 ? cs2[1] :
-                                              *reinterpret_cast<const float2*>(a.rope + ((size_t)t * hp + jj) * 2));
-                            const float rs = s.rstd[t];
-                            const float va = yv(t, 0, j) * rs, vb = yv(t, 0, f.h + j) * rs;
-                            if (sl < 0) continue;                         // inactive row: no query, no cache slot
-                            const float ra = va * cs.x - vb * cs.y, rb = vb * cs.x + va * cs.y;
-                            if (hg < a.Hq) {
-                                // attention operands: q * log2(e) / sqrt(hd) as bf16 hi + lo (softmax runs on exp2)
-                                const size_t o = ((size_t)t * a.Hq + hg) * HD + jj;
-                                split_store(ra * scale * 1.4426950408889634f, a.q_hi + o, a.q_lo + o);
-                                split_store(rb * scale * 1.4426950408889634f, a.q_hi + o + hp, a.q_lo + o + hp);
-                            } else {
-                                const int sq = ahead == 0 ? sq2[0] : (ahead == 1 ? sq2[1] : a.rm.seq[t]), kv = hg >= a.Hq + a.Hkv ? 1 : 0;
-                                if (sl >= a.cap || (unsigned)sq >= (unsigned)a.max_batch) continue;   // never past the cache
-                                __nv_bfloat16* c = a.cache + idx_cache(layer, a.max_batch, sq, kv, a.Hkv, hg - a.Hq - kv * a.Hkv, a.cap, sl, HD);
-                                c[jj] = __float2bfloat16_rn(kv ? va : ra);
-                                c[jj + hp] = __float2bfloat16_rn(kv ? vb : rb);
-                            }
-                        }
-                    } else if (kind == FW_GATEUP) {
-                        for (int i = e; i < nr * nf; i += FW_EPI) {
-                            const int t = r0 + i / nf, j = i % nf, n = f0 + j;
-                            if (n >= a.F) continue;
-                            const float rs = s.rstd[t];
-                            const float g = yv(t, 0, j) * rs, up = yv(t, 1, j) * rs;
-                            store_terms(g / (1.f + expf(-g)) * up, a.x_f + (size_t)t * terms * a.F + n, a.F, terms);
-                        }
-                    } else if (kind == FW_LM && a.lm_plain) {
-                        for (int i = e; i < nr * nf; i += FW_EPI) {
-                            const int t = r0 + i / nf, jl = i % nf, q = jl / f.h, n = f0 + jl;
-                            if (n < a.V) a.logits[(size_t)t * a.V + n] = yv(t, q, jl - q * f.h) * s.rstd[t];
-                        }
-                    } else if (kind == FW_LM) {
-                        // a warp per row: maximum, sum of exponentials, arg-max of the perturbed logits over the tile
-                        for (int t = r0 + w; t < r1; t += 8) {
-                            float z[8], m = -CUDART_INF_F, bv = -CUDART_INF_F, sum = 0.f;
-                            int bi = 0x7fffffff;
-                            const float rs = s.rstd[t];
-                            if (t != w)
-#pragma unroll
-                                for (int i = 0; i < 8; ++i) {
-                                    const int n = f0 + lane + 32 * i;
-                                    u8[i] = (lane + 32 * i < nf && n < a.V) ? a.uniforms[(size_t)(t / a.R) * a.V + n] : 0.5f;
-                                }
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                const int jl = lane + 32 * i, n = f0 + jl, q = jl >= f.h ? 1 : 0;
-                                const bool in = jl < nf && n < a.V;
-                                z[i] = in ? yv(t, q, jl - q * f.h) * rs : -CUDART_INF_F;
-                                m = fmaxf(m, z[i]);
-                                const float pz = in ? z[i] - logf(-logf(u8[i])) : -CUDART_INF_F;
-                                if (in && (pz > bv || (pz == bv && n < bi))) { bv = pz; bi = n; }
-                            }
-#pragma unroll
-                            for (int o = 16; o > 0; o >>= 1) {
-                                m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-                                const float v2 = __shfl_xor_sync(0xffffffffu, bv, o);
-                                const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
-                                if (v2 > bv || (v2 == bv && i2 < bi)) { bv = v2; bi = i2; }
-                            }
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) sum += z[i] == -CUDART_INF_F ? 0.f : expf(z[i] - m);
-#pragma unroll
-                            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-                            if (lane == 0) a.lm_part[idx_lm_part(t, f.n_tiles, tile)] = make_float4(m, sum, bv, __int_as_float(bi));
-                        }
-                        // logit of each node's token under its parent row, where it falls into this tile
-                        for (int t = e; t < T; t += FW_EPI) {
-                            const int pr = a.rm.prow[t];
-                            if (pr < r0 || pr >= r1) continue;
-                            const int tk = a.rm.tok[t] - f0, q = tk >= f.h ? 1 : 0;
-                            if (tk >= 0 && tk < nf) a.node_z[t] = yv(pr, q, tk - q * f.h) * s.rstd[pr];
-                        }
-                    } else {
-                        // residual: a warp per row; emits the next operand rows and the row's share of its sum of squares
-                        float* sq = kind == FW_O ? a.sumsq_b : a.sumsq_a;
-                        for (int t = r0 + w; t < r1; t += 8) {
-                            float ss = 0.f;
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                const int jl = lane + 32 * i, n = f0 + jl;
-                                if (jl >= nf || n >= a.d) continue;
-                                float* hp = a.hidden + (size_t)t * a.d + n;
-                                const float y = yv(t, 0, jl) + (t == w ? pre[i] : __ldcg(hp));
-                                *hp = y;
-                                store_terms(y * gn[i], a.x_d + (size_t)t * terms * a.d + n, a.d, terms);
-                                ss += y * y;
-                            }
-#pragma unroll
-                            for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-                            if (lane == 0) sq[(size_t)tile * TC_X_ROWS + t] = ss;
-                        }
-                    }
-                    if (r1 < T || tile + n_cta < f.n_tiles) bar_n(1, FW_EPI);       // Y is rewritten by the next rows or tile
-                    }
-                    if (!ok) break;
-                }
-                if (!ok) break;
+                ok = epi_phase<FW_LM, HD>(a, s, Y, p, layer, tcount, e, t_lane, cta);
             }
-            if (kind != FW_LM) {
+            if (kind != FW_LM && ok) {
                 // phase barrier: the release covers the whole group's stores (the readers' proxy fence follows their acquire)
                 bar_n(1, FW_EPI);
                 if (e == 0) {
@@ -921,7 +1026,12 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
         f.b_off = f.nbox * f.box_bytes;
         if (f.b_off + f.kb * a.cols * 128 > FW_SLOT || f.nbox * f.S * a.cols > FW_ACC) return false;
         if ((k == FW_O || k == FW_DOWN) && f.n_tiles > n_cta) return false;
-        if (FW_UNION / (8 * (f.nbox * f.S * f.hr + 4) * 4) < 1) return false;
+        // one box: the MMAs along k alternate between two accumulators where they fit and there are two
+        f.dual = f.nbox == 1 && 2 * f.S * a.cols <= FW_ACC && f.steps * (f.kb / f.S) >= 2 ? 1 : 0;
+        const int per = a.terms == 3 ? 5 : 8;              // rows of one drain load
+        const int fit = FW_UNION / (per * (f.nbox * f.S * f.hr + 4) * 4);
+        if (fit < 1) return false;
+        f.blk = std::min(up_div(T, per), fit) * per;
     }
     return true;
 }
@@ -933,7 +1043,7 @@ size_t fw_parts_max(const mtad_model_desc& d, int n_cta, bool lm) {
 }
 
 cudaError_t launch_forward(const FwArgs& a, cudaStream_t st) {
-    const size_t smem = 1024 + (size_t)NS * FW_SLOT + FW_UNION + sizeof(FwTail);
+    const size_t smem = (size_t)NS * FW_SLOT + FW_UNION + sizeof(FwTail);
     auto go = [&](auto kernel) -> cudaError_t {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e != cudaSuccess) return e;

@@ -24,6 +24,7 @@ struct FwPhase {
     int kb, flat, S, steps;               // k-blocks of a box, its map's view, k-blocks side by side in the MMA, steps of a tile
     int box_bytes, b_off;                 // bytes of one weight box, offset of the operand rows in the slot
     int k_blocks, K;
+    int dual, blk;                        // two accumulators for one box; rows that the epilogue takes at a time
 };
 enum { FW_QKV = 0, FW_ATTN = 1, FW_O = 2, FW_GATEUP = 3, FW_DOWN = 4, FW_LM = 5 };
 
