@@ -44,6 +44,7 @@ constexpr int FW_EPI = 256;
 constexpr int FW_UNION = 32 * 1024;       // epilogue tile Y, or the attention's query and probability tiles
 constexpr int NS = FW_SLOTS;
 constexpr int FW_ACC = 240;               // accumulator columns of a tile, of 256 (the drain reads up to 15 columns further)
+constexpr float FW_LAZY = 8.f;            // log2 of how far a score may exceed its row's reference value
 constexpr int FW_TM_D = 128;              // attention: tensor-memory columns 0 / 64 scores, 128 / 192 outputs
 
 __device__ __forceinline__ bool grid_wait(const int* c, int want, volatile int* abort_flag) {
@@ -58,6 +59,21 @@ __device__ __forceinline__ bool grid_wait(const int* c, int want, volatile int* 
     return false;
 }
 __device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async;" ::: "memory"); }
+__device__ __forceinline__ uint2 pack4(float x, float y, float z, float w) {
+    const __nv_bfloat162 p = __floats2bfloat162_rn(x, y), q = __floats2bfloat162_rn(z, w);
+    return make_uint2(*reinterpret_cast<const uint32_t*>(&p), *reinterpret_cast<const uint32_t*>(&q));
+}
+__device__ __forceinline__ void store_bf4(const float* v, __nv_bfloat16* d) {
+    *reinterpret_cast<uint2*>(d) = pack4(v[0], v[1], v[2], v[3]);
+}
+// four values times `scale` as bf16 hi and lo parts
+__device__ __forceinline__ void split_store4(const float* v, float scale, __nv_bfloat16* hi, __nv_bfloat16* lo) {
+    const float x = v[0] * scale, y = v[1] * scale, z = v[2] * scale, w = v[3] * scale;
+    const uint2 h = pack4(x, y, z, w);
+    *reinterpret_cast<uint2*>(hi) = h;
+    *reinterpret_cast<uint2*>(lo) = pack4(x - __uint_as_float(h.x << 16), y - __uint_as_float(h.x & 0xffff0000u),
+                                          z - __uint_as_float(h.y << 16), w - __uint_as_float(h.y & 0xffff0000u));
+}
 // barrier and consensus of `n` threads
 __device__ __forceinline__ bool all_of(int id, int n, bool ok) {
     uint32_t r;
@@ -143,7 +159,9 @@ __device__ __forceinline__ void attn_next(AttnPos& it, const SeqMeta* meta, int 
 
 struct FwTail {
     SeqMeta meta[MTAD_MAX_BATCH];
-    float rstd[64];
+    float rstd[FW_MAX_ROWS];
+    int slot[FW_MAX_ROWS];                // cache slot of a row, -1: inactive
+    uint8_t rowb[FW_MAX_ROWS];            // its sequence within the call
     float smx[2][16][4];                  // row maxima of the four softmax warps
     float sf[2][16];                      // rescale factor of the running output, per tile buffer
     float sl[2][4][16];                   // row sums of the softmax warps
@@ -159,23 +177,27 @@ static_assert(NS * FW_SLOT + FW_UNION + sizeof(FwTail) <= 227 * 1024, "shared me
 // The epilogue group's part of one projection: row statistics, then per tile the accumulators -> Y in shared memory ->
 // the fused epilogue.  KIND is a template parameter so that the phase's geometry is read straight from the launch
 // parameters; index arithmetic and global loads stand ahead of the wait for the accumulator, because everything after it
-// is a chain of latencies between the last weight and the next phase's first.
-template <int KIND, int HD>
+// is a chain of latencies between the last weight and the next phase's first.  FEW (up to eight rows): an element per
+// thread, as little code as possible (with a warp or two per scheduler, and code that runs once a phase, time goes by the
+// instruction); otherwise four neighbouring features per thread.
+template <int KIND, int HD, bool FEW>
 __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, int p, int layer, int& tcount, int e,
                                           uint32_t tmem_lane, int cta) {
     const FwPhase& f = a.ph[KIND];
     if (cta >= f.n_tiles) return true;
     volatile int* abort_flag = s.abort_flag;
+    constexpr int V = FEW ? 1 : 4;                         // features per item
     const int lane = e & 31, w = e >> 5, quad = w & 3, half = w >> 2;
     const int T = a.T, terms = a.terms, cols = a.cols, n_cta = a.n_cta;
     const int hr = f.hr, S = f.S, nbox = f.nbox;
     const int yb = S * hr, ys = nbox * yb + 4;             // columns of Y that a box takes, row stride of Y
     const int nf = KIND == FW_LM ? nbox * f.h : f.h;       // features (pairs) of a tile
-    const int per = terms == 3 ? 5 : 8, blk = f.blk;       // rows of a drain load, rows that Y holds at a time
+    const int nv = nf / V;                                 // items of a row
+    const int per = terms == 3 ? 5 : 8, blk = FEW ? 8 : f.blk;      // rows of a drain load, rows that Y holds at a time
     // a lane's slice of the S k-blocks that the MMA takes side by side is tl / hr; a warp's lanes may lie in several
     const int tl = quad * 32 + lane, my = tl / hr;
     const int s0 = S > 1 ? quad * 32 / hr : 0, s1 = S > 1 ? min(S - 1, (quad * 32 + 31) / hr) : 0;
-    const int it0 = e / nf, ij0 = e - it0 * nf, dt = FW_EPI / nf, dj = FW_EPI - dt * nf;    // this thread's items (row, feature)
+    const int it0 = e / nv, ij0 = (e - it0 * nv) * V, dt = FW_EPI / nv, dj = (FW_EPI - dt * nv) * V;    // items (row, feature)
     bool ok = true;
     if (KIND == FW_QKV || KIND == FW_GATEUP || KIND == FW_LM) {
         // scale of the deferred RMSNorm: the rows' sums of squares come from every block
@@ -188,42 +210,40 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
         const int parts = KIND == FW_GATEUP ? a.ph[FW_O].n_tiles : (p == 0 ? a.parts0 : a.ph[FW_DOWN].n_tiles);
         for (int r = w; r < T; r += 8) {
             float v = 0.f;
+#pragma unroll 5
             for (int q = lane; q < parts; q += 32) v += __ldcg(sq + (size_t)q * TC_X_ROWS + r);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
             if (lane == 0) s.rstd[r] = rsqrtf(v * a.inv_dim + a.eps);
         }
     }
-    const FwLayer* L = a.layers + layer;
+    const __nv_bfloat16* gain = nullptr;
+    if (KIND == FW_O) gain = a.layers[layer].gain_ffn;
+    if (KIND == FW_DOWN) gain = a.layers[layer].gain_next;
     for (int tile = cta; tile < f.n_tiles; tile += n_cta, ++tcount) {
         const int buf = tcount & 1, f0 = tile * nf;        // f0: first feature (O, down, gate / up, LM head)
         // ---- what the first items need besides the accumulator
-        // QKV
         const int hg = KIND == FW_QKV ? tile / f.u : 0, j0 = KIND == FW_QKV ? (tile - hg * f.u) * f.h : 0;
-        constexpr int NI = 4;                              // items per thread whose loads are in flight together
-        int sl4[NI], sq4[NI];
-        float2 cs4[NI];
-        auto qkv_load = [&](int t, int j) {
+        constexpr int NI = FEW ? 2 : 1;                    // QKV: items per thread and round
+        float cs[NI][2 * V];                               // cosines and sines of an item's pairs
+        auto rope_load = [&](int t, int j) {
 #pragma unroll
             for (int q = 0; q < NI; ++q) {
-                sl4[q] = -1;
                 if (t < T && j0 + j < HD / 2) {
-                    cs4[q] = *reinterpret_cast<const float2*>(a.rope + ((size_t)t * (HD / 2) + j0 + j) * 2);
-                    sl4[q] = a.rm.slot[t];
-                    sq4[q] = a.rm.seq[t];
+                    const float* src = a.rope + ((size_t)t * (HD / 2) + j0 + j) * 2;
+                    if (V == 4) {
+#pragma unroll
+                        for (int x = 0; x < V / 2; ++x)
+                            *reinterpret_cast<float4*>(&cs[q][4 * x]) = *reinterpret_cast<const float4*>(src + 4 * x);
+                    } else {
+                        *reinterpret_cast<float2*>(&cs[q][0]) = *reinterpret_cast<const float2*>(src);
+                    }
                 }
                 t += dt; j += dj;
                 if (j >= nf) { j -= nf; ++t; }
             }
         };
-        // O, down: the residual rows w, w + 8, ... of the first 32 features
-        float hid[NI], gain0 = 0.f;
-        const __nv_bfloat16* gain = KIND == FW_O ? L->gain_ffn : L->gain_next;
-        auto res_load = [&](int t, int n, bool in) {
-#pragma unroll
-            for (int q = 0; q < NI; ++q)
-                hid[q] = (in && t + 8 * q < T) ? __ldcg(a.hidden + (size_t)(t + 8 * q) * a.d + n) : 0.f;
-        };
+        float hid = 0.f, gain0 = 0.f;                      // O, down with few rows: the residual element of (row w, feature lane)
         float u8[8];
         auto lm_load = [&](int t) {
 #pragma unroll
@@ -232,11 +252,10 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                 u8[i] = (t < T && jl < nf && n < a.V) ? a.uniforms[(size_t)(t / a.R) * a.V + n] : 0.5f;
             }
         };
-        if (KIND == FW_QKV) qkv_load(it0, ij0);
-        if (KIND == FW_O || KIND == FW_DOWN) {
-            const bool in = lane < nf && f0 + lane < a.d;
-            if (in) gain0 = __bfloat162float(gain[f0 + lane]);
-            res_load(w, f0 + lane, in);
+        if (KIND == FW_QKV) rope_load(it0, ij0);
+        if (FEW && (KIND == FW_O || KIND == FW_DOWN) && lane < nf && f0 + lane < a.d) {
+            gain0 = __bfloat162float(gain[f0 + lane]);
+            if (w < T) hid = __ldcg(a.hidden + (size_t)w * a.d + f0 + lane);
         }
         if (KIND == FW_LM && !a.lm_plain) lm_load(w);
         // (one thread polls: 256 of them would take the shared-memory pipe away from the copies' barriers)
@@ -262,7 +281,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                     }
                     if (my == sl && tl < yb) {
                         float* y = Y + (rb - r0) * ys + b * yb + tl;
-                        if (terms == 3) {
+                        if (FEW || terms == 3) {
 #pragma unroll
                             for (int j = 0; j < 5; ++j)
                                 if (rb + j < r1) y[j * ys] = v[3 * j] + (v[3 * j + 1] + v[3 * j + 2]);
@@ -280,66 +299,119 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                 if (lane == 0) mbar_arrive(smem_u32(&s.tempty[buf]));
             }
             bar_n(1, FW_EPI);
-            // value of (row of the block, box, weight row): the S slices lie side by side
-            auto yv = [&](int t, int q, int row) -> float {
+            // values of (row of the block, box, weight rows `row` ..): the S slices lie side by side
+            auto yv1 = [&](int t, int q, int row) -> float {
                 const float* y = Y + t * ys + q * yb + row;
                 float v = y[0];
-#pragma unroll 4
+                if (S == 4) return (v + y[hr]) + (y[2 * hr] + y[3 * hr]);
                 for (int sl = 1; sl < S; ++sl) v += y[sl * hr];
                 return v;
             };
+            auto yv = [&](int t, int q, int row, float* o) {
+                if (V == 1) { o[0] = yv1(t, q, row); return; }
+                const float* y = Y + t * ys + q * yb + row;
+                float4 v = *reinterpret_cast<const float4*>(y);
+                for (int sl = 1; sl < S; ++sl) {
+                    const float4 x = *reinterpret_cast<const float4*>(y + sl * hr);
+                    v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w;
+                }
+                o[0] = v.x; o[V - 3 > 0 ? 1 : 0] = v.y; o[V - 2 > 0 ? 2 % V : 0] = v.z; o[V - 1] = v.w;
+            };
             if (KIND == FW_QKV) {
                 constexpr int hp = HD / 2;
-                const float scale = rsqrtf((float)HD);
+                const float scale = rsqrtf((float)HD) * 1.4426950408889634f;      // (the attention's softmax runs on exp2)
                 int t = it0, j = ij0;
-                for (int i = e; i < nr * nf; i += NI * FW_EPI) {
-                    if (r0 > 0 || i != e) qkv_load(r0 + t, j);
+                for (int i = e; i < nr * nv; i += NI * FW_EPI) {
+                    if (FEW ? i != e : r0 > 0 && i == e) rope_load(r0 + t, j);
 #pragma unroll
                     for (int q = 0; q < NI; ++q) {
-                        const int jj = j0 + j;
-                        if (t < nr && jj < hp && sl4[q] >= 0) {           // (no slot: an inactive row has no query and no keys)
-                            const float rs = s.rstd[r0 + t];
-                            const float va = yv(t, 0, j) * rs, vb = yv(t, 0, f.h + j) * rs;
-                            const float2 cs = cs4[q];
-                            const float ra = va * cs.x - vb * cs.y, rb2 = vb * cs.x + va * cs.y;
+                        const int jj = j0 + j, tt = r0 + t;
+                        int tn = t + dt, jn = j + dj;                     // the next item
+                        if (jn >= nf) { jn -= nf; ++tn; }
+                        float c[2 * V];
+#pragma unroll
+                        for (int x = 0; x < 2 * V; ++x) c[x] = cs[q][x];
+                        if (!FEW && i + FW_EPI < nr * nv) rope_load(r0 + tn, jn);        // ahead by one round
+                        const int sl = t < nr ? s.slot[tt] : -1;
+                        if (jj < hp && sl >= 0) {                         // (no slot: an inactive row has no query and no keys)
+                            const float rs = s.rstd[tt];
+                            float va[V], vb[V];
+                            yv(t, 0, j, va);
+                            yv(t, 0, f.h + j, vb);
+                            const bool rot = hg < a.Hq + a.Hkv;
+#pragma unroll
+                            for (int x = 0; x < V; ++x) {
+                                const float ya = va[x] * rs, yb2 = vb[x] * rs;
+                                va[x] = rot ? ya * c[2 * x] - yb2 * c[2 * x + 1] : ya;
+                                vb[x] = rot ? yb2 * c[2 * x] + ya * c[2 * x + 1] : yb2;
+                            }
                             if (hg < a.Hq) {
-                                // attention operands: q * log2(e) / sqrt(hd) as bf16 hi + lo (softmax runs on exp2)
-                                const size_t o = ((size_t)(r0 + t) * a.Hq + hg) * HD + jj;
-                                split_store(ra * scale * 1.4426950408889634f, a.q_hi + o, a.q_lo + o);
-                                split_store(rb2 * scale * 1.4426950408889634f, a.q_hi + o + hp, a.q_lo + o + hp);
-                            } else if (sl4[q] < a.cap && (unsigned)sq4[q] < (unsigned)a.max_batch) {   // never past the cache
-                                const int kv = hg >= a.Hq + a.Hkv ? 1 : 0;
-                                __nv_bfloat16* c = a.cache + idx_cache(layer, a.max_batch, sq4[q], kv, a.Hkv, hg - a.Hq - kv * a.Hkv,
-                                                                       a.cap, sl4[q], HD);
-                                c[jj] = __float2bfloat16_rn(kv ? va : ra);
-                                c[jj + hp] = __float2bfloat16_rn(kv ? vb : rb2);
+                                // attention operands: q * log2(e) / sqrt(hd) as bf16 hi + lo
+                                const size_t o = ((size_t)tt * a.Hq + hg) * HD + jj;
+                                if (V == 1) {
+                                    split_store(va[0] * scale, a.q_hi + o, a.q_lo + o);
+                                    split_store(vb[0] * scale, a.q_hi + o + hp, a.q_lo + o + hp);
+                                } else {
+                                    split_store4(va, scale, a.q_hi + o, a.q_lo + o);
+                                    split_store4(vb, scale, a.q_hi + o + hp, a.q_lo + o + hp);
+                                }
+                            } else {
+                                const int sq = s.meta[s.rowb[tt]].seq, kv = rot ? 0 : 1;
+                                if (sl < a.cap && (unsigned)sq < (unsigned)a.max_batch) {   // never past the cache
+                                    __nv_bfloat16* d = a.cache + idx_cache(layer, a.max_batch, sq, kv, a.Hkv, hg - a.Hq - kv * a.Hkv,
+                                                                           a.cap, sl, HD) + jj;
+                                    if (V == 1) {
+                                        d[0] = __float2bfloat16_rn(va[0]);
+                                        d[hp] = __float2bfloat16_rn(vb[0]);
+                                    } else {
+                                        store_bf4(va, d);
+                                        store_bf4(vb, d + hp);
+                                    }
+                                }
                             }
                         }
-                        t += dt; j += dj;
-                        if (j >= nf) { j -= nf; ++t; }
+                        t = tn; j = jn;
                     }
                 }
             } else if (KIND == FW_GATEUP) {
                 int t = it0, j = ij0;
-                for (int i = e; i < nr * nf; i += 2 * FW_EPI) {
+#pragma unroll 2
+                for (int i = e; i < nr * nv; i += FW_EPI) {
+                    const int n = f0 + j;
+                    if (n < a.F) {
+                        const float rs = s.rstd[r0 + t];
+                        float g[V], u[V];
+                        yv(t, 0, j, g);
+                        yv(t, 1, j, u);
 #pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        const int n = f0 + j;
-                        if (t < nr && n < a.F) {
-                            const float rs = s.rstd[r0 + t];
-                            const float g = yv(t, 0, j) * rs, up = yv(t, 1, j) * rs;
-                            store_terms(g / (1.f + expf(-g)) * up, a.x_f + (size_t)(r0 + t) * terms * a.F + n, a.F, terms);
+                        for (int x = 0; x < V; ++x) {
+                            const float gx = g[x] * rs;
+                            g[x] = gx / (1.f + expf(-gx)) * (u[x] * rs);
                         }
-                        t += dt; j += dj;
-                        if (j >= nf) { j -= nf; ++t; }
+                        __nv_bfloat16* o = a.x_f + (size_t)(r0 + t) * terms * a.F + n;
+                        if (V == 1) store_terms(g[0], o, a.F, terms);
+                        else store_terms4(make_float4(g[0], g[1 % V], g[2 % V], g[3 % V]), o, a.F, terms);
                     }
+                    t += dt; j += dj;
+                    if (j >= nf) { j -= nf; ++t; }
                 }
             } else if (KIND == FW_LM) {
                 if (a.lm_plain) {
                     int t = it0, j = ij0;
-                    for (int i = e; i < nr * nf; i += FW_EPI) {
+#pragma unroll 2
+                    for (int i = e; i < nr * nv; i += FW_EPI) {
                         const int q = j >= f.h ? 1 : 0, n = f0 + j;
-                        if (n < a.V) a.logits[(size_t)(r0 + t) * a.V + n] = yv(t, q, j - q * f.h) * s.rstd[r0 + t];
+                        float z[V];
+                        yv(t, q, j - q * f.h, z);
+                        const float rs = s.rstd[r0 + t];
+                        float* o = a.logits + (size_t)(r0 + t) * a.V + n;
+                        if (V == 4 && (a.V & 3) == 0) {
+                            if (n < a.V) *reinterpret_cast<float4*>(o) = make_float4(z[0] * rs, z[1 % V] * rs, z[2 % V] * rs, z[3 % V] * rs);
+                        } else {
+#pragma unroll
+                            for (int x = 0; x < V; ++x)
+                                if (n + x < a.V) o[x] = z[x] * rs;
+                        }
                         t += dt; j += dj;
                         if (j >= nf) { j -= nf; ++t; }
                     }
@@ -354,7 +426,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                         for (int i = 0; i < 8; ++i) {
                             const int jl = lane + 32 * i, n = f0 + jl, q = jl >= f.h ? 1 : 0;
                             const bool in = jl < nf && n < a.V;
-                            z[i] = in ? yv(t - r0, q, jl - q * f.h) * rs : -CUDART_INF_F;
+                            z[i] = in ? yv1(t - r0, q, jl - q * f.h) * rs : -CUDART_INF_F;
                             m = fmaxf(m, z[i]);
                             const float pz = in ? z[i] - logf(-logf(u8[i])) : -CUDART_INF_F;
                             if (in && (pz > bv || (pz == bv && n < bi))) { bv = pz; bi = n; }
@@ -377,39 +449,55 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                         const int pr = a.rm.prow[t];
                         if (pr < r0 || pr >= r1) continue;
                         const int tk = a.rm.tok[t] - f0, q = tk >= f.h ? 1 : 0;
-                        if (tk >= 0 && tk < nf) a.node_z[t] = yv(pr - r0, q, tk - q * f.h) * s.rstd[pr];
+                        if (tk >= 0 && tk < nf) a.node_z[t] = yv1(pr - r0, q, tk - q * f.h) * s.rstd[pr];
                     }
                 }
-            } else {
-                // residual: a warp per row, four rows at a time; emits the next operand rows and the rows' share of their sums
-                // of squares
-                float* sq = KIND == FW_O ? a.sumsq_b : a.sumsq_a;
-                for (int t = r0 + w; t < r1; t += 8 * NI) {
-                    float ss[NI] = {};
-                    for (int jl = lane; jl < nf; jl += 32) {
+            } else if (FEW) {
+                // residual, a warp per row: emits the next operand rows and the row's share of its sum of squares
+                if (w < T) {
+                    float ss = 0.f;
+                    for (int jl = lane; jl < nf && f0 + jl < a.d; jl += 32) {
                         const int n = f0 + jl;
-                        const bool in = n < a.d;
-                        const bool first = t == w && jl == lane;
-                        if (!first) res_load(t, n, in);
-                        const float g = jl == lane ? gain0 : (in ? __bfloat162float(gain[n]) : 0.f);
-#pragma unroll
-                        for (int q = 0; q < NI; ++q) {
-                            const int tt = t + 8 * q;
-                            if (in && tt < r1) {
-                                const float y = yv(tt - r0, 0, jl) + hid[q];
-                                a.hidden[(size_t)tt * a.d + n] = y;
-                                store_terms(y * g, a.x_d + (size_t)tt * terms * a.d + n, a.d, terms);
-                                ss[q] += y * y;
-                            }
-                        }
+                        if (jl != lane) { hid = __ldcg(a.hidden + (size_t)w * a.d + n); gain0 = __bfloat162float(gain[n]); }
+                        const float y = yv1(w, 0, jl) + hid;
+                        a.hidden[(size_t)w * a.d + n] = y;
+                        store_terms(y * gain0, a.x_d + (size_t)w * 3 * a.d + n, a.d, 3);
+                        ss += y * y;
                     }
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1)
+                    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+                    if (lane == 0) (KIND == FW_O ? a.sumsq_b : a.sumsq_a)[(size_t)tile * TC_X_ROWS + w] = ss;
+                }
+            } else {
+                // residual, four features per item; the items' sums of squares meet in Y (each over its own first element)
+                int t = it0, j = ij0;
+#pragma unroll 2
+                for (int i = e; i < nr * nv; i += FW_EPI) {
+                    const int n = f0 + j;
+                    float ss = 0.f;
+                    if (n < a.d) {
+                        float4* hp = reinterpret_cast<float4*>(a.hidden + (size_t)(r0 + t) * a.d + n);
+                        const float4 h4 = __ldcg(hp);
+                        float g[4], v[V];
 #pragma unroll
-                        for (int q = 0; q < NI; ++q) ss[q] += __shfl_xor_sync(0xffffffffu, ss[q], o);
+                        for (int x = 0; x < 4; ++x) g[x] = __bfloat162float(gain[n + x]);
+                        yv(t, 0, j, v);
+                        const float4 y = make_float4(v[0] + h4.x, v[1 % V] + h4.y, v[2 % V] + h4.z, v[3 % V] + h4.w);
+                        *hp = y;
+                        store_terms4(make_float4(y.x * g[0], y.y * g[1], y.z * g[2], y.w * g[3]),
+                                     a.x_d + (size_t)(r0 + t) * terms * a.d + n, a.d, terms);
+                        ss = (y.x * y.x + y.y * y.y) + (y.z * y.z + y.w * y.w);
+                    }
+                    Y[t * ys + j] = ss;
+                    t += dt; j += dj;
+                    if (j >= nf) { j -= nf; ++t; }
+                }
+                bar_n(1, FW_EPI);
+                for (int tr = w; tr < nr; tr += 8) {
+                    float ss = lane < nv ? Y[tr * ys + lane * V] : 0.f;       // (nv <= 32: at most 128 features)
 #pragma unroll
-                    for (int q = 0; q < NI; ++q)
-                        if (lane == q && t + 8 * q < r1) sq[(size_t)tile * TC_X_ROWS + t + 8 * q] = ss[q];
+                    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+                    if (lane == 0) (KIND == FW_O ? a.sumsq_b : a.sumsq_a)[(size_t)tile * TC_X_ROWS + r0 + tr] = ss;
                 }
             }
             if (r1 < T || tile + n_cta < f.n_tiles) bar_n(1, FW_EPI);       // Y is rewritten by the next rows or tile
@@ -418,7 +506,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
     return true;
 }
 
-template <int HD, int NQP>
+template <int HD, int NQP, bool FEW>
 __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_constant__ FwArgs a) {
     constexpr int NCH = HD / 64;                       // 64-element chunks of a head row
     constexpr int NQ2 = 2 * NQP;                       // query rows as hi and lo parts
@@ -442,6 +530,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         m.nkeys = min(m.L + __ldcg(a.rm.n_spec + b), a.pieces * FW_KEYS);
         m.seq = __ldcg(a.rm.call_seq + b);
         s.meta[b] = m;
+    }
+    for (int t = threadIdx.x; t < T; t += FW_THREADS) {
+        s.slot[t] = __ldcg(a.rm.slot + t);
+        s.rowb[t] = (uint8_t)(t / a.R);
     }
     if (threadIdx.x == 0) {
         for (int i = 0; i < NS; ++i) {
@@ -762,35 +854,52 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
 #pragma unroll
                             for (int r = 0; r < NQP; ++r) v[r] = ((vis >> r) & 1u) ? c[r] + c[NQP + r] : -CUDART_INF_F;
                         }
-                        float wm[NQP];
+                        // The reference value m of a row follows its maximum lazily: it moves only when a score exceeds it by
+                        // more than 2^8 (numerators and sums stay well inside fp32, and bf16 hi + lo keep their precision), so
+                        // the row maxima over 128 lanes are formed on a segment's first tile and hardly ever after.
+                        bool calm = !fresh;
 #pragma unroll
-                        for (int r = 0; r < NQP; ++r) wm[r] = v[r];
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                            for (int r = 0; r < NQP; ++r) wm[r] = fmaxf(wm[r], __shfl_xor_sync(0xffffffffu, wm[r], o));
-#pragma unroll
-                        for (int r = 0; r < NQP; ++r)
-                            if (lane == r) s.smx[b][r][quad] = wm[r];
+                        for (int r = 0; r < NQP; ++r) {
+                            if (r >= n_q) break;
+                            calm = calm && v[r] <= m[r] + FW_LAZY;
+                        }
                         // the buffers P and sf of this tile are free once the output warps are done with the tile before the last
                         ok = warp_wait(smem_u32(&s.oempty[b]), par ^ 1u, abort_flag, ok, lane);
-                        ok = all_of(2, 128, ok);
+                        if (!all_of(2, 128, calm && ok)) {
+                            float wm[NQP];
+#pragma unroll
+                            for (int r = 0; r < NQP; ++r) wm[r] = v[r];
+#pragma unroll
+                            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                                for (int r = 0; r < NQP; ++r) wm[r] = fmaxf(wm[r], __shfl_xor_sync(0xffffffffu, wm[r], o));
+#pragma unroll
+                            for (int r = 0; r < NQP; ++r)
+                                if (lane == r) s.smx[b][r][quad] = wm[r];
+                            ok = all_of(2, 128, ok);
+#pragma unroll
+                            for (int r = 0; r < NQP; ++r) {
+                                const float4 q4 = *reinterpret_cast<const float4*>(s.smx[b][r]);
+                                const float mn = fmaxf(m[r], fmaxf(fmaxf(q4.x, q4.y), fmaxf(q4.z, q4.w)));
+                                const float f = mn == -CUDART_INF_F ? 1.f : exp2f(m[r] - mn);
+                                m[r] = mn;
+                                l[r] *= f;
+                                if (kl == r) s.sf[b][r] = f;
+                            }
+                        } else if (kl < NQP) {
+                            s.sf[b][kl] = 1.f;
+                        }
                         uint8_t* pt = Ps + b * P_BYTES + (kl >> 6) * (NQ2 * 128) + (kl & 7) * 2;
                         const int pc = (kl & 63) >> 3;
 #pragma unroll
                         for (int r = 0; r < NQP; ++r) {
-                            const float4 q4 = *reinterpret_cast<const float4*>(s.smx[b][r]);
-                            const float mn = fmaxf(m[r], fmaxf(fmaxf(q4.x, q4.y), fmaxf(q4.z, q4.w)));
-                            const float mz = mn == -CUDART_INF_F ? 0.f : mn;
-                            const float f = exp2f(m[r] - mz);                                   // exp2(-inf) = 0
-                            const float pv = exp2f(v[r] - mz);
-                            m[r] = mn;
-                            l[r] = l[r] * f + pv;
-                            if (kl == r) s.sf[b][r] = f;
+                            if (r >= n_q) break;                              // (rows without a query: their output columns are not read)
+                            const float pv = exp2f(v[r] - (m[r] == -CUDART_INF_F ? 0.f : m[r]));        // exp2(-inf) = 0
+                            l[r] += pv;
                             const __nv_bfloat16 hi = __float2bfloat16_rn(pv);
-                            *reinterpret_cast<__nv_bfloat16*>(pt + r * 128 + ((pc ^ (r & 7)) << 4)) = hi;
-                            *reinterpret_cast<__nv_bfloat16*>(pt + (NQP + r) * 128 + ((pc ^ (r & 7)) << 4)) =
-                                __float2bfloat16_rn(pv - __bfloat162float(hi));
+                            uint8_t* d = pt + ((pc ^ (r & 7)) << 4);
+                            *reinterpret_cast<__nv_bfloat16*>(d + r * 128) = hi;
+                            *reinterpret_cast<__nv_bfloat16*>(d + (NQP + r) * 128) = __float2bfloat16_rn(pv - __bfloat162float(hi));
                         }
                         if ((it.tile + 1) * FW_KEYS > nkeys) {
                             // rows of V past the last key: their probabilities are 0, but 0 x (stale value) must not make a NaN
@@ -926,15 +1035,15 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     }
                 }
             } else if (kind == FW_QKV) {
-                ok = epi_phase<FW_QKV, HD>(a, s, Y, p, layer, tcount, e, t_lane, cta);
+                ok = epi_phase<FW_QKV, HD, FEW>(a, s, Y, p, layer, tcount, e, t_lane, cta);
             } else if (kind == FW_O) {
-                ok = epi_phase<FW_O, HD>(a, s, Y, p, layer, tcount, e, t_lane, cta);
+                ok = epi_phase<FW_O, HD, FEW>(a, s, Y, p, layer, tcount, e, t_lane, cta);
             } else if (kind == FW_GATEUP) {
-                ok = epi_phase<FW_GATEUP, HD>(a, s, Y, p, layer, tcount, e, t_lane, cta);
+                ok = epi_phase<FW_GATEUP, HD, FEW>(a, s, Y, p, layer, tcount, e, t_lane, cta);
             } else if (kind == FW_DOWN) {
-                ok = epi_phase<FW_DOWN, HD>(a, s, Y, p, layer, tcount, e, t_lane, cta);
+                ok = epi_phase<FW_DOWN, HD, FEW>(a, s, Y, p, layer, tcount, e, t_lane, cta);
             } else {
-                ok = epi_phase<FW_LM, HD>(a, s, Y, p, layer, tcount, e, t_lane, cta);
+                ok = epi_phase<FW_LM, HD, FEW>(a, s, Y, p, layer, tcount, e, t_lane, cta);
             }
             if (kind != FW_LM && ok) {
                 // phase barrier: the release covers the whole group's stores (the readers' proxy fence follows their acquire)
@@ -1004,7 +1113,7 @@ void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta) {
 bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
     const int T = B * R, G = d.n_q_heads / d.n_kv_heads;
     if (d.head_dim != 64 && d.head_dim != 128) return false;
-    if (T > 64 || G * R > FW_MAX_QROWS || B > MTAD_MAX_BATCH) return false;
+    if (T > FW_MAX_ROWS || G * R > FW_MAX_QROWS || B > MTAD_MAX_BATCH) return false;
     if (d.d_model >= 8192 && T > 32) return false;          // the accurate K / V projection has launches of its own
     fw_geometry(a.ph, d, n_cta);
     a.T = T; a.B = B; a.R = R; a.terms = tc_terms(T);
@@ -1059,9 +1168,14 @@ cudaError_t launch_forward(const FwArgs& a, cudaStream_t st) {
         cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, kernel, a);
     };
-    const bool few = (a.Hq / a.Hkv) * a.R <= 8;
-    if (a.hd == 128) return few ? go(forward_kernel<128, 8>) : go(forward_kernel<128, 16>);
-    return few ? go(forward_kernel<64, 8>) : go(forward_kernel<64, 16>);
+    // instantiations: head size, query rows of a KV head, few rows in all
+    const bool q8 = (a.Hq / a.Hkv) * a.R <= 8, few = a.T <= 8;
+    if (a.hd == 128) {
+        if (few) return q8 ? go(forward_kernel<128, 8, true>) : go(forward_kernel<128, 16, true>);
+        return q8 ? go(forward_kernel<128, 8, false>) : go(forward_kernel<128, 16, false>);
+    }
+    if (few) return q8 ? go(forward_kernel<64, 8, true>) : go(forward_kernel<64, 16, true>);
+    return q8 ? go(forward_kernel<64, 8, false>) : go(forward_kernel<64, 16, false>);
 }
 
 }  // namespace mtad

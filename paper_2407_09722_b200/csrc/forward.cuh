@@ -8,6 +8,7 @@ namespace mtad {
 constexpr int FW_SLOT = 48 * 1024;        // bytes of one ring slot: one step of a projection, or 128 keys of K or V
 constexpr int FW_SLOTS = 4;
 constexpr int FW_KEYS = 128;              // keys of an attention tile
+constexpr int FW_MAX_ROWS = 56;           // rows of a call
 constexpr int FW_MAX_COLS = 112;          // operand rows (terms x rows) of a call
 constexpr int FW_MAX_QROWS = 16;          // query rows of one KV head and sequence
 
