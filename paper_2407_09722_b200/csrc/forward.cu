@@ -28,6 +28,8 @@
 // others run into their own limits at the grid barrier.
 #include <math_constants.h>
 
+#include <cstddef>
+
 #include <algorithm>
 
 #include "forward.cuh"
@@ -162,7 +164,7 @@ struct FwTail {
     float rstd[FW_MAX_ROWS];
     int slot[FW_MAX_ROWS];                // cache slot of a row, -1: inactive
     uint8_t rowb[FW_MAX_ROWS];            // its sequence within the call
-    float smx[2][16][4];                  // row maxima of the four softmax warps
+    alignas(16) float smx[2][16][4];           // row maxima of the four softmax warps
     float sf[2][16];                      // rescale factor of the running output, per tile buffer
     float sl[2][4][16];                   // row sums of the softmax warps
     float sm[2][16];                      // row reference values
@@ -172,6 +174,7 @@ struct FwTail {
     int abort_flag[2];
     int last[2];
 };
+static_assert(offsetof(FwTail, smx) % 16 == 0 && offsetof(FwTail, full) % 8 == 0, "alignment of the tail");
 static_assert(NS * FW_SLOT + FW_UNION + sizeof(FwTail) <= 227 * 1024, "shared memory of the forward");
 
 // The epilogue group's part of one projection: row statistics, then per tile the accumulators -> Y in shared memory ->
