@@ -46,7 +46,7 @@ constexpr int FW_EPI = 256;
 constexpr int FW_UNION = 32 * 1024;       // epilogue tile Y, or the attention's query and probability tiles
 constexpr int NS = FW_SLOTS;
 constexpr int FW_ACC = 240;               // accumulator columns of a tile, of 256 (the drain reads up to 15 columns further)
-constexpr float FW_LAZY = 8.f;            // log2 of how far a score may exceed its row's reference value
+constexpr float FW_LAZY = 64.f;           // log2 of how far a score may exceed its row's reference value
 constexpr int FW_TM_D = 128;              // attention: tensor-memory columns 0 / 64 scores, 128 / 192 outputs
 
 __device__ __forceinline__ bool grid_wait(const int* c, int want, volatile int* abort_flag) {
@@ -169,7 +169,7 @@ struct FwTail {
     float sl[2][4][16];                   // row sums of the softmax warps
     float sm[2][16];                      // row reference values
     uint64_t full[NS], empty[NS];
-    uint64_t tfull[2], tempty[2], sfull[2], pfull[2], ofull[2], oempty[2], qfull[2];
+    uint64_t tfull[2], tempty[2], sfull[2], pfull[2], ofull[2], oempty[2], qfull[2], lfull[2];
     uint32_t tmem_ptr;
     int abort_flag[2];
     int last[2];
@@ -509,6 +509,54 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
     return true;
 }
 
+// Merge of a (sequence, KV head)'s pieces by the 128 output threads of the block that arrived last: four output elements a
+// thread, the pieces in order (deterministic) and six at a time, so that their loads are in flight together.
+template <int HD, int NQP>
+__device__ __noinline__ void merge_pieces(const FwArgs& a, const FwTail& s, const AttnPos& q, int n_piece, int G, int kl) {
+    const int nrows = s.meta[q.bi].nrows, n_q = min(G * nrows, NQP);
+    for (int i = kl; i < n_q * (HD / 4); i += 128) {
+        const int r = i / (HD / 4), c4 = i % (HD / 4);
+        const int hq = G == 1 ? 0 : r / nrows, t = q.bi * a.R + r - hq * nrows, h = q.g * G + hq;
+        const size_t o = ((size_t)t * a.Hq + h) * a.pieces;
+        const float2* ml = reinterpret_cast<const float2*>(a.part + (size_t)a.T * a.Hq * a.pieces * HD) + o;
+        const float4* po = reinterpret_cast<const float4*>(a.part + o * HD) + c4;
+        constexpr int NP = 6;
+        float M = -CUDART_INF_F, ls = 0.f;
+        float4 o4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k0 = 0; k0 < n_piece; k0 += NP) {
+            float2 v[NP];
+            float4 y[NP];
+#pragma unroll
+            for (int k = 0; k < NP; ++k) {
+                const int kk = min(k0 + k, n_piece - 1);
+                v[k] = __ldcg(ml + kk);
+                y[k] = __ldcg(po + (size_t)kk * (HD / 4));
+                if (k0 + k >= n_piece) v[k].x = -CUDART_INF_F;
+            }
+            float mn = M;
+#pragma unroll
+            for (int k = 0; k < NP; ++k) mn = fmaxf(mn, v[k].x);
+            const float mz = mn == -CUDART_INF_F ? 0.f : mn;
+            const float fo = exp2f(M - mz);
+            ls *= fo;
+            o4.x *= fo; o4.y *= fo; o4.z *= fo; o4.w *= fo;
+            M = mn;
+#pragma unroll
+            for (int k = 0; k < NP; ++k) {
+                const float wg = exp2f(v[k].x - mz);
+                if (wg != 0.f) {                       // (a piece without a visible key wrote no sum worth multiplying)
+                    ls += wg * v[k].y;
+                    o4.x += wg * y[k].x; o4.y += wg * y[k].y; o4.z += wg * y[k].z; o4.w += wg * y[k].w;
+                }
+            }
+        }
+        const float f = 1.f / ls;
+        store_terms4(make_float4(o4.x * f, o4.y * f, o4.z * f, o4.w * f),
+                     a.x_a + (size_t)t * a.terms * a.Hq * HD + (size_t)h * HD + c4 * 4, (size_t)a.Hq * HD, a.terms);
+    }
+    if (kl == 0) a.acnt[q.bi * a.Hkv + q.g] = 0;       // ready for the next layer
+}
+
 template <int HD, int NQP, bool FEW>
 __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_constant__ FwArgs a) {
     constexpr int NCH = HD / 64;                       // 64-element chunks of a head row
@@ -551,6 +599,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
             mbar_init(smem_u32(&s.ofull[i]), 1);
             mbar_init(smem_u32(&s.oempty[i]), 4);
             mbar_init(smem_u32(&s.qfull[i]), 4);
+            mbar_init(smem_u32(&s.lfull[i]), 4);
         }
         s.abort_flag[0] = 0;
         s.abort_flag[1] = (int)(a.wait_limit ? a.wait_limit : WAIT_LIMIT);
@@ -799,37 +848,68 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 if (!ok) break;
                 pos += ring_qkv;
                 const int G = a.Hq / a.Hkv, kl = quad * 32 + lane;    // this thread's key of a tile, or its head dimension
-                float m[NQP], l[NQP], acc[NQP];
                 AttnPos it = a_first;
-                for (int i = 0; i < a_n; ++i) {
-                    const SeqMeta sm = s.meta[it.bi];
-                    const int nrows = sm.nrows, L = sm.L, nkeys = sm.nkeys;
-                    const int n_q = min(G * nrows, NQP);
-                    const int t0 = it.bi * a.R, h0 = it.g * G;        // query row r: row t0 + r % nrows, head h0 + r / nrows
-                    const bool fresh = i == 0 || it.tile == 0;
-                    const int b = at & 1;
-                    const uint32_t par = (uint32_t)(at >> 1) & 1u;
-                    if (fresh) {
+                if (half == 0) {
+                    // -------- softmax: a lane per key
+                    // query rows of (sequence, KV head) -> buffer `qb`, hi rows then lo rows, K-major; the first two segments'
+                    // go out at once, a later segment's when the one two before it has ended
+                    auto load_q = [&](const AttnPos& q, int qb) {
+                        const int nrows = s.meta[q.bi].nrows, n_q = min(G * nrows, NQP);
+                        uint8_t* dst = Qs + qb * Q_BYTES;
 #pragma unroll
-                        for (int r = 0; r < NQP; ++r) { m[r] = -CUDART_INF_F; l[r] = 0.f; acc[r] = 0.f; }
+                        for (int x = 0; x < NQ2 * (HD / 8) / 128; ++x) {
+                            const int idx = kl + x * 128, row = idx / (HD / 8), c = idx % (HD / 8), r = row & (NQP - 1);
+                            const bool valid = r < n_q;
+                            const int rr = valid ? r : 0, hq = G == 1 ? 0 : rr / nrows;
+                            const __nv_bfloat16* src = (row >= NQP ? a.q_lo : a.q_hi) +
+                                ((size_t)(q.bi * a.R + rr - hq * nrows) * a.Hq + q.g * G + hq) * HD + c * 8;
+                            cp_async16(smem_u32(dst + (c >> 3) * (NQ2 * 128) + row * 128 + (((c & 7) ^ (row & 7)) << 4)), src, valid);
+                        }
+                        asm volatile("cp.async.commit_group;" ::: "memory");
+                    };
+                    auto q_ready = [&](int qb) {
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&s.qfull[qb]));
+                    };
+                    // the segment that follows `q` in this block's range, if there is one (x: first item of q's segment end)
+                    AttnPos ahead = a_first;
+                    int ahead_i = 0;
+                    auto next_seg = [&]() -> bool {
+                        const int left = ahead.nt - ahead.tile;
+                        ahead_i += left;
+                        if (ahead_i >= a_n) return false;
+                        ahead.tile = ahead.nt - 1;
+                        attn_next(ahead, s.meta, a.B, a.Hkv);
+                        return true;
+                    };
+                    bool more = a_n > 0;
+                    if (more) {
+                        load_q(ahead, as & 1);
+                        more = next_seg();
+                        if (more) {
+                            load_q(ahead, (as + 1) & 1);
+                            asm volatile("cp.async.wait_group 1;" ::: "memory");
+                            q_ready(as & 1);
+                            asm volatile("cp.async.wait_group 0;" ::: "memory");
+                            q_ready((as + 1) & 1);
+                        } else {
+                            asm volatile("cp.async.wait_group 0;" ::: "memory");
+                            q_ready(as & 1);
+                        }
                     }
-                    if (half == 0) {
-                        // -------- softmax: a lane per key
+                    float m[NQP], l[NQP];
+                    for (int i = 0; i < a_n; ++i) {
+                        const SeqMeta sm = s.meta[it.bi];
+                        const int nrows = sm.nrows, L = sm.L, nkeys = sm.nkeys;
+                        const int n_q = min(G * nrows, NQP);
+                        const int t0 = it.bi * a.R;                   // query row r: row t0 + r % nrows, head g * G + r / nrows
+                        const bool fresh = i == 0 || it.tile == 0;
+                        const int b = at & 1;
+                        const uint32_t par = (uint32_t)(at >> 1) & 1u;
                         if (fresh) {
-                            uint8_t* q = Qs + (as & 1) * Q_BYTES;
 #pragma unroll
-                            for (int x = 0; x < NQ2 * (HD / 8) / 128; ++x) {
-                                const int idx = kl + x * 128, row = idx / (HD / 8), c = idx % (HD / 8), r = row & (NQP - 1);
-                                const bool valid = r < n_q;
-                                const int rr = valid ? r : 0, hq = G == 1 ? 0 : rr / nrows;
-                                const __nv_bfloat16* src = (row >= NQP ? a.q_lo : a.q_hi) +
-                                    ((size_t)(t0 + rr - hq * nrows) * a.Hq + h0 + hq) * HD + c * 8;
-                                cp_async16(smem_u32(q + (c >> 3) * (NQ2 * 128) + row * 128 + (((c & 7) ^ (row & 7)) << 4)), src, valid);
-                            }
-                            asm volatile("cp.async.wait_all;" ::: "memory");
-                            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(smem_u32(&s.qfull[as & 1]));
+                            for (int r = 0; r < NQP; ++r) { m[r] = -CUDART_INF_F; l[r] = 0.f; }
                         }
                         const int j = it.tile * FW_KEYS + kl;
                         // which query rows see this thread's key: all of a committed one; of a draft row those that have it
@@ -858,8 +938,9 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             for (int r = 0; r < NQP; ++r) v[r] = ((vis >> r) & 1u) ? c[r] + c[NQP + r] : -CUDART_INF_F;
                         }
                         // The reference value m of a row follows its maximum lazily: it moves only when a score exceeds it by
-                        // more than 2^8 (numerators and sums stay well inside fp32, and bf16 hi + lo keep their precision), so
-                        // the row maxima over 128 lanes are formed on a segment's first tile and hardly ever after.
+                        // more than 2^64 (numerators and sums stay well inside the exponent range that fp32 and bf16 share, and
+                        // a common factor costs no precision), so the row maxima over 128 lanes are formed on a segment's first
+                        // tile and hardly ever after.
                         bool calm = !fresh;
 #pragma unroll
                         for (int r = 0; r < NQP; ++r) {
@@ -919,24 +1000,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(smem_u32(&s.pfull[b]));
-                    } else {
-                        // -------- output: a lane per head dimension
-                        ok = warp_wait(smem_u32(&s.ofull[b]), par, abort_flag, ok, lane);
-                        tc_fence_after();
-                        float c[NQ2];
-                        if (NQ2 == 16) tc_ld16(t_lane + FW_TM_D + b * 64, c);
-                        else { tc_ld16(t_lane + FW_TM_D + b * 64, c); tc_ld16(t_lane + FW_TM_D + b * 64 + 16, c + 16); }
-#pragma unroll
-                        for (int r = 0; r < NQP; ++r) acc[r] = acc[r] * s.sf[b][r] + (c[r] + c[NQP + r]);
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&s.oempty[b]));
-                    }
-                    ++at;
-                    if (i + 1 == a_n || it.tile + 1 == it.nt) {
-                        // -------- end of a segment: the row sums meet, then the rows leave (final, or as a piece)
-                        const int sb = as & 1;
-                        if (half == 0) {
+                        ++at;
+                        if (i + 1 == a_n || it.tile + 1 == it.nt) {
+                            // -------- end of a segment: the rows' sums and reference values for the output warps
+                            const int sb = as & 1;
 #pragma unroll
                             for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
@@ -946,97 +1013,83 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                                 if (lane == r) s.sl[sb][quad][r] = l[r];
                                 if (kl == r) s.sm[sb][r] = m[r];
                             }
-                        }
-                        const int first = it.f0 / a_per, n_piece = (it.f0 + it.nt - 1) / a_per - first + 1, piece = cta - first;
-                        ok = all_of(1, FW_EPI, ok);
-                        if (half == 1 && ok && (HD == 128 || kl < HD)) {
-#pragma unroll
-                            for (int r = 0; r < NQP; ++r) {
-                                if (r >= n_q) continue;
-                                const int hq = G == 1 ? 0 : r / nrows, t = t0 + r - hq * nrows, h = h0 + hq;
-                                const float ls = (s.sl[sb][0][r] + s.sl[sb][1][r]) + (s.sl[sb][2][r] + s.sl[sb][3][r]);
-                                if (n_piece == 1) {
-                                    store_terms(acc[r] / ls, a.x_a + (size_t)t * terms * a.Hq * HD + (size_t)h * HD + kl,
-                                                (size_t)a.Hq * HD, terms);
-                                } else {
-                                    const size_t o = ((size_t)t * a.Hq + h) * a.pieces + piece;
-                                    a.part[o * HD + kl] = acc[r];
-                                    if (kl == 0)
-                                        reinterpret_cast<float2*>(a.part + (size_t)T * a.Hq * a.pieces * HD)[o] = make_float2(s.sm[sb][r], ls);
-                                }
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(smem_u32(&s.lfull[sb]));
+                            // the scores of this segment are formed, its query buffer is free
+                            if (more) more = next_seg();
+                            if (more) {
+                                load_q(ahead, sb);
+                                asm volatile("cp.async.wait_group 0;" ::: "memory");
+                                q_ready(sb);
                             }
+                            ++as;
                         }
-                        ++as;
+                        if (i + 1 < a_n) attn_next(it, s.meta, a.B, a.Hkv);
                     }
-                    if (i + 1 < a_n) attn_next(it, s.meta, a.B, a.Hkv);
-                }
-                pos += 2 * a_n + ring_other;
-                // pieces shared with other blocks (at most the first and the last segment): the last to arrive merges
-                if (a_n > 0) {
-                    ok = all_of(1, FW_EPI, ok);
-                    if (!ok) break;
-                    if (e < 2) {
-                        const AttnPos q = e == 0 ? a_first : it;
-                        const int n_piece = (q.f0 + q.nt - 1) / a_per - q.f0 / a_per + 1;
-                        int last = 0;
-                        if (n_piece > 1 && (e == 0 || it.f0 != a_first.f0)) {
-                            int old;
-                            asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;"
-                                         : "=r"(old) : "l"(a.acnt + q.bi * a.Hkv + q.g) : "memory");
-                            last = old + 1 == n_piece;
+                } else {
+                    // -------- output: a lane per head dimension
+                    float acc[NQP];
+                    for (int i = 0; i < a_n; ++i) {
+                        const int nrows = s.meta[it.bi].nrows, n_q = min(G * nrows, NQP);
+                        const int t0 = it.bi * a.R, h0 = it.g * G;
+                        const bool fresh = i == 0 || it.tile == 0, ends = i + 1 == a_n || it.tile + 1 == it.nt;
+                        const int b = at & 1, sb = as & 1;
+                        if (fresh) {
+#pragma unroll
+                            for (int r = 0; r < NQP; ++r) acc[r] = 0.f;
                         }
-                        s.last[e] = last;
-                    }
-                    bar_n(1, FW_EPI);
-                    for (int x = 0; x < 2; ++x) {
-                        if (!s.last[x]) continue;
-                        const AttnPos q = x == 0 ? a_first : it;
-                        const int nrows = s.meta[q.bi].nrows, n_q = min(G * nrows, NQP);
-                        const int n_piece = (q.f0 + q.nt - 1) / a_per - q.f0 / a_per + 1;
-                        for (int i = e; i < n_q * (HD / 4); i += FW_EPI) {
-                            const int r = i / (HD / 4), c4 = i % (HD / 4);
-                            const int hq = G == 1 ? 0 : r / nrows, t = q.bi * a.R + r - hq * nrows, h = q.g * G + hq;
-                            const size_t o = ((size_t)t * a.Hq + h) * a.pieces;
-                            const float2* ml = reinterpret_cast<const float2*>(a.part + (size_t)T * a.Hq * a.pieces * HD) + o;
-                            const float4* po = reinterpret_cast<const float4*>(a.part + o * HD) + c4;
-                            // pieces in order (deterministic), six at a time: their loads are in flight together
-                            constexpr int NP = 6;
-                            float M = -CUDART_INF_F, ls = 0.f;
-                            float4 o4 = make_float4(0.f, 0.f, 0.f, 0.f);
-                            for (int k0 = 0; k0 < n_piece; k0 += NP) {
-                                float2 v[NP];
-                                float4 y[NP];
+                        ok = warp_wait(smem_u32(&s.ofull[b]), (uint32_t)(at >> 1) & 1u, abort_flag, ok, lane);
+                        tc_fence_after();
+                        float c[NQ2];
+                        if (NQ2 == 16) tc_ld16(t_lane + FW_TM_D + b * 64, c);
+                        else { tc_ld16(t_lane + FW_TM_D + b * 64, c); tc_ld16(t_lane + FW_TM_D + b * 64 + 16, c + 16); }
 #pragma unroll
-                                for (int k = 0; k < NP; ++k) {
-                                    const int kk = min(k0 + k, n_piece - 1);
-                                    v[k] = __ldcg(ml + kk);
-                                    y[k] = __ldcg(po + (size_t)kk * (HD / 4));
-                                    if (k0 + k >= n_piece) v[k].x = -CUDART_INF_F;
-                                }
-                                float mn = M;
+                        for (int r = 0; r < NQP; ++r) acc[r] = acc[r] * s.sf[b][r] + (c[r] + c[NQP + r]);
+                        if (ends) {
+                            // the rows leave: final, or as a piece that the block arriving last merges with the others
+                            const int first = it.f0 / a_per, n_piece = (it.f0 + it.nt - 1) / a_per - first + 1, piece = cta - first;
+                            ok = warp_wait(smem_u32(&s.lfull[sb]), (uint32_t)(as >> 1) & 1u, abort_flag, ok, lane);
+                            if (ok && (HD == 128 || kl < HD)) {
 #pragma unroll
-                                for (int k = 0; k < NP; ++k) mn = fmaxf(mn, v[k].x);
-                                const float mz = mn == -CUDART_INF_F ? 0.f : mn;
-                                const float fo = exp2f(M - mz);
-                                ls *= fo;
-                                o4.x *= fo; o4.y *= fo; o4.z *= fo; o4.w *= fo;
-                                M = mn;
-#pragma unroll
-                                for (int k = 0; k < NP; ++k) {
-                                    const float wg = exp2f(v[k].x - mz);
-                                    if (wg != 0.f) {
-                                        ls += wg * v[k].y;
-                                        o4.x += wg * y[k].x; o4.y += wg * y[k].y; o4.z += wg * y[k].z; o4.w += wg * y[k].w;
+                                for (int r = 0; r < NQP; ++r) {
+                                    if (r >= n_q) break;
+                                    const int hq = G == 1 ? 0 : r / nrows, t = t0 + r - hq * nrows, h = h0 + hq;
+                                    const float ls = (s.sl[sb][0][r] + s.sl[sb][1][r]) + (s.sl[sb][2][r] + s.sl[sb][3][r]);
+                                    if (n_piece == 1) {
+                                        store_terms(acc[r] / ls, a.x_a + (size_t)t * terms * a.Hq * HD + (size_t)h * HD + kl,
+                                                    (size_t)a.Hq * HD, terms);
+                                    } else {
+                                        const size_t o = ((size_t)t * a.Hq + h) * a.pieces + piece;
+                                        a.part[o * HD + kl] = acc[r];
+                                        if (kl == 0)
+                                            reinterpret_cast<float2*>(a.part + (size_t)T * a.Hq * a.pieces * HD)[o] =
+                                                make_float2(s.sm[sb][r], ls);
                                     }
                                 }
                             }
-                            const float f = 1.f / ls;
-                            store_terms4(make_float4(o4.x * f, o4.y * f, o4.z * f, o4.w * f),
-                                         a.x_a + (size_t)t * terms * a.Hq * HD + (size_t)h * HD + c4 * 4, (size_t)a.Hq * HD, terms);
+                            if (n_piece > 1) {
+                                bar_n(3, 128);
+                                if (kl == 0) {
+                                    int old;
+                                    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;"
+                                                 : "=r"(old) : "l"(a.acnt + it.bi * a.Hkv + it.g) : "memory");
+                                    s.last[0] = old + 1 == n_piece;
+                                }
+                                bar_n(3, 128);
+                                if (s.last[0]) merge_pieces<HD, NQP>(a, s, it, n_piece, G, kl);
+                            }
+                            ++as;
                         }
-                        if (e == 0) a.acnt[q.bi * a.Hkv + q.g] = 0;       // ready for the next layer
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&s.oempty[b]));
+                        ++at;
+                        if (i + 1 < a_n) attn_next(it, s.meta, a.B, a.Hkv);
                     }
                 }
+                pos += 2 * a_n + ring_other;
+                ok = all_of(1, FW_EPI, ok);
+                if (!ok) break;
             } else if (kind == FW_QKV) {
                 ok = epi_phase<FW_QKV, HD, FEW>(a, s, Y, p, layer, tcount, e, t_lane, cta);
             } else if (kind == FW_O) {
