@@ -18,12 +18,12 @@
 //
 // Attention: keys as the M dimension.  The (sequence, KV head, 128-key tile) items are dealt out evenly, in order.
 //   S^T = K Q^T   A = K tile as it lies in the cache, B = query rows (bf16 hi rows, then lo rows)
-//   P = exp2(S - m), a thread per key, written to shared memory as bf16 hi and lo
-//   O^T += V^T P  A = V tile (MN-major), B = P; a thread per head dimension adds it to its registers
+//   P = exp2(S - m), a thread per key and half of the query rows, written to shared memory as bf16 hi and lo
+//   O^T += V^T P  A = V tile (MN-major), B = P; a thread per head dimension and half of the rows adds it to its registers
 // Pieces of a (sequence, KV head) held by several blocks meet in global memory; the block that arrives last merges them.
 //
 // Warps: 0 weight and K / V producer (TMA), 1 operand-row producer (TMA; waits for the phase before), 2 and 3 MMA issuers
-// (3 owns the tensor memory), 4..11 epilogue; in the attention 4..7 softmax (a lane per key) and 8..11 output (a lane per dimension).
+// (3 owns the tensor memory), 4..11 epilogue and softmax.
 // Every wait is bounded; a block that gives up raises MTAD_ST_TIMEOUT for every sequence of the call and leaves, and the
 // others run into their own limits at the grid barrier.
 #include <math_constants.h>
@@ -164,17 +164,16 @@ struct FwTail {
     float rstd[FW_MAX_ROWS];
     int slot[FW_MAX_ROWS];                // cache slot of a row, -1: inactive
     uint8_t rowb[FW_MAX_ROWS];            // its sequence within the call
-    alignas(16) float smx[2][16][4];           // row maxima of the four softmax warps
-    float sf[2][16];                      // rescale factor of the running output, per tile buffer
-    float sl[2][4][16];                   // row sums of the softmax warps
-    float sm[2][16];                      // row reference values
+    alignas(16) float smx[2][8][4];       // attention, per half of the rows: row maxima of the four warps
+    alignas(16) float sl[2][2][8][4];     // row sums of the four warps, two segments
+    float sm[2][8];                       // first scores of a segment
     uint64_t full[NS], empty[NS];
-    uint64_t tfull[2], tempty[2], sfull[2], pfull[2], ofull[2], oempty[2], qfull[2], lfull[2];
+    uint64_t tfull[2], tempty[2], sfull[2], pfull[2], ofull[2], qfull[2];
     uint32_t tmem_ptr;
     int abort_flag[2];
     int last[2];
 };
-static_assert(offsetof(FwTail, smx) % 16 == 0 && offsetof(FwTail, full) % 8 == 0, "alignment of the tail");
+static_assert(offsetof(FwTail, smx) % 16 == 0 && offsetof(FwTail, sl) % 16 == 0 && offsetof(FwTail, full) % 8 == 0, "alignment of the tail");
 static_assert(NS * FW_SLOT + FW_UNION + sizeof(FwTail) <= 227 * 1024, "shared memory of the forward");
 
 // The epilogue group's part of one projection: row statistics, then per tile the accumulators -> Y in shared memory ->
@@ -509,12 +508,12 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
     return true;
 }
 
-// Merge of a (sequence, KV head)'s pieces by the 128 output threads of the block that arrived last: four output elements a
+// Merge of a (sequence, KV head)'s pieces by the epilogue threads of the block that arrived last: four output elements a
 // thread, the pieces in order (deterministic) and six at a time, so that their loads are in flight together.
 template <int HD, int NQP>
-__device__ __noinline__ void merge_pieces(const FwArgs& a, const FwTail& s, const AttnPos& q, int n_piece, int G, int kl) {
+__device__ __forceinline__ void merge_pieces(const FwArgs& a, const FwTail& s, const AttnPos& q, int n_piece, int G, int e) {
     const int nrows = s.meta[q.bi].nrows, n_q = min(G * nrows, NQP);
-    for (int i = kl; i < n_q * (HD / 4); i += 128) {
+    for (int i = e; i < n_q * (HD / 4); i += FW_EPI) {
         const int r = i / (HD / 4), c4 = i % (HD / 4);
         const int hq = G == 1 ? 0 : r / nrows, t = q.bi * a.R + r - hq * nrows, h = q.g * G + hq;
         const size_t o = ((size_t)t * a.Hq + h) * a.pieces;
@@ -554,7 +553,7 @@ __device__ __noinline__ void merge_pieces(const FwArgs& a, const FwTail& s, cons
         store_terms4(make_float4(o4.x * f, o4.y * f, o4.z * f, o4.w * f),
                      a.x_a + (size_t)t * a.terms * a.Hq * HD + (size_t)h * HD + c4 * 4, (size_t)a.Hq * HD, a.terms);
     }
-    if (kl == 0) a.acnt[q.bi * a.Hkv + q.g] = 0;       // ready for the next layer
+    if (e == 0) a.acnt[q.bi * a.Hkv + q.g] = 0;       // ready for the next layer
 }
 
 template <int HD, int NQP, bool FEW>
@@ -595,11 +594,9 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
             mbar_init(smem_u32(&s.tfull[i]), 2);
             mbar_init(smem_u32(&s.tempty[i]), 8);
             mbar_init(smem_u32(&s.sfull[i]), 1);
-            mbar_init(smem_u32(&s.pfull[i]), 4);
+            mbar_init(smem_u32(&s.pfull[i]), 8);
             mbar_init(smem_u32(&s.ofull[i]), 1);
-            mbar_init(smem_u32(&s.oempty[i]), 4);
-            mbar_init(smem_u32(&s.qfull[i]), 4);
-            mbar_init(smem_u32(&s.lfull[i]), 4);
+            mbar_init(smem_u32(&s.qfull[i]), 8);
         }
         s.abort_flag[0] = 0;
         s.abort_flag[1] = (int)(a.wait_limit ? a.wait_limit : WAIT_LIMIT);
@@ -620,7 +617,16 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     for (int b = 0; b < a.B; ++b) a_tot += attn_tiles(s.meta[b]) * a.Hkv;
     const int a_per = max(1, (a_tot + n_cta - 1) / n_cta);
     const int a_lo = min(cta * a_per, a_tot), a_n = min(a_lo + a_per, a_tot) - a_lo;
-    const AttnPos a_first = attn_find(s.meta, a.B, a.Hkv, a_lo);
+    // This block's items in the order it takes them: if its range holds more than one segment (run of tiles of one sequence
+    // and KV head), the first segment comes last, because it ends with the tile that holds the call's own rows and cannot
+    // be requested before the phase has been released.  a_wrap: where the order returns to the front of the range.
+    const AttnPos a_zero = attn_find(s.meta, a.B, a.Hkv, a_lo), a_last = attn_find(s.meta, a.B, a.Hkv, max(a_lo, a_lo + a_n - 1));
+    const int a_rot = a_zero.nt - a_zero.tile < a_n ? a_zero.nt - a_zero.tile : 0, a_wrap = a_n - a_rot;
+    const AttnPos a_first = a_rot ? attn_find(s.meta, a.B, a.Hkv, a_lo + a_rot) : a_zero;
+    auto attn_step = [&](AttnPos& it, int next) {          // item `next` of the order, from the one before
+        if (next == a_wrap) it = a_zero;
+        else attn_next(it, s.meta, a.B, a.Hkv);
+    };
     auto slot_ptr = [&](int pos) { return smem_u32(smem) + (uint32_t)(pos % NS) * FW_SLOT; };
     auto full_bar = [&](int pos) { return smem_u32(&s.full[pos % NS]); };
     auto empty_bar = [&](int pos) { return smem_u32(&s.empty[pos % NS]); };
@@ -640,7 +646,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 if (kind == FW_ATTN) {
                     bool waited = false;
                     AttnPos it = a_first;
-                    for (int i = 0; i < a_n && ok; ++i, attn_next(it, s.meta, a.B, a.Hkv)) {
+                    for (int i = 0; i < a_n && ok; attn_step(it, ++i)) {
                         const SeqMeta sm = s.meta[it.bi];
                         const int plane = ((layer * a.max_batch + sm.seq) * 2) * a.Hkv + it.g;
                         if (!waited && (it.tile + 1) * FW_KEYS > sm.L) {
@@ -747,8 +753,8 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 if (me == 0) {
                     constexpr uint32_t idesc_s = IDESC | ((uint32_t)(NQ2 >> 3) << 17);
                     AttnPos it = a_first;
-                    for (int i = 0; i < a_n; ++i, attn_next(it, s.meta, a.B, a.Hkv)) {
-                        const bool fresh = i == 0 || it.tile == 0;
+                    for (int i = 0; i < a_n; attn_step(it, ++i)) {
+                        const bool fresh = i == 0 || i == a_wrap || it.tile == 0;
                         if (fresh && i > 0) ++as;
                         const int kpos = pos + 2 * i, b = (at + i) & 1;
                         // query rows of the segment, the K tile, and the score buffer (read by the softmax two tiles ago)
@@ -772,9 +778,9 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     for (int i = 0; i < a_n; ++i) {
                         const int vpos = pos + 2 * i + 1, b = (at + i) & 1;
                         const uint32_t par = (uint32_t)((at + i) >> 1) & 1u;
+                        // (the probabilities' arrival also says that every epilogue warp has read the output two tiles ago)
                         ok = mbar_wait_warp(smem_u32(&s.pfull[b]), par, abort_flag) &&
-                             mbar_wait_warp(full_bar(vpos), ring_par(vpos), abort_flag) &&
-                             mbar_wait_warp(smem_u32(&s.oempty[b]), par ^ 1u, abort_flag);
+                             mbar_wait_warp(full_bar(vpos), ring_par(vpos), abort_flag);
                         if (!ok) break;
                         tc_fence_after();
                         const uint64_t va = smem_desc_mn(slot_ptr(vpos)), pa = smem_desc(smem_u32(Ps) + b * P_BYTES);
@@ -847,249 +853,253 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 ok = all_of(1, FW_EPI, ok);
                 if (!ok) break;
                 pos += ring_qkv;
-                const int G = a.Hq / a.Hkv, kl = quad * 32 + lane;    // this thread's key of a tile, or its head dimension
-                AttnPos it = a_first;
-                if (half == 0) {
-                    // -------- softmax: a lane per key
-                    // query rows of (sequence, KV head) -> buffer `qb`, hi rows then lo rows, K-major; the first two segments'
-                    // go out at once, a later segment's when the one two before it has ended
-                    auto load_q = [&](const AttnPos& q, int qb) {
-                        const int nrows = s.meta[q.bi].nrows, n_q = min(G * nrows, NQP);
-                        uint8_t* dst = Qs + qb * Q_BYTES;
+                const int G = a.Hq / a.Hkv, kl = quad * 32 + lane;    // this thread's key of a tile, later its head dimension
+                constexpr int NR = NQP / 2;                           // this thread's query rows: half, half + 2, ...
+                // query rows of (sequence, KV head) -> buffer `qb`, hi rows then lo rows, K-major
+                auto load_q = [&](const AttnPos& q, int qb) {
+                    const int nrows = s.meta[q.bi].nrows, n_q = min(G * nrows, NQP);
+                    uint8_t* dst = Qs + qb * Q_BYTES;
 #pragma unroll
-                        for (int x = 0; x < NQ2 * (HD / 8) / 128; ++x) {
-                            const int idx = kl + x * 128, row = idx / (HD / 8), c = idx % (HD / 8), r = row & (NQP - 1);
-                            const bool valid = r < n_q;
-                            const int rr = valid ? r : 0, hq = G == 1 ? 0 : rr / nrows;
-                            const __nv_bfloat16* src = (row >= NQP ? a.q_lo : a.q_hi) +
-                                ((size_t)(q.bi * a.R + rr - hq * nrows) * a.Hq + q.g * G + hq) * HD + c * 8;
-                            cp_async16(smem_u32(dst + (c >> 3) * (NQ2 * 128) + row * 128 + (((c & 7) ^ (row & 7)) << 4)), src, valid);
-                        }
-                        asm volatile("cp.async.commit_group;" ::: "memory");
-                    };
-                    auto q_ready = [&](int qb) {
-                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&s.qfull[qb]));
-                    };
-                    // the segment that follows `q` in this block's range, if there is one (x: first item of q's segment end)
-                    AttnPos ahead = a_first;
-                    int ahead_i = 0;
-                    auto next_seg = [&]() -> bool {
-                        const int left = ahead.nt - ahead.tile;
-                        ahead_i += left;
-                        if (ahead_i >= a_n) return false;
-                        ahead.tile = ahead.nt - 1;
-                        attn_next(ahead, s.meta, a.B, a.Hkv);
-                        return true;
-                    };
-                    bool more = a_n > 0;
+                    for (int idx = e; idx < NQ2 * (HD / 8); idx += FW_EPI) {
+                        const int row = idx / (HD / 8), c = idx % (HD / 8), r = row & (NQP - 1);
+                        const bool valid = r < n_q;
+                        const int rr = valid ? r : 0, hq = G == 1 ? 0 : rr / nrows;
+                        const __nv_bfloat16* src = (row >= NQP ? a.q_lo : a.q_hi) +
+                            ((size_t)(q.bi * a.R + rr - hq * nrows) * a.Hq + q.g * G + hq) * HD + c * 8;
+                        cp_async16(smem_u32(dst + (c >> 3) * (NQ2 * 128) + row * 128 + (((c & 7) ^ (row & 7)) << 4)), src, valid);
+                    }
+                    asm volatile("cp.async.commit_group;" ::: "memory");
+                };
+                auto q_ready = [&](int qb) {
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&s.qfull[qb]));
+                };
+                // the first two segments' query rows go out at once, a later segment's when the one two before it has ended
+                AttnPos ahead = a_first;
+                int ahead_i = 0;
+                bool more = a_n > 0;
+                auto next_seg = [&]() {
+                    const int n = min(ahead.nt - ahead.tile, (ahead_i < a_wrap ? a_wrap : a_n) - ahead_i);
+                    ahead.tile += n - 1;
+                    ahead_i += n;
+                    more = ahead_i < a_n;
+                    if (more) attn_step(ahead, ahead_i);
+                };
+                if (more) {
+                    load_q(ahead, as & 1);
+                    next_seg();
                     if (more) {
-                        load_q(ahead, as & 1);
-                        more = next_seg();
-                        if (more) {
-                            load_q(ahead, (as + 1) & 1);
-                            asm volatile("cp.async.wait_group 1;" ::: "memory");
-                            q_ready(as & 1);
-                            asm volatile("cp.async.wait_group 0;" ::: "memory");
-                            q_ready((as + 1) & 1);
-                        } else {
-                            asm volatile("cp.async.wait_group 0;" ::: "memory");
-                            q_ready(as & 1);
-                        }
+                        load_q(ahead, (as + 1) & 1);
+                        asm volatile("cp.async.wait_group 1;" ::: "memory");
+                        q_ready(as & 1);
+                        asm volatile("cp.async.wait_group 0;" ::: "memory");
+                        q_ready((as + 1) & 1);
+                    } else {
+                        asm volatile("cp.async.wait_group 0;" ::: "memory");
+                        q_ready(as & 1);
                     }
-                    float m[NQP], l[NQP];
-                    for (int i = 0; i < a_n; ++i) {
-                        const SeqMeta sm = s.meta[it.bi];
-                        const int nrows = sm.nrows, L = sm.L, nkeys = sm.nkeys;
-                        const int n_q = min(G * nrows, NQP);
-                        const int t0 = it.bi * a.R;                   // query row r: row t0 + r % nrows, head g * G + r / nrows
-                        const bool fresh = i == 0 || it.tile == 0;
-                        const int b = at & 1;
-                        const uint32_t par = (uint32_t)(at >> 1) & 1u;
-                        if (fresh) {
+                }
+                AttnPos it = a_first;
+                float m[NR], l[NR], acc[NR];
+                // output of the tile before: this thread's head dimension of its rows, out of tensor memory
+                auto output = [&](int tile_no) {
+                    const int b = tile_no & 1;
+                    ok = warp_wait(smem_u32(&s.ofull[b]), (uint32_t)(tile_no >> 1) & 1u, abort_flag, ok, lane);
+                    tc_fence_after();
+                    float c[NQ2];
+                    if (NQ2 == 16) tc_ld16(t_lane + FW_TM_D + b * 64, c);
+                    else { tc_ld16(t_lane + FW_TM_D + b * 64, c); tc_ld16(t_lane + FW_TM_D + b * 64 + 16, c + 16); }
 #pragma unroll
-                            for (int r = 0; r < NQP; ++r) { m[r] = -CUDART_INF_F; l[r] = 0.f; }
-                        }
-                        const int j = it.tile * FW_KEYS + kl;
-                        // which query rows see this thread's key: all of a committed one; of a draft row those that have it
-                        // among their ancestors and themselves; none past the last key
-                        uint32_t vis = 0xffffffffu;
-                        if ((it.tile + 1) * FW_KEYS > L) {
-                            const int sr = j - L;
-                            vis = j < nkeys ? 0xffffffffu : 0u;
-                            if (sr >= 0 && vis) {
-                                vis = 0;
+                    for (int x = 0; x < NR; ++x)
+                        acc[x] += half == 0 ? c[2 * x] + c[NQP + 2 * x] : c[2 * x + 1] + c[NQP + 2 * x + 1];
+                };
+                // end of a segment: the rows' sums over the lanes, then the rows leave - final, or as a piece
+                auto finish = [&](const AttnPos& q) {
+                    const int sb = as & 1;
 #pragma unroll
-                                for (int r = 0; r < NQP; ++r) {
-                                    const int rr = r < n_q ? (G == 1 ? r : r % nrows) : 0;
-                                    vis |= ((a.rm.mask[(size_t)(t0 + rr) * MTAD_MASK_WORDS + (sr >> 5)] >> (sr & 31)) & 1u) << r;
+                    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                        for (int x = 0; x < NR; ++x) l[x] += __shfl_xor_sync(0xffffffffu, l[x], o);
+#pragma unroll
+                    for (int x = 0; x < NR; ++x)
+                        if (lane == x) s.sl[sb][half][x][quad] = l[x];
+                    ok = all_of(2 + half, 128, ok);
+                    const int nrows = s.meta[q.bi].nrows, n_q = min(G * nrows, NQP);
+                    const int first = q.f0 / a_per, n_piece = (q.f0 + q.nt - 1) / a_per - first + 1, piece = cta - first;
+                    if (ok && (HD == 128 || kl < HD)) {
+#pragma unroll
+                        for (int x = 0; x < NR; ++x) {
+                            const int r = 2 * x + half;
+                            if (r < n_q) {
+                                const int hq = G == 1 ? 0 : r / nrows, t = q.bi * a.R + r - hq * nrows, h = q.g * G + hq;
+                                const float4 l4 = *reinterpret_cast<const float4*>(s.sl[sb][half][x]);
+                                const float ls = (l4.x + l4.y) + (l4.z + l4.w);
+                                if (n_piece == 1) {
+                                    store_terms(acc[x] / ls, a.x_a + (size_t)t * terms * a.Hq * HD + (size_t)h * HD + kl,
+                                                (size_t)a.Hq * HD, terms);
+                                } else {
+                                    const size_t o = ((size_t)t * a.Hq + h) * a.pieces + piece;
+                                    a.part[o * HD + kl] = acc[x];
+                                    if (kl == 0)
+                                        reinterpret_cast<float2*>(a.part + (size_t)T * a.Hq * a.pieces * HD)[o] = make_float2(m[x], ls);
                                 }
                             }
                         }
-                        ok = warp_wait(smem_u32(&s.sfull[b]), par, abort_flag, ok, lane);
-                        tc_fence_after();
-                        float v[NQP];
-                        {
-                            float c[NQ2];
-                            if (NQ2 == 16) tc_ld16(t_lane + b * 64, c);
-                            else { tc_ld16(t_lane + b * 64, c); tc_ld16(t_lane + b * 64 + 16, c + 16); }
-#pragma unroll
-                            for (int r = 0; r < NQP; ++r) v[r] = ((vis >> r) & 1u) ? c[r] + c[NQP + r] : -CUDART_INF_F;
-                        }
-                        // The reference value m of a row follows its maximum lazily: it moves only when a score exceeds it by
-                        // more than 2^64 (numerators and sums stay well inside the exponent range that fp32 and bf16 share, and
-                        // a common factor costs no precision), so the row maxima over 128 lanes are formed on a segment's first
-                        // tile and hardly ever after.
-                        bool calm = !fresh;
-#pragma unroll
-                        for (int r = 0; r < NQP; ++r) {
-                            if (r >= n_q) break;
-                            calm = calm && v[r] <= m[r] + FW_LAZY;
-                        }
-                        // the buffers P and sf of this tile are free once the output warps are done with the tile before the last
-                        ok = warp_wait(smem_u32(&s.oempty[b]), par ^ 1u, abort_flag, ok, lane);
-                        if (!all_of(2, 128, calm && ok)) {
-                            float wm[NQP];
-#pragma unroll
-                            for (int r = 0; r < NQP; ++r) wm[r] = v[r];
-#pragma unroll
-                            for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                                for (int r = 0; r < NQP; ++r) wm[r] = fmaxf(wm[r], __shfl_xor_sync(0xffffffffu, wm[r], o));
-#pragma unroll
-                            for (int r = 0; r < NQP; ++r)
-                                if (lane == r) s.smx[b][r][quad] = wm[r];
-                            ok = all_of(2, 128, ok);
-#pragma unroll
-                            for (int r = 0; r < NQP; ++r) {
-                                const float4 q4 = *reinterpret_cast<const float4*>(s.smx[b][r]);
-                                const float mn = fmaxf(m[r], fmaxf(fmaxf(q4.x, q4.y), fmaxf(q4.z, q4.w)));
-                                const float f = mn == -CUDART_INF_F ? 1.f : exp2f(m[r] - mn);
-                                m[r] = mn;
-                                l[r] *= f;
-                                if (kl == r) s.sf[b][r] = f;
-                            }
-                        } else if (kl < NQP) {
-                            s.sf[b][kl] = 1.f;
-                        }
-                        uint8_t* pt = Ps + b * P_BYTES + (kl >> 6) * (NQ2 * 128) + (kl & 7) * 2;
-                        const int pc = (kl & 63) >> 3;
-#pragma unroll
-                        for (int r = 0; r < NQP; ++r) {
-                            if (r >= n_q) break;                              // (rows without a query: their output columns are not read)
-                            const float pv = exp2f(v[r] - (m[r] == -CUDART_INF_F ? 0.f : m[r]));        // exp2(-inf) = 0
-                            l[r] += pv;
-                            const __nv_bfloat16 hi = __float2bfloat16_rn(pv);
-                            uint8_t* d = pt + ((pc ^ (r & 7)) << 4);
-                            *reinterpret_cast<__nv_bfloat16*>(d + r * 128) = hi;
-                            *reinterpret_cast<__nv_bfloat16*>(d + (NQP + r) * 128) = __float2bfloat16_rn(pv - __bfloat162float(hi));
-                        }
-                        if ((it.tile + 1) * FW_KEYS > nkeys) {
-                            // rows of V past the last key: their probabilities are 0, but 0 x (stale value) must not make a NaN
-                            const int vpos = pos + 2 * i + 1;
-                            ok = warp_wait(full_bar(vpos), ring_par(vpos), abort_flag, ok, lane);
-                            if (ok && j >= nkeys) {
-                                uint8_t* vs = smem + (size_t)(vpos % NS) * FW_SLOT + kl * 128;
-#pragma unroll
-                                for (int c = 0; c < NCH * 8; ++c)
-                                    *reinterpret_cast<uint4*>(vs + (c >> 3) * (FW_KEYS * 128) + (c & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
-                            }
-                        }
-                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&s.pfull[b]));
-                        ++at;
-                        if (i + 1 == a_n || it.tile + 1 == it.nt) {
-                            // -------- end of a segment: the rows' sums and reference values for the output warps
-                            const int sb = as & 1;
-#pragma unroll
-                            for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                                for (int r = 0; r < NQP; ++r) l[r] += __shfl_xor_sync(0xffffffffu, l[r], o);
-#pragma unroll
-                            for (int r = 0; r < NQP; ++r) {
-                                if (lane == r) s.sl[sb][quad][r] = l[r];
-                                if (kl == r) s.sm[sb][r] = m[r];
-                            }
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(smem_u32(&s.lfull[sb]));
-                            // the scores of this segment are formed, its query buffer is free
-                            if (more) more = next_seg();
-                            if (more) {
-                                load_q(ahead, sb);
-                                asm volatile("cp.async.wait_group 0;" ::: "memory");
-                                q_ready(sb);
-                            }
-                            ++as;
-                        }
-                        if (i + 1 < a_n) attn_next(it, s.meta, a.B, a.Hkv);
                     }
-                } else {
-                    // -------- output: a lane per head dimension
-                    float acc[NQP];
-                    for (int i = 0; i < a_n; ++i) {
-                        const int nrows = s.meta[it.bi].nrows, n_q = min(G * nrows, NQP);
-                        const int t0 = it.bi * a.R, h0 = it.g * G;
-                        const bool fresh = i == 0 || it.tile == 0, ends = i + 1 == a_n || it.tile + 1 == it.nt;
-                        const int b = at & 1, sb = as & 1;
-                        if (fresh) {
-#pragma unroll
-                            for (int r = 0; r < NQP; ++r) acc[r] = 0.f;
+                    if (more) next_seg();
+                    if (more) {                                           // (the scores of this segment are formed, its query buffer is free)
+                        load_q(ahead, sb);
+                        asm volatile("cp.async.wait_group 0;" ::: "memory");
+                        q_ready(sb);
+                    }
+                    ++as;
+                };
+                AttnPos prev = it;
+                for (int i = 0; i < a_n; ++i) {
+                    const bool fresh = i == 0 || i == a_wrap || it.tile == 0;
+                    if (fresh) {
+                        if (i > 0) {
+                            output(at - 1);
+                            finish(prev);
                         }
-                        ok = warp_wait(smem_u32(&s.ofull[b]), (uint32_t)(at >> 1) & 1u, abort_flag, ok, lane);
-                        tc_fence_after();
+#pragma unroll
+                        for (int x = 0; x < NR; ++x) { m[x] = -CUDART_INF_F; l[x] = 0.f; acc[x] = 0.f; }
+                    }
+                    const SeqMeta sm = s.meta[it.bi];
+                    const int nrows = sm.nrows, L = sm.L, nkeys = sm.nkeys;
+                    const int n_q = min(G * nrows, NQP);
+                    const int t0 = it.bi * a.R;                       // query row r: row t0 + r % nrows, head g * G + r / nrows
+                    const int b = at & 1;
+                    const uint32_t par = (uint32_t)(at >> 1) & 1u;
+                    const int j = it.tile * FW_KEYS + kl;
+                    // which of this thread's rows see its key: all of a committed one; of a draft row those that have it among
+                    // their ancestors and themselves; none past the last key
+                    uint32_t vis = 0xffffffffu;
+                    if ((it.tile + 1) * FW_KEYS > L) {
+                        const int sr = j - L;
+                        vis = j < nkeys ? 0xffffffffu : 0u;
+                        if (sr >= 0 && vis) {
+                            vis = 0;
+#pragma unroll
+                            for (int x = 0; x < NR; ++x) {
+                                const int r = 2 * x + half, rr = r < n_q ? (G == 1 ? r : r % nrows) : 0;
+                                vis |= ((a.rm.mask[(size_t)(t0 + rr) * MTAD_MASK_WORDS + (sr >> 5)] >> (sr & 31)) & 1u) << x;
+                            }
+                        }
+                    }
+                    ok = warp_wait(smem_u32(&s.sfull[b]), par, abort_flag, ok, lane);
+                    tc_fence_after();
+                    float v[NR];
+                    {
                         float c[NQ2];
-                        if (NQ2 == 16) tc_ld16(t_lane + FW_TM_D + b * 64, c);
-                        else { tc_ld16(t_lane + FW_TM_D + b * 64, c); tc_ld16(t_lane + FW_TM_D + b * 64 + 16, c + 16); }
+                        if (NQ2 == 16) tc_ld16(t_lane + b * 64, c);
+                        else { tc_ld16(t_lane + b * 64, c); tc_ld16(t_lane + b * 64 + 16, c + 16); }
 #pragma unroll
-                        for (int r = 0; r < NQP; ++r) acc[r] = acc[r] * s.sf[b][r] + (c[r] + c[NQP + r]);
-                        if (ends) {
-                            // the rows leave: final, or as a piece that the block arriving last merges with the others
-                            const int first = it.f0 / a_per, n_piece = (it.f0 + it.nt - 1) / a_per - first + 1, piece = cta - first;
-                            ok = warp_wait(smem_u32(&s.lfull[sb]), (uint32_t)(as >> 1) & 1u, abort_flag, ok, lane);
-                            if (ok && (HD == 128 || kl < HD)) {
-#pragma unroll
-                                for (int r = 0; r < NQP; ++r) {
-                                    if (r >= n_q) break;
-                                    const int hq = G == 1 ? 0 : r / nrows, t = t0 + r - hq * nrows, h = h0 + hq;
-                                    const float ls = (s.sl[sb][0][r] + s.sl[sb][1][r]) + (s.sl[sb][2][r] + s.sl[sb][3][r]);
-                                    if (n_piece == 1) {
-                                        store_terms(acc[r] / ls, a.x_a + (size_t)t * terms * a.Hq * HD + (size_t)h * HD + kl,
-                                                    (size_t)a.Hq * HD, terms);
-                                    } else {
-                                        const size_t o = ((size_t)t * a.Hq + h) * a.pieces + piece;
-                                        a.part[o * HD + kl] = acc[r];
-                                        if (kl == 0)
-                                            reinterpret_cast<float2*>(a.part + (size_t)T * a.Hq * a.pieces * HD)[o] =
-                                                make_float2(s.sm[sb][r], ls);
-                                    }
-                                }
-                            }
-                            if (n_piece > 1) {
-                                bar_n(3, 128);
-                                if (kl == 0) {
-                                    int old;
-                                    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;"
-                                                 : "=r"(old) : "l"(a.acnt + it.bi * a.Hkv + it.g) : "memory");
-                                    s.last[0] = old + 1 == n_piece;
-                                }
-                                bar_n(3, 128);
-                                if (s.last[0]) merge_pieces<HD, NQP>(a, s, it, n_piece, G, kl);
-                            }
-                            ++as;
+                        for (int x = 0; x < NR; ++x) {
+                            const float y = half == 0 ? c[2 * x] + c[NQP + 2 * x] : c[2 * x + 1] + c[NQP + 2 * x + 1];
+                            v[x] = ((vis >> x) & 1u) ? y : -CUDART_INF_F;
                         }
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&s.oempty[b]));
-                        ++at;
-                        if (i + 1 < a_n) attn_next(it, s.meta, a.B, a.Hkv);
                     }
+                    // The reference value m of a row need not be its maximum: numerators and sums have the exponent range that
+                    // fp32 and bf16 share, and a common factor costs no precision.  A segment starts with the score of its first
+                    // key, and m moves to the maximum only when a score exceeds it by more than 2^64 (or no key was seen yet).
+                    if (fresh) {
+                        if (kl == 0)
+#pragma unroll
+                            for (int x = 0; x < NR; ++x) s.sm[half][x] = v[x];
+                        bar_n(2 + half, 128);
+#pragma unroll
+                        for (int x = 0; x < NR; ++x) m[x] = s.sm[half][x];
+                    }
+                    bool calm = true;
+#pragma unroll
+                    for (int x = 0; x < NR; ++x) calm = calm && v[x] <= m[x] + FW_LAZY && m[x] > -CUDART_INF_F;
+                    float f[NR];
+#pragma unroll
+                    for (int x = 0; x < NR; ++x) f[x] = 1.f;
+                    const bool quiet = all_of(2 + half, 128, calm);
+                    if (!quiet) {
+                        float wm[NR];
+#pragma unroll
+                        for (int x = 0; x < NR; ++x) wm[x] = v[x];
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                            for (int x = 0; x < NR; ++x) wm[x] = fmaxf(wm[x], __shfl_xor_sync(0xffffffffu, wm[x], o));
+#pragma unroll
+                        for (int x = 0; x < NR; ++x)
+                            if (lane == x) s.smx[half][x][quad] = wm[x];
+                        bar_n(2 + half, 128);
+#pragma unroll
+                        for (int x = 0; x < NR; ++x) {
+                            const float4 q4 = *reinterpret_cast<const float4*>(s.smx[half][x]);
+                            const float mn = fmaxf(m[x], fmaxf(fmaxf(q4.x, q4.y), fmaxf(q4.z, q4.w)));
+                            f[x] = mn == -CUDART_INF_F ? 1.f : exp2f(m[x] - mn);
+                            m[x] = mn;
+                            l[x] *= f[x];
+                        }
+                        bar_n(2 + half, 128);                         // (smx is free again)
+                    }
+                    uint8_t* pt = Ps + b * P_BYTES + (kl >> 6) * (NQ2 * 128) + (kl & 7) * 2 + half * 128;
+                    const int pc = (kl & 63) >> 3;
+#pragma unroll
+                    for (int x = 0; x < NR; ++x) {
+                        const float pv = exp2f(v[x] - (m[x] == -CUDART_INF_F ? 0.f : m[x]));        // exp2(-inf) = 0
+                        l[x] += pv;
+                        const __nv_bfloat16 hi = __float2bfloat16_rn(pv);
+                        uint8_t* d = pt + ((pc ^ ((2 * x + half) & 7)) << 4);
+                        *reinterpret_cast<__nv_bfloat16*>(d + 2 * x * 128) = hi;
+                        *reinterpret_cast<__nv_bfloat16*>(d + (NQP + 2 * x) * 128) = __float2bfloat16_rn(pv - __bfloat162float(hi));
+                    }
+                    if ((it.tile + 1) * FW_KEYS > nkeys) {
+                        // rows of V past the last key: their probabilities are 0, but 0 x (stale value) must not make a NaN
+                        const int vpos = pos + 2 * i + 1;
+                        ok = warp_wait(full_bar(vpos), ring_par(vpos), abort_flag, ok, lane);
+                        if (ok && j >= nkeys) {
+                            uint8_t* vs = smem + (size_t)(vpos % NS) * FW_SLOT + kl * 128 + half * 64;
+#pragma unroll
+                            for (int c = 0; c < NCH * 4; ++c)
+                                *reinterpret_cast<uint4*>(vs + (c >> 2) * (FW_KEYS * 128) + (c & 3) * 16) = make_uint4(0u, 0u, 0u, 0u);
+                        }
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    if (!fresh) output(at - 1);                       // (tile i - 1 of the same segment, while this one's output is formed)
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&s.pfull[b]));
+                    if (!quiet)
+#pragma unroll
+                        for (int x = 0; x < NR; ++x) acc[x] *= f[x];
+                    ++at;
+                    prev = it;
+                    if (i + 1 < a_n) attn_step(it, i + 1);
+                }
+                if (a_n > 0) {
+                    output(at - 1);
+                    finish(prev);
                 }
                 pos += 2 * a_n + ring_other;
                 ok = all_of(1, FW_EPI, ok);
                 if (!ok) break;
+                // pieces shared with other blocks (at most the first and the last of this block's range): who arrives last merges
+                if (a_n > 0) {
+                    if (e < 2) {
+                        const AttnPos q = e == 0 ? a_zero : a_last;
+                        const int n_piece = (q.f0 + q.nt - 1) / a_per - q.f0 / a_per + 1;
+                        int last = 0;
+                        if (n_piece > 1 && (e == 0 || a_last.f0 != a_zero.f0)) {
+                            int old;
+                            asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;"
+                                         : "=r"(old) : "l"(a.acnt + q.bi * a.Hkv + q.g) : "memory");
+                            last = old + 1 == n_piece ? n_piece : 0;
+                        }
+                        s.last[e] = last;
+                    }
+                    bar_n(1, FW_EPI);
+                    for (int x = 0; x < 2; ++x)
+                        if (s.last[x]) merge_pieces<HD, NQP>(a, s, x == 0 ? a_zero : a_last, s.last[x], G, e);
+                }
             } else if (kind == FW_QKV) {
                 ok = epi_phase<FW_QKV, HD, FEW>(a, s, Y, p, layer, tcount, e, t_lane, cta);
             } else if (kind == FW_O) {
