@@ -254,8 +254,9 @@ size_t carve(mtad_ctx* c, const mtad_model_desc* t, const mtad_model_desc* a, in
     sc.tc_counters = k.take<int32_t>(max_tiles, "tc_counters");
     sc.lm_part = k.take<float4>(Tc * std::max(lm_tiles, mx([](const mtad_model_desc* m) { return fw_parts_max(*m, kCtas, true); })),
                                 "lm_part");
-    sc.fw_sync_words = (int)mx([&](const mtad_model_desc* m) { return fw_sync_words(m->layers, max_batch, m->n_kv_heads); });
+    sc.fw_sync_words = (int)mx([&](const mtad_model_desc* m) { return fw_sync_words(m->layers, max_batch, m->n_kv_heads, kCtas); });
     sc.fw_sync = k.take<int32_t>(sc.fw_sync_words, "fw_sync");
+    sc.fw_part = k.take<float>((size_t)kCtas * FW_MAX_ROWS * TC_TILE_N, "fw_part");
     FwLayer* fw_t = k.take<FwLayer>(t->layers, "fw_target");
     FwLayer* fw_a = a ? k.take<FwLayer>(a->layers, "fw_aux") : nullptr;
     sc.node_z = k.take<float>(T, "node_z");
@@ -403,24 +404,24 @@ bool build_weight_maps(const ModelView& m, WeightMaps& w) {
 bool build_forward_table(const ModelView& m, FwLayer* dev, CUtensorMap* lm) {
     const mtad_model_desc& d = m.d;
     if (d.head_dim != 64 && d.head_dim != 128) return false;
-    FwPhase ph[6];
-    fw_geometry(ph, d, kCtas);
     const int qd = d.n_q_heads * d.head_dim, hp = d.head_dim / 2;
     std::vector<FwLayer> tab(d.layers);
     for (int c = 0; c < FW_CLASSES; ++c) {
+        FwPhase ph[6];
+        fw_geometry(ph, d, kCtas, c);
         for (int l = 0; l < d.layers; ++l) {
             CUtensorMap* w = tab[l].w[c];
             const FwPhase &q = ph[FW_QKV], &o = ph[FW_O], &g = ph[FW_GATEUP], &dn = ph[FW_DOWN];
-            if (tc_make_pair_map(w, m.w(l, 1), d.n_q_heads, hp, d.d_model, q.h, q.kbc[c]) ||
-                tc_make_pair_map(w + 1, m.w(l, 2), d.n_kv_heads, hp, d.d_model, q.h, q.kbc[c]) ||
-                tc_make_pair_map(w + 2, m.w(l, 3), d.n_kv_heads, hp, d.d_model, q.h, q.kbc[c]) ||
-                tc_make_kb_map(w + 3, m.w(l, 4), d.d_model, qd, o.h, o.kbc[c]) ||
-                tc_make_kb_map(w + 4, m.w(l, 6), d.d_ffn, d.d_model, g.h, g.kbc[c]) ||
-                tc_make_kb_map(w + 5, m.w(l, 7), d.d_ffn, d.d_model, g.h, g.kbc[c]) ||
-                tc_make_kb_map(w + 6, m.w(l, 8), d.d_model, d.d_ffn, dn.h, dn.kbc[c]))
+            if (tc_make_pair_map(w, m.w(l, 1), d.n_q_heads, hp, d.d_model, q.h, q.kb) ||
+                tc_make_pair_map(w + 1, m.w(l, 2), d.n_kv_heads, hp, d.d_model, q.h, q.kb) ||
+                tc_make_pair_map(w + 2, m.w(l, 3), d.n_kv_heads, hp, d.d_model, q.h, q.kb) ||
+                tc_make_kb_map(w + 3, m.w(l, 4), d.d_model, qd, o.h, o.kb) ||
+                tc_make_kb_map(w + 4, m.w(l, 6), d.d_ffn, d.d_model, g.h, g.kb) ||
+                tc_make_kb_map(w + 5, m.w(l, 7), d.d_ffn, d.d_model, g.h, g.kb) ||
+                tc_make_kb_map(w + 6, m.w(l, 8), d.d_model, d.d_ffn, dn.h, dn.kb))
                 return false;
         }
-        if (tc_make_kb_map(lm + c, d.lm_head, d.vocab, d.d_model, ph[FW_LM].h, ph[FW_LM].kbc[c])) return false;
+        if (tc_make_kb_map(lm + c, d.lm_head, d.vocab, d.d_model, ph[FW_LM].h, ph[FW_LM].kb)) return false;
     }
     for (int l = 0; l < d.layers; ++l) {
         tab[l].gain_ffn = m.w(l, 5);
@@ -451,6 +452,7 @@ bool build_forward_plan(ForwardPlan& fp, const Scratch& sc, const RowMeta& rm, c
     a.max_batch = m.max_batch; a.cap = d.kv_capacity;
     a.parts0 = 1; a.inv_dim = 1.f / (float)d.d_model; a.eps = d.rms_eps;
     a.sync = sc.fw_sync; a.acnt = sc.fw_sync + 5 * d.layers + 1;
+    a.kcnt = a.acnt + (size_t)m.max_batch * d.n_kv_heads; a.kpart = sc.fw_part;
     a.sumsq_a = sc.sumsq_a; a.sumsq_b = sc.sumsq_b; a.hidden = sc.hidden;
     a.x_d = sc.xd; a.x_a = sc.xa; a.x_f = sc.xf; a.q_hi = sc.q_hi; a.q_lo = sc.q_lo;
     a.cache = static_cast<__nv_bfloat16*>(d.kv_cache);
@@ -1169,7 +1171,9 @@ void audit_forward(Audit& au, const mtad_ctx& c, const ModelView& m, int B, int 
         au.ws("xa", idx_xrow(T - 1, terms, terms - 1, qd, qd - 1) + 1);
         au.ws("xf", idx_xrow(T - 1, terms, terms - 1, d.d_ffn, d.d_ffn - 1) + 1);
         au.ws("attn_part", (size_t)T * Hq * pieces * (hd + 2));
-        au.ws("fw_sync", fw_sync_words(d.layers, m.max_batch, Hkv));
+        au.ws("fw_sync", fw_sync_words(d.layers, m.max_batch, Hkv, kCtas));
+        for (const FwPhase* f : {&a.ph[FW_O], &a.ph[FW_DOWN]})
+            if (f->c > 1) au.ws("fw_part", (size_t)f->n_tiles * T * f->h);
         au.ws(&m == &c.target ? "fw_target" : "fw_aux", d.layers);
         if (lm_plain) au.ws("logits", (size_t)T * d.vocab);
         else au.ws("lm_part", idx_lm_part(T - 1, a.ph[FW_LM].n_tiles, a.ph[FW_LM].n_tiles - 1) + 1);

@@ -134,6 +134,7 @@ struct Scratch {
     DraftPart* draft_part;   // [max_batch][MTAD_MAX_BEAM][MTAD_DRAFT_CHUNKS], only with an auxiliary model
     int32_t* fw_sync;        // one-launch forward: phase counters and the attention's arrival counters
     int fw_sync_words;
+    float* fw_part;          // partial sums of its split projections
     WarpPart* warp_part;     // [T][MTAD_DRAFT_CHUNKS]
     WarpRow* warp_row;       // [T]
 };

@@ -31,6 +31,7 @@
 #include <cstddef>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "forward.cuh"
 #include "tc_device.cuh"
@@ -44,7 +45,6 @@ constexpr int FW_THREADS = 32 * 12;
 constexpr int FW_EPI_WARP0 = 4;
 constexpr int FW_EPI = 256;
 constexpr int FW_UNION = 32 * 1024;       // epilogue tile Y, or the attention's query and probability tiles
-constexpr int NS = FW_SLOTS;
 constexpr int FW_ACC = 240;               // accumulator columns of a tile, of 256 (the drain reads up to 15 columns further)
 constexpr float FW_LAZY = 64.f;           // log2 of how far a score may exceed its row's reference value
 constexpr int FW_TM_D = 128;              // attention: tensor-memory columns 0 / 64 scores, 128 / 192 outputs
@@ -167,14 +167,14 @@ struct FwTail {
     alignas(16) float smx[2][8][4];       // attention, per half of the rows: row maxima of the four warps
     alignas(16) float sl[2][2][8][4];     // row sums of the four warps, two segments
     float sm[2][8];                       // first scores of a segment
-    uint64_t full[NS], empty[NS];
+    uint64_t full[4], empty[4];
     uint64_t tfull[2], tempty[2], sfull[2], pfull[2], ofull[2], qfull[2];
     uint32_t tmem_ptr;
     int abort_flag[2];
     int last[2];
 };
 static_assert(offsetof(FwTail, smx) % 16 == 0 && offsetof(FwTail, sl) % 16 == 0 && offsetof(FwTail, full) % 8 == 0, "alignment of the tail");
-static_assert(NS * FW_SLOT + FW_UNION + sizeof(FwTail) <= 227 * 1024, "shared memory of the forward");
+static_assert(FW_RING + FW_UNION + sizeof(FwTail) <= 227 * 1024, "shared memory of the forward");
 
 // The epilogue group's part of one projection: row statistics, then per tile the accumulators -> Y in shared memory ->
 // the fused epilogue.  KIND is a template parameter so that the phase's geometry is read straight from the launch
@@ -209,7 +209,8 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
             if (!ok) return false;
         }
         const float* sq = KIND == FW_GATEUP ? a.sumsq_b : a.sumsq_a;
-        const int parts = KIND == FW_GATEUP ? a.ph[FW_O].n_tiles : (p == 0 ? a.parts0 : a.ph[FW_DOWN].n_tiles);
+        const FwPhase& from = a.ph[KIND == FW_GATEUP ? FW_O : FW_DOWN];
+        const int parts = KIND != FW_GATEUP && p == 0 ? a.parts0 : (FEW ? from.n_tiles : from.n_tiles / from.c);
         for (int r = w; r < T; r += 8) {
             float v = 0.f;
 #pragma unroll 5
@@ -219,11 +220,18 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
             if (lane == 0) s.rstd[r] = rsqrtf(v * a.inv_dim + a.eps);
         }
     }
+    if (!FEW && (KIND == FW_O || KIND == FW_DOWN)) {
+        // the residual stream comes from other blocks where O and down are cut differently
+        if (e == 0) ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
+        ok = all_of(1, FW_EPI, ok);
+        if (!ok) return false;
+    }
     const __nv_bfloat16* gain = nullptr;
     if (KIND == FW_O) gain = a.layers[layer].gain_ffn;
     if (KIND == FW_DOWN) gain = a.layers[layer].gain_next;
     for (int tile = cta; tile < f.n_tiles; tile += n_cta, ++tcount) {
-        const int buf = tcount & 1, f0 = tile * nf;        // f0: first feature (O, down, gate / up, LM head)
+        const bool split = !FEW && (KIND == FW_O || KIND == FW_DOWN) && f.c > 1;
+        const int buf = tcount & 1, f0 = (split ? tile / f.c : tile) * nf;     // f0: first feature (O, down, gate / up, LM head)
         // ---- what the first items need besides the accumulator
         const int hg = KIND == FW_QKV ? tile / f.u : 0, j0 = KIND == FW_QKV ? (tile - hg * f.u) * f.h : 0;
         constexpr int NI = FEW ? 2 : 1;                    // QKV: items per thread and round
@@ -471,35 +479,74 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                     if (lane == 0) (KIND == FW_O ? a.sumsq_b : a.sumsq_a)[(size_t)tile * TC_X_ROWS + w] = ss;
                 }
             } else {
-                // residual, four features per item; the items' sums of squares meet in Y (each over its own first element)
-                int t = it0, j = ij0;
+                // residual, four features per item; the items' sums of squares meet in Y (each over its own first element).
+                // A split tile: the blocks that share it leave their partial sums in global memory, wait for one another and
+                // finish a share of the rows each, adding the partial sums in block order (deterministic).
+                int t = it0, j = ij0, ra = 0, rn = nr;     // rows [ra, rn) of this block of rows are finished here
+                if (split) {
+                    float* mine = a.kpart + (size_t)tile * T * nf;
 #pragma unroll 2
-                for (int i = e; i < nr * nv; i += FW_EPI) {
+                    for (int i = e; i < nr * nv; i += FW_EPI) {
+                        float v[V];
+                        yv(t, 0, j, v);
+                        __stcg(reinterpret_cast<float4*>(mine + (size_t)(r0 + t) * nf + j), make_float4(v[0], v[1 % V], v[2 % V], v[3 % V]));
+                        t += dt; j += dj;
+                        if (j >= nf) { j -= nf; ++t; }
+                    }
+                    bar_n(1, FW_EPI);                      // (Y is free again; every partial sum of these rows is on its way)
+                    if (r1 < T) continue;
+                    if (e == 0) {
+                        int32_t* cnt = a.kcnt + (KIND == FW_O ? 0 : n_cta) + tile / f.c;
+                        asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(cnt) : "memory");
+                        ok = grid_wait(cnt, f.c * (layer + 1), abort_flag);
+                    }
+                    ok = all_of(1, FW_EPI, ok);
+                    if (!ok) return false;
+                    const int kp = tile % f.c;
+                    ra = T * kp / f.c;
+                    rn = T * (kp + 1) / f.c;
+                    t = ra + it0; j = ij0;
+                }
+                const int rb0 = split ? 0 : r0, ystr = split ? nf : ys;
+                const float* parts = a.kpart + (size_t)(split ? tile / f.c * f.c : 0) * T * nf;
+#pragma unroll 2
+                for (int i = e; i < (rn - ra) * nv; i += FW_EPI) {
                     const int n = f0 + j;
                     float ss = 0.f;
                     if (n < a.d) {
-                        float4* hp = reinterpret_cast<float4*>(a.hidden + (size_t)(r0 + t) * a.d + n);
-                        const float4 h4 = __ldcg(hp);
+                        float4* hp = reinterpret_cast<float4*>(a.hidden + (size_t)(rb0 + t) * a.d + n);
+                        float4 y = __ldcg(hp);
                         float g[4], v[V];
 #pragma unroll
                         for (int x = 0; x < 4; ++x) g[x] = __bfloat162float(gain[n + x]);
-                        yv(t, 0, j, v);
-                        const float4 y = make_float4(v[0] + h4.x, v[1 % V] + h4.y, v[2 % V] + h4.z, v[3 % V] + h4.w);
+                        if (split) {
+                            float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+                            for (int k = 0; k < f.c; ++k) {
+                                const float4 x = __ldcg(reinterpret_cast<const float4*>(parts + ((size_t)k * T + t) * nf + j));
+                                q.x += x.x; q.y += x.y; q.z += x.z; q.w += x.w;
+                            }
+                            v[0] = q.x; v[1 % V] = q.y; v[2 % V] = q.z; v[3 % V] = q.w;
+                        } else {
+                            yv(t, 0, j, v);
+                        }
+                        y.x += v[0]; y.y += v[1 % V]; y.z += v[2 % V]; y.w += v[3 % V];
                         *hp = y;
                         store_terms4(make_float4(y.x * g[0], y.y * g[1], y.z * g[2], y.w * g[3]),
-                                     a.x_d + (size_t)(r0 + t) * terms * a.d + n, a.d, terms);
+                                     a.x_d + (size_t)(rb0 + t) * terms * a.d + n, a.d, terms);
                         ss = (y.x * y.x + y.y * y.y) + (y.z * y.z + y.w * y.w);
                     }
-                    Y[t * ys + j] = ss;
+                    Y[(t - ra) * ystr + j] = ss;
                     t += dt; j += dj;
                     if (j >= nf) { j -= nf; ++t; }
                 }
                 bar_n(1, FW_EPI);
-                for (int tr = w; tr < nr; tr += 8) {
-                    float ss = lane < nv ? Y[tr * ys + lane * V] : 0.f;       // (nv <= 32: at most 128 features)
+                for (int tr = w; tr < rn - ra; tr += 8) {
+                    float ss = lane < nv ? Y[tr * ystr + lane * V] : 0.f;       // (nv <= 32: at most 128 features)
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-                    if (lane == 0) (KIND == FW_O ? a.sumsq_b : a.sumsq_a)[(size_t)tile * TC_X_ROWS + r0 + tr] = ss;
+                    if (lane == 0)
+                        (KIND == FW_O ? a.sumsq_b : a.sumsq_a)[(size_t)(split ? tile / f.c : tile) * TC_X_ROWS + rb0 + ra + tr] = ss;
                 }
             }
             if (r1 < T || tile + n_cta < f.n_tiles) bar_n(1, FW_EPI);       // Y is rewritten by the next rows or tile
@@ -556,15 +603,16 @@ __device__ __forceinline__ void merge_pieces(const FwArgs& a, const FwTail& s, c
     if (e == 0) a.acnt[q.bi * a.Hkv + q.g] = 0;       // ready for the next layer
 }
 
-template <int HD, int NQP, bool FEW>
+template <int HD, int NQP, bool FEW, int NS>
 __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_constant__ FwArgs a) {
     constexpr int NCH = HD / 64;                       // 64-element chunks of a head row
     constexpr int NQ2 = 2 * NQP;                       // query rows as hi and lo parts
     constexpr uint32_t KV_BYTES = FW_KEYS * HD * 2;
     constexpr int Q_BYTES = NQ2 * HD * 2;              // one query tile
     constexpr int P_BYTES = NQ2 * FW_KEYS * 2;         // one probability tile
+    constexpr int FW_SLOT = FW_RING / NS;
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t* uni = smem + (size_t)NS * FW_SLOT;
+    uint8_t* uni = smem + FW_RING;
     FwTail& s = *reinterpret_cast<FwTail*>(uni + FW_UNION);
     float* Y = reinterpret_cast<float*>(uni);
     uint8_t* Qs = uni;                                 // [2][Q_BYTES]
@@ -631,6 +679,9 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     auto full_bar = [&](int pos) { return smem_u32(&s.full[pos % NS]); };
     auto empty_bar = [&](int pos) { return smem_u32(&s.empty[pos % NS]); };
     auto ring_par = [&](int pos) { return (uint32_t)(pos / NS) & 1u; };
+    // steps [k0, k1) of a tile: all of them, or this block's share
+    auto k_first = [&](const FwPhase& f, int tile) { return f.c > 1 ? (tile % f.c) * f.steps / f.c : 0; };
+    auto k_end = [&](const FwPhase& f, int tile) { return f.c > 1 ? (tile % f.c + 1) * f.steps / f.c : f.steps; };
     // kind of phase p
     auto kind_of = [&](int p) { return p == n_phases - 1 ? (int)FW_LM : p % 5; };
 
@@ -692,8 +743,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         row = tile * f.h;
                     } else {
                         m = kind == FW_O ? w + 3 : (kind == FW_DOWN ? w + 6 : &a.lm);
+                        if (f.c > 1) row = tile / f.c * f.h;
                     }
-                    for (int step = 0; step < f.steps; ++step, ++pos) {
+                    const int k1 = k_end(f, tile);
+                    for (int step = k_first(f, tile); step < k1; ++step, ++pos) {
                         ok = mbar_wait(empty_bar(pos), ring_par(pos) ^ 1u, abort_flag);
                         if (!ok) break;
                         const uint32_t bar = full_bar(pos), base = slot_ptr(pos);
@@ -728,14 +781,16 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
                     proxy_fence();
                 }
-                for (int tile = cta; tile < f.n_tiles && ok; tile += n_cta)
-                    for (int step = 0; step < f.steps; ++step, ++pos) {
+                for (int tile = cta; tile < f.n_tiles && ok; tile += n_cta) {
+                    const int k1 = k_end(f, tile);
+                    for (int step = k_first(f, tile); step < k1; ++step, ++pos) {
                         ok = mbar_wait(empty_bar(pos), ring_par(pos) ^ 1u, abort_flag);
                         if (!ok) break;
                         const uint32_t bar = full_bar(pos), base = slot_ptr(pos) + f.b_off;
                         if (!a.debug_no_operands)
                             tma_load_3d(base, m, bar, f.flat ? step * TC_TILE_K : 0, 0, f.flat ? 0 : step * f.kb, HINT_KEEP);
                     }
+                }
             }
         }
     } else if (warp < FW_EPI_WARP0) {
@@ -811,7 +866,8 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 const uint32_t d = tmem + buf * 256 + me * sc;
                 uint32_t acc = 0;
                 int turn = 0;                              // dual: MMAs along k alternate between the warps
-                for (int step = 0; step < f.steps; ++step, ++pos) {
+                const int k1 = k_end(f, tile);
+                for (int step = k_first(f, tile); step < k1; ++step, ++pos) {
                     ok = mbar_wait_warp(full_bar(pos), ring_par(pos), abort_flag);
                     if (!ok) break;
                     tc_fence_after();
@@ -843,7 +899,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         const uint32_t t_lane = tmem + ((uint32_t)(quad * 32) << 16);
         int tcount = 0, at = 0, as = 0, pos = 0;
         bool ok = true;
-        auto steps_of = [&](const FwPhase& f) { return cta < f.n_tiles ? ((f.n_tiles - 1 - cta) / n_cta + 1) * f.steps : 0; };
+        auto steps_of = [&](const FwPhase& f) {
+            if (cta >= f.n_tiles) return 0;
+            return f.c > 1 ? k_end(f, cta) - k_first(f, cta) : ((f.n_tiles - 1 - cta) / n_cta + 1) * f.steps;
+        };
         const int ring_other = steps_of(a.ph[FW_O]) + steps_of(a.ph[FW_GATEUP]) + steps_of(a.ph[FW_DOWN]);
         const int ring_qkv = steps_of(a.ph[FW_QKV]);
         for (int p = 0; p < n_phases && ok; ++p) {
@@ -1135,20 +1194,43 @@ int up8(int x) { return (x + 7) / 8 * 8; }
 
 }  // namespace
 
-void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta) {
+void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta, int cls) {
     const int qd = d.n_q_heads * d.head_dim, hp = d.head_dim / 2, heads = d.n_q_heads + 2 * d.n_kv_heads;
+    const int cols = FW_CLASS[cls].cols, slot = FW_RING / FW_CLASS[cls].slots;
+    for (int k = 0; k < 6; ++k) ph[k].c = ph[k].u = 1;
     // rows of a matrix: one tile per SM, in whole groups of eight rows (swizzle atoms)
-    auto rows = [&](FwPhase& f, int N, int nbox, int cut) {
+    auto rows = [&](FwPhase& f, int N, int K, int nbox, int cut) {
+        f.K = K;
+        f.k_blocks = up_div(K, TC_TILE_K);
         f.nbox = nbox;
         f.h = f.hr = std::min(128, std::max(8, up8(up_div(N, n_cta * cut))));
         f.n_tiles = up_div(N, f.h * cut);
-        f.u = 1;
     };
-    rows(ph[FW_O], d.d_model, 1, 1);
-    rows(ph[FW_DOWN], d.d_model, 1, 1);
-    rows(ph[FW_GATEUP], d.d_ffn, 2, 1);
+    rows(ph[FW_O], d.d_model, qd, 1, 1);
+    rows(ph[FW_DOWN], d.d_model, d.d_ffn, 1, 1);
+    rows(ph[FW_GATEUP], d.d_ffn, d.d_model, 2, 1);
     const int lm_boxes = up_div(d.vocab, n_cta) > 64 ? 2 : 1;
-    rows(ph[FW_LM], d.vocab, lm_boxes, lm_boxes);
+    rows(ph[FW_LM], d.vocab, d.d_model, lm_boxes, lm_boxes);
+    // O and down: a tile's k-range over c blocks where that pays.  With many operand rows the SMs' intake bounds a narrow
+    // tile (every block reads all operand rows of its k-blocks, about 100 GB/s an SM from L2); c blocks on a tile c times as
+    // wide read them a c-th as often, and pay about 3.5 us to exchange their partial sums.
+    for (int k : {FW_O, FW_DOWN}) {
+        FwPhase& f = ph[k];
+        double best = 1e30;
+        for (int c = 1; c <= 4; ++c) {
+            const int h = std::max(8, up8(up_div(d.d_model, n_cta / c)));
+            if (c > 1 && (h > 128 || f.k_blocks < 8 * c || cls < 2)) break;
+            const double intake = (double)(h + cols) * 128.0 * up_div(f.k_blocks, c) / 100e3;
+            const double floor_us = 2.0 * d.d_model * f.K / 6.5e6;
+            const double us = std::max(intake, floor_us) + (c > 1 ? 3.5 : 0.0);
+            if (us < best) {
+                best = us;
+                f.c = c;
+                f.h = f.hr = std::min(128, h);
+                f.n_tiles = up_div(d.d_model, f.h) * c;
+            }
+        }
+    }
     // QKV: the rotary pairs of a head in u tiles, as many as the SMs allow
     FwPhase& q = ph[FW_QKV];
     q.u = std::max(1, std::min(n_cta / heads, hp / 4));
@@ -1157,22 +1239,21 @@ void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta) {
     q.hr = 2 * q.h;
     q.nbox = 1;
     q.n_tiles = heads * q.u;
-    ph[FW_O].K = qd;
-    ph[FW_DOWN].K = d.d_ffn;
-    ph[FW_LM].K = ph[FW_GATEUP].K = q.K = d.d_model;
-    static const int class_cols[FW_CLASSES] = {16, 32, 64, FW_MAX_COLS};
+    q.K = d.d_model;
+    q.k_blocks = up_div(q.K, TC_TILE_K);
     for (int k = 0; k < 6; ++k) {
         if (k == FW_ATTN) continue;
         FwPhase& f = ph[k];
-        f.k_blocks = up_div(f.K, TC_TILE_K);
-        for (int c = 0; c < FW_CLASSES; ++c) {
-            int kb = FW_SLOT / ((f.nbox * f.hr + class_cols[c]) * 128);
-            kb = std::min(std::min(kb, f.k_blocks), 16);
-            // a multiple of the k-blocks that the MMA can take side by side
-            const int S = std::min(TC_TILE_N / f.hr, FW_ACC / (class_cols[c] * f.nbox));
-            if (S > 1 && kb > S) kb -= kb % S;
-            f.kbc[c] = (f.K % TC_TILE_K || kb < 1) ? 1 : kb;
-        }
+        int kb = slot / ((f.nbox * f.hr + cols) * 128);
+        kb = std::min(std::min(kb, f.k_blocks), 16);
+        // a multiple of the k-blocks that the MMA can take side by side
+        const int S = std::min(TC_TILE_N / f.hr, FW_ACC / (cols * f.nbox));
+        if (S > 1 && kb > S) kb -= kb % S;
+        f.kb = (f.K % TC_TILE_K || kb < 1) ? 1 : kb;
+        f.flat = tc_kb_flat(f.K, f.kb) ? 1 : 0;
+        f.steps = up_div(f.k_blocks, f.kb);
+        f.box_bytes = f.hr * 128 * f.kb;
+        f.b_off = f.nbox * f.box_bytes;
     }
 }
 
@@ -1181,28 +1262,24 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
     if (d.head_dim != 64 && d.head_dim != 128) return false;
     if (T > FW_MAX_ROWS || G * R > FW_MAX_QROWS || B > MTAD_MAX_BATCH) return false;
     if (d.d_model >= 8192 && T > 32) return false;          // the accurate K / V projection has launches of its own
-    fw_geometry(a.ph, d, n_cta);
     a.T = T; a.B = B; a.R = R; a.terms = tc_terms(T);
     a.cols = (a.terms * T + 15) / 16 * 16;
     if (a.cols > FW_MAX_COLS) return false;
-    a.cls = a.cols <= 16 ? 0 : (a.cols <= 32 ? 1 : (a.cols <= 64 ? 2 : 3));
+    a.cls = T <= 8 ? 0 : 2;                                // (four slots and the lean epilogues: up to eight rows)
+    while (FW_CLASS[a.cls].cols < a.cols) ++a.cls;
+    fw_geometry(a.ph, d, n_cta, a.cls);
     a.n_cta = n_cta; a.n_layers = d.layers;
     a.d = d.d_model; a.F = d.d_ffn; a.V = d.vocab; a.Hq = d.n_q_heads; a.Hkv = d.n_kv_heads; a.hd = d.head_dim;
     for (int k = 0; k < 6; ++k) {
         if (k == FW_ATTN) continue;
         FwPhase& f = a.ph[k];
-        f.kb = f.kbc[a.cls];
-        f.flat = tc_kb_flat(f.K, f.kb) ? 1 : 0;
         f.S = 1;
         for (int S = 2; S <= f.kb; ++S)
             if (f.kb % S == 0 && S * f.hr <= TC_TILE_N && S * a.cols * f.nbox <= FW_ACC) f.S = S;
-        f.steps = up_div(f.k_blocks, f.kb);
-        f.box_bytes = f.hr * 128 * f.kb;
-        f.b_off = f.nbox * f.box_bytes;
-        if (f.b_off + f.kb * a.cols * 128 > FW_SLOT || f.nbox * f.S * a.cols > FW_ACC) return false;
-        if ((k == FW_O || k == FW_DOWN) && f.n_tiles > n_cta) return false;
-        // one box: the MMAs along k alternate between two accumulators where they fit and there are two
-        f.dual = f.nbox == 1 && 2 * f.S * a.cols <= FW_ACC && f.steps * (f.kb / f.S) >= 2 ? 1 : 0;
+        if (f.b_off + f.kb * a.cols * 128 > FW_RING / FW_CLASS[a.cls].slots || f.nbox * f.S * a.cols > FW_ACC) return false;
+        if ((k == FW_O || k == FW_DOWN) && (f.n_tiles > n_cta || f.steps < f.c)) return false;
+        // one box: the MMAs along k alternate between two accumulators where they fit and every block has two
+        f.dual = f.nbox == 1 && 2 * f.S * a.cols <= FW_ACC && f.steps / f.c * (f.kb / f.S) >= 2 ? 1 : 0;
         const int per = a.terms == 3 ? 5 : 8;              // rows of one drain load
         const int fit = FW_UNION / (per * (f.nbox * f.S * f.hr + 4) * 4);
         if (fit < 1) return false;
@@ -1212,13 +1289,18 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
 }
 
 size_t fw_parts_max(const mtad_model_desc& d, int n_cta, bool lm) {
-    FwPhase ph[6];
-    fw_geometry(ph, d, n_cta);
-    return (size_t)ph[lm ? FW_LM : FW_O].n_tiles;
+    size_t most = 0;
+    for (int c = 0; c < FW_CLASSES; ++c) {
+        FwPhase ph[6];
+        fw_geometry(ph, d, n_cta, c);
+        for (int k : {FW_O, FW_DOWN, FW_LM})
+            if ((k == FW_LM) == lm) most = std::max(most, (size_t)(ph[k].n_tiles / ph[k].c));
+    }
+    return most;
 }
 
 cudaError_t launch_forward(const FwArgs& a, cudaStream_t st) {
-    const size_t smem = (size_t)NS * FW_SLOT + FW_UNION + sizeof(FwTail);
+    const size_t smem = (size_t)FW_RING + FW_UNION + sizeof(FwTail);
     auto go = [&](auto kernel) -> cudaError_t {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e != cudaSuccess) return e;
@@ -1234,14 +1316,15 @@ cudaError_t launch_forward(const FwArgs& a, cudaStream_t st) {
         cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, kernel, a);
     };
-    // instantiations: head size, query rows of a KV head, few rows in all
+    // instantiations: head size, query rows of a KV head, few rows in all, ring slots
     const bool q8 = (a.Hq / a.Hkv) * a.R <= 8, few = a.T <= 8;
-    if (a.hd == 128) {
-        if (few) return q8 ? go(forward_kernel<128, 8, true>) : go(forward_kernel<128, 16, true>);
-        return q8 ? go(forward_kernel<128, 8, false>) : go(forward_kernel<128, 16, false>);
-    }
-    if (few) return q8 ? go(forward_kernel<64, 8, true>) : go(forward_kernel<64, 16, true>);
-    return q8 ? go(forward_kernel<64, 8, false>) : go(forward_kernel<64, 16, false>);
+    auto pick = [&](auto hd, auto nqp) -> cudaError_t {
+        constexpr int HD = decltype(hd)::value, NQP = decltype(nqp)::value;
+        return few ? go(forward_kernel<HD, NQP, true, FW_CLASS[0].slots>) : go(forward_kernel<HD, NQP, false, FW_CLASS[2].slots>);
+    };
+    using std::integral_constant;
+    if (a.hd == 128) return q8 ? pick(integral_constant<int, 128>{}, integral_constant<int, 8>{}) : pick(integral_constant<int, 128>{}, integral_constant<int, 16>{});
+    return q8 ? pick(integral_constant<int, 64>{}, integral_constant<int, 8>{}) : pick(integral_constant<int, 64>{}, integral_constant<int, 16>{});
 }
 
 }  // namespace mtad

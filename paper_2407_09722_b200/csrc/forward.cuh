@@ -5,8 +5,8 @@
 
 namespace mtad {
 
-constexpr int FW_SLOT = 48 * 1024;        // bytes of one ring slot: one step of a projection, or 128 keys of K or V
-constexpr int FW_SLOTS = 4;
+constexpr int FW_RING = 192 * 1024;       // the copy ring: four slots, or three where the operand rows are many; a slot
+                                          // holds one step of a projection, or 128 keys of K or V
 constexpr int FW_KEYS = 128;              // keys of an attention tile
 constexpr int FW_MAX_ROWS = 56;           // rows of a call
 constexpr int FW_MAX_COLS = 112;          // operand rows (terms x rows) of a call
@@ -14,15 +14,17 @@ constexpr int FW_MAX_QROWS = 16;          // query rows of one KV head and seque
 
 // Tile geometry of one projection.  A step brings nbox boxes of hr weight rows x kb k-blocks (one copy each) and one box of
 // operand rows.  nbox = 1: the rows of h features (QKV: of h rotary pairs of a head, hr = 2 h); nbox = 2: h gate rows and
-// the h matching up rows, or 2 h rows of the LM head.  h depends on the matrix and the SM count alone; kb is the most that
-// a ring slot holds for the call's operand rows, in FW_CLASSES steps, so that the weight maps are encoded once per model.
+// the h matching up rows, or 2 h rows of the LM head.  The geometry depends on the matrix, the SM count and the class of
+// the call's operand rows, so that the weight maps are encoded once per model: kb is the most that a ring slot holds.
 // Big boxes matter twice: a thread issues a copy about every quarter of a microsecond whatever its size, and rows of 256
 // bytes and more pass at 70 GB/s per SM where rows of 128 bytes pass at 43.
-constexpr int FW_CLASSES = 4;             // operand rows up to 16, 32, 64, 112
+constexpr int FW_CLASSES = 5;
+struct FwClass { int cols, slots; };      // operand rows up to, ring slots
+constexpr FwClass FW_CLASS[FW_CLASSES] = {{16, 4}, {32, 4}, {64, 3}, {80, 3}, {FW_MAX_COLS, 3}};
 struct FwPhase {
     int h, hr, nbox, n_tiles, u;          // u: tiles per head (QKV)
-    int kbc[FW_CLASSES];                  // kb by class
-    int kb, flat, S, steps;               // k-blocks of a box, its map's view, k-blocks side by side in the MMA, steps of a tile
+    int c;                                // O, down: blocks that share a tile's k-range (their partial sums meet in global memory)
+    int kb, flat, S, steps;               // k-blocks of a box, its map's view, k-blocks side by side in the MMA, steps of all k-blocks
     int box_bytes, b_off;                 // bytes of one weight box, offset of the operand rows in the slot
     int k_blocks, K;
     int dual, blk;                        // two accumulators for one box; rows that the epilogue takes at a time
@@ -46,6 +48,8 @@ struct FwArgs {
     long long cap;
     float inv_dim, eps;
     int32_t *sync, *acnt;                 // phase counters, arrival counters of the attention's (sequence, KV head) pairs
+    int32_t* kcnt;                        // arrivals at the split tiles of O, then of down
+    float* kpart;                         // their partial sums [block][row][feature]
     float *sumsq_a, *sumsq_b, *hidden;
     __nv_bfloat16 *x_d, *x_a, *x_f, *q_hi, *q_lo, *cache;
     const float* rope;
@@ -59,14 +63,16 @@ struct FwArgs {
     int debug_no_operands;
 };
 
-// Host side.  fw_geometry fills what the matrices alone decide; fw_plan the rest for a call of B x R rows and returns
-// false where the one-launch forward does not apply.  fw_parts_max: tiles of the LM head (lm) or of O / down, i.e. the
+// Host side.  fw_geometry fills the geometry of class cls; fw_plan the rest for a call of B x R rows and returns false
+// where the one-launch forward does not apply.  fw_parts_max: most tiles of the LM head (lm) or of O / down, i.e. the
 // partial results that a row of a call has.
-void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta);
+void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta, int cls);
 bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta);
 size_t fw_parts_max(const mtad_model_desc& d, int n_cta, bool lm);
 // words of the phase and arrival counters (zeroed by the row preparation of every call)
-inline size_t fw_sync_words(int layers, int max_batch, int Hkv) { return (size_t)5 * layers + 1 + (size_t)max_batch * Hkv; }
+inline size_t fw_sync_words(int layers, int max_batch, int Hkv, int n_cta) {
+    return (size_t)5 * layers + 1 + (size_t)max_batch * Hkv + 2 * (size_t)n_cta;
+}
 cudaError_t launch_forward(const FwArgs& a, cudaStream_t st);
 
 }  // namespace mtad
