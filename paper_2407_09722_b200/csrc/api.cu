@@ -1164,7 +1164,7 @@ void audit_forward(Audit& au, const mtad_ctx& c, const ModelView& m, int B, int 
         const long long cap = d.kv_capacity, total = std::min<long long>(len_ub, cap) + R;
         const long long slot_max = std::min<long long>(len_ub + R - 1, cap - 1), pieces = (total + FW_KEYS - 1) / FW_KEYS;
         for (const FwPhase* f : {&a.ph[FW_O], &a.ph[FW_DOWN]})
-            for (const char* n : {"sumsq_a", "sumsq_b"}) au.ws(n, (size_t)(f->n_tiles - 1) * TC_X_ROWS + T);
+            for (const char* n : {"sumsq_a", "sumsq_b"}) au.ws(n, (size_t)(f->n_tiles / f->c - 1) * TC_X_ROWS + T);
         au.ws("hidden", (size_t)(T - 1) * d.d_model + d.d_model);
         au.ws("q_hi", (size_t)T * qd);
         au.ws("q_lo", (size_t)T * qd);

@@ -60,6 +60,11 @@ __device__ __forceinline__ bool grid_wait(const int* c, int want, volatile int* 
     *abort_flag = 1;
     return false;
 }
+// The layer table's tensor maps lie in global memory, where the host wrote them: an SM's descriptor cache may still hold
+// what an earlier table had at the same address (a context that is gone), so each is acquired before its first use.
+__device__ __forceinline__ void map_acquire(const CUtensorMap* m) {
+    asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
+}
 __device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async;" ::: "memory"); }
 __device__ __forceinline__ uint2 pack4(float x, float y, float z, float w) {
     const __nv_bfloat162 p = __floats2bfloat162_rn(x, y), q = __floats2bfloat162_rn(z, w);
@@ -720,12 +725,6 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     }
                     continue;
                 }
-                if (kind == FW_QKV && layer + 1 < a.n_layers) {
-                    const CUtensorMap* nm = L[1].w[a.cls];
-#pragma unroll
-                    for (int i = 0; i < 7; ++i)
-                        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(nm + i)) : "memory");
-                }
                 const FwPhase& f = a.ph[kind];
                 const CUtensorMap* w = L->w[a.cls];
                 const uint32_t bytes = (uint32_t)(f.nbox * f.box_bytes + f.kb * cols * 128);
@@ -744,6 +743,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     } else {
                         m = kind == FW_O ? w + 3 : (kind == FW_DOWN ? w + 6 : &a.lm);
                         if (f.c > 1) row = tile / f.c * f.h;
+                    }
+                    if (kind != FW_LM) {
+                        map_acquire(m);
+                        if (kind == FW_GATEUP) map_acquire(m + 1);
                     }
                     const int k1 = k_end(f, tile);
                     for (int step = k_first(f, tile); step < k1; ++step, ++pos) {
@@ -892,6 +895,8 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 if (ok) tc_commit_one(one, smem_u32(&s.tfull[buf]));
             }
         }
+        if (!ok)               // gave up: the MMAs in flight end before the block frees its tensor memory and leaves
+            for (int i = 0; i < 64; ++i) __nanosleep(1000);
     } else {
         // ---------------- epilogue warps
         const int e = threadIdx.x - 32 * FW_EPI_WARP0;   // 0..255
