@@ -815,10 +815,14 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         const bool fresh = i == 0 || i == a_wrap || it.tile == 0;
                         if (fresh && i > 0) ++as;
                         const int kpos = pos + 2 * i, b = (at + i) & 1;
-                        // query rows of the segment, the K tile, and the score buffer (read by the softmax two tiles ago)
+                        // Query rows of the segment, the score buffer (read by the softmax two tiles ago), and the K tile.  With an odd
+                        // ring the K tile's slot held the V tile of two tiles ago, whose arrival this warp has not followed: its
+                        // barrier may be a phase behind, and the parity would then name the phase before the one meant.  The output
+                        // of that tile being complete says that the V tile has come and gone.
+                        const uint32_t before = ((uint32_t)((at + i) >> 1) & 1u) ^ 1u;
                         ok = (!fresh || mbar_wait_warp(smem_u32(&s.qfull[as & 1]), (uint32_t)(as >> 1) & 1u, abort_flag)) &&
-                             mbar_wait_warp(full_bar(kpos), ring_par(kpos), abort_flag) &&
-                             mbar_wait_warp(smem_u32(&s.pfull[b]), ((uint32_t)((at + i) >> 1) & 1u) ^ 1u, abort_flag);
+                             mbar_wait_warp(smem_u32(NS % 2 ? &s.ofull[b] : &s.pfull[b]), before, abort_flag) &&
+                             mbar_wait_warp(full_bar(kpos), ring_par(kpos), abort_flag);
                         if (!ok) break;
                         tc_fence_after();
                         const uint64_t ka = smem_desc(slot_ptr(kpos)), qa = smem_desc(smem_u32(Qs) + (as & 1) * Q_BYTES);
