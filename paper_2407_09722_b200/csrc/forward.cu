@@ -815,10 +815,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         const bool fresh = i == 0 || i == a_wrap || it.tile == 0;
                         if (fresh && i > 0) ++as;
                         const int kpos = pos + 2 * i, b = (at + i) & 1;
-                        // Query rows of the segment, the score buffer (read by the softmax two tiles ago), and the K tile.  With an odd
-                        // ring the K tile's slot held the V tile of two tiles ago, whose arrival this warp has not followed: its
-                        // barrier may be a phase behind, and the parity would then name the phase before the one meant.  The output
-                        // of that tile being complete says that the V tile has come and gone.
+                        // Query rows of the segment, the score buffer (read by the softmax two tiles ago), and the K tile.  With an
+                        // odd ring the K tile's slot held the V tile of two tiles ago, whose arrival this warp has not followed:
+                        // the slot's barrier may be a phase behind, and the parity would then name the phase before the one
+                        // meant.  The output of that tile being complete says that the V tile has come and gone.
                         const uint32_t before = ((uint32_t)((at + i) >> 1) & 1u) ^ 1u;
                         ok = (!fresh || mbar_wait_warp(smem_u32(&s.qfull[as & 1]), (uint32_t)(as >> 1) & 1u, abort_flag)) &&
                              mbar_wait_warp(smem_u32(NS % 2 ? &s.ofull[b] : &s.pfull[b]), before, abort_flag) &&
@@ -835,6 +835,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         tc_commit_one(one, empty_bar(kpos));
                     }
                     if (a_n > 0) ++as;
+                    if (NS % 2 && a_n > 1 && ok) {     // (the next phase's first slot held the last V tile but one)
+                        const int n = at + a_n - 2;
+                        ok = mbar_wait_warp(smem_u32(&s.ofull[n & 1]), (uint32_t)(n >> 1) & 1u, abort_flag);
+                    }
                 } else {
                     constexpr uint32_t idesc_o = IDESC | (1u << 15) | ((uint32_t)(NQ2 >> 3) << 17);
                     for (int i = 0; i < a_n; ++i) {
