@@ -254,7 +254,7 @@ size_t carve(mtad_ctx* c, const mtad_model_desc* t, const mtad_model_desc* a, in
     sc.tc_counters = k.take<int32_t>(max_tiles, "tc_counters");
     sc.lm_part = k.take<float4>(Tc * std::max(lm_tiles, mx([](const mtad_model_desc* m) { return fw_parts_max(*m, kCtas, true); })),
                                 "lm_part");
-    sc.fw_sync_words = (int)mx([&](const mtad_model_desc* m) { return fw_sync_words(m->layers, max_batch, m->n_kv_heads, kCtas); });
+    sc.fw_sync_words = (int)mx([&](const mtad_model_desc* m) { return fw_sync_words(*m, max_batch, kCtas); });
     sc.fw_sync = k.take<int32_t>(sc.fw_sync_words, "fw_sync");
     sc.fw_part = k.take<float>((size_t)kCtas * FW_MAX_ROWS * TC_TILE_N, "fw_part");
     FwLayer* fw_t = k.take<FwLayer>(t->layers, "fw_target");
@@ -452,7 +452,7 @@ bool build_forward_plan(ForwardPlan& fp, const Scratch& sc, const RowMeta& rm, c
     a.max_batch = m.max_batch; a.cap = d.kv_capacity;
     a.parts0 = 1; a.inv_dim = 1.f / (float)d.d_model; a.eps = d.rms_eps;
     a.sync = sc.fw_sync; a.acnt = sc.fw_sync + 5 * d.layers + 1;
-    a.kcnt = a.acnt + (size_t)m.max_batch * d.n_kv_heads; a.kpart = sc.fw_part;
+    a.kcnt = a.acnt + fw_pairs(d, m.max_batch); a.kpart = sc.fw_part;
     a.sumsq_a = sc.sumsq_a; a.sumsq_b = sc.sumsq_b; a.hidden = sc.hidden;
     a.x_d = sc.xd; a.x_a = sc.xa; a.x_f = sc.xf; a.q_hi = sc.q_hi; a.q_lo = sc.q_lo;
     a.cache = static_cast<__nv_bfloat16*>(d.kv_cache);
@@ -1171,7 +1171,7 @@ void audit_forward(Audit& au, const mtad_ctx& c, const ModelView& m, int B, int 
         au.ws("xa", idx_xrow(T - 1, terms, terms - 1, qd, qd - 1) + 1);
         au.ws("xf", idx_xrow(T - 1, terms, terms - 1, d.d_ffn, d.d_ffn - 1) + 1);
         au.ws("attn_part", (size_t)T * Hq * pieces * (hd + 2));
-        au.ws("fw_sync", fw_sync_words(d.layers, m.max_batch, Hkv, kCtas));
+        au.ws("fw_sync", fw_sync_words(d, m.max_batch, kCtas));
         for (const FwPhase* f : {&a.ph[FW_O], &a.ph[FW_DOWN]})
             if (f->c > 1) au.ws("fw_part", (size_t)f->n_tiles * T * f->h);
         au.ws(&m == &c.target ? "fw_target" : "fw_aux", d.layers);

@@ -45,9 +45,9 @@ constexpr int FW_THREADS = 32 * 12;
 constexpr int FW_EPI_WARP0 = 4;
 constexpr int FW_EPI = 256;
 constexpr int FW_UNION = 32 * 1024;       // epilogue tile Y, or the attention's query and probability tiles
-constexpr int FW_ACC = 240;               // accumulator columns of a tile, of 256 (the drain reads up to 15 columns further)
+constexpr int FW_ACC = 240;               // accumulator columns of a tile, of 256 (the drain reads up to 15 columns further),
+constexpr int FW_ACC_ONE = 496;           // or of 512 where a tile takes both buffers
 constexpr float FW_LAZY = 64.f;           // log2 of how far a score may exceed its row's reference value
-constexpr int FW_TM_D = 128;              // attention: tensor-memory columns 0 / 64 scores, 128 / 192 outputs
 
 __device__ __forceinline__ bool grid_wait(const int* c, int want, volatile int* abort_flag) {
     const uint32_t limit = (uint32_t)abort_flag[1];
@@ -164,21 +164,26 @@ __device__ __forceinline__ void attn_next(AttnPos& it, const SeqMeta* meta, int 
     if (it.bi < B) it.nt = attn_tiles(meta[it.bi]);
 }
 
+// What the attention's epilogue warps tell one another, for NR rows in each half of them
+template <int NR>
+struct alignas(16) FwAttn {
+    float smx[2][NR][4];                  // row maxima of the four warps
+    float sl[2][2][NR][4];                // row sums of the four warps, two segments
+    float sm[2][NR];                      // first scores of a segment
+};
 struct FwTail {
     SeqMeta meta[MTAD_MAX_BATCH];
     float rstd[FW_MAX_ROWS];
     int slot[FW_MAX_ROWS];                // cache slot of a row, -1: inactive
     uint8_t rowb[FW_MAX_ROWS];            // its sequence within the call
-    alignas(16) float smx[2][8][4];       // attention, per half of the rows: row maxima of the four warps
-    alignas(16) float sl[2][2][8][4];     // row sums of the four warps, two segments
-    float sm[2][8];                       // first scores of a segment
+    FwAttn<FW_QROWS / 2> attn;            // (the wide attention's lies behind its query tile)
     uint64_t full[4], empty[4];
     uint64_t tfull[2], tempty[2], sfull[2], pfull[2], ofull[2], qfull[2];
     uint32_t tmem_ptr;
     int abort_flag[2];
     int last[2];
 };
-static_assert(offsetof(FwTail, smx) % 16 == 0 && offsetof(FwTail, sl) % 16 == 0 && offsetof(FwTail, full) % 8 == 0, "alignment of the tail");
+static_assert(offsetof(FwTail, attn) % 16 == 0 && offsetof(FwTail, full) % 8 == 0, "alignment of the tail");
 static_assert(FW_RING + FW_UNION + sizeof(FwTail) <= 227 * 1024, "shared memory of the forward");
 
 // The epilogue group's part of one projection: row statistics, then per tile the accumulators -> Y in shared memory ->
@@ -278,7 +283,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
         ok = all_of(1, FW_EPI, ok);
         if (!ok) return false;
         tc_fence_after();
-        const uint32_t t_acc = tmem_lane + buf * 256;
+        const uint32_t t_acc = tmem_lane + (f.both ? 0 : buf * 256);
         for (int r0 = 0; r0 < T; r0 += blk) {
             const int r1 = min(T, r0 + blk), nr = r1 - r0;
             // ---- accumulators -> Y[row][box][lane], the terms of a row added up
@@ -564,10 +569,11 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
 // thread, the pieces in order (deterministic) and six at a time, so that their loads are in flight together.
 template <int HD, int NQP>
 __device__ __forceinline__ void merge_pieces(const FwArgs& a, const FwTail& s, const AttnPos& q, int n_piece, int G, int e) {
-    const int nrows = s.meta[q.bi].nrows, n_q = min(G * nrows, NQP);
+    const int nqb = NQP > FW_QROWS ? a.nqb : 1, g = q.g / nqb, r0 = (q.g - g * nqb) * a.qrows;
+    const int nrows = s.meta[q.bi].nrows, n_q = min(G * nrows - r0, a.qrows);
     for (int i = e; i < n_q * (HD / 4); i += FW_EPI) {
-        const int r = i / (HD / 4), c4 = i % (HD / 4);
-        const int hq = G == 1 ? 0 : r / nrows, t = q.bi * a.R + r - hq * nrows, h = q.g * G + hq;
+        const int r = r0 + i / (HD / 4), c4 = i % (HD / 4);
+        const int hq = G == 1 ? 0 : r / nrows, t = q.bi * a.R + r - hq * nrows, h = g * G + hq;
         const size_t o = ((size_t)t * a.Hq + h) * a.pieces;
         const float2* ml = reinterpret_cast<const float2*>(a.part + (size_t)a.T * a.Hq * a.pieces * HD) + o;
         const float4* po = reinterpret_cast<const float4*>(a.part + o * HD) + c4;
@@ -605,7 +611,7 @@ __device__ __forceinline__ void merge_pieces(const FwArgs& a, const FwTail& s, c
         store_terms4(make_float4(o4.x * f, o4.y * f, o4.z * f, o4.w * f),
                      a.x_a + (size_t)t * a.terms * a.Hq * HD + (size_t)h * HD + c4 * 4, (size_t)a.Hq * HD, a.terms);
     }
-    if (e == 0) a.acnt[q.bi * a.Hkv + q.g] = 0;       // ready for the next layer
+    if (e == 0) a.acnt[q.bi * a.Hkv * nqb + q.g] = 0; // ready for the next layer
 }
 
 template <int HD, int NQP, bool FEW, int NS>
@@ -616,12 +622,19 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     constexpr int Q_BYTES = NQ2 * HD * 2;              // one query tile
     constexpr int P_BYTES = NQ2 * FW_KEYS * 2;         // one probability tile
     constexpr int FW_SLOT = FW_RING / NS;
+    // Wide attention: up to 40 query rows, whose tiles outgrow the union.  The probabilities of a tile lie behind its V tile, in
+    // the rest of the ring slot (free by then: the slot's item before it was used before this tile's scores were formed, as
+    // long as that item is the K tile of the tile before, three items ago), and there is one query tile instead of two.
+    constexpr bool WIDE = NQP > FW_QROWS;
+    static_assert(!WIDE || (NS == 3 && (int)KV_BYTES + P_BYTES <= FW_SLOT && Q_BYTES + (int)sizeof(FwAttn<NQP / 2>) <= FW_UNION), "wide attention");
+    constexpr int TM = WIDE ? 128 : 64;                // attention: tensor-memory columns 0 / TM scores, 2 TM / 3 TM outputs
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* uni = smem + FW_RING;
     FwTail& s = *reinterpret_cast<FwTail*>(uni + FW_UNION);
     float* Y = reinterpret_cast<float*>(uni);
-    uint8_t* Qs = uni;                                 // [2][Q_BYTES]
+    uint8_t* Qs = uni;                                 // [2][Q_BYTES], wide: [Q_BYTES]
     uint8_t* Ps = uni + 2 * Q_BYTES;                   // [2][P_BYTES]
+    const int nqb = WIDE ? a.nqb : 1, heads = a.Hkv * nqb;           // attention: (KV head, query block)s of a sequence
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const int cta = (int)blockIdx.x, n_cta = a.n_cta;
     const int T = a.T, cols = a.cols, terms = a.terms;
@@ -667,18 +680,18 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     const uint32_t tmem = s.tmem_ptr;
     volatile int* abort_flag = s.abort_flag;
     int a_tot = 0;
-    for (int b = 0; b < a.B; ++b) a_tot += attn_tiles(s.meta[b]) * a.Hkv;
+    for (int b = 0; b < a.B; ++b) a_tot += attn_tiles(s.meta[b]) * heads;
     const int a_per = max(1, (a_tot + n_cta - 1) / n_cta);
     const int a_lo = min(cta * a_per, a_tot), a_n = min(a_lo + a_per, a_tot) - a_lo;
     // This block's items in the order it takes them: if its range holds more than one segment (run of tiles of one sequence
     // and KV head), the first segment comes last, because it ends with the tile that holds the call's own rows and cannot
     // be requested before the phase has been released.  a_wrap: where the order returns to the front of the range.
-    const AttnPos a_zero = attn_find(s.meta, a.B, a.Hkv, a_lo), a_last = attn_find(s.meta, a.B, a.Hkv, max(a_lo, a_lo + a_n - 1));
+    const AttnPos a_zero = attn_find(s.meta, a.B, heads, a_lo), a_last = attn_find(s.meta, a.B, heads, max(a_lo, a_lo + a_n - 1));
     const int a_rot = a_zero.nt - a_zero.tile < a_n ? a_zero.nt - a_zero.tile : 0, a_wrap = a_n - a_rot;
-    const AttnPos a_first = a_rot ? attn_find(s.meta, a.B, a.Hkv, a_lo + a_rot) : a_zero;
+    const AttnPos a_first = a_rot ? attn_find(s.meta, a.B, heads, a_lo + a_rot) : a_zero;
     auto attn_step = [&](AttnPos& it, int next) {          // item `next` of the order, from the one before
         if (next == a_wrap) it = a_zero;
-        else attn_next(it, s.meta, a.B, a.Hkv);
+        else attn_next(it, s.meta, a.B, heads);
     };
     auto slot_ptr = [&](int pos) { return smem_u32(smem) + (uint32_t)(pos % NS) * FW_SLOT; };
     auto full_bar = [&](int pos) { return smem_u32(&s.full[pos % NS]); };
@@ -704,7 +717,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     AttnPos it = a_first;
                     for (int i = 0; i < a_n && ok; attn_step(it, ++i)) {
                         const SeqMeta sm = s.meta[it.bi];
-                        const int plane = ((layer * a.max_batch + sm.seq) * 2) * a.Hkv + it.g;
+                        const int plane = ((layer * a.max_batch + sm.seq) * 2) * a.Hkv + it.g / nqb;
                         if (!waited && (it.tile + 1) * FW_KEYS > sm.L) {
                             ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
                             proxy_fence();
@@ -825,10 +838,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                              mbar_wait_warp(full_bar(kpos), ring_par(kpos), abort_flag);
                         if (!ok) break;
                         tc_fence_after();
-                        const uint64_t ka = smem_desc(slot_ptr(kpos)), qa = smem_desc(smem_u32(Qs) + (as & 1) * Q_BYTES);
+                        const uint64_t ka = smem_desc(slot_ptr(kpos)), qa = smem_desc(smem_u32(Qs) + (WIDE ? 0 : as & 1) * Q_BYTES);
 #pragma unroll
                         for (int ks = 0; ks < HD / 16; ++ks)
-                            tc_mma_one(one, tmem + b * 64, ka + (ks >> 2) * (FW_KEYS * 8) + (ks & 3) * 2,
+                            tc_mma_one(one, tmem + b * TM, ka + (ks >> 2) * (FW_KEYS * 8) + (ks & 3) * 2,
                                        qa + (ks >> 2) * (NQ2 * 8) + (ks & 3) * 2, idesc_s, ks > 0 ? 1u : 0u);
                         tc_commit_one(one, smem_u32(&s.sfull[b]));
                         tc_commit_one(one, empty_bar(kpos));
@@ -849,10 +862,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                              mbar_wait_warp(full_bar(vpos), ring_par(vpos), abort_flag);
                         if (!ok) break;
                         tc_fence_after();
-                        const uint64_t va = smem_desc_mn(slot_ptr(vpos)), pa = smem_desc(smem_u32(Ps) + b * P_BYTES);
+                        const uint64_t va = smem_desc_mn(slot_ptr(vpos)), pa = smem_desc(WIDE ? slot_ptr(vpos) + KV_BYTES : smem_u32(Ps) + b * P_BYTES);
 #pragma unroll
                         for (int ks = 0; ks < FW_KEYS / 16; ++ks)
-                            tc_mma_one(one, tmem + FW_TM_D + b * 64, va + ks * 128, pa + (ks >> 2) * (NQ2 * 8) + (ks & 3) * 2,
+                            tc_mma_one(one, tmem + (2 + b) * TM, va + ks * 128, pa + (ks >> 2) * (NQ2 * 8) + (ks & 3) * 2,
                                        idesc_o, ks > 0 ? 1u : 0u);
                         tc_commit_one(one, smem_u32(&s.ofull[b]));
                         tc_commit_one(one, empty_bar(vpos));
@@ -871,10 +884,12 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
             for (int tile = cta; tile < f.n_tiles && ok; tile += n_cta, ++tcount) {
                 const int buf = tcount & 1;
                 ok = mbar_wait_warp(smem_u32(&s.tempty[buf]), ((uint32_t)(tcount >> 1) & 1u) ^ 1u, abort_flag);
+                if (f.both && tcount > 0)              // (its accumulators take the columns of the tile before as well)
+                    ok = ok && mbar_wait_warp(smem_u32(&s.tempty[buf ^ 1]), (uint32_t)((tcount - 1) >> 1) & 1u, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
                 const bool mine = me == 0 || nbox == 2 || dual;
-                const uint32_t d = tmem + buf * 256 + me * sc;
+                const uint32_t d = tmem + (f.both ? 0 : buf * 256) + me * sc;
                 uint32_t acc = 0;
                 int turn = 0;                              // dual: MMAs along k alternate between the warps
                 const int k1 = k_end(f, tile);
@@ -926,18 +941,36 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 if (!ok) break;
                 pos += ring_qkv;
                 const int G = a.Hq / a.Hkv, kl = quad * 32 + lane;    // this thread's key of a tile, later its head dimension
-                constexpr int NR = NQP / 2;                           // this thread's query rows: half, half + 2, ...
+                constexpr int NR = NQP / 2;                           // this thread's query rows: half, half + 2, ...; wide:
+                auto row_of = [&](int x) { return WIDE ? half * NR + x : 2 * x + half; };        // NR neighbouring ones
+                auto& sa = *reinterpret_cast<FwAttn<WIDE ? NR : FW_QROWS / 2>*>(WIDE ? Qs + Q_BYTES : reinterpret_cast<uint8_t*>(&s.attn));
+                // scores or outputs at column `col`: this thread's rows, hi and lo parts added up
+                auto tm_rows = [&](int col, float* v) {
+                    if constexpr (WIDE) {
+                        tc_ld20_sum(t_lane + col + half * NR, t_lane + col + NQP + half * NR, v);
+                    } else {
+                        float c[NQ2];
+                        if (NQ2 == 16) tc_ld16(t_lane + col, c);
+                        else { tc_ld16(t_lane + col, c); tc_ld16(t_lane + col + 16, c + NQ2 - 16); }
+#pragma unroll
+                        for (int x = 0; x < NR; ++x) v[x] = half == 0 ? c[2 * x] + c[NQP + 2 * x] : c[2 * x + 1] + c[NQP + 2 * x + 1];
+                    }
+                };
+                // query rows of a segment: KV head, first row, how many
+                auto q_head = [&](const AttnPos& q) { return WIDE ? q.g / nqb : q.g; };
+                auto q_base = [&](const AttnPos& q) { return WIDE ? q.g % nqb * a.qrows : 0; };
+                auto q_count = [&](const AttnPos& q) { return min(G * s.meta[q.bi].nrows - q_base(q), a.qrows); };
                 // query rows of (sequence, KV head) -> buffer `qb`, hi rows then lo rows, K-major
                 auto load_q = [&](const AttnPos& q, int qb) {
-                    const int nrows = s.meta[q.bi].nrows, n_q = min(G * nrows, NQP);
-                    uint8_t* dst = Qs + qb * Q_BYTES;
+                    const int nrows = s.meta[q.bi].nrows, n_q = q_count(q), rb = q_base(q);
+                    uint8_t* dst = Qs + (WIDE ? 0 : qb) * Q_BYTES;
 #pragma unroll
                     for (int idx = e; idx < NQ2 * (HD / 8); idx += FW_EPI) {
-                        const int row = idx / (HD / 8), c = idx % (HD / 8), r = row & (NQP - 1);
+                        const int row = idx / (HD / 8), c = idx % (HD / 8), r = row >= NQP ? row - NQP : row;
                         const bool valid = r < n_q;
-                        const int rr = valid ? r : 0, hq = G == 1 ? 0 : rr / nrows;
+                        const int rr = valid ? rb + r : 0, hq = G == 1 ? 0 : rr / nrows;
                         const __nv_bfloat16* src = (row >= NQP ? a.q_lo : a.q_hi) +
-                            ((size_t)(q.bi * a.R + rr - hq * nrows) * a.Hq + q.g * G + hq) * HD + c * 8;
+                            ((size_t)(q.bi * a.R + rr - hq * nrows) * a.Hq + q_head(q) * G + hq) * HD + c * 8;
                         cp_async16(smem_u32(dst + (c >> 3) * (NQ2 * 128) + row * 128 + (((c & 7) ^ (row & 7)) << 4)), src, valid);
                     }
                     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -947,7 +980,8 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&s.qfull[qb]));
                 };
-                // the first two segments' query rows go out at once, a later segment's when the one two before it has ended
+                // the first two segments' query rows go out at once, a later segment's when the one two before it has ended (wide:
+                // the first one's, and a later one's when the scores of the one before it have been formed)
                 AttnPos ahead = a_first;
                 int ahead_i = 0;
                 bool more = a_n > 0;
@@ -961,7 +995,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 if (more) {
                     load_q(ahead, as & 1);
                     next_seg();
-                    if (more) {
+                    if (!WIDE && more) {
                         load_q(ahead, (as + 1) & 1);
                         asm volatile("cp.async.wait_group 1;" ::: "memory");
                         q_ready(as & 1);
@@ -979,12 +1013,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     const int b = tile_no & 1;
                     ok = warp_wait(smem_u32(&s.ofull[b]), (uint32_t)(tile_no >> 1) & 1u, abort_flag, ok, lane);
                     tc_fence_after();
-                    float c[NQ2];
-                    if (NQ2 == 16) tc_ld16(t_lane + FW_TM_D + b * 64, c);
-                    else { tc_ld16(t_lane + FW_TM_D + b * 64, c); tc_ld16(t_lane + FW_TM_D + b * 64 + 16, c + 16); }
+                    float c[NR];
+                    tm_rows((2 + b) * TM, c);
 #pragma unroll
-                    for (int x = 0; x < NR; ++x)
-                        acc[x] += half == 0 ? c[2 * x] + c[NQP + 2 * x] : c[2 * x + 1] + c[NQP + 2 * x + 1];
+                    for (int x = 0; x < NR; ++x) acc[x] += c[x];
                 };
                 // end of a segment: the rows' sums over the lanes, then the rows leave - final, or as a piece
                 auto finish = [&](const AttnPos& q) {
@@ -995,17 +1027,17 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         for (int x = 0; x < NR; ++x) l[x] += __shfl_xor_sync(0xffffffffu, l[x], o);
 #pragma unroll
                     for (int x = 0; x < NR; ++x)
-                        if (lane == x) s.sl[sb][half][x][quad] = l[x];
+                        if (lane == x) sa.sl[sb][half][x][quad] = l[x];
                     ok = all_of(2 + half, 128, ok);
-                    const int nrows = s.meta[q.bi].nrows, n_q = min(G * nrows, NQP);
+                    const int nrows = s.meta[q.bi].nrows, n_q = q_count(q), rb = q_base(q), g = q_head(q);
                     const int first = q.f0 / a_per, n_piece = (q.f0 + q.nt - 1) / a_per - first + 1, piece = cta - first;
                     if (ok && (HD == 128 || kl < HD)) {
 #pragma unroll
                         for (int x = 0; x < NR; ++x) {
-                            const int r = 2 * x + half;
+                            const int r = row_of(x);
                             if (r < n_q) {
-                                const int hq = G == 1 ? 0 : r / nrows, t = q.bi * a.R + r - hq * nrows, h = q.g * G + hq;
-                                const float4 l4 = *reinterpret_cast<const float4*>(s.sl[sb][half][x]);
+                                const int hq = G == 1 ? 0 : (rb + r) / nrows, t = q.bi * a.R + rb + r - hq * nrows, h = g * G + hq;
+                                const float4 l4 = *reinterpret_cast<const float4*>(sa.sl[sb][half][x]);
                                 const float ls = (l4.x + l4.y) + (l4.z + l4.w);
                                 if (n_piece == 1) {
                                     store_terms(acc[x] / ls, a.x_a + (size_t)t * terms * a.Hq * HD + (size_t)h * HD + kl,
@@ -1019,8 +1051,8 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             }
                         }
                     }
-                    if (more) next_seg();
-                    if (more) {                                           // (the scores of this segment are formed, its query buffer is free)
+                    if (!WIDE && more) next_seg();
+                    if (!WIDE && more) {                                  // (the scores of this segment are formed, its query buffer is free)
                         load_q(ahead, sb);
                         asm volatile("cp.async.wait_group 0;" ::: "memory");
                         q_ready(sb);
@@ -1040,8 +1072,9 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     }
                     const SeqMeta sm = s.meta[it.bi];
                     const int nrows = sm.nrows, L = sm.L, nkeys = sm.nkeys;
-                    const int n_q = min(G * nrows, NQP);
+                    const int n_q = q_count(it), rb = q_base(it);
                     const int t0 = it.bi * a.R;                       // query row r: row t0 + r % nrows, head g * G + r / nrows
+                    const bool turn = WIDE && i + 1 < a_n && (i + 1 == a_wrap || it.tile + 1 == it.nt);     // the segment's last
                     const int b = at & 1;
                     const uint32_t par = (uint32_t)(at >> 1) & 1u;
                     const int j = it.tile * FW_KEYS + kl;
@@ -1055,7 +1088,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             vis = 0;
 #pragma unroll
                             for (int x = 0; x < NR; ++x) {
-                                const int r = 2 * x + half, rr = r < n_q ? (G == 1 ? r : r % nrows) : 0;
+                                const int r = row_of(x), rr = r < n_q ? (G == 1 ? rb + r : (rb + r) % nrows) : 0;
                                 vis |= ((a.rm.mask[(size_t)(t0 + rr) * MTAD_MASK_WORDS + (sr >> 5)] >> (sr & 31)) & 1u) << x;
                             }
                         }
@@ -1063,26 +1096,20 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     ok = warp_wait(smem_u32(&s.sfull[b]), par, abort_flag, ok, lane);
                     tc_fence_after();
                     float v[NR];
-                    {
-                        float c[NQ2];
-                        if (NQ2 == 16) tc_ld16(t_lane + b * 64, c);
-                        else { tc_ld16(t_lane + b * 64, c); tc_ld16(t_lane + b * 64 + 16, c + 16); }
+                    tm_rows(b * TM, v);
 #pragma unroll
-                        for (int x = 0; x < NR; ++x) {
-                            const float y = half == 0 ? c[2 * x] + c[NQP + 2 * x] : c[2 * x + 1] + c[NQP + 2 * x + 1];
-                            v[x] = ((vis >> x) & 1u) ? y : -CUDART_INF_F;
-                        }
-                    }
+                    for (int x = 0; x < NR; ++x) v[x] = ((vis >> x) & 1u) ? v[x] : -CUDART_INF_F;
+                    if (turn) load_q(ahead, 0);                       // (this segment's scores are formed, the query tile is free)
                     // The reference value m of a row need not be its maximum: numerators and sums have the exponent range that
                     // fp32 and bf16 share, and a common factor costs no precision.  A segment starts with the score of its first
                     // key, and m moves to the maximum only when a score exceeds it by more than 2^64 (or no key was seen yet).
                     if (fresh) {
                         if (kl == 0)
 #pragma unroll
-                            for (int x = 0; x < NR; ++x) s.sm[half][x] = v[x];
+                            for (int x = 0; x < NR; ++x) sa.sm[half][x] = v[x];
                         bar_n(2 + half, 128);
 #pragma unroll
-                        for (int x = 0; x < NR; ++x) m[x] = s.sm[half][x];
+                        for (int x = 0; x < NR; ++x) m[x] = sa.sm[half][x];
                     }
                     bool calm = true;
 #pragma unroll
@@ -1101,11 +1128,11 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             for (int x = 0; x < NR; ++x) wm[x] = fmaxf(wm[x], __shfl_xor_sync(0xffffffffu, wm[x], o));
 #pragma unroll
                         for (int x = 0; x < NR; ++x)
-                            if (lane == x) s.smx[half][x][quad] = wm[x];
+                            if (lane == x) sa.smx[half][x][quad] = wm[x];
                         bar_n(2 + half, 128);
 #pragma unroll
                         for (int x = 0; x < NR; ++x) {
-                            const float4 q4 = *reinterpret_cast<const float4*>(s.smx[half][x]);
+                            const float4 q4 = *reinterpret_cast<const float4*>(sa.smx[half][x]);
                             const float mn = fmaxf(m[x], fmaxf(fmaxf(q4.x, q4.y), fmaxf(q4.z, q4.w)));
                             f[x] = mn == -CUDART_INF_F ? 1.f : exp2f(m[x] - mn);
                             m[x] = mn;
@@ -1113,16 +1140,18 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         }
                         bar_n(2 + half, 128);                         // (smx is free again)
                     }
-                    uint8_t* pt = Ps + b * P_BYTES + (kl >> 6) * (NQ2 * 128) + (kl & 7) * 2 + half * 128;
+                    uint8_t* pt = (WIDE ? smem + (size_t)((pos + 2 * i + 1) % NS) * FW_SLOT + KV_BYTES : Ps + b * P_BYTES) +
+                                  (kl >> 6) * (NQ2 * 128) + (kl & 7) * 2 + row_of(0) * 128;
+                    constexpr int RS = WIDE ? 128 : 256;              // bytes between this thread's rows
                     const int pc = (kl & 63) >> 3;
 #pragma unroll
                     for (int x = 0; x < NR; ++x) {
                         const float pv = exp2f(v[x] - (m[x] == -CUDART_INF_F ? 0.f : m[x]));        // exp2(-inf) = 0
                         l[x] += pv;
                         const __nv_bfloat16 hi = __float2bfloat16_rn(pv);
-                        uint8_t* d = pt + ((pc ^ ((2 * x + half) & 7)) << 4);
-                        *reinterpret_cast<__nv_bfloat16*>(d + 2 * x * 128) = hi;
-                        *reinterpret_cast<__nv_bfloat16*>(d + (NQP + 2 * x) * 128) = __float2bfloat16_rn(pv - __bfloat162float(hi));
+                        uint8_t* d = pt + ((pc ^ (row_of(x) & 7)) << 4) + x * RS;
+                        *reinterpret_cast<__nv_bfloat16*>(d) = hi;
+                        *reinterpret_cast<__nv_bfloat16*>(d + NQP * 128) = __float2bfloat16_rn(pv - __bfloat162float(hi));
                     }
                     if ((it.tile + 1) * FW_KEYS > nkeys) {
                         // rows of V past the last key: their probabilities are 0, but 0 x (stale value) must not make a NaN
@@ -1140,6 +1169,11 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&s.pfull[b]));
+                    if (turn) {
+                        asm volatile("cp.async.wait_group 0;" ::: "memory");
+                        q_ready((as + 1) & 1);
+                        next_seg();
+                    }
                     if (!quiet)
 #pragma unroll
                         for (int x = 0; x < NR; ++x) acc[x] *= f[x];
@@ -1163,7 +1197,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         if (n_piece > 1 && (e == 0 || a_last.f0 != a_zero.f0)) {
                             int old;
                             asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;"
-                                         : "=r"(old) : "l"(a.acnt + q.bi * a.Hkv + q.g) : "memory");
+                                         : "=r"(old) : "l"(a.acnt + q.bi * heads + q.g) : "memory");
                             last = old + 1 == n_piece ? n_piece : 0;
                         }
                         s.last[e] = last;
@@ -1273,12 +1307,15 @@ void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta, int cls) {
 bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
     const int T = B * R, G = d.n_q_heads / d.n_kv_heads;
     if (d.head_dim != 64 && d.head_dim != 128) return false;
-    if (T > FW_MAX_ROWS || G * R > FW_MAX_QROWS || B > MTAD_MAX_BATCH) return false;
+    if (T > FW_MAX_ROWS || B > MTAD_MAX_BATCH) return false;
     if (d.d_model >= 8192 && T > 32) return false;          // the accurate K / V projection has launches of its own
     a.T = T; a.B = B; a.R = R; a.terms = tc_terms(T);
     a.cols = (a.terms * T + 15) / 16 * 16;
     if (a.cols > FW_MAX_COLS) return false;
-    a.cls = T <= 8 ? 0 : 2;                                // (four slots and the lean epilogues: up to eight rows)
+    const bool wide = G * R > FW_QROWS;
+    a.nqb = wide ? up_div(G * R, FW_QROWS_WIDE) : 1;
+    a.qrows = up_div(G * R, a.nqb);
+    a.cls = T <= 8 && !wide ? 0 : 2;                       // (four slots and the lean epilogues: up to eight rows)
     while (FW_CLASS[a.cls].cols < a.cols) ++a.cls;
     fw_geometry(a.ph, d, n_cta, a.cls);
     a.n_cta = n_cta; a.n_layers = d.layers;
@@ -1289,7 +1326,8 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
         f.S = 1;
         for (int S = 2; S <= f.kb; ++S)
             if (f.kb % S == 0 && S * f.hr <= TC_TILE_N && S * a.cols * f.nbox <= FW_ACC) f.S = S;
-        if (f.b_off + f.kb * a.cols * 128 > FW_RING / FW_CLASS[a.cls].slots || f.nbox * f.S * a.cols > FW_ACC) return false;
+        if (f.b_off + f.kb * a.cols * 128 > FW_RING / FW_CLASS[a.cls].slots || f.nbox * f.S * a.cols > FW_ACC_ONE) return false;
+        f.both = f.nbox * f.S * a.cols > FW_ACC ? 1 : 0;
         if ((k == FW_O || k == FW_DOWN) && (f.n_tiles > n_cta || f.steps < f.c)) return false;
         // one box: the MMAs along k alternate between two accumulators where they fit and every block has two
         f.dual = f.nbox == 1 && 2 * f.S * a.cols <= FW_ACC && f.steps / f.c * (f.kb / f.S) >= 2 ? 1 : 0;
@@ -1329,15 +1367,15 @@ cudaError_t launch_forward(const FwArgs& a, cudaStream_t st) {
         cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, kernel, a);
     };
-    // instantiations: head size, query rows of a KV head, few rows in all, ring slots
-    const bool q8 = (a.Hq / a.Hkv) * a.R <= 8, few = a.T <= 8;
-    auto pick = [&](auto hd, auto nqp) -> cudaError_t {
-        constexpr int HD = decltype(hd)::value, NQP = decltype(nqp)::value;
-        return few ? go(forward_kernel<HD, NQP, true, FW_CLASS[0].slots>) : go(forward_kernel<HD, NQP, false, FW_CLASS[2].slots>);
+    // instantiations: head size, query rows of an attention item, few rows in all, ring slots
+    auto pick = [&](auto hd) -> cudaError_t {
+        constexpr int HD = decltype(hd)::value, NF = FW_CLASS[0].slots, NM = FW_CLASS[2].slots;
+        const bool q8 = (a.Hq / a.Hkv) * a.R <= 8, q16 = (a.Hq / a.Hkv) * a.R <= FW_QROWS;
+        if (a.cls < 2) return q8 ? go(forward_kernel<HD, 8, true, NF>) : go(forward_kernel<HD, FW_QROWS, true, NF>);
+        if (q8) return go(forward_kernel<HD, 8, false, NM>);
+        return q16 ? go(forward_kernel<HD, FW_QROWS, false, NM>) : go(forward_kernel<HD, FW_QROWS_WIDE, false, NM>);
     };
-    using std::integral_constant;
-    if (a.hd == 128) return q8 ? pick(integral_constant<int, 128>{}, integral_constant<int, 8>{}) : pick(integral_constant<int, 128>{}, integral_constant<int, 16>{});
-    return q8 ? pick(integral_constant<int, 64>{}, integral_constant<int, 8>{}) : pick(integral_constant<int, 64>{}, integral_constant<int, 16>{});
+    return a.hd == 128 ? pick(std::integral_constant<int, 128>{}) : pick(std::integral_constant<int, 64>{});
 }
 
 }  // namespace mtad

@@ -8,9 +8,10 @@ namespace mtad {
 constexpr int FW_RING = 192 * 1024;       // the copy ring: four slots, or three where the operand rows are many; a slot
                                           // holds one step of a projection, or 128 keys of K or V
 constexpr int FW_KEYS = 128;              // keys of an attention tile
-constexpr int FW_MAX_ROWS = 56;           // rows of a call
-constexpr int FW_MAX_COLS = 112;          // operand rows (terms x rows) of a call
-constexpr int FW_MAX_QROWS = 16;          // query rows of one KV head and sequence
+constexpr int FW_MAX_ROWS = 72;           // rows of a call
+constexpr int FW_MAX_COLS = 144;          // operand rows (terms x rows) of a call
+constexpr int FW_QROWS = 16;              // query rows of one KV head and sequence that an attention item takes at most,
+constexpr int FW_QROWS_WIDE = 40;         // or in the wide variant: more are cut into blocks of equal size
 
 // Tile geometry of one projection.  A step brings nbox boxes of hr weight rows x kb k-blocks (one copy each) and one box of
 // operand rows.  nbox = 1: the rows of h features (QKV: of h rotary pairs of a head, hr = 2 h); nbox = 2: h gate rows and
@@ -18,16 +19,17 @@ constexpr int FW_MAX_QROWS = 16;          // query rows of one KV head and seque
 // the call's operand rows, so that the weight maps are encoded once per model: kb is the most that a ring slot holds.
 // Big boxes matter twice: a thread issues a copy about every quarter of a microsecond whatever its size, and rows of 256
 // bytes and more pass at 70 GB/s per SM where rows of 128 bytes pass at 43.
-constexpr int FW_CLASSES = 5;
+constexpr int FW_CLASSES = 6;
 struct FwClass { int cols, slots; };      // operand rows up to, ring slots
-constexpr FwClass FW_CLASS[FW_CLASSES] = {{16, 4}, {32, 4}, {64, 3}, {80, 3}, {FW_MAX_COLS, 3}};
+constexpr FwClass FW_CLASS[FW_CLASSES] = {{16, 4}, {32, 4}, {64, 3}, {80, 3}, {112, 3}, {FW_MAX_COLS, 3}};
 struct FwPhase {
     int h, hr, nbox, n_tiles, u;          // u: tiles per head (QKV)
     int c;                                // O, down: blocks that share a tile's k-range (their partial sums meet in global memory)
     int kb, flat, S, steps;               // k-blocks of a box, its map's view, k-blocks side by side in the MMA, steps of all k-blocks
     int box_bytes, b_off;                 // bytes of one weight box, offset of the operand rows in the slot
     int k_blocks, K;
-    int dual, blk;                        // two accumulators for one box; rows that the epilogue takes at a time
+    int dual, both, blk;                  // two accumulators for one box; a tile takes both accumulator buffers; rows that the
+                                          // epilogue takes at a time
 };
 enum { FW_QKV = 0, FW_ATTN = 1, FW_O = 2, FW_GATEUP = 3, FW_DOWN = 4, FW_LM = 5 };
 
@@ -43,11 +45,12 @@ struct FwArgs {
     const FwLayer* layers;
     int n_layers, n_cta;
     int T, terms, cols, B, R, d, F, V, Hq, Hkv, hd, max_batch, lm_plain;
+    int nqb, qrows;                       // wide attention: blocks that a sequence's query rows of a KV head are cut into, rows of a block
     int pieces;                           // stride of the attention partials: pieces per (row, head)
     int parts0;                           // statistics of the prepared rows: parts of sumsq_a
     long long cap;
     float inv_dim, eps;
-    int32_t *sync, *acnt;                 // phase counters, arrival counters of the attention's (sequence, KV head) pairs
+    int32_t *sync, *acnt;                 // phase counters, arrival counters of the attention's (sequence, KV head, query block)s
     int32_t* kcnt;                        // arrivals at the split tiles of O, then of down
     float* kpart;                         // their partial sums [block][row][feature]
     float *sumsq_a, *sumsq_b, *hidden;
@@ -69,9 +72,14 @@ struct FwArgs {
 void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta, int cls);
 bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta);
 size_t fw_parts_max(const mtad_model_desc& d, int n_cta, bool lm);
+// (sequence, KV head, query block)s of a call at most: B * ceil(G R / rows) with B R <= FW_MAX_ROWS
+inline size_t fw_pairs(const mtad_model_desc& d, int max_batch) {
+    const int G = d.n_q_heads / d.n_kv_heads;
+    return (size_t)d.n_kv_heads * ((G * FW_MAX_ROWS + FW_QROWS_WIDE - 1) / FW_QROWS_WIDE + max_batch);
+}
 // words of the phase and arrival counters (zeroed by the row preparation of every call)
-inline size_t fw_sync_words(int layers, int max_batch, int Hkv, int n_cta) {
-    return (size_t)5 * layers + 1 + (size_t)max_batch * Hkv + 2 * (size_t)n_cta;
+inline size_t fw_sync_words(const mtad_model_desc& d, int max_batch, int n_cta) {
+    return (size_t)5 * d.layers + 1 + fw_pairs(d, max_batch) + 2 * (size_t)n_cta;
 }
 cudaError_t launch_forward(const FwArgs& a, cudaStream_t st);
 
