@@ -169,7 +169,7 @@ template <int NR>
 struct alignas(16) FwAttn {
     float smx[2][NR][4];                  // row maxima of the four warps
     float sl[2][2][NR][4];                // row sums of the four warps, two segments
-    float sm[2][NR];                      // first scores of a segment
+    float sm[2][NR];                      // reference values
 };
 struct FwTail {
     SeqMeta meta[MTAD_MAX_BATCH];
@@ -182,6 +182,7 @@ struct FwTail {
     uint32_t tmem_ptr;
     int abort_flag[2];
     int last[2];
+    AttnPos apos[3];                      // attention items of this block: the lowest, the highest, the one it takes first
 };
 static_assert(offsetof(FwTail, attn) % 16 == 0 && offsetof(FwTail, full) % 8 == 0, "alignment of the tail");
 static_assert(FW_RING + FW_UNION + sizeof(FwTail) <= 227 * 1024, "shared memory of the forward");
@@ -205,7 +206,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
     const int yb = S * hr, ys = nbox * yb + 4;             // columns of Y that a box takes, row stride of Y
     const int nf = KIND == FW_LM ? nbox * f.h : f.h;       // features (pairs) of a tile
     const int nv = nf / V;                                 // items of a row
-    const int per = terms == 3 ? 5 : 8, blk = FEW ? 8 : f.blk;      // rows of a drain load, rows that Y holds at a time
+    const int per = terms == 3 ? 5 : 16, blk = FEW ? 8 : f.blk;      // rows of a drain load, rows that Y holds at a time
     // a lane's slice of the S k-blocks that the MMA takes side by side is tl / hr; a warp's lanes may lie in several
     const int tl = quad * 32 + lane, my = tl / hr;
     const int s0 = S > 1 ? quad * 32 / hr : 0, s1 = S > 1 ? min(S - 1, (quad * 32 + 31) / hr) : 0;
@@ -291,25 +292,36 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
             if (nbox == 2) b = half;                       // the two warps of a quadrant share out the boxes, or the row groups
             for (; rb < r1; rb += nbox == 1 ? 2 * per : per)
                 for (int sl = s0; sl <= s1; ++sl) {
-                    float v[16];
-                    tc_ld16(t_acc + (b * S + sl) * cols + rb * terms, v);
-                    if (f.dual) {
-                        float v2[16];
-                        tc_ld16(t_acc + (S + sl) * cols + rb * terms, v2);
+                    float* y = Y + (rb - r0) * ys + b * yb + tl;
+                    const bool here = my == sl && tl < yb;
+                    if (FEW || terms == 3) {
+                        float v[16];
+                        tc_ld16(t_acc + (b * S + sl) * cols + rb * 3, v);
+                        if (f.dual) {
+                            float v2[16];
+                            tc_ld16(t_acc + (S + sl) * cols + rb * 3, v2);
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) v[j] += v2[j];
-                    }
-                    if (my == sl && tl < yb) {
-                        float* y = Y + (rb - r0) * ys + b * yb + tl;
-                        if (FEW || terms == 3) {
+                            for (int j = 0; j < 16; ++j) v[j] += v2[j];
+                        }
+                        if (here)
 #pragma unroll
                             for (int j = 0; j < 5; ++j)
                                 if (rb + j < r1) y[j * ys] = v[3 * j] + (v[3 * j + 1] + v[3 * j + 2]);
-                        } else {
+                    } else {
+                        float v[32];
+                        tc_ld32(t_acc + (b * S + sl) * cols + rb * 2, v);
+                        if (f.dual)
 #pragma unroll
-                            for (int j = 0; j < 8; ++j)
+                            for (int h = 0; h < 32; h += 16) {
+                                float v2[16];
+                                tc_ld16(t_acc + (S + sl) * cols + rb * 2 + h, v2);
+#pragma unroll
+                                for (int j = 0; j < 16; ++j) v[h + j] += v2[j];
+                            }
+                        if (here)
+#pragma unroll
+                            for (int j = 0; j < 16; ++j)
                                 if (rb + j < r1) y[j * ys] = v[2 * j] + v[2 * j + 1];
-                        }
                     }
                     __syncwarp();
                 }
@@ -686,9 +698,14 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     // This block's items in the order it takes them: if its range holds more than one segment (run of tiles of one sequence
     // and KV head), the first segment comes last, because it ends with the tile that holds the call's own rows and cannot
     // be requested before the phase has been released.  a_wrap: where the order returns to the front of the range.
-    const AttnPos a_zero = attn_find(s.meta, a.B, heads, a_lo), a_last = attn_find(s.meta, a.B, heads, max(a_lo, a_lo + a_n - 1));
+    const AttnPos &a_zero = s.apos[0], &a_last = s.apos[1], &a_first = s.apos[2];
+    if (threadIdx.x == 0) {
+        s.apos[0] = attn_find(s.meta, a.B, heads, a_lo);
+        s.apos[1] = attn_find(s.meta, a.B, heads, max(a_lo, a_lo + a_n - 1));
+        s.apos[2] = attn_find(s.meta, a.B, heads, a_lo + (s.apos[0].nt - s.apos[0].tile < a_n ? s.apos[0].nt - s.apos[0].tile : 0));
+    }
+    __syncthreads();
     const int a_rot = a_zero.nt - a_zero.tile < a_n ? a_zero.nt - a_zero.tile : 0, a_wrap = a_n - a_rot;
-    const AttnPos a_first = a_rot ? attn_find(s.meta, a.B, heads, a_lo + a_rot) : a_zero;
     auto attn_step = [&](AttnPos& it, int next) {          // item `next` of the order, from the one before
         if (next == a_wrap) it = a_zero;
         else attn_next(it, s.meta, a.B, heads);
@@ -1007,6 +1024,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     }
                 }
                 AttnPos it = a_first;
+                // (The reference values lie in shared memory too: wide, they would not fit the registers beside the rest.)
                 float m[NR], l[NR], acc[NR];
                 // output of the tile before: this thread's head dimension of its rows, out of tensor memory
                 auto output = [&](int tile_no) {
@@ -1046,7 +1064,8 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                                     const size_t o = ((size_t)t * a.Hq + h) * a.pieces + piece;
                                     a.part[o * HD + kl] = acc[x];
                                     if (kl == 0)
-                                        reinterpret_cast<float2*>(a.part + (size_t)T * a.Hq * a.pieces * HD)[o] = make_float2(m[x], ls);
+                                        reinterpret_cast<float2*>(a.part + (size_t)T * a.Hq * a.pieces * HD)[o] =
+                                            make_float2(WIDE ? sa.sm[half][x] : m[x], ls);
                                 }
                             }
                         }
@@ -1059,14 +1078,14 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     }
                     ++as;
                 };
-                AttnPos prev = it;
                 for (int i = 0; i < a_n; ++i) {
-                    const bool fresh = i == 0 || i == a_wrap || it.tile == 0;
+                    const bool fresh = i == 0 || i == a_wrap || it.tile + 1 == it.nt;     // (it: the item before)
+                    if (fresh && i > 0) {
+                        output(at - 1);
+                        finish(it);
+                    }
+                    if (i > 0) attn_step(it, i);
                     if (fresh) {
-                        if (i > 0) {
-                            output(at - 1);
-                            finish(prev);
-                        }
 #pragma unroll
                         for (int x = 0; x < NR; ++x) { m[x] = -CUDART_INF_F; l[x] = 0.f; acc[x] = 0.f; }
                     }
@@ -1084,7 +1103,16 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     if ((it.tile + 1) * FW_KEYS > L) {
                         const int sr = j - L;
                         vis = j < nkeys ? 0xffffffffu : 0u;
-                        if (sr >= 0 && vis) {
+                        if (WIDE && sr >= 0 && vis) {
+                            const uint32_t* words = a.rm.mask + (size_t)t0 * MTAD_MASK_WORDS + (sr >> 5);
+                            int r = row_of(0), rr = (rb + min(r, n_q - 1)) % nrows;
+                            vis = 0;
+#pragma unroll
+                            for (int x = 0; x < NR; ++x) {
+                                vis |= ((words[rr * MTAD_MASK_WORDS] >> (sr & 31)) & 1u) << x;
+                                if (++r < n_q && ++rr == nrows) rr = 0;
+                            }
+                        } else if (sr >= 0 && vis) {
                             vis = 0;
 #pragma unroll
                             for (int x = 0; x < NR; ++x) {
@@ -1108,17 +1136,16 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
 #pragma unroll
                             for (int x = 0; x < NR; ++x) sa.sm[half][x] = v[x];
                         bar_n(2 + half, 128);
+                    }
+                    if (WIDE || fresh)
 #pragma unroll
                         for (int x = 0; x < NR; ++x) m[x] = sa.sm[half][x];
-                    }
                     bool calm = true;
 #pragma unroll
                     for (int x = 0; x < NR; ++x) calm = calm && v[x] <= m[x] + FW_LAZY && m[x] > -CUDART_INF_F;
-                    float f[NR];
-#pragma unroll
-                    for (int x = 0; x < NR; ++x) f[x] = 1.f;
                     const bool quiet = all_of(2 + half, 128, calm);
                     if (!quiet) {
+                        if (!fresh) output(at - 1);                   // (before the reference moves)
                         float wm[NR];
 #pragma unroll
                         for (int x = 0; x < NR; ++x) wm[x] = v[x];
@@ -1134,10 +1161,14 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         for (int x = 0; x < NR; ++x) {
                             const float4 q4 = *reinterpret_cast<const float4*>(sa.smx[half][x]);
                             const float mn = fmaxf(m[x], fmaxf(fmaxf(q4.x, q4.y), fmaxf(q4.z, q4.w)));
-                            f[x] = mn == -CUDART_INF_F ? 1.f : exp2f(m[x] - mn);
+                            const float f = mn == -CUDART_INF_F ? 1.f : exp2f(m[x] - mn);
                             m[x] = mn;
-                            l[x] *= f[x];
+                            l[x] *= f;
+                            acc[x] *= f;
                         }
+                        if (WIDE && kl == 0)
+#pragma unroll
+                            for (int x = 0; x < NR; ++x) sa.sm[half][x] = m[x];
                         bar_n(2 + half, 128);                         // (smx is free again)
                     }
                     uint8_t* pt = (WIDE ? smem + (size_t)((pos + 2 * i + 1) % NS) * FW_SLOT + KV_BYTES : Ps + b * P_BYTES) +
@@ -1165,7 +1196,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         }
                     }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    if (!fresh) output(at - 1);                       // (tile i - 1 of the same segment, while this one's output is formed)
+                    if (quiet && !fresh) output(at - 1);              // (tile i - 1 of the same segment, while this one's output is formed)
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&s.pfull[b]));
@@ -1174,16 +1205,11 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         q_ready((as + 1) & 1);
                         next_seg();
                     }
-                    if (!quiet)
-#pragma unroll
-                        for (int x = 0; x < NR; ++x) acc[x] *= f[x];
                     ++at;
-                    prev = it;
-                    if (i + 1 < a_n) attn_step(it, i + 1);
                 }
                 if (a_n > 0) {
                     output(at - 1);
-                    finish(prev);
+                    finish(it);
                 }
                 pos += 2 * a_n + ring_other;
                 ok = all_of(1, FW_EPI, ok);
@@ -1331,7 +1357,7 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
         if ((k == FW_O || k == FW_DOWN) && (f.n_tiles > n_cta || f.steps < f.c)) return false;
         // one box: the MMAs along k alternate between two accumulators where they fit and every block has two
         f.dual = f.nbox == 1 && 2 * f.S * a.cols <= FW_ACC && f.steps / f.c * (f.kb / f.S) >= 2 ? 1 : 0;
-        const int per = a.terms == 3 ? 5 : 8;              // rows of one drain load
+        const int per = a.terms == 3 ? 5 : 16;             // rows of one drain load
         const int fit = FW_UNION / (per * (f.nbox * f.S * f.hr + 4) * 4);
         if (fit < 1) return false;
         f.blk = std::min(up_div(T, per), fit) * per;
