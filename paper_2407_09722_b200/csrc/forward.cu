@@ -577,16 +577,49 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
     return true;
 }
 
-// Merge of a (sequence, KV head)'s pieces by the epilogue threads of the block that arrived last: four output elements a
+__device__ __forceinline__ float exp2_ftz(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// Sums over the 32 lanes of N values in about 2 N instructions instead of 10 N: at each step a lane passes on half of its
+// values and keeps the other half.  Leaves one sum in v[0] and returns which (N: none; several lanes may hold the same).
+template <int N>
+__device__ __forceinline__ int lane_sums(float* v, int lane) {
+    int n = N, idx = 0, have = N;
+#pragma unroll
+    for (int bit = 16; bit > 0; bit >>= 1) {
+        if (n > 1) {
+            const int h = (n + 1) / 2;                     // the lanes with this bit keep the upper half of the values
+            const bool up = lane & bit;
+#pragma unroll
+            for (int k = 0; k < (N + 1) / 2; ++k)
+                if (k < h) {
+                    const float hiv = h + k < n ? v[h + k] : 0.f;
+                    const float mine = up ? hiv : v[k], other = up ? v[k] : hiv;
+                    v[k] = mine + __shfl_xor_sync(0xffffffffu, other, bit);
+                }
+            idx += up ? h : 0;
+            have = up ? have - h : min(have, h);
+            n = h;
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], bit);
+        }
+    }
+    return have > 0 ? idx : N;
+}
+
+// Merge of rows [ra, rn) of a (sequence, KV head, query block)'s pieces by the epilogue threads: four output elements a
 // thread, the pieces in order (deterministic) and six at a time, so that their loads are in flight together.
 template <int HD, int NQP>
-__device__ __forceinline__ void merge_pieces(const FwArgs& a, const FwTail& s, const AttnPos& q, int n_piece, int G, int e) {
+__device__ __forceinline__ void merge_pieces(const FwArgs& a, const FwTail& s, const AttnPos& q, int n_piece, int G, int e, int kp) {
     const int nqb = NQP > FW_QROWS ? a.nqb : 1, g = q.g / nqb, r0 = (q.g - g * nqb) * a.qrows;
-    const int nrows = s.meta[q.bi].nrows, n_q = min(G * nrows - r0, a.qrows);
-    for (int i = e; i < n_q * (HD / 4); i += FW_EPI) {
+    const int nrows = s.meta[q.bi].nrows, n_q = max(0, min(G * nrows - r0, a.qrows));
+    const int ra = kp < 0 ? 0 : n_q * kp / n_piece, rn = kp < 0 ? n_q : n_q * (kp + 1) / n_piece;
+    for (int i = ra * (HD / 4) + e; i < rn * (HD / 4); i += FW_EPI) {
         const int r = r0 + i / (HD / 4), c4 = i % (HD / 4);
         const int hq = G == 1 ? 0 : r / nrows, t = q.bi * a.R + r - hq * nrows, h = g * G + hq;
-        const size_t o = ((size_t)t * a.Hq + h) * a.pieces;
+        const size_t o = ((size_t)(q.bi * a.Hkv + g) * G * a.R + r) * a.pieces;
         const float2* ml = reinterpret_cast<const float2*>(a.part + (size_t)a.T * a.Hq * a.pieces * HD) + o;
         const float4* po = reinterpret_cast<const float4*>(a.part + o * HD) + c4;
         constexpr int NP = 6;
@@ -623,7 +656,6 @@ __device__ __forceinline__ void merge_pieces(const FwArgs& a, const FwTail& s, c
         store_terms4(make_float4(o4.x * f, o4.y * f, o4.z * f, o4.w * f),
                      a.x_a + (size_t)t * a.terms * a.Hq * HD + (size_t)h * HD + c4 * 4, (size_t)a.Hq * HD, a.terms);
     }
-    if (e == 0) a.acnt[q.bi * a.Hkv * nqb + q.g] = 0; // ready for the next layer
 }
 
 template <int HD, int NQP, bool FEW, int NS>
@@ -1039,34 +1071,41 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 // end of a segment: the rows' sums over the lanes, then the rows leave - final, or as a piece
                 auto finish = [&](const AttnPos& q) {
                     const int sb = as & 1;
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                        for (int x = 0; x < NR; ++x) l[x] += __shfl_xor_sync(0xffffffffu, l[x], o);
-#pragma unroll
-                    for (int x = 0; x < NR; ++x)
-                        if (lane == x) sa.sl[sb][half][x][quad] = l[x];
+                    const int which = lane_sums<NR>(l, lane);
+                    if (which < NR) sa.sl[sb][half][which][quad] = l[0];
                     ok = all_of(2 + half, 128, ok);
                     const int nrows = s.meta[q.bi].nrows, n_q = q_count(q), rb = q_base(q), g = q_head(q);
                     const int first = q.f0 / a_per, n_piece = (q.f0 + q.nt - 1) / a_per - first + 1, piece = cta - first;
-                    if (ok && (HD == 128 || kl < HD)) {
+                    auto row_sum = [&](int x) {
+                        const float4 l4 = *reinterpret_cast<const float4*>(sa.sl[sb][half][x]);
+                        return (l4.x + l4.y) + (l4.z + l4.w);
+                    };
+                    // (code that runs once a phase costs its instructions' way from L2: keep the loops over rows short)
+                    if (ok && n_piece > 1) {
+                        const size_t o = ((size_t)(q.bi * a.Hkv + g) * G * a.R + rb + row_of(0)) * a.pieces + piece;
+                        constexpr int DR = WIDE ? 1 : 2;
+                        float* po = a.part + o * HD + kl;
+                        const int left = n_q - row_of(0);
+                        if (HD == 128 || kl < HD)
+#pragma unroll
+                            for (int x = 0; x < NR; ++x, po += DR * a.pieces * HD)
+                                if (DR * x < left) *po = acc[x];
+                        float2* ml = reinterpret_cast<float2*>(a.part + (size_t)T * a.Hq * a.pieces * HD) + o;
+                        if (WIDE) {
+                            if (kl < NR && kl < left) ml[kl * a.pieces] = make_float2(sa.sm[half][kl], row_sum(kl));
+                        } else if (kl == 0) {
+#pragma unroll
+                            for (int x = 0; x < NR; ++x)
+                                if (DR * x < left) ml[DR * x * a.pieces] = make_float2(m[x], row_sum(x));
+                        }
+                    } else if (ok && (HD == 128 || kl < HD)) {
 #pragma unroll
                         for (int x = 0; x < NR; ++x) {
                             const int r = row_of(x);
                             if (r < n_q) {
                                 const int hq = G == 1 ? 0 : (rb + r) / nrows, t = q.bi * a.R + rb + r - hq * nrows, h = g * G + hq;
-                                const float4 l4 = *reinterpret_cast<const float4*>(sa.sl[sb][half][x]);
-                                const float ls = (l4.x + l4.y) + (l4.z + l4.w);
-                                if (n_piece == 1) {
-                                    store_terms(acc[x] / ls, a.x_a + (size_t)t * terms * a.Hq * HD + (size_t)h * HD + kl,
-                                                (size_t)a.Hq * HD, terms);
-                                } else {
-                                    const size_t o = ((size_t)t * a.Hq + h) * a.pieces + piece;
-                                    a.part[o * HD + kl] = acc[x];
-                                    if (kl == 0)
-                                        reinterpret_cast<float2*>(a.part + (size_t)T * a.Hq * a.pieces * HD)[o] =
-                                            make_float2(WIDE ? sa.sm[half][x] : m[x], ls);
-                                }
+                                store_terms(acc[x] / row_sum(x), a.x_a + (size_t)t * terms * a.Hq * HD + (size_t)h * HD + kl,
+                                            (size_t)a.Hq * HD, terms);
                             }
                         }
                     }
@@ -1078,6 +1117,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     }
                     ++as;
                 };
+                int L = 0, nkeys = 0;
                 for (int i = 0; i < a_n; ++i) {
                     const bool fresh = i == 0 || i == a_wrap || it.tile + 1 == it.nt;     // (it: the item before)
                     if (fresh && i > 0) {
@@ -1089,10 +1129,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
 #pragma unroll
                         for (int x = 0; x < NR; ++x) { m[x] = -CUDART_INF_F; l[x] = 0.f; acc[x] = 0.f; }
                     }
-                    const SeqMeta sm = s.meta[it.bi];
-                    const int nrows = sm.nrows, L = sm.L, nkeys = sm.nkeys;
-                    const int n_q = q_count(it), rb = q_base(it);
-                    const int t0 = it.bi * a.R;                       // query row r: row t0 + r % nrows, head g * G + r / nrows
+                    if (fresh) { L = s.meta[it.bi].L; nkeys = s.meta[it.bi].nkeys; }
                     const bool turn = WIDE && i + 1 < a_n && (i + 1 == a_wrap || it.tile + 1 == it.nt);     // the segment's last
                     const int b = at & 1;
                     const uint32_t par = (uint32_t)(at >> 1) & 1u;
@@ -1101,7 +1138,8 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     // their ancestors and themselves; none past the last key
                     uint32_t vis = 0xffffffffu;
                     if ((it.tile + 1) * FW_KEYS > L) {
-                        const int sr = j - L;
+                        const int sr = j - L, nrows = s.meta[it.bi].nrows, n_q = q_count(it), rb = q_base(it);
+                        const int t0 = it.bi * a.R;                   // query row r: row t0 + r % nrows, head g * G + r / nrows
                         vis = j < nkeys ? 0xffffffffu : 0u;
                         if (WIDE && sr >= 0 && vis) {
                             const uint32_t* words = a.rm.mask + (size_t)t0 * MTAD_MASK_WORDS + (sr >> 5);
@@ -1177,7 +1215,8 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     const int pc = (kl & 63) >> 3;
 #pragma unroll
                     for (int x = 0; x < NR; ++x) {
-                        const float pv = exp2f(v[x] - (m[x] == -CUDART_INF_F ? 0.f : m[x]));        // exp2(-inf) = 0
+                        // (exp2(-inf) = 0; results below 2^-126 of a sum of at least 1, the reference being a key's score, go to 0)
+                        const float pv = exp2_ftz(v[x] - (m[x] == -CUDART_INF_F ? 0.f : m[x]));
                         l[x] += pv;
                         const __nv_bfloat16 hi = __float2bfloat16_rn(pv);
                         uint8_t* d = pt + ((pc ^ (row_of(x) & 7)) << 4) + x * RS;
@@ -1215,6 +1254,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 ok = all_of(1, FW_EPI, ok);
                 if (!ok) break;
                 // pieces shared with other blocks (at most the first and the last of this block's range): who arrives last merges
+                // them; with many rows the blocks wait for one another and take a share of the rows each
                 if (a_n > 0) {
                     if (e < 2) {
                         const AttnPos q = e == 0 ? a_zero : a_last;
@@ -1224,13 +1264,19 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             int old;
                             asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;"
                                          : "=r"(old) : "l"(a.acnt + q.bi * heads + q.g) : "memory");
-                            last = old + 1 == n_piece ? n_piece : 0;
+                            last = WIDE || old + 1 == n_piece * (layer + 1) ? n_piece : 0;
                         }
                         s.last[e] = last;
+                        __syncwarp(3u);
+                        if (WIDE && last) ok = grid_wait(a.acnt + q.bi * heads + q.g, n_piece * (layer + 1), abort_flag);
                     }
-                    bar_n(1, FW_EPI);
+                    ok = all_of(1, FW_EPI, ok);
+                    if (!ok) break;
                     for (int x = 0; x < 2; ++x)
-                        if (s.last[x]) merge_pieces<HD, NQP>(a, s, x == 0 ? a_zero : a_last, s.last[x], G, e);
+                        if (s.last[x]) {
+                            const AttnPos q = x == 0 ? a_zero : a_last;
+                            merge_pieces<HD, NQP>(a, s, q, s.last[x], G, e, WIDE ? cta - q.f0 / a_per : -1);
+                        }
                 }
             } else if (kind == FW_QKV) {
                 ok = epi_phase<FW_QKV, HD, FEW>(a, s, Y, p, layer, tcount, e, t_lane, cta);
