@@ -47,10 +47,6 @@ constexpr int FW_EPI = 256;
 constexpr int FW_UNION = 32 * 1024;       // epilogue tile Y, or the attention's query and probability tiles
 constexpr int FW_ACC = 240;               // accumulator columns of a tile, of 256 (the drain reads up to 15 columns further),
 constexpr int FW_ACC_ONE = 496;           // or of 512 where a tile takes both buffers
-#ifndef FW_REHEARSE
-#define FW_REHEARSE 1
-#endif
-constexpr bool REHEARSE = FW_REHEARSE;
 constexpr float FW_LAZY = 64.f;           // log2 of how far a score may exceed its row's reference value
 
 __device__ __forceinline__ bool grid_wait(const int* c, int want, volatile int* abort_flag) {
@@ -74,54 +70,16 @@ __device__ __forceinline__ uint2 pack4(float x, float y, float z, float w) {
     const __nv_bfloat162 p = __floats2bfloat162_rn(x, y), q = __floats2bfloat162_rn(z, w);
     return make_uint2(*reinterpret_cast<const uint32_t*>(&p), *reinterpret_cast<const uint32_t*>(&q));
 }
-// Stores that happen only if `on`, without a branch: what they store is computed either way (see the rehearsal below)
-__device__ __forceinline__ void put(bool on, __nv_bfloat16* p, __nv_bfloat16 v) {
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.global.b16 [%0], %1;\n\t}" ::"l"(p),
-                 "h"(__bfloat16_as_ushort(v)), "r"(on ? 1u : 0u) : "memory");
+__device__ __forceinline__ void store_bf4(const float* v, __nv_bfloat16* d) {
+    *reinterpret_cast<uint2*>(d) = pack4(v[0], v[1], v[2], v[3]);
 }
-__device__ __forceinline__ void put(bool on, float* p, float v) {
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.global.f32 [%0], %1;\n\t}" ::"l"(p), "f"(v),
-                 "r"(on ? 1u : 0u) : "memory");
-}
-__device__ __forceinline__ void put(bool on, __nv_bfloat16* p, uint2 v) {
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t@q st.global.v2.b32 [%0], {%1, %2};\n\t}" ::"l"(p), "r"(v.x),
-                 "r"(v.y), "r"(on ? 1u : 0u) : "memory");
-}
-__device__ __forceinline__ void put(bool on, void* p, float4 v) {
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %5, 0;\n\t@q st.global.v4.f32 [%0], {%1, %2, %3, %4};\n\t}" ::"l"(p),
-                 "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(on ? 1u : 0u) : "memory");
-}
-__device__ __forceinline__ void put_bf4(bool on, const float* v, __nv_bfloat16* d) { put(on, d, pack4(v[0], v[1], v[2], v[3])); }
-// one value, or four times `scale`, as bf16 hi and lo parts
-__device__ __forceinline__ void put_split(bool on, float y, __nv_bfloat16* hi, __nv_bfloat16* lo) {
-    const __nv_bfloat16 h = __float2bfloat16_rn(y);
-    put(on, hi, h);
-    put(on, lo, __float2bfloat16_rn(y - __bfloat162float(h)));
-}
-__device__ __forceinline__ void put_split4(bool on, const float* v, float scale, __nv_bfloat16* hi, __nv_bfloat16* lo) {
+// four values times `scale` as bf16 hi and lo parts
+__device__ __forceinline__ void split_store4(const float* v, float scale, __nv_bfloat16* hi, __nv_bfloat16* lo) {
     const float x = v[0] * scale, y = v[1] * scale, z = v[2] * scale, w = v[3] * scale;
     const uint2 h = pack4(x, y, z, w);
-    put(on, hi, h);
-    put(on, lo, pack4(x - __uint_as_float(h.x << 16), y - __uint_as_float(h.x & 0xffff0000u),
-                      z - __uint_as_float(h.y << 16), w - __uint_as_float(h.y & 0xffff0000u)));
-}
-// store_terms and store_terms4
-__device__ __forceinline__ void put_terms(bool on, float y, __nv_bfloat16* x, size_t K, int terms) {
-    const __nv_bfloat16 h = __float2bfloat16_rn(y);
-    put(on, x, h);
-    const float r = y - __bfloat162float(h);
-    const __nv_bfloat16 l = __float2bfloat16_rn(r);
-    put(on, x + K, l);
-    put(on && terms == 3, x + 2 * K, __float2bfloat16_rn(r - __bfloat162float(l)));
-}
-__device__ __forceinline__ void put_terms4(bool on, float4 v, __nv_bfloat16* x, size_t K, int terms) {
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        const uint2 w = pack4(v.x, v.y, v.z, v.w);
-        put(on && j < terms, x + (size_t)j * K, w);
-        v.x -= __uint_as_float(w.x << 16); v.y -= __uint_as_float(w.x & 0xffff0000u);
-        v.z -= __uint_as_float(w.y << 16); v.w -= __uint_as_float(w.y & 0xffff0000u);
-    }
+    *reinterpret_cast<uint2*>(hi) = h;
+    *reinterpret_cast<uint2*>(lo) = pack4(x - __uint_as_float(h.x << 16), y - __uint_as_float(h.x & 0xffff0000u),
+                                          z - __uint_as_float(h.y << 16), w - __uint_as_float(h.y & 0xffff0000u));
 }
 // barrier and consensus of `n` threads
 __device__ __forceinline__ bool all_of(int id, int n, bool ok) {
@@ -315,12 +273,6 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                 u8[i] = (t < T && jl < nf && n < a.V) ? a.uniforms[(size_t)(t / a.R) * a.V + n] : 0.5f;
             }
         };
-        // A rehearsal: the epilogue runs once while the accumulator is still being formed, on the buffer that lies idle and with
-        // its stores held back.  Its instructions come from L2 otherwise, at a few bytes a cycle, after the last MMA; this
-        // way they wait in the SM.
-#pragma unroll 1
-        for (int pass = REHEARSE && tile == cta && !f.both && !split ? 0 : 1; pass < 2; ++pass) {
-        const bool on = pass == 1;
         if (KIND == FW_QKV) rope_load(it0, ij0);
         if (FEW && (KIND == FW_O || KIND == FW_DOWN) && lane < nf && f0 + lane < a.d) {
             gain0 = __bfloat162float(gain[f0 + lane]);
@@ -328,15 +280,13 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
         }
         if (KIND == FW_LM && !a.lm_plain) lm_load(w);
         // (one thread polls: 256 of them would take the shared-memory pipe away from the copies' barriers)
-        if (on) {
-            if (e == 0) ok = mbar_wait(smem_u32(&s.tfull[buf]), (uint32_t)(tcount >> 1) & 1u, abort_flag);
-            ok = all_of(1, FW_EPI, ok);
-            if (!ok) return false;
-            tc_fence_after();
-        }
-        const uint32_t t_acc = tmem_lane + (f.both ? 0 : (on ? buf : buf ^ 1) * 256);
-        for (int r0 = 0; r0 < (on ? T : 1); r0 += blk) {
-            const int r1 = on ? min(T, r0 + blk) : min(T, min(8, blk)), nr = r1 - r0;
+        if (e == 0) ok = mbar_wait(smem_u32(&s.tfull[buf]), (uint32_t)(tcount >> 1) & 1u, abort_flag);
+        ok = all_of(1, FW_EPI, ok);
+        if (!ok) return false;
+        tc_fence_after();
+        const uint32_t t_acc = tmem_lane + (f.both ? 0 : buf * 256);
+        for (int r0 = 0; r0 < T; r0 += blk) {
+            const int r1 = min(T, r0 + blk), nr = r1 - r0;
             // ---- accumulators -> Y[row][box][lane], the terms of a row added up
             int b = 0, rb = r0 + (nbox == 1 ? half * per : 0);
             if (nbox == 2) b = half;                       // the two warps of a quadrant share out the boxes, or the row groups
@@ -375,7 +325,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                     }
                     __syncwarp();
                 }
-            if (on && r1 == T) {
+            if (r1 == T) {
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&s.tempty[buf]));
@@ -431,11 +381,11 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                                 // attention operands: q * log2(e) / sqrt(hd) as bf16 hi + lo
                                 const size_t o = ((size_t)tt * a.Hq + hg) * HD + jj;
                                 if (V == 1) {
-                                    put_split(on, va[0] * scale, a.q_hi + o, a.q_lo + o);
-                                    put_split(on, vb[0] * scale, a.q_hi + o + hp, a.q_lo + o + hp);
+                                    split_store(va[0] * scale, a.q_hi + o, a.q_lo + o);
+                                    split_store(vb[0] * scale, a.q_hi + o + hp, a.q_lo + o + hp);
                                 } else {
-                                    put_split4(on, va, scale, a.q_hi + o, a.q_lo + o);
-                                    put_split4(on, vb, scale, a.q_hi + o + hp, a.q_lo + o + hp);
+                                    split_store4(va, scale, a.q_hi + o, a.q_lo + o);
+                                    split_store4(vb, scale, a.q_hi + o + hp, a.q_lo + o + hp);
                                 }
                             } else {
                                 const int sq = s.meta[s.rowb[tt]].seq, kv = rot ? 0 : 1;
@@ -443,11 +393,11 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                                     __nv_bfloat16* d = a.cache + idx_cache(layer, a.max_batch, sq, kv, a.Hkv, hg - a.Hq - kv * a.Hkv,
                                                                            a.cap, sl, HD) + jj;
                                     if (V == 1) {
-                                        put(on, d, __float2bfloat16_rn(va[0]));
-                                        put(on, d + hp, __float2bfloat16_rn(vb[0]));
+                                        d[0] = __float2bfloat16_rn(va[0]);
+                                        d[hp] = __float2bfloat16_rn(vb[0]);
                                     } else {
-                                        put_bf4(on, va, d);
-                                        put_bf4(on, vb, d + hp);
+                                        store_bf4(va, d);
+                                        store_bf4(vb, d + hp);
                                     }
                                 }
                             }
@@ -471,8 +421,8 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                             g[x] = gx / (1.f + expf(-gx)) * (u[x] * rs);
                         }
                         __nv_bfloat16* o = a.x_f + (size_t)(r0 + t) * terms * a.F + n;
-                        if (V == 1) put_terms(on, g[0], o, a.F, terms);
-                        else put_terms4(on, make_float4(g[0], g[1 % V], g[2 % V], g[3 % V]), o, a.F, terms);
+                        if (V == 1) store_terms(g[0], o, a.F, terms);
+                        else store_terms4(make_float4(g[0], g[1 % V], g[2 % V], g[3 % V]), o, a.F, terms);
                     }
                     t += dt; j += dj;
                     if (j >= nf) { j -= nf; ++t; }
@@ -488,11 +438,11 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                         const float rs = s.rstd[r0 + t];
                         float* o = a.logits + (size_t)(r0 + t) * a.V + n;
                         if (V == 4 && (a.V & 3) == 0) {
-                            if (n < a.V) put(on, o, make_float4(z[0] * rs, z[1 % V] * rs, z[2 % V] * rs, z[3 % V] * rs));
+                            if (n < a.V) *reinterpret_cast<float4*>(o) = make_float4(z[0] * rs, z[1 % V] * rs, z[2 % V] * rs, z[3 % V] * rs);
                         } else {
 #pragma unroll
                             for (int x = 0; x < V; ++x)
-                                if (n + x < a.V) put(on, o + x, z[x] * rs);
+                                if (n + x < a.V) o[x] = z[x] * rs;
                         }
                         t += dt; j += dj;
                         if (j >= nf) { j -= nf; ++t; }
@@ -524,31 +474,31 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                         for (int i = 0; i < 8; ++i) sum += z[i] == -CUDART_INF_F ? 0.f : expf(z[i] - m);
 #pragma unroll
                         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-                        if (lane == 0) put(on, a.lm_part + idx_lm_part(t, f.n_tiles, tile), make_float4(m, sum, bv, __int_as_float(bi)));
+                        if (lane == 0) a.lm_part[idx_lm_part(t, f.n_tiles, tile)] = make_float4(m, sum, bv, __int_as_float(bi));
                     }
                     // logit of each node's token under its parent row, where it falls into this tile
                     for (int t = e; t < T; t += FW_EPI) {
                         const int pr = a.rm.prow[t];
                         if (pr < r0 || pr >= r1) continue;
                         const int tk = a.rm.tok[t] - f0, q = tk >= f.h ? 1 : 0;
-                        if (tk >= 0 && tk < nf) put(on, a.node_z + t, yv1(pr - r0, q, tk - q * f.h) * s.rstd[pr]);
+                        if (tk >= 0 && tk < nf) a.node_z[t] = yv1(pr - r0, q, tk - q * f.h) * s.rstd[pr];
                     }
                 }
             } else if (FEW) {
                 // residual, a warp per row: emits the next operand rows and the row's share of its sum of squares
                 if (w < T) {
-                    float ss = 0.f, h = hid, g = gain0;
+                    float ss = 0.f;
                     for (int jl = lane; jl < nf && f0 + jl < a.d; jl += 32) {
                         const int n = f0 + jl;
-                        if (jl != lane) { h = __ldcg(a.hidden + (size_t)w * a.d + n); g = __bfloat162float(gain[n]); }
-                        const float y = yv1(w, 0, jl) + h;
-                        put(on, a.hidden + (size_t)w * a.d + n, y);
-                        put_terms(on, y * g, a.x_d + (size_t)w * 3 * a.d + n, a.d, 3);
+                        if (jl != lane) { hid = __ldcg(a.hidden + (size_t)w * a.d + n); gain0 = __bfloat162float(gain[n]); }
+                        const float y = yv1(w, 0, jl) + hid;
+                        a.hidden[(size_t)w * a.d + n] = y;
+                        store_terms(y * gain0, a.x_d + (size_t)w * 3 * a.d + n, a.d, 3);
                         ss += y * y;
                     }
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-                    if (lane == 0) put(on, (KIND == FW_O ? a.sumsq_b : a.sumsq_a) + (size_t)tile * TC_X_ROWS + w, ss);
+                    if (lane == 0) (KIND == FW_O ? a.sumsq_b : a.sumsq_a)[(size_t)tile * TC_X_ROWS + w] = ss;
                 }
             } else {
                 // residual, four features per item; the items' sums of squares meet in Y (each over its own first element).
@@ -603,8 +553,8 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                             yv(t, 0, j, v);
                         }
                         y.x += v[0]; y.y += v[1 % V]; y.z += v[2 % V]; y.w += v[3 % V];
-                        put(on, hp, y);
-                        put_terms4(on, make_float4(y.x * g[0], y.y * g[1], y.z * g[2], y.w * g[3]),
+                        *hp = y;
+                        store_terms4(make_float4(y.x * g[0], y.y * g[1], y.z * g[2], y.w * g[3]),
                                      a.x_d + (size_t)(rb0 + t) * terms * a.d + n, a.d, terms);
                         ss = (y.x * y.x + y.y * y.y) + (y.z * y.z + y.w * y.w);
                     }
@@ -618,11 +568,10 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
                     if (lane == 0)
-                        put(on, (KIND == FW_O ? a.sumsq_b : a.sumsq_a) + (size_t)(split ? tile / f.c : tile) * TC_X_ROWS + rb0 + ra + tr, ss);
+                        (KIND == FW_O ? a.sumsq_b : a.sumsq_a)[(size_t)(split ? tile / f.c : tile) * TC_X_ROWS + rb0 + ra + tr] = ss;
                 }
             }
-            if (!on || r1 < T || tile + n_cta < f.n_tiles) bar_n(1, FW_EPI);       // Y is rewritten by the next rows or tile
-        }
+            if (r1 < T || tile + n_cta < f.n_tiles) bar_n(1, FW_EPI);       // Y is rewritten by the next rows or tile
         }
     }
     return true;
