@@ -1173,7 +1173,7 @@ void audit_forward(Audit& au, const mtad_ctx& c, const ModelView& m, int B, int 
         au.ws("attn_part", (size_t)T * Hq * pieces * (hd + 2));
         au.ws("fw_sync", fw_sync_words(d, m.max_batch, kCtas));
         for (const FwPhase* f : {&a.ph[FW_O], &a.ph[FW_DOWN]})
-            if (f->c > 1) au.ws("fw_part", (size_t)f->n_tiles * T * f->h);
+            if (f->c > 1) au.ws("fw_part", (size_t)f->n_tiles * T * f->S * f->hr);
         au.ws(&m == &c.target ? "fw_target" : "fw_aux", d.layers);
         if (lm_plain) au.ws("logits", (size_t)T * d.vocab);
         else au.ws("lm_part", idx_lm_part(T - 1, a.ph[FW_LM].n_tiles, a.ph[FW_LM].n_tiles - 1) + 1);

@@ -187,6 +187,115 @@ struct FwTail {
 static_assert(offsetof(FwTail, attn) % 16 == 0 && offsetof(FwTail, full) % 8 == 0, "alignment of the tail");
 static_assert(FW_RING + FW_UNION + sizeof(FwTail) <= 227 * 1024, "shared memory of the forward");
 
+// O or down where c blocks share the k-range of a tile: each leaves its accumulators in global memory as they lie in tensor
+// memory (a row's features, the S slices side by side), the blocks wait for one another, and each finishes a share of the
+// rows, a warp per row, adding the parts in order (deterministic).
+template <int KIND>
+__device__ __forceinline__ bool split_residual(const FwArgs& a, FwTail& s, const FwPhase& f, int layer, int tcount, int e,
+                                               uint32_t tmem_lane, int tile) {
+    volatile int* abort_flag = s.abort_flag;
+    const int lane = e & 31, w = e >> 5, quad = w & 3, half = w >> 2;
+    const int T = a.T, terms = a.terms, cols = a.cols, S = f.S, hr = f.hr, yb = S * hr, c = f.c;
+    const int tl = quad * 32 + lane, my = tl / hr, s0 = quad * 32 / hr, s1 = min(S - 1, (quad * 32 + 31) / hr);
+    const int per = terms == 3 ? 5 : 8, buf = tcount & 1;
+    const int kp = tile % c, ra = T * kp / c, rn = T * (kp + 1) / c, n = tile / c * hr + 4 * lane;
+    const bool in = 4 * lane < hr && n < a.d;
+    constexpr int RW = 3;                                  // rows of a warp whose loads are in flight together
+    float4 hid[RW];
+    auto load_hid = [&](int t0) {
+#pragma unroll
+        for (int x = 0; x < RW; ++x)
+            hid[x] = in && t0 + 8 * x < rn ? __ldcg(reinterpret_cast<const float4*>(a.hidden + (size_t)(t0 + 8 * x) * a.d + n))
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    load_hid(ra + w);
+    float g[4];
+    const __nv_bfloat16* gain = KIND == FW_O ? a.layers[layer].gain_ffn : a.layers[layer].gain_next;
+#pragma unroll
+    for (int x = 0; x < 4; ++x) g[x] = in ? __bfloat162float(gain[n + x]) : 0.f;
+    bool ok = true;
+    if (e == 0) ok = mbar_wait(smem_u32(&s.tfull[buf]), (uint32_t)(tcount >> 1) & 1u, abort_flag);
+    ok = all_of(1, FW_EPI, ok);
+    if (!ok) return false;
+    tc_fence_after();
+    const uint32_t t_acc = tmem_lane + (f.both ? 0 : buf * 256);
+    float* mine = a.kpart + (size_t)tile * T * yb + tl;
+    for (int rb = half * per; rb < T; rb += 2 * per)
+        for (int sl = s0; sl <= s1; ++sl) {
+            float v[16];
+            const uint32_t at = t_acc + sl * cols + rb * terms;
+            tc_ld16(at, v);
+            if (f.dual) {
+                float v2[16];
+                tc_ld16(at + S * cols, v2);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[j] += v2[j];
+            }
+            if (my == sl && tl < yb) {
+                float* y = mine + (size_t)rb * yb;
+                if (terms == 3) {
+#pragma unroll
+                    for (int j = 0; j < 5; ++j, y += yb)
+                        if (rb + j < T) __stcg(y, v[3 * j] + (v[3 * j + 1] + v[3 * j + 2]));
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j, y += yb)
+                        if (rb + j < T) __stcg(y, v[2 * j] + v[2 * j + 1]);
+                }
+            }
+            __syncwarp();
+        }
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(&s.tempty[buf]));
+    bar_n(1, FW_EPI);
+    if (e == 0) {
+        int32_t* cnt = a.kcnt + (KIND == FW_O ? 0 : a.n_cta) + tile / c;
+        asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(cnt) : "memory");
+        ok = grid_wait(cnt, c * (layer + 1), abort_flag);
+    }
+    ok = all_of(1, FW_EPI, ok);
+    if (!ok) return false;
+    const float* parts = a.kpart + (size_t)(tile / c * c) * T * yb + 4 * lane;
+    for (int t0 = ra + w; t0 < rn; t0 += 8 * RW) {
+        if (t0 != ra + w) load_hid(t0);
+        float4 q[RW];
+#pragma unroll
+        for (int x = 0; x < RW; ++x) q[x] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (in) {
+            const float* p = parts + (size_t)t0 * yb;
+            int sl = 0;
+#pragma unroll 4
+            for (int k = 0; k < c * S; ++k) {
+#pragma unroll
+                for (int x = 0; x < RW; ++x) {
+                    if (t0 + 8 * x >= rn) continue;
+                    const float4 z = __ldcg(reinterpret_cast<const float4*>(p + (size_t)(8 * x) * yb));
+                    q[x].x += z.x; q[x].y += z.y; q[x].z += z.z; q[x].w += z.w;
+                }
+                if (++sl == S) { sl = 0; p += (size_t)T * yb - (S - 1) * hr; }
+                else p += hr;
+            }
+        }
+#pragma unroll
+        for (int x = 0; x < RW; ++x) {
+            const int t = t0 + 8 * x;
+            if (t >= rn) continue;                         // (the whole warp)
+            float ss = 0.f;
+            if (in) {
+                const float4 y = make_float4(q[x].x + hid[x].x, q[x].y + hid[x].y, q[x].z + hid[x].z, q[x].w + hid[x].w);
+                *reinterpret_cast<float4*>(a.hidden + (size_t)t * a.d + n) = y;
+                store_terms4(make_float4(y.x * g[0], y.y * g[1], y.z * g[2], y.w * g[3]), a.x_d + (size_t)t * terms * a.d + n, a.d, terms);
+                ss = (y.x * y.x + y.y * y.y) + (y.z * y.z + y.w * y.w);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+            if (lane == 0) (KIND == FW_O ? a.sumsq_b : a.sumsq_a)[(size_t)(tile / c) * TC_X_ROWS + t] = ss;
+        }
+    }
+    return true;
+}
+
 // The epilogue group's part of one projection: row statistics, then per tile the accumulators -> Y in shared memory ->
 // the fused epilogue.  KIND is a template parameter so that the phase's geometry is read straight from the launch
 // parameters; index arithmetic and global loads stand ahead of the wait for the accumulator, because everything after it
@@ -240,9 +349,13 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
     const __nv_bfloat16* gain = nullptr;
     if (KIND == FW_O) gain = a.layers[layer].gain_ffn;
     if (KIND == FW_DOWN) gain = a.layers[layer].gain_next;
+    if (!FEW && (KIND == FW_O || KIND == FW_DOWN) && f.c > 1) {
+        ok = split_residual<KIND>(a, s, f, layer, tcount, e, tmem_lane, cta);
+        ++tcount;
+        return ok;
+    }
     for (int tile = cta; tile < f.n_tiles; tile += n_cta, ++tcount) {
-        const bool split = !FEW && (KIND == FW_O || KIND == FW_DOWN) && f.c > 1;
-        const int buf = tcount & 1, f0 = (split ? tile / f.c : tile) * nf;     // f0: first feature (O, down, gate / up, LM head)
+        const int buf = tcount & 1, f0 = tile * nf;        // f0: first feature (O, down, gate / up, LM head)
         // ---- what the first items need besides the accumulator
         const int hg = KIND == FW_QKV ? tile / f.u : 0, j0 = KIND == FW_QKV ? (tile - hg * f.u) * f.h : 0;
         constexpr int NI = FEW ? 2 : 1;                    // QKV: items per thread and round
@@ -501,74 +614,35 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                     if (lane == 0) (KIND == FW_O ? a.sumsq_b : a.sumsq_a)[(size_t)tile * TC_X_ROWS + w] = ss;
                 }
             } else {
-                // residual, four features per item; the items' sums of squares meet in Y (each over its own first element).
-                // A split tile: the blocks that share it leave their partial sums in global memory, wait for one another and
-                // finish a share of the rows each, adding the partial sums in block order (deterministic).
-                int t = it0, j = ij0, ra = 0, rn = nr;     // rows [ra, rn) of this block of rows are finished here
-                if (split) {
-                    float* mine = a.kpart + (size_t)tile * T * nf;
+                // residual, four features per item; the items' sums of squares meet in Y (each over its own first element)
+                int t = it0, j = ij0;
 #pragma unroll 2
-                    for (int i = e; i < nr * nv; i += FW_EPI) {
-                        float v[V];
-                        yv(t, 0, j, v);
-                        __stcg(reinterpret_cast<float4*>(mine + (size_t)(r0 + t) * nf + j), make_float4(v[0], v[1 % V], v[2 % V], v[3 % V]));
-                        t += dt; j += dj;
-                        if (j >= nf) { j -= nf; ++t; }
-                    }
-                    bar_n(1, FW_EPI);                      // (Y is free again; every partial sum of these rows is on its way)
-                    if (r1 < T) continue;
-                    if (e == 0) {
-                        int32_t* cnt = a.kcnt + (KIND == FW_O ? 0 : n_cta) + tile / f.c;
-                        asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(cnt) : "memory");
-                        ok = grid_wait(cnt, f.c * (layer + 1), abort_flag);
-                    }
-                    ok = all_of(1, FW_EPI, ok);
-                    if (!ok) return false;
-                    const int kp = tile % f.c;
-                    ra = T * kp / f.c;
-                    rn = T * (kp + 1) / f.c;
-                    t = ra + it0; j = ij0;
-                }
-                const int rb0 = split ? 0 : r0, ystr = split ? nf : ys;
-                const float* parts = a.kpart + (size_t)(split ? tile / f.c * f.c : 0) * T * nf;
-#pragma unroll 2
-                for (int i = e; i < (rn - ra) * nv; i += FW_EPI) {
+                for (int i = e; i < nr * nv; i += FW_EPI) {
                     const int n = f0 + j;
                     float ss = 0.f;
                     if (n < a.d) {
-                        float4* hp = reinterpret_cast<float4*>(a.hidden + (size_t)(rb0 + t) * a.d + n);
+                        float4* hp = reinterpret_cast<float4*>(a.hidden + (size_t)(r0 + t) * a.d + n);
                         float4 y = __ldcg(hp);
                         float g[4], v[V];
 #pragma unroll
                         for (int x = 0; x < 4; ++x) g[x] = __bfloat162float(gain[n + x]);
-                        if (split) {
-                            float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-                            for (int k = 0; k < f.c; ++k) {
-                                const float4 x = __ldcg(reinterpret_cast<const float4*>(parts + ((size_t)k * T + t) * nf + j));
-                                q.x += x.x; q.y += x.y; q.z += x.z; q.w += x.w;
-                            }
-                            v[0] = q.x; v[1 % V] = q.y; v[2 % V] = q.z; v[3 % V] = q.w;
-                        } else {
-                            yv(t, 0, j, v);
-                        }
+                        yv(t, 0, j, v);
                         y.x += v[0]; y.y += v[1 % V]; y.z += v[2 % V]; y.w += v[3 % V];
                         *hp = y;
                         store_terms4(make_float4(y.x * g[0], y.y * g[1], y.z * g[2], y.w * g[3]),
-                                     a.x_d + (size_t)(rb0 + t) * terms * a.d + n, a.d, terms);
+                                     a.x_d + (size_t)(r0 + t) * terms * a.d + n, a.d, terms);
                         ss = (y.x * y.x + y.y * y.y) + (y.z * y.z + y.w * y.w);
                     }
-                    Y[(t - ra) * ystr + j] = ss;
+                    Y[t * ys + j] = ss;
                     t += dt; j += dj;
                     if (j >= nf) { j -= nf; ++t; }
                 }
                 bar_n(1, FW_EPI);
-                for (int tr = w; tr < rn - ra; tr += 8) {
-                    float ss = lane < nv ? Y[tr * ystr + lane * V] : 0.f;       // (nv <= 32: at most 128 features)
+                for (int tr = w; tr < nr; tr += 8) {
+                    float ss = lane < nv ? Y[tr * ys + lane * V] : 0.f;       // (nv <= 32: at most 128 features)
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-                    if (lane == 0)
-                        (KIND == FW_O ? a.sumsq_b : a.sumsq_a)[(size_t)(split ? tile / f.c : tile) * TC_X_ROWS + rb0 + ra + tr] = ss;
+                    if (lane == 0) (KIND == FW_O ? a.sumsq_b : a.sumsq_a)[(size_t)tile * TC_X_ROWS + r0 + tr] = ss;
                 }
             }
             if (r1 < T || tile + n_cta < f.n_tiles) bar_n(1, FW_EPI);       // Y is rewritten by the next rows or tile
