@@ -46,6 +46,7 @@ struct ForwardPlan {
     int kv_terms = 0;
     bool maps = false;                 // tensor maps encoded (false: decomposition only, for the extent audit)
     bool one_launch = false;           // the whole forward is one launch (fw), g stays empty
+    bool fw_attn = false;              // the attention is the one-launch forward's, a launch of its own per layer (fw)
     FwArgs fw{};
     double fw_bytes = 0.0;
 };
@@ -430,6 +431,17 @@ bool build_forward_table(const ModelView& m, FwLayer* dev, CUtensorMap* lm) {
     return cudaMemcpy(dev, tab.data(), sizeof(FwLayer) * tab.size(), cudaMemcpyHostToDevice) == cudaSuccess;
 }
 
+bool mma_attention(const ModelView& m) {
+    return m.kv_map_ok && (m.d.head_dim == 64 || m.d.head_dim == 128);
+}
+
+// what the attention needs of the context
+void fw_common(FwArgs& a, const Scratch& sc, const RowMeta& rm, const ModelView& m) {
+    a.max_batch = m.max_batch; a.cap = m.d.kv_capacity; a.kv = m.kv_map;
+    a.sync = sc.fw_sync; a.acnt = sc.fw_sync + 5 * m.d.layers + 1;
+    a.x_a = sc.xa; a.q_hi = sc.q_hi; a.q_lo = sc.q_lo; a.rm = rm; a.part = sc.attn_part;
+}
+
 // The one-launch plan of a call of B x R rows: everything that the calls of this shape share.  `with_maps` as build_plan.
 bool build_forward_plan(ForwardPlan& fp, const Scratch& sc, const RowMeta& rm, const ModelView& m, const FwLayer* table,
                         const CUtensorMap* lm, int B, int R, bool lm_plain, bool with_maps) {
@@ -445,18 +457,16 @@ bool build_forward_plan(ForwardPlan& fp, const Scratch& sc, const RowMeta& rm, c
             if (tc_make_kb_map(&a.x[k], x, 2 * TC_X_ROWS, a.ph[k].K, a.cols, a.ph[k].kb)) return false;
         }
         a.lm = lm[a.cls];
-        a.kv = m.kv_map;
     }
     a.layers = table;
     a.lm_plain = lm_plain ? 1 : 0;
-    a.max_batch = m.max_batch; a.cap = d.kv_capacity;
+    fw_common(a, sc, rm, m);
     a.parts0 = 1; a.inv_dim = 1.f / (float)d.d_model; a.eps = d.rms_eps;
-    a.sync = sc.fw_sync; a.acnt = sc.fw_sync + 5 * d.layers + 1;
     a.kcnt = a.acnt + fw_pairs(d, m.max_batch); a.kpart = sc.fw_part;
     a.sumsq_a = sc.sumsq_a; a.sumsq_b = sc.sumsq_b; a.hidden = sc.hidden;
-    a.x_d = sc.xd; a.x_a = sc.xa; a.x_f = sc.xf; a.q_hi = sc.q_hi; a.q_lo = sc.q_lo;
+    a.x_d = sc.xd; a.x_f = sc.xf;
     a.cache = static_cast<__nv_bfloat16*>(d.kv_cache);
-    a.rope = sc.rope; a.rm = rm; a.part = sc.attn_part;
+    a.rope = sc.rope;
     a.lm_part = sc.lm_part; a.logits = sc.logits; a.node_z = sc.node_z;
     const double kvd = (double)d.n_kv_heads * d.head_dim;
     fp.fw_bytes = 2.0 * d.layers * ((double)d.d_model * (2.0 * qd + 2.0 * kvd + 3.0 * d.d_ffn)) + 2.0 * d.vocab * d.d_model;
@@ -466,9 +476,6 @@ bool build_forward_plan(ForwardPlan& fp, const Scratch& sc, const RowMeta& rm, c
     return true;
 }
 
-bool mma_attention(const ModelView& m) {
-    return m.kv_map_ok && (m.d.head_dim == 64 || m.d.head_dim == 128);
-}
 
 // K/V tiles of the tensor-core attention arrive by TMA: one map over the whole cache of a model
 void build_kv_map(ModelView& m) {
@@ -622,6 +629,9 @@ int build_plan(ForwardPlan& fp, const Scratch& sc, const RowMeta& rm, const Mode
     fp.maps = with_maps;
     fp.split_kv = split_kv;
     fp.kv_terms = tkv;
+    // The attention of many query rows per KV head: at 1032 rows of a KV head and 1024 keys (64 heads, 8 KV heads) FIGURES
+    fp.fw_attn = mma_attention(m) && fw_attn_plan(fp.fw, d, B, R, kCtas);
+    if (fp.fw_attn) fw_common(fp.fw, sc, rm, m);
     return MTAD_OK;
 }
 
@@ -681,7 +691,11 @@ int forward_rows_tc(mtad_ctx* ctx, const ModelView& m, const WeightMaps& wm, int
     for (size_t i = 0; i < fp.g.size(); ++i) {
         if (fp.g[i].attn_before) {                               // the O projection: the attention pass feeds it
             const int l = layer++;
-            if (mma_attention(m)) {
+            if (fp.fw_attn) {
+                fp.fw.status = status; fp.fw.wait_limit = ctx->wait_limit;
+                fp.fw.pieces = (int)((total + FW_KEYS - 1) / FW_KEYS);
+                RUN(MTAD_K_ATTN, 0, 1, launch_forward_attention(fp.fw, l, s));
+            } else if (mma_attention(m)) {
                 const AttnSplit as = attn_split(m, B, R, total);
                 RUN(MTAD_K_ATTN, 0, 2, launch_attention_mma(m, l, ctx->rm, sc, B, R, as.ns, as.nsp, status, pdl, s));
                 RUN(MTAD_K_ATTN, 0, 0, launch_attention_combine(m, ctx->rm, sc, B, R, as.ns, true, pdl, s));
@@ -1227,6 +1241,10 @@ void audit_forward(Audit& au, const mtad_ctx& c, const ModelView& m, int B, int 
     }
     // attention: split-KV partials of the last row, head and split; combined rows and the O projection's operand rows
     const long long total = std::min<long long>(len_ub, cap) + R;
+    if (fp.fw_attn) {
+        au.ws("attn_part", (size_t)T * Hq * ((total + FW_KEYS - 1) / FW_KEYS) * (hd + 2));
+        au.ws("fw_sync", fw_sync_words(d, m.max_batch, kCtas));
+    }
     const AttnSplit as = attn_split(m, B, R, total);
     au.ws("attn_part", idx_attn_part(T - 1, Hq, Hq - 1, as.ns, as.ns - 1, hd) + hd + 2);
     au.ws("attn", (size_t)T * qd);

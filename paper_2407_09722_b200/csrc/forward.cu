@@ -48,6 +48,7 @@ constexpr int FW_UNION = 32 * 1024;       // epilogue tile Y, or the attention's
 constexpr int FW_ACC = 240;               // accumulator columns of a tile, of 256 (the drain reads up to 15 columns further),
 constexpr int FW_ACC_ONE = 496;           // or of 512 where a tile takes both buffers
 constexpr float FW_LAZY = 64.f;           // log2 of how far a score may exceed its row's reference value
+constexpr float FW_UNSEEN = -1e30f;       // the reference value of a row that has seen no key
 
 __device__ __forceinline__ bool grid_wait(const int* c, int want, volatile int* abort_flag) {
     const uint32_t limit = (uint32_t)abort_flag[1];
@@ -765,7 +766,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         m.seq = __ldcg(a.rm.call_seq + b);
         s.meta[b] = m;
     }
-    for (int t = threadIdx.x; t < T; t += FW_THREADS) {
+    for (int t = threadIdx.x; t < min(T, FW_MAX_ROWS); t += FW_THREADS) {     // (more rows: the attention alone)
         s.slot[t] = __ldcg(a.rm.slot + t);
         s.rowb[t] = (uint8_t)(t / a.R);
     }
@@ -832,11 +833,11 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         if (lane == 0) {
             int pos = 0;
             bool ok = true;
-            for (int p = 0; p < n_phases && ok; ++p) {
+            for (int p = a.p_lo; p < a.p_hi && ok; ++p) {
                 const int kind = kind_of(p), layer = p / 5;
                 const FwLayer* L = a.layers + layer;
                 if (kind == FW_ATTN) {
-                    bool waited = false;
+                    bool waited = p == a.p_lo;
                     AttnPos it = a_first;
                     for (int i = 0; i < a_n && ok; attn_step(it, ++i)) {
                         const SeqMeta sm = s.meta[it.bi];
@@ -911,12 +912,12 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         if (lane == 0) {
             int pos = 0;
             bool ok = true;
-            for (int p = 0; p < n_phases && ok; ++p) {
+            for (int p = a.p_lo; p < a.p_hi && ok; ++p) {
                 const int kind = kind_of(p);
                 if (kind == FW_ATTN) { pos += 2 * a_n; continue; }
                 const FwPhase& f = a.ph[kind];
                 const CUtensorMap* m = &a.x[kind];
-                if (p > 0) {
+                if (p > a.p_lo) {
                     ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
                     proxy_fence();
                 }
@@ -941,7 +942,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         const int me = warp - 2;
         int pos = 0, tcount = 0, at = 0, as = 0;       // ring position, projection tiles, attention tiles, segments so far
         bool ok = true;
-        for (int p = 0; p < n_phases && ok; ++p) {
+        for (int p = a.p_lo; p < a.p_hi && ok; ++p) {
             const int kind = kind_of(p);
             if (kind == FW_ATTN) {
                 if (me == 0) {
@@ -1056,13 +1057,13 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         };
         const int ring_other = steps_of(a.ph[FW_O]) + steps_of(a.ph[FW_GATEUP]) + steps_of(a.ph[FW_DOWN]);
         const int ring_qkv = steps_of(a.ph[FW_QKV]);
-        for (int p = 0; p < n_phases && ok; ++p) {
+        for (int p = a.p_lo; p < a.p_hi && ok; ++p) {
             const int kind = kind_of(p), layer = p / 5;
             if (kind == FW_ATTN) {
-                if (e == 0) ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
+                if (e == 0 && p > a.p_lo) ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
                 ok = all_of(1, FW_EPI, ok);
                 if (!ok) break;
-                pos += ring_qkv;
+                if (p > a.p_lo) pos += ring_qkv;
                 const int G = a.Hq / a.Hkv, kl = quad * 32 + lane;    // this thread's key of a tile, later its head dimension
                 constexpr int NR = NQP / 2;                           // this thread's query rows: half, half + 2, ...; wide:
                 auto row_of = [&](int x) { return WIDE ? half * NR + x : 2 * x + half; };        // NR neighbouring ones
@@ -1201,7 +1202,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     if (i > 0) attn_step(it, i);
                     if (fresh) {
 #pragma unroll
-                        for (int x = 0; x < NR; ++x) { m[x] = -CUDART_INF_F; l[x] = 0.f; acc[x] = 0.f; }
+                        for (int x = 0; x < NR; ++x) { m[x] = FW_UNSEEN; l[x] = 0.f; acc[x] = 0.f; }
                     }
                     if (fresh) { L = s.meta[it.bi].L; nkeys = s.meta[it.bi].nkeys; }
                     const bool turn = WIDE && i + 1 < a_n && (i + 1 == a_wrap || it.tile + 1 == it.nt);     // the segment's last
@@ -1237,8 +1238,9 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     tc_fence_after();
                     float v[NR];
                     tm_rows(b * TM, v);
+                    if (__any_sync(0xffffffffu, vis != 0xffffffffu))
 #pragma unroll
-                    for (int x = 0; x < NR; ++x) v[x] = ((vis >> x) & 1u) ? v[x] : -CUDART_INF_F;
+                        for (int x = 0; x < NR; ++x) v[x] = ((vis >> x) & 1u) ? v[x] : -CUDART_INF_F;
                     if (turn) load_q(ahead, 0);                       // (this segment's scores are formed, the query tile is free)
                     // The reference value m of a row need not be its maximum: numerators and sums have the exponent range that
                     // fp32 and bf16 share, and a common factor costs no precision.  A segment starts with the score of its first
@@ -1246,21 +1248,22 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     if (fresh) {
                         if (kl == 0)
 #pragma unroll
-                            for (int x = 0; x < NR; ++x) sa.sm[half][x] = v[x];
+                            for (int x = 0; x < NR; ++x) sa.sm[half][x] = fmaxf(v[x], FW_UNSEEN);
                         bar_n(2 + half, 128);
                     }
                     if (WIDE || fresh)
 #pragma unroll
                         for (int x = 0; x < NR; ++x) m[x] = sa.sm[half][x];
-                    bool calm = true;
+                    float most = -CUDART_INF_F;
 #pragma unroll
-                    for (int x = 0; x < NR; ++x) calm = calm && v[x] <= m[x] + FW_LAZY && m[x] > -CUDART_INF_F;
-                    const bool quiet = all_of(2 + half, 128, calm);
+                    for (int x = 0; x < NR; ++x) { v[x] -= m[x]; most = fmaxf(most, v[x]); }
+                    const bool quiet = all_of(2 + half, 128, most <= FW_LAZY);
                     if (!quiet) {
                         if (!fresh) output(at - 1);                   // (before the reference moves)
                         float wm[NR];
+                        tm_rows(b * TM, v);
 #pragma unroll
-                        for (int x = 0; x < NR; ++x) wm[x] = v[x];
+                        for (int x = 0; x < NR; ++x) wm[x] = v[x] = ((vis >> x) & 1u) ? v[x] : -CUDART_INF_F;
 #pragma unroll
                         for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
@@ -1273,8 +1276,9 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         for (int x = 0; x < NR; ++x) {
                             const float4 q4 = *reinterpret_cast<const float4*>(sa.smx[half][x]);
                             const float mn = fmaxf(m[x], fmaxf(fmaxf(q4.x, q4.y), fmaxf(q4.z, q4.w)));
-                            const float f = mn == -CUDART_INF_F ? 1.f : exp2f(m[x] - mn);
+                            const float f = exp2f(m[x] - mn);
                             m[x] = mn;
+                            v[x] -= mn;
                             l[x] *= f;
                             acc[x] *= f;
                         }
@@ -1290,7 +1294,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
 #pragma unroll
                     for (int x = 0; x < NR; ++x) {
                         // (exp2(-inf) = 0; results below 2^-126 of a sum of at least 1, the reference being a key's score, go to 0)
-                        const float pv = exp2_ftz(v[x] - (m[x] == -CUDART_INF_F ? 0.f : m[x]));
+                        const float pv = exp2_ftz(v[x]);
                         l[x] += pv;
                         const __nv_bfloat16 hi = __float2bfloat16_rn(pv);
                         uint8_t* d = pt + ((pc ^ (row_of(x) & 7)) << 4) + x * RS;
@@ -1465,6 +1469,7 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
     while (FW_CLASS[a.cls].cols < a.cols) ++a.cls;
     fw_geometry(a.ph, d, n_cta, a.cls);
     a.n_cta = n_cta; a.n_layers = d.layers;
+    a.p_lo = 0; a.p_hi = 5 * d.layers + 1;
     a.d = d.d_model; a.F = d.d_ffn; a.V = d.vocab; a.Hq = d.n_q_heads; a.Hkv = d.n_kv_heads; a.hd = d.head_dim;
     for (int k = 0; k < 6; ++k) {
         if (k == FW_ATTN) continue;
@@ -1483,6 +1488,23 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
         f.blk = std::min(up_div(T, per), fit) * per;
     }
     return true;
+}
+
+bool fw_attn_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
+    const int G = d.n_q_heads / d.n_kv_heads;
+    if ((d.head_dim != 64 && d.head_dim != 128) || G * R <= FW_QROWS || B * R > TC_MAX_ROWS || B > MTAD_MAX_BATCH) return false;
+    a.T = B * R; a.B = B; a.R = R; a.terms = tc_terms(a.T); a.cls = 2;
+    a.nqb = up_div(G * R, FW_QROWS_WIDE);
+    a.qrows = up_div(G * R, a.nqb);
+    a.n_cta = n_cta; a.n_layers = d.layers;
+    a.Hq = d.n_q_heads; a.Hkv = d.n_kv_heads; a.hd = d.head_dim;
+    return true;
+}
+
+cudaError_t launch_forward_attention(FwArgs& a, int layer, cudaStream_t st) {
+    a.p_lo = 5 * layer + FW_ATTN;
+    a.p_hi = a.p_lo + 1;
+    return launch_forward(a, st);
 }
 
 size_t fw_parts_max(const mtad_model_desc& d, int n_cta, bool lm) {

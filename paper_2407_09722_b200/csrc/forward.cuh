@@ -44,6 +44,7 @@ struct FwArgs {
     FwPhase ph[6];                        // by kind; the entry of the attention is unused
     const FwLayer* layers;
     int n_layers, n_cta;
+    int p_lo, p_hi;                       // phases of this launch: all, or one attention
     int T, terms, cols, B, R, d, F, V, Hq, Hkv, hd, max_batch, lm_plain;
     int nqb, qrows;                       // wide attention: blocks that a sequence's query rows of a KV head are cut into, rows of a block
     int pieces;                           // stride of the attention partials: pieces per (row, head)
@@ -71,16 +72,20 @@ struct FwArgs {
 // partial results that a row of a call has.
 void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta, int cls);
 bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta);
+// The attention alone, wide variant, for a call whose projections run as launches of their own; run for one layer with
+// launch_forward_attention.
+bool fw_attn_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta);
 size_t fw_parts_max(const mtad_model_desc& d, int n_cta, bool lm);
-// (sequence, KV head, query block)s of a call at most: B * ceil(G R / rows) with B R <= FW_MAX_ROWS
+// (sequence, KV head, query block)s of a call at most: B * ceil(G R / rows) with B R <= TC_MAX_ROWS
 inline size_t fw_pairs(const mtad_model_desc& d, int max_batch) {
     const int G = d.n_q_heads / d.n_kv_heads;
-    return (size_t)d.n_kv_heads * ((G * FW_MAX_ROWS + FW_QROWS_WIDE - 1) / FW_QROWS_WIDE + max_batch);
+    return (size_t)d.n_kv_heads * ((G * TC_MAX_ROWS + FW_QROWS_WIDE - 1) / FW_QROWS_WIDE + max_batch);
 }
 // words of the phase and arrival counters (zeroed by the row preparation of every call)
 inline size_t fw_sync_words(const mtad_model_desc& d, int max_batch, int n_cta) {
     return (size_t)5 * d.layers + 1 + fw_pairs(d, max_batch) + 2 * (size_t)n_cta;
 }
 cudaError_t launch_forward(const FwArgs& a, cudaStream_t st);
+cudaError_t launch_forward_attention(FwArgs& a, int layer, cudaStream_t st);
 
 }  // namespace mtad
