@@ -741,11 +741,12 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     constexpr int Q_BYTES = NQ2 * HD * 2;              // one query tile
     constexpr int P_BYTES = NQ2 * FW_KEYS * 2;         // one probability tile
     constexpr int FW_SLOT = FW_RING / NS;
-    // Wide attention: up to 40 query rows, whose tiles outgrow the union.  The probabilities of a tile lie behind its V tile, in
-    // the rest of the ring slot (free by then: the slot's item before it was used before this tile's scores were formed, as
-    // long as that item is the K tile of the tile before, three items ago), and there is one query tile instead of two.
-    constexpr bool WIDE = NQP > FW_QROWS;
-    static_assert(!WIDE || (NS == 3 && (int)KV_BYTES + P_BYTES <= FW_SLOT && Q_BYTES + (int)sizeof(FwAttn<NQP / 2>) <= FW_UNION), "wide attention");
+    // Wide attention: up to 40 query rows, whose tiles outgrow the union.  There is one query tile instead of two, and the
+    // probabilities lie in the ring, behind the K and V tiles, which do not fill their slots: with three slots behind V; with
+    // four the second 64 keys behind K.  That space is a tile's own: an item that fills its slot (a step of a projection) came
+    // before the attention, or comes after the output has been formed (PBK: so the last two K tiles are released only then).
+    constexpr bool WIDE = NQP > FW_QROWS, PBK = WIDE && NS == 4;
+    static_assert(!WIDE || ((int)KV_BYTES + P_BYTES / (PBK ? 2 : 1) <= FW_SLOT && Q_BYTES + (int)sizeof(FwAttn<NQP / 2>) <= FW_UNION), "wide attention");
     constexpr int TM = WIDE ? 128 : 64;                // attention: tensor-memory columns 0 / TM scores, 2 TM / 3 TM outputs
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* uni = smem + FW_RING;
@@ -968,8 +969,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             tc_mma_one(one, tmem + b * TM, ka + (ks >> 2) * (FW_KEYS * 8) + (ks & 3) * 2,
                                        qa + (ks >> 2) * (NQ2 * 8) + (ks & 3) * 2, idesc_s, ks > 0 ? 1u : 0u);
                         tc_commit_one(one, smem_u32(&s.sfull[b]));
-                        tc_commit_one(one, empty_bar(kpos));
-                        tc_commit_one(one, empty_bar(kpos));
+                        if (!PBK || i < a_n - 2) {
+                            tc_commit_one(one, empty_bar(kpos));
+                            tc_commit_one(one, empty_bar(kpos));
+                        }
                     }
                     if (a_n > 0) ++as;
                     if (NS % 2 && a_n > 1 && ok) {     // (the next phase's first slot held the last V tile but one)
@@ -987,13 +990,18 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         if (!ok) break;
                         tc_fence_after();
                         const uint64_t va = smem_desc_mn(slot_ptr(vpos)), pa = smem_desc(WIDE ? slot_ptr(vpos) + KV_BYTES : smem_u32(Ps) + b * P_BYTES);
+                        const uint64_t pb = PBK ? smem_desc(slot_ptr(vpos - 1) + KV_BYTES) : pa + NQ2 * 8;       // keys 64 ..
 #pragma unroll
                         for (int ks = 0; ks < FW_KEYS / 16; ++ks)
-                            tc_mma_one(one, tmem + (2 + b) * TM, va + ks * 128, pa + (ks >> 2) * (NQ2 * 8) + (ks & 3) * 2,
+                            tc_mma_one(one, tmem + (2 + b) * TM, va + ks * 128, (ks < 4 ? pa : pb) + (ks & 3) * 2,
                                        idesc_o, ks > 0 ? 1u : 0u);
                         tc_commit_one(one, smem_u32(&s.ofull[b]));
                         tc_commit_one(one, empty_bar(vpos));
                         tc_commit_one(one, empty_bar(vpos));
+                        if (PBK && i >= a_n - 2) {
+                            tc_commit_one(one, empty_bar(vpos - 1));
+                            tc_commit_one(one, empty_bar(vpos - 1));
+                        }
                     }
                 }
                 at += a_n;
@@ -1287,8 +1295,8 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             for (int x = 0; x < NR; ++x) sa.sm[half][x] = m[x];
                         bar_n(2 + half, 128);                         // (smx is free again)
                     }
-                    uint8_t* pt = (WIDE ? smem + (size_t)((pos + 2 * i + 1) % NS) * FW_SLOT + KV_BYTES : Ps + b * P_BYTES) +
-                                  (kl >> 6) * (NQ2 * 128) + (kl & 7) * 2 + row_of(0) * 128;
+                    uint8_t* pt = (WIDE ? smem + (size_t)((pos + 2 * i + (PBK && kl >= 64 ? 0 : 1)) % NS) * FW_SLOT + KV_BYTES : Ps + b * P_BYTES) +
+                                  (PBK ? 0 : kl >> 6) * (NQ2 * 128) + (kl & 7) * 2 + row_of(0) * 128;
                     constexpr int RS = WIDE ? 128 : 256;              // bytes between this thread's rows
                     const int pc = (kl & 63) >> 3;
 #pragma unroll
@@ -1493,7 +1501,7 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
 bool fw_attn_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
     const int G = d.n_q_heads / d.n_kv_heads;
     if ((d.head_dim != 64 && d.head_dim != 128) || G * R <= FW_QROWS || B * R > TC_MAX_ROWS || B > MTAD_MAX_BATCH) return false;
-    a.T = B * R; a.B = B; a.R = R; a.terms = tc_terms(a.T); a.cls = 2;
+    a.T = B * R; a.B = B; a.R = R; a.terms = tc_terms(a.T); a.cls = FW_CLASSES - 1;
     a.nqb = up_div(G * R, FW_QROWS_WIDE);
     a.qrows = up_div(G * R, a.nqb);
     a.n_cta = n_cta; a.n_layers = d.layers;
@@ -1537,11 +1545,18 @@ cudaError_t launch_forward(const FwArgs& a, cudaStream_t st) {
     };
     // instantiations: head size, query rows of an attention item, few rows in all, ring slots
     auto pick = [&](auto hd) -> cudaError_t {
-        constexpr int HD = decltype(hd)::value, NF = FW_CLASS[0].slots, NM = FW_CLASS[2].slots;
-        const bool q8 = (a.Hq / a.Hkv) * a.R <= 8, q16 = (a.Hq / a.Hkv) * a.R <= FW_QROWS;
-        if (a.cls < 2) return q8 ? go(forward_kernel<HD, 8, true, NF>) : go(forward_kernel<HD, FW_QROWS, true, NF>);
-        if (q8) return go(forward_kernel<HD, 8, false, NM>);
-        return q16 ? go(forward_kernel<HD, FW_QROWS, false, NM>) : go(forward_kernel<HD, FW_QROWS_WIDE, false, NM>);
+        constexpr int HD = decltype(hd)::value;
+        const int n_q = (a.Hq / a.Hkv) * a.R;
+        auto rows = [&](auto few, auto slots) -> cudaError_t {
+            constexpr bool FEW = decltype(few)::value;
+            constexpr int NS = decltype(slots)::value;
+            if (n_q <= 8) return go(forward_kernel<HD, 8, FEW, NS>);
+            if (FEW || n_q <= FW_QROWS) return go(forward_kernel<HD, FW_QROWS, FEW, NS>);
+            return go(forward_kernel<HD, FEW ? FW_QROWS : FW_QROWS_WIDE, FEW, NS>);
+        };
+        using std::integral_constant;
+        if (a.cls < 2) return rows(std::true_type{}, integral_constant<int, 4>{});
+        return FW_CLASS[a.cls].slots == 3 ? rows(std::false_type{}, integral_constant<int, 3>{}) : rows(std::false_type{}, integral_constant<int, 4>{});
     };
     return a.hd == 128 ? pick(std::integral_constant<int, 128>{}) : pick(std::integral_constant<int, 64>{});
 }
