@@ -20,20 +20,8 @@ constexpr int FW_QROWS_WIDE = 40;         // or in the wide variant: more are cu
 // Big boxes matter twice: a thread issues a copy about every quarter of a microsecond whatever its size, and rows of 256
 // bytes and more pass at 70 GB/s per SM where rows of 128 bytes pass at 43.
 constexpr int FW_CLASSES = 6;
-#ifndef FWS64
-#define FWS64 3
-#endif
-#ifndef FWS80
-#define FWS80 3
-#endif
-#ifndef FWS112
-#define FWS112 3
-#endif
-#ifndef FWS144
-#define FWS144 4
-#endif
 struct FwClass { int cols, slots; };      // operand rows up to, ring slots
-constexpr FwClass FW_CLASS[FW_CLASSES] = {{16, 4}, {32, 4}, {64, FWS64}, {80, FWS80}, {112, FWS112}, {FW_MAX_COLS, FWS144}};
+constexpr FwClass FW_CLASS[FW_CLASSES] = {{16, 4}, {32, 4}, {64, 4}, {80, 3}, {112, 3}, {FW_MAX_COLS, 4}};
 struct FwPhase {
     int h, hr, nbox, n_tiles, u;          // u: tiles per head (QKV)
     int c;                                // O, down: blocks that share a tile's k-range (their partial sums meet in global memory)
