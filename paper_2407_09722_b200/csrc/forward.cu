@@ -203,7 +203,6 @@ struct FwTail {
     uint8_t rowb[FW_MAX_ROWS];            // its sequence within the call
     FwAttn<FW_QROWS / 2> attn;            // (the wide attention's lies behind its query tile)
     uint64_t full[FW_BARS], empty[FW_BARS];
-    int kv_pos, kv_slot;                  // the attention's first item in the ring
     int issued;                           // items whose place was found free, as far as slots are new
     uint64_t tfull[2], tempty[2], sfull[2], pfull[2], ofull[2], qfull[2];
     uint32_t tmem_ptr;
@@ -1137,22 +1136,15 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         };
         for (int p = a.p_lo; p < a.p_hi && ok; ++p) {
             const int kind = kind_of(p), layer = p / 5;
+            if (kind != FW_ATTN && cta < a.ph[kind].n_tiles) {
+                r.enter(a.ph[kind].ns, a.ph[kind].sz);
+                r.skip(steps_of(a.ph[kind]));
+            }
             if (kind == FW_ATTN) {
-                if (e == 0) {                                         // (one thread, while it would wait)
-                    for (int k : {FW_O, FW_GATEUP, FW_DOWN, FW_QKV}) {
-                        const FwPhase& f = a.ph[k];
-                        if (p == a.p_lo || cta >= f.n_tiles || (layer == 0 && k != FW_QKV)) continue;
-                        r.enter(f.ns, f.sz);
-                        r.skip(steps_of(f));
-                    }
-                    if (a_n > 0) r.enter(KV_SLOTS, KV_SLOT);
-                    s.kv_pos = r.pos;
-                    s.kv_slot = r.slot;
-                }
                 if (e == 0 && p > a.p_lo) ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
                 ok = all_of(1, FW_EPI, ok);
                 if (!ok) break;
-                const int kv_pos = s.kv_pos, kv_slot = s.kv_slot;
+                if (a_n > 0) r.enter(KV_SLOTS, KV_SLOT);
                 const int G = a.Hq / a.Hkv, kl = quad * 32 + lane;    // this thread's key of a tile, later its head dimension
                 constexpr int NR = NQP / 2;                           // this thread's query rows: half, half + 2, ...; wide:
                 auto row_of = [&](int x) { return WIDE ? half * NR + x : 2 * x + half; };        // NR neighbouring ones
@@ -1376,7 +1368,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             for (int x = 0; x < NR; ++x) sa.sm[half][x] = m[x];
                         bar_n(2 + half, 128);                         // (smx is free again)
                     }
-                    uint8_t* pt = (WIDE ? smem + (kv_slot + 2 * i + (kl >= 64 ? 0 : 1)) % KV_SLOTS * KV_SLOT + KV_BYTES
+                    uint8_t* pt = (WIDE ? smem + (r.slot + 2 * i + (kl >= 64 ? 0 : 1)) % KV_SLOTS * KV_SLOT + KV_BYTES
                                         : Ps + b * P_BYTES + (kl >> 6) * (NQ2 * 128)) + (kl & 7) * 2 + row_of(0) * 128;
                     constexpr int RS = WIDE ? 128 : 256;              // bytes between this thread's rows
                     const int pc = (kl & 63) >> 3;
@@ -1392,10 +1384,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     }
                     if ((it.tile + 1) * FW_KEYS > nkeys) {
                         // rows of V past the last key: their probabilities are 0, but 0 x (stale value) must not make a NaN
-                        const int vpos = kv_pos + 2 * i + 1;
+                        const int vpos = r.pos + 2 * i + 1;
                         ok = warp_wait(full_bar(vpos), ring_par(vpos), abort_flag, ok, lane);
                         if (ok && j >= nkeys) {
-                            uint8_t* vs = smem + (kv_slot + 2 * i + 1) % KV_SLOTS * KV_SLOT + kl * 128 + half * 64;
+                            uint8_t* vs = smem + (r.slot + 2 * i + 1) % KV_SLOTS * KV_SLOT + kl * 128 + half * 64;
 #pragma unroll
                             for (int c = 0; c < NCH * 4; ++c)
                                 *reinterpret_cast<uint4*>(vs + (c >> 2) * (FW_KEYS * 128) + (c & 3) * 16) = make_uint4(0u, 0u, 0u, 0u);
@@ -1417,7 +1409,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     output(at - 1);
                     finish(it);
                 }
-                if (e == 0 && a_n > 0) r.skip(2 * a_n);
+                if (a_n > 0) r.skip(2 * a_n);
                 ok = all_of(1, FW_EPI, ok);
                 if (!ok) break;
                 // pieces shared with other blocks (at most the first and the last of this block's range): who arrives last merges
@@ -1542,11 +1534,10 @@ void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta, int cls) {
             const int ns = std::min(FW_SLOTS, FW_RING / (kb * one));
             if (ns < 3 || (S > 1 && kb > S && kb % S)) continue;
             double flight = (double)ns * kb * one * (kb == 1 ? 0.85 : kb * one < 40 * 1024 ? 0.93 : 1.0) * (ns == 3 ? 0.97 : 1.0);
-            if (ns == 4 && f.k_blocks * one <= 2 * FW_RING) flight *= 1.5;
-            if (few) flight = ns >= 4 ? kb : 0;
+            if (ns == 4 && (few || f.k_blocks * one <= 2 * FW_RING)) flight *= few ? 1.3 : 1.5;
             if (flight > best) { best = flight; f.kb = kb; }
         }
-        f.ns = few ? 4 : std::min(FW_SLOTS, FW_RING / (f.kb * one));
+        f.ns = std::min(FW_SLOTS, FW_RING / (f.kb * one));
         f.sz = FW_RING / f.ns / 1024 * 1024;
         f.flat = tc_kb_flat(f.K, f.kb) ? 1 : 0;
         f.steps = up_div(f.k_blocks, f.kb);
