@@ -48,7 +48,6 @@ constexpr int FW_UNION = 32 * 1024;       // epilogue tile Y, or the attention's
 constexpr int FW_ACC = 240;               // accumulator columns of a tile, of 256 (the drain reads up to 15 columns further),
 constexpr int FW_ACC_ONE = 496;           // or of 512 where a tile takes both buffers
 constexpr int FW_BARS = 8;                // barriers of the copy ring, one per item in turn
-constexpr int FW_SIDE = 8;                // k-blocks side by side in an MMA at most (the epilogue adds up as many values)
 constexpr int FW_SLOTS = 6;               // slots of the ring at most
 constexpr float FW_LAZY = 64.f;           // log2 of how far a score may exceed its row's reference value
 constexpr float FW_UNSEEN = -1e30f;       // the reference value of a row that has seen no key
@@ -1527,14 +1526,14 @@ void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta, int cls) {
         // the k-blocks that the MMA can take side by side.  Changing the slots costs about a slot's worth of bytes in flight, so
         // phases with as many slots have slots of one size, and four are preferred where rows or steps are few.
         const bool few = cls < 2;
-        const int S = std::min(FW_SIDE, std::min(TC_TILE_N / f.hr, FW_ACC / (cols * f.nbox))), one = (f.nbox * f.hr + cols) * 128;
+        const int S = std::min(TC_TILE_N / f.hr, FW_ACC / (cols * f.nbox)), one = (f.nbox * f.hr + cols) * 128;
         double best = 0;
         f.kb = 1;
         for (int kb = f.K % TC_TILE_K ? 1 : std::min(f.k_blocks, 16); kb >= 1; --kb) {
             const int ns = std::min(FW_SLOTS, FW_RING / (kb * one));
             if (ns < 3 || (S > 1 && kb > S && kb % S)) continue;
             double flight = (double)ns * kb * one * (kb == 1 ? 0.85 : kb * one < 40 * 1024 ? 0.93 : 1.0) * (ns == 3 ? 0.97 : 1.0);
-            if (ns == 4 && (few || f.k_blocks * one <= 2 * FW_RING)) flight *= few ? 1.3 : 1.5;
+            if (ns == 4 && (few || f.k_blocks * one <= 2 * FW_RING)) flight *= few ? 1.1 : 1.5;
             if (flight > best) { best = flight; f.kb = kb; }
         }
         f.ns = std::min(FW_SLOTS, FW_RING / (f.kb * one));
@@ -1567,7 +1566,7 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
         if (k == FW_ATTN) continue;
         FwPhase& f = a.ph[k];
         f.S = 1;
-        for (int S = 2; S <= std::min(f.kb, FW_SIDE); ++S)
+        for (int S = 2; S <= f.kb; ++S)
             if (f.kb % S == 0 && S * f.hr <= TC_TILE_N && S * a.cols * f.nbox <= FW_ACC) f.S = S;
         if (f.ns < 2 || f.b_off + f.kb * a.cols * 128 > f.sz || f.nbox * f.S * a.cols > FW_ACC_ONE) return false;
         f.both = f.nbox * f.S * a.cols > FW_ACC ? 1 : 0;
