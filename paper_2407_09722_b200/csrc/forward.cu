@@ -769,7 +769,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     // K.  That space is a tile's own: a projection's items came before the attention, or come after the output has been formed
     // (the last two K tiles are released only then).
     constexpr bool WIDE = NQP > FW_QROWS;
-    constexpr int KV_SLOTS = WIDE || FEW ? 4 : FW_SLOTS, KV_SLOT = FW_RING / KV_SLOTS;
+    constexpr int KV_SLOTS = WIDE ? 4 : FW_SLOTS, KV_SLOT = WIDE ? FW_RING / 4 : (int)KV_BYTES;
     static_assert(!WIDE || ((int)KV_BYTES + P_BYTES / 2 <= KV_SLOT && Q_BYTES + (int)sizeof(FwAttn<NQP / 2>) <= FW_UNION), "wide attention");
     constexpr int TM = WIDE ? 128 : 64;                // attention: tensor-memory columns 0 / TM scores, 2 TM / 3 TM outputs
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -1523,21 +1523,18 @@ void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta, int cls) {
         FwPhase& f = ph[k];
         // k-blocks of a step: as many bytes in flight as the ring holds, in three slots at least; rows of one k-block (128
         // bytes) pass slower than longer ones, and a step takes its producer 0.3 us, which small ones do not last; a multiple of
-        // the k-blocks that the MMA can take side by side.  Changing the slots costs about a slot's worth of bytes in flight, so
-        // phases with as many slots have slots of one size, and four are preferred where rows or steps are few.
-        const bool few = cls < 2;
+        // the k-blocks that the MMA can take side by side
         const int S = std::min(TC_TILE_N / f.hr, FW_ACC / (cols * f.nbox)), one = (f.nbox * f.hr + cols) * 128;
         double best = 0;
         f.kb = 1;
         for (int kb = f.K % TC_TILE_K ? 1 : std::min(f.k_blocks, 16); kb >= 1; --kb) {
             const int ns = std::min(FW_SLOTS, FW_RING / (kb * one));
             if (ns < 3 || (S > 1 && kb > S && kb % S)) continue;
-            double flight = (double)ns * kb * one * (kb == 1 ? 0.85 : kb * one < 40 * 1024 ? 0.93 : 1.0) * (ns == 3 ? 0.97 : 1.0);
-            if (ns == 4 && (few || f.k_blocks * one <= 2 * FW_RING)) flight *= few ? 1.1 : 1.5;
+            const double flight = (double)ns * kb * one * (kb == 1 ? 0.85 : kb * one < 40 * 1024 ? 0.93 : 1.0) * (ns == 3 ? 0.97 : 1.0);
             if (flight > best) { best = flight; f.kb = kb; }
         }
-        f.ns = std::min(FW_SLOTS, FW_RING / (f.kb * one));
-        f.sz = FW_RING / f.ns / 1024 * 1024;
+        f.sz = f.kb * one;
+        f.ns = std::min(FW_SLOTS, FW_RING / f.sz);
         f.flat = tc_kb_flat(f.K, f.kb) ? 1 : 0;
         f.steps = up_div(f.k_blocks, f.kb);
         f.box_bytes = f.hr * 128 * f.kb;
