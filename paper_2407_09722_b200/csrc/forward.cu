@@ -172,14 +172,13 @@ __device__ __forceinline__ void attn_next(AttnPos& it, const SeqMeta* meta, int 
 // microseconds.  Every role walks the same items in the same order and so knows where each lies: item `pos` of the launch uses
 // barriers pos % FW_BARS, and a phase's first slot follows the memory that the one before used last.
 struct Ring {
-    int pos = 0, slot = 0, ns = 1, sz = 0, since = 0;      // since: the first item with the present slots
+    int pos = 0, slot = 0, ns = 1, sz = 0;
     __device__ __forceinline__ void enter(int n, int size) {
         if (size == sz) return;
         slot = sz ? (slot * sz + size - 1) / size : 0;
         if (slot >= n) slot = 0;
         ns = n;
         sz = size;
-        since = pos;
     }
     __device__ __forceinline__ void skip(int n) { pos += n; slot = (slot + n) % ns; }
     __device__ __forceinline__ void next() {
@@ -202,7 +201,9 @@ struct FwTail {
     uint8_t rowb[FW_MAX_ROWS];            // its sequence within the call
     FwAttn<FW_QROWS / 2> attn;            // (the wide attention's lies behind its query tile)
     uint64_t full[FW_BARS], empty[FW_BARS];
-    int issued;                           // items whose place was found free, as far as slots are new
+    int lo[FW_BARS];                      // (weight producer) where the last items lie in the ring, their sizes
+    int size[FW_BARS];
+    int issued;                           // items that have their place and their byte count
     uint64_t tfull[2], tempty[2], sfull[2], pfull[2], ofull[2], qfull[2];
     uint32_t tmem_ptr;
     int abort_flag[2];
@@ -797,6 +798,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     }
     if (threadIdx.x == 0) {
         for (int i = 0; i < FW_BARS; ++i) {
+            s.size[i] = 0;
             mbar_init(smem_u32(&s.full[i]), 1);
             mbar_init(smem_u32(&s.empty[i]), 2);       // both MMA warps
         }
@@ -858,35 +860,27 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         // ---------------- weight and K / V producer: walks all phases; only the K / V tiles that hold this call's own
         // rows wait for the phase that writes them
         if (lane == 0) {
-            Ring r, was;                               // was: at the change to the present slots
+            Ring r;
+            int since = 0;                             // the first item with the present slots
             bool ok = true;
             auto enter = [&](int n, int size) {
-                if (size != r.sz) was = r;
+                if (size != r.sz) since = r.pos;
                 r.enter(n, size);
             };
-            auto used = [&](int q) { ok = ok && (q < 0 || mbar_wait(empty_bar(q), ring_par(q), abort_flag)); };
-            // The item's place is free when the item one turn before it has been used.  While the slots are new it is when the
-            // items before the change that overlap it have been: the old items follow one another in the ring from where the
-            // new slots began, and are used in this order (K and V tiles in pairs).  Slots that the old items did not all take hold
-            // what came before those.  An item before pos - FW_BARS has been used when that one has, and has no barrier any more.
+            // The item's place is free: the item one turn before it has been used; while the slots are new, every item that
+            // overlaps it and the one that used its barriers.
             auto acquire = [&](uint32_t bytes) {
-                if (r.pos - r.since >= FW_BARS) {
-                    used(r.pos - r.ns);
-                } else {
-                    if (r.pos - r.since >= r.ns) {
-                        used(r.pos - r.ns);
-                    } else if (was.sz) {
-                        const int begin = was.slot * was.sz, end = (r.slot + 1) * r.sz;
-                        const int span = end - begin + (r.slot * r.sz < begin ? was.ns * was.sz : 0);
-                        int q = was.pos - was.ns + min(was.ns, (span + was.sz - 1) / was.sz) - 1;
-                        if (q < was.since) q = was.since - 1;
-                        if (q - 1 > r.pos - FW_BARS) used(q - 1);
-                        if (q > r.pos - FW_BARS) used(q);
-                    }
-                    used(r.pos - FW_BARS);
-                    if (ok) asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(smem_u32(&s.issued)), "r"(r.pos + 1) : "memory");
-                }
-                if (ok) mbar_expect_tx(full_bar(r.pos), bytes);
+                const int at = r.slot * r.sz;
+                if (r.pos - since >= r.ns) ok = mbar_wait(empty_bar(r.pos - r.ns), ring_par(r.pos - r.ns), abort_flag);
+                if (r.pos - since < FW_BARS)
+                    for (int q = max(0, r.pos - FW_BARS); q < r.pos && ok; ++q)
+                        if (q == r.pos - FW_BARS || (s.lo[q % FW_BARS] < at + r.sz && at < s.lo[q % FW_BARS] + s.size[q % FW_BARS]))
+                            ok = mbar_wait(empty_bar(q), ring_par(q), abort_flag);
+                if (!ok) return;
+                s.lo[r.pos % FW_BARS] = at;
+                s.size[r.pos % FW_BARS] = r.sz;
+                mbar_expect_tx(full_bar(r.pos), bytes);
+                asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(smem_u32(&s.issued)), "r"(r.pos + 1) : "memory");
             };
             for (int p = a.p_lo; p < a.p_hi && ok; ++p) {
                 const int kind = kind_of(p), layer = p / 5;
@@ -967,8 +961,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         if (lane == 0) {
             Ring r;
             bool ok = true;
-            auto issued = [&]() -> bool {              // the item's place is free: see above
-                if (r.pos - r.since >= FW_BARS) return mbar_wait(empty_bar(r.pos - r.ns), ring_par(r.pos - r.ns), abort_flag);
+            auto issued = [&]() -> bool {              // the weight producer has acquired item r.pos
                 const uint32_t limit = (uint32_t)abort_flag[1];
                 for (uint32_t it = 0; it < limit; ++it) {
                     int v;
