@@ -47,8 +47,6 @@ constexpr int FW_EPI = 256;
 constexpr int FW_UNION = 32 * 1024;       // epilogue tile Y, or the attention's query and probability tiles
 constexpr int FW_ACC = 240;               // accumulator columns of a tile, of 256 (the drain reads up to 15 columns further),
 constexpr int FW_ACC_ONE = 496;           // or of 512 where a tile takes both buffers
-constexpr int FW_BARS = 8;                // barriers of the copy ring, one per item in turn
-constexpr int FW_SLOTS = 6;               // slots of the ring at most
 constexpr float FW_LAZY = 64.f;           // log2 of how far a score may exceed its row's reference value
 constexpr float FW_UNSEEN = -1e30f;       // the reference value of a row that has seen no key
 
@@ -167,26 +165,6 @@ __device__ __forceinline__ void attn_next(AttnPos& it, const SeqMeta* meta, int 
     if (it.bi < B) it.nt = attn_tiles(meta[it.bi]);
 }
 
-// The copy ring.  Its memory is cut into slots of the size that a phase's items need, so that whatever the phase close to all
-// of it is in flight: an SM's intake is bytes in flight over latency, and the latency with every SM at it is above two
-// microseconds.  Every role walks the same items in the same order and so knows where each lies: item `pos` of the launch uses
-// barriers pos % FW_BARS, and a phase's first slot follows the memory that the one before used last.
-struct Ring {
-    int pos = 0, slot = 0, ns = 1, sz = 0;
-    __device__ __forceinline__ void enter(int n, int size) {
-        if (size == sz) return;
-        slot = sz ? (slot * sz + size - 1) / size : 0;
-        if (slot >= n) slot = 0;
-        ns = n;
-        sz = size;
-    }
-    __device__ __forceinline__ void skip(int n) { pos += n; slot = (slot + n) % ns; }
-    __device__ __forceinline__ void next() {
-        ++pos;
-        if (++slot == ns) slot = 0;
-    }
-};
-
 // What the attention's epilogue warps tell one another, for NR rows in each half of them
 template <int NR>
 struct alignas(16) FwAttn {
@@ -200,10 +178,7 @@ struct FwTail {
     int slot[FW_MAX_ROWS];                // cache slot of a row, -1: inactive
     uint8_t rowb[FW_MAX_ROWS];            // its sequence within the call
     FwAttn<FW_QROWS / 2> attn;            // (the wide attention's lies behind its query tile)
-    uint64_t full[FW_BARS], empty[FW_BARS];
-    int lo[FW_BARS];                      // (weight producer) where the last items lie in the ring, their sizes
-    int size[FW_BARS];
-    int issued;                           // items that have their place and their byte count
+    uint64_t full[4], empty[4];
     uint64_t tfull[2], tempty[2], sfull[2], pfull[2], ofull[2], qfull[2];
     uint32_t tmem_ptr;
     int abort_flag[2];
@@ -758,20 +733,20 @@ __device__ __forceinline__ void merge_pieces(const FwArgs& a, const FwTail& s, c
     }
 }
 
-template <int HD, int NQP, bool FEW>
+template <int HD, int NQP, bool FEW, int NS>
 __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_constant__ FwArgs a) {
     constexpr int NCH = HD / 64;                       // 64-element chunks of a head row
     constexpr int NQ2 = 2 * NQP;                       // query rows as hi and lo parts
     constexpr uint32_t KV_BYTES = FW_KEYS * HD * 2;
     constexpr int Q_BYTES = NQ2 * HD * 2;              // one query tile
     constexpr int P_BYTES = NQ2 * FW_KEYS * 2;         // one probability tile
+    constexpr int FW_SLOT = FW_RING / NS;
     // Wide attention: up to 40 query rows, whose tiles outgrow the union.  There is one query tile instead of two, and the
-    // probabilities lie in the ring, in slots that the K and V tiles do not fill: the first 64 keys behind V, the others behind
-    // K.  That space is a tile's own: a projection's items came before the attention, or come after the output has been formed
-    // (the last two K tiles are released only then).
-    constexpr bool WIDE = NQP > FW_QROWS;
-    constexpr int KV_SLOTS = WIDE ? 4 : FW_SLOTS, KV_SLOT = WIDE ? FW_RING / 4 : (int)KV_BYTES;
-    static_assert(!WIDE || ((int)KV_BYTES + P_BYTES / 2 <= KV_SLOT && Q_BYTES + (int)sizeof(FwAttn<NQP / 2>) <= FW_UNION), "wide attention");
+    // probabilities lie in the ring, behind the K and V tiles, which do not fill their slots: with three slots behind V; with
+    // four the second 64 keys behind K.  That space is a tile's own: an item that fills its slot (a step of a projection) came
+    // before the attention, or comes after the output has been formed (PBK: so the last two K tiles are released only then).
+    constexpr bool WIDE = NQP > FW_QROWS, PBK = WIDE && NS == 4;
+    static_assert(!WIDE || ((int)KV_BYTES + P_BYTES / (PBK ? 2 : 1) <= FW_SLOT && Q_BYTES + (int)sizeof(FwAttn<NQP / 2>) <= FW_UNION), "wide attention");
     constexpr int TM = WIDE ? 128 : 64;                // attention: tensor-memory columns 0 / TM scores, 2 TM / 3 TM outputs
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* uni = smem + FW_RING;
@@ -797,8 +772,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         s.rowb[t] = (uint8_t)(t / a.R);
     }
     if (threadIdx.x == 0) {
-        for (int i = 0; i < FW_BARS; ++i) {
-            s.size[i] = 0;
+        for (int i = 0; i < NS; ++i) {
             mbar_init(smem_u32(&s.full[i]), 1);
             mbar_init(smem_u32(&s.empty[i]), 2);       // both MMA warps
         }
@@ -810,7 +784,6 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
             mbar_init(smem_u32(&s.ofull[i]), 1);
             mbar_init(smem_u32(&s.qfull[i]), 8);
         }
-        s.issued = 0;
         s.abort_flag[0] = 0;
         s.abort_flag[1] = (int)(a.wait_limit ? a.wait_limit : WAIT_LIMIT);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -845,11 +818,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         if (next == a_wrap) it = a_zero;
         else attn_next(it, s.meta, a.B, heads);
     };
-    auto kv_ptr = [&](int slot) { return smem_u32(smem) + (uint32_t)(slot % KV_SLOTS * KV_SLOT); };
-    auto slot_ptr = [&](const Ring& r) { return smem_u32(smem) + (uint32_t)(r.slot * r.sz); };
-    auto full_bar = [&](int pos) { return smem_u32(&s.full[pos % FW_BARS]); };
-    auto empty_bar = [&](int pos) { return smem_u32(&s.empty[pos % FW_BARS]); };
-    auto ring_par = [&](int pos) { return (uint32_t)(pos / FW_BARS) & 1u; };
+    auto slot_ptr = [&](int pos) { return smem_u32(smem) + (uint32_t)(pos % NS) * FW_SLOT; };
+    auto full_bar = [&](int pos) { return smem_u32(&s.full[pos % NS]); };
+    auto empty_bar = [&](int pos) { return smem_u32(&s.empty[pos % NS]); };
+    auto ring_par = [&](int pos) { return (uint32_t)(pos / NS) & 1u; };
     // steps [k0, k1) of a tile: all of them, or this block's share
     auto k_first = [&](const FwPhase& f, int tile) { return f.c > 1 ? (tile % f.c) * f.steps / f.c : 0; };
     auto k_end = [&](const FwPhase& f, int tile) { return f.c > 1 ? (tile % f.c + 1) * f.steps / f.c : f.steps; };
@@ -860,35 +832,14 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         // ---------------- weight and K / V producer: walks all phases; only the K / V tiles that hold this call's own
         // rows wait for the phase that writes them
         if (lane == 0) {
-            Ring r;
-            int since = 0;                             // the first item with the present slots
+            int pos = 0;
             bool ok = true;
-            auto enter = [&](int n, int size) {
-                if (size != r.sz) since = r.pos;
-                r.enter(n, size);
-            };
-            // The item's place is free: the item one turn before it has been used; while the slots are new, every item that
-            // overlaps it and the one that used its barriers.
-            auto acquire = [&](uint32_t bytes) {
-                const int at = r.slot * r.sz;
-                if (r.pos - since >= r.ns) ok = mbar_wait(empty_bar(r.pos - r.ns), ring_par(r.pos - r.ns), abort_flag);
-                if (r.pos - since < FW_BARS)
-                    for (int q = max(0, r.pos - FW_BARS); q < r.pos && ok; ++q)
-                        if (q == r.pos - FW_BARS || (s.lo[q % FW_BARS] < at + r.sz && at < s.lo[q % FW_BARS] + s.size[q % FW_BARS]))
-                            ok = mbar_wait(empty_bar(q), ring_par(q), abort_flag);
-                if (!ok) return;
-                s.lo[r.pos % FW_BARS] = at;
-                s.size[r.pos % FW_BARS] = r.sz;
-                mbar_expect_tx(full_bar(r.pos), bytes);
-                asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(smem_u32(&s.issued)), "r"(r.pos + 1) : "memory");
-            };
             for (int p = a.p_lo; p < a.p_hi && ok; ++p) {
                 const int kind = kind_of(p), layer = p / 5;
                 const FwLayer* L = a.layers + layer;
                 if (kind == FW_ATTN) {
                     bool waited = p == a.p_lo;
                     AttnPos it = a_first;
-                    if (a_n > 0) enter(KV_SLOTS, KV_SLOT);
                     for (int i = 0; i < a_n && ok; attn_step(it, ++i)) {
                         const SeqMeta sm = s.meta[it.bi];
                         const int plane = ((layer * a.max_batch + sm.seq) * 2) * a.Hkv + it.g / nqb;
@@ -897,10 +848,11 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             proxy_fence();
                             waited = true;
                         }
-                        for (int kv = 0; kv < 2 && ok; ++kv, r.next()) {
-                            acquire(KV_BYTES);
+                        for (int kv = 0; kv < 2 && ok; ++kv, ++pos) {
+                            ok = mbar_wait(empty_bar(pos), ring_par(pos) ^ 1u, abort_flag);
                             if (!ok) break;
-                            const uint32_t bar = full_bar(r.pos), dst = slot_ptr(r);
+                            const uint32_t bar = full_bar(pos), dst = slot_ptr(pos);
+                            mbar_expect_tx(bar, KV_BYTES);
 #pragma unroll
                             for (int c = 0; c < NCH; ++c)
 #pragma unroll
@@ -912,7 +864,6 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     continue;
                 }
                 const FwPhase& f = a.ph[kind];
-                if (cta < f.n_tiles) enter(f.ns, f.sz);
                 const CUtensorMap* w = L->w[a.cls];
                 const uint32_t bytes = (uint32_t)(f.nbox * f.box_bytes + f.kb * cols * 128);
                 for (int tile = cta; tile < f.n_tiles && ok; tile += n_cta) {
@@ -936,11 +887,12 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         if (kind == FW_GATEUP) map_acquire(m + 1);
                     }
                     const int k1 = k_end(f, tile);
-                    for (int step = k_first(f, tile); step < k1; ++step, r.next()) {
-                        acquire(bytes);
+                    for (int step = k_first(f, tile); step < k1; ++step, ++pos) {
+                        ok = mbar_wait(empty_bar(pos), ring_par(pos) ^ 1u, abort_flag);
                         if (!ok) break;
-                        const uint32_t bar = full_bar(r.pos), base = slot_ptr(r);
+                        const uint32_t bar = full_bar(pos), base = slot_ptr(pos);
                         const int kx = f.flat ? step * TC_TILE_K : 0, kz = f.flat ? 0 : step * f.kb;
+                        mbar_expect_tx(bar, bytes);
                         if (kind == FW_QKV) {
                             tma_load_4d(base, m, bar, kx, row, half, kz, HINT_STREAM);
                         } else {
@@ -953,33 +905,18 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 }
             }
             if (!ok)       // give the copies in flight a bounded chance to land before the block exits
-                for (int j = max(0, r.pos - FW_BARS); j < r.pos; ++j)
+                for (int j = max(0, pos - NS); j < pos; ++j)
                     for (uint32_t it = 0; it < (1u << 12) && !mbar_test(full_bar(j), ring_par(j)); ++it) __nanosleep(64);
         }
     } else if (warp == 1) {
         // ---------------- operand-row producer: the rows of a phase exist once every block has finished the one before
         if (lane == 0) {
-            Ring r;
+            int pos = 0;
             bool ok = true;
-            auto issued = [&]() -> bool {              // the weight producer has acquired item r.pos
-                const uint32_t limit = (uint32_t)abort_flag[1];
-                for (uint32_t it = 0; it < limit; ++it) {
-                    int v;
-                    asm volatile("ld.acquire.cta.shared.s32 %0, [%1];" : "=r"(v) : "r"(smem_u32(&s.issued)) : "memory");
-                    if (v > r.pos) return true;
-                    if ((it & 31u) == 31u && *abort_flag) return false;
-                }
-                *abort_flag = 1;
-                return false;
-            };
             for (int p = a.p_lo; p < a.p_hi && ok; ++p) {
                 const int kind = kind_of(p);
-                if (kind == FW_ATTN) {
-                    if (a_n > 0) { r.enter(KV_SLOTS, KV_SLOT); r.skip(2 * a_n); }
-                    continue;
-                }
+                if (kind == FW_ATTN) { pos += 2 * a_n; continue; }
                 const FwPhase& f = a.ph[kind];
-                if (cta < f.n_tiles) r.enter(f.ns, f.sz);
                 const CUtensorMap* m = &a.x[kind];
                 if (p > a.p_lo) {
                     ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
@@ -987,10 +924,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 }
                 for (int tile = cta; tile < f.n_tiles && ok; tile += n_cta) {
                     const int k1 = k_end(f, tile);
-                    for (int step = k_first(f, tile); step < k1; ++step, r.next()) {
-                        ok = issued();
+                    for (int step = k_first(f, tile); step < k1; ++step, ++pos) {
+                        ok = mbar_wait(empty_bar(pos), ring_par(pos) ^ 1u, abort_flag);
                         if (!ok) break;
-                        const uint32_t bar = full_bar(r.pos), base = slot_ptr(r) + f.b_off;
+                        const uint32_t bar = full_bar(pos), base = slot_ptr(pos) + f.b_off;
                         if (!a.debug_no_operands)
                             tma_load_3d(base, m, bar, f.flat ? step * TC_TILE_K : 0, 0, f.flat ? 0 : step * f.kb, HINT_KEEP);
                     }
@@ -1004,14 +941,11 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (8u << 24);      // bf16 x bf16 -> fp32, M = 128
         const uint32_t one = elect_one();
         const int me = warp - 2;
-        Ring r;
-        int tcount = 0, at = 0, as = 0;                // projection tiles, attention tiles, segments so far
+        int pos = 0, tcount = 0, at = 0, as = 0;       // ring position, projection tiles, attention tiles, segments so far
         bool ok = true;
         for (int p = a.p_lo; p < a.p_hi && ok; ++p) {
             const int kind = kind_of(p);
             if (kind == FW_ATTN) {
-                if (a_n > 0) r.enter(KV_SLOTS, KV_SLOT);
-                const int pos = r.pos;
                 if (me == 0) {
                     constexpr uint32_t idesc_s = IDESC | ((uint32_t)(NQ2 >> 3) << 17);
                     AttnPos it = a_first;
@@ -1019,26 +953,32 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         const bool fresh = i == 0 || i == a_wrap || it.tile == 0;
                         if (fresh && i > 0) ++as;
                         const int kpos = pos + 2 * i, b = (at + i) & 1;
-                        // Query rows of the segment, the score buffer (read by the softmax two tiles ago), and the K tile.  (An even
-                        // number of barriers: the one of a K tile was a K tile's before, whose arrival this warp has seen.  A
-                        // wait for a parity is only good for who has seen the phase before.)
+                        // Query rows of the segment, the score buffer (read by the softmax two tiles ago), and the K tile.  With an
+                        // odd ring the K tile's slot held the V tile of two tiles ago, whose arrival this warp has not followed:
+                        // the slot's barrier may be a phase behind, and the parity would then name the phase before the one
+                        // meant.  The output of that tile being complete says that the V tile has come and gone.
+                        const uint32_t before = ((uint32_t)((at + i) >> 1) & 1u) ^ 1u;
                         ok = (!fresh || mbar_wait_warp(smem_u32(&s.qfull[as & 1]), (uint32_t)(as >> 1) & 1u, abort_flag)) &&
-                             mbar_wait_warp(smem_u32(&s.pfull[b]), ((uint32_t)((at + i) >> 1) & 1u) ^ 1u, abort_flag) &&
+                             mbar_wait_warp(smem_u32(NS % 2 ? &s.ofull[b] : &s.pfull[b]), before, abort_flag) &&
                              mbar_wait_warp(full_bar(kpos), ring_par(kpos), abort_flag);
                         if (!ok) break;
                         tc_fence_after();
-                        const uint64_t ka = smem_desc(kv_ptr(r.slot + 2 * i)), qa = smem_desc(smem_u32(Qs) + (WIDE ? 0 : as & 1) * Q_BYTES);
+                        const uint64_t ka = smem_desc(slot_ptr(kpos)), qa = smem_desc(smem_u32(Qs) + (WIDE ? 0 : as & 1) * Q_BYTES);
 #pragma unroll
                         for (int ks = 0; ks < HD / 16; ++ks)
                             tc_mma_one(one, tmem + b * TM, ka + (ks >> 2) * (FW_KEYS * 8) + (ks & 3) * 2,
                                        qa + (ks >> 2) * (NQ2 * 8) + (ks & 3) * 2, idesc_s, ks > 0 ? 1u : 0u);
                         tc_commit_one(one, smem_u32(&s.sfull[b]));
-                        if (!WIDE || i < a_n - 2) {
+                        if (!PBK || i < a_n - 2) {
                             tc_commit_one(one, empty_bar(kpos));
                             tc_commit_one(one, empty_bar(kpos));
                         }
                     }
                     if (a_n > 0) ++as;
+                    if (NS % 2 && a_n > 1 && ok) {     // (the next phase's first slot held the last V tile but one)
+                        const int n = at + a_n - 2;
+                        ok = mbar_wait_warp(smem_u32(&s.ofull[n & 1]), (uint32_t)(n >> 1) & 1u, abort_flag);
+                    }
                 } else {
                     constexpr uint32_t idesc_o = IDESC | (1u << 15) | ((uint32_t)(NQ2 >> 3) << 17);
                     for (int i = 0; i < a_n; ++i) {
@@ -1049,9 +989,8 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                              mbar_wait_warp(full_bar(vpos), ring_par(vpos), abort_flag);
                         if (!ok) break;
                         tc_fence_after();
-                        const uint32_t v0 = kv_ptr(r.slot + 2 * i + 1);
-                        const uint64_t va = smem_desc_mn(v0), pa = smem_desc(WIDE ? v0 + KV_BYTES : smem_u32(Ps) + b * P_BYTES);
-                        const uint64_t pb = WIDE ? smem_desc(kv_ptr(r.slot + 2 * i) + KV_BYTES) : pa + NQ2 * 8;       // keys 64 ..
+                        const uint64_t va = smem_desc_mn(slot_ptr(vpos)), pa = smem_desc(WIDE ? slot_ptr(vpos) + KV_BYTES : smem_u32(Ps) + b * P_BYTES);
+                        const uint64_t pb = PBK ? smem_desc(slot_ptr(vpos - 1) + KV_BYTES) : pa + NQ2 * 8;       // keys 64 ..
 #pragma unroll
                         for (int ks = 0; ks < FW_KEYS / 16; ++ks)
                             tc_mma_one(one, tmem + (2 + b) * TM, va + ks * 128, (ks < 4 ? pa : pb) + (ks & 3) * 2,
@@ -1059,18 +998,17 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         tc_commit_one(one, smem_u32(&s.ofull[b]));
                         tc_commit_one(one, empty_bar(vpos));
                         tc_commit_one(one, empty_bar(vpos));
-                        if (WIDE && i >= a_n - 2) {
+                        if (PBK && i >= a_n - 2) {
                             tc_commit_one(one, empty_bar(vpos - 1));
                             tc_commit_one(one, empty_bar(vpos - 1));
                         }
                     }
                 }
                 at += a_n;
-                if (a_n > 0) r.skip(2 * a_n);
+                pos += 2 * a_n;
                 continue;
             }
             const FwPhase& f = a.ph[kind];
-            if (cta < f.n_tiles) r.enter(f.ns, f.sz);
             const int groups = f.kb / f.S, sc = f.S * cols, nbox = f.nbox;      // MMAs along k, accumulator columns of a box
             const bool dual = f.dual != 0;
             const uint32_t idesc = IDESC | ((uint32_t)(sc >> 3) << 17);
@@ -1087,12 +1025,12 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 uint32_t acc = 0;
                 int turn = 0;                              // dual: MMAs along k alternate between the warps
                 const int k1 = k_end(f, tile);
-                for (int step = k_first(f, tile); step < k1; ++step, r.next()) {
-                    ok = mbar_wait_warp(full_bar(r.pos), ring_par(r.pos), abort_flag);
+                for (int step = k_first(f, tile); step < k1; ++step, ++pos) {
+                    ok = mbar_wait_warp(full_bar(pos), ring_par(pos), abort_flag);
                     if (!ok) break;
                     tc_fence_after();
                     if (mine) {
-                        const uint32_t base = slot_ptr(r);
+                        const uint32_t base = slot_ptr(pos);
                         uint64_t ad = smem_desc(base), bd = smem_desc(base + f.b_off);
                         if (nbox == 2) ad += (uint32_t)(me * f.box_bytes) >> 4;
                         for (int gr = 0; gr < groups; ++gr, ad += a_step, bd += b_step) {
@@ -1107,7 +1045,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             }
                         }
                     }
-                    tc_commit_one(one, empty_bar(r.pos));
+                    tc_commit_one(one, empty_bar(pos));
                 }
                 if (ok) tc_commit_one(one, smem_u32(&s.tfull[buf]));
             }
@@ -1119,24 +1057,21 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         const int e = threadIdx.x - 32 * FW_EPI_WARP0;   // 0..255
         const int quad = warp & 3, half = (warp - FW_EPI_WARP0) >> 2;     // TMEM lane quadrant; which of its two warps
         const uint32_t t_lane = tmem + ((uint32_t)(quad * 32) << 16);
-        int tcount = 0, at = 0, as = 0;
-        Ring r;
+        int tcount = 0, at = 0, as = 0, pos = 0;
         bool ok = true;
         auto steps_of = [&](const FwPhase& f) {
             if (cta >= f.n_tiles) return 0;
             return f.c > 1 ? k_end(f, cta) - k_first(f, cta) : ((f.n_tiles - 1 - cta) / n_cta + 1) * f.steps;
         };
+        const int ring_other = steps_of(a.ph[FW_O]) + steps_of(a.ph[FW_GATEUP]) + steps_of(a.ph[FW_DOWN]);
+        const int ring_qkv = steps_of(a.ph[FW_QKV]);
         for (int p = a.p_lo; p < a.p_hi && ok; ++p) {
             const int kind = kind_of(p), layer = p / 5;
-            if (kind != FW_ATTN && cta < a.ph[kind].n_tiles) {
-                r.enter(a.ph[kind].ns, a.ph[kind].sz);
-                r.skip(steps_of(a.ph[kind]));
-            }
             if (kind == FW_ATTN) {
                 if (e == 0 && p > a.p_lo) ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
                 ok = all_of(1, FW_EPI, ok);
                 if (!ok) break;
-                if (a_n > 0) r.enter(KV_SLOTS, KV_SLOT);
+                if (p > a.p_lo) pos += ring_qkv;
                 const int G = a.Hq / a.Hkv, kl = quad * 32 + lane;    // this thread's key of a tile, later its head dimension
                 constexpr int NR = NQP / 2;                           // this thread's query rows: half, half + 2, ...; wide:
                 auto row_of = [&](int x) { return WIDE ? half * NR + x : 2 * x + half; };        // NR neighbouring ones
@@ -1360,8 +1295,8 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             for (int x = 0; x < NR; ++x) sa.sm[half][x] = m[x];
                         bar_n(2 + half, 128);                         // (smx is free again)
                     }
-                    uint8_t* pt = (WIDE ? smem + (r.slot + 2 * i + (kl >= 64 ? 0 : 1)) % KV_SLOTS * KV_SLOT + KV_BYTES
-                                        : Ps + b * P_BYTES + (kl >> 6) * (NQ2 * 128)) + (kl & 7) * 2 + row_of(0) * 128;
+                    uint8_t* pt = (WIDE ? smem + (size_t)((pos + 2 * i + (PBK && kl >= 64 ? 0 : 1)) % NS) * FW_SLOT + KV_BYTES : Ps + b * P_BYTES) +
+                                  (PBK ? 0 : kl >> 6) * (NQ2 * 128) + (kl & 7) * 2 + row_of(0) * 128;
                     constexpr int RS = WIDE ? 128 : 256;              // bytes between this thread's rows
                     const int pc = (kl & 63) >> 3;
 #pragma unroll
@@ -1376,10 +1311,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     }
                     if ((it.tile + 1) * FW_KEYS > nkeys) {
                         // rows of V past the last key: their probabilities are 0, but 0 x (stale value) must not make a NaN
-                        const int vpos = r.pos + 2 * i + 1;
+                        const int vpos = pos + 2 * i + 1;
                         ok = warp_wait(full_bar(vpos), ring_par(vpos), abort_flag, ok, lane);
                         if (ok && j >= nkeys) {
-                            uint8_t* vs = smem + (r.slot + 2 * i + 1) % KV_SLOTS * KV_SLOT + kl * 128 + half * 64;
+                            uint8_t* vs = smem + (size_t)(vpos % NS) * FW_SLOT + kl * 128 + half * 64;
 #pragma unroll
                             for (int c = 0; c < NCH * 4; ++c)
                                 *reinterpret_cast<uint4*>(vs + (c >> 2) * (FW_KEYS * 128) + (c & 3) * 16) = make_uint4(0u, 0u, 0u, 0u);
@@ -1401,7 +1336,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     output(at - 1);
                     finish(it);
                 }
-                if (a_n > 0) r.skip(2 * a_n);
+                pos += 2 * a_n + ring_other;
                 ok = all_of(1, FW_EPI, ok);
                 if (!ok) break;
                 // pieces shared with other blocks (at most the first and the last of this block's range): who arrives last merges
@@ -1466,7 +1401,7 @@ int up8(int x) { return (x + 7) / 8 * 8; }
 
 void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta, int cls) {
     const int qd = d.n_q_heads * d.head_dim, hp = d.head_dim / 2, heads = d.n_q_heads + 2 * d.n_kv_heads;
-    const int cols = FW_CLASS[cls];
+    const int cols = FW_CLASS[cls].cols, slot = FW_RING / FW_CLASS[cls].slots;
     for (int k = 0; k < 6; ++k) ph[k].c = ph[k].u = 1;
     // rows of a matrix: one tile per SM, in whole groups of eight rows (swizzle atoms)
     auto rows = [&](FwPhase& f, int N, int K, int nbox, int cut) {
@@ -1514,20 +1449,12 @@ void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta, int cls) {
     for (int k = 0; k < 6; ++k) {
         if (k == FW_ATTN) continue;
         FwPhase& f = ph[k];
-        // k-blocks of a step: as many bytes in flight as the ring holds, in three slots at least; rows of one k-block (128
-        // bytes) pass slower than longer ones, and a step takes its producer 0.3 us, which small ones do not last; a multiple of
-        // the k-blocks that the MMA can take side by side
-        const int S = std::min(TC_TILE_N / f.hr, FW_ACC / (cols * f.nbox)), one = (f.nbox * f.hr + cols) * 128;
-        double best = 0;
-        f.kb = 1;
-        for (int kb = f.K % TC_TILE_K ? 1 : std::min(f.k_blocks, 16); kb >= 1; --kb) {
-            const int ns = std::min(FW_SLOTS, FW_RING / (kb * one));
-            if (ns < 3 || (S > 1 && kb > S && kb % S)) continue;
-            const double flight = (double)ns * kb * one * (kb == 1 ? 0.85 : kb * one < 40 * 1024 ? 0.93 : 1.0) * (ns == 3 ? 0.97 : 1.0);
-            if (flight > best) { best = flight; f.kb = kb; }
-        }
-        f.sz = f.kb * one;
-        f.ns = std::min(FW_SLOTS, FW_RING / f.sz);
+        int kb = slot / ((f.nbox * f.hr + cols) * 128);
+        kb = std::min(std::min(kb, f.k_blocks), 16);
+        // a multiple of the k-blocks that the MMA can take side by side
+        const int S = std::min(TC_TILE_N / f.hr, FW_ACC / (cols * f.nbox));
+        if (S > 1 && kb > S) kb -= kb % S;
+        f.kb = (f.K % TC_TILE_K || kb < 1) ? 1 : kb;
         f.flat = tc_kb_flat(f.K, f.kb) ? 1 : 0;
         f.steps = up_div(f.k_blocks, f.kb);
         f.box_bytes = f.hr * 128 * f.kb;
@@ -1546,8 +1473,8 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
     const bool wide = G * R > FW_QROWS;
     a.nqb = wide ? up_div(G * R, FW_QROWS_WIDE) : 1;
     a.qrows = up_div(G * R, a.nqb);
-    a.cls = T <= 8 && !wide ? 0 : 2;                       // (the lean epilogues: up to eight rows)
-    while (FW_CLASS[a.cls] < a.cols) ++a.cls;
+    a.cls = T <= 8 && !wide ? 0 : 2;                       // (four slots and the lean epilogues: up to eight rows)
+    while (FW_CLASS[a.cls].cols < a.cols) ++a.cls;
     fw_geometry(a.ph, d, n_cta, a.cls);
     a.n_cta = n_cta; a.n_layers = d.layers;
     a.p_lo = 0; a.p_hi = 5 * d.layers + 1;
@@ -1558,7 +1485,7 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
         f.S = 1;
         for (int S = 2; S <= f.kb; ++S)
             if (f.kb % S == 0 && S * f.hr <= TC_TILE_N && S * a.cols * f.nbox <= FW_ACC) f.S = S;
-        if (f.ns < 2 || f.b_off + f.kb * a.cols * 128 > f.sz || f.nbox * f.S * a.cols > FW_ACC_ONE) return false;
+        if (f.b_off + f.kb * a.cols * 128 > FW_RING / FW_CLASS[a.cls].slots || f.nbox * f.S * a.cols > FW_ACC_ONE) return false;
         f.both = f.nbox * f.S * a.cols > FW_ACC ? 1 : 0;
         if ((k == FW_O || k == FW_DOWN) && (f.n_tiles > n_cta || f.steps < f.c)) return false;
         // one box: the MMAs along k alternate between two accumulators where they fit and every block has two
@@ -1616,13 +1543,20 @@ cudaError_t launch_forward(const FwArgs& a, cudaStream_t st) {
         cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, kernel, a);
     };
-    // instantiations: head size, query rows of an attention item, few rows in all
+    // instantiations: head size, query rows of an attention item, few rows in all, ring slots
     auto pick = [&](auto hd) -> cudaError_t {
         constexpr int HD = decltype(hd)::value;
         const int n_q = (a.Hq / a.Hkv) * a.R;
-        if (a.cls < 2) return n_q <= 8 ? go(forward_kernel<HD, 8, true>) : go(forward_kernel<HD, FW_QROWS, true>);
-        if (n_q <= 8) return go(forward_kernel<HD, 8, false>);
-        return n_q <= FW_QROWS ? go(forward_kernel<HD, FW_QROWS, false>) : go(forward_kernel<HD, FW_QROWS_WIDE, false>);
+        auto rows = [&](auto few, auto slots) -> cudaError_t {
+            constexpr bool FEW = decltype(few)::value;
+            constexpr int NS = decltype(slots)::value;
+            if (n_q <= 8) return go(forward_kernel<HD, 8, FEW, NS>);
+            if (FEW || n_q <= FW_QROWS) return go(forward_kernel<HD, FW_QROWS, FEW, NS>);
+            return go(forward_kernel<HD, FEW ? FW_QROWS : FW_QROWS_WIDE, FEW, NS>);
+        };
+        using std::integral_constant;
+        if (a.cls < 2) return rows(std::true_type{}, integral_constant<int, 4>{});
+        return FW_CLASS[a.cls].slots == 3 ? rows(std::false_type{}, integral_constant<int, 3>{}) : rows(std::false_type{}, integral_constant<int, 4>{});
     };
     return a.hd == 128 ? pick(std::integral_constant<int, 128>{}) : pick(std::integral_constant<int, 64>{});
 }

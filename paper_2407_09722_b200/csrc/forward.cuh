@@ -5,8 +5,8 @@
 
 namespace mtad {
 
-constexpr int FW_RING = 192 * 1024;       // the copy ring, cut into slots as large as one step of a projection, or 128 keys
-                                          // of K or V
+constexpr int FW_RING = 192 * 1024;       // the copy ring: four slots, or three where the operand rows are many; a slot
+                                          // holds one step of a projection, or 128 keys of K or V
 constexpr int FW_KEYS = 128;              // keys of an attention tile
 constexpr int FW_MAX_ROWS = 72;           // rows of a call
 constexpr int FW_MAX_COLS = 144;          // operand rows (terms x rows) of a call
@@ -16,17 +16,17 @@ constexpr int FW_QROWS_WIDE = 40;         // or in the wide variant: more are cu
 // Tile geometry of one projection.  A step brings nbox boxes of hr weight rows x kb k-blocks (one copy each) and one box of
 // operand rows.  nbox = 1: the rows of h features (QKV: of h rotary pairs of a head, hr = 2 h); nbox = 2: h gate rows and
 // the h matching up rows, or 2 h rows of the LM head.  The geometry depends on the matrix, the SM count and the class of
-// the call's operand rows, so that the weight maps are encoded once per model.
+// the call's operand rows, so that the weight maps are encoded once per model: kb is the most that a ring slot holds.
 // Big boxes matter twice: a thread issues a copy about every quarter of a microsecond whatever its size, and rows of 256
 // bytes and more pass at 70 GB/s per SM where rows of 128 bytes pass at 43.
 constexpr int FW_CLASSES = 6;
-constexpr int FW_CLASS[FW_CLASSES] = {16, 32, 64, 80, 112, FW_MAX_COLS};      // operand rows up to
+struct FwClass { int cols, slots; };      // operand rows up to, ring slots
+constexpr FwClass FW_CLASS[FW_CLASSES] = {{16, 4}, {32, 4}, {64, 4}, {80, 3}, {112, 3}, {FW_MAX_COLS, 4}};
 struct FwPhase {
     int h, hr, nbox, n_tiles, u;          // u: tiles per head (QKV)
     int c;                                // O, down: blocks that share a tile's k-range (their partial sums meet in global memory)
     int kb, flat, S, steps;               // k-blocks of a box, its map's view, k-blocks side by side in the MMA, steps of all k-blocks
     int box_bytes, b_off;                 // bytes of one weight box, offset of the operand rows in the slot
-    int sz, ns;                           // bytes of a slot, slots of the ring
     int k_blocks, K;
     int dual, both, blk;                  // two accumulators for one box; a tile takes both accumulator buffers; rows that the
                                           // epilogue takes at a time
