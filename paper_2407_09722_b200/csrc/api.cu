@@ -19,7 +19,6 @@ using namespace mtad;
 // per tensor-memory accumulator, the pieces being added in fp32 (relative error about 4e-7 instead of 4e-6 at K = 8192)
 static const int kQkvSegCap = 8;
 static const int kCtas = 148;   // SMs the tensor-core GEMM spreads over
-static const bool kOneLaunchForward = true;
 
 // Host-side tensor maps of one model's weight matrices.
 struct WeightMaps {                      // index 0, 1, 2: tiles of 128, 256, 512 rows (1, 2, 4 halves)
@@ -844,7 +843,7 @@ int mtad_create(const mtad_model_desc* target, const mtad_model_desc* aux, int m
         if (e == cudaSuccess) e = cudaMemset(ctx->ws_base + r.off + r.count * r.elem, 0xC5, kCanaryBytes);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) { delete ctx; return MTAD_E_CUDA; }
-    if (ctx->use_tc && kOneLaunchForward) {
+    if (ctx->use_tc) {
         ctx->fw_ok[0] = ctx->target.kv_map_ok && build_forward_table(ctx->target, ctx->fw_target, ctx->fw_lm[0]);
         ctx->fw_ok[1] = aux && ctx->amaps.ok && ctx->aux.kv_map_ok && build_forward_table(ctx->aux, ctx->fw_aux, ctx->fw_lm[1]);
     }
@@ -1172,7 +1171,7 @@ void audit_forward(Audit& au, const mtad_ctx& c, const ModelView& m, int B, int 
     au.ws("xd", idx_xrow(T - 1, terms, terms - 1, d.d_model, d.d_model - 1) + 1);
     au.ws("sumsq_a", T);
     ForwardPlan fp;
-    if (kOneLaunchForward && build_forward_plan(fp, c.sc, c.rm, m, nullptr, nullptr, B, R, lm_plain, false)) {
+    if (build_forward_plan(fp, c.sc, c.rm, m, nullptr, nullptr, B, R, lm_plain, false)) {
         // the one-launch forward: what its epilogues and its attention index
         const FwArgs& a = fp.fw;
         const long long cap = d.kv_capacity, total = std::min<long long>(len_ub, cap) + R;

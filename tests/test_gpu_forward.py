@@ -1,0 +1,62 @@
+"""The one-launch decoder forward at the edges of its variants: row counts where the operand class, the epilogue or the
+number of bf16 terms changes, key counts around its 128-key tiles, query rows per KV head around the sizes of an
+attention item, split and unsplit projections, and one call beyond its rows whose attention alone it forms.  Compared
+with the CPU oracle; the tolerances are derived in parity.py."""
+import pytest
+
+import mtad_synth as S
+from paper_2407_09722_b200 import binding as Bn
+from tests.parity import GpuModel, SeqCase, ParityStats, compare, gemm_eps
+
+pytestmark = pytest.mark.gpu
+
+# layers, d_model, query heads, KV heads, head_dim, d_ffn, vocab
+SHAPES = {
+    "hd64": S.ModelShape(2, 1024, 16, 16, 64, 4096, 1000),       # down is split over four blocks from nine rows on
+    "gqa128": S.ModelShape(2, 512, 8, 2, 128, 1024, 640),        # four query rows per row of a call
+    "odd": S.ModelShape(3, 320, 5, 5, 64, 1000, 777),            # neither features nor k-blocks divide evenly
+}
+
+
+@pytest.fixture(scope="module")
+def models():
+    made = {}
+
+    def get(name):
+        if name not in made:
+            made.clear()                                         # one at a time on the device
+            made[name] = GpuModel(SHAPES[name], max_batch=8, max_nodes=80, capacity=420)
+        return made[name]
+
+    return get
+
+
+@pytest.mark.parametrize("shape,rows,tree,lengths", [
+    ("hd64", 1, None, [127]),
+    ("hd64", 8, None, [128]),
+    ("hd64", 9, None, [120]),
+    ("hd64", 8, None, [0, 127, 128, 300]),
+    ("hd64", 33, (4, 8, 4), [250]),
+    ("hd64", 7, None, [1, 60, 121, 122, 129, 200, 256, 333]),
+    ("hd64", 57, (7, 8, 4), [100]),
+    ("hd64", 9, None, [0, 5, 119, 120, 128, 247, 300, 384]),
+    ("gqa128", 4, None, [129]),
+    ("gqa128", 5, None, [255]),
+    ("gqa128", 65, (8, 8, 2), [130]),
+    ("gqa128", 73, (9, 8, 4), [128]),
+    ("odd", 6, None, [64, 65]),
+    ("odd", 33, (4, 8, 2), [64]),
+])
+def test_forward_edges(models, shape, rows, tree, lengths):
+    gm, sh = models(shape), SHAPES[shape]
+    B, stats = len(lengths), ParityStats()
+    cases = []
+    for b, L in enumerate(lengths):
+        gm.inject(b, L)
+        t = S.beam_tree(*tree, sh.vocab, stream=70 + b) if tree else S.chain_tree(rows - 1, sh.vocab, stream=50 + b)
+        assert len(t.tok) == rows - 1
+        cases.append(SeqCase(b, L, int(S.token_ids(9, (21 << 40) | b, 1, sh.vocab)[0]), t))
+    u = S.bonus_uniforms(9, rows, B, sh.vocab, "cuda")
+    compare(gm, cases, Bn.log_tau(0.3), u, chain=tree is None, stats=stats)
+    assert stats.ok(), stats
+    assert stats.cache_ok(sh.layers, gemm_eps(B * rows, max(sh.d_ffn, sh.d_model)))
