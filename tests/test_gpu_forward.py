@@ -59,4 +59,11 @@ def test_forward_edges(models, shape, rows, tree, lengths):
     u = S.bonus_uniforms(9, rows, B, sh.vocab, "cuda")
     compare(gm, cases, Bn.log_tau(0.3), u, chain=tree is None, stats=stats)
     assert stats.ok(), stats
-    assert stats.cache_ok(sh.layers, gemm_eps(B * rows, max(sh.d_ffn, sh.d_model)))
+    flips = 1.0 - stats.cache_exact / stats.cache_rows
+    if min(lengths) >= 60:
+        assert stats.cache_ok(sh.layers, gemm_eps(B * rows, max(sh.d_ffn, sh.d_model)))
+    else:
+        # A row with next to no committed keys attends to this call's own: where their values rounded the other way (a
+        # bf16 step, at most 2^-8 of the value, in a share `flips` of the elements), its output moves by 2^-9 sqrt(flips)
+        # of the largest value in the mean square, and by four times that at most.  cache_ok leaves this out.
+        assert flips <= 0.1 and stats.cache_max_excess <= 2.0 ** -7 * flips ** 0.5 * stats.cache_scale
