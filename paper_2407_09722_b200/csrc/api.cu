@@ -256,7 +256,7 @@ size_t carve(mtad_ctx* c, const mtad_model_desc* t, const mtad_model_desc* a, in
                                 "lm_part");
     sc.fw_sync_words = (int)mx([&](const mtad_model_desc* m) { return fw_sync_words(*m, max_batch, kCtas); });
     sc.fw_sync = k.take<int32_t>(sc.fw_sync_words, "fw_sync");
-    sc.fw_part = k.take<float>((size_t)kCtas * FW_MAX_ROWS * TC_TILE_N, "fw_part");
+    sc.fw_part = k.take<float>((size_t)kCtas * FW_MAX_ROWS * 2 * TC_TILE_N, "fw_part");
     FwLayer* fw_t = k.take<FwLayer>(t->layers, "fw_target");
     FwLayer* fw_a = a ? k.take<FwLayer>(a->layers, "fw_aux") : nullptr;
     sc.node_z = k.take<float>(T, "node_z");
@@ -1185,8 +1185,8 @@ void audit_forward(Audit& au, const mtad_ctx& c, const ModelView& m, int B, int 
         au.ws("xf", idx_xrow(T - 1, terms, terms - 1, d.d_ffn, d.d_ffn - 1) + 1);
         au.ws("attn_part", (size_t)T * Hq * pieces * (hd + 2));
         au.ws("fw_sync", fw_sync_words(d, m.max_batch, kCtas));
-        for (const FwPhase* f : {&a.ph[FW_O], &a.ph[FW_DOWN]})
-            if (f->c > 1) au.ws("fw_part", (size_t)f->n_tiles * T * f->S * f->hr);
+        for (const FwPhase* f : {&a.ph[FW_QKV], &a.ph[FW_O], &a.ph[FW_DOWN]})
+            if (f->c > 1) au.ws("fw_part", (size_t)f->n_tiles * T * f->nbox * f->S * f->hr);
         au.ws(&m == &c.target ? "fw_target" : "fw_aux", d.layers);
         if (lm_plain) au.ws("logits", (size_t)T * d.vocab);
         else au.ws("lm_part", idx_lm_part(T - 1, a.ph[FW_LM].n_tiles, a.ph[FW_LM].n_tiles - 1) + 1);

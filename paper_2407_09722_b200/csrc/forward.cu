@@ -297,6 +297,90 @@ __device__ __forceinline__ bool split_residual(const FwArgs& a, FwTail& s, const
     return true;
 }
 
+// QKV where c blocks share the k-range of a tile of two heads (128 rows each): the same exchange, then a warp per row, four
+// rotary pairs of a head a lane.
+template <int HD>
+__device__ __forceinline__ bool split_qkv(const FwArgs& a, FwTail& s, const FwPhase& f, int layer, int tcount, int e,
+                                          uint32_t tmem_lane, int tile) {
+    volatile int* abort_flag = s.abort_flag;
+    constexpr int hp = HD / 2;
+    const int lane = e & 31, w = e >> 5, quad = w & 3, half = w >> 2;
+    const int T = a.T, terms = a.terms, cols = a.cols, c = f.c, buf = tcount & 1, per = terms == 3 ? 5 : 8;
+    const int kp = tile % c, ra = T * kp / c, rn = T * (kp + 1) / c;
+    bool ok = true;
+    if (e == 0) ok = mbar_wait(smem_u32(&s.tfull[buf]), (uint32_t)(tcount >> 1) & 1u, abort_flag);
+    ok = all_of(1, FW_EPI, ok);
+    if (!ok) return false;
+    tc_fence_after();
+    const uint32_t t_acc = tmem_lane + (f.both ? 0 : buf * 256) + half * cols;     // the two warps of a quadrant: a head each
+    float* y = a.kpart + (size_t)tile * T * 256 + half * 128 + quad * 32 + lane;
+    for (int rb = 0; rb < T; rb += per) {
+        float v[16];
+        tc_ld16(t_acc + rb * terms, v);
+        if (terms == 3) {
+#pragma unroll
+            for (int j = 0; j < 5; ++j, y += 256)
+                if (rb + j < T) __stcg(y, v[3 * j] + (v[3 * j + 1] + v[3 * j + 2]));
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j, y += 256)
+                if (rb + j < T) __stcg(y, v[2 * j] + v[2 * j + 1]);
+        }
+        __syncwarp();
+    }
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(&s.tempty[buf]));
+    bar_n(1, FW_EPI);
+    if (e == 0) {
+        int32_t* cnt = a.kcnt + 2 * a.n_cta + tile / c;
+        asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(cnt) : "memory");
+        ok = grid_wait(cnt, c * (layer + 1), abort_flag);
+    }
+    ok = all_of(1, FW_EPI, ok);
+    if (!ok) return false;
+    const int box = lane >> 4, j = (lane & 15) * 4, hg = tile / c * 2 + box, heads = a.Hq + 2 * a.Hkv;
+    const bool rot = hg < a.Hq + a.Hkv;
+    const float scale = rsqrtf((float)HD) * 1.4426950408889634f;
+    const float* parts = a.kpart + (size_t)(tile / c * c) * T * 256 + box * 128 + j;
+#pragma unroll 2
+    for (int t = ra + w; t < rn; t += 8) {
+        const int sl = s.slot[t];
+        if (j >= hp || hg >= heads || sl < 0) continue;
+        float va[4] = {0.f, 0.f, 0.f, 0.f}, vb[4] = {0.f, 0.f, 0.f, 0.f}, cs[8];
+        const float* rp = a.rope + ((size_t)t * hp + j) * 2;
+        *reinterpret_cast<float4*>(cs) = *reinterpret_cast<const float4*>(rp);
+        *reinterpret_cast<float4*>(cs + 4) = *reinterpret_cast<const float4*>(rp + 4);
+#pragma unroll 4
+        for (int k = 0; k < c; ++k) {
+            const float* p = parts + ((size_t)k * T + t) * 256;
+            const float4 x = __ldcg(reinterpret_cast<const float4*>(p)), z = __ldcg(reinterpret_cast<const float4*>(p + hp));
+            va[0] += x.x; va[1] += x.y; va[2] += x.z; va[3] += x.w;
+            vb[0] += z.x; vb[1] += z.y; vb[2] += z.z; vb[3] += z.w;
+        }
+        const float rs = s.rstd[t];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            const float ya = va[x] * rs, yb = vb[x] * rs;
+            va[x] = rot ? ya * cs[2 * x] - yb * cs[2 * x + 1] : ya;
+            vb[x] = rot ? yb * cs[2 * x] + ya * cs[2 * x + 1] : yb;
+        }
+        if (hg < a.Hq) {
+            const size_t o = ((size_t)t * a.Hq + hg) * HD + j;
+            split_store4(va, scale, a.q_hi + o, a.q_lo + o);
+            split_store4(vb, scale, a.q_hi + o + hp, a.q_lo + o + hp);
+        } else {
+            const int sq = s.meta[s.rowb[t]].seq, kv = rot ? 0 : 1;
+            if (sl < a.cap && (unsigned)sq < (unsigned)a.max_batch) {                  // never past the cache
+                __nv_bfloat16* d = a.cache + idx_cache(layer, a.max_batch, sq, kv, a.Hkv, hg - a.Hq - kv * a.Hkv, a.cap, sl, HD) + j;
+                store_bf4(va, d);
+                store_bf4(vb, d + hp);
+            }
+        }
+    }
+    return true;
+}
+
 // The epilogue group's part of one projection: row statistics, then per tile the accumulators -> Y in shared memory ->
 // the fused epilogue.  KIND is a template parameter so that the phase's geometry is read straight from the launch
 // parameters; index arithmetic and global loads stand ahead of the wait for the accumulator, because everything after it
@@ -355,6 +439,12 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
         ++tcount;
         return ok;
     }
+    if constexpr (!FEW && KIND == FW_QKV && HD == 128)
+        if (f.c > 1) {
+            ok = split_qkv<HD>(a, s, f, layer, tcount, e, tmem_lane, cta);
+            ++tcount;
+            return ok;
+        }
     for (int tile = cta; tile < f.n_tiles; tile += n_cta, ++tcount) {
         const int buf = tcount & 1, f0 = tile * nf;        // f0: first feature (O, down, gate / up, LM head)
         // ---- what the first items need besides the accumulator
@@ -870,11 +960,21 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     // the tile's first box: map, row coordinate (QKV: pair and half-head coordinates)
                     const CUtensorMap* m = w;
                     int row = tile * f.nbox * f.h, half = 0;
-                    if (kind == FW_QKV) {
+                    const CUtensorMap* m2 = m;         // QKV, a tile of two heads: the second
+                    int half2 = 0;
+                    auto of_head = [&](int hg, const CUtensorMap*& map, int& pos2) {
+                        pos2 = 2 * (hg < a.Hq ? hg : (hg < a.Hq + a.Hkv ? hg - a.Hq : hg - a.Hq - a.Hkv));
+                        map = w + (hg < a.Hq ? 0 : (hg < a.Hq + a.Hkv ? 1 : 2));
+                    };
+                    if (kind == FW_QKV && f.nbox == 2) {
+                        const int hg = tile / f.c * 2;
+                        row = 0;
+                        of_head(hg, m, half);
+                        of_head(min(hg + 1, a.Hq + 2 * a.Hkv - 1), m2, half2);
+                    } else if (kind == FW_QKV) {
                         const int hg = tile / f.u;
                         row = (tile - hg * f.u) * f.h;
-                        half = 2 * (hg < a.Hq ? hg : (hg < a.Hq + a.Hkv ? hg - a.Hq : hg - a.Hq - a.Hkv));
-                        m = w + (hg < a.Hq ? 0 : (hg < a.Hq + a.Hkv ? 1 : 2));
+                        of_head(hg, m, half);
                     } else if (kind == FW_GATEUP) {
                         m = w + 4;
                         row = tile * f.h;
@@ -885,6 +985,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     if (kind != FW_LM) {
                         map_acquire(m);
                         if (kind == FW_GATEUP) map_acquire(m + 1);
+                        if (kind == FW_QKV && f.nbox == 2) map_acquire(m2);
                     }
                     const int k1 = k_end(f, tile);
                     for (int step = k_first(f, tile); step < k1; ++step, ++pos) {
@@ -895,6 +996,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         mbar_expect_tx(bar, bytes);
                         if (kind == FW_QKV) {
                             tma_load_4d(base, m, bar, kx, row, half, kz, HINT_STREAM);
+                            if (f.nbox == 2) tma_load_4d(base + f.box_bytes, m2, bar, kx, row, half2, kz, HINT_STREAM);
                         } else {
                             tma_load_3d(base, m, bar, kx, row, kz, HINT_STREAM);
                             if (f.nbox == 2)
@@ -1399,9 +1501,15 @@ int up8(int x) { return (x + 7) / 8 * 8; }
 
 }  // namespace
 
+// Ring slots: those of the class, or four where steps are few (auxiliary model of width 1024, eight sequences of four beams:
+// six draft steps 1147 us with three, 1120 with four) and a step of two boxes of 128 rows fits.
+static int fw_slots(const mtad_model_desc& d, int cls) {
+    return d.d_model <= 2048 && (256 + FW_CLASS[cls].cols) * 128 <= FW_RING / 4 ? 4 : FW_CLASS[cls].slots;
+}
+
 void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta, int cls) {
     const int qd = d.n_q_heads * d.head_dim, hp = d.head_dim / 2, heads = d.n_q_heads + 2 * d.n_kv_heads;
-    const int cols = FW_CLASS[cls].cols, slot = FW_RING / FW_CLASS[cls].slots;
+    const int cols = FW_CLASS[cls].cols, slot = FW_RING / fw_slots(d, cls);
     for (int k = 0; k < 6; ++k) ph[k].c = ph[k].u = 1;
     // rows of a matrix: one tile per SM, in whole groups of eight rows (swizzle atoms)
     auto rows = [&](FwPhase& f, int N, int K, int nbox, int cut) {
@@ -1446,6 +1554,23 @@ void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta, int cls) {
     q.n_tiles = heads * q.u;
     q.K = d.d_model;
     q.k_blocks = up_div(q.K, TC_TILE_K);
+    // The same split for QKV, two heads of 128 on a tile: it meets the operand rows half as often and spreads over all SMs
+    // (7B, 32 heads: 96 tiles of one head leave a third of them idle), at about 4.5 us for the exchange.
+    if (d.head_dim == 128 && q.u == 1 && cls >= 2) {
+        const double floor_us = 2.0 * heads * 128 * q.K / 6.5e6;
+        double best = std::max((128.0 + cols) * 128.0 * q.k_blocks / 85e3, floor_us) - 2.0;
+        for (int c = 2; c <= 4; ++c) {
+            const int tiles = up_div(heads, 2) * c;
+            if (tiles > n_cta || q.k_blocks < 8 * c || (256 + cols) * 128 > slot) break;
+            const double us = std::max((256.0 + cols) * 128.0 * up_div(q.k_blocks, c) / 85e3, floor_us) + 4.5;
+            if (us < best) {
+                best = us;
+                q.c = c;
+                q.nbox = 2;
+                q.n_tiles = tiles;
+            }
+        }
+    }
     for (int k = 0; k < 6; ++k) {
         if (k == FW_ATTN) continue;
         FwPhase& f = ph[k];
@@ -1475,6 +1600,7 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
     a.qrows = up_div(G * R, a.nqb);
     a.cls = T <= 8 && !wide ? 0 : 2;                       // (four slots and the lean epilogues: up to eight rows)
     while (FW_CLASS[a.cls].cols < a.cols) ++a.cls;
+    a.slots = fw_slots(d, a.cls);
     fw_geometry(a.ph, d, n_cta, a.cls);
     a.n_cta = n_cta; a.n_layers = d.layers;
     a.p_lo = 0; a.p_hi = 5 * d.layers + 1;
@@ -1485,9 +1611,9 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
         f.S = 1;
         for (int S = 2; S <= f.kb; ++S)
             if (f.kb % S == 0 && S * f.hr <= TC_TILE_N && S * a.cols * f.nbox <= FW_ACC) f.S = S;
-        if (f.b_off + f.kb * a.cols * 128 > FW_RING / FW_CLASS[a.cls].slots || f.nbox * f.S * a.cols > FW_ACC_ONE) return false;
+        if (f.b_off + f.kb * a.cols * 128 > FW_RING / a.slots || f.nbox * f.S * a.cols > FW_ACC_ONE) return false;
         f.both = f.nbox * f.S * a.cols > FW_ACC ? 1 : 0;
-        if ((k == FW_O || k == FW_DOWN) && (f.n_tiles > n_cta || f.steps < f.c)) return false;
+        if ((k == FW_O || k == FW_DOWN || f.c > 1) && (f.n_tiles > n_cta || f.steps < f.c)) return false;
         // one box: the MMAs along k alternate between two accumulators where they fit and every block has two
         f.dual = f.nbox == 1 && 2 * f.S * a.cols <= FW_ACC && f.steps / f.c * (f.kb / f.S) >= 2 ? 1 : 0;
         const int per = a.terms == 3 ? 5 : 16;             // rows of one drain load
@@ -1501,7 +1627,7 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
 bool fw_attn_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
     const int G = d.n_q_heads / d.n_kv_heads;
     if ((d.head_dim != 64 && d.head_dim != 128) || G * R <= FW_QROWS || B * R > TC_MAX_ROWS || B > MTAD_MAX_BATCH) return false;
-    a.T = B * R; a.B = B; a.R = R; a.terms = tc_terms(a.T); a.cls = FW_CLASSES - 1;
+    a.T = B * R; a.B = B; a.R = R; a.terms = tc_terms(a.T); a.cls = FW_CLASSES - 1; a.slots = 4;
     a.nqb = up_div(G * R, FW_QROWS_WIDE);
     a.qrows = up_div(G * R, a.nqb);
     a.n_cta = n_cta; a.n_layers = d.layers;
@@ -1556,7 +1682,7 @@ cudaError_t launch_forward(const FwArgs& a, cudaStream_t st) {
         };
         using std::integral_constant;
         if (a.cls < 2) return rows(std::true_type{}, integral_constant<int, 4>{});
-        return FW_CLASS[a.cls].slots == 3 ? rows(std::false_type{}, integral_constant<int, 3>{}) : rows(std::false_type{}, integral_constant<int, 4>{});
+        return a.slots == 3 ? rows(std::false_type{}, integral_constant<int, 3>{}) : rows(std::false_type{}, integral_constant<int, 4>{});
     };
     return a.hd == 128 ? pick(std::integral_constant<int, 128>{}) : pick(std::integral_constant<int, 64>{});
 }

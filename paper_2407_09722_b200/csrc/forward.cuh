@@ -21,10 +21,11 @@ constexpr int FW_QROWS_WIDE = 40;         // or in the wide variant: more are cu
 // bytes and more pass at 70 GB/s per SM where rows of 128 bytes pass at 43.
 constexpr int FW_CLASSES = 6;
 struct FwClass { int cols, slots; };      // operand rows up to, ring slots
-constexpr FwClass FW_CLASS[FW_CLASSES] = {{16, 4}, {32, 4}, {64, 4}, {80, 3}, {112, 3}, {FW_MAX_COLS, 4}};
+constexpr FwClass FW_CLASS[FW_CLASSES] = {{16, 4}, {32, 4}, {64, 4}, {80, 3}, {112, 3}, {FW_MAX_COLS, 3}};
 struct FwPhase {
     int h, hr, nbox, n_tiles, u;          // u: tiles per head (QKV)
-    int c;                                // O, down: blocks that share a tile's k-range (their partial sums meet in global memory)
+    int c;                                // blocks that share a tile's k-range (their partial sums meet in global memory): O, down,
+                                          // and QKV, where a tile then is two heads
     int kb, flat, S, steps;               // k-blocks of a box, its map's view, k-blocks side by side in the MMA, steps of all k-blocks
     int box_bytes, b_off;                 // bytes of one weight box, offset of the operand rows in the slot
     int k_blocks, K;
@@ -40,7 +41,7 @@ struct alignas(64) FwLayer {              // device table, one entry per layer
 
 struct FwArgs {
     CUtensorMap x[6], lm, kv;             // operand rows by kind
-    int cls;
+    int cls, slots;                       // class of the operand rows, ring slots
     FwPhase ph[6];                        // by kind; the entry of the attention is unused
     const FwLayer* layers;
     int n_layers, n_cta;
@@ -52,7 +53,7 @@ struct FwArgs {
     long long cap;
     float inv_dim, eps;
     int32_t *sync, *acnt;                 // phase counters, arrival counters of the attention's (sequence, KV head, query block)s
-    int32_t* kcnt;                        // arrivals at the split tiles of O, then of down
+    int32_t* kcnt;                        // arrivals at the split tiles of O, of down, of QKV
     float* kpart;                         // their partial sums [block][row][feature]
     float *sumsq_a, *sumsq_b, *hidden;
     __nv_bfloat16 *x_d, *x_a, *x_f, *q_hi, *q_lo, *cache;
@@ -83,7 +84,7 @@ inline size_t fw_pairs(const mtad_model_desc& d, int max_batch) {
 }
 // words of the phase and arrival counters (zeroed by the row preparation of every call)
 inline size_t fw_sync_words(const mtad_model_desc& d, int max_batch, int n_cta) {
-    return (size_t)5 * d.layers + 1 + fw_pairs(d, max_batch) + 2 * (size_t)n_cta;
+    return (size_t)5 * d.layers + 1 + fw_pairs(d, max_batch) + 3 * (size_t)n_cta;
 }
 cudaError_t launch_forward(const FwArgs& a, cudaStream_t st);
 cudaError_t launch_forward_attention(FwArgs& a, int layer, cudaStream_t st);
