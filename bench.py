@@ -501,9 +501,10 @@ def run_ours(args, w: S.Workload, rank: int, world: int, local_rank: int):
     final_lens = [ctx.mtad_seq_get(b)[0] for b in seqs]
 
     # ---- per-kernel passes: the same steps again under the library's event brackets -------------------------------
-    # grouped: one event pair around every run of consecutive launches of a class (the four projections between two
-    # attention passes keep their programmatic overlap, as in the timed steps); isolated: one pair per launch (an
-    # event between two launches serialises them, so every kernel is timed as if it stood alone)
+    # grouped: one event pair around every run of consecutive launches of a class (where the forward is a chain of
+    # launches, the four projections between two attention passes keep their programmatic overlap, as in the timed
+    # steps); isolated: one pair per launch (an event between two launches serialises them, so every kernel is timed as
+    # if it stood alone)
     prof_steps = min(args.steps, 4)
 
     def profile_pass(grouped: bool):
@@ -530,11 +531,15 @@ def run_ours(args, w: S.Workload, rank: int, world: int, local_rank: int):
     prof_total = sum(v["ms"] for v in prof.values())
     alg_per_launch = gemm["bytes"] / max(gemm["launches"], 1)
     ratio = NCU_TRAFFIC_RATIO.get(w.name)
+    one_launch = gemm["launches"] == prof_steps
     roofline = {"bound": "hbm",
-                "kernel": "the weight-streaming GEMMs (tc_gemm_cluster_kernel / tc_gemm_cluster_big_kernel / tc_gemm_kernel: "
+                "kernel": "forward_kernel (the decoder forward as one cooperative launch; bytes: all weight matrices + LM "
+                          "head, without the K/V tiles that it reads as well)" if one_launch else
+                          "the weight-streaming GEMMs (tc_gemm_cluster_kernel / tc_gemm_cluster_big_kernel / tc_gemm_kernel: "
                           "all weight matrices + LM head)", "achieved": achieved,
                 "peak": peak, "peak_kind": peak_kind, "unit": "GB/s", "frac": achieved / peak,
-                "timing": "CUDA events on the launching stream around every run of consecutive GEMM launches "
+                "timing": "CUDA events on the launching stream around the launch" if one_launch else
+                          "CUDA events on the launching stream around every run of consecutive GEMM launches "
                           "(O, gate/up, down, next QKV or LM head), summed and divided by the launches",
                 "algorithmic_bytes_per_launch": alg_per_launch,
                 # DRAM read + write bytes per launch: the ratio to the algorithmic bytes was taken with ncu on the

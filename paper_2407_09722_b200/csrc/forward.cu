@@ -498,6 +498,26 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                 for (int sl = s0; sl <= s1; ++sl) {
                     float* y = Y + (rb - r0) * ys + b * yb + tl;
                     const bool here = my == sl && tl < yb;
+                    if (FEW && s1 > s0 && !f.dual) {
+                        // narrow slices, several in a warp's lanes: up to four at a time, and a lane keeps its own
+                        const uint32_t at = t_acc + b * S * cols + rb * 3;
+                        float v[4][16];
+                        for (int q0 = s0; q0 <= s1; q0 += 4) {
+                            auto col = [&](int q) { return at + min(q0 + q, s1) * cols; };
+                            tc_ld16x4(col(0), col(1), col(2), col(3), v);
+                            const int q = my - q0;
+                            if (q >= 0 && q < 4 && tl < yb)
+#pragma unroll
+                                for (int j = 0; j < 5; ++j) {
+                                    float o = 0.f;
+#pragma unroll
+                                    for (int i = 0; i < 4; ++i)
+                                        if (i == q) o = v[i][3 * j] + (v[i][3 * j + 1] + v[i][3 * j + 2]);
+                                    if (rb + j < r1) y[j * ys] = o;
+                                }
+                        }
+                        break;
+                    }
                     if (FEW || terms == 3) {
                         float v[16];
                         tc_ld16(t_acc + (b * S + sl) * cols + rb * 3, v);
@@ -540,6 +560,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                 const float* y = Y + t * ys + q * yb + row;
                 float v = y[0];
                 if (S == 4) return (v + y[hr]) + (y[2 * hr] + y[3 * hr]);
+#pragma unroll 4
                 for (int sl = 1; sl < S; ++sl) v += y[sl * hr];
                 return v;
             };
