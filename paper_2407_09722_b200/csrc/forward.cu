@@ -8,7 +8,11 @@
 // leave the ring, the first ones of the next (or the committed K / V tiles of the attention) take their place, so HBM
 // stays busy across the barrier for as long as the ring is deep.  Two more things keep the boundary short: every block
 // owns whole output features (the features are cut into one tile per SM, not into 128-row tiles), so no partial sum leaves
-// an SM; and only the call's terms x rows operand rows are multiplied (16 columns for five rows).
+// an SM while rows are few; and only the call's terms x rows operand rows are multiplied (16 columns for five rows).
+// Measured (chain of launches -> one launch, a whole verification step): 7B, 5 rows 3.55 -> 3.02 ms (weights and K / V in
+// 2.2 ms at copy speed), 33 rows 4.40 -> 3.50, 65 rows 5.94 -> 4.65; 13B, 8 x 7 rows 9.8 -> 8.6; two-layer auxiliary
+// model of width 768, four draft steps 523 -> 434 us.  A phase costs its bytes plus about 3 us (barrier 1.1, first operand
+// rows 0.8, last MMA to last store 1.2 and up).
 //
 // Contraction.  Weights are the 128-row MMA operand A, the operand rows (two or three bf16 terms per activation, see
 // store_terms) operand B.  Where a block owns at most 64 features, the MMA takes S k-blocks at once: their weights lie
@@ -21,6 +25,10 @@
 //   P = exp2(S - m), a thread per key and half of the query rows, written to shared memory as bf16 hi and lo
 //   O^T += V^T P  A = V tile (MN-major), B = P; a thread per head dimension and half of the rows adds it to its registers
 // Pieces of a (sequence, KV head) held by several blocks meet in global memory; the block that arrives last merges them.
+// An item takes up to 8 or 16 query rows of a KV head, or 40 in the wide variant (an instantiation each: the softmax's time
+// goes with the rows, padding included; beyond 40 a thread's 20 rows would leave its registers), and more are cut into
+// blocks of equal size.  Per tile 0.75 us at 8 rows, 1.6 at 40, against 1.3 us that K and V take at copy speed.  7B, 65 rows
+// on 2048 keys: 39 -> 32 us a layer against `mma.sync` warps; 64 heads on 8 KV heads, 129 rows: 167 -> 40.
 //
 // Warps: 0 weight and K / V producer (TMA), 1 operand-row producer (TMA; waits for the phase before), 2 and 3 MMA issuers
 // (3 owns the tensor memory), 4..11 epilogue and softmax.
@@ -1547,7 +1555,8 @@ void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta, int cls) {
     rows(ph[FW_LM], d.vocab, d.d_model, lm_boxes, lm_boxes);
     // O and down: a tile's k-range over c blocks where that pays.  With many operand rows the SMs' intake bounds a narrow
     // tile (every block reads all operand rows of its k-blocks, about 100 GB/s an SM from L2); c blocks on a tile c times as
-    // wide read them a c-th as often, and pay about 3.5 us to exchange their partial sums.
+    // wide read them a c-th as often, and pay about 3.5 us to exchange their partial sums.  13B, 56 rows: O and down 24 and
+    // 48 us a layer unsplit, 17 and 32.5 over three blocks each.
     for (int k : {FW_O, FW_DOWN}) {
         FwPhase& f = ph[k];
         double best = 1e30;
@@ -1576,7 +1585,8 @@ void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta, int cls) {
     q.K = d.d_model;
     q.k_blocks = up_div(q.K, TC_TILE_K);
     // The same split for QKV, two heads of 128 on a tile: it meets the operand rows half as often and spreads over all SMs
-    // (7B, 32 heads: 96 tiles of one head leave a third of them idle), at about 4.5 us for the exchange.
+    // (7B, 32 heads: 96 tiles of one head leave a third of them idle), at about 4.5 us for the exchange.  7B, 65 rows: 35 ->
+    // 26 us a layer; at 33 rows both ways take 24.
     if (d.head_dim == 128 && q.u == 1 && cls >= 2) {
         const double floor_us = 2.0 * heads * 128 * q.K / 6.5e6;
         double best = std::max((128.0 + cols) * 128.0 * q.k_blocks / 85e3, floor_us) - 2.0;
@@ -1619,7 +1629,8 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
     const bool wide = G * R > FW_QROWS;
     a.nqb = wide ? up_div(G * R, FW_QROWS_WIDE) : 1;
     a.qrows = up_div(G * R, a.nqb);
-    a.cls = T <= 8 && !wide ? 0 : 2;                       // (four slots and the lean epilogues: up to eight rows)
+    // Up to eight rows the lean epilogues (an element per thread, a warp per row: beyond, a row would wait for its turn).
+    a.cls = T <= 8 && !wide ? 0 : 2;
     while (FW_CLASS[a.cls].cols < a.cols) ++a.cls;
     a.slots = fw_slots(d, a.cls);
     fw_geometry(a.ph, d, n_cta, a.cls);

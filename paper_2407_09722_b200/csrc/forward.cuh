@@ -19,6 +19,8 @@ constexpr int FW_QROWS_WIDE = 40;         // or in the wide variant: more are cu
 // the call's operand rows, so that the weight maps are encoded once per model: kb is the most that a ring slot holds.
 // Big boxes matter twice: a thread issues a copy about every quarter of a microsecond whatever its size, and rows of 256
 // bytes and more pass at 70 GB/s per SM where rows of 128 bytes pass at 43.
+// Three larger slots from 80 operand rows on, where a slot of a quarter of the ring holds one k-block only: 13B, 56 rows 8.64 ms
+// with three, 8.75 with four; 7B, 33 rows 3.50 and 3.62.  At up to 64 four are as good (7B, 18 rows 3.98 and 3.96).
 constexpr int FW_CLASSES = 6;
 struct FwClass { int cols, slots; };      // operand rows up to, ring slots
 constexpr FwClass FW_CLASS[FW_CLASSES] = {{16, 4}, {32, 4}, {64, 4}, {80, 3}, {112, 3}, {FW_MAX_COLS, 3}};
