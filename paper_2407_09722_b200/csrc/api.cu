@@ -629,7 +629,7 @@ int build_plan(ForwardPlan& fp, const Scratch& sc, const RowMeta& rm, const Mode
     fp.split_kv = split_kv;
     fp.kv_terms = tkv;
     // The attention of more than 16 query rows per KV head: 64 heads, 8 KV heads, 129 rows on 1024 keys 167 us a layer in
-    // attn_mma_kernel, 40 here.  With fewer that one is as fast, without a cooperative launch between the projections.
+    // attn_mma_kernel, 77 here.  With fewer that one is as fast, without a cooperative launch between the projections.
     fp.fw_attn = mma_attention(m) && fw_attn_plan(fp.fw, d, B, R, kCtas);
     if (fp.fw_attn) fw_common(fp.fw, sc, rm, m);
     return MTAD_OK;
@@ -778,7 +778,7 @@ int verify_common(mtad_ctx* ctx, int B, const int32_t* seqs, const int32_t* n_no
                              out->status, s));
     if (spd) {
         SpdArgs sa{B, R, D, tok, logq_ref, spd_accept_uniform, bonus_uniform};
-        RUN(MTAD_K_ACCEPT, 0, 1, launch_spd_accept(ctx->target, ctx->rm, ctx->sc, sa, *out, s));
+        RUN(MTAD_K_ACCEPT, 0, 3, launch_spd_accept(ctx->target, ctx->rm, ctx->sc, sa, *out, ctx->use_pdl, s));
     } else {
         AcceptArgs aa{B, R, D, tok, parent, logq_ref, log_tau};
         RUN(MTAD_K_ACCEPT, 0, 1, launch_accept(ctx->rm, ctx->sc, aa, *out, s));

@@ -363,7 +363,7 @@ struct SpdArgs {
     const float* resample_uniform;  // [B, V]
 };
 cudaError_t launch_spd_accept(const ModelView& m, const RowMeta& rm, const Scratch& sc, const SpdArgs& a,
-                              const mtad_result& out, cudaStream_t st);
+                              const mtad_result& out, bool pdl, cudaStream_t st);
 cudaError_t launch_accept(const RowMeta& rm, const Scratch& sc, const AcceptArgs& a, const mtad_result& out,
                           cudaStream_t st);
 cudaError_t launch_kv_commit(const ModelView& m, const SeqState& s, int B, const int32_t* call_seq_dev,

@@ -28,7 +28,7 @@
 // An item takes up to 8 or 16 query rows of a KV head, or 40 in the wide variant (an instantiation each: the softmax's time
 // goes with the rows, padding included; beyond 40 a thread's 20 rows would leave its registers), and more are cut into
 // blocks of equal size.  Per tile 0.75 us at 8 rows, 1.6 at 40, against 1.3 us that K and V take at copy speed.  7B, 65 rows
-// on 2048 keys: 39 -> 32 us a layer against `mma.sync` warps; 64 heads on 8 KV heads, 129 rows: 167 -> 40.
+// on 2048 keys: 39 -> 32 us a layer against `mma.sync` warps; 64 heads on 8 KV heads, 129 rows, 1024 keys: 167 -> 77.
 //
 // Warps: 0 weight and K / V producer (TMA), 1 operand-row producer (TMA; waits for the phase before), 2 and 3 MMA issuers
 // (3 owns the tensor memory), 4..11 epilogue and softmax.
