@@ -265,18 +265,27 @@ __global__ void __launch_bounds__(256) draft_pick_kernel(const float* __restrict
     __shared__ float l_y[MTAD_MAX_CAND];                           // the layer's nodes: perturbed score, flat pair,
     __shared__ int l_flat[MTAD_MAX_CAND], l_rank[MTAD_MAX_CAND];   // rank among the kept beams (-1: not kept)
     const DraftPart* pp = part + (size_t)bi * MTAD_MAX_BEAM * nch;
-    if (tid < n_beams) {
-        // log-sum-exp of beam row tid: chunks in order
-        const DraftPart* pj = pp + (size_t)tid * nch;
-        float M = -CUDART_INF_F;
-        for (int c = 0; c < nch; ++c) M = fmaxf(M, pj[c].m);
-        float a = 0.f;
-        for (int c = 0; c < nch; ++c) a += (pj[c].m == -CUDART_INF_F) ? 0.f : pj[c].s * expf(pj[c].m - M);
-        s_lse[tid] = M + logf(a);
-        const int slot = step == 0 ? -1 : (step - 1) * beam + tid;
-        s_slot[tid] = slot;
-        s_tree[tid] = slot < 0 ? -1 : ds.tree_id[seq * MTAD_DRAFT_NODES + slot];
-        s_lq[tid] = slot < 0 ? 0.f : ds.node_logq[seq * MTAD_DRAFT_NODES + slot];
+    // Log-sum-exp of a beam row: a warp per row, a lane per chunk, combined in a fixed order.  (A thread per row that walked the
+    // chunks took 2 us longer a step: its loads and exponentials one after the other.)
+    static_assert(MTAD_DRAFT_CHUNKS <= 32, "a lane per chunk");
+    for (int j = tid >> 5; j < n_beams; j += 8) {
+        const int lane = tid & 31, slot = step == 0 ? -1 : (step - 1) * beam + j;
+        const DraftPart* pj = pp + (size_t)j * nch;
+        const float mc = lane < nch ? pj[lane].m : -CUDART_INF_F, sc = lane < nch ? pj[lane].s : 0.f;
+        const int tree = slot < 0 ? -1 : ds.tree_id[seq * MTAD_DRAFT_NODES + slot];
+        const float lq = slot < 0 ? 0.f : ds.node_logq[seq * MTAD_DRAFT_NODES + slot];
+        float M = mc;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+        float a = mc == -CUDART_INF_F ? 0.f : sc * expf(mc - M);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (lane == 0) {
+            s_lse[j] = M + logf(a);
+            s_slot[j] = slot;
+            s_tree[j] = tree;
+            s_lq[j] = lq;
+        }
     }
     __syncthreads();
     const int per_beam = nch * kpb;                                // candidates of one beam row
