@@ -53,8 +53,9 @@ constexpr int FW_THREADS = 32 * 12;
 constexpr int FW_EPI_WARP0 = 4;
 constexpr int FW_EPI = 256;
 constexpr int FW_UNION = 32 * 1024;       // epilogue tile Y, or the attention's query and probability tiles
-constexpr int FW_ACC = 240;               // accumulator columns of a tile, of 256 (the drain reads up to 15 columns further),
+constexpr int FW_ACC = 240;               // accumulator columns of a tile, of 256 (the drain reads up to 16 columns further),
 constexpr int FW_ACC_ONE = 496;           // or of 512 where a tile takes both buffers
+static_assert(FW_ACC + 16 <= 256 && FW_ACC_ONE + 16 <= 512, "columns that a drain reads");
 constexpr float FW_LAZY = 64.f;           // log2 of how far a score may exceed its row's reference value
 constexpr float FW_UNSEEN = -1e30f;       // the reference value of a row that has seen no key
 
@@ -132,6 +133,22 @@ __device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr) {
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
     const int n = valid ? 16 : 0;                      // src-size 0: the 16 bytes are zero-filled
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+}
+
+// 16 columns of a box's `na` accumulators (up to four), `stride` columns apart, added up
+__device__ __forceinline__ void acc_ld16(uint32_t at, int stride, int na, float* v) {
+    if (na == 1) {
+        tc_ld16(at, v);
+        return;
+    }
+    tc_ld16_sum(at, at + stride, v);
+    if (na > 2) {
+        float w[16];
+        if (na > 3) tc_ld16_sum(at + 2 * stride, at + 3 * stride, w);
+        else tc_ld16(at + 2 * stride, w);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] += w[j];
+    }
 }
 
 // What a call's sequence looks like to the attention
@@ -232,14 +249,7 @@ __device__ __forceinline__ bool split_residual(const FwArgs& a, FwTail& s, const
     for (int rb = half * per; rb < T; rb += 2 * per)
         for (int sl = s0; sl <= s1; ++sl) {
             float v[16];
-            const uint32_t at = t_acc + sl * cols + rb * terms;
-            tc_ld16(at, v);
-            if (f.dual) {
-                float v2[16];
-                tc_ld16(at + S * cols, v2);
-#pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] += v2[j];
-            }
+            acc_ld16(t_acc + sl * cols + rb * terms, S * cols, f.na, v);
             if (my == sl && tl < yb) {
                 float* y = mine + (size_t)rb * yb;
                 if (terms == 3) {
@@ -324,7 +334,7 @@ __device__ __forceinline__ bool split_qkv(const FwArgs& a, FwTail& s, const FwPh
     float* y = a.kpart + (size_t)tile * T * 256 + half * 128 + quad * 32 + lane;
     for (int rb = 0; rb < T; rb += per) {
         float v[16];
-        tc_ld16(t_acc + rb * terms, v);
+        acc_ld16(t_acc + rb * terms, 2 * cols, f.na, v);
         if (terms == 3) {
 #pragma unroll
             for (int j = 0; j < 5; ++j, y += 256)
@@ -389,6 +399,47 @@ __device__ __forceinline__ bool split_qkv(const FwArgs& a, FwTail& s, const FwPh
     return true;
 }
 
+__device__ __forceinline__ int up16(int x) { return (x + 15) & ~15; }
+
+// End of a part of a tile's k-range other than the last (two boxes, a warp of a quadrant each; one slice): the rows' sums so
+// far go to the tensor-memory columns from f.stash on, and the accumulators are free.
+__device__ __forceinline__ bool put_by(const FwArgs& a, FwTail& s, const FwPhase& f, int part, int tcount, int e, uint32_t tmem_lane) {
+    const int lane = e & 31, half = e >> 7, T = a.T, cols = a.cols, buf = tcount & 1;
+    bool ok = true;
+    if (e == 0) ok = mbar_wait(smem_u32(&s.tfull[buf]), (uint32_t)(tcount >> 1) & 1u, s.abort_flag);
+    ok = all_of(1, FW_EPI, ok);
+    if (!ok) return false;
+    tc_fence_after();
+    const uint32_t at = tmem_lane + (f.both ? 0 : buf * 256) + half * cols, st = tmem_lane + f.stash + half * up16(T);
+    for (int rb = 0; rb < T; rb += 16) {
+        float r[16];
+        if (a.terms == 3) {
+            float v[48];
+#pragma unroll
+            for (int h = 0; h < 3; ++h) acc_ld16(at + rb * 3 + 16 * h, 2 * cols, f.na, v + 16 * h);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) r[j] = v[3 * j] + (v[3 * j + 1] + v[3 * j + 2]);
+        } else {
+            float v[32];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) acc_ld16(at + rb * 2 + 16 * h, 2 * cols, f.na, v + 16 * h);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) r[j] = v[2 * j] + v[2 * j + 1];
+        }
+        if (part > 0) {
+            float o[16];
+            tc_ld16(st + rb, o);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) r[j] += o[j];
+        }
+        tc_st16(st + rb, r);
+    }
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(&s.tempty[buf]));
+    return true;
+}
+
 // The epilogue group's part of one projection: row statistics, then per tile the accumulators -> Y in shared memory ->
 // the fused epilogue.  KIND is a template parameter so that the phase's geometry is read straight from the launch
 // parameters; index arithmetic and global loads stand ahead of the wait for the accumulator, because everything after it
@@ -404,7 +455,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
     constexpr int V = FEW ? 1 : 4;                         // features per item
     const int lane = e & 31, w = e >> 5, quad = w & 3, half = w >> 2;
     const int T = a.T, terms = a.terms, cols = a.cols, n_cta = a.n_cta;
-    const int hr = f.hr, S = f.S, nbox = f.nbox;
+    const int hr = f.hr, S = f.S, nbox = f.nbox, na = f.na, acc_stride = nbox * S * cols;
     const int yb = S * hr, ys = nbox * yb + 4;             // columns of Y that a box takes, row stride of Y
     const int nf = KIND == FW_LM ? nbox * f.h : f.h;       // features (pairs) of a tile
     const int nv = nf / V;                                 // items of a row
@@ -454,7 +505,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
             return ok;
         }
     for (int tile = cta; tile < f.n_tiles; tile += n_cta, ++tcount) {
-        const int buf = tcount & 1, f0 = tile * nf;        // f0: first feature (O, down, gate / up, LM head)
+        const int f0 = tile * nf;                          // first feature (O, down, gate / up, LM head)
         // ---- what the first items need besides the accumulator
         const int hg = KIND == FW_QKV ? tile / f.u : 0, j0 = KIND == FW_QKV ? (tile - hg * f.u) * f.h : 0;
         constexpr int NI = FEW ? 2 : 1;                    // QKV: items per thread and round
@@ -491,12 +542,24 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
             if (w < T) hid = __ldcg(a.hidden + (size_t)w * a.d + f0 + lane);
         }
         if (KIND == FW_LM && !a.lm_plain) lm_load(w);
+        if (!FEW && KIND == FW_GATEUP)
+            for (int sg = 0; sg + 1 < f.segs; ++sg, ++tcount)
+                if (!put_by(a, s, f, sg, tcount, e, tmem_lane)) return false;
+        const int buf = tcount & 1;
         // (one thread polls: 256 of them would take the shared-memory pipe away from the copies' barriers)
         if (e == 0) ok = mbar_wait(smem_u32(&s.tfull[buf]), (uint32_t)(tcount >> 1) & 1u, abort_flag);
         ok = all_of(1, FW_EPI, ok);
         if (!ok) return false;
         tc_fence_after();
         const uint32_t t_acc = tmem_lane + (f.both ? 0 : buf * 256);
+        auto add_put_by = [&](int b, int rb, float* v) {   // what the tile's earlier parts left of 16 rows
+            if (!FEW && KIND == FW_GATEUP && f.segs > 1) {
+                float o[16];
+                tc_ld16(tmem_lane + f.stash + b * up16(T) + rb, o);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[j] += o[j];
+            }
+        };
         for (int r0 = 0; r0 < T; r0 += blk) {
             const int r1 = min(T, r0 + blk), nr = r1 - r0;
             // ---- accumulators -> Y[row][box][lane], the terms of a row added up
@@ -506,7 +569,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                 for (int sl = s0; sl <= s1; ++sl) {
                     float* y = Y + (rb - r0) * ys + b * yb + tl;
                     const bool here = my == sl && tl < yb;
-                    if (FEW && s1 > s0 && !f.dual) {
+                    if (FEW && s1 > s0 && na == 1) {
                         // narrow slices, several in a warp's lanes: up to four at a time, and a lane keeps its own
                         const uint32_t at = t_acc + b * S * cols + rb * 3;
                         float v[4][16];
@@ -528,32 +591,30 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                     }
                     if (FEW || terms == 3) {
                         float v[16];
-                        tc_ld16(t_acc + (b * S + sl) * cols + rb * 3, v);
-                        if (f.dual) {
-                            float v2[16];
-                            tc_ld16(t_acc + (S + sl) * cols + rb * 3, v2);
+                        acc_ld16(t_acc + (b * S + sl) * cols + rb * 3, acc_stride, na, v);
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) v[j] += v2[j];
-                        }
+                        for (int j = 0; j < 5; ++j) v[j] = v[3 * j] + (v[3 * j + 1] + v[3 * j + 2]);
+                        add_put_by(b, rb, v);
                         if (here)
 #pragma unroll
                             for (int j = 0; j < 5; ++j)
-                                if (rb + j < r1) y[j * ys] = v[3 * j] + (v[3 * j + 1] + v[3 * j + 2]);
+                                if (rb + j < r1) y[j * ys] = v[j];
                     } else {
                         float v[32];
-                        tc_ld32(t_acc + (b * S + sl) * cols + rb * 2, v);
-                        if (f.dual)
+                        const uint32_t at = t_acc + (b * S + sl) * cols + rb * 2;
+                        if (na == 1) {
+                            tc_ld32(at, v);
+                        } else {
+                            acc_ld16(at, acc_stride, na, v);
+                            acc_ld16(at + 16, acc_stride, na, v + 16);
+                        }
 #pragma unroll
-                            for (int h = 0; h < 32; h += 16) {
-                                float v2[16];
-                                tc_ld16(t_acc + (S + sl) * cols + rb * 2 + h, v2);
-#pragma unroll
-                                for (int j = 0; j < 16; ++j) v[h + j] += v2[j];
-                            }
+                        for (int j = 0; j < 16; ++j) v[j] = v[2 * j] + v[2 * j + 1];
+                        add_put_by(b, rb, v);
                         if (here)
 #pragma unroll
                             for (int j = 0; j < 16; ++j)
-                                if (rb + j < r1) y[j * ys] = v[2 * j] + v[2 * j + 1];
+                                if (rb + j < r1) y[j * ys] = v[j];
                     }
                     __syncwarp();
                 }
@@ -1141,44 +1202,42 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
             }
             const FwPhase& f = a.ph[kind];
             const int groups = f.kb / f.S, sc = f.S * cols, nbox = f.nbox;      // MMAs along k, accumulator columns of a box
-            const bool dual = f.dual != 0;
+            const int na = f.na;
             const uint32_t idesc = IDESC | ((uint32_t)(sc >> 3) << 17);
             const uint32_t a_step = f.S * f.hr * 8, b_step = sc * 8;            // 16-byte units
-            for (int tile = cta; tile < f.n_tiles && ok; tile += n_cta, ++tcount) {
-                const int buf = tcount & 1;
-                ok = mbar_wait_warp(smem_u32(&s.tempty[buf]), ((uint32_t)(tcount >> 1) & 1u) ^ 1u, abort_flag);
-                if (f.both && tcount > 0)              // (its accumulators take the columns of the tile before as well)
-                    ok = ok && mbar_wait_warp(smem_u32(&s.tempty[buf ^ 1]), (uint32_t)((tcount - 1) >> 1) & 1u, abort_flag);
-                if (!ok) break;
-                tc_fence_after();
-                const bool mine = me == 0 || nbox == 2 || dual;
-                const uint32_t d = tmem + (f.both ? 0 : buf * 256) + me * sc;
-                uint32_t acc = 0;
-                int turn = 0;                              // dual: MMAs along k alternate between the warps
-                const int k1 = k_end(f, tile);
-                for (int step = k_first(f, tile); step < k1; ++step, ++pos) {
-                    ok = mbar_wait_warp(full_bar(pos), ring_par(pos), abort_flag);
+            for (int tile = cta; tile < f.n_tiles && ok; tile += n_cta) {
+                const int k0 = k_first(f, tile), k1 = k_end(f, tile);
+                for (int sg = 0; sg < f.segs && ok; ++sg, ++tcount) {
+                    const int buf = tcount & 1;
+                    ok = mbar_wait_warp(smem_u32(&s.tempty[buf]), ((uint32_t)(tcount >> 1) & 1u) ^ 1u, abort_flag);
+                    if (f.both && tcount > 0)          // (its accumulators take the columns of the tile before as well)
+                        ok = ok && mbar_wait_warp(smem_u32(&s.tempty[buf ^ 1]), (uint32_t)((tcount - 1) >> 1) & 1u, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
-                    if (mine) {
+                    const uint32_t d0 = tmem + (f.both ? 0 : buf * 256) + (nbox == 2 ? me * sc : 0);
+                    int turn = 0;                      // accumulator of the next MMA along k; one box: warp `me` forms every other one
+                    uint32_t acc = 0;                  // (the first round over the accumulators begins them)
+                    const int end = k0 + (k1 - k0) * (sg + 1) / f.segs;
+                    for (int step = k0 + (k1 - k0) * sg / f.segs; step < end; ++step, ++pos) {
+                        ok = mbar_wait_warp(full_bar(pos), ring_par(pos), abort_flag);
+                        if (!ok) break;
+                        tc_fence_after();
                         const uint32_t base = slot_ptr(pos);
                         uint64_t ad = smem_desc(base), bd = smem_desc(base + f.b_off);
                         if (nbox == 2) ad += (uint32_t)(me * f.box_bytes) >> 4;
                         for (int gr = 0; gr < groups; ++gr, ad += a_step, bd += b_step) {
-                            if (dual) {
-                                turn ^= 1;
-                                if (turn == me) continue;
-                            }
+                            if (nbox == 2 || (turn & 1) == me) {
+                                const uint32_t d = d0 + turn * nbox * sc;
 #pragma unroll
-                            for (int k4 = 0; k4 < TC_TILE_K / 16; ++k4) {
-                                tc_mma_one(one, d, ad + k4 * 2, bd + k4 * 2, idesc, acc);
-                                acc = 1u;
+                                for (int k4 = 0; k4 < TC_TILE_K / 16; ++k4)
+                                    tc_mma_one(one, d, ad + k4 * 2, bd + k4 * 2, idesc, k4 > 0 ? 1u : acc);
                             }
+                            if (++turn == na) { turn = 0; acc = 1u; }
                         }
+                        tc_commit_one(one, empty_bar(pos));
                     }
-                    tc_commit_one(one, empty_bar(pos));
+                    if (ok) tc_commit_one(one, smem_u32(&s.tfull[buf]));
                 }
-                if (ok) tc_commit_one(one, smem_u32(&s.tfull[buf]));
             }
         }
         if (!ok)               // gave up: the MMAs in flight end before the block frees its tensor memory and leaves
@@ -1644,10 +1703,40 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
         for (int S = 2; S <= f.kb; ++S)
             if (f.kb % S == 0 && S * f.hr <= TC_TILE_N && S * a.cols * f.nbox <= FW_ACC) f.S = S;
         if (f.b_off + f.kb * a.cols * 128 > FW_RING / a.slots || f.nbox * f.S * a.cols > FW_ACC_ONE) return false;
-        f.both = f.nbox * f.S * a.cols > FW_ACC ? 1 : 0;
         if ((k == FW_O || k == FW_DOWN || f.c > 1) && (f.n_tiles > n_cta || f.steps < f.c)) return false;
-        // one box: the MMAs along k alternate between two accumulators where they fit and every block has two
-        f.dual = f.nbox == 1 && 2 * f.S * a.cols <= FW_ACC && f.steps / f.c * (f.kb / f.S) >= 2 ? 1 : 0;
+        // Accumulators.  At every addition into an accumulator the tensor core cuts off what fp32 does not hold, toward zero,
+        // so a sum's error goes with the k-blocks that one accumulator takes (6.9e-8 each).  A box has as many accumulators as
+        // keep them below `cap`, which take the k-blocks in turn and are added by the epilogue (one box: at least two where the
+        // tile keeps to its buffer, so that both issuing warps have one).  The caps are about what the chain of launches,
+        // whose blocks share a tile's k-range, leaves to an accumulator; its error against 64 bits is the measure.  7B, 4096 ->
+        // 11008 -> 4096: gate / up 7.5e-6 there, 11.2e-6 with one accumulator, 8.0e-6 with two; down of 65 rows 2.2, 3.2 and
+        // 1.7e-6.  It costs 1 % of a step of five rows, 2 % of one of 65.
+        const int cap = std::max(4, k == FW_QKV ? std::min(f.k_blocks / 2, 43) : (k == FW_O ? f.k_blocks / 4 : (k == FW_GATEUP ?
+                                f.k_blocks / 2 : (k == FW_DOWN ? f.k_blocks / 6 : f.k_blocks))));
+        const int base = f.nbox * f.S * a.cols, most = f.n_tiles <= n_cta ? FW_ACC_ONE : FW_ACC;
+        const int fewest = f.steps / f.c * (f.kb / f.S);          // MMAs along k of a block, at least and at most
+        const int longest = up_div(f.steps, f.c) * (f.kb / f.S);
+        const int room = std::max(1, std::min(std::min(4, fewest), most / base));
+        f.na = f.nbox == 1 && 2 * base <= FW_ACC ? std::min(2, room) : 1;
+        while (f.na < room && up_div(longest, f.na) > cap) ++f.na;
+        f.both = f.na * base > FW_ACC ? 1 : 0;
+        // Gate / up of many rows: two boxes leave room for one or two accumulators each, and the k-range of a tile is taken
+        // in parts instead, after each of which the sums move to other columns of the tensor memory.
+        f.segs = 1;
+        f.stash = 0;
+        if (k == FW_GATEUP && a.cls >= 2 && f.S == 1 && up_div(longest, f.na) > cap) {
+            const int put = 2 * ((a.T + 15) / 16 * 16);
+            for (int n = f.na; n >= 1; --n) {
+                const int segs = up_div(up_div(longest, n), cap), used = n * base;
+                const bool one = used <= FW_ACC && used + put <= 256;
+                if ((!one && (f.n_tiles > n_cta || used + put > 512)) || f.steps / segs * f.kb < n) continue;
+                f.na = n;
+                f.segs = segs;
+                f.both = one ? 0 : 1;
+                f.stash = used;
+                break;
+            }
+        }
         const int per = a.terms == 3 ? 5 : 16;             // rows of one drain load
         const int fit = FW_UNION / (per * (f.nbox * f.S * f.hr + 4) * 4);
         if (fit < 1) return false;

@@ -31,8 +31,10 @@ struct FwPhase {
     int kb, flat, S, steps;               // k-blocks of a box, its map's view, k-blocks side by side in the MMA, steps of all k-blocks
     int box_bytes, b_off;                 // bytes of one weight box, offset of the operand rows in the slot
     int k_blocks, K;
-    int dual, both, blk;                  // two accumulators for one box; a tile takes both accumulator buffers; rows that the
-                                          // epilogue takes at a time
+    int na, segs;                         // accumulators of a box, which take the MMAs along k in turn; parts of a tile's k-range
+                                          // after which the accumulators are put by and begun afresh
+    int both, stash, blk;                 // a tile takes both accumulator buffers; tensor-memory column where the parts are put
+                                          // by; rows that the epilogue takes at a time
 };
 enum { FW_QKV = 0, FW_ATTN = 1, FW_O = 2, FW_GATEUP = 3, FW_DOWN = 4, FW_LM = 5 };
 
