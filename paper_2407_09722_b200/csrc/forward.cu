@@ -22,7 +22,7 @@
 //
 // Attention: keys as the M dimension.  The (sequence, KV head, 128-key tile) items are dealt out evenly, in order.
 //   S^T = K Q^T   A = K tile as it lies in the cache, B = query rows (bf16 hi rows, then lo rows)
-//   P = exp2(S - m), a thread per key and half of the query rows, written to shared memory as bf16 hi and lo
+//   P = exp2(S - m), a thread per key and half of the query rows, written to shared memory as three bf16 terms
 //   O^T += V^T P  A = V tile (MN-major), B = P; a thread per head dimension and half of the rows adds it to its registers
 // Pieces of a (sequence, KV head) held by several blocks meet in global memory; the block that arrives last merges them.
 // An item takes up to 8 or 16 query rows of a KV head, or 40 in the wide variant (an instantiation each: the softmax's time
@@ -919,15 +919,23 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     constexpr int NQ2 = 2 * NQP;                       // query rows as hi and lo parts
     constexpr uint32_t KV_BYTES = FW_KEYS * HD * 2;
     constexpr int Q_BYTES = NQ2 * HD * 2;              // one query tile
-    constexpr int P_BYTES = NQ2 * FW_KEYS * 2;         // one probability tile
+    // Probabilities as three terms, exactly.  Two leave 2^-18 of each, and with one reference value for all keys of a tile even
+    // the largest is not exact (mma.sync warps had a maximum for every 16 or 64 keys, whose probability is 1): 400 keys of a
+    // 64-wide head 2.85e-6 of the output off, 2.45 with mma.sync, 1.40 with three terms.  A tile takes 3 % longer.
+    constexpr int NP3 = 3 * NQP;
+    constexpr int P_N = (NP3 + 15) / 16 * 16;          // N of the output MMA: may read up to eight rows past the tile
+    constexpr int P_BYTES = NP3 * FW_KEYS * 2;         // one probability tile
     constexpr int FW_SLOT = FW_RING / NS;
-    // Wide attention: up to 40 query rows, whose tiles outgrow the union.  There is one query tile instead of two, and the
-    // probabilities lie in the ring, behind the K and V tiles, which do not fill their slots: with three slots behind V; with
-    // four the second 64 keys behind K.  That space is a tile's own: an item that fills its slot (a step of a projection) came
-    // before the attention, or comes after the output has been formed (PBK: so the last two K tiles are released only then).
-    constexpr bool WIDE = NQP > FW_QROWS, PBK = WIDE && NS == 4;
-    static_assert(!WIDE || ((int)KV_BYTES + P_BYTES / (PBK ? 2 : 1) <= FW_SLOT && Q_BYTES + (int)sizeof(FwAttn<NQP / 2>) <= FW_UNION), "wide attention");
+    // From nine query rows on the tiles outgrow the union, and the probabilities lie in the ring, behind the K and V tiles, which
+    // do not fill their slots: behind V; wide (up to 40 query rows; one query tile instead of two) and with four slots the second
+    // 64 keys behind K.  That space is a tile's own: an item that fills its slot (a step of a projection) came before the
+    // attention, or comes after the output has been formed (PBK: so the last two K tiles are released only then).
+    constexpr bool PRING = NQP > 8, WIDE = NQP > FW_QROWS, PBK = WIDE && NS == 4;
+    static_assert(!PRING || (int)KV_BYTES + P_BYTES / (PBK ? 2 : 1) + (P_N - NP3) * 128 <= FW_SLOT, "probabilities in the ring");
+    static_assert((WIDE ? Q_BYTES + (int)sizeof(FwAttn<NQP / 2>) : 2 * Q_BYTES + (PRING ? 0 : 2 * P_BYTES + (P_N - NP3) * 128)) <= FW_UNION,
+                  "query rows and probabilities");
     constexpr int TM = WIDE ? 128 : 64;                // attention: tensor-memory columns 0 / TM scores, 2 TM / 3 TM outputs
+    static_assert(P_N <= TM, "output columns");
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* uni = smem + FW_RING;
     FwTail& s = *reinterpret_cast<FwTail*>(uni + FW_UNION);
@@ -1172,7 +1180,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         ok = mbar_wait_warp(smem_u32(&s.ofull[n & 1]), (uint32_t)(n >> 1) & 1u, abort_flag);
                     }
                 } else {
-                    constexpr uint32_t idesc_o = IDESC | (1u << 15) | ((uint32_t)(NQ2 >> 3) << 17);
+                    constexpr uint32_t idesc_o = IDESC | (1u << 15) | ((uint32_t)(P_N >> 3) << 17);
                     for (int i = 0; i < a_n; ++i) {
                         const int vpos = pos + 2 * i + 1, b = (at + i) & 1;
                         const uint32_t par = (uint32_t)((at + i) >> 1) & 1u;
@@ -1181,8 +1189,8 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                              mbar_wait_warp(full_bar(vpos), ring_par(vpos), abort_flag);
                         if (!ok) break;
                         tc_fence_after();
-                        const uint64_t va = smem_desc_mn(slot_ptr(vpos)), pa = smem_desc(WIDE ? slot_ptr(vpos) + KV_BYTES : smem_u32(Ps) + b * P_BYTES);
-                        const uint64_t pb = PBK ? smem_desc(slot_ptr(vpos - 1) + KV_BYTES) : pa + NQ2 * 8;       // keys 64 ..
+                        const uint64_t va = smem_desc_mn(slot_ptr(vpos)), pa = smem_desc(PRING ? slot_ptr(vpos) + KV_BYTES : smem_u32(Ps) + b * P_BYTES);
+                        const uint64_t pb = PBK ? smem_desc(slot_ptr(vpos - 1) + KV_BYTES) : pa + NP3 * 8;       // keys 64 ..
 #pragma unroll
                         for (int ks = 0; ks < FW_KEYS / 16; ++ks)
                             tc_mma_one(one, tmem + (2 + b) * TM, va + ks * 128, (ks < 4 ? pa : pb) + (ks & 3) * 2,
@@ -1266,16 +1274,34 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                 constexpr int NR = NQP / 2;                           // this thread's query rows: half, half + 2, ...; wide:
                 auto row_of = [&](int x) { return WIDE ? half * NR + x : 2 * x + half; };        // NR neighbouring ones
                 auto& sa = *reinterpret_cast<FwAttn<WIDE ? NR : FW_QROWS / 2>*>(WIDE ? Qs + Q_BYTES : reinterpret_cast<uint8_t*>(&s.attn));
-                // scores or outputs at column `col`: this thread's rows, hi and lo parts added up
+                // scores at column `col`: this thread's rows, hi and lo parts added up
                 auto tm_rows = [&](int col, float* v) {
                     if constexpr (WIDE) {
                         tc_ld20_sum(t_lane + col + half * NR, t_lane + col + NQP + half * NR, v);
                     } else {
                         float c[NQ2];
-                        if (NQ2 == 16) tc_ld16(t_lane + col, c);
-                        else { tc_ld16(t_lane + col, c); tc_ld16(t_lane + col + 16, c + NQ2 - 16); }
+                        if constexpr (NQ2 == 16) tc_ld16(t_lane + col, c);
+                        else tc_ld32(t_lane + col, c);
 #pragma unroll
                         for (int x = 0; x < NR; ++x) v[x] = half == 0 ? c[2 * x] + c[NQP + 2 * x] : c[2 * x + 1] + c[NQP + 2 * x + 1];
+                    }
+                };
+                // the same for outputs, which have three parts
+                auto tm_out = [&](int col, float* v) {
+                    if constexpr (WIDE) {
+                        float c[NR];
+                        tc_ld20_sum(t_lane + col + NQP + half * NR, t_lane + col + 2 * NQP + half * NR, v);
+                        tc_ld20(t_lane + col + half * NR, c);
+#pragma unroll
+                        for (int x = 0; x < NR; ++x) v[x] += c[x];
+                    } else {
+                        float c[NP3 > 32 ? 48 : 32];
+                        if constexpr (NP3 > 32) tc_ld48(t_lane + col, c);
+                        else tc_ld32(t_lane + col, c);
+#pragma unroll
+                        for (int x = 0; x < NR; ++x)
+                            v[x] = half == 0 ? c[2 * x] + (c[NQP + 2 * x] + c[2 * NQP + 2 * x])
+                                             : c[2 * x + 1] + (c[NQP + 2 * x + 1] + c[2 * NQP + 2 * x + 1]);
                     }
                 };
                 // query rows of a segment: KV head, first row, how many
@@ -1337,7 +1363,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     ok = warp_wait(smem_u32(&s.ofull[b]), (uint32_t)(tile_no >> 1) & 1u, abort_flag, ok, lane);
                     tc_fence_after();
                     float c[NR];
-                    tm_rows((2 + b) * TM, c);
+                    tm_out((2 + b) * TM, c);
 #pragma unroll
                     for (int x = 0; x < NR; ++x) acc[x] += c[x];
                 };
@@ -1485,8 +1511,8 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             for (int x = 0; x < NR; ++x) sa.sm[half][x] = m[x];
                         bar_n(2 + half, 128);                         // (smx is free again)
                     }
-                    uint8_t* pt = (WIDE ? smem + (size_t)((pos + 2 * i + (PBK && kl >= 64 ? 0 : 1)) % NS) * FW_SLOT + KV_BYTES : Ps + b * P_BYTES) +
-                                  (PBK ? 0 : kl >> 6) * (NQ2 * 128) + (kl & 7) * 2 + row_of(0) * 128;
+                    uint8_t* pt = (PRING ? smem + (size_t)((pos + 2 * i + (PBK && kl >= 64 ? 0 : 1)) % NS) * FW_SLOT + KV_BYTES : Ps + b * P_BYTES) +
+                                  (PBK ? 0 : kl >> 6) * (NP3 * 128) + (kl & 7) * 2 + row_of(0) * 128;
                     constexpr int RS = WIDE ? 128 : 256;              // bytes between this thread's rows
                     const int pc = (kl & 63) >> 3;
 #pragma unroll
@@ -1497,7 +1523,10 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         const __nv_bfloat16 hi = __float2bfloat16_rn(pv);
                         uint8_t* d = pt + ((pc ^ (row_of(x) & 7)) << 4) + x * RS;
                         *reinterpret_cast<__nv_bfloat16*>(d) = hi;
-                        *reinterpret_cast<__nv_bfloat16*>(d + NQP * 128) = __float2bfloat16_rn(pv - __bfloat162float(hi));
+                        const float rest = pv - __bfloat162float(hi);
+                        const __nv_bfloat16 lo = __float2bfloat16_rn(rest);
+                        *reinterpret_cast<__nv_bfloat16*>(d + NQP * 128) = lo;
+                        *reinterpret_cast<__nv_bfloat16*>(d + 2 * NQP * 128) = __float2bfloat16_rn(rest - __bfloat162float(lo));
                     }
                     if ((it.tile + 1) * FW_KEYS > nkeys) {
                         // rows of V past the last key: their probabilities are 0, but 0 x (stale value) must not make a NaN
