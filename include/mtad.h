@@ -237,7 +237,8 @@ int kv_commit(mtad_ctx* ctx, int B, const int32_t* seqs, const mtad_result* res,
  * The K/V rows of the root and the draft tokens are left in cache slots kv_len .. kv_len + gamma, as after
  * mtad_verify_chain; there is no commit step, the caller keeps the rows it accepts.
  * Limits and sharing: returns MTAD_E_WORKSPACE when the model shape or gamma needs more scratch than the array
- * holds (mtad_workspace_bytes(target, NULL, 1, gamma) tells how much).  All calls on a device share the one array,
+ * holds.  What mtad_workspace_bytes(target, NULL, 1, gamma) reports is enough; somewhat less is too: without room for the
+ * arrays of the one-launch forward the step runs as a chain of launches.  All calls on a device share the one array,
  * which still contains the previous call's data: the library re-zeroes the whole array whenever the model or gamma
  * changes (after synchronising the device, so that earlier calls still running on any stream are over) and the
  * split-K counters at the start of every call, but two calls whose GPU work overlaps (different streams, different threads) race

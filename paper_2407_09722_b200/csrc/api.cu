@@ -163,13 +163,15 @@ bool model_ptrs_ok(const mtad_model_desc* m) {
     return true;
 }
 
-// Lays out the workspace; with base == nullptr only measures it.
-size_t carve(mtad_ctx* c, const mtad_model_desc* t, const mtad_model_desc* a, int max_batch, int max_nodes,
+// Lays out the workspace; with base == nullptr only measures it.  one_launch = false leaves out what only the one-launch
+// forward and its attention use.
+size_t carve(mtad_ctx* c, const mtad_model_desc* t, const mtad_model_desc* a, int max_batch, int max_nodes, bool one_launch,
              void* base, std::vector<Region>* log = nullptr) {
     Carver k(base);
     k.log = log;
     const size_t T = (size_t)max_batch * (max_nodes + 1);
     auto mx = [&](auto f) { size_t v = f(t); if (a) v = std::max(v, (size_t)f(a)); return v; };
+    auto fw = [&](auto f) { return one_launch ? mx(f) : (size_t)0; };
     const size_t d = mx([](const mtad_model_desc* m) { return (size_t)m->d_model; });
     const size_t qkv = mx([](const mtad_model_desc* m) { return (size_t)(m->n_q_heads + 2 * m->n_kv_heads) * m->head_dim; });
     const size_t qd = mx([](const mtad_model_desc* m) { return (size_t)m->n_q_heads * m->head_dim; });
@@ -225,7 +227,7 @@ size_t carve(mtad_ctx* c, const mtad_model_desc* t, const mtad_model_desc* a, in
     sc.xkv = k.take<__nv_bfloat16>((size_t)2 * TC_X_ROWS * d, "xkv");
     const size_t dt = (d + TC_TILE_N - 1) / TC_TILE_N;
     // (the one-launch forward leaves a part per block that owns features)
-    const size_t sq_parts = std::max(dt, mx([](const mtad_model_desc* m) { return fw_parts_max(*m, kCtas, false); }));
+    const size_t sq_parts = std::max(dt, fw([](const mtad_model_desc* m) { return fw_parts_max(*m, kCtas, false); }));
     sc.sumsq_a = k.take<float>(sq_parts * TC_X_ROWS, "sumsq_a");
     sc.sumsq_b = k.take<float>(sq_parts * TC_X_ROWS, "sumsq_b");
     size_t ws_tiles = 0, max_tiles = 0, lm_tiles = 0;
@@ -252,13 +254,14 @@ size_t carve(mtad_ctx* c, const mtad_model_desc* t, const mtad_model_desc* a, in
     if (a) shape_ws(a);
     sc.tc_ws = k.take<float>(ws_tiles * rpad * TC_TILE_N, "tc_ws");
     sc.tc_counters = k.take<int32_t>(max_tiles, "tc_counters");
-    sc.lm_part = k.take<float4>(Tc * std::max(lm_tiles, mx([](const mtad_model_desc* m) { return fw_parts_max(*m, kCtas, true); })),
+    sc.lm_part = k.take<float4>(Tc * std::max(lm_tiles, fw([](const mtad_model_desc* m) { return fw_parts_max(*m, kCtas, true); })),
                                 "lm_part");
-    sc.fw_sync_words = (int)mx([&](const mtad_model_desc* m) { return fw_sync_words(*m, max_batch, kCtas); });
+    sc.fw_sync_words = (int)fw([&](const mtad_model_desc* m) { return fw_sync_words(*m, max_batch, kCtas); });
     sc.fw_sync = k.take<int32_t>(sc.fw_sync_words, "fw_sync");
-    sc.fw_part = k.take<float>((size_t)kCtas * FW_MAX_ROWS * 2 * TC_TILE_N, "fw_part");
-    FwLayer* fw_t = k.take<FwLayer>(t->layers, "fw_target");
-    FwLayer* fw_a = a ? k.take<FwLayer>(a->layers, "fw_aux") : nullptr;
+    sc.fw_part = k.take<float>(fw([&](const mtad_model_desc* m) { return fw_part_floats(*m, kCtas, max_batch, max_nodes + 1); }),
+                               "fw_part");
+    FwLayer* fw_t = k.take<FwLayer>(one_launch ? t->layers : 0, "fw_target");
+    FwLayer* fw_a = a ? k.take<FwLayer>(one_launch ? a->layers : 0, "fw_aux") : nullptr;
     sc.node_z = k.take<float>(T, "node_z");
     sc.draft_part = a ? k.take<DraftPart>((size_t)max_batch * MTAD_MAX_BEAM * MTAD_DRAFT_CHUNKS, "draft_part") : nullptr;
     sc.warp_part = k.take<WarpPart>(T * MTAD_DRAFT_CHUNKS, "warp_part");
@@ -630,7 +633,7 @@ int build_plan(ForwardPlan& fp, const Scratch& sc, const RowMeta& rm, const Mode
     fp.kv_terms = tkv;
     // The attention of more than 16 query rows per KV head: 64 heads, 8 KV heads, 129 rows on 1024 keys 167 us a layer in
     // attn_mma_kernel, 77 here.  With fewer that one is as fast, without a cooperative launch between the projections.
-    fp.fw_attn = mma_attention(m) && fw_attn_plan(fp.fw, d, B, R, kCtas);
+    fp.fw_attn = sc.fw_sync_words > 0 && mma_attention(m) && fw_attn_plan(fp.fw, d, B, R, kCtas);
     if (fp.fw_attn) fw_common(fp.fw, sc, rm, m);
     return MTAD_OK;
 }
@@ -798,17 +801,31 @@ int mtad_workspace_bytes(const mtad_model_desc* target, const mtad_model_desc* a
     if (!out_bytes || !model_ok(target) || (aux && !model_ok(aux))) return MTAD_E_INVALID;
     if (max_batch < 1 || max_nodes < 0) return MTAD_E_INVALID;
     if (max_batch > MTAD_MAX_BATCH || max_nodes > MTAD_MAX_NODES) return MTAD_E_CAPACITY;
-    *out_bytes = carve(nullptr, target, aux, max_batch, max_nodes, nullptr);
+    *out_bytes = carve(nullptr, target, aux, max_batch, max_nodes, true, nullptr);
     return MTAD_OK;
 }
 
 int mtad_create(const mtad_model_desc* target, const mtad_model_desc* aux, int max_batch, int max_nodes,
                 void* workspace, size_t workspace_bytes, mtad_ctx** out) {
+    return create_context(target, aux, max_batch, max_nodes, true, workspace, workspace_bytes, out);
+}
+
+}  // extern "C"
+
+namespace mtad {
+
+size_t workspace_need(const mtad_model_desc* target, int max_batch, int max_nodes, bool one_launch) {
+    return carve(nullptr, target, nullptr, max_batch, max_nodes, one_launch, nullptr);
+}
+
+int create_context(const mtad_model_desc* target, const mtad_model_desc* aux, int max_batch, int max_nodes, bool one_launch,
+                   void* workspace, size_t workspace_bytes, mtad_ctx** out) {
     if (!out) return MTAD_E_INVALID;
     *out = nullptr;
     size_t need = 0;
     int rc = mtad_workspace_bytes(target, aux, max_batch, max_nodes, &need);
     if (rc != MTAD_OK) return rc;
+    if (!one_launch) need = carve(nullptr, target, aux, max_batch, max_nodes, false, nullptr);
     if (!model_ptrs_ok(target) || (aux && !model_ptrs_ok(aux))) return MTAD_E_INVALID;
     if (aux && aux->vocab != target->vocab) return MTAD_E_INVALID;
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) || workspace_bytes < need) return MTAD_E_WORKSPACE;
@@ -827,7 +844,7 @@ int mtad_create(const mtad_model_desc* target, const mtad_model_desc* aux, int m
     ctx->T_max = max_batch * (max_nodes + 1);
     ctx->len_ub.assign(max_batch, 0);
     ctx->npend_ub.assign(max_batch, 1);
-    carve(ctx, target, aux, max_batch, max_nodes, workspace, &ctx->regions);
+    carve(ctx, target, aux, max_batch, max_nodes, one_launch, workspace, &ctx->regions);
     ctx->ws_base = static_cast<char*>(workspace);
     // tensor-core path unless MTAD_PATH=simt asks for the CUDA-core kernels (or a weight pointer is not 16-byte aligned)
     const char* path = getenv("MTAD_PATH");
@@ -844,13 +861,17 @@ int mtad_create(const mtad_model_desc* target, const mtad_model_desc* aux, int m
         if (e == cudaSuccess) e = cudaMemset(ctx->ws_base + r.off + r.count * r.elem, 0xC5, kCanaryBytes);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) { delete ctx; return MTAD_E_CUDA; }
-    if (ctx->use_tc) {
+    if (ctx->use_tc && one_launch) {
         ctx->fw_ok[0] = ctx->target.kv_map_ok && build_forward_table(ctx->target, ctx->fw_target, ctx->fw_lm[0]);
         ctx->fw_ok[1] = aux && ctx->amaps.ok && ctx->aux.kv_map_ok && build_forward_table(ctx->aux, ctx->fw_aux, ctx->fw_lm[1]);
     }
     *out = ctx;
     return MTAD_OK;
 }
+
+}  // namespace mtad
+
+extern "C" {
 
 int mtad_destroy(mtad_ctx* ctx) {
     if (ctx)
@@ -1275,7 +1296,7 @@ int mtad_audit_extents(const mtad_model_desc* target, const mtad_model_desc* aux
     fill(c.target, target);
     if (aux) { fill(c.aux, aux); c.has_aux = true; }
     c.max_batch = max_batch; c.max_nodes = max_nodes;
-    carve(&c, target, aux, max_batch, max_nodes, nullptr, &au.regions);
+    carve(&c, target, aux, max_batch, max_nodes, true, nullptr, &au.regions);
     const int D = gamma > 0 ? gamma : 1;
     if (call == MTAD_AUDIT_VERIFY) {
         const int R = nodes + 1;

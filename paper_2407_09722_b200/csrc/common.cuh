@@ -387,4 +387,10 @@ cudaError_t launch_aux_commit(const ModelView& aux, const SeqState& s, const Dra
 cudaError_t launch_seq_set(const SeqState& s, int seq, int kv_len, int root, int aux_len, int npend,
                            const int32_t* pend_host, cudaStream_t st);
 
+// A context whose workspace may leave out what only the one-launch forward uses (one_launch = false: every call runs as a chain
+// of launches), and the bytes it takes.
+size_t workspace_need(const mtad_model_desc* target, int max_batch, int max_nodes, bool one_launch);
+int create_context(const mtad_model_desc* target, const mtad_model_desc* aux, int max_batch, int max_nodes, bool one_launch,
+                   void* workspace, size_t workspace_bytes, mtad_ctx** out);
+
 }  // namespace mtad

@@ -1624,6 +1624,10 @@ static int fw_slots(const mtad_model_desc& d, int cls) {
     return d.d_model <= 2048 && (256 + FW_CLASS[cls].cols) * 128 <= FW_RING / 4 ? 4 : FW_CLASS[cls].slots;
 }
 
+// Up to eight rows the lean epilogues (an element per thread, a warp per row: beyond, a row would wait for its turn), which know
+// no split projections.
+static bool fw_few(int T, int query_rows) { return T <= 8 && query_rows <= FW_QROWS; }
+
 void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta, int cls) {
     const int qd = d.n_q_heads * d.head_dim, hp = d.head_dim / 2, heads = d.n_q_heads + 2 * d.n_kv_heads;
     const int cols = FW_CLASS[cls].cols, slot = FW_RING / fw_slots(d, cls);
@@ -1717,8 +1721,7 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
     const bool wide = G * R > FW_QROWS;
     a.nqb = wide ? up_div(G * R, FW_QROWS_WIDE) : 1;
     a.qrows = up_div(G * R, a.nqb);
-    // Up to eight rows the lean epilogues (an element per thread, a warp per row: beyond, a row would wait for its turn).
-    a.cls = T <= 8 && !wide ? 0 : 2;
+    a.cls = fw_few(T, G * R) ? 0 : 2;
     while (FW_CLASS[a.cls].cols < a.cols) ++a.cls;
     a.slots = fw_slots(d, a.cls);
     fw_geometry(a.ph, d, n_cta, a.cls);
@@ -1800,6 +1803,19 @@ size_t fw_parts_max(const mtad_model_desc& d, int n_cta, bool lm) {
             if ((k == FW_LM) == lm) most = std::max(most, (size_t)(ph[k].n_tiles / ph[k].c));
     }
     return most;
+}
+
+size_t fw_part_floats(const mtad_model_desc& d, int n_cta, int max_batch, int max_rows) {
+    const int T = max_batch * max_rows;
+    if (fw_few(T, d.n_q_heads / d.n_kv_heads * max_rows)) return 0;
+    size_t most = 0;
+    for (int c = 2; c < FW_CLASSES; ++c) {
+        FwPhase ph[6];
+        fw_geometry(ph, d, n_cta, c);
+        for (int k : {FW_QKV, FW_O, FW_DOWN})               // (a box's k-blocks side by side are 128 rows at most)
+            if (ph[k].c > 1) most = std::max(most, (size_t)ph[k].n_tiles * ph[k].nbox * TC_TILE_N);
+    }
+    return most * std::min(T, FW_MAX_ROWS);
 }
 
 cudaError_t launch_forward(const FwArgs& a, cudaStream_t st) {

@@ -90,6 +90,8 @@ inline size_t fw_pairs(const mtad_model_desc& d, int max_batch) {
 inline size_t fw_sync_words(const mtad_model_desc& d, int max_batch, int n_cta) {
     return (size_t)5 * d.layers + 1 + fw_pairs(d, max_batch) + 3 * (size_t)n_cta;
 }
+// partial sums of the split projections of calls of up to max_batch x max_rows rows
+size_t fw_part_floats(const mtad_model_desc& d, int n_cta, int max_batch, int max_rows);
 cudaError_t launch_forward(const FwArgs& a, cudaStream_t st);
 cudaError_t launch_forward_attention(FwArgs& a, int layer, cudaStream_t st);
 

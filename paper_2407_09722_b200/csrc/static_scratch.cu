@@ -45,7 +45,9 @@ extern "C" int mtad_verify_chain_static(const mtad_model_desc* target, int32_t k
     size_t need = 0;
     int rc = mtad_workspace_bytes(target, nullptr, 1, gamma, &need);
     if (rc != MTAD_OK) return rc;
-    if (need > (size_t)MTAD_STATIC_SCRATCH_BYTES) return MTAD_E_WORKSPACE;   // model or chain too large for the array
+    // what is too large for the array with the one-launch forward's tables and partial sums may fit without
+    const bool one_launch = need <= (size_t)MTAD_STATIC_SCRATCH_BYTES;
+    if (!one_launch && mtad::workspace_need(target, 1, gamma, false) > (size_t)MTAD_STATIC_SCRATCH_BYTES) return MTAD_E_WORKSPACE;
 
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return MTAD_E_CUDA;
@@ -65,7 +67,7 @@ extern "C" int mtad_verify_chain_static(const mtad_model_desc* target, int32_t k
         if (p.ctx) { mtad_destroy(p.ctx); p.ctx = nullptr; }
         // mtad_create lays the step's scratch out inside the array and zeroes it (the array still holds the
         // previous caller's data); it allocates no device memory itself.
-        rc = mtad_create(target, nullptr, 1, gamma, p.scratch, MTAD_STATIC_SCRATCH_BYTES, &p.ctx);
+        rc = mtad::create_context(target, nullptr, 1, gamma, one_launch, p.scratch, MTAD_STATIC_SCRATCH_BYTES, &p.ctx);
         if (rc != MTAD_OK) { p.ctx = nullptr; return rc; }
         p.desc = *target;
         p.lw.assign(target->layer_weights, target->layer_weights + (size_t)target->layers * MTAD_LAYER_TENSORS);
