@@ -107,7 +107,9 @@ int mtad_workspace_bytes(const mtad_model_desc* target, const mtad_model_desc* a
 
 /* Create a context.  workspace: device memory, 256-byte aligned, at least mtad_workspace_bytes(); it is zeroed
  * and the call synchronises the device.  The descriptors (and the host pointer arrays in them) are copied; the
- * device memory they point to stays the caller's.  All sequences start empty (L = 0, root token 0). */
+ * device memory they point to stays the caller's.  All sequences start empty (L = 0, root token 0).  Calls of up to 72
+ * rows run their decoder forward as one cooperative launch of 148 blocks with an SM each; where the device, or the part
+ * of it that the process may use, has fewer SMs, as a chain of launches (the results differ by fp32 rounding). */
 int mtad_create(const mtad_model_desc* target, const mtad_model_desc* aux, int max_batch, int max_nodes,
                 void* workspace, size_t workspace_bytes, mtad_ctx** out);
 int mtad_destroy(mtad_ctx* ctx);
@@ -304,6 +306,11 @@ int mtad_debug_region(const mtad_ctx* ctx, const char* name, size_t* offset, siz
  * and every sequence of the call reports MTAD_ST_TIMEOUT.  The kernels return normally; a later call with the hook
  * switched off is unaffected. */
 int mtad_debug_set_wait(mtad_ctx* ctx, unsigned int wait_limit, int no_operands);
+
+/* Test hook: path 0 runs every call of the context as a chain of launches, as on a device that cannot hold the blocks of
+ * the one-launch forward at once; 1 goes back to the default; 2 lets its launches be refused by the driver once, as
+ * when the process is given fewer SMs later on. */
+int mtad_debug_set_path(mtad_ctx* ctx, int path);
 
 const char* mtad_status_str(int status);
 int mtad_last_cuda_error(const mtad_ctx* ctx);

@@ -48,7 +48,7 @@ EXPORTS = ("mtad_workspace_bytes", "mtad_create", "mtad_destroy", "mtad_seq_set"
            "mtad_profile_begin", "mtad_profile_end", "mtad_kernel_launches", "mtad_verify_chain_static",
            "mtad_debug_gemm", "mtad_set_warp", "mtad_set_draft_warp", "mtad_profile_grouped",
            "mtad_verify_chain_spd", "mtad_seq_hint", "mtad_debug_set_wait", "mtad_audit_extents",
-           "mtad_debug_check_canaries", "mtad_debug_region")
+           "mtad_debug_check_canaries", "mtad_debug_region", "mtad_debug_set_path")
 MTAD_STATIC_SCRATCH_BYTES = 16 << 20
 MTAD_ST_TIMEOUT, MTAD_ST_AUX_PENDING, MTAD_ST_NONFINITE, MTAD_ST_RANGE = 32, 64, 128, 256      # device status bits (mtad.h)
 KERNEL_CLASSES = ("prepare", "norm", "gemm", "rope_append", "attention", "lm_reduce", "accept", "commit")
@@ -78,6 +78,7 @@ def load_library() -> C.CDLL:
     lib.mtad_seq_hint.argtypes = [P, I, C.c_int32]
     lib.mtad_audit_extents.argtypes = [MD, MD, I, I, I, I, I, I, I, C.c_int64, C.POINTER(Extent), I, C.POINTER(I)]
     lib.mtad_debug_set_wait.argtypes = [P, C.c_uint, I]
+    lib.mtad_debug_set_path.argtypes = [P, I]
     lib.mtad_debug_region.argtypes = [P, C.c_char_p, C.POINTER(C.c_size_t), C.POINTER(C.c_size_t), C.POINTER(C.c_size_t)]
     lib.mtad_debug_check_canaries.argtypes = [P, P, C.POINTER(C.c_char_p)]
     lib.mtad_profile_grouped.argtypes = [P, I]
@@ -251,6 +252,9 @@ class Context:
     def mtad_debug_set_wait(self, wait_limit: int, no_operands: bool):
         self._check(self._lib.mtad_debug_set_wait(self.handle, wait_limit, 1 if no_operands else 0),
                     "mtad_debug_set_wait")
+
+    def mtad_debug_set_path(self, path: int):
+        self._check(self._lib.mtad_debug_set_path(self.handle, path), "mtad_debug_set_path")
 
     def region(self, name: str, dtype) -> torch.Tensor:
         """View of the workspace array `name` (a live view of device memory, for tests)."""

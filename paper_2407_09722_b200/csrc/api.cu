@@ -57,7 +57,9 @@ struct mtad_ctx {
     WeightMaps tmaps, amaps;
     FwLayer *fw_target = nullptr, *fw_aux = nullptr;   // device tables of the one-launch forward (in the workspace)
     CUtensorMap fw_lm[2][FW_CLASSES];                  // its LM-head maps: target, auxiliary model
-    bool fw_ok[2] = {false, false};
+    bool fw_ok[2] = {false, false};                    // the table and maps of the target, of the auxiliary model are there
+    bool resident = false;              // a cooperative launch of kCtas blocks is possible, as far as is known
+    bool refuse_resident = false;       // debug: such launches ask for more blocks than fit
     bool use_tc = false, use_pdl = false;
     size_t tc_ws_floats = 0, tc_counter_n = 0, xf_elems = 0;
     ModelView target, aux;
@@ -490,7 +492,7 @@ void build_kv_map(ModelView& m) {
 // Builds the plan.  with_maps = false leaves out everything that needs the driver (the operand-row tensor maps) and
 // the weight maps: what is left is the index arithmetic of the launches.
 int build_plan(ForwardPlan& fp, const Scratch& sc, const RowMeta& rm, const ModelView& m, const WeightMaps* wm, int B,
-               int R, bool lm_plain, bool with_maps, bool split_kv_ok) {
+               int R, bool lm_plain, bool with_maps, bool split_kv_ok, bool fw_attn_ok) {
     const int T = B * R;
     const mtad_model_desc& d = m.d;
     const int qd = d.n_q_heads * d.head_dim, kvd = d.n_kv_heads * d.head_dim;
@@ -633,7 +635,7 @@ int build_plan(ForwardPlan& fp, const Scratch& sc, const RowMeta& rm, const Mode
     fp.kv_terms = tkv;
     // The attention of more than 16 query rows per KV head: 64 heads, 8 KV heads, 129 rows on 1024 keys 167 us a layer in
     // attn_mma_kernel, 77 here.  With fewer that one is as fast, without a cooperative launch between the projections.
-    fp.fw_attn = sc.fw_sync_words > 0 && mma_attention(m) && fw_attn_plan(fp.fw, d, B, R, kCtas);
+    fp.fw_attn = fw_attn_ok && mma_attention(m) && fw_attn_plan(fp.fw, d, B, R, kCtas);
     if (fp.fw_attn) fw_common(fp.fw, sc, rm, m);
     return MTAD_OK;
 }
@@ -660,19 +662,33 @@ int forward_rows_tc(mtad_ctx* ctx, const ModelView& m, const WeightMaps& wm, int
     if (it == ctx->plans.end()) {
         ForwardPlan fp;
         const bool aux = &m == &ctx->aux;
-        if (!(ctx->fw_ok[aux] && build_forward_plan(fp, sc, ctx->rm, m, aux ? ctx->fw_aux : ctx->fw_target, ctx->fw_lm[aux], B, R,
+        if (!(ctx->resident && ctx->fw_ok[aux] && build_forward_plan(fp, sc, ctx->rm, m, aux ? ctx->fw_aux : ctx->fw_target, ctx->fw_lm[aux], B, R,
                                                     lm_plain, true))) {
             fp = ForwardPlan();
-            if (int rc = build_plan(fp, sc, ctx->rm, m, &wm, B, R, lm_plain, true, !aux)) return rc;
+            if (int rc = build_plan(fp, sc, ctx->rm, m, &wm, B, R, lm_plain, true, !aux, ctx->resident)) return rc;
         }
         it = ctx->plans.emplace(key, std::move(fp)).first;
     }
     ForwardPlan& fp = it->second;
+    // A cooperative launch that the driver refuses, because the process may use fewer SMs now than when the context was made:
+    // nothing has been launched then, and this call and those that follow run as a chain of launches.
+    auto too_large = [&](int rc) {
+        if (rc != MTAD_E_CUDA || ctx->last_cuda != (int)cudaErrorCooperativeLaunchTooLarge) return false;
+        (void)cudaGetLastError();
+        ctx->last_cuda = 0;
+        ctx->resident = false;
+        return true;
+    };
     if (fp.one_launch) {
         fp.fw.status = status; fp.fw.uniforms = uniforms;
         fp.fw.wait_limit = ctx->wait_limit; fp.fw.debug_no_operands = ctx->debug_no_operands;
         fp.fw.pieces = (int)((total + FW_KEYS - 1) / FW_KEYS);
-        RUN(MTAD_K_GEMM, fp.fw_bytes, 1, launch_forward(fp.fw, s));
+        const int rc = timed(ctx, MTAD_K_GEMM, fp.fw_bytes, 1, s, [&] { return launch_forward(fp.fw, s, ctx->refuse_resident); });
+        if (too_large(rc)) {
+            ctx->plans.clear();
+            return forward_rows_tc(ctx, m, wm, B, R, len_ub, uniforms, status, lm_plain, s);
+        }
+        if (rc != MTAD_OK) return rc;
         if (!lm_plain) RUN(MTAD_K_LMRED, 0, 2, launch_lm_merge(m, ctx->rm, sc, B, R, fp.lm_tiles128, uniforms, status, s));
         return MTAD_OK;
     }
@@ -694,15 +710,19 @@ int forward_rows_tc(mtad_ctx* ctx, const ModelView& m, const WeightMaps& wm, int
     for (size_t i = 0; i < fp.g.size(); ++i) {
         if (fp.g[i].attn_before) {                               // the O projection: the attention pass feeds it
             const int l = layer++;
-            if (fp.fw_attn) {
+            bool done = false;
+            if (fp.fw_attn && ctx->resident) {
                 fp.fw.status = status; fp.fw.wait_limit = ctx->wait_limit;
                 fp.fw.pieces = (int)((total + FW_KEYS - 1) / FW_KEYS);
-                RUN(MTAD_K_ATTN, 0, 1, launch_forward_attention(fp.fw, l, s));
-            } else if (mma_attention(m)) {
+                const int rc = timed(ctx, MTAD_K_ATTN, 0, 1, s, [&] { return launch_forward_attention(fp.fw, l, s, ctx->refuse_resident); });
+                if (rc != MTAD_OK && !too_large(rc)) return rc;
+                done = rc == MTAD_OK;
+            }
+            if (!done && mma_attention(m)) {
                 const AttnSplit as = attn_split(m, B, R, total);
                 RUN(MTAD_K_ATTN, 0, 2, launch_attention_mma(m, l, ctx->rm, sc, B, R, as.ns, as.nsp, status, pdl, s));
                 RUN(MTAD_K_ATTN, 0, 0, launch_attention_combine(m, ctx->rm, sc, B, R, as.ns, true, pdl, s));
-            } else {
+            } else if (!done) {
                 int nsplit = (int)std::min<long long>(attn_split_cap(d.n_q_heads), (total + MTAD_ATTN_TILE - 1) / MTAD_ATTN_TILE);
                 nsplit = std::max(1, std::min(nsplit, (4 * 148 + d.n_q_heads * B - 1) / (d.n_q_heads * B)));
                 long long chunk = (total + nsplit - 1) / nsplit;
@@ -861,6 +881,8 @@ int create_context(const mtad_model_desc* target, const mtad_model_desc* aux, in
         if (e == cudaSuccess) e = cudaMemset(ctx->ws_base + r.off + r.count * r.elem, 0xC5, kCanaryBytes);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) { delete ctx; return MTAD_E_CUDA; }
+    // (a plan made while such launches were possible is used only as long as they are)
+    ctx->resident = ctx->use_tc && one_launch && forward_fits(kCtas);
     if (ctx->use_tc && one_launch) {
         ctx->fw_ok[0] = ctx->target.kv_map_ok && build_forward_table(ctx->target, ctx->fw_target, ctx->fw_lm[0]);
         ctx->fw_ok[1] = aux && ctx->amaps.ok && ctx->aux.kv_map_ok && build_forward_table(ctx->aux, ctx->fw_aux, ctx->fw_lm[1]);
@@ -1031,6 +1053,14 @@ int mtad_debug_set_wait(mtad_ctx* ctx, unsigned int wait_limit, int no_operands)
     return MTAD_OK;
 }
 
+int mtad_debug_set_path(mtad_ctx* ctx, int path) {
+    if (!ctx || path < 0 || path > 2) return MTAD_E_INVALID;
+    ctx->plans.clear();
+    ctx->refuse_resident = path == 2;
+    ctx->resident = path != 0 && ctx->use_tc && ctx->sc.fw_sync_words > 0 && forward_fits(kCtas);
+    return MTAD_OK;
+}
+
 int mtad_seq_get(mtad_ctx* ctx, int seq, int32_t* kv_len, int32_t* root_token, void* stream) {
     if (!ctx || seq < 0 || seq >= ctx->max_batch) return MTAD_E_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -1194,7 +1224,8 @@ void audit_forward(Audit& au, const mtad_ctx& c, const ModelView& m, int B, int 
     au.ws("sumsq_a", T);
     ForwardPlan fp;
     if (build_forward_plan(fp, c.sc, c.rm, m, nullptr, nullptr, B, R, lm_plain, false)) {
-        // the one-launch forward: what its epilogues and its attention index
+        // the one-launch forward: what its epilogues and its attention index (and, below, the chain of launches that the call
+        // takes on a device that cannot hold the one launch)
         const FwArgs& a = fp.fw;
         const long long cap = d.kv_capacity, total = std::min<long long>(len_ub, cap) + R;
         const long long slot_max = std::min<long long>(len_ub + R - 1, cap - 1), pieces = (total + FW_KEYS - 1) / FW_KEYS;
@@ -1217,10 +1248,9 @@ void audit_forward(Audit& au, const mtad_ctx& c, const ModelView& m, int B, int 
         au.ext("operand rows of a box", a.cols, 2 * TC_X_ROWS);
         au.ext("kv_map_planes", (size_t)((d.layers - 1) * m.max_batch + (m.max_batch - 1)) * 2 * Hkv + 2 * Hkv,
                (size_t)d.layers * m.max_batch * 2 * Hkv);
-        return;
     }
     fp = ForwardPlan();
-    build_plan(fp, c.sc, c.rm, m, nullptr, B, R, lm_plain, false, &m == &c.target);
+    build_plan(fp, c.sc, c.rm, m, nullptr, B, R, lm_plain, false, &m == &c.target, true);
     if (fp.split_kv) au.ws("xkv", idx_xrow(T - 1, fp.kv_terms, fp.kv_terms - 1, d.d_model, d.d_model - 1) + 1);
     const long long cap = d.kv_capacity;
     const long long slot_max = std::min<long long>(len_ub + R - 1, cap - 1);     // prepare refuses rows past the capacity

@@ -1788,10 +1788,10 @@ bool fw_attn_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) 
     return true;
 }
 
-cudaError_t launch_forward_attention(FwArgs& a, int layer, cudaStream_t st) {
+cudaError_t launch_forward_attention(FwArgs& a, int layer, cudaStream_t st, bool refuse) {
     a.p_lo = 5 * layer + FW_ATTN;
     a.p_hi = a.p_lo + 1;
-    return launch_forward(a, st);
+    return launch_forward(a, st, refuse);
 }
 
 size_t fw_parts_max(const mtad_model_desc& d, int n_cta, bool lm) {
@@ -1818,13 +1818,22 @@ size_t fw_part_floats(const mtad_model_desc& d, int n_cta, int max_batch, int ma
     return most * std::min(T, FW_MAX_ROWS);
 }
 
-cudaError_t launch_forward(const FwArgs& a, cudaStream_t st) {
+bool forward_fits(int n_cta) {
+    int dev = 0, sms = 0, coop = 0, smem = 0;
+    // (a block per SM: each asks for nearly all of an SM's shared memory)
+    return cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
+           sms >= n_cta && coop && smem >= 227 * 1024;
+}
+
+cudaError_t launch_forward(const FwArgs& a, cudaStream_t st, bool refuse) {
     const size_t smem = (size_t)FW_RING + FW_UNION + sizeof(FwTail);
     auto go = [&](auto kernel) -> cudaError_t {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(a.n_cta);
+        cfg.gridDim = dim3(refuse ? 1 << 20 : a.n_cta);
         cfg.blockDim = dim3(FW_THREADS);
         cfg.dynamicSmemBytes = smem;
         cfg.stream = st;

@@ -92,7 +92,10 @@ inline size_t fw_sync_words(const mtad_model_desc& d, int max_batch, int n_cta) 
 }
 // partial sums of the split projections of calls of up to max_batch x max_rows rows
 size_t fw_part_floats(const mtad_model_desc& d, int n_cta, int max_batch, int max_rows);
-cudaError_t launch_forward(const FwArgs& a, cudaStream_t st);
-cudaError_t launch_forward_attention(FwArgs& a, int layer, cudaStream_t st);
+// Its blocks wait on one another: whether the current device holds n_cta of them at once.  A launch that does not fit returns
+// cudaErrorCooperativeLaunchTooLarge and does nothing (`refuse`, for tests: ask for more blocks than any device holds).
+bool forward_fits(int n_cta);
+cudaError_t launch_forward(const FwArgs& a, cudaStream_t st, bool refuse = false);
+cudaError_t launch_forward_attention(FwArgs& a, int layer, cudaStream_t st, bool refuse = false);
 
 }  // namespace mtad

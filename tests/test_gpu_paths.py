@@ -1,0 +1,43 @@
+"""A device, or a part of one, that cannot hold the blocks of the one-launch forward at once: its calls, and those whose
+attention alone is such a launch, run as a chain of launches with the attention of mma.sync warps, whether that is known
+when the context is made or the driver refuses the launch later.  Compared with the CPU oracle at the edges of that
+attention's variants (query rows per KV head: a packed tile, one, two, up to four, five and more tiles of 16)."""
+import numpy as np
+import pytest
+import torch
+
+import mtad_synth as S
+from paper_2407_09722_b200 import binding as Bn
+from tests.parity import GpuModel, SeqCase, ParityStats, compare
+
+pytestmark = pytest.mark.gpu
+MHA64 = S.ModelShape(2, 256, 4, 4, 64, 688, 1000)
+GQA128 = S.ModelShape(2, 512, 8, 2, 128, 1024, 640)              # four query rows of a KV head per row of a call
+
+
+def _compare(gm, rows, tree, lengths, it=0):
+    sh, stats, cases = gm.shape, ParityStats(), []
+    for b, L in enumerate(lengths):
+        gm.inject(b, L)
+        t = S.beam_tree(*tree, sh.vocab, stream=270 + b) if tree else S.chain_tree(rows - 1, sh.vocab, stream=250 + b)
+        assert len(t.tok) == rows - 1
+        cases.append(SeqCase(b, L, int(S.token_ids(9, (23 << 40) | b, 1, sh.vocab)[0]), t))
+    compare(gm, cases, Bn.log_tau(0.3), S.bonus_uniforms(9, rows + it, len(lengths), sh.vocab, "cuda"), chain=tree is None,
+            stats=stats)
+    assert stats.ok(), stats
+
+
+@pytest.mark.parametrize("path", [0, 2])
+@pytest.mark.parametrize("shape,rows,tree,lengths", [
+    (MHA64, 5, None, [130]), (MHA64, 9, None, [64]), (MHA64, 17, (4, 4, 2), [100]), (MHA64, 33, (4, 8, 4), [65]),
+    (MHA64, 71, (7, 10, 2), [129]), (MHA64, 97, (8, 12, 4), [200]), (GQA128, 2, None, [63, 1]), (GQA128, 7, None, [90, 128, 5]),
+    (GQA128, 33, (4, 8, 4), [127])])
+def test_chain_of_launches(shape, rows, tree, lengths, path):
+    gm = GpuModel(shape, max_batch=len(lengths), max_nodes=rows, capacity=320)
+    launches = []
+    for it, p in enumerate((path, 1)):                           # and back: the plans of the other path are not kept
+        gm.ctx.mtad_debug_set_path(p)
+        n = Bn.mtad_kernel_launches()
+        _compare(gm, rows, tree, lengths, it)
+        launches.append(Bn.mtad_kernel_launches() - n)
+    assert launches[0] > launches[1] or rows * len(lengths) > 72, launches
