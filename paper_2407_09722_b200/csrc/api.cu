@@ -53,7 +53,7 @@ struct ForwardPlan {
 struct mtad_ctx {
     std::vector<Region> regions;        // the workspace's arrays, each followed by kCanaryBytes of guard pattern
     char* ws_base = nullptr;
-    std::map<uint64_t, ForwardPlan> plans;   // by (model, sequences, rows per sequence, LM-head mode)
+    std::map<uint64_t, ForwardPlan> plans;   // by (model, sequences, rows per sequence, LM-head mode, one launch or a chain)
     WeightMaps tmaps, amaps;
     FwLayer *fw_target = nullptr, *fw_aux = nullptr;   // device tables of the one-launch forward (in the workspace)
     CUtensorMap fw_lm[2][FW_CLASSES];                  // its LM-head maps: target, auxiliary model
@@ -633,8 +633,7 @@ int build_plan(ForwardPlan& fp, const Scratch& sc, const RowMeta& rm, const Mode
     fp.maps = with_maps;
     fp.split_kv = split_kv;
     fp.kv_terms = tkv;
-    // The attention of more than 16 query rows per KV head: 64 heads, 8 KV heads, 129 rows on 1024 keys 167 us a layer in
-    // attn_mma_kernel, 77 here.  With fewer that one is as fast, without a cooperative launch between the projections.
+    // (taken where fw_attn_pays; up to 16 query rows per KV head attn_mma_kernel always)
     fp.fw_attn = fw_attn_ok && mma_attention(m) && fw_attn_plan(fp.fw, d, B, R, kCtas);
     if (fp.fw_attn) fw_common(fp.fw, sc, rm, m);
     return MTAD_OK;
@@ -656,13 +655,14 @@ int forward_rows_tc(mtad_ctx* ctx, const ModelView& m, const WeightMaps& wm, int
     const Scratch& sc = ctx->sc;
     const long long total = std::min<long long>(len_ub, d.kv_capacity) + R;
     const bool pdl = ctx->use_pdl;
+    const bool one = ctx->resident && ctx->fw_ok[&m == &ctx->aux] && fw_pays(d, B, R, total);
     const uint64_t key = ((uint64_t)(&m == &ctx->aux ? 1 : 0) << 40) | ((uint64_t)B << 24) | ((uint64_t)R << 8) |
-                         (lm_plain ? 1u : 0u);
+                         (lm_plain ? 1u : 0u) | (one ? 2u : 0u);
     auto it = ctx->plans.find(key);
     if (it == ctx->plans.end()) {
         ForwardPlan fp;
         const bool aux = &m == &ctx->aux;
-        if (!(ctx->resident && ctx->fw_ok[aux] && build_forward_plan(fp, sc, ctx->rm, m, aux ? ctx->fw_aux : ctx->fw_target, ctx->fw_lm[aux], B, R,
+        if (!(one && build_forward_plan(fp, sc, ctx->rm, m, aux ? ctx->fw_aux : ctx->fw_target, ctx->fw_lm[aux], B, R,
                                                     lm_plain, true))) {
             fp = ForwardPlan();
             if (int rc = build_plan(fp, sc, ctx->rm, m, &wm, B, R, lm_plain, true, !aux, ctx->resident)) return rc;
@@ -711,7 +711,7 @@ int forward_rows_tc(mtad_ctx* ctx, const ModelView& m, const WeightMaps& wm, int
         if (fp.g[i].attn_before) {                               // the O projection: the attention pass feeds it
             const int l = layer++;
             bool done = false;
-            if (fp.fw_attn && ctx->resident) {
+            if (fp.fw_attn && ctx->resident && fw_attn_pays(d, B, R, total)) {
                 fp.fw.status = status; fp.fw.wait_limit = ctx->wait_limit;
                 fp.fw.pieces = (int)((total + FW_KEYS - 1) / FW_KEYS);
                 const int rc = timed(ctx, MTAD_K_ATTN, 0, 1, s, [&] { return launch_forward_attention(fp.fw, l, s, ctx->refuse_resident); });

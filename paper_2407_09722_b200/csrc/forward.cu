@@ -1777,6 +1777,34 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
     return true;
 }
 
+// A (sequence, KV head) costs the attention of the one launch about 2 us beside its tiles, and a tile takes as long with one
+// query row as with eight.  With heads of 128 its tiles are bound by their bytes all the same (64 sequences of one row, 7B
+// width: 0.96..1.01 of the chain); with heads of 64 the mma.sync warps, which spread over more blocks, are faster from some
+// number of sequences on.  Measured, chain -> one launch, us of a step (eight layers of width 2048, 32 heads of 64): 64 x 1
+// rows, 64 / 512 / 2048 / 4096 keys 1111 -> 1196, 1343 -> 1498, 2050 -> 2616, 3011 -> 4045; 40 x 1, 2048 keys 1520 -> 1667;
+// 32 x 1, 2048 keys 1383 -> 1454; 28 x 2, 4096 keys 1958 -> 1909; 24 x 1 1646 -> 1628; 18 x 4, 2048 and 4096 keys 1306 ->
+// 1286, 1618 -> 1712; 8 x 8, 8192 and 16384 keys 1430 -> 1455, 2076 -> 2201.  A draft of the 13B pair (16 heads), 64 x 1, 2048
+// keys 1404 -> 1643; 32 x 2 1127 -> 1159; 32 x 1 1023 -> 1002.
+bool fw_pays(const mtad_model_desc& d, int B, int R, long long total) {
+    if (d.head_dim != 64) return true;
+    const long long heads = (long long)B * d.n_kv_heads, tiles = heads * ((total + FW_KEYS - 1) / FW_KEYS);
+    return B <= 32 && heads < 1000 && (B * R < 64 || (B < 32 && tiles < 80 * 148));
+}
+
+// The launch of its own costs 7..10 us more a layer than attn_mma_kernel's two, which overlap their neighbours; it gains by
+// its tiles: with more than 96 query rows per KV head, six tiles of 16, that kernel takes them in rounds, and with heads of
+// 128 it is slower by the key from 17 rows on.  Measured a step of eight layers, attn_mma_kernel -> here, us: 64 heads of 128
+// on 8 KV heads, 129 rows, 1024 keys 7682 -> 6770, 6 x 18 rows 5317 -> 5359, 2048 keys 5704 -> 5441; 32 heads of 128 on as
+// many, 81 rows, 16 / 1024 / 4096 keys 1588 -> 1644, 1770 -> 1719, 2119 -> 1964; 129 rows 2780 -> 2695, 3028 -> 2833, 3944 ->
+// 3140; 6 x 18 rows, 1024 and 4096 keys 2089 -> 2136, 2681 -> 2586; 32 heads of 64 on as many, 81 rows 945 -> 996, 996 ->
+// 1076, 1133 -> 1308; 97 rows, 64 and 2048 keys 1013 -> 1050, 1293 -> 1195; 32 heads of 64 on 8, 4 x 30 rows, 256 and 2048
+// keys 1052 -> 1074, 1298 -> 1220; 81 rows 1049 -> 978, 1209 -> 1101.
+bool fw_attn_pays(const mtad_model_desc& d, int B, int R, long long total) {
+    const int tiles = (d.n_q_heads / d.n_kv_heads * R + 15) / 16;
+    if (total >= 2048) return tiles > 6 || (d.head_dim == 128 && B <= 8);
+    return B <= 4 && tiles > (d.head_dim == 128 ? 6 : 9);
+}
+
 bool fw_attn_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
     const int G = d.n_q_heads / d.n_kv_heads;
     if ((d.head_dim != 64 && d.head_dim != 128) || G * R <= FW_QROWS || B * R > TC_MAX_ROWS || B > MTAD_MAX_BATCH) return false;

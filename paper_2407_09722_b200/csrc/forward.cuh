@@ -80,6 +80,10 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta);
 // The attention alone, wide variant, for a call whose projections run as launches of their own; run for one layer with
 // launch_forward_attention.
 bool fw_attn_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta);
+// Whether the one-launch forward of a call of B x R rows, of up to `total` keys a sequence, is the faster one; the same of the
+// wide attention as a launch of its own.
+bool fw_pays(const mtad_model_desc& d, int B, int R, long long total);
+bool fw_attn_pays(const mtad_model_desc& d, int B, int R, long long total);
 size_t fw_parts_max(const mtad_model_desc& d, int n_cta, bool lm);
 // (sequence, KV head, query block)s of a call at most: B * ceil(G R / rows) with B R <= TC_MAX_ROWS
 inline size_t fw_pairs(const mtad_model_desc& d, int max_batch) {

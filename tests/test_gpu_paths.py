@@ -41,3 +41,37 @@ def test_chain_of_launches(shape, rows, tree, lengths, path):
         _compare(gm, rows, tree, lengths, it)
         launches.append(Bn.mtad_kernel_launches() - n)
     assert launches[0] > launches[1] or rows * len(lengths) > 72, launches
+
+
+@pytest.mark.parametrize("shape,rows,tree,lengths,chain", [
+    (S.ModelShape(1, 256, 32, 32, 64, 512, 500), 1, None, [40 + 5 * b for b in range(33)], True),      # 33 sequences
+    (S.ModelShape(1, 256, 32, 32, 64, 512, 500), 2, None, [30 + 9 * b for b in range(31)], False),     # 31 x 32 KV heads
+    (S.ModelShape(1, 256, 32, 32, 64, 512, 500), 1, None, [64] * 32, True),                            # 32 x 32
+    (S.ModelShape(1, 256, 2, 2, 64, 512, 500), 2, None, [20 + b for b in range(32)], True),            # 64 rows of 32
+    (S.ModelShape(1, 256, 2, 2, 128, 512, 500), 2, None, [20 + b for b in range(32)], False),          # heads of 128
+    (MHA64, 81, (5, 16, 4), [90], True), (MHA64, 97, (8, 12, 4), [90], True),                          # six tiles of 16, seven
+    (MHA64, 145, (9, 16, 4), [90], False), (GQA128, 81, (5, 16, 4), [90], False),
+])
+def test_the_faster_way_is_taken(shape, rows, tree, lengths, chain):
+    """Few long calls as one launch (beyond 72 rows: their attention), calls of many sequences with heads of 64 as a chain."""
+    gm = GpuModel(shape, max_batch=len(lengths), max_nodes=max(rows - 1, 1), capacity=480)
+    launches = []
+    for it, path in enumerate((1, 0)):
+        gm.ctx.mtad_debug_set_path(path)
+        n = Bn.mtad_kernel_launches()
+        _compare(gm, rows, tree, lengths, it)
+        launches.append(Bn.mtad_kernel_launches() - n)
+    assert (launches[0] == launches[1]) == chain, launches
+
+
+
+@pytest.mark.parametrize("shape,wide", [(S.ModelShape(2, 256, 2, 2, 128, 512, 500), True), (MHA64, False)])
+def test_keys_from_which_the_wide_attention_is_taken(shape, wide):
+    """Three tiles of query rows a KV head: mma.sync warps up to 2047 keys, and with heads of 64 beyond them."""
+    gm = GpuModel(shape, max_batch=2, max_nodes=40, capacity=2100)
+    used = []
+    for L in (2006, 2007):
+        n = Bn.mtad_kernel_launches()
+        _compare(gm, 41, (4, 10, 2), [L, 50], L)
+        used.append(Bn.mtad_kernel_launches() - n)
+    assert used[0] - used[1] == (shape.layers if wide else 0), used        # (two launches a layer, one)
