@@ -107,7 +107,7 @@ int mtad_workspace_bytes(const mtad_model_desc* target, const mtad_model_desc* a
 
 /* Create a context.  workspace: device memory, 256-byte aligned, at least mtad_workspace_bytes(); it is zeroed
  * and the call synchronises the device.  The descriptors (and the host pointer arrays in them) are copied; the
- * device memory they point to stays the caller's.  All sequences start empty (L = 0, root token 0).  Calls of up to 72
+ * device memory they point to stays the caller's.  All sequences start empty (L = 0, root token 0).  Calls of up to 80
  * rows run their decoder forward as one cooperative launch of 148 blocks with an SM each; where the device, or the part
  * of it that the process may use, has fewer SMs, as a chain of launches (the results differ by fp32 rounding). */
 int mtad_create(const mtad_model_desc* target, const mtad_model_desc* aux, int max_batch, int max_nodes,

@@ -56,6 +56,7 @@ constexpr int FW_UNION = 32 * 1024;       // epilogue tile Y, or the attention's
 constexpr int FW_ACC = 240;               // accumulator columns of a tile, of 256 (the drain reads up to 16 columns further),
 constexpr int FW_ACC_ONE = 496;           // or of 512 where a tile takes both buffers
 static_assert(FW_ACC + 16 <= 256 && FW_ACC_ONE + 16 <= 512, "columns that a drain reads");
+static_assert(2 * FW_MAX_COLS + 2 * FW_MAX_ROWS <= 512 && FW_MAX_ROWS % 16 == 0, "gate / up with the sums put by");
 constexpr float FW_LAZY = 64.f;           // log2 of how far a score may exceed its row's reference value
 constexpr float FW_UNSEEN = -1e30f;       // the reference value of a row that has seen no key
 

@@ -8,8 +8,12 @@ namespace mtad {
 constexpr int FW_RING = 192 * 1024;       // the copy ring: four slots, or three where the operand rows are many; a slot
                                           // holds one step of a projection, or 128 keys of K or V
 constexpr int FW_KEYS = 128;              // keys of an attention tile
-constexpr int FW_MAX_ROWS = 72;           // rows of a call
-constexpr int FW_MAX_COLS = 144;          // operand rows (terms x rows) of a call
+// Rows of a call.  Gate / up ends them: two boxes of 2 x 80 accumulator columns and the rows' sums put by between the parts
+// of a tile's k-range (2 x 80 more) are 480 of the 512 columns of tensor memory.  Speed does not: eight layers of the 7B shape
+// on 1024 keys, chain of launches -> one launch, 65 / 73 / 77 rows 1500 -> 1197, 1610 -> 1272, 1626 -> 1285 us, and in a trial
+// without the sums put by (less exact than the chain) 101 rows 1997 -> 1444; 13B, 77 rows 1978 -> 1746.
+constexpr int FW_MAX_ROWS = 80;
+constexpr int FW_MAX_COLS = 160;          // operand rows (terms x rows) of a call
 constexpr int FW_QROWS = 16;              // query rows of one KV head and sequence that an attention item takes at most,
 constexpr int FW_QROWS_WIDE = 40;         // or in the wide variant: more are cut into blocks of equal size
 
@@ -21,9 +25,9 @@ constexpr int FW_QROWS_WIDE = 40;         // or in the wide variant: more are cu
 // bytes and more pass at 70 GB/s per SM where rows of 128 bytes pass at 43.
 // Three larger slots from 80 operand rows on, where a slot of a quarter of the ring holds one k-block only: 13B, 56 rows 8.64 ms
 // with three, 8.75 with four; 7B, 33 rows 3.50 and 3.62.  At up to 64 four are as good (7B, 18 rows 3.98 and 3.96).
-constexpr int FW_CLASSES = 6;
+constexpr int FW_CLASSES = 7;
 struct FwClass { int cols, slots; };      // operand rows up to, ring slots
-constexpr FwClass FW_CLASS[FW_CLASSES] = {{16, 4}, {32, 4}, {64, 4}, {80, 3}, {112, 3}, {FW_MAX_COLS, 3}};
+constexpr FwClass FW_CLASS[FW_CLASSES] = {{16, 4}, {32, 4}, {64, 4}, {80, 3}, {112, 3}, {144, 3}, {FW_MAX_COLS, 3}};
 struct FwPhase {
     int h, hr, nbox, n_tiles, u;          // u: tiles per head (QKV)
     int c;                                // blocks that share a tile's k-range (their partial sums meet in global memory): O, down,

@@ -44,6 +44,9 @@ def models():
     ("gqa128", 5, None, [255]),
     ("gqa128", 65, (8, 8, 2), [130]),
     ("gqa128", 73, (9, 8, 4), [128]),
+    ("hd64", 10, None, [9, 64, 120, 121, 127, 128, 255, 300]),   # the most rows
+    ("gqa128", 77, (4, 19, 1), [200]),
+    ("gqa128", 81, (5, 16, 4), [128]),                           # one more: the attention alone
     ("odd", 6, None, [64, 65]),
     ("odd", 33, (4, 8, 2), [64]),
 ])

@@ -40,7 +40,7 @@ def test_chain_of_launches(shape, rows, tree, lengths, path):
         n = Bn.mtad_kernel_launches()
         _compare(gm, rows, tree, lengths, it)
         launches.append(Bn.mtad_kernel_launches() - n)
-    assert launches[0] > launches[1] or rows * len(lengths) > 72, launches
+    assert launches[0] > launches[1] or rows * len(lengths) > 80, launches
 
 
 @pytest.mark.parametrize("shape,rows,tree,lengths,chain", [
@@ -53,7 +53,7 @@ def test_chain_of_launches(shape, rows, tree, lengths, path):
     (MHA64, 145, (9, 16, 4), [90], False), (GQA128, 81, (5, 16, 4), [90], False),
 ])
 def test_the_faster_way_is_taken(shape, rows, tree, lengths, chain):
-    """Few long calls as one launch (beyond 72 rows: their attention), calls of many sequences with heads of 64 as a chain."""
+    """Few long calls as one launch (beyond 80 rows: their attention), calls of many sequences with heads of 64 as a chain."""
     gm = GpuModel(shape, max_batch=len(lengths), max_nodes=max(rows - 1, 1), capacity=480)
     launches = []
     for it, path in enumerate((1, 0)):

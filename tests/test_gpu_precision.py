@@ -93,7 +93,7 @@ def _layer_errors(sh, batch, rows, length, tree):
 # matrix over eight blocks; 3.2e-6 with a quarter, which is what two bf16 terms may add to (2.2e-6).
 @pytest.mark.parametrize("batch,rows,tree", [(1, 1, None), (1, 5, None), (1, 9, None), (3, 6, None), (1, 32, None),
                                              (1, 33, (4, 8, 4)), (1, 41, (4, 10, 2)), (8, 7, None), (1, 57, (4, 14, 2)),
-                                             (1, 65, (4, 16, 4)), (1, 71, (7, 10, 2))])
+                                             (1, 65, (4, 16, 4)), (1, 71, (7, 10, 2)), (8, 10, None)])
 def test_accumulators_take_a_part_of_the_k_range(batch, rows, tree):
     e = _layer_errors(S.ModelShape(1, 4096, 32, 32, 128, 11008, 1000), batch, rows, 300, tree)
     many = batch * rows > 32
@@ -108,7 +108,7 @@ def test_accumulators_take_a_part_of_the_k_range(batch, rows, tree):
     (12, 12, 64, 1, 1, None), (12, 12, 64, 1, 5, None), (6, 6, 128, 1, 8, None), (12, 12, 64, 1, 12, None),
     (6, 6, 128, 1, 16, None), (12, 3, 64, 2, 4, None), (12, 12, 64, 1, 17, None), (12, 3, 64, 3, 7, None),
     (12, 12, 64, 8, 7, None), (12, 12, 64, 1, 33, (4, 8, 4)), (6, 6, 128, 1, 41, (4, 10, 2)), (12, 12, 64, 1, 65, (8, 8, 2)),
-    (6, 6, 128, 1, 73, (9, 8, 4))])
+    (6, 6, 128, 1, 73, (9, 8, 4)), (12, 12, 64, 8, 10, None), (6, 6, 128, 1, 97, (8, 12, 4))])
 def test_probabilities_are_exact(heads, kv_heads, head_dim, batch, rows, tree):
     e = _layer_errors(S.ModelShape(1, 768, heads, kv_heads, head_dim, 1024, 1000), batch, rows, 400, tree)
     assert e["attention"] <= (3.3e-6 if batch * rows > 32 else 2.1e-6), e
