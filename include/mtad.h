@@ -176,7 +176,9 @@ int mtad_set_draft_warp(mtad_ctx* ctx, int top_k, float top_p);
  * The chain of Algorithm 1 is best_path with logq_ref.  kv_commit after a verification of this tree (or of that
  * chain) also rolls the auxiliary cache forward: accepted nodes that were beams of a layer before the last keep
  * their keys and values, an accepted node that the auxiliary model never ran (last layer, or a candidate that was
- * not kept) is replayed by the next draft together with the extra token. */
+ * not kept) is replayed by the next draft together with the extra token.
+ * A bounded wait that gave up in a draft (its nodes are then meaningless) is reported by the verification of the same
+ * sequences that follows: MTAD_ST_TIMEOUT, nothing accepted, and kv_commit leaves them as they were before the draft. */
 int mtad_draft(mtad_ctx* ctx, int B, const int32_t* seqs, int gamma, int beam_width, int keep_all_candidates,
                const float* uniforms, int32_t* n_nodes, int32_t* tok, int32_t* parent, int32_t* depth,
                float* node_logq, float* logq_ref, int32_t* best_path, void* stream);

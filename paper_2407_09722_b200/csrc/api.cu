@@ -282,6 +282,7 @@ size_t carve(mtad_ctx* c, const mtad_model_desc* t, const mtad_model_desc* a, in
     ds.tree2slot = k.take<int32_t>((size_t)max_batch * MTAD_DRAFT_NODES, "ds_tree2slot");
     ds.nb = k.take<int32_t>((size_t)max_batch * MTAD_MAX_DEPTH, "ds_nb");
     ds.n_tree = k.take<int32_t>((size_t)max_batch, "ds_n_tree");
+    ds.status = k.take<uint32_t>((size_t)max_batch, "ds_status");
     if (c) {
         c->ds = ds;
         c->st = st; c->rm = rm; c->sc = sc;
@@ -774,6 +775,8 @@ int verify_common(mtad_ctx* ctx, int B, const int32_t* seqs, const int32_t* n_no
     PrepareArgs pa{};
     for (int i = 0; i < B; ++i) pa.seqs.v[i] = seqs[i];
     pa.B = B; pa.R = R; pa.max_depth = D; pa.n_nodes = n_nodes; pa.tok = tok; pa.parent = parent;
+    if (ctx->draft_active && ctx->draft_B == B && memcmp(seqs, ctx->draft_seqs, sizeof(int32_t) * B) == 0)
+        pa.draft_status = ctx->ds.status;
     const bool tc = ctx->use_tc && ctx->tmaps.ok && B * R <= TC_MAX_ROWS;
     if (tc) {
         pa.gain0 = ctx->target.w(0, 0); pa.x = ctx->sc.xd; pa.terms = tc_terms(B * R);
@@ -1115,7 +1118,7 @@ int mtad_draft(mtad_ctx* ctx, int B, const int32_t* seqs, int gamma, int beam_wi
         // keys of the auxiliary cache: committed ones, the pending rows and every node drafted so far
         const long long keys_ub = ub + 1 + (long long)step * beam_width;
         int rc;
-        if (tc && B * R <= TC_MAX_ROWS) rc = forward_rows_tc(ctx, m, ctx->amaps, B, R, keys_ub, nullptr, nullptr, true, s);
+        if (tc && B * R <= TC_MAX_ROWS) rc = forward_rows_tc(ctx, m, ctx->amaps, B, R, keys_ub, nullptr, ctx->ds.status, true, s);
         else rc = forward_rows(ctx, m, B, R, keys_ub, s);
         if (rc != MTAD_OK) return rc;
         if (dwarp) {

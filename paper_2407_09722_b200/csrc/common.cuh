@@ -71,6 +71,7 @@ struct DraftState {
     // and the nodes written to the caller's tree so far.
     int32_t* nb;           // [max_batch][MTAD_MAX_DEPTH]
     int32_t* n_tree;       // [max_batch]
+    uint32_t* status;      // [max_batch] by place in the call: MTAD_ST_TIMEOUT of the draft's forwards, for the verification
 };
 
 struct DraftOut {          // caller's device arrays of mtad_draft
@@ -314,6 +315,7 @@ struct PrepareArgs {
     const int32_t* n_nodes;    // device [B] or nullptr (all sequences have R-1 nodes)
     const int32_t* tok;        // device [B, R-1]
     const int32_t* parent;     // device [B, R-1] or nullptr (chain)
+    const uint32_t* draft_status;   // of the draft that these sequences come from, or nullptr
     // tensor-core path (null otherwise): first layer's norm gains, operand rows and row statistics to emit
     const __nv_bfloat16* gain0;
     __nv_bfloat16* x;

@@ -110,6 +110,7 @@ __global__ void prepare_kernel(const __nv_bfloat16* __restrict__ embed, int d, i
             mask[0] |= 1u;
             if (tok < 0 || tok >= vocab) { st |= MTAD_ST_BAD_TOKEN; tok = 0; }
         }
+        if (r == 0 && a.draft_status) st |= a.draft_status[bi];
         if (st) atomicOr(&status[bi], st);
         rm.tok[t] = tok;
         rm.depth[t] = depth;

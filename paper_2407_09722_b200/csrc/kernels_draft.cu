@@ -65,7 +65,7 @@ __global__ void draft_prepare_kernel(const __nv_bfloat16* __restrict__ embed, in
     if (threadIdx.x == 0) {
         const int L = step == 0 ? s.aux_len[seq] : ds.base_len[seq];
         const int P = step == 0 ? s.aux_npend[seq] : ds.npend[seq];
-        if (step == 0 && r == 0) { ds.base_len[seq] = L; ds.npend[seq] = P; }
+        if (step == 0 && r == 0) { ds.base_len[seq] = L; ds.npend[seq] = P; ds.status[bi] = 0; }
         uint32_t mask[MTAD_MASK_WORDS];
 #pragma unroll
         for (int i = 0; i < MTAD_MASK_WORDS; ++i) mask[i] = 0;

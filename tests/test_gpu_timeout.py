@@ -47,3 +47,36 @@ def test_wait_runs_out_then_context_recovers(gamma):
         cases = [SeqCase(s, L, 3 + s, S.chain_tree(gamma, V, stream=80 + 8 * it + s)) for s in seqs]
         compare(gm, cases, math.log(0.3), S.bonus_uniforms(6, it, 3, V, "cuda"), chain=True, stats=stats)
     assert stats.ok() and stats.near_ties <= 2, stats
+
+
+def test_wait_runs_out_in_a_draft():
+    """The verification that follows reports it for every sequence of the draft, nothing is committed, and the next draft's
+    verification is fine again."""
+    W = S.WORKLOADS["tiny"]
+    gamma, beam, L, V = 3, 2, 20, W.target.vocab
+    gm = GpuModel(W.target, max_batch=2, max_nodes=16, capacity=128, aux=W.aux, aux_capacity=128)
+    seqs, n = [0, 1], gamma * beam
+    i32, f32 = dict(dtype=torch.int32, device="cuda"), dict(dtype=torch.float32, device="cuda")
+    for s in seqs:
+        gm.inject(s, L)
+        gm.inject_aux(s, L)
+    u, u_draft = S.bonus_uniforms(5, 0, 2, V, "cuda"), S.bonus_uniforms(6, 0, 2 * gamma * beam, V, "cuda").view(2, gamma, beam, V)
+    tok, parent, depth = (torch.zeros(2, n, **i32) for _ in range(3))
+    logq, ref, best = torch.zeros(2, n, **f32), torch.zeros(2, gamma, **f32), torch.zeros(2, gamma, **i32)
+    res = M.ResultBuffers(2, n, gamma)
+    for path in (0, 1):
+        gm.ctx.mtad_debug_set_path(path)
+        for fails in (True, False):
+            for s in seqs:
+                gm.ctx.mtad_seq_set(s, L, 3 + s)
+            gm.ctx.mtad_debug_set_wait(*((2000, True) if fails else (0, False)))
+            gm.ctx.mtad_draft(seqs, gamma, beam, u_draft, tok, parent, depth, logq, ref, best)
+            gm.ctx.mtad_debug_set_wait(0, False)
+            gm.ctx.mtad_verify_tree(seqs, None, n, gamma, tok, parent, ref, math.log(0.1), u, res)
+            gm.ctx.kv_commit(seqs, res)
+            h = res.host()
+            if fails:
+                assert all(x & Bn.MTAD_ST_TIMEOUT for x in h["status"].tolist()) and h["n_out"].tolist() == [0, 0]
+                assert [gm.ctx.mtad_seq_get(s) for s in seqs] == [(L, 3), (L, 4)]
+            else:
+                assert h["status"].tolist() == [0, 0] and min(h["n_out"].tolist()) >= 1
