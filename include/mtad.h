@@ -303,8 +303,10 @@ int mtad_debug_check_canaries(mtad_ctx* ctx, void* stream, const char** damaged)
  * element count and element size.  For tests that inspect intermediate results. */
 int mtad_debug_region(const mtad_ctx* ctx, const char* name, size_t* offset, size_t* count, size_t* elem_bytes);
 
-/* Test hook for the time-out path: wait_limit = iterations a bounded wait inside the GEMM kernels may poll (0: the
- * default); no_operands != 0 makes the GEMM kernels leave out their operand-row copies, so the waits on them run out
+/* Test hook for the time-out path: wait_limit = polls that a bounded wait inside the GEMM kernels and the one-launch
+ * forward may take (0: the default, 2^20; a poll of a barrier may suspend the thread for a system-dependent time, so
+ * this bounds a number and not a time); no_operands = 1 makes them leave out their operand-row copies, 2 makes the
+ * one-launch forward's attention leave out its key and value tiles, so that the waits on them run out
  * and every sequence of the call reports MTAD_ST_TIMEOUT.  The kernels return normally; a later call with the hook
  * switched off is unaffected. */
 int mtad_debug_set_wait(mtad_ctx* ctx, unsigned int wait_limit, int no_operands);

@@ -249,9 +249,8 @@ class Context:
     def mtad_seq_hint(self, seq: int, kv_len: int):
         self._check(self._lib.mtad_seq_hint(self.handle, seq, kv_len), "mtad_seq_hint")
 
-    def mtad_debug_set_wait(self, wait_limit: int, no_operands: bool):
-        self._check(self._lib.mtad_debug_set_wait(self.handle, wait_limit, 1 if no_operands else 0),
-                    "mtad_debug_set_wait")
+    def mtad_debug_set_wait(self, wait_limit: int, no_operands: int):
+        self._check(self._lib.mtad_debug_set_wait(self.handle, wait_limit, int(no_operands)), "mtad_debug_set_wait")
 
     def mtad_debug_set_path(self, path: int):
         self._check(self._lib.mtad_debug_set_path(self.handle, path), "mtad_debug_set_path")

@@ -79,7 +79,7 @@ struct mtad_ctx {
     int32_t last_seqs[MTAD_MAX_BATCH];
     int last_cuda = 0;
     unsigned int wait_limit = 0;        // debug: iteration limit of the GEMM kernels' bounded waits (0: default)
-    int debug_no_operands = 0;          // debug: the GEMM kernels' operand-row copies are left out (waits run out)
+    int debug_no_operands = 0;          // debug: copies that are left out (waits run out): 1 operand rows, 2 K and V tiles
     int warp_k = 0;                     // 0: unwarped target rows
     float warp_p = 1.f;
     int dwarp_k = 0;                    // 0: the draft samples from the unwarped auxiliary rows
@@ -697,7 +697,7 @@ int forward_rows_tc(mtad_ctx* ctx, const ModelView& m, const WeightMaps& wm, int
         GemmDesc& gd = fp.g[i];
         TcGemmParams& p = gd.p;
         p.status = status; p.uniforms = uniforms;
-        p.wait_limit = ctx->wait_limit; p.debug_no_operands = ctx->debug_no_operands;
+        p.wait_limit = ctx->wait_limit; p.debug_no_operands = ctx->debug_no_operands == 1;
 #ifdef MTAD_TRACE
         p.trace = trace_slot(gd.cluster, p.mode,
                              gd.cluster ? p.n_tiles * p.csize : (p.total_units + p.units_per_cta - 1) / p.units_per_cta,
@@ -713,7 +713,7 @@ int forward_rows_tc(mtad_ctx* ctx, const ModelView& m, const WeightMaps& wm, int
             const int l = layer++;
             bool done = false;
             if (fp.fw_attn && ctx->resident && fw_attn_pays(d, B, R, total)) {
-                fp.fw.status = status; fp.fw.wait_limit = ctx->wait_limit;
+                fp.fw.status = status; fp.fw.wait_limit = ctx->wait_limit; fp.fw.debug_no_operands = ctx->debug_no_operands;
                 fp.fw.pieces = (int)((total + FW_KEYS - 1) / FW_KEYS);
                 const int rc = timed(ctx, MTAD_K_ATTN, 0, 1, s, [&] { return launch_forward_attention(fp.fw, l, s, ctx->refuse_resident); });
                 if (rc != MTAD_OK && !too_large(rc)) return rc;
@@ -1050,9 +1050,9 @@ int mtad_debug_region(const mtad_ctx* ctx, const char* name, size_t* offset, siz
 }
 
 int mtad_debug_set_wait(mtad_ctx* ctx, unsigned int wait_limit, int no_operands) {
-    if (!ctx) return MTAD_E_INVALID;
+    if (!ctx || no_operands < 0 || no_operands > 2) return MTAD_E_INVALID;
     ctx->wait_limit = wait_limit;
-    ctx->debug_no_operands = no_operands ? 1 : 0;
+    ctx->debug_no_operands = no_operands;
     return MTAD_OK;
 }
 

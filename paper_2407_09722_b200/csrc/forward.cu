@@ -32,7 +32,7 @@
 //
 // Warps: 0 weight and K / V producer (TMA), 1 operand-row producer (TMA; waits for the phase before), 2 and 3 MMA issuers
 // (3 owns the tensor memory), 4..11 epilogue and softmax.
-// Every wait is bounded; a block that gives up raises MTAD_ST_TIMEOUT for every sequence of the call and leaves, and the
+// Every wait is bounded by a number of polls (WAIT_LIMIT); a block that gives up raises MTAD_ST_TIMEOUT for every sequence of the call and leaves, and the
 // others run into their own limits at the grid barrier.
 #include <math_constants.h>
 
@@ -1042,6 +1042,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                             if (!ok) break;
                             const uint32_t bar = full_bar(pos), dst = slot_ptr(pos);
                             mbar_expect_tx(bar, KV_BYTES);
+                            if (a.debug_no_operands == 2) continue;
 #pragma unroll
                             for (int c = 0; c < NCH; ++c)
 #pragma unroll
@@ -1129,7 +1130,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         ok = mbar_wait(empty_bar(pos), ring_par(pos) ^ 1u, abort_flag);
                         if (!ok) break;
                         const uint32_t bar = full_bar(pos), base = slot_ptr(pos) + f.b_off;
-                        if (!a.debug_no_operands)
+                        if (a.debug_no_operands != 1)
                             tma_load_3d(base, m, bar, f.flat ? step * TC_TILE_K : 0, 0, f.flat ? 0 : step * f.kb, HINT_KEEP);
                     }
                 }

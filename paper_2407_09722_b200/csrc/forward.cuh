@@ -73,7 +73,7 @@ struct FwArgs {
     float *logits, *node_z;
     uint32_t* status;
     unsigned int wait_limit;
-    int debug_no_operands;
+    int debug_no_operands;                // test hook: 1 no operand rows, 2 no K and V tiles are copied, so the waits on them run out
 };
 
 // Host side.  fw_geometry fills the geometry of class cls; fw_plan the rest for a call of B x R rows and returns false

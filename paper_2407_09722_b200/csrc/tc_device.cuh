@@ -9,9 +9,10 @@
 namespace mtad {
 namespace tcdev {
 
-// A wait gives up after this many polls (some tenths of a second).  A poll is an mbarrier.try_wait, which may park the
-// thread for a while: a parked warp takes no issue slots from the warps that work, and no hand-over waits for the rest of
-// a sleep.
+// A wait gives up after this many polls.  This bounds a number and not a time: a poll of a barrier is an mbarrier.try_wait,
+// which may park the thread for a while that the hardware chooses, and one of a counter in global memory is a load from L2
+// (half a microsecond and more).  A parked warp takes no issue slots from the warps that work, and no hand-over waits for the
+// rest of a sleep.
 constexpr uint32_t WAIT_LIMIT = 1u << 20;
 constexpr int MAX_STAGES = 12;
 constexpr int EPI_THREADS = 128;

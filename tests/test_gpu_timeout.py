@@ -1,7 +1,8 @@
-"""The time-out path of the GEMM kernels: a bounded wait that runs out must end in MTAD_ST_TIMEOUT for every
-sequence of the call, the kernels must return normally, kv_commit must leave those sequences alone, and the next call
-on the same context must match the oracle again.  The wait is made to run out on the host's request (the operand-row
-copies are left out, so the barrier they would complete is never completed); nothing faults and nothing hangs."""
+"""The time-out path of the one-launch forward, the GEMM kernels and the wide attention: a bounded wait that runs out must
+end in MTAD_ST_TIMEOUT for every sequence of the call, the kernels must return normally, kv_commit must leave those
+sequences alone, and the next call on the same context must match the oracle again.  The wait is made to run out on the
+host's request (copies are left out, so the barrier they would complete is never completed); nothing faults and nothing
+hangs."""
 import math
 
 import pytest
@@ -14,12 +15,26 @@ from tests.parity import GpuModel, SeqCase, ParityStats, compare
 
 pytestmark = pytest.mark.gpu
 TINY = S.WORKLOADS["tiny"].target
+GQA128 = S.ModelShape(2, 512, 8, 2, 128, 1024, 640)
 
 
-@pytest.mark.parametrize("gamma", [4, 11])      # 5 rows: the few-row cluster kernel and (gate / up) the stream-K kernel; 12 rows x 3 sequences = 36: the many-row cluster kernel
+@pytest.mark.parametrize("gamma", [4, 11])      # 15 and 36 rows: three and two bf16 terms
 def test_wait_runs_out_then_context_recovers(gamma):
-    gm = GpuModel(TINY, max_batch=3, max_nodes=16, capacity=128)
-    V = TINY.vocab
+    _runs_out_then_recovers(TINY, gamma, path=1, left_out=1)
+
+
+# as a chain of launches: 15 rows take the few-row cluster kernel and (gate / up) the stream-K kernel, 36 the many-row cluster
+# kernel; in one launch without keys and values; 84 rows of four query heads per KV head: the wide attention of its own
+@pytest.mark.parametrize("shape,gamma,path,left_out", [(TINY, 4, 0, 1), (TINY, 11, 0, 1), (TINY, 4, 1, 2), (TINY, 27, 0, 1),
+                                                       (GQA128, 27, 1, 2)])
+def test_every_kernel_that_waits(shape, gamma, path, left_out):
+    _runs_out_then_recovers(shape, gamma, path, left_out)
+
+
+def _runs_out_then_recovers(shape, gamma, path, left_out):
+    gm = GpuModel(shape, max_batch=3, max_nodes=32, capacity=128)
+    gm.ctx.mtad_debug_set_path(path)
+    V = shape.vocab
     seqs, L = [0, 1, 2], 20
     for s in seqs:
         gm.inject(s, L)
@@ -29,7 +44,7 @@ def test_wait_runs_out_then_context_recovers(gamma):
     lq = torch.tensor([t.logq for t in trees], dtype=torch.float32, device="cuda")
     u = S.bonus_uniforms(5, 0, 3, V, "cuda")
     res = M.ResultBuffers(3, gamma, gamma)
-    gm.ctx.mtad_debug_set_wait(2000, True)
+    gm.ctx.mtad_debug_set_wait(2000, left_out)
     gm.ctx.mtad_verify_chain(seqs, gamma, tok, lq, math.log(0.1), u, res)
     gm.ctx.kv_commit(seqs, res)
     torch.cuda.synchronize()                      # the kernels came back: no fault, no hang
