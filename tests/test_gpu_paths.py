@@ -75,3 +75,14 @@ def test_keys_from_which_the_wide_attention_is_taken(shape, wide):
         _compare(gm, 41, (4, 10, 2), [L, 50], L)
         used.append(Bn.mtad_kernel_launches() - n)
     assert used[0] - used[1] == (shape.layers if wide else 0), used        # (two launches a layer, one)
+
+
+@pytest.mark.parametrize("shape,rows", [(MHA64, 5), (S.ModelShape(2, 256, 2, 2, 128, 512, 500), 6), (GQA128, 5)])
+def test_stale_partials_of_ragged_batches(shape, rows):
+    """Beyond 80 rows, few of them per sequence: the attention of mma.sync warps, whose splits past a short sequence's keys are
+    empty.  What earlier calls left in their partials must not matter, a NaN neither."""
+    lengths = [0, 250, 1, 64, 63, 190, 7, 128, 33, 3, 255, 70, 100, 0, 129, 20, 200]
+    gm = GpuModel(shape, max_batch=len(lengths), max_nodes=rows, capacity=320)
+    for it in range(2):
+        gm.ctx.region("attn_part", torch.float32).fill_(float("nan"))
+        _compare(gm, rows, None, lengths, it)
