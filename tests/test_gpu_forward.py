@@ -1,6 +1,6 @@
 """The one-launch decoder forward at the edges of its variants: row counts where the operand class, the epilogue or the
 number of bf16 terms changes, key counts around its 128-key tiles, query rows per KV head around the sizes of an
-attention item, split and unsplit projections, and one call beyond its rows whose attention alone it forms.  Compared
+attention item, split and unsplit projections, its most rows, and one call beyond them whose attention alone it forms.  Compared
 with the CPU oracle; the tolerances are derived in parity.py."""
 import pytest
 
@@ -69,4 +69,6 @@ def test_forward_edges(models, shape, rows, tree, lengths):
         # A row with next to no committed keys attends to this call's own: where their values rounded the other way (a
         # bf16 step, at most 2^-8 of the value, in a share `flips` of the elements), its output moves by 2^-9 sqrt(flips)
         # of the largest value in the mean square, and by four times that at most.  cache_ok leaves this out.
-        assert flips <= 0.1 and stats.cache_max_excess <= 2.0 ** -7 * flips ** 0.5 * stats.cache_scale
+        # The share itself is bounded from above by 0.29 (the first layer's as in cache_ok, the second's with the output moved
+        # as said); measured 5e-3..6e-3, held to five times that.
+        assert flips <= 0.03 and stats.cache_max_excess <= 2.0 ** -7 * flips ** 0.5 * stats.cache_scale
