@@ -2,11 +2,13 @@
 attention alone is such a launch, run as a chain of launches with the attention of mma.sync warps, whether that is known
 when the context is made or the driver refuses the launch later.  Compared with the CPU oracle at the edges of that
 attention's variants (query rows per KV head: a packed tile, one, two, up to four, five and more tiles of 16)."""
-import numpy as np
+import threading
+
 import pytest
 import torch
 
 import mtad_synth as S
+import paper_2407_09722_b200 as M
 from paper_2407_09722_b200 import binding as Bn
 from tests.parity import GpuModel, SeqCase, ParityStats, compare
 
@@ -86,3 +88,61 @@ def test_stale_partials_of_ragged_batches(shape, rows):
     for it in range(2):
         gm.ctx.region("attn_part", torch.float32).fill_(float("nan"))
         _compare(gm, rows, None, lengths, it)
+
+
+def _chain_call(gm, L, gamma, seed):
+    t, V = S.chain_tree(gamma, gm.shape.vocab, stream=seed), gm.shape.vocab
+    gm.inject(0, L)
+    gm.ctx.mtad_seq_set(0, L, 3)
+    tok = torch.tensor([t.tok], dtype=torch.int32, device="cuda")
+    lq = torch.tensor([t.logq], dtype=torch.float32, device="cuda")
+    res, u = M.ResultBuffers(1, gamma, gamma), S.bonus_uniforms(9, seed, 1, V, "cuda")
+    return res, lambda stream=None: gm.ctx.mtad_verify_chain([0], gamma, tok, lq, Bn.log_tau(0.3), u, res, stream=stream)
+
+
+def _same(a, b):
+    return all(torch.equal(a[k], b[k]) for k in ("eta", "winner", "n_out", "out_tok", "out_lp", "node_lp", "row_lse", "status"))
+
+
+@pytest.mark.parametrize("gamma,path", [(4, 1), (4, 0), (30, 1)])
+def test_capture(gamma, path):
+    """A verification recorded in a CUDA graph and replayed gives what the call gives."""
+    gm = GpuModel(MHA64, max_batch=1, max_nodes=32, capacity=320)
+    gm.ctx.mtad_debug_set_path(path)
+    res, call = _chain_call(gm, 150, gamma, 3)
+    call()
+    torch.cuda.synchronize()
+    want = res.host()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call()
+    for _ in range(2):
+        res.buf.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert _same(res.host(), want)
+    del graph
+
+
+def test_two_contexts_on_two_streams():
+    """Calls of two contexts, each on its own stream and thread: what one of them waits for never depends on the other."""
+    made = []
+    for k, sh in enumerate((MHA64, GQA128)):
+        gm = GpuModel(sh, max_batch=1, max_nodes=32, capacity=320)
+        res, call = _chain_call(gm, 140 + 20 * k, 8 + 16 * k, 5 + k)
+        call()
+        torch.cuda.synchronize()
+        made.append((gm, res, call, res.host(), torch.cuda.Stream()))
+
+    def work(k):
+        for _ in range(40):
+            made[k][2](made[k][4])
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    for gm, res, call, want, _ in made:
+        assert _same(res.host(), want)
