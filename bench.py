@@ -28,9 +28,9 @@ import mtad_synth as S  # noqa: E402
 
 TAU = 0.1
 SEED = 0
-# (DRAM read + write) / weight bytes of the forward launch, ncu on the 4-layer workloads (profiles/forward_7b_4l.md); the
-# others of the shape with their own share of K / V bytes, which the launch reads too; no figure for other shapes
-NCU_TRAFFIC_RATIO = {"7b_chain": 1.086, "7b_chain_4l": 1.076, "7b_chain_l512": 1.025, "7b_tree": 1.108, "7b_tree_4l": 1.098}
+# (DRAM read + write) / (weights + committed K / V) of the forward launch, ncu on the 4-layer workloads (profiles/forward_7b_4l.md):
+# chain and tree of the 7B shape; no figure for other shapes
+NCU_TRAFFIC_RATIO = {"7b_chain": 1.005, "7b_chain_4l": 1.005, "7b_chain_l512": 1.005, "7b_tree": 1.025, "7b_tree_4l": 1.025}
 
 
 def measured_peaks():
@@ -531,6 +531,7 @@ def run_ours(args, w: S.Workload, rank: int, world: int, local_rank: int):
     prof_total = sum(v["ms"] for v in prof.values())
     alg_per_launch = gemm["bytes"] / max(gemm["launches"], 1)
     ratio = NCU_TRAFFIC_RATIO.get(w.name)
+    kv_per_launch = w.target.kv_bytes_per_token() * float(sum((a + c) / 2 for a, c in zip(lens, final_lens)))
     one_launch = gemm["launches"] == prof_steps
     roofline = {"bound": "hbm",
                 "kernel": "forward_kernel (the decoder forward as one cooperative launch; bytes: all weight matrices + LM "
@@ -542,9 +543,9 @@ def run_ours(args, w: S.Workload, rank: int, world: int, local_rank: int):
                           "CUDA events on the launching stream around every run of consecutive GEMM launches "
                           "(O, gate/up, down, next QKV or LM head), summed and divided by the launches",
                 "algorithmic_bytes_per_launch": alg_per_launch,
-                # DRAM read + write bytes per launch: the ratio to the algorithmic bytes was taken with ncu on the
-                # 4-layer workload of the same shape
-                "traffic": alg_per_launch * ratio if ratio else None,
+                # DRAM read + write bytes per launch: the ratio to weights and K / V, which the launch reads as well, was taken
+                # with ncu on the 4-layer workload of the same shape
+                "traffic": (alg_per_launch + kv_per_launch) * ratio if ratio and one_launch else None,
                 "launches_per_step": gemm["launches"] / prof_steps,
                 "avg_launch_us": 1e3 * gemm["ms"] / max(gemm["launches"], 1),
                 "share_of_step": gemm["ms"] / prof_total if prof_total else None,

@@ -9,10 +9,11 @@
 // stays busy across the barrier for as long as the ring is deep.  Two more things keep the boundary short: every block
 // owns whole output features (the features are cut into one tile per SM, not into 128-row tiles), so no partial sum leaves
 // an SM while rows are few; and only the call's terms x rows operand rows are multiplied (16 columns for five rows).
-// Measured (chain of launches -> one launch, a whole verification step): 7B, 5 rows 3.55 -> 3.02 ms (weights and K / V in
-// 2.2 ms at copy speed), 33 rows 4.40 -> 3.50, 65 rows 5.94 -> 4.65; 13B, 8 x 7 rows 9.8 -> 8.6; two-layer auxiliary
-// model of width 768, four draft steps 523 -> 434 us.  A phase costs its bytes plus about 3 us (barrier 1.1, first operand
-// rows 0.8, last MMA to last store 1.2 and up).
+// Measured (chain of launches -> one launch, a whole verification step): 7B, 5 rows 3.55 -> 3.07 ms (weights and K / V in
+// 2.2 ms at copy speed), 33 rows 4.37 -> 3.56, 65 rows 5.90 -> 4.81; 13B, 8 x 7 rows 9.41 -> 8.50; two-layer auxiliary
+// model of width 768, four draft steps 520 -> 439 us.  A phase of a large model costs its bytes plus about 3 us (barrier 1.1,
+// first operand rows 0.8, last MMA to last store 1.2 and up); the phases of the auxiliary model, which move next to nothing,
+// take about 8, and the attention of a chain 10 more than its bytes.
 //
 // Contraction.  Weights are the 128-row MMA operand A, the operand rows (two or three bf16 terms per activation, see
 // store_terms) operand B.  Where a block owns at most 64 features, the MMA takes S k-blocks at once: their weights lie
@@ -27,13 +28,14 @@
 // Pieces of a (sequence, KV head) held by several blocks meet in global memory; the block that arrives last merges them.
 // An item takes up to 8 or 16 query rows of a KV head, or 40 in the wide variant (an instantiation each: the softmax's time
 // goes with the rows, padding included; beyond 40 a thread's 20 rows would leave its registers), and more are cut into
-// blocks of equal size.  Per tile 0.75 us at 8 rows, 1.6 at 40, against 1.3 us that K and V take at copy speed.  7B, 65 rows
-// on 2048 keys: 39 -> 32 us a layer against `mma.sync` warps; 64 heads on 8 KV heads, 129 rows, 1024 keys: 167 -> 77.
+// blocks of equal size.  Per tile 0.75 us at 8 rows, 1.6 at 40, against 1.3 us that K and V take at copy speed (before the
+// third term of P).  7B, 65 rows on 2048 keys: 39 -> 35 us a layer against `mma.sync` warps; 64 heads on 8 KV heads, 129 rows,
+// 1024 keys: a layer of the whole step 960 -> 846.
 //
 // Warps: 0 weight and K / V producer (TMA), 1 operand-row producer (TMA; waits for the phase before), 2 and 3 MMA issuers
 // (3 owns the tensor memory), 4..11 epilogue and softmax.
-// Every wait is bounded by a number of polls (WAIT_LIMIT); a block that gives up raises MTAD_ST_TIMEOUT for every sequence of the call and leaves, and the
-// others run into their own limits at the grid barrier.
+// Every wait is bounded by a number of polls (WAIT_LIMIT); a block that gives up raises MTAD_ST_TIMEOUT for every sequence of
+// the call and leaves, and the others run into their own limits at the grid barrier.
 #include <math_constants.h>
 
 #include <cstddef>
@@ -922,7 +924,8 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     constexpr int Q_BYTES = NQ2 * HD * 2;              // one query tile
     // Probabilities as three terms, exactly.  Two leave 2^-18 of each, and with one reference value for all keys of a tile even
     // the largest is not exact (mma.sync warps had a maximum for every 16 or 64 keys, whose probability is 1): 400 keys of a
-    // 64-wide head 2.85e-6 of the output off, 2.45 with mma.sync, 1.40 with three terms.  A tile takes 3 % longer.
+    // 64-wide head 2.85e-6 of the output off, 2.45 with mma.sync, 1.40 with three terms.  Costs about 3 us a layer of 65 rows at 7B width (the step
+    // 4830 -> 4930 us), below 1 % of a step of five.
     constexpr int NP3 = 3 * NQP;
     constexpr int P_N = (NP3 + 15) / 16 * 16;          // N of the output MMA: may read up to eight rows past the tile
     constexpr int P_BYTES = NP3 * FW_KEYS * 2;         // one probability tile
@@ -1650,7 +1653,8 @@ void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta, int cls) {
     // O and down: a tile's k-range over c blocks where that pays.  With many operand rows the SMs' intake bounds a narrow
     // tile (every block reads all operand rows of its k-blocks, about 100 GB/s an SM from L2); c blocks on a tile c times as
     // wide read them a c-th as often, and pay about 3.5 us to exchange their partial sums.  13B, 56 rows: O and down 24 and
-    // 48 us a layer unsplit, 17 and 32.5 over three blocks each.
+    // 48 us a layer unsplit, 17 and 32.5 over three blocks each.  The rates and what an exchange costs are fitted to the phases'
+    // times at 7B and 13B width and 33, 56 and 65 rows; they only rank the splits.
     for (int k : {FW_O, FW_DOWN}) {
         FwPhase& f = ph[k];
         double best = 1e30;
@@ -1680,7 +1684,8 @@ void fw_geometry(FwPhase ph[6], const mtad_model_desc& d, int n_cta, int cls) {
     q.k_blocks = up_div(q.K, TC_TILE_K);
     // The same split for QKV, two heads of 128 on a tile: it meets the operand rows half as often and spreads over all SMs
     // (7B, 32 heads: 96 tiles of one head leave a third of them idle), at about 4.5 us for the exchange.  7B, 65 rows: 35 ->
-    // 26 us a layer; at 33 rows both ways take 24.
+    // 26 us a layer; at 33 rows both ways take 24, and the unsplit one, which needs no exchange buffer, is taken unless the split
+    // is estimated 2 us faster (the 2.0).  The lower rate is that of the wider boxes: 256 weight rows beside the operand rows.
     if (d.head_dim == 128 && q.u == 1 && cls >= 2) {
         const double floor_us = 2.0 * heads * 128 * q.K / 6.5e6;
         double best = std::max((128.0 + cols) * 128.0 * q.k_blocks / 85e3, floor_us) - 2.0;

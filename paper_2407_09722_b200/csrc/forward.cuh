@@ -20,11 +20,13 @@ constexpr int FW_QROWS_WIDE = 40;         // or in the wide variant: more are cu
 // Tile geometry of one projection.  A step brings nbox boxes of hr weight rows x kb k-blocks (one copy each) and one box of
 // operand rows.  nbox = 1: the rows of h features (QKV: of h rotary pairs of a head, hr = 2 h); nbox = 2: h gate rows and
 // the h matching up rows, or 2 h rows of the LM head.  The geometry depends on the matrix, the SM count and the class of
-// the call's operand rows, so that the weight maps are encoded once per model: kb is the most that a ring slot holds.
+// the call's operand rows, so that the weight maps are encoded once per model and class (seven sets, 49 maps and 6.3 KB a layer):
+// kb is the most that a ring slot holds.
 // Big boxes matter twice: a thread issues a copy about every quarter of a microsecond whatever its size, and rows of 256
 // bytes and more pass at 70 GB/s per SM where rows of 128 bytes pass at 43.
 // Three larger slots from 80 operand rows on, where a slot of a quarter of the ring holds one k-block only: 13B, 56 rows 8.64 ms
 // with three, 8.75 with four; 7B, 33 rows 3.50 and 3.62.  At up to 64 four are as good (7B, 18 rows 3.98 and 3.96).
+// Beyond 128 operand rows the split QKV's step, two boxes of 128 rows, does not fit a quarter of the ring at all.
 constexpr int FW_CLASSES = 7;
 struct FwClass { int cols, slots; };      // operand rows up to, ring slots
 constexpr FwClass FW_CLASS[FW_CLASSES] = {{16, 4}, {32, 4}, {64, 4}, {80, 3}, {112, 3}, {144, 3}, {FW_MAX_COLS, 3}};
