@@ -72,3 +72,22 @@ def test_forward_edges(models, shape, rows, tree, lengths):
         # The share itself is bounded from above by 0.29 (the first layer's as in cache_ok, the second's with the output moved
         # as said); measured 5e-3..6e-3, held to five times that.
         assert flips <= 0.03 and stats.cache_max_excess <= 2.0 ** -7 * flips ** 0.5 * stats.cache_scale
+
+
+@pytest.mark.parametrize("shape,rows,tree,lengths", [
+    ("hd64", 5, None, [1290]),                                   # 16 heads of 11 tiles: pieces of two, the last of one
+    ("hd64", 5, None, [1100, 1030]),                             # 32 of nine: three, one more than dealt out evenly
+    ("hd64", 6, None, [140, 700, 1280]),                         # of different lengths
+    ("hd64", 5, None, [2170, 300, 2300, 1500]),                  # 64: no pieces, blocks of several heads
+    ("hd64", 33, (4, 8, 4), [1290]),                             # wide items
+])
+def test_attention_pieces(shape, rows, tree, lengths):
+    """Where the keys of a (sequence, KV head) are cut into pieces of a block each, and where blocks take runs of tiles."""
+    sh, B, stats = SHAPES[shape], len(lengths), ParityStats()
+    gm, cases = GpuModel(sh, max_batch=B, max_nodes=rows - 1, capacity=2400), []
+    for b, L in enumerate(lengths):
+        gm.inject(b, L)
+        t = S.beam_tree(*tree, sh.vocab, stream=90 + b) if tree else S.chain_tree(rows - 1, sh.vocab, stream=90 + b)
+        cases.append(SeqCase(b, L, int(S.token_ids(9, (22 << 40) | b, 1, sh.vocab)[0]), t))
+    compare(gm, cases, Bn.log_tau(0.3), S.bonus_uniforms(9, 90 + rows, B, sh.vocab, "cuda"), chain=tree is None, stats=stats)
+    assert stats.ok() and stats.cache_ok(sh.layers, gemm_eps(B * rows, sh.d_ffn)), stats
