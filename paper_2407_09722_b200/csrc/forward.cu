@@ -78,7 +78,9 @@ __device__ __forceinline__ bool grid_wait(const int* c, int want, volatile int* 
 __device__ __forceinline__ void map_acquire(const CUtensorMap* m) {
     asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
 }
-__device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async;" ::: "memory"); }
+// before TMA reads what other SMs wrote to global memory (after the acquire that saw it); the form for all state spaces, which also
+// waits for this thread's shared memory, takes 0.3 us longer a phase
+__device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 __device__ __forceinline__ uint2 pack4(float x, float y, float z, float w) {
     const __nv_bfloat162 p = __floats2bfloat162_rn(x, y), q = __floats2bfloat162_rn(z, w);
     return make_uint2(*reinterpret_cast<const uint32_t*>(&p), *reinterpret_cast<const uint32_t*>(&q));
@@ -215,6 +217,62 @@ __device__ __forceinline__ int attn_cut(const SeqMeta* meta, int B, int heads, i
     }
     return blocks;
 }
+
+// Where a tile's weights lie: map and row coordinate of its boxes (QKV: pair and half-head coordinates).
+struct TileSrc {
+    const CUtensorMap *m, *m2;
+    int row, row2, half, half2;
+};
+__device__ __forceinline__ TileSrc tile_src(const FwArgs& a, int kind, int layer, int tile) {
+    const FwPhase& f = a.ph[kind];
+    const CUtensorMap* w = a.layers[layer].w[a.cls];           // (not read for the LM head)
+    TileSrc t{w, w, tile * f.nbox * f.h, 0, 0, 0};
+    auto of_head = [&](int hg, const CUtensorMap*& map, int& pos) {
+        pos = 2 * (hg < a.Hq ? hg : (hg < a.Hq + a.Hkv ? hg - a.Hq : hg - a.Hq - a.Hkv));
+        map = w + (hg < a.Hq ? 0 : (hg < a.Hq + a.Hkv ? 1 : 2));
+    };
+    if (kind == FW_QKV && f.nbox == 2) {                       // a tile of two heads
+        const int hg = tile / f.c * 2;
+        t.row = 0;
+        of_head(hg, t.m, t.half);
+        of_head(min(hg + 1, a.Hq + 2 * a.Hkv - 1), t.m2, t.half2);
+    } else if (kind == FW_QKV) {
+        const int hg = tile / f.u;
+        t.row = (tile - hg * f.u) * f.h;
+        of_head(hg, t.m, t.half);
+    } else if (kind == FW_GATEUP) {
+        t.m = w + 4;
+        t.m2 = w + 5;
+        t.row = t.row2 = tile * f.h;
+    } else if (kind == FW_LM) {
+        t.m = t.m2 = &a.lm;
+        t.row2 = t.row + f.h;
+    } else {
+        t.m = kind == FW_O ? w + 3 : w + 6;
+        if (f.c > 1) t.row = tile / f.c * f.h;
+    }
+    if (kind != FW_LM) {
+        map_acquire(t.m);
+        if (f.nbox == 2) map_acquire(t.m2);
+    }
+    return t;
+}
+// one step of a tile's weights to the ring slot at `base`
+__device__ __forceinline__ void copy_step(const FwArgs& a, int kind, const TileSrc& t, int step, uint32_t base, uint32_t bar) {
+    const FwPhase& f = a.ph[kind];
+    const int kx = f.flat ? step * TC_TILE_K : 0, kz = f.flat ? 0 : step * f.kb;
+    mbar_expect_tx(bar, (uint32_t)(f.nbox * f.box_bytes + f.kb * a.cols * 128));
+    if (kind == FW_QKV) {
+        tma_load_4d(base, t.m, bar, kx, t.row, t.half, kz, HINT_STREAM);
+        if (f.nbox == 2) tma_load_4d(base + f.box_bytes, t.m2, bar, kx, t.row, t.half2, kz, HINT_STREAM);
+    } else {
+        tma_load_3d(base, t.m, bar, kx, t.row, kz, HINT_STREAM);
+        if (f.nbox == 2) tma_load_3d(base + f.box_bytes, t.m2, bar, kx, t.row2, kz, HINT_STREAM);
+    }
+}
+// steps [k_first, k_end) of a tile are its block's: all of them, or its share
+__device__ __forceinline__ int k_first(const FwPhase& f, int tile) { return f.c > 1 ? (tile % f.c) * f.steps / f.c : 0; }
+__device__ __forceinline__ int k_end(const FwPhase& f, int tile) { return f.c > 1 ? (tile % f.c + 1) * f.steps / f.c : f.steps; }
 
 // What the attention's epilogue warps tell one another, for NR rows in each half of them
 template <int NR>
@@ -975,18 +1033,11 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     const int cta = (int)blockIdx.x, n_cta = a.n_cta;
     const int T = a.T, cols = a.cols, terms = a.terms;
     const int n_phases = 5 * a.n_layers + 1;
-    for (int b = threadIdx.x; b < a.B; b += FW_THREADS) {
-        SeqMeta m;
-        m.nrows = __ldcg(a.rm.n_rows + b);
-        m.L = __ldcg(a.rm.kv_base + b);
-        m.nkeys = min(m.L + __ldcg(a.rm.n_spec + b), a.pieces * FW_KEYS);
-        m.seq = __ldcg(a.rm.call_seq + b);
-        s.meta[b] = m;
-    }
-    for (int t = threadIdx.x; t < min(T, FW_MAX_ROWS); t += FW_THREADS) {     // (more rows: the attention alone)
-        s.slot[t] = __ldcg(a.rm.slot + t);
-        s.rowb[t] = (uint8_t)(t / a.R);
-    }
+    auto slot_ptr = [&](int pos) { return smem_u32(smem) + (uint32_t)(pos % NS) * FW_SLOT; };
+    auto full_bar = [&](int pos) { return smem_u32(&s.full[pos % NS]); };
+    auto empty_bar = [&](int pos) { return smem_u32(&s.empty[pos % NS]); };
+    auto ring_par = [&](int pos) { return (uint32_t)(pos / NS) & 1u; };
+    int n_pre = 0;                                     // (thread 0)
     if (threadIdx.x == 0) {
         for (int i = 0; i < NS; ++i) {
             mbar_init(smem_u32(&s.full[i]), 1);
@@ -1004,6 +1055,27 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         s.abort_flag[1] = (int)(a.wait_limit ? a.wait_limit : WAIT_LIMIT);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        // The first projection's weights wait for nothing: as many steps as the ring holds are asked for before the rest of the
+        // block's set-up, which takes 2 us.
+        if (a.p_lo % 5 == FW_QKV && a.p_lo < 5 * a.n_layers && cta < a.ph[FW_QKV].n_tiles) {
+            const FwPhase& f = a.ph[FW_QKV];
+            const TileSrc src = tile_src(a, FW_QKV, a.p_lo / 5, cta);
+            const int k0 = k_first(f, cta);
+            n_pre = min(NS, k_end(f, cta) - k0);
+            for (int i = 0; i < n_pre; ++i) copy_step(a, FW_QKV, src, k0 + i, slot_ptr(i), full_bar(i));
+        }
+    }
+    for (int b = (int)threadIdx.x - 32; b >= 0 && b < a.B; b += FW_THREADS - 32) {         // (not the warp that issues copies)
+        SeqMeta m;
+        m.nrows = __ldcg(a.rm.n_rows + b);
+        m.L = __ldcg(a.rm.kv_base + b);
+        m.nkeys = min(m.L + __ldcg(a.rm.n_spec + b), a.pieces * FW_KEYS);
+        m.seq = __ldcg(a.rm.call_seq + b);
+        s.meta[b] = m;
+    }
+    for (int t = (int)threadIdx.x - 32; t >= 0 && t < min(T, FW_MAX_ROWS); t += FW_THREADS - 32) {     // (more rows: the attention alone)
+        s.slot[t] = __ldcg(a.rm.slot + t);
+        s.rowb[t] = (uint8_t)(t / a.R);
     }
     if (warp == 3) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s.tmem_ptr)), "r"(512)
@@ -1021,7 +1093,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     // and KV head), the first segment comes last, because it ends with the tile that holds the call's own rows and cannot
     // be requested before the phase has been released.  a_wrap: where the order returns to the front of the range.
     const AttnPos &a_zero = s.apos[0], &a_last = s.apos[1], &a_first = s.apos[2];
-    if (warp == 0) {
+    if (warp == 1) {
         // Dealt out evenly, a block's tiles may be of two (sequence, KV head)s or more, and the end of each (sums over the keys,
         // output to global memory, the next one's first scores) costs as much as two tiles and a half: pieces that keep to one are
         // taken where they are at most two tiles longer, a lane per length tried.  7B chain, 32 heads of 17 tiles: pieces of
@@ -1051,13 +1123,6 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
         if (next == a_wrap) it = a_zero;
         else attn_next(it, s.meta, a.B, heads);
     };
-    auto slot_ptr = [&](int pos) { return smem_u32(smem) + (uint32_t)(pos % NS) * FW_SLOT; };
-    auto full_bar = [&](int pos) { return smem_u32(&s.full[pos % NS]); };
-    auto empty_bar = [&](int pos) { return smem_u32(&s.empty[pos % NS]); };
-    auto ring_par = [&](int pos) { return (uint32_t)(pos / NS) & 1u; };
-    // steps [k0, k1) of a tile: all of them, or this block's share
-    auto k_first = [&](const FwPhase& f, int tile) { return f.c > 1 ? (tile % f.c) * f.steps / f.c : 0; };
-    auto k_end = [&](const FwPhase& f, int tile) { return f.c > 1 ? (tile % f.c + 1) * f.steps / f.c : f.steps; };
     // kind of phase p
     auto kind_of = [&](int p) { return p == n_phases - 1 ? (int)FW_LM : p % 5; };
 
@@ -1069,7 +1134,6 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
             bool ok = true;
             for (int p = a.p_lo; p < a.p_hi && ok; ++p) {
                 const int kind = kind_of(p), layer = p / 5;
-                const FwLayer* L = a.layers + layer;
                 if (kind == FW_ATTN) {
                     bool waited = p == a.p_lo;
                     AttnPos it = a_first;
@@ -1098,55 +1162,14 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     continue;
                 }
                 const FwPhase& f = a.ph[kind];
-                const CUtensorMap* w = L->w[a.cls];
-                const uint32_t bytes = (uint32_t)(f.nbox * f.box_bytes + f.kb * cols * 128);
                 for (int tile = cta; tile < f.n_tiles && ok; tile += n_cta) {
-                    // the tile's first box: map, row coordinate (QKV: pair and half-head coordinates)
-                    const CUtensorMap* m = w;
-                    int row = tile * f.nbox * f.h, half = 0;
-                    const CUtensorMap* m2 = m;         // QKV, a tile of two heads: the second
-                    int half2 = 0;
-                    auto of_head = [&](int hg, const CUtensorMap*& map, int& pos2) {
-                        pos2 = 2 * (hg < a.Hq ? hg : (hg < a.Hq + a.Hkv ? hg - a.Hq : hg - a.Hq - a.Hkv));
-                        map = w + (hg < a.Hq ? 0 : (hg < a.Hq + a.Hkv ? 1 : 2));
-                    };
-                    if (kind == FW_QKV && f.nbox == 2) {
-                        const int hg = tile / f.c * 2;
-                        row = 0;
-                        of_head(hg, m, half);
-                        of_head(min(hg + 1, a.Hq + 2 * a.Hkv - 1), m2, half2);
-                    } else if (kind == FW_QKV) {
-                        const int hg = tile / f.u;
-                        row = (tile - hg * f.u) * f.h;
-                        of_head(hg, m, half);
-                    } else if (kind == FW_GATEUP) {
-                        m = w + 4;
-                        row = tile * f.h;
-                    } else {
-                        m = kind == FW_O ? w + 3 : (kind == FW_DOWN ? w + 6 : &a.lm);
-                        if (f.c > 1) row = tile / f.c * f.h;
-                    }
-                    if (kind != FW_LM) {
-                        map_acquire(m);
-                        if (kind == FW_GATEUP) map_acquire(m + 1);
-                        if (kind == FW_QKV && f.nbox == 2) map_acquire(m2);
-                    }
+                    const TileSrc src = tile_src(a, kind, layer, tile);
                     const int k1 = k_end(f, tile);
                     for (int step = k_first(f, tile); step < k1; ++step, ++pos) {
+                        if (pos < n_pre) continue;
                         ok = mbar_wait(empty_bar(pos), ring_par(pos) ^ 1u, abort_flag);
                         if (!ok) break;
-                        const uint32_t bar = full_bar(pos), base = slot_ptr(pos);
-                        const int kx = f.flat ? step * TC_TILE_K : 0, kz = f.flat ? 0 : step * f.kb;
-                        mbar_expect_tx(bar, bytes);
-                        if (kind == FW_QKV) {
-                            tma_load_4d(base, m, bar, kx, row, half, kz, HINT_STREAM);
-                            if (f.nbox == 2) tma_load_4d(base + f.box_bytes, m2, bar, kx, row, half2, kz, HINT_STREAM);
-                        } else {
-                            tma_load_3d(base, m, bar, kx, row, kz, HINT_STREAM);
-                            if (f.nbox == 2)
-                                tma_load_3d(base + f.box_bytes, kind == FW_GATEUP ? m + 1 : m, bar, kx,
-                                            kind == FW_GATEUP ? row : row + f.h, kz, HINT_STREAM);
-                        }
+                        copy_step(a, kind, src, step, slot_ptr(pos), full_bar(pos));
                     }
                 }
             }
