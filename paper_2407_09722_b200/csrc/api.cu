@@ -59,6 +59,7 @@ struct mtad_ctx {
     CUtensorMap fw_lm[2][FW_CLASSES];                  // its LM-head maps: target, auxiliary model
     bool fw_ok[2] = {false, false};                    // the table and maps of the target, of the auxiliary model are there
     bool resident = false;              // a cooperative launch of kCtas blocks is possible, as far as is known
+    bool counters_stale = false;        // the split-K arrival counters have yet to be zeroed for this call
     bool refuse_resident = false;       // debug: such launches ask for more blocks than fit
     bool use_tc = false, use_pdl = false;
     size_t tc_ws_floats = 0, tc_counter_n = 0, xf_elems = 0;
@@ -209,6 +210,7 @@ size_t carve(mtad_ctx* c, const mtad_model_desc* t, const mtad_model_desc* a, in
     sc.qkv = k.take<float>(T * qkv, "qkv");
     sc.attn = k.take<float>(T * qd, "attn");
     sc.act = k.take<float>(T * F, "act");
+    sc.arrive = reinterpret_cast<int32_t*>(sc.act);
     sc.rope = k.take<float>(T * hh * 2, "rope");
     sc.attn_part = k.take<float>(T * part, "attn_part");
     sc.q_hi = k.take<__nv_bfloat16>(T * qd, "q_hi");
@@ -647,18 +649,36 @@ AttnSplit attn_split(const ModelView& m, int B, int R, long long total) {
     return {nsp, (int)(((total + 63) / 64 + nsp - 1) / nsp)};
 }
 
+bool takes_one_launch(const mtad_ctx* ctx, const ModelView& m, int B, int R, long long total) {
+    return ctx->resident && ctx->fw_ok[&m == &ctx->aux] && fw_pays(m.d, B, R, total);
+}
+uint64_t plan_key(const mtad_ctx* ctx, const ModelView& m, int B, int R, bool lm_plain, bool one) {
+    return ((uint64_t)(&m == &ctx->aux ? 1 : 0) << 40) | ((uint64_t)B << 24) | ((uint64_t)R << 8) | (lm_plain ? 1u : 0u) | (one ? 2u : 0u);
+}
+
+// A launch that gave up on a wait leaves split-K arrival counters behind: every call that uses them starts from zero.  They are
+// zeroed here unless the call's (first) forward is known to be one launch, which has none; else ahead of the first that is not.
+int begin_forwards(mtad_ctx* ctx, const ModelView& m, int B, int R, long long len_ub, bool lm_plain, cudaStream_t s) {
+    const bool one = takes_one_launch(ctx, m, B, R, std::min<long long>(len_ub, m.d.kv_capacity) + R);
+    const auto it = ctx->plans.find(plan_key(ctx, m, B, R, lm_plain, one));
+    ctx->counters_stale = it != ctx->plans.end() && it->second.one_launch;
+    if (!ctx->counters_stale) CU(cudaMemsetAsync(ctx->sc.tc_counters, 0, sizeof(int32_t) * ctx->tc_counter_n, s));
+    return MTAD_OK;
+}
+
 // The forward on the tensor-core path: every projection is one launch of the TMA + tcgen05 GEMM with a fused
 // epilogue; activations travel between launches as bf16 operand rows plus per-row sums of squares, so the RMSNorm is
-// applied as a per-row scale in the consumer's epilogue.  Leaves lm_part / node_z for launch_lm_merge.
+// applied as a per-row scale in the consumer's epilogue.  Ends in plain logits, or in the acceptance.
+// `accept`: what the acceptance needs, which follows in the launch that merges the LM head's partials (null: plain logits).
 int forward_rows_tc(mtad_ctx* ctx, const ModelView& m, const WeightMaps& wm, int B, int R, long long len_ub,
-                    const float* uniforms, uint32_t* status, bool lm_plain, cudaStream_t s) {
+                    const float* uniforms, uint32_t* status, const AcceptArgs* accept, const mtad_result* out, cudaStream_t s) {
+    const bool lm_plain = accept == nullptr;
     const mtad_model_desc& d = m.d;
     const Scratch& sc = ctx->sc;
     const long long total = std::min<long long>(len_ub, d.kv_capacity) + R;
     const bool pdl = ctx->use_pdl;
-    const bool one = ctx->resident && ctx->fw_ok[&m == &ctx->aux] && fw_pays(d, B, R, total);
-    const uint64_t key = ((uint64_t)(&m == &ctx->aux ? 1 : 0) << 40) | ((uint64_t)B << 24) | ((uint64_t)R << 8) |
-                         (lm_plain ? 1u : 0u) | (one ? 2u : 0u);
+    const bool one = takes_one_launch(ctx, m, B, R, total);
+    const uint64_t key = plan_key(ctx, m, B, R, lm_plain, one);
     auto it = ctx->plans.find(key);
     if (it == ctx->plans.end()) {
         ForwardPlan fp;
@@ -687,11 +707,15 @@ int forward_rows_tc(mtad_ctx* ctx, const ModelView& m, const WeightMaps& wm, int
         const int rc = timed(ctx, MTAD_K_GEMM, fp.fw_bytes, 1, s, [&] { return launch_forward(fp.fw, s, ctx->refuse_resident); });
         if (too_large(rc)) {
             ctx->plans.clear();
-            return forward_rows_tc(ctx, m, wm, B, R, len_ub, uniforms, status, lm_plain, s);
+            return forward_rows_tc(ctx, m, wm, B, R, len_ub, uniforms, status, accept, out, s);
         }
         if (rc != MTAD_OK) return rc;
-        if (!lm_plain) RUN(MTAD_K_LMRED, 0, 2, launch_lm_merge(m, ctx->rm, sc, B, R, fp.lm_tiles128, uniforms, status, s));
+        if (accept) RUN(MTAD_K_LMRED, 0, 1, launch_lm_accept(m, ctx->rm, sc, fp.lm_tiles128, uniforms, *accept, *out, pdl, s));
         return MTAD_OK;
+    }
+    if (ctx->counters_stale) {
+        CU(cudaMemsetAsync(sc.tc_counters, 0, sizeof(int32_t) * ctx->tc_counter_n, s));
+        ctx->counters_stale = false;
     }
     auto launch = [&](size_t i) -> int {
         GemmDesc& gd = fp.g[i];
@@ -733,7 +757,7 @@ int forward_rows_tc(mtad_ctx* ctx, const ModelView& m, const WeightMaps& wm, int
         }
         if (int rc = launch(i)) return rc;
     }
-    if (!lm_plain) RUN(MTAD_K_LMRED, 0, 2, launch_lm_merge(m, ctx->rm, sc, B, R, fp.lm_tiles128, uniforms, status, s));
+    if (accept) RUN(MTAD_K_LMRED, 0, 1, launch_lm_accept(m, ctx->rm, sc, fp.lm_tiles128, uniforms, *accept, *out, pdl, s));
     return MTAD_OK;
 }
 
@@ -770,8 +794,9 @@ int verify_common(mtad_ctx* ctx, int B, const int32_t* seqs, const int32_t* n_no
     for (int i = 0; i < B; ++i) ub = std::max(ub, ctx->len_ub[seqs[i]]);
 
     CU(cudaMemsetAsync(out->status, 0, sizeof(uint32_t) * B, s));
-    // a launch that gave up on a wait leaves split-K arrival counters behind: every call starts from zero
-    CU(cudaMemsetAsync(ctx->sc.tc_counters, 0, sizeof(int32_t) * ctx->tc_counter_n, s));
+    const bool spd = spd_accept_uniform != nullptr;
+    const bool warped = ctx->warp_k > 0 && !spd;   // warped rows are made from plain logits, after the forward
+    if (int rc = begin_forwards(ctx, ctx->target, B, R, ub, warped || spd, s)) return rc;
     PrepareArgs pa{};
     for (int i = 0; i < B; ++i) pa.seqs.v[i] = seqs[i];
     pa.B = B; pa.R = R; pa.max_depth = D; pa.n_nodes = n_nodes; pa.tok = tok; pa.parent = parent;
@@ -786,10 +811,10 @@ int verify_common(mtad_ctx* ctx, int B, const int32_t* seqs, const int32_t* n_no
         pa.sumsq_out = ctx->sc.sumsq_a;
     }
     RUN(MTAD_K_PREPARE, 0, 1, launch_prepare(ctx->target, ctx->st, ctx->rm, ctx->sc, pa, out->status, s));
-    const bool spd = spd_accept_uniform != nullptr;
-    const bool warped = ctx->warp_k > 0 && !spd;   // warped rows are made from plain logits, after the forward
+    const AcceptArgs aa{B, R, D, tok, parent, logq_ref, log_tau};
+    const bool fused = tc && !warped && !spd;
     if (tc) {
-        int rc = forward_rows_tc(ctx, ctx->target, ctx->tmaps, B, R, ub, bonus_uniform, out->status, warped || spd, s);
+        int rc = forward_rows_tc(ctx, ctx->target, ctx->tmaps, B, R, ub, bonus_uniform, out->status, fused ? &aa : nullptr, out, s);
         if (rc != MTAD_OK) return rc;
     } else {
         int rc = forward_rows(ctx, ctx->target, B, R, ub, s);
@@ -805,9 +830,8 @@ int verify_common(mtad_ctx* ctx, int B, const int32_t* seqs, const int32_t* n_no
     if (spd) {
         SpdArgs sa{B, R, D, tok, logq_ref, spd_accept_uniform, bonus_uniform};
         RUN(MTAD_K_ACCEPT, 0, 3, launch_spd_accept(ctx->target, ctx->rm, ctx->sc, sa, *out, ctx->use_pdl, s));
-    } else {
-        AcceptArgs aa{B, R, D, tok, parent, logq_ref, log_tau};
-        RUN(MTAD_K_ACCEPT, 0, 1, launch_accept(ctx->rm, ctx->sc, aa, *out, s));
+    } else if (!fused) {
+        RUN(MTAD_K_ACCEPT, 0, 1, launch_accept(ctx->rm, ctx->sc, aa, *out, ctx->use_pdl, s));
     }
     ctx->last_B = B; ctx->last_R = R; ctx->last_D = D;
     ctx->last_chain = (parent == nullptr);
@@ -1110,15 +1134,16 @@ int mtad_draft(mtad_ctx* ctx, int B, const int32_t* seqs, int gamma, int beam_wi
     for (int i = 0; i < B; ++i) sl.v[i] = seqs[i];
     DraftOut out{n_nodes, tok, parent, depth, node_logq, logq_ref, best_path};
     const bool tc = ctx->use_tc && ctx->amaps.ok;
-    CU(cudaMemsetAsync(ctx->sc.tc_counters, 0, sizeof(int32_t) * ctx->tc_counter_n, s));
+    if (int rc = begin_forwards(ctx, m, B, R0, ub + 1, true, s)) return rc;
     for (int step = 0; step < gamma; ++step) {
         const int R = step == 0 ? R0 : beam_width;
-        RUN(MTAD_K_PREPARE, 0, 1, launch_draft_prepare(m, ctx->st, ctx->ds, ctx->rm, ctx->sc, sl, B, R, step, beam_width,
-                                                       tc && B * R <= TC_MAX_ROWS, dwarp, ctx->use_pdl, s));
+        if (step == 0 || dwarp)                         // (otherwise the selection of the step before made the rows)
+            RUN(MTAD_K_PREPARE, 0, 1, launch_draft_prepare(m, ctx->st, ctx->ds, ctx->rm, ctx->sc, sl, B, R, step, beam_width,
+                                                           tc && B * R <= TC_MAX_ROWS, dwarp, ctx->use_pdl, s));
         // keys of the auxiliary cache: committed ones, the pending rows and every node drafted so far
         const long long keys_ub = ub + 1 + (long long)step * beam_width;
         int rc;
-        if (tc && B * R <= TC_MAX_ROWS) rc = forward_rows_tc(ctx, m, ctx->amaps, B, R, keys_ub, nullptr, ctx->ds.status, true, s);
+        if (tc && B * R <= TC_MAX_ROWS) rc = forward_rows_tc(ctx, m, ctx->amaps, B, R, keys_ub, nullptr, ctx->ds.status, nullptr, nullptr, s);
         else rc = forward_rows(ctx, m, B, R, keys_ub, s);
         if (rc != MTAD_OK) return rc;
         if (dwarp) {
@@ -1128,7 +1153,10 @@ int mtad_draft(mtad_ctx* ctx, int B, const int32_t* seqs, int gamma, int beam_wi
                                                                keep_all, uniforms, out, s));
             continue;
         }
-        RUN(MTAD_K_LMRED, 0, 2, launch_draft_select(m, ctx->ds, ctx->sc, sl, B, R, step, gamma, beam_width, keep_all, uniforms, out,
+        if (!(tc && B * R <= TC_MAX_ROWS))              // (the CUDA-core forward has written over the counters)
+            CU(cudaMemsetAsync(ctx->sc.arrive, 0, sizeof(int32_t) * B, s));
+        RUN(MTAD_K_LMRED, 0, 1, launch_draft_select(m, ctx->ds, ctx->sc, sl, B, R, step, gamma, beam_width, keep_all, uniforms, out,
+                                                     ctx->st, ctx->rm, step + 1 < gamma, tc && B * beam_width <= TC_MAX_ROWS,
                                                      ctx->use_pdl, s));
     }
     ctx->draft_active = true;
@@ -1167,20 +1195,18 @@ int kv_commit(mtad_ctx* ctx, int B, const int32_t* seqs, const mtad_result* res,
     if (!seqs_ok(ctx, B, seqs)) return MTAD_E_INVALID;
     if (B != ctx->last_B || memcmp(seqs, ctx->last_seqs, sizeof(int32_t) * B) != 0) return MTAD_E_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    // auxiliary cache: after a draft its accepted rows are kept; otherwise the accepted tokens wait for replay
+    const bool after_draft = ctx->has_aux && ctx->draft_active && ctx->draft_B == B &&
+                             memcmp(seqs, ctx->draft_seqs, sizeof(int32_t) * B) == 0;
+    const int mode = after_draft ? (ctx->last_chain ? 0 : 1) : 2;
+    RUN(MTAD_K_COMMIT, 0, 2,
+        launch_commit(ctx->target, ctx->has_aux ? &ctx->aux : nullptr, ctx->st, ctx->ds, B, ctx->rm.call_seq, *res, ctx->last_D, mode,
+                      ctx->use_pdl, s));
     if (ctx->has_aux) {
-        // auxiliary cache: after a draft its accepted rows are kept; otherwise the accepted tokens wait for replay
-        const bool after_draft = ctx->draft_active && ctx->draft_B == B &&
-                                 memcmp(seqs, ctx->draft_seqs, sizeof(int32_t) * B) == 0;
-        const int mode = after_draft ? (ctx->last_chain ? 0 : 1) : 2;
-        RUN(MTAD_K_COMMIT, 0, 2,
-            launch_aux_commit(ctx->aux, ctx->st, ctx->ds, B, ctx->rm.call_seq, *res, ctx->last_D, mode, s));
         for (int i = 0; i < B; ++i)
             ctx->npend_ub[seqs[i]] = after_draft ? 2 : std::min(ctx->npend_ub[seqs[i]] + ctx->last_D + 1, MTAD_MAX_DEPTH + 1);
         ctx->draft_active = false;
     }
-    RUN(MTAD_K_COMMIT, 0, 1, launch_kv_commit(ctx->target, ctx->st, B, ctx->rm.call_seq, *res, ctx->last_D, s));
-    RUN(MTAD_K_COMMIT, 0, 1, launch_seq_advance(ctx->st, B, ctx->rm.call_seq, *res, ctx->last_D, ctx->max_batch,
-                                              (long long)ctx->target.d.kv_capacity, s));
     for (int i = 0; i < B; ++i)
         ctx->len_ub[seqs[i]] = std::min<long long>(ctx->len_ub[seqs[i]] + ctx->last_D + 1, ctx->target.d.kv_capacity);
     ctx->last_B = 0;

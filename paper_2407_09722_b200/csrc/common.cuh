@@ -130,6 +130,8 @@ struct Scratch {
     float* sumsq_b;      // [tiles(d)][256] the same after the O projection
     float* tc_ws;        // split-K partial tiles
     int32_t* tc_counters;
+    int32_t* arrive;         // [max_batch] blocks of a sequence that have finished their part of a launch whose last one goes on.
+                             // Lies over `act`, which the CUDA-core forward alone uses; 0 between launches of the other path.
     float4* lm_part;     // [T][tiles(V)]
     float* node_z;       // [T]
     DraftPart* draft_part;   // [max_batch][MTAD_MAX_BEAM][MTAD_DRAFT_CHUNKS], only with an auxiliary model
@@ -221,17 +223,17 @@ __device__ __forceinline__ void store_terms4(float4 v, __nv_bfloat16* x, size_t 
 }
 
 // One embedding row -> the fp32 hidden row and (tensor-core path) its bf16 operand terms times the first norm's gain;
-// returns this thread's share of the row's sum of squares.  16-byte loads, four in flight per thread: a scalar loop
+// returns this thread's (`tid` of `n_thr`) share of the row's sum of squares.  16-byte loads, four in flight per thread: a scalar loop
 // whose loads wait behind the previous iteration's stores pays one DRAM latency per element (32 us for a 4096-wide
 // row).  d is a multiple of 8; rows that are not 16-byte aligned take the scalar loop.
 __device__ __forceinline__ float embed_row(const __nv_bfloat16* __restrict__ src_row, bool ok, int d,
                                            float* __restrict__ hidden_row, const __nv_bfloat16* __restrict__ gain,
-                                           __nv_bfloat16* x_row, int terms) {
+                                           __nv_bfloat16* x_row, int terms, int tid, int n_thr) {
     float ss = 0.f;
     const bool vec = ((reinterpret_cast<uintptr_t>(src_row) | reinterpret_cast<uintptr_t>(hidden_row) |
                        reinterpret_cast<uintptr_t>(gain) | reinterpret_cast<uintptr_t>(x_row)) & 15) == 0;
     if (!vec) {
-        for (int i = threadIdx.x; i < d; i += blockDim.x) {
+        for (int i = tid; i < d; i += n_thr) {
             const float v = ok ? __bfloat162float(src_row[i]) : 0.f;
             hidden_row[i] = v;
             if (x_row) {
@@ -244,17 +246,17 @@ __device__ __forceinline__ float embed_row(const __nv_bfloat16* __restrict__ src
     const int nv = d >> 3;
     const uint4* src = reinterpret_cast<const uint4*>(src_row);
     const uint4* gsrc = reinterpret_cast<const uint4*>(gain);
-    for (int c0 = threadIdx.x; c0 < nv; c0 += 4 * blockDim.x) {
+    for (int c0 = tid; c0 < nv; c0 += 4 * n_thr) {
         uint4 q[4], gq[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const int c = c0 + k * blockDim.x;
+            const int c = c0 + k * n_thr;
             q[k] = (ok && c < nv) ? __ldg(src + c) : make_uint4(0u, 0u, 0u, 0u);
             gq[k] = (x_row && c < nv) ? __ldg(gsrc + c) : make_uint4(0u, 0u, 0u, 0u);
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const int c = c0 + k * blockDim.x;
+            const int c = c0 + k * n_thr;
             if (c >= nv) continue;
             const uint32_t w[4] = {q[k].x, q[k].y, q[k].z, q[k].w}, gw[4] = {gq[k].x, gq[k].y, gq[k].z, gq[k].w};
             float v[8];
@@ -342,8 +344,6 @@ cudaError_t launch_attention_mma(const ModelView& m, int layer, const RowMeta& r
                                  int nsplit, int nsp, uint32_t* status, bool pdl, cudaStream_t st);
 cudaError_t launch_attention_combine(const ModelView& m, const RowMeta& rm, const Scratch& sc, int B, int R, int nsplit,
                                      bool emit_split, bool pdl, cudaStream_t st);
-cudaError_t launch_lm_merge(const ModelView& m, const RowMeta& rm, const Scratch& sc, int B, int R, int n_tiles,
-                            const float* bonus_uniform, uint32_t* status, cudaStream_t st);
 cudaError_t launch_lm_reduce(const ModelView& m, const RowMeta& rm, const Scratch& sc, int B, int R,
                              const float* bonus_uniform, const int32_t* tok, const int32_t* parent,
                              uint32_t* status, cudaStream_t st);
@@ -357,6 +357,9 @@ struct AcceptArgs {
     const float* logq_ref;     // [B, max_depth]
     float log_tau;
 };
+// Merge of the LM head's partials, the nodes' log-probabilities and the acceptance, one launch.
+cudaError_t launch_lm_accept(const ModelView& m, const RowMeta& rm, const Scratch& sc, int n_tiles, const float* bonus_uniform,
+                             const AcceptArgs& a, const mtad_result& out, bool pdl, cudaStream_t st);
 struct SpdArgs {
     int B, R, max_depth;
     const int32_t* tok;             // [B, R-1]
@@ -366,26 +369,24 @@ struct SpdArgs {
 };
 cudaError_t launch_spd_accept(const ModelView& m, const RowMeta& rm, const Scratch& sc, const SpdArgs& a,
                               const mtad_result& out, bool pdl, cudaStream_t st);
-cudaError_t launch_accept(const RowMeta& rm, const Scratch& sc, const AcceptArgs& a, const mtad_result& out,
+cudaError_t launch_accept(const RowMeta& rm, const Scratch& sc, const AcceptArgs& a, const mtad_result& out, bool pdl,
                           cudaStream_t st);
-cudaError_t launch_kv_commit(const ModelView& m, const SeqState& s, int B, const int32_t* call_seq_dev,
-                             const mtad_result& res, int max_depth, cudaStream_t st);
-cudaError_t launch_seq_advance(const SeqState& s, int B, const int32_t* call_seq_dev, const mtad_result& res,
-                               int max_depth, int max_batch, long long cap, cudaStream_t st);
 cudaError_t launch_draft_prepare(const ModelView& m, const SeqState& s, const DraftState& ds, const RowMeta& rm,
                                  const Scratch& sc, const SeqList& seqs, int B, int R, int step, int beam, bool tc,
                                  bool warped, bool pdl, cudaStream_t st);
 cudaError_t launch_draft_select(const ModelView& m, const DraftState& ds, const Scratch& sc, const SeqList& seqs, int B,
                                 int R, int step, int gamma, int beam, int keep_all, const float* uniforms,
-                                const DraftOut& out, bool pdl, cudaStream_t st);
+                                const DraftOut& out, const SeqState& s, const RowMeta& rm, bool next, bool tc, bool pdl,
+                                cudaStream_t st);
 cudaError_t launch_draft_select_warped(const ModelView& m, const DraftState& ds, const Scratch& sc, const SeqList& seqs,
                                        int B, int R, int step, int gamma, int beam, int keep_all, const float* uniforms,
                                        const DraftOut& out, cudaStream_t st);
 cudaError_t launch_warp_rows_only(const ModelView& m, const RowMeta& rm, const Scratch& sc, int B, int R, int top_k,
                                   float top_p, const float* uni, cudaStream_t st);
-cudaError_t launch_aux_commit(const ModelView& aux, const SeqState& s, const DraftState& ds, int B,
-                              const int32_t* call_seq_dev, const mtad_result& res, int max_depth, int mode,
-                              cudaStream_t st);
+// Roll-forward after a verification: the accepted rows of both caches, then the sequences' states.  aux null: no auxiliary model;
+// mode: 0 / 1 after a draft (chain, tree), 2 without one.
+cudaError_t launch_commit(const ModelView& m, const ModelView* aux, const SeqState& s, const DraftState& ds, int B,
+                          const int32_t* call_seq_dev, const mtad_result& res, int max_depth, int mode, bool pdl, cudaStream_t st);
 cudaError_t launch_seq_set(const SeqState& s, int seq, int kv_len, int root, int aux_len, int npend,
                            const int32_t* pend_host, cudaStream_t st);
 

@@ -71,7 +71,7 @@ cudaError_t launch_seq_set(const SeqState& s, int seq, int kv_len, int root, int
 __global__ void prepare_kernel(const __nv_bfloat16* __restrict__ embed, int d, int vocab, int hd, RopeInv rinv,
                                long long kv_capacity, SeqState s, RowMeta rm, float* __restrict__ hidden,
                                float* __restrict__ rope, PrepareArgs a, uint32_t* status, int32_t* __restrict__ sync,
-                               int sync_words) {
+                               int sync_words, int32_t* __restrict__ arrive) {
     const int t = blockIdx.x, bi = t / a.R, r = t % a.R;
     for (int i = t * blockDim.x + threadIdx.x; i < sync_words; i += gridDim.x * blockDim.x) sync[i] = 0;
     const int seq = a.seqs.v[bi];
@@ -126,6 +126,7 @@ __global__ void prepare_kernel(const __nv_bfloat16* __restrict__ embed, int d, i
         }
         rm.prow[t] = pr;
         if (r == 0) {
+            arrive[bi] = 0;
             rm.n_rows[bi] = seq_ok ? nn + 1 : 0;
             rm.n_spec[bi] = seq_ok ? nn + 1 : 0;
             rm.kv_base[bi] = L;
@@ -139,7 +140,7 @@ __global__ void prepare_kernel(const __nv_bfloat16* __restrict__ embed, int d, i
     const int tok = sh_tok;
     const bool ok = sh_ok;
     float ss = embed_row(embed + (size_t)tok * d, ok, d, hidden + (size_t)t * d, a.gain0,
-                         a.x ? a.x + (size_t)t * a.terms * d : nullptr, a.terms);
+                         a.x ? a.x + (size_t)t * a.terms * d : nullptr, a.terms, threadIdx.x, blockDim.x);
     if (a.x) {
         __shared__ float red[32];
         ss = block_sum(ss, red);                     // (also orders the hidden row's stores before the loop below)
@@ -163,7 +164,7 @@ cudaError_t launch_prepare(const ModelView& m, const SeqState& s, const RowMeta&
     prepare_kernel<<<a.B * a.R, 128, 0, st>>>(static_cast<const __nv_bfloat16*>(m.d.embed), m.d.d_model, m.d.vocab,
                                               m.d.head_dim, rope_inv((double)m.d.rope_base, m.d.head_dim),
                                               (long long)m.d.kv_capacity, s, rm,
-                                              sc.hidden, sc.rope, a, status, sc.fw_sync, sc.fw_sync_words);
+                                              sc.hidden, sc.rope, a, status, sc.fw_sync, sc.fw_sync_words, sc.arrive);
     return cudaGetLastError();
 }
 
@@ -442,92 +443,34 @@ cudaError_t launch_lm_reduce(const ModelView& m, const RowMeta& rm, const Scratc
     return e;
 }
 
-// Merge of the LM-head kernel's per-(row, vocab tile) partials, in tile order: log-sum-exp, Gumbel-argmax candidate
-// and its log-probability per row, then the log-probability of every node's token under its parent row.
-__global__ void lm_merge_kernel(const float4* __restrict__ part, int n_tiles, int V, int R,
-                                const float* __restrict__ uni, const int32_t* __restrict__ slot,
-                                float* __restrict__ row_lse, int32_t* __restrict__ row_cand,
-                                float* __restrict__ row_cand_lp, uint32_t* status) {
-    const int t = blockIdx.x, bi = t / R;
-    if (slot[t] < 0) {
-        if (threadIdx.x == 0) { row_lse[t] = 0.f; row_cand[t] = 0; row_cand_lp[t] = 0.f; }
-        return;
-    }
-    float m = -CUDART_INF_F, s = 0.f;
-    Best best{-CUDART_INF_F, 0x7fffffff};
-    for (int j = threadIdx.x; j < n_tiles; j += blockDim.x) {
-        const float4 q = part[idx_lm_part(t, n_tiles, j)];
-        const float mm = fmaxf(m, q.x);
-        s = (m == -CUDART_INF_F ? 0.f : s * expf(m - mm)) + (q.x == -CUDART_INF_F ? 0.f : q.y * expf(q.x - mm));
-        m = mm;
-        best = better(best, Best{q.z, __float_as_int(q.w)});
-    }
-    __shared__ float sm[256], ss[256], sv[256];
-    __shared__ int si[256];
-    sm[threadIdx.x] = m; ss[threadIdx.x] = s; sv[threadIdx.x] = best.v; si[threadIdx.x] = best.i;
-    __syncthreads();
-    for (int o = blockDim.x >> 1; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            const float m1 = sm[threadIdx.x], m2 = sm[threadIdx.x + o];
-            const float mm = fmaxf(m1, m2);
-            const float s1 = (m1 == -CUDART_INF_F) ? 0.f : ss[threadIdx.x] * expf(m1 - mm);
-            const float s2 = (m2 == -CUDART_INF_F) ? 0.f : ss[threadIdx.x + o] * expf(m2 - mm);
-            sm[threadIdx.x] = mm; ss[threadIdx.x] = s1 + s2;
-            const Best b = better(Best{sv[threadIdx.x], si[threadIdx.x]},
-                                  Best{sv[threadIdx.x + o], si[threadIdx.x + o]});
-            sv[threadIdx.x] = b.v; si[threadIdx.x] = b.i;
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        const float lse = sm[0] + logf(ss[0]);
-        // a row of NaN logits wins no comparison and leaves no candidate: flag it instead of indexing with it
-        const bool none = (unsigned)si[0] >= (unsigned)V;
-        if (none || !isfinite(lse)) atomicOr(&status[bi], MTAD_ST_NONFINITE);
-        const int c = none ? 0 : si[0];
-        row_lse[t] = lse;
-        row_cand[t] = c;
-        // the partial keeps logit + noise; take the noise off again to get the candidate's logit
-        const float g = -logf(-logf(uni[(size_t)bi * V + c]));
-        row_cand_lp[t] = (sv[0] - g) - lse;
-    }
-}
-
-__global__ void node_lp_from_z_kernel(const float* __restrict__ node_z, const int32_t* __restrict__ prow,
-                                      const float* __restrict__ row_lse, float* __restrict__ node_lp, int T) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= T) return;
-    const int pr = prow[t];
-    node_lp[t] = pr >= 0 ? node_z[t] - row_lse[pr] : 0.f;
-}
-
-cudaError_t launch_lm_merge(const ModelView& m, const RowMeta& rm, const Scratch& sc, int B, int R, int n_tiles,
-                            const float* bonus_uniform, uint32_t* status, cudaStream_t st) {
-    lm_merge_kernel<<<B * R, 256, 0, st>>>(sc.lm_part, n_tiles, m.d.vocab, R, bonus_uniform, rm.slot, sc.row_lse,
-                                           sc.row_cand, sc.row_cand_lp, status);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    node_lp_from_z_kernel<<<(B * R + 127) / 128, 128, 0, st>>>(sc.node_z, rm.prow, sc.row_lse, sc.node_lp, B * R);
-    return cudaGetLastError();
-}
-
 // ---------------------------------------------------------------------------------------------------------------
-// accept / select: one warp per sequence
+// accept / select: one warp per sequence.  (L2 loads: in launch_lm_accept other blocks of the same launch wrote these.)
 // ---------------------------------------------------------------------------------------------------------------
 
-__global__ void accept_kernel(RowMeta rm, Scratch sc, AcceptArgs a, mtad_result out) {
-    const int bi = blockIdx.x, lane = threadIdx.x;
+struct AcceptShared {
+    float LP[MTAD_MAX_NODES + 1];
+    int16_t parent[MTAD_MAX_NODES + 1];
+};
+
+__device__ __forceinline__ void accept_seq(const RowMeta& rm, const Scratch& sc, const AcceptArgs& a, const mtad_result& out,
+                                           AcceptShared& sh, int bi, int lane) {
     const int R = a.R, N = R - 1, D = a.max_depth;
-    __shared__ float LP[MTAD_MAX_NODES + 1];
+    float* LP = sh.LP;
     const int nrows = rm.n_rows[bi];
-    const bool bad = (out.status[bi] != 0) || nrows == 0;
+    const bool bad = (__ldcg(out.status + bi) != 0) || nrows == 0;
     const int nn = bad ? 0 : nrows - 1;
     const int t0 = bi * R;
-    // joint log-likelihood along each path: LP[n] = LP[parent(n)] + lp[n] in node order (fp32)
+    // joint log-likelihood along each path: LP[n] = LP[parent(n)] + lp[n] in node order (fp32).  The nodes' own terms and parents
+    // are fetched side by side first: one lane that fetched them as it went took 7 us at 64 nodes.
+    for (int n = lane; n < nn; n += 32) {
+        LP[n] = __ldcg(sc.node_lp + t0 + n + 1);
+        sh.parent[n] = (int16_t)(a.parent ? a.parent[bi * N + n] : n - 1);
+    }
+    __syncwarp();
     if (lane == 0) {
         for (int n = 0; n < nn; ++n) {
-            const int p = a.parent ? a.parent[bi * N + n] : n - 1;
-            LP[n] = (p < 0 ? 0.f : LP[p]) + sc.node_lp[t0 + n + 1];
+            const int p = sh.parent[n];
+            LP[n] = (p < 0 ? 0.f : LP[p]) + LP[n];
         }
     }
     __syncwarp();
@@ -561,12 +504,12 @@ __global__ void accept_kernel(RowMeta rm, Scratch sc, AcceptArgs a, mtad_result 
     for (int o = 16; o > 0; o >>= 1) tie = fminf(tie, __shfl_xor_sync(0xffffffffu, tie, o));
 
     if (out.node_LP) for (int n = lane; n < N; n += 32) out.node_LP[bi * N + n] = n < nn ? LP[n] : 0.f;
-    if (out.node_lp) for (int n = lane; n < N; n += 32) out.node_lp[bi * N + n] = n < nn ? sc.node_lp[t0 + n + 1] : 0.f;
+    if (out.node_lp) for (int n = lane; n < N; n += 32) out.node_lp[bi * N + n] = n < nn ? __ldcg(sc.node_lp + t0 + n + 1) : 0.f;
     for (int r = lane; r < R; r += 32) {
         const bool v = !bad && r < nrows;
-        if (out.row_lse) out.row_lse[bi * R + r] = v ? sc.row_lse[t0 + r] : 0.f;
-        if (out.row_cand) out.row_cand[bi * R + r] = v ? sc.row_cand[t0 + r] : 0;
-        if (out.row_cand_lp) out.row_cand_lp[bi * R + r] = v ? sc.row_cand_lp[t0 + r] : 0.f;
+        if (out.row_lse) out.row_lse[bi * R + r] = v ? __ldcg(sc.row_lse + t0 + r) : 0.f;
+        if (out.row_cand) out.row_cand[bi * R + r] = v ? __ldcg(sc.row_cand + t0 + r) : 0;
+        if (out.row_cand_lp) out.row_cand_lp[bi * R + r] = v ? __ldcg(sc.row_cand_lp + t0 + r) : 0.f;
     }
     if (lane == 0) {
         if (bad) {
@@ -582,93 +525,103 @@ __global__ void accept_kernel(RowMeta rm, Scratch sc, AcceptArgs a, mtad_result 
         for (int i = eta - 1; i >= 0 && cur >= 0; --i) {
             out.path[bi * D + i] = cur;
             out.out_tok[bi * (D + 1) + i] = a.tok[bi * N + cur];
-            out.out_lp[bi * (D + 1) + i] = sc.node_lp[t0 + cur + 1];
-            cur = a.parent ? a.parent[bi * N + cur] : cur - 1;
+            out.out_lp[bi * (D + 1) + i] = __ldcg(sc.node_lp + t0 + cur + 1);
+            cur = sh.parent[cur];
         }
         const int wrow = t0 + bn + 1;
-        out.out_tok[bi * (D + 1) + eta] = sc.row_cand[wrow];
-        out.out_lp[bi * (D + 1) + eta] = sc.row_cand_lp[wrow];
+        out.out_tok[bi * (D + 1) + eta] = __ldcg(sc.row_cand + wrow);
+        out.out_lp[bi * (D + 1) + eta] = __ldcg(sc.row_cand_lp + wrow);
         if (out.margin) { out.margin[bi * 2] = m_acc; out.margin[bi * 2 + 1] = tie; }
     }
 }
 
-cudaError_t launch_accept(const RowMeta& rm, const Scratch& sc, const AcceptArgs& a, const mtad_result& out,
+__global__ void accept_kernel(RowMeta rm, Scratch sc, AcceptArgs a, mtad_result out) {
+    __shared__ AcceptShared sh;
+    pdl_wait();
+    pdl_trigger();
+    accept_seq(rm, sc, a, out, sh, blockIdx.x, threadIdx.x);
+}
+
+cudaError_t launch_accept(const RowMeta& rm, const Scratch& sc, const AcceptArgs& a, const mtad_result& out, bool pdl,
                           cudaStream_t st) {
-    accept_kernel<<<a.B, 32, 0, st>>>(rm, sc, a, out);
-    return cudaGetLastError();
+    return launch_pdl(accept_kernel, dim3(a.B), dim3(32), 0, st, pdl, rm, sc, a, out);
 }
 
-// ---------------------------------------------------------------------------------------------------------------
-// KV commit: node path[i] (slot L + 1 + path[i]) moves to position L + 1 + i.  One block per (layer, K|V, kv head,
-// sequence) reads all rows it moves before writing any (a destination may be a later move's source).
-// ---------------------------------------------------------------------------------------------------------------
-
-__global__ void kv_commit_kernel(__nv_bfloat16* __restrict__ cache, const int32_t* __restrict__ call_seq,
-                                 const int32_t* __restrict__ kv_len, mtad_result res, int D, int max_batch, int Hkv,
-                                 int hd, long long cap) {
-    const int bi = blockIdx.y;
-    if (res.status[bi] != 0) return;
-    const int eta = res.eta[bi];
-    if (eta <= 0) return;
-    const int seq = call_seq[bi];
-    if ((unsigned)seq >= (unsigned)max_batch) return;
-    const int L = kv_len[seq];
-    // every source and destination row inside the cache, or nothing moves (seq_advance_kernel flags the sequence)
-    if (eta > D || L < 0 || (long long)L + 1 + eta > cap) return;
-    for (int r = 0; r < eta; ++r) {
-        const int pn = res.path[bi * D + r];
-        if (pn < 0 || (long long)L + 1 + pn >= cap) return;
-    }
-    const int head = blockIdx.x % Hkv;
-    const int kv = (blockIdx.x / Hkv) & 1;
-    const int layer = blockIdx.x / (2 * Hkv);
-    __nv_bfloat16* base = cache + idx_cache(layer, max_batch, seq, kv, Hkv, head, cap, 0, hd);
-    extern __shared__ __nv_bfloat16 buf[];
-    for (int i = threadIdx.x; i < eta * hd; i += blockDim.x) {
-        const int r = i / hd, j = i % hd;
-        buf[i] = base[(size_t)(L + 1 + res.path[bi * D + r]) * hd + j];
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < eta * hd; i += blockDim.x) {
-        const int r = i / hd, j = i % hd;
-        base[(size_t)(L + 1 + r) * hd + j] = buf[i];
-    }
-}
-
-__global__ void seq_advance_kernel(SeqState s, const int32_t* __restrict__ call_seq, mtad_result res, int D, int B,
-                                   int max_batch, long long cap) {
-    const int bi = blockIdx.x * blockDim.x + threadIdx.x;
-    if (bi >= B || res.status[bi] != 0) return;
-    const int seq = call_seq[bi];
-    const int eta = res.eta[bi];
-    bool ok = (unsigned)seq < (unsigned)max_batch && eta >= 0 && eta <= D;
-    if (ok) {
-        const long long L = s.kv_len[seq];
-        ok = L >= 0 && L + 1 + eta <= cap;
-        for (int r = 0; r < eta && ok; ++r) {
-            const int pn = res.path[bi * D + r];
-            ok = pn >= 0 && L + 1 + pn < cap;
+// A block per row: merge of the LM-head kernel's per-(row, vocab tile) partials, in tile order: log-sum-exp, Gumbel-argmax
+// candidate and its log-probability.  The block of a sequence that finishes last goes on: the log-probability of every
+// node's token under its parent row, then the acceptance.  (As launches of their own these two cost 3 us each, which is most of what
+// follows the forward in a step of a small model.)
+__global__ void __launch_bounds__(256) lm_accept_kernel(const float4* __restrict__ part, int n_tiles, int V,
+                                                        const float* __restrict__ uni, RowMeta rm, Scratch sc, AcceptArgs a,
+                                                        mtad_result out) {
+    const int R = a.R, t = blockIdx.x, bi = t / R;
+    __shared__ float sm[256], ss[256], sv[256];
+    __shared__ int si[256];
+    __shared__ AcceptShared sh;
+    __shared__ bool last;
+    pdl_wait();
+    pdl_trigger();
+    const bool active = rm.slot[t] >= 0;
+    if (active) {
+        float m = -CUDART_INF_F, s = 0.f;
+        Best best{-CUDART_INF_F, 0x7fffffff};
+        for (int j = threadIdx.x; j < n_tiles; j += blockDim.x) {
+            const float4 q = part[idx_lm_part(t, n_tiles, j)];
+            const float mm = fmaxf(m, q.x);
+            s = (m == -CUDART_INF_F ? 0.f : s * expf(m - mm)) + (q.x == -CUDART_INF_F ? 0.f : q.y * expf(q.x - mm));
+            m = mm;
+            best = better(best, Best{q.z, __float_as_int(q.w)});
+        }
+        sm[threadIdx.x] = m; ss[threadIdx.x] = s; sv[threadIdx.x] = best.v; si[threadIdx.x] = best.i;
+        __syncthreads();
+        for (int o = blockDim.x >> 1; o > 0; o >>= 1) {
+            if (threadIdx.x < o) {
+                const float m1 = sm[threadIdx.x], m2 = sm[threadIdx.x + o];
+                const float mm = fmaxf(m1, m2);
+                const float s1 = (m1 == -CUDART_INF_F) ? 0.f : ss[threadIdx.x] * expf(m1 - mm);
+                const float s2 = (m2 == -CUDART_INF_F) ? 0.f : ss[threadIdx.x + o] * expf(m2 - mm);
+                sm[threadIdx.x] = mm; ss[threadIdx.x] = s1 + s2;
+                const Best b = better(Best{sv[threadIdx.x], si[threadIdx.x]},
+                                      Best{sv[threadIdx.x + o], si[threadIdx.x + o]});
+                sv[threadIdx.x] = b.v; si[threadIdx.x] = b.i;
+            }
+            __syncthreads();
         }
     }
-    if (!ok) { atomicOr(&res.status[bi], MTAD_ST_RANGE); return; }
-    s.kv_len[seq] += eta + 1;
-    s.root_tok[seq] = res.out_tok[bi * (D + 1) + eta];
+    if (threadIdx.x == 0) {
+        if (active) {
+            const float lse = sm[0] + logf(ss[0]);
+            // a row of NaN logits wins no comparison and leaves no candidate: flag it instead of indexing with it
+            const bool none = (unsigned)si[0] >= (unsigned)V;
+            if (none || !isfinite(lse)) atomicOr(&out.status[bi], MTAD_ST_NONFINITE);
+            const int c = none ? 0 : si[0];
+            sc.row_lse[t] = lse;
+            sc.row_cand[t] = c;
+            // the partial keeps logit + noise; take the noise off again to get the candidate's logit
+            const float g = -logf(-logf(uni[(size_t)bi * V + c]));
+            sc.row_cand_lp[t] = (sv[0] - g) - lse;
+        } else {
+            sc.row_lse[t] = 0.f; sc.row_cand[t] = 0; sc.row_cand_lp[t] = 0.f;
+        }
+        __threadfence();
+        last = atomicAdd(sc.arrive + bi, 1) == R - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+    for (int r = threadIdx.x; r < R; r += blockDim.x) {
+        const int row = bi * R + r, pr = rm.prow[row];
+        sc.node_lp[row] = pr >= 0 ? sc.node_z[row] - __ldcg(sc.row_lse + pr) : 0.f;
+    }
+    if (threadIdx.x == 0) sc.arrive[bi] = 0;
+    __syncthreads();
+    if (threadIdx.x < 32) accept_seq(rm, sc, a, out, sh, bi, threadIdx.x);
 }
 
-cudaError_t launch_kv_commit(const ModelView& m, const SeqState& s, int B, const int32_t* call_seq_dev,
-                             const mtad_result& res, int max_depth, cudaStream_t st) {
-    dim3 grid(m.d.layers * 2 * m.d.n_kv_heads, B);
-    const size_t smem = (size_t)(max_depth > 0 ? max_depth : 1) * m.d.head_dim * sizeof(__nv_bfloat16);
-    kv_commit_kernel<<<grid, 128, smem, st>>>(static_cast<__nv_bfloat16*>(m.d.kv_cache), call_seq_dev, s.kv_len, res,
-                                              max_depth, m.max_batch, m.d.n_kv_heads, m.d.head_dim,
-                                              (long long)m.d.kv_capacity);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_seq_advance(const SeqState& s, int B, const int32_t* call_seq_dev, const mtad_result& res,
-                               int max_depth, int max_batch, long long cap, cudaStream_t st) {
-    seq_advance_kernel<<<1, 64, 0, st>>>(s, call_seq_dev, res, max_depth, B, max_batch, cap);
-    return cudaGetLastError();
+cudaError_t launch_lm_accept(const ModelView& m, const RowMeta& rm, const Scratch& sc, int n_tiles, const float* bonus_uniform,
+                             const AcceptArgs& a, const mtad_result& out, bool pdl, cudaStream_t st) {
+    return launch_pdl(lm_accept_kernel, dim3(a.B * a.R), dim3(256), 0, st, pdl, (const float4*)sc.lm_part, n_tiles, m.d.vocab,
+                      bonus_uniform, rm, sc, a, out);
 }
 
 }  // namespace mtad
