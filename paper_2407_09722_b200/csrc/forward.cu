@@ -544,7 +544,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
     const int yb = S * hr, ys = nbox * yb + 4;             // columns of Y that a box takes, row stride of Y
     const int nf = KIND == FW_LM ? nbox * f.h : f.h;       // features (pairs) of a tile
     const int nv = nf / V;                                 // items of a row
-    const int per = terms == 3 ? 5 : 16, blk = FEW ? 8 : f.blk;      // rows of a drain load, rows that Y holds at a time
+    const int per = terms == 3 ? 5 : (!FEW && KIND == FW_GATEUP && f.S == 1 ? 8 : 16), blk = FEW ? 8 : f.blk;      // rows of a drain load, rows that Y holds at a time
     // a lane's slice of the S k-blocks that the MMA takes side by side is tl / hr; a warp's lanes may lie in several
     const int tl = quad * 32 + lane, my = tl / hr;
     const int s0 = S > 1 ? quad * 32 / hr : 0, s1 = S > 1 ? min(S - 1, (quad * 32 + 31) / hr) : 0;
@@ -645,6 +645,46 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                 for (int j = 0; j < 16; ++j) v[j] += o[j];
             }
         };
+        if constexpr (!FEW && KIND == FW_GATEUP)
+            if (f.S == 1) {
+                // A thread has a feature's gate and up sums of every row in its tensor-memory lane: no way through shared memory, the
+                // two warps of a quadrant take the rows in turn, eight at a time (terms three: five).
+                const int n = f0 + tl;
+                const bool in = tl < f.h && n < a.F;
+                if (quad * 32 < f.h)
+                    for (int rb = half * per; rb < T; rb += 2 * per) {
+                        float v[2][16];
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            acc_ld16(t_acc + q * cols + rb * terms, acc_stride, na, v[q]);
+                            if (terms == 3) {
+#pragma unroll
+                                for (int j = 0; j < 5; ++j) v[q][j] = v[q][3 * j] + (v[q][3 * j + 1] + v[q][3 * j + 2]);
+                            } else {
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) v[q][j] = v[q][2 * j] + v[q][2 * j + 1];
+                            }
+                            if (f.segs > 1) {
+                                float o[8];
+                                tc_ld8(tmem_lane + f.stash + q * up16(T) + rb, o);
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) v[q][j] += o[j];
+                            }
+                        }
+                        __nv_bfloat16* o = a.x_f + (size_t)rb * terms * a.F + n;
+#pragma unroll
+                        for (int j = 0; j < 8; ++j, o += (size_t)terms * a.F) {
+                            if (j >= per || rb + j >= T) break;
+                            const float rs = s.rstd[rb + j], gx = v[0][j] * rs;
+                            if (in) store_terms(gx / (1.f + expf(-gx)) * (v[1][j] * rs), o, a.F, terms);
+                        }
+                        __syncwarp();
+                    }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&s.tempty[buf]));
+                continue;
+            }
         for (int r0 = 0; r0 < T; r0 += blk) {
             const int r1 = min(T, r0 + blk), nr = r1 - r0;
             // ---- accumulators -> Y[row][box][lane], the terms of a row added up
@@ -949,53 +989,70 @@ __device__ __forceinline__ int lane_sums(float* v, int lane) {
     return have > 0 ? idx : N;
 }
 
-// Merge of rows [ra, rn) of a (sequence, KV head, query block)'s pieces by the epilogue threads: four output elements a
-// thread, the pieces in order (deterministic) and six at a time, so that their loads are in flight together.
-template <int HD, int NQP>
-__device__ __forceinline__ void merge_pieces(const FwArgs& a, const FwTail& s, const AttnPos& q, int n_piece, int G, int e, int kp) {
+// Merge of rows [ra, rn) of a (sequence, KV head, query block)'s pieces by the epilogue threads: four output elements of NI rows
+// a thread, the pieces in order (deterministic) and NP at a time, so that their loads are in flight together.
+template <int HD, int NQP, int NP, int NI>
+__device__ __forceinline__ void merge_rows(const FwArgs& a, const FwTail& s, const AttnPos& q, int n_piece, int G, int e, int kp) {
     const int nqb = NQP > FW_QROWS ? a.nqb : 1, g = q.g / nqb, r0 = (q.g - g * nqb) * a.qrows;
     const int nrows = s.meta[q.bi].nrows, n_q = max(0, min(G * nrows - r0, a.qrows));
     const int ra = kp < 0 ? 0 : n_q * kp / n_piece, rn = kp < 0 ? n_q : n_q * (kp + 1) / n_piece;
-    for (int i = ra * (HD / 4) + e; i < rn * (HD / 4); i += FW_EPI) {
-        const int r = r0 + i / (HD / 4), c4 = i % (HD / 4);
-        const int hq = G == 1 ? 0 : r / nrows, t = q.bi * a.R + r - hq * nrows, h = g * G + hq;
-        const size_t o = ((size_t)(q.bi * a.Hkv + g) * G * a.R + r) * a.pieces;
+    constexpr int DR = FW_EPI / (HD / 4);              // rows that the group takes at a time
+    const int c4 = e % (HD / 4);
+    for (int rr = ra + e / (HD / 4); rr < rn; rr += DR * NI) {
+        const size_t o = ((size_t)(q.bi * a.Hkv + g) * G * a.R + r0) * a.pieces;
         const float2* ml = reinterpret_cast<const float2*>(a.part + (size_t)a.T * a.Hq * a.pieces * HD) + o;
         const float4* po = reinterpret_cast<const float4*>(a.part + o * HD) + c4;
-        constexpr int NP = 6;
-        float M = -CUDART_INF_F, ls = 0.f;
-        float4 o4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        float M[NI], ls[NI];
+        float4 o4[NI];
+#pragma unroll
+        for (int x = 0; x < NI; ++x) { M[x] = -CUDART_INF_F; ls[x] = 0.f; o4[x] = make_float4(0.f, 0.f, 0.f, 0.f); }
         for (int k0 = 0; k0 < n_piece; k0 += NP) {
-            float2 v[NP];
-            float4 y[NP];
+            float2 v[NI][NP];
+            float4 y[NI][NP];
 #pragma unroll
-            for (int k = 0; k < NP; ++k) {
-                const int kk = min(k0 + k, n_piece - 1);
-                v[k] = __ldcg(ml + kk);
-                y[k] = __ldcg(po + (size_t)kk * (HD / 4));
-                if (k0 + k >= n_piece) v[k].x = -CUDART_INF_F;
-            }
-            float mn = M;
+            for (int x = 0; x < NI; ++x)
 #pragma unroll
-            for (int k = 0; k < NP; ++k) mn = fmaxf(mn, v[k].x);
-            const float mz = mn == -CUDART_INF_F ? 0.f : mn;
-            const float fo = exp2f(M - mz);
-            ls *= fo;
-            o4.x *= fo; o4.y *= fo; o4.z *= fo; o4.w *= fo;
-            M = mn;
+                for (int k = 0; k < NP; ++k) {
+                    const int i = min(rr + DR * x, rn - 1) * a.pieces + min(k0 + k, n_piece - 1);
+                    v[x][k] = __ldcg(ml + i);
+                    y[x][k] = __ldcg(po + (size_t)i * (HD / 4));
+                    if (k0 + k >= n_piece) v[x][k].x = -CUDART_INF_F;
+                }
 #pragma unroll
-            for (int k = 0; k < NP; ++k) {
-                const float wg = exp2f(v[k].x - mz);
-                if (wg != 0.f) {                       // (a piece without a visible key wrote no sum worth multiplying)
-                    ls += wg * v[k].y;
-                    o4.x += wg * y[k].x; o4.y += wg * y[k].y; o4.z += wg * y[k].z; o4.w += wg * y[k].w;
+            for (int x = 0; x < NI; ++x) {
+                float mn = M[x];
+#pragma unroll
+                for (int k = 0; k < NP; ++k) mn = fmaxf(mn, v[x][k].x);
+                const float mz = mn == -CUDART_INF_F ? 0.f : mn;
+                const float fo = exp2f(M[x] - mz);
+                ls[x] *= fo;
+                o4[x].x *= fo; o4[x].y *= fo; o4[x].z *= fo; o4[x].w *= fo;
+                M[x] = mn;
+#pragma unroll
+                for (int k = 0; k < NP; ++k) {
+                    const float wg = exp2f(v[x][k].x - mz);
+                    if (wg != 0.f) {                   // (a piece without a visible key wrote no sum worth multiplying)
+                        ls[x] += wg * v[x][k].y;
+                        o4[x].x += wg * y[x][k].x; o4[x].y += wg * y[x][k].y; o4[x].z += wg * y[x][k].z; o4[x].w += wg * y[x][k].w;
+                    }
                 }
             }
         }
-        const float f = 1.f / ls;
-        store_terms4(make_float4(o4.x * f, o4.y * f, o4.z * f, o4.w * f),
-                     a.x_a + (size_t)t * a.terms * a.Hq * HD + (size_t)h * HD + c4 * 4, (size_t)a.Hq * HD, a.terms);
+#pragma unroll
+        for (int x = 0; x < NI; ++x) {
+            if (rr + DR * x >= rn) continue;
+            const int r = r0 + rr + DR * x, hq = G == 1 ? 0 : r / nrows, t = q.bi * a.R + r - hq * nrows, h = g * G + hq;
+            const float f = 1.f / ls[x];
+            store_terms4(make_float4(o4[x].x * f, o4[x].y * f, o4[x].z * f, o4[x].w * f),
+                         a.x_a + (size_t)t * a.terms * a.Hq * HD + (size_t)h * HD + c4 * 4, (size_t)a.Hq * HD, a.terms);
+        }
     }
+}
+// Wide items have many rows in few pieces: a thread's rows are fetched side by side.
+template <int HD, int NQP>
+__device__ __forceinline__ void merge_pieces(const FwArgs& a, const FwTail& s, const AttnPos& q, int n_piece, int G, int e, int kp) {
+    if (NQP > FW_QROWS && n_piece <= 2) merge_rows<HD, NQP, 2, 3>(a, s, q, n_piece, G, e, kp);
+    else merge_rows<HD, NQP, 6, 1>(a, s, q, n_piece, G, e, kp);
 }
 
 template <int HD, int NQP, bool FEW, int NS>
