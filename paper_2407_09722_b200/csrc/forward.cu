@@ -156,19 +156,6 @@ __device__ __forceinline__ void acc_ld16(uint32_t at, int stride, int na, float*
     }
 }
 
-// 16 rows of two terms, or five of three, of a box's accumulators, the terms of a row added up (v: room for 32)
-__device__ __forceinline__ void acc_rows(uint32_t at, int stride, int na, int terms, float* v) {
-    acc_ld16(at, stride, na, v);
-    if (terms == 3) {
-#pragma unroll
-        for (int j = 0; j < 5; ++j) v[j] = v[3 * j] + (v[3 * j + 1] + v[3 * j + 2]);
-    } else {
-        acc_ld16(at + 16, stride, na, v + 16);
-#pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = v[2 * j] + v[2 * j + 1];
-    }
-}
-
 // What a call's sequence looks like to the attention
 struct SeqMeta {
     int nrows, L, nkeys, seq;
@@ -321,7 +308,7 @@ __device__ __forceinline__ bool split_residual(const FwArgs& a, FwTail& s, const
     const int lane = e & 31, w = e >> 5, quad = w & 3, half = w >> 2;
     const int T = a.T, terms = a.terms, cols = a.cols, S = f.S, hr = f.hr, yb = S * hr, c = f.c;
     const int tl = quad * 32 + lane, my = tl / hr, s0 = quad * 32 / hr, s1 = min(S - 1, (quad * 32 + 31) / hr);
-    const int per = terms == 3 ? 5 : 16, buf = tcount & 1;
+    const int per = terms == 3 ? 5 : 8, buf = tcount & 1;
     const int kp = tile % c, ra = T * kp / c, rn = T * (kp + 1) / c, n = tile / c * hr + 4 * lane;
     const bool in = 4 * lane < hr && n < a.d;
     constexpr int RW = 3;                                  // rows of a warp whose loads are in flight together
@@ -346,13 +333,19 @@ __device__ __forceinline__ bool split_residual(const FwArgs& a, FwTail& s, const
     float* mine = a.kpart + (size_t)tile * T * yb + tl;
     for (int rb = half * per; rb < T; rb += 2 * per)
         for (int sl = s0; sl <= s1; ++sl) {
-            float v[32];
-            acc_rows(t_acc + sl * cols + rb * terms, S * cols, f.na, terms, v);
+            float v[16];
+            acc_ld16(t_acc + sl * cols + rb * terms, S * cols, f.na, v);
             if (my == sl && tl < yb) {
                 float* y = mine + (size_t)rb * yb;
+                if (terms == 3) {
 #pragma unroll
-                for (int j = 0; j < 16; ++j, y += yb)
-                    if (j < per && rb + j < T) __stcg(y, v[j]);
+                    for (int j = 0; j < 5; ++j, y += yb)
+                        if (rb + j < T) __stcg(y, v[3 * j] + (v[3 * j + 1] + v[3 * j + 2]));
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j, y += yb)
+                        if (rb + j < T) __stcg(y, v[2 * j] + v[2 * j + 1]);
+                }
             }
             __syncwarp();
         }
@@ -374,26 +367,18 @@ __device__ __forceinline__ bool split_residual(const FwArgs& a, FwTail& s, const
 #pragma unroll
         for (int x = 0; x < RW; ++x) q[x] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (in) {
-            // (four parts at a time, their loads in flight together: one after the other they took 0.7 us each)
             const float* p = parts + (size_t)t0 * yb;
             int sl = 0;
-            for (int k0 = 0; k0 < c * S; k0 += 4) {
-                float4 z[4][RW];
+#pragma unroll 4
+            for (int k = 0; k < c * S; ++k) {
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-#pragma unroll
-                    for (int x = 0; x < RW; ++x)
-                        z[k][x] = k0 + k < c * S && t0 + 8 * x < rn ? __ldcg(reinterpret_cast<const float4*>(p + (size_t)(8 * x) * yb))
-                                                                   : make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (++sl == S) { sl = 0; p += (size_t)T * yb - (S - 1) * hr; }
-                    else p += hr;
+                for (int x = 0; x < RW; ++x) {
+                    if (t0 + 8 * x >= rn) continue;
+                    const float4 z = __ldcg(reinterpret_cast<const float4*>(p + (size_t)(8 * x) * yb));
+                    q[x].x += z.x; q[x].y += z.y; q[x].z += z.z; q[x].w += z.w;
                 }
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-#pragma unroll
-                    for (int x = 0; x < RW; ++x) {
-                        q[x].x += z[k][x].x; q[x].y += z[k][x].y; q[x].z += z[k][x].z; q[x].w += z[k][x].w;
-                    }
+                if (++sl == S) { sl = 0; p += (size_t)T * yb - (S - 1) * hr; }
+                else p += hr;
             }
         }
 #pragma unroll
@@ -423,7 +408,7 @@ __device__ __forceinline__ bool split_qkv(const FwArgs& a, FwTail& s, const FwPh
     volatile int* abort_flag = s.abort_flag;
     constexpr int hp = HD / 2;
     const int lane = e & 31, w = e >> 5, quad = w & 3, half = w >> 2;
-    const int T = a.T, terms = a.terms, cols = a.cols, c = f.c, buf = tcount & 1, per = terms == 3 ? 5 : 16;
+    const int T = a.T, terms = a.terms, cols = a.cols, c = f.c, buf = tcount & 1, per = terms == 3 ? 5 : 8;
     const int kp = tile % c, ra = T * kp / c, rn = T * (kp + 1) / c;
     bool ok = true;
     if (e == 0) ok = mbar_wait(smem_u32(&s.tfull[buf]), (uint32_t)(tcount >> 1) & 1u, abort_flag);
@@ -433,12 +418,17 @@ __device__ __forceinline__ bool split_qkv(const FwArgs& a, FwTail& s, const FwPh
     const uint32_t t_acc = tmem_lane + (f.both ? 0 : buf * 256) + half * cols;     // the two warps of a quadrant: a head each
     float* y = a.kpart + (size_t)tile * T * 256 + half * 128 + quad * 32 + lane;
     for (int rb = 0; rb < T; rb += per) {
-        float v[32];
-        acc_rows(t_acc + rb * terms, 2 * cols, f.na, terms, v);
+        float v[16];
+        acc_ld16(t_acc + rb * terms, 2 * cols, f.na, v);
+        if (terms == 3) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j)
-            if (j < per && rb + j < T) __stcg(y + j * 256, v[j]);
-        y += per * 256;
+            for (int j = 0; j < 5; ++j, y += 256)
+                if (rb + j < T) __stcg(y, v[3 * j] + (v[3 * j + 1] + v[3 * j + 2]));
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j, y += 256)
+                if (rb + j < T) __stcg(y, v[2 * j] + v[2 * j + 1]);
+        }
         __syncwarp();
     }
     tc_fence_before();
@@ -456,6 +446,7 @@ __device__ __forceinline__ bool split_qkv(const FwArgs& a, FwTail& s, const FwPh
     const bool rot = hg < a.Hq + a.Hkv;
     const float scale = rsqrtf((float)HD) * 1.4426950408889634f;
     const float* parts = a.kpart + (size_t)(tile / c * c) * T * 256 + box * 128 + j;
+#pragma unroll 2
     for (int t = ra + w; t < rn; t += 8) {
         const int sl = s.slot[t];
         if (j >= hp || hg >= heads || sl < 0) continue;
@@ -463,17 +454,12 @@ __device__ __forceinline__ bool split_qkv(const FwArgs& a, FwTail& s, const FwPh
         const float* rp = a.rope + ((size_t)t * hp + j) * 2;
         *reinterpret_cast<float4*>(cs) = *reinterpret_cast<const float4*>(rp);
         *reinterpret_cast<float4*>(cs + 4) = *reinterpret_cast<const float4*>(rp + 4);
-        float4 px[4], pz[4];                               // (at most four parts: their loads in flight together)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
+#pragma unroll 4
+        for (int k = 0; k < c; ++k) {
             const float* p = parts + ((size_t)k * T + t) * 256;
-            px[k] = k < c ? __ldcg(reinterpret_cast<const float4*>(p)) : make_float4(0.f, 0.f, 0.f, 0.f);
-            pz[k] = k < c ? __ldcg(reinterpret_cast<const float4*>(p + hp)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            va[0] += px[k].x; va[1] += px[k].y; va[2] += px[k].z; va[3] += px[k].w;
-            vb[0] += pz[k].x; vb[1] += pz[k].y; vb[2] += pz[k].z; vb[3] += pz[k].w;
+            const float4 x = __ldcg(reinterpret_cast<const float4*>(p)), z = __ldcg(reinterpret_cast<const float4*>(p + hp));
+            va[0] += x.x; va[1] += x.y; va[2] += x.z; va[3] += x.w;
+            vb[0] += z.x; vb[1] += z.y; vb[2] += z.z; vb[3] += z.w;
         }
         const float rs = s.rstd[t];
 #pragma unroll
@@ -574,38 +560,13 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
         const float* sq = KIND == FW_GATEUP ? a.sumsq_b : a.sumsq_a;
         const FwPhase& from = a.ph[KIND == FW_GATEUP ? FW_O : FW_DOWN];
         const int parts = KIND != FW_GATEUP && p == 0 ? a.parts0 : (FEW ? from.n_tiles : from.n_tiles / from.c);
-        if (FEW) {
-            for (int r = w; r < T; r += 8) {
-                float v = 0.f;
+        for (int r = w; r < T; r += 8) {
+            float v = 0.f;
 #pragma unroll 5
-                for (int q = lane; q < parts; q += 32) v += __ldcg(sq + (size_t)q * TC_X_ROWS + r);
+            for (int q = lane; q < parts; q += 32) v += __ldcg(sq + (size_t)q * TC_X_ROWS + r);
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                if (lane == 0) s.rstd[r] = rsqrtf(v * a.inv_dim + a.eps);
-            }
-        } else {
-            // A lane per row and every eighth part a warp, so that a load is whole lines and the parts' loads are in flight together.
-            // (A warp per row, a lane per part, took 1 us a row: with 32 rows of a small model this ended 3 us after the
-            // accumulators, twice a layer.)
-            constexpr int NX = (FW_MAX_ROWS + 31) / 32;
-            float v[NX];
-#pragma unroll
-            for (int x = 0; x < NX; ++x) v[x] = 0.f;
-#pragma unroll 6
-            for (int q = w; q < parts; q += 8)
-#pragma unroll
-                for (int x = 0; x < NX; ++x)
-                    if (lane + 32 * x < T) v[x] += __ldcg(sq + (size_t)q * TC_X_ROWS + lane + 32 * x);
-#pragma unroll
-            for (int x = 0; x < NX; ++x)
-                if (lane + 32 * x < T) Y[w * (32 * NX) + lane + 32 * x] = v[x];
-            bar_n(1, FW_EPI);
-            if (e < T) {
-                float t = 0.f;
-#pragma unroll
-                for (int q = 0; q < 8; ++q) t += Y[q * (32 * NX) + e];
-                s.rstd[e] = rsqrtf(t * a.inv_dim + a.eps);
-            }
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0) s.rstd[r] = rsqrtf(v * a.inv_dim + a.eps);
         }
     }
     if (!FEW && (KIND == FW_O || KIND == FW_DOWN)) {
