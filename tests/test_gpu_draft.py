@@ -166,6 +166,37 @@ def test_draft_wide_vocabulary():
     assert skipped <= 1
 
 
+@pytest.mark.parametrize("V,b,keep_all", [
+    (24, 2, True),               # fewer tokens than a warp has lanes
+    (1025, 8, False),            # two chunks, the second one token shorter
+    (1025, 8, True),             # 64 candidates of a chunk
+    (33000, 4, False),           # five tokens a thread
+    (70000, 8, False),           # chunks of more tokens than a thread's list holds
+])
+def test_draft_selection_edges(V, b, keep_all):
+    """The selection's chunks, lists and merges at their edges, and the rows that it makes for the next step (two sequences)."""
+    gamma, N = 2, 2 * (b * b if keep_all else b)
+    gm = GpuModel(S.ModelShape(1, 128, 2, 2, 64, 344, V), max_batch=2, max_nodes=max(16, N), capacity=192,
+                  aux=S.ModelShape(1, 128, 2, 2, 64, 512, V), aux_capacity=192)
+    lens, roots, skipped = [20, 33], [7, 11], 0
+    for q in range(2):
+        gm.inject(q, lens[q])
+        gm.inject_aux(q, lens[q])
+        gm.ctx.mtad_seq_set(q, lens[q], roots[q], aux_len=lens[q])
+    caches = [gm.aux_cache_bits(q, lens[q]) for q in range(2)]
+    u = S.uniforms(0, (34 << 40) | V, 2 * gamma * b * V, "cuda").view(2, gamma, b, V)
+    g = _draft_gpu_batch(gm, [0, 1], gamma, b, u, keep_all)
+    for q in range(2):
+        dr = O.draft_beam(gm.oracle_aux(), caches[q], lens[q], [roots[q]], gamma, b, u[q].cpu().numpy(), keep_all=keep_all)
+        if dr.min_gap < draft_gap(keep_all):
+            skipped += 1
+            continue
+        assert g["tok"][q].tolist() == dr.tok and g["parent"][q].tolist() == dr.parent
+        assert g["depth"][q].tolist() == dr.depth and g["best_path"][q].tolist() == dr.best_path
+        assert np.max(np.abs(g["node_logq"][q].cpu().numpy() - np.asarray(dr.logq))) < 2e-5
+    assert skipped <= 1 and gm.ctx.mtad_debug_check_canaries() == ""
+
+
 def test_draft_rejects_bad_arguments():
     gm = GpuModel(W.target, max_batch=1, max_nodes=40, capacity=128, aux=W.aux, aux_capacity=128)
     V = W.target.vocab
