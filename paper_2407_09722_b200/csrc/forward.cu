@@ -301,8 +301,7 @@ static_assert(FW_RING + FW_UNION + sizeof(FwTail) <= 227 * 1024, "shared memory 
 // O or down where c blocks share the k-range of a tile: each leaves its accumulators in global memory as they lie in tensor
 // memory (a row's features, the S slices side by side), the blocks wait for one another, and each finishes a share of the
 // rows, a warp per row, adding the parts in order (deterministic).
-template <int KIND>
-__device__ __forceinline__ bool split_residual(const FwArgs& a, FwTail& s, const FwPhase& f, int layer, int tcount, int e,
+__device__ __forceinline__ bool split_residual(const FwArgs& a, FwTail& s, const FwPhase& f, bool is_o, int layer, int tcount, int e,
                                                uint32_t tmem_lane, int tile) {
     volatile int* abort_flag = s.abort_flag;
     const int lane = e & 31, w = e >> 5, quad = w & 3, half = w >> 2;
@@ -321,7 +320,7 @@ __device__ __forceinline__ bool split_residual(const FwArgs& a, FwTail& s, const
     };
     load_hid(ra + w);
     float g[4];
-    const __nv_bfloat16* gain = KIND == FW_O ? a.layers[layer].gain_ffn : a.layers[layer].gain_next;
+    const __nv_bfloat16* gain = is_o ? a.layers[layer].gain_ffn : a.layers[layer].gain_next;
 #pragma unroll
     for (int x = 0; x < 4; ++x) g[x] = in ? __bfloat162float(gain[n + x]) : 0.f;
     bool ok = true;
@@ -354,7 +353,7 @@ __device__ __forceinline__ bool split_residual(const FwArgs& a, FwTail& s, const
     if (lane == 0) mbar_arrive(smem_u32(&s.tempty[buf]));
     bar_n(1, FW_EPI);
     if (e == 0) {
-        int32_t* cnt = a.kcnt + (KIND == FW_O ? 0 : a.n_cta) + tile / c;
+        int32_t* cnt = a.kcnt + (is_o ? 0 : a.n_cta) + tile / c;
         asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(cnt) : "memory");
         ok = grid_wait(cnt, c * (layer + 1), abort_flag);
     }
@@ -394,7 +393,7 @@ __device__ __forceinline__ bool split_residual(const FwArgs& a, FwTail& s, const
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-            if (lane == 0) (KIND == FW_O ? a.sumsq_b : a.sumsq_a)[(size_t)(tile / c) * TC_X_ROWS + t] = ss;
+            if (lane == 0) (is_o ? a.sumsq_b : a.sumsq_a)[(size_t)(tile / c) * TC_X_ROWS + t] = ss;
         }
     }
     return true;
@@ -533,13 +532,14 @@ __device__ __forceinline__ bool put_by(const FwArgs& a, FwTail& s, const FwPhase
 // instruction); otherwise four neighbouring features per thread.
 template <int KIND, int HD, bool FEW>
 __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, int p, int layer, int& tcount, int e,
-                                          uint32_t tmem_lane, int cta) {
-    const FwPhase& f = a.ph[KIND];
+                                          uint32_t tmem_lane, int cta, int kind) {
+    const FwPhase& f = a.ph[KIND == FW_O ? kind : KIND];               // (O and down are one instance)
+    const bool is_o = kind == FW_O;
     if (cta >= f.n_tiles) return true;
     volatile int* abort_flag = s.abort_flag;
     constexpr int V = FEW ? 1 : 4;                         // features per item
     const int lane = e & 31, w = e >> 5, quad = w & 3, half = w >> 2;
-    const int T = a.T, terms = a.terms, cols = a.cols, n_cta = a.n_cta;
+    const int T = a.T, terms = FEW ? 3 : a.terms, cols = a.cols, n_cta = a.n_cta;
     const int hr = f.hr, S = f.S, nbox = f.nbox, na = f.na, acc_stride = nbox * S * cols;
     const int yb = S * hr, ys = nbox * yb + 4;             // columns of Y that a box takes, row stride of Y
     const int nf = KIND == FW_LM ? nbox * f.h : f.h;       // features (pairs) of a tile
@@ -594,17 +594,16 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
             }
         }
     }
-    if (!FEW && (KIND == FW_O || KIND == FW_DOWN)) {
+    if (!FEW && (KIND == FW_O)) {
         // the residual stream comes from other blocks where O and down are cut differently
         if (e == 0) ok = grid_wait(a.sync + p - 1, n_cta, abort_flag);
         ok = all_of(1, FW_EPI, ok);
         if (!ok) return false;
     }
     const __nv_bfloat16* gain = nullptr;
-    if (KIND == FW_O) gain = a.layers[layer].gain_ffn;
-    if (KIND == FW_DOWN) gain = a.layers[layer].gain_next;
-    if (!FEW && (KIND == FW_O || KIND == FW_DOWN) && f.c > 1) {
-        ok = split_residual<KIND>(a, s, f, layer, tcount, e, tmem_lane, cta);
+    if (KIND == FW_O) gain = is_o ? a.layers[layer].gain_ffn : a.layers[layer].gain_next;
+    if (!FEW && (KIND == FW_O) && f.c > 1) {
+        ok = split_residual(a, s, f, is_o, layer, tcount, e, tmem_lane, cta);
         ++tcount;
         return ok;
     }
@@ -618,7 +617,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
         const int f0 = tile * nf;                          // first feature (O, down, gate / up, LM head)
         // ---- what the first items need besides the accumulator
         const int hg = KIND == FW_QKV ? tile / f.u : 0, j0 = KIND == FW_QKV ? (tile - hg * f.u) * f.h : 0;
-        constexpr int NI = FEW ? 2 : 1;                    // QKV: items per thread and round
+        constexpr int NI = 1;                              // QKV: items per thread and round
         float cs[NI][2 * V];                               // cosines and sines of an item's pairs
         auto rope_load = [&](int t, int j) {
 #pragma unroll
@@ -638,16 +637,22 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
             }
         };
         float hid = 0.f, gain0 = 0.f;                      // O, down with few rows: the residual element of (row w, feature lane)
-        float u8[8];
+        float gum[8];                                      // LM head: the Gumbel noise of the warp's tokens, one draw per sequence
+        int gum_seq = -1;
         auto lm_load = [&](int t) {
+            const int sq = t / a.R;
+            if (t >= T || sq == gum_seq) return;
+            gum_seq = sq;
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const int jl = lane + 32 * i, n = f0 + jl;
-                u8[i] = (t < T && jl < nf && n < a.V) ? a.uniforms[(size_t)(t / a.R) * a.V + n] : 0.5f;
+                gum[i] = (jl < nf && n < a.V) ? a.uniforms[(size_t)sq * a.V + n] : 0.5f;
             }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) gum[i] = logf(-logf(gum[i]));
         };
         if (KIND == FW_QKV) rope_load(it0, ij0);
-        if (FEW && (KIND == FW_O || KIND == FW_DOWN) && lane < nf && f0 + lane < a.d) {
+        if (FEW && (KIND == FW_O) && lane < nf && f0 + lane < a.d) {
             gain0 = __bfloat162float(gain[f0 + lane]);
             if (w < T) hid = __ldcg(a.hidden + (size_t)w * a.d + f0 + lane);
         }
@@ -779,7 +784,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                 const float* y = Y + t * ys + q * yb + row;
                 float v = y[0];
                 if (S == 4) return (v + y[hr]) + (y[2 * hr] + y[3 * hr]);
-#pragma unroll 4
+#pragma unroll 1
                 for (int sl = 1; sl < S; ++sl) v += y[sl * hr];
                 return v;
             };
@@ -851,7 +856,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                 }
             } else if (KIND == FW_GATEUP) {
                 int t = it0, j = ij0;
-#pragma unroll 2
+#pragma unroll(FEW ? 1 : 2)
                 for (int i = e; i < nr * nv; i += FW_EPI) {
                     const int n = f0 + j;
                     if (n < a.F) {
@@ -874,7 +879,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
             } else if (KIND == FW_LM) {
                 if (a.lm_plain) {
                     int t = it0, j = ij0;
-#pragma unroll 2
+#pragma unroll(FEW ? 1 : 2)
                     for (int i = e; i < nr * nv; i += FW_EPI) {
                         const int q = j >= f.h ? 1 : 0, n = f0 + j;
                         float z[V];
@@ -904,7 +909,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                             const bool in = jl < nf && n < a.V;
                             z[i] = in ? yv1(t - r0, q, jl - q * f.h) * rs : -CUDART_INF_F;
                             m = fmaxf(m, z[i]);
-                            const float pz = in ? z[i] - logf(-logf(u8[i])) : -CUDART_INF_F;
+                            const float pz = in ? z[i] - gum[i] : -CUDART_INF_F;
                             if (in && (pz > bv || (pz == bv && n < bi))) { bv = pz; bi = n; }
                         }
 #pragma unroll
@@ -942,7 +947,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                     }
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-                    if (lane == 0) (KIND == FW_O ? a.sumsq_b : a.sumsq_a)[(size_t)tile * TC_X_ROWS + w] = ss;
+                    if (lane == 0) (is_o ? a.sumsq_b : a.sumsq_a)[(size_t)tile * TC_X_ROWS + w] = ss;
                 }
             } else {
                 // residual, four features per item; the items' sums of squares meet in Y (each over its own first element)
@@ -973,7 +978,7 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                     float ss = lane < nv ? Y[tr * ys + lane * V] : 0.f;       // (nv <= 32: at most 128 features)
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-                    if (lane == 0) (KIND == FW_O ? a.sumsq_b : a.sumsq_a)[(size_t)tile * TC_X_ROWS + r0 + tr] = ss;
+                    if (lane == 0) (is_o ? a.sumsq_b : a.sumsq_a)[(size_t)tile * TC_X_ROWS + r0 + tr] = ss;
                 }
             }
             if (r1 < T || tile + n_cta < f.n_tiles) bar_n(1, FW_EPI);       // Y is rewritten by the next rows or tile
@@ -1113,7 +1118,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     const int nqb = WIDE ? a.nqb : 1, heads = a.Hkv * nqb;           // attention: (KV head, query block)s of a sequence
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const int cta = (int)blockIdx.x, n_cta = a.n_cta;
-    const int T = a.T, cols = a.cols, terms = a.terms;
+    const int T = a.T, cols = a.cols, terms = FEW ? 3 : a.terms;
     const int n_phases = 5 * a.n_layers + 1;
     auto slot_ptr = [&](int pos) { return smem_u32(smem) + (uint32_t)(pos % NS) * FW_SLOT; };
     auto full_bar = [&](int pos) { return smem_u32(&s.full[pos % NS]); };
@@ -1568,12 +1573,13 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     ++as;
                 };
                 int L = 0, nkeys = 0;
-                for (int i = 0; i < a_n; ++i) {
-                    const bool fresh = i == 0 || i == a_wrap || it.tile + 1 == it.nt;     // (it: the item before)
+                for (int i = 0; a_n > 0; ++i) {
+                    const bool fresh = i == 0 || i == a_wrap || i == a_n || it.tile + 1 == it.nt;     // (it: the item before)
                     if (fresh && i > 0) {
                         output(at - 1);
                         finish(it);
                     }
+                    if (i == a_n) break;
                     if (i > 0) attn_step(it, i);
                     if (fresh) {
 #pragma unroll
@@ -1702,10 +1708,6 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                     }
                     ++at;
                 }
-                if (a_n > 0) {
-                    output(at - 1);
-                    finish(it);
-                }
                 pos += 2 * a_n + ring_other;
                 ok = all_of(1, FW_EPI, ok);
                 if (!ok) break;
@@ -1735,15 +1737,13 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
                         }
                 }
             } else if (kind == FW_QKV) {
-                ok = epi_phase<FW_QKV, HD, FEW>(a, s, Y, p, layer, tcount, e, t_lane, cta);
-            } else if (kind == FW_O) {
-                ok = epi_phase<FW_O, HD, FEW>(a, s, Y, p, layer, tcount, e, t_lane, cta);
+                ok = epi_phase<FW_QKV, HD, FEW>(a, s, Y, p, layer, tcount, e, t_lane, cta, kind);
+            } else if (kind == FW_O || kind == FW_DOWN) {
+                ok = epi_phase<FW_O, HD, FEW>(a, s, Y, p, layer, tcount, e, t_lane, cta, kind);
             } else if (kind == FW_GATEUP) {
-                ok = epi_phase<FW_GATEUP, HD, FEW>(a, s, Y, p, layer, tcount, e, t_lane, cta);
-            } else if (kind == FW_DOWN) {
-                ok = epi_phase<FW_DOWN, HD, FEW>(a, s, Y, p, layer, tcount, e, t_lane, cta);
+                ok = epi_phase<FW_GATEUP, HD, FEW>(a, s, Y, p, layer, tcount, e, t_lane, cta, kind);
             } else {
-                ok = epi_phase<FW_LM, HD, FEW>(a, s, Y, p, layer, tcount, e, t_lane, cta);
+                ok = epi_phase<FW_LM, HD, FEW>(a, s, Y, p, layer, tcount, e, t_lane, cta, kind);
             }
             if (kind != FW_LM && ok) {
                 // phase barrier: the release covers the whole group's stores (the readers' proxy fence follows their acquire)
