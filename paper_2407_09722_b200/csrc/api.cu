@@ -1246,7 +1246,7 @@ void audit_forward(Audit& au, const mtad_ctx& c, const ModelView& m, int B, int 
                           "row_cand_lp", "node_z"})
         au.ws(n, T);
     au.ws("rm_mask", (size_t)T * MTAD_MASK_WORDS);
-    for (const char* n : {"rm_n_rows", "rm_n_spec", "rm_kv_base", "rm_call_seq"}) au.ws(n, B);
+    for (const char* n : {"rm_n_rows", "rm_n_spec", "rm_kv_base", "rm_call_seq", "act"}) au.ws(n, B);     // (act: Scratch::arrive)
     au.ws("hidden", (size_t)T * d.d_model);
     au.ws("rope", ((size_t)(T - 1) * (hd / 2) + (hd / 2 - 1)) * 2 + 2);
     au.ws("xd", idx_xrow(T - 1, terms, terms - 1, d.d_model, d.d_model - 1) + 1);

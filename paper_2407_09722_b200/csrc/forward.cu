@@ -9,11 +9,14 @@
 // stays busy across the barrier for as long as the ring is deep.  Two more things keep the boundary short: every block
 // owns whole output features (the features are cut into one tile per SM, not into 128-row tiles), so no partial sum leaves
 // an SM while rows are few; and only the call's terms x rows operand rows are multiplied (16 columns for five rows).
-// Measured (chain of launches -> one launch, a whole verification step): 7B, 5 rows 3.55 -> 3.07 ms (weights and K / V in
-// 2.2 ms at copy speed), 33 rows 4.37 -> 3.56, 65 rows 5.90 -> 4.81; 13B, 8 x 7 rows 9.41 -> 8.50; two-layer auxiliary
-// model of width 768, four draft steps 520 -> 439 us.  A phase of a large model costs its bytes plus about 3 us (barrier 1.1,
-// first operand rows 0.8, last MMA to last store 1.2 and up); the phases of the auxiliary model, which move next to nothing,
-// take about 8, and the attention of a chain 10 more than its bytes.
+// Measured (chain of launches -> one launch, a whole verification step): 7B, 5 rows 3.55 -> 2.91 ms (weights and K / V in
+// 2.2 ms at copy speed), 33 rows 4.37 -> 3.57, 65 rows 5.90 -> 4.79; 13B, 8 x 7 rows 9.41 -> 8.80; two-layer auxiliary
+// model of width 768, four draft steps 520 -> 378 us.  A phase of a large model costs its bytes plus about 3 us (barrier 1.1,
+// first operand rows 0.6, last MMA to last store 1.2 and up); the phases of the auxiliary model, which move next to nothing,
+// take about 6, and the attention of a chain 7 more than its bytes.  Much of that is waiting for instructions: what an epilogue
+// executes runs once a phase, and a layer's worth of it does not fit an SM's instruction cache (four layers of 7B, 5 rows: 6.2k
+// misses of 23.8k lookups an SM, 8.1k of 26.6k before the code of few rows was made smaller).  Code here should be short before
+// it is clever: unrolled groups of loads that saved round trips made a step slower.
 //
 // Contraction.  Weights are the 128-row MMA operand A, the operand rows (two or three bf16 terms per activation, see
 // store_terms) operand B.  Where a block owns at most 64 features, the MMA takes S k-blocks at once: their weights lie
