@@ -414,8 +414,13 @@ __device__ __forceinline__ void draft_pick(const float* __restrict__ logits, int
         const int n = step * per_layer + m;
         int k = keep_all ? -1 : m, b = keep_all ? m : -1;  // its rank among the kept beams, its place among the beams' best
         if (keep_all) {
+            // Fewer pairs than beams (scores of NaN): the ranks that no pair took go to the first nodes without one, so that every
+            // beam of the next step has a token and a mask, as in the plain tree.
+            int free = 0;
+            if (!valid)
+                for (int q = 0; q < m; ++q) free += sh.bflat[q] == 0x7fffffff;
             for (int q = 0; q < beam; ++q)
-                if (valid && sh.kflat[q] == f) k = q;
+                if (sh.kflat[q] == f && (valid || free-- == 0)) k = q;
         } else {
             for (int q = 0; q < kpb; ++q)
                 if (sh.bflat[j * kpb + q] == f) b = j * kpb + q;

@@ -197,6 +197,34 @@ def test_draft_selection_edges(V, b, keep_all):
     assert skipped <= 1 and gm.ctx.mtad_debug_check_canaries() == ""
 
 
+@pytest.mark.parametrize("keep_all", [False, True])
+def test_draft_without_candidates(keep_all):
+    """Rows without one finite score (a NaN logit): every beam of every layer still gets a token, a parent and a mask, the same
+    whatever an earlier draft left behind."""
+    gamma, b, L, V = 3, 4, 24, W.target.vocab
+    per_layer = b * b if keep_all else b
+    gm = GpuModel(W.target, max_batch=1, max_nodes=gamma * per_layer, capacity=128, aux=W.aux, aux_capacity=128)
+    gm.inject(0, L)
+    gm.inject_aux(0, L)
+    gm.ctx.mtad_seq_set(0, L, 5, aux_len=L)
+    u = S.uniforms(0, (36 << 40) | 1, gamma * b * V, "cuda").view(1, gamma, b, V)
+    for _ in range(20):                              # (on different SMs)
+        _draft_gpu(gm, 0, gamma, b, u, keep_all)
+    gm.aux_weights["lm_head"][5] = float("nan")
+    g = _draft_gpu(gm, 0, gamma, b, u, keep_all)
+    assert g["tok"].unique().tolist() == [0] and g["best_path"][0].tolist() == [s * per_layer for s in range(gamma)]
+    assert g["parent"].view(gamma, per_layer).tolist() == [[(s - 1) * per_layer if s else -1] * per_layer for s in range(gamma)]
+
+    def region(name, n, dtype=torch.int32):
+        return gm.ctx.region(name, dtype)[:n].tolist()
+
+    assert region("ds_node_tok", gamma * b) == [0] * (gamma * b)
+    assert region("ds_tree_id", gamma * b) == [s * per_layer + k for s in range(gamma) for k in range(b)]
+    # the last step's rows: the pending token, the first beam of the first layer, themselves
+    assert region("rm_tok", b) == [0] * b and region("rm_slot", b) == [L + 1 + b + r for r in range(b)]
+    assert region("rm_mask", b * 8) == [w for r in range(b) for w in [3 | 1 << (1 + b + r)] + [0] * 7]
+
+
 def test_draft_rejects_bad_arguments():
     gm = GpuModel(W.target, max_batch=1, max_nodes=40, capacity=128, aux=W.aux, aux_capacity=128)
     V = W.target.vocab
