@@ -575,24 +575,26 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
         } else {
             // A lane per row and every eighth part a warp, so that a load is whole lines and the parts' loads are in flight together.
             // (A warp per row, a lane per part, took 1 us a row: with 32 rows of a small model this ended 3 us after the
-            // accumulators, twice a layer.)
-            constexpr int NX = (FW_MAX_ROWS + 31) / 32;
-            float v[NX];
+            // accumulators, twice a layer.)  Added in the order of 32 lanes and a butterfly, which is also that of few rows: no chain is
+            // longer than five parts (one sum a warp lost up to 1e-6 of a row's, tests/test_gpu_row_sums.py).
+            constexpr int NX = (FW_MAX_ROWS + 31) / 32, NQ = 20;             // (NQ x 8 parts: those of 148 blocks)
+#pragma unroll 1
+            for (int r = lane; r - lane < T; r += 32) {
+                float v[4] = {0.f, 0.f, 0.f, 0.f};
+                for (int q0 = w; q0 < parts; q0 += 8 * NQ) {
+                    float x[NQ];
 #pragma unroll
-            for (int x = 0; x < NX; ++x) v[x] = 0.f;
-#pragma unroll 6
-            for (int q = w; q < parts; q += 8)
+                    for (int k = 0; k < NQ; ++k) x[k] = q0 + 8 * k < parts && r < T ? __ldcg(sq + (size_t)(q0 + 8 * k) * TC_X_ROWS + r) : 0.f;
 #pragma unroll
-                for (int x = 0; x < NX; ++x)
-                    if (lane + 32 * x < T) v[x] += __ldcg(sq + (size_t)q * TC_X_ROWS + lane + 32 * x);
-#pragma unroll
-            for (int x = 0; x < NX; ++x)
-                if (lane + 32 * x < T) Y[w * (32 * NX) + lane + 32 * x] = v[x];
+                    for (int k = 0; k < NQ; ++k) v[k % 4] += x[k];
+                }
+                Y[w * (32 * NX) + r] = (v[0] + v[2]) + (v[1] + v[3]);
+            }
             bar_n(1, FW_EPI);
             if (e < T) {
-                float t = 0.f;
-#pragma unroll
-                for (int q = 0; q < 8; ++q) t += Y[q * (32 * NX) + e];
+                constexpr int q = 32 * NX;
+                const float* y = Y + e;
+                const float t = ((y[0] + y[4 * q]) + (y[2 * q] + y[6 * q])) + ((y[q] + y[5 * q]) + (y[3 * q] + y[7 * q]));
                 s.rstd[e] = rsqrtf(t * a.inv_dim + a.eps);
             }
         }
