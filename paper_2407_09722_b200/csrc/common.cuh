@@ -223,25 +223,33 @@ __device__ __forceinline__ void store_terms4(float4 v, __nv_bfloat16* x, size_t 
 }
 
 // One embedding row -> the fp32 hidden row and (tensor-core path) its bf16 operand terms times the first norm's gain;
-// returns this thread's (`tid` of `n_thr`) share of the row's sum of squares.  16-byte loads, four in flight per thread: a scalar loop
-// whose loads wait behind the previous iteration's stores pays one DRAM latency per element (32 us for a 4096-wide
-// row).  d is a multiple of 8; rows that are not 16-byte aligned take the scalar loop.
-__device__ __forceinline__ float embed_row(const __nv_bfloat16* __restrict__ src_row, bool ok, int d,
-                                           float* __restrict__ hidden_row, const __nv_bfloat16* __restrict__ gain,
-                                           __nv_bfloat16* x_row, int terms, int tid, int n_thr) {
-    float ss = 0.f;
+// returns this thread's (`tid` of `n_thr`) shares of the row's sum of squares: one, or those that four threads of four times as
+// many would have (a warp alone that keeps one sum a lane adds 128 squares of a 4096-wide row in a chain).  16-byte loads, four
+// in flight per thread: a scalar loop whose loads wait behind the previous iteration's stores pays one DRAM latency per element (32 us for a
+// 4096-wide row).  d is a multiple of 8; rows that are not 16-byte aligned take the scalar loop.
+template <int NS>
+__device__ __forceinline__ void embed_row(const __nv_bfloat16* __restrict__ src_row, bool ok, int d,
+                                          float* __restrict__ hidden_row, const __nv_bfloat16* __restrict__ gain,
+                                          __nv_bfloat16* x_row, int terms, int tid, int n_thr, float (&ss)[NS]) {
+    static_assert(NS == 1 || NS == 4, "shares of a thread");
+#pragma unroll
+    for (int k = 0; k < NS; ++k) ss[k] = 0.f;
     const bool vec = ((reinterpret_cast<uintptr_t>(src_row) | reinterpret_cast<uintptr_t>(hidden_row) |
                        reinterpret_cast<uintptr_t>(gain) | reinterpret_cast<uintptr_t>(x_row)) & 15) == 0;
     if (!vec) {
-        for (int i = tid; i < d; i += n_thr) {
-            const float v = ok ? __bfloat162float(src_row[i]) : 0.f;
-            hidden_row[i] = v;
-            if (x_row) {
-                store_terms(v * __bfloat162float(gain[i]), x_row + i, d, terms);
-                ss += v * v;
+        for (int i0 = tid; i0 < d; i0 += NS * n_thr)
+#pragma unroll
+            for (int k = 0; k < NS; ++k) {
+                const int i = i0 + k * n_thr;
+                if (i >= d) break;
+                const float v = ok ? __bfloat162float(src_row[i]) : 0.f;
+                hidden_row[i] = v;
+                if (x_row) {
+                    store_terms(v * __bfloat162float(gain[i]), x_row + i, d, terms);
+                    ss[k] += v * v;
+                }
             }
-        }
-        return ss;
+        return;
     }
     const int nv = d >> 3;
     const uint4* src = reinterpret_cast<const uint4*>(src_row);
@@ -274,12 +282,11 @@ __device__ __forceinline__ float embed_row(const __nv_bfloat16* __restrict__ src
                     store_terms(v[2 * e] * __uint_as_float(gw[e] << 16), x_row + (size_t)c * 8 + 2 * e, d, terms);
                     store_terms(v[2 * e + 1] * __uint_as_float(gw[e] & 0xffff0000u), x_row + (size_t)c * 8 + 2 * e + 1, d,
                                 terms);
-                    ss += v[2 * e] * v[2 * e] + v[2 * e + 1] * v[2 * e + 1];
+                    ss[k % NS] += v[2 * e] * v[2 * e] + v[2 * e + 1] * v[2 * e + 1];
                 }
             }
         }
     }
-    return ss;
 }
 
 // Rotary frequencies base^(-2i/hd), i < hd/2, computed once on the host in double and passed to the kernels that

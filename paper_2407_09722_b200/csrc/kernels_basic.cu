@@ -139,11 +139,12 @@ __global__ void prepare_kernel(const __nv_bfloat16* __restrict__ embed, int d, i
     __syncthreads();
     const int tok = sh_tok;
     const bool ok = sh_ok;
-    float ss = embed_row(embed + (size_t)tok * d, ok, d, hidden + (size_t)t * d, a.gain0,
-                         a.x ? a.x + (size_t)t * a.terms * d : nullptr, a.terms, threadIdx.x, blockDim.x);
+    float share[1];
+    embed_row(embed + (size_t)tok * d, ok, d, hidden + (size_t)t * d, a.gain0, a.x ? a.x + (size_t)t * a.terms * d : nullptr, a.terms,
+              threadIdx.x, blockDim.x, share);
     if (a.x) {
         __shared__ float red[32];
-        ss = block_sum(ss, red);                     // (also orders the hidden row's stores before the loop below)
+        const float ss = block_sum(share[0], red);                     // (also orders the hidden row's stores before the loop below)
         if (threadIdx.x == 0) a.sumsq_out[t] = ss;
         if (a.x2)
             for (int i = threadIdx.x; i < d; i += blockDim.x)

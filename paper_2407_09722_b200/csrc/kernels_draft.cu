@@ -167,11 +167,12 @@ __global__ void draft_prepare_kernel(DraftRows a, DraftState ds, SeqList seqs, i
             cache[idx_cache(layer, max_batch, seq, kv, Hkv, head, a.cap, row.hole, hd) + j] = __float2bfloat16_rn(0.f);
         }
     }
-    float ss = embed_row(a.embed + (size_t)row.tok * d, row.ok, d, a.hidden + (size_t)t * d, a.gain0,
-                         a.x ? a.x + (size_t)t * a.terms * d : nullptr, a.terms, threadIdx.x, blockDim.x);
+    float share[1];
+    embed_row(a.embed + (size_t)row.tok * d, row.ok, d, a.hidden + (size_t)t * d, a.gain0, a.x ? a.x + (size_t)t * a.terms * d : nullptr,
+              a.terms, threadIdx.x, blockDim.x, share);
     if (a.x) {
         __shared__ float red[32];
-        ss = wsum(ss);
+        const float ss = wsum(share[0]);
         if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -513,8 +514,11 @@ __global__ void __launch_bounds__(256) draft_select_kernel(const float* __restri
                                   npend + step * beam + warp, true, -1, sh.pick.kmask[warp], beam);
         __syncwarp();
         const int t = bi * beam + warp;
-        const float ss = wsum(embed_row(rows.embed + (size_t)row[warp].tok * d, row[warp].ok, d, rows.hidden + (size_t)t * d, rows.gain0,
-                                        rows.x ? rows.x + (size_t)t * rows.terms * d : nullptr, rows.terms, lane, 32));
+        float share[4], ss = 0.f;
+        embed_row(rows.embed + (size_t)row[warp].tok * d, row[warp].ok, d, rows.hidden + (size_t)t * d, rows.gain0,
+                  rows.x ? rows.x + (size_t)t * rows.terms * d : nullptr, rows.terms, lane, 32, share);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) ss += wsum(share[k]);
         if (rows.x && lane == 0) rows.sumsq[t] = ss;
     }
     __syncthreads();
