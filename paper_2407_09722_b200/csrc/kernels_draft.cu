@@ -761,13 +761,13 @@ struct CommitCache {
 };
 
 // Node path[i] (cache slot L + 1 + path[i], of the auxiliary model base + beam slot) moves to position L + 1 + i (base + i).  Blocks
-// 0 .. nt - 1 of a sequence share out the target's (layer, K|V, KV head)s, the others the auxiliary model's; all rows of one are
-// read before any is written (a destination may be a later move's source).  Rows that stay where they are (an accepted
-// chain) are left alone.
+// 0 .. nt - 1 of a sequence share out the target's rows, the others the auxiliary model's, in columns of 16 bytes (what every attention
+// kernel reads at a time) of a (layer, K|V, KV head): a thread reads its column of all rows before it writes any (a destination may
+// be a later move's source), so the loads of the rows are in flight together and no thread waits for another.  Rows that stay
+// where they are (an accepted chain) are left alone.
 __global__ void __launch_bounds__(128) commit_kernel(CommitCache tg, CommitCache ax, SeqState s, DraftState ds,
                                                      const int32_t* __restrict__ call_seq, mtad_result res, int D, int mode,
                                                      int max_batch, int nt) {
-    extern __shared__ __nv_bfloat16 buf[];
     __shared__ int src[MTAD_MAX_DEPTH];
     __shared__ int n_rows, dst, moved, stop;
     const int bi = blockIdx.y, tid = threadIdx.x;
@@ -793,8 +793,9 @@ __global__ void __launch_bounds__(128) commit_kernel(CommitCache tg, CommitCache
         moved = stop = 0;
     }
     __syncthreads();
-    if (n_rows == 0) return;
-    if (tid < n_rows) {
+    const int n = n_rows;
+    if (n == 0) return;
+    if (tid < n) {
         const int from = target ? res.path[bi * D + tid] : aux_slot_of(ds, res, bi, seq, D, mode, tid);
         src[tid] = from;
         if (from != tid) moved = 1;
@@ -803,14 +804,24 @@ __global__ void __launch_bounds__(128) commit_kernel(CommitCache tg, CommitCache
     __syncthreads();
     if (stop || !moved) return;
     const CommitCache& c = target ? tg : ax;
-    const int n = n_rows * c.hd, blocks = target ? nt : (int)gridDim.x - nt;
-    for (int pl = target ? blockIdx.x : blockIdx.x - nt; pl < c.planes; pl += blocks) {
-        const int head = pl % c.Hkv, kv = (pl / c.Hkv) & 1, layer = pl / (2 * c.Hkv);
-        __nv_bfloat16* b = c.cache + idx_cache(layer, max_batch, seq, kv, c.Hkv, head, c.cap, dst, c.hd);
-        for (int i = tid; i < n; i += blockDim.x) buf[i] = b[(size_t)src[i / c.hd] * c.hd + i % c.hd];
-        __syncthreads();
-        for (int i = tid; i < n; i += blockDim.x) b[i] = buf[i];
-        __syncthreads();
+    const int cols = c.hd / 8, items = c.planes * cols, step = (target ? nt : (int)gridDim.x - nt) * 128;
+    for (int i = (target ? blockIdx.x : blockIdx.x - nt) * 128 + tid; i < items; i += step) {
+        const int pl = i / cols, head = pl % c.Hkv, kv = (pl / c.Hkv) & 1, layer = pl / (2 * c.Hkv);
+        uint4* b = reinterpret_cast<uint4*>(c.cache + idx_cache(layer, max_batch, seq, kv, c.Hkv, head, c.cap, dst, c.hd)) + i % cols;
+        constexpr int NV = 8;
+        if (n <= NV) {
+            uint4 v[NV];
+#pragma unroll
+            for (int r = 0; r < NV; ++r)
+                if (r < n) v[r] = b[(size_t)src[r] * cols];
+#pragma unroll
+            for (int r = 0; r < NV; ++r)
+                if (r < n) b[(size_t)r * cols] = v[r];
+        } else {
+            uint4 v[MTAD_MAX_DEPTH];
+            for (int r = 0; r < n; ++r) v[r] = b[(size_t)src[r] * cols];
+            for (int r = 0; r < n; ++r) b[(size_t)r * cols] = v[r];
+        }
     }
 }
 
@@ -861,9 +872,14 @@ cudaError_t launch_commit(const ModelView& m, const ModelView* aux, const SeqSta
                            (long long)v.d.kv_capacity};
     };
     const CommitCache tg = cache_of(m), ax = aux ? cache_of(*aux) : CommitCache{};
-    const int most = std::max(16, 4 * 148 / B), nt = std::min(tg.planes, most), na = aux && mode != 2 ? std::min(ax.planes, most) : 0;
-    const size_t smem = (size_t)std::max(max_depth, 1) * std::max(tg.hd, ax.hd) * sizeof(__nv_bfloat16);
-    cudaError_t e = launch_pdl(commit_kernel, dim3(nt + na, B), dim3(128), smem, st, pdl, tg, ax, s, ds, call_seq_dev, res, max_depth,
+    // A thread per 16-byte column while a wave (8 blocks an SM) holds that many, then several a thread.  What bounds it is the moved rows'
+    // traffic where there is some, and otherwise its chain of a few dependent loads and two launches.  us with the launch after it: 40
+    // layers of 40 heads, 8 sequences, 6 rows of 128 moved each 24, 20 rows 83 (a block per plane, elements of two bytes through shared
+    // memory: 91 and 239; 592 blocks that took the planes in turn: 169 and 509); 32 x 32 heads, 4 rows, 1 / 64 sequences 11 / 56 (15 / 297,
+    // 19 / 360); nothing to move 9 (17..89 with a block per plane).
+    auto blocks = [&](const CommitCache& c) { return std::min((c.planes * (c.hd / 8) + 127) / 128, std::max(16, 8 * 148 / B)); };
+    const int nt = blocks(tg), na = aux && mode != 2 ? blocks(ax) : 0;
+    cudaError_t e = launch_pdl(commit_kernel, dim3(nt + na, B), dim3(128), 0, st, pdl, tg, ax, s, ds, call_seq_dev, res, max_depth,
                                mode, m.max_batch, nt);
     if (e != cudaSuccess) return e;
     return launch_pdl(advance_kernel, dim3(1), dim3(64), 0, st, pdl, s, ds, call_seq_dev, res, max_depth, mode, B, m.max_batch,
