@@ -7,6 +7,7 @@
 #include <math_constants.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -250,23 +251,29 @@ __device__ __forceinline__ void draft_scan(const float* __restrict__ logits, int
     const float* z = logits + (size_t)(bi * R + row) * V;
     const float* ub = uni + (((size_t)bi * gamma + step) * beam + j) * V;
     const int len = (V + nch - 1) / nch, v0 = c * len, v1 = min(V, v0 + len);
-    constexpr int NL = MTAD_MAX_BEAM;
+    // A list of NL tokens a thread.  A longer chunk (vocabulary above 65536) takes more passes, in which the warp's kpb best so far
+    // take the lists' first places.
+    constexpr int NL = MTAD_MAX_BEAM, HELD = MTAD_MAX_CAND / 32;
+    static_assert(HELD < NL, "room for tokens beside the best so far");
     float m = -CUDART_INF_F, sum = 0.f;
-    Cand loc[NL];
-    if (len <= 256 * NL) {
+    auto pass = [&](int at, auto held_places) {
+        constexpr int held = decltype(held_places)::value;
         // all of a thread's tokens at once
         float zv[NL], uv[NL];
+        Cand loc[NL];
 #pragma unroll
-        for (int k = 0; k < NL; ++k) {
-            const int v = v0 + tid + 256 * k;
+        for (int k = held; k < NL; ++k) {
+            const int v = at + tid + 256 * (k - held);
             zv[k] = v < v1 ? z[v] : -CUDART_INF_F;
             uv[k] = v < v1 ? ub[v] : 0.5f;
         }
+        const float before_max = m;
 #pragma unroll
-        for (int k = 0; k < NL; ++k) m = fmaxf(m, zv[k]);
+        for (int k = held; k < NL; ++k) m = fmaxf(m, zv[k]);
+        if (held && m != before_max) sum = before_max == -CUDART_INF_F ? 0.f : sum * expf(before_max - m);
 #pragma unroll
-        for (int k = 0; k < NL; ++k) {
-            const int v = v0 + tid + 256 * k;
+        for (int k = held; k < NL; ++k) {
+            const int v = at + tid + 256 * (k - held);
             loc[k] = Cand{-CUDART_INF_F, 0x7fffffff};
             if (256 * k < len && v < v1) {
                 sum += m == -CUDART_INF_F ? 0.f : (zv[k] == m ? 1.f : expf(zv[k] - m));
@@ -274,23 +281,34 @@ __device__ __forceinline__ void draft_scan(const float* __restrict__ logits, int
                 if (y == y) loc[k] = Cand{y, v};             // (NaN is no candidate)
             }
         }
-    } else {
-        // more tokens than the list holds: its NL best, sorted
 #pragma unroll
-        for (int k = 0; k < NL; ++k) loc[k] = Cand{-CUDART_INF_F, 0x7fffffff};
-        for (int v = v0 + tid; v < v1; v += 256) {
-            const float zv = z[v];
-            if (zv > m) { sum = sum * expf(m - zv) + 1.f; m = zv; }
-            else sum += expf(zv - m);
-            const Cand cd{zv - logf(-logf(ub[v])), v};
-            if (before(cd, loc[NL - 1])) {
-                loc[NL - 1] = cd;
+        for (int k = 0; k < held; ++k) {
+            const int r = lane + 32 * k;
+            loc[k] = r < kpb ? Cand{sh.y[warp][r], sh.v[warp][r]} : Cand{-CUDART_INF_F, 0x7fffffff};
+        }
+        __syncwarp();
+        // the warp's kpb best
+        Cand top = loc[0];
 #pragma unroll
-                for (int k = NL - 1; k > 0; --k)
-                    if (before(loc[k], loc[k - 1])) { const Cand tmp = loc[k]; loc[k] = loc[k - 1]; loc[k - 1] = tmp; }
+        for (int q = 1; q < NL; ++q)
+            if (before(loc[q], top)) top = loc[q];
+        for (int k = 0; k < kpb; ++k) {
+            const Cand win = warp_best(top);
+            if (lane == 0) { sh.y[warp][k] = win.y; sh.v[warp][k] = win.flat; }
+            if (top.flat == win.flat && win.flat != 0x7fffffff) {        // the owner takes it off its list (tokens are unique)
+                top = Cand{-CUDART_INF_F, 0x7fffffff};
+#pragma unroll
+                for (int q = 0; q < NL; ++q) {
+                    if (loc[q].flat == win.flat) loc[q] = Cand{-CUDART_INF_F, 0x7fffffff};
+                    if (before(loc[q], top)) top = loc[q];
+                }
             }
         }
-    }
+        __syncwarp();
+    };
+    pass(v0, std::integral_constant<int, 0>{});
+#pragma unroll 1
+    for (int at = v0 + 256 * NL; at < v1; at += 256 * (NL - HELD)) pass(at, std::integral_constant<int, HELD>{});
     // the chunk's maximum and sum of exponentials (fixed combination order: butterfly, then warps in order)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -300,23 +318,6 @@ __device__ __forceinline__ void draft_scan(const float* __restrict__ logits, int
         m = M;
     }
     if (lane == 0) { sh.m[warp] = m; sh.s[warp] = sum; }
-    // the warp's kpb best
-    Cand top = loc[0];
-#pragma unroll
-    for (int q = 1; q < NL; ++q)
-        if (before(loc[q], top)) top = loc[q];
-    for (int k = 0; k < kpb; ++k) {
-        const Cand win = warp_best(top);
-        if (lane == 0) { sh.y[warp][k] = win.y; sh.v[warp][k] = win.flat; }
-        if (top.flat == win.flat && win.flat != 0x7fffffff) {            // the owner takes it off its list (tokens are unique)
-            top = Cand{-CUDART_INF_F, 0x7fffffff};
-#pragma unroll
-            for (int q = 0; q < NL; ++q) {
-                if (loc[q].flat == win.flat) loc[q] = Cand{-CUDART_INF_F, 0x7fffffff};
-                if (before(loc[q], top)) top = loc[q];
-            }
-        }
-    }
     __syncthreads();
     if (warp) return;
     DraftPart* dst = part + ((size_t)(bi * MTAD_MAX_BEAM + j)) * nch + c;

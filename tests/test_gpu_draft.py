@@ -225,6 +225,41 @@ def test_draft_without_candidates(keep_all):
     assert region("rm_mask", b * 8) == [w for r in range(b) for w in [3 | 1 << (1 + b + r)] + [0] * 7]
 
 
+@pytest.mark.parametrize("V", [65536, 65537, 70000, 131104])
+def test_draft_selection_passes(V):
+    """Chunks of more tokens than a block's lists hold: the 64 best of the only row, with more of them than a list's places on the
+    tokens of one thread, and a row whose first logit is minus infinity.  Held against the logits that the device left."""
+    b, L = 8, 20
+    shape = S.ModelShape(1, 128, 2, 2, 64, 344, V)
+    gm = GpuModel(shape, max_batch=1, max_nodes=b * b, capacity=64, aux=shape, aux_capacity=64)
+    gm.inject(0, L)
+    gm.inject_aux(0, L)
+    gm.ctx.mtad_seq_set(0, L, 7, aux_len=L)
+    u = S.uniforms(0, (37 << 40) | V, b * V, "cuda").view(1, 1, b, V)
+    length = -(-V // 32)
+    for c in range(5):                                             # a thread's tokens lie 256 apart
+        own = torch.arange(c * length + 17 * c, (c + 1) * length, 256, device="cuda")
+        u[0, 0, 0, own] = 1 - 2.0 ** -24 * (20 + 3 * (torch.arange(len(own), device="cuda") * 5 + c))
+    seen = set()
+    for weight in (0.0, 3e38, -3e38):                              # (of one of the signs a token's logit is minus infinity)
+        if weight:
+            gm.aux_weights["lm_head"][0] = 0
+            gm.aux_weights["lm_head"][0, :8] = weight
+        g = _draft_gpu(gm, 0, 1, b, u, True)
+        z = gm.ctx.region("logits", torch.float32)[:V].double()
+        seen.add(float(z[0]))
+        if torch.isnan(z).any() or z.max() == math.inf:
+            continue
+        y = z - torch.log(-torch.log(u[0, 0, 0].double()))
+        best = y.topk(b * b + 1)
+        lq = z.log_softmax(0)
+        tok = g["tok"][0].long()
+        assert (best.values[:-1] - y[tok]).abs().max() < 1e-5 and len(set(tok.tolist())) == b * b
+        assert (best.values.diff().abs().min() < 1e-5) or torch.equal(tok, best.indices[:-1])
+        assert (g["node_logq"][0] - lq[tok]).abs().max() < 1e-5
+    assert -math.inf in seen and len(seen) == 3
+
+
 def test_draft_rejects_bad_arguments():
     gm = GpuModel(W.target, max_batch=1, max_nodes=40, capacity=128, aux=W.aux, aux_capacity=128)
     V = W.target.vocab
