@@ -1135,9 +1135,10 @@ int mtad_draft(mtad_ctx* ctx, int B, const int32_t* seqs, int gamma, int beam_wi
     DraftOut out{n_nodes, tok, parent, depth, node_logq, logq_ref, best_path};
     const bool tc = ctx->use_tc && ctx->amaps.ok;
     if (int rc = begin_forwards(ctx, m, B, R0, ub + 1, true, s)) return rc;
+    const bool ahead = !dwarp && draft_rows_ahead(m.d);
     for (int step = 0; step < gamma; ++step) {
         const int R = step == 0 ? R0 : beam_width;
-        if (step == 0 || dwarp)                         // (otherwise the selection of the step before made the rows)
+        if (step == 0 || !ahead)                        // (otherwise the selection of the step before made the rows)
             RUN(MTAD_K_PREPARE, 0, 1, launch_draft_prepare(m, ctx->st, ctx->ds, ctx->rm, ctx->sc, sl, B, R, step, beam_width,
                                                            tc && B * R <= TC_MAX_ROWS, dwarp, ctx->use_pdl, s));
         // keys of the auxiliary cache: committed ones, the pending rows and every node drafted so far
@@ -1156,7 +1157,7 @@ int mtad_draft(mtad_ctx* ctx, int B, const int32_t* seqs, int gamma, int beam_wi
         if (!(tc && B * R <= TC_MAX_ROWS))              // (the CUDA-core forward has written over the counters)
             CU(cudaMemsetAsync(ctx->sc.arrive, 0, sizeof(int32_t) * B, s));
         RUN(MTAD_K_LMRED, 0, 1, launch_draft_select(m, ctx->ds, ctx->sc, sl, B, R, step, gamma, beam_width, keep_all, uniforms, out,
-                                                     ctx->st, ctx->rm, step + 1 < gamma, tc && B * beam_width <= TC_MAX_ROWS,
+                                                     ctx->st, ctx->rm, ahead && step + 1 < gamma, tc && B * beam_width <= TC_MAX_ROWS,
                                                      ctx->use_pdl, s));
     }
     ctx->draft_active = true;

@@ -278,12 +278,13 @@ __device__ __forceinline__ void embed_row(const __nv_bfloat16* __restrict__ src_
             h4[1] = make_float4(v[4], v[5], v[6], v[7]);
             if (x_row) {
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    store_terms(v[2 * e] * __uint_as_float(gw[e] << 16), x_row + (size_t)c * 8 + 2 * e, d, terms);
-                    store_terms(v[2 * e + 1] * __uint_as_float(gw[e] & 0xffff0000u), x_row + (size_t)c * 8 + 2 * e + 1, d,
-                                terms);
-                    ss[k % NS] += v[2 * e] * v[2 * e] + v[2 * e + 1] * v[2 * e + 1];
-                }
+                for (int e = 0; e < 4; e += 2)
+                    store_terms4(make_float4(v[2 * e] * __uint_as_float(gw[e] << 16), v[2 * e + 1] * __uint_as_float(gw[e] & 0xffff0000u),
+                                             v[2 * e + 2] * __uint_as_float(gw[e + 1] << 16),
+                                             v[2 * e + 3] * __uint_as_float(gw[e + 1] & 0xffff0000u)),
+                                 x_row + (size_t)c * 8 + 2 * e, d, terms);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) ss[k % NS] += v[2 * e] * v[2 * e] + v[2 * e + 1] * v[2 * e + 1];
             }
         }
     }
@@ -381,6 +382,7 @@ cudaError_t launch_accept(const RowMeta& rm, const Scratch& sc, const AcceptArgs
 cudaError_t launch_draft_prepare(const ModelView& m, const SeqState& s, const DraftState& ds, const RowMeta& rm,
                                  const Scratch& sc, const SeqList& seqs, int B, int R, int step, int beam, bool tc,
                                  bool warped, bool pdl, cudaStream_t st);
+bool draft_rows_ahead(const mtad_model_desc& d);      // the selection makes the next step's rows
 cudaError_t launch_draft_select(const ModelView& m, const DraftState& ds, const Scratch& sc, const SeqList& seqs, int B,
                                 int R, int step, int gamma, int beam, int keep_all, const float* uniforms,
                                 const DraftOut& out, const SeqState& s, const RowMeta& rm, bool next, bool tc, bool pdl,

@@ -206,8 +206,8 @@ cudaError_t launch_draft_prepare(const ModelView& m, const SeqState& s, const Dr
 // joint score of a pair is t + (log q(beam) - lse(row)), a per-row constant added in fp32 (monotone), so a pair
 // among the overall `beam` largest is among the `beam` largest of its chunk.  Then the block of a sequence that finishes last
 // (draft_pick) merges the chunks of every row in chunk order, scores the surviving pairs and takes the `beam` largest
-// (ties to the lower flat index beam * V + token), writes the new layer of the tree, and makes the next step's rows from
-// it.  As three launches - scan, pick, rows - a step of the 7B pair spent 21 us between two forwards.
+// (ties to the lower flat index beam * V + token), writes the new layer of the tree, and of a narrow model (draft_rows_ahead)
+// makes the next step's rows from it.  As three launches - scan, pick, rows - a step of the 7B pair spent 21 us between two forwards.
 // ---------------------------------------------------------------------------------------------------------------
 
 __device__ __forceinline__ Cand warp_best(Cand c) {
@@ -480,7 +480,7 @@ __device__ __forceinline__ void draft_pick(const float* __restrict__ logits, int
     }
 }
 
-__global__ void __launch_bounds__(256) draft_select_kernel(const float* __restrict__ logits, int V, int R, int step, int gamma,
+__global__ void __launch_bounds__(256, 4) draft_select_kernel(const float* __restrict__ logits, int V, int R, int step, int gamma,
                                                            int beam, int keep_all, int kpb, const float* __restrict__ uni,
                                                            DraftState ds, SeqList seqs, DraftPart* part, int nch, DraftOut out,
                                                            DraftRows rows, bool next) {
@@ -692,6 +692,12 @@ cudaError_t launch_draft_select_warped(const ModelView& m, const DraftState& ds,
                                                 out);
     return cudaGetLastError();
 }
+
+// A sequence's rows of the next step are made by one block at the end of the selection, a warp a row, which saves a launch; as a launch of
+// their own they have a block each.  Drafts of four steps, us, one way and the other: width 512, 4 beams 228 / 232; 768, 1 / 4 / 8 beams
+// 209 / 214, 233 / 235, 265 / 267, eight sequences of four 310 / 313; 1024, 4 beams 238 / 239, eight sequences of eight 383 / 381; 1536, 4 and 8
+// beams 241 / 240, 281 / 277; 2048 256 / 254, 299 / 291; 4096 306 / 299, 366 / 345; 8192 412 / 393, 481 / 436.
+bool draft_rows_ahead(const mtad_model_desc& d) { return d.d_model <= 1024; }
 
 // next: the next step's rows too; tc: as operand rows of the tensor-core path.
 cudaError_t launch_draft_select(const ModelView& m, const DraftState& ds, const Scratch& sc, const SeqList& seqs, int B,

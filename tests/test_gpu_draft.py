@@ -397,3 +397,26 @@ def batched_iterations(target, aux, lens, gamma, b, capacity, aux_capacity, iter
             assert gm.ctx.mtad_seq_get(s) == (st["L"], st["root"])
     assert skipped <= B
     assert gm.ctx.mtad_debug_check_canaries() == ""
+
+
+@pytest.mark.parametrize("d,b", [(1024, 4), (1032, 4), (4096, 1)])
+def test_draft_wide_models(d, b):
+    """Where the next step's rows are made by the selection, and where by a launch of their own."""
+    V, gamma, L = 500, 3, 20
+    gm = GpuModel(S.ModelShape(1, 128, 2, 2, 64, 344, V), max_batch=1, max_nodes=16, capacity=64,
+                  aux=S.ModelShape(1, d, 2, 2, 64, 512, V), aux_capacity=64)
+    gm.inject(0, L)
+    gm.inject_aux(0, L)
+    gm.ctx.mtad_seq_set(0, L, 7, aux_len=L)
+    acache, skipped = gm.aux_cache_bits(0, L), 0
+    for it in range(3):
+        u = S.uniforms(0, (38 << 40) | it, gamma * b * V, "cuda").view(1, gamma, b, V)
+        g = _draft_gpu(gm, 0, gamma, b, u)
+        dr = O.draft_beam(gm.oracle_aux(), acache, L, [7], gamma, b, u[0].cpu().numpy())
+        if dr.min_gap < draft_gap(False):
+            skipped += 1
+            continue
+        assert g["tok"][0].tolist() == dr.tok and g["parent"][0].tolist() == dr.parent
+        assert g["best_path"][0].tolist() == dr.best_path
+        assert np.max(np.abs(g["node_logq"][0].cpu().numpy() - np.asarray(dr.logq))) < 2e-5
+    assert skipped <= 1 and gm.ctx.mtad_debug_check_canaries() == ""
