@@ -74,20 +74,48 @@ def test_forward_edges(models, shape, rows, tree, lengths):
         assert flips <= 0.03 and stats.cache_max_excess <= 2.0 ** -7 * flips ** 0.5 * stats.cache_scale
 
 
-@pytest.mark.parametrize("shape,rows,tree,lengths", [
-    ("hd64", 5, None, [1290]),                                   # 16 heads of 11 tiles: pieces of two, the last of one
-    ("hd64", 5, None, [1100, 1030]),                             # 32 of nine: three, one more than dealt out evenly
-    ("hd64", 6, None, [140, 700, 1280]),                         # of different lengths
-    ("hd64", 5, None, [2170, 300, 2300, 1500]),                  # 64: no pieces, blocks of several heads
-    ("hd64", 33, (4, 8, 4), [1290]),                             # wide items
+def piece_length(sh, rows, lengths):
+    """Key tiles of a piece of a (sequence, KV head, query block): dealt out evenly over 148 blocks, or up to two more, where the pieces
+    fit the blocks.  0: they do not, blocks take runs of tiles over several heads."""
+    query_rows = sh.n_q_heads // sh.n_kv_heads * rows
+    heads = sh.n_kv_heads * (-(-query_rows // 40) if query_rows > 16 else 1)
+    tiles = [-(-(L + rows) // 128) for L in lengths]
+    even = -(-sum(tiles) * heads // 148)
+    return next((n for n in (even, even + 1, even + 2) if sum(-(-t // n) for t in tiles) * heads <= 148), 0)
+
+
+SHAPES["h20"] = S.ModelShape(2, 640, 20, 20, 64, 1024, 500)
+SHAPES["h20x128"] = S.ModelShape(2, 512, 20, 20, 128, 1024, 500)
+
+
+@pytest.mark.parametrize("shape,rows,tree,lengths,piece", [
+    ("hd64", 5, None, [1290], 2),                                # 16 heads of 11 tiles: the last piece has one
+    ("hd64", 5, None, [1100, 1030], 3),                          # 32 of nine: one more than dealt out evenly
+    ("hd64", 6, None, [140, 700, 1280], 3),                      # of different lengths
+    ("hd64", 5, None, [2170, 300, 2300, 1500], 7),               # 64: one more
+    ("hd64", 33, (4, 8, 4), [1290], 2),                          # wide items
+    ("h20x128", 2, None, [1290, 700], 3),                        # few rows
+    ("h20x128", 7, None, [1290, 700], 3),
+    # wide: 24 query rows of a KV head.  Long, because cache_ok leaves out that a share of 2e-3 of the first layer's elements rounds
+    # the other way: of n own rows beside L keys, each as heavy as another, that moves an output by up to 4 x 2^-9 sqrt(2e-3) n / L
+    # of the largest value: 3e-6 at six rows and 700 keys, more than cache_ok's 2e-6, as measured (3.4e-6); 1.2e-6 at 1800.
+    ("gqa128", 6, None, [2290, 1800], 1),
+    ("h20", 1, None, [127, 300, 64, 513, 128, 1000, 90, 255], 0),             # 160 (sequence, KV head)s, few rows
+    ("h20x128", 1, None, [127, 300, 64, 513, 128, 1000, 90, 255], 0),
+    ("hd64", 3, None, [70, 130, 200, 300, 125, 126, 64, 400, 253, 254, 90, 100], 0),
+    ("h20x128", 7, None, [127, 300, 64, 513, 121, 122, 90, 255], 0),
+    ("hd64", 16, None, [760, 880, 753, 800, 879], 0),            # 80 of seven tiles, items of 16 rows
+    ("h20", 17, None, [760, 879, 752, 800], 0),                  # the same, wide items
+    ("h20x128", 17, None, [760, 879, 752, 800], 0),
 ])
-def test_attention_pieces(shape, rows, tree, lengths):
+def test_attention_pieces(shape, rows, tree, lengths, piece):
     """Where the keys of a (sequence, KV head) are cut into pieces of a block each, and where blocks take runs of tiles."""
     sh, B, stats = SHAPES[shape], len(lengths), ParityStats()
-    gm, cases = GpuModel(sh, max_batch=B, max_nodes=rows - 1, capacity=2400), []
+    assert piece_length(sh, rows, lengths) == piece
+    gm, cases = GpuModel(sh, max_batch=B, max_nodes=max(rows - 1, 1), capacity=max(lengths) + 100), []
     for b, L in enumerate(lengths):
         gm.inject(b, L)
         t = S.beam_tree(*tree, sh.vocab, stream=90 + b) if tree else S.chain_tree(rows - 1, sh.vocab, stream=90 + b)
         cases.append(SeqCase(b, L, int(S.token_ids(9, (22 << 40) | b, 1, sh.vocab)[0]), t))
     compare(gm, cases, Bn.log_tau(0.3), S.bonus_uniforms(9, 90 + rows, B, sh.vocab, "cuda"), chain=tree is None, stats=stats)
-    assert stats.ok() and stats.cache_ok(sh.layers, gemm_eps(B * rows, sh.d_ffn)), stats
+    assert stats.ok() and stats.cache_ok(sh.layers, gemm_eps(B * rows, max(sh.d_ffn, sh.q_dim))), stats
