@@ -622,23 +622,17 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
         const int f0 = tile * nf;                          // first feature (O, down, gate / up, LM head)
         // ---- what the first items need besides the accumulator
         const int hg = KIND == FW_QKV ? tile / f.u : 0, j0 = KIND == FW_QKV ? (tile - hg * f.u) * f.h : 0;
-        constexpr int NI = 1;                              // QKV: items per thread and round
-        float cs[NI][2 * V];                               // cosines and sines of an item's pairs
+        float cs[2 * V];                                   // QKV: cosines and sines of an item's pairs
         auto rope_load = [&](int t, int j) {
+            if (t < T && j0 + j < HD / 2) {
+                const float* src = a.rope + ((size_t)t * (HD / 2) + j0 + j) * 2;
+                if (V == 4) {
 #pragma unroll
-            for (int q = 0; q < NI; ++q) {
-                if (t < T && j0 + j < HD / 2) {
-                    const float* src = a.rope + ((size_t)t * (HD / 2) + j0 + j) * 2;
-                    if (V == 4) {
-#pragma unroll
-                        for (int x = 0; x < V / 2; ++x)
-                            *reinterpret_cast<float4*>(&cs[q][4 * x]) = *reinterpret_cast<const float4*>(src + 4 * x);
-                    } else {
-                        *reinterpret_cast<float2*>(&cs[q][0]) = *reinterpret_cast<const float2*>(src);
-                    }
+                    for (int x = 0; x < V / 2; ++x)
+                        *reinterpret_cast<float4*>(&cs[4 * x]) = *reinterpret_cast<const float4*>(src + 4 * x);
+                } else {
+                    *reinterpret_cast<float2*>(&cs[0]) = *reinterpret_cast<const float2*>(src);
                 }
-                t += dt; j += dj;
-                if (j >= nf) { j -= nf; ++t; }
             }
         };
         float hid = 0.f, gain0 = 0.f;                      // O, down with few rows: the residual element of (row w, feature lane)
@@ -672,14 +666,6 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
         if (!ok) return false;
         tc_fence_after();
         const uint32_t t_acc = tmem_lane + (f.both ? 0 : buf * 256);
-        auto add_put_by = [&](int b, int rb, float* v) {   // what the tile's earlier parts left of 16 rows
-            if (!FEW && KIND == FW_GATEUP && f.segs > 1) {
-                float o[16];
-                tc_ld16(tmem_lane + f.stash + b * up16(T) + rb, o);
-#pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] += o[j];
-            }
-        };
         if constexpr (!FEW && KIND == FW_GATEUP)
             if (f.S == 1) {
                 // A thread has a feature's gate and up sums of every row in its tensor-memory lane: no way through shared memory, the
@@ -754,7 +740,6 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                         acc_ld16(t_acc + (b * S + sl) * cols + rb * 3, acc_stride, na, v);
 #pragma unroll
                         for (int j = 0; j < 5; ++j) v[j] = v[3 * j] + (v[3 * j + 1] + v[3 * j + 2]);
-                        add_put_by(b, rb, v);
                         if (here)
 #pragma unroll
                             for (int j = 0; j < 5; ++j)
@@ -770,7 +755,6 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                         }
 #pragma unroll
                         for (int j = 0; j < 16; ++j) v[j] = v[2 * j] + v[2 * j + 1];
-                        add_put_by(b, rb, v);
                         if (here)
 #pragma unroll
                             for (int j = 0; j < 16; ++j)
@@ -807,57 +791,54 @@ __device__ __forceinline__ bool epi_phase(const FwArgs& a, FwTail& s, float* Y, 
                 constexpr int hp = HD / 2;
                 const float scale = rsqrtf((float)HD) * 1.4426950408889634f;      // (the attention's softmax runs on exp2)
                 int t = it0, j = ij0;
-                for (int i = e; i < nr * nv; i += NI * FW_EPI) {
+                for (int i = e; i < nr * nv; i += FW_EPI) {
                     if (FEW ? i != e : r0 > 0 && i == e) rope_load(r0 + t, j);
+                    const int jj = j0 + j, tt = r0 + t;
+                    int tn = t + dt, jn = j + dj;                     // the next item
+                    if (jn >= nf) { jn -= nf; ++tn; }
+                    float c[2 * V];
 #pragma unroll
-                    for (int q = 0; q < NI; ++q) {
-                        const int jj = j0 + j, tt = r0 + t;
-                        int tn = t + dt, jn = j + dj;                     // the next item
-                        if (jn >= nf) { jn -= nf; ++tn; }
-                        float c[2 * V];
+                    for (int x = 0; x < 2 * V; ++x) c[x] = cs[x];
+                    if (!FEW && i + FW_EPI < nr * nv) rope_load(r0 + tn, jn);        // ahead by one round
+                    const int sl = s.slot[tt];
+                    if (jj < hp && sl >= 0) {                         // (no slot: an inactive row has no query and no keys)
+                        const float rs = s.rstd[tt];
+                        float va[V], vb[V];
+                        yv(t, 0, j, va);
+                        yv(t, 0, f.h + j, vb);
+                        const bool rot = hg < a.Hq + a.Hkv;
 #pragma unroll
-                        for (int x = 0; x < 2 * V; ++x) c[x] = cs[q][x];
-                        if (!FEW && i + FW_EPI < nr * nv) rope_load(r0 + tn, jn);        // ahead by one round
-                        const int sl = t < nr ? s.slot[tt] : -1;
-                        if (jj < hp && sl >= 0) {                         // (no slot: an inactive row has no query and no keys)
-                            const float rs = s.rstd[tt];
-                            float va[V], vb[V];
-                            yv(t, 0, j, va);
-                            yv(t, 0, f.h + j, vb);
-                            const bool rot = hg < a.Hq + a.Hkv;
-#pragma unroll
-                            for (int x = 0; x < V; ++x) {
-                                const float ya = va[x] * rs, yb2 = vb[x] * rs;
-                                va[x] = rot ? ya * c[2 * x] - yb2 * c[2 * x + 1] : ya;
-                                vb[x] = rot ? yb2 * c[2 * x] + ya * c[2 * x + 1] : yb2;
-                            }
-                            if (hg < a.Hq) {
-                                // attention operands: q * log2(e) / sqrt(hd) as bf16 hi + lo
-                                const size_t o = ((size_t)tt * a.Hq + hg) * HD + jj;
-                                if (V == 1) {
-                                    split_store(va[0] * scale, a.q_hi + o, a.q_lo + o);
-                                    split_store(vb[0] * scale, a.q_hi + o + hp, a.q_lo + o + hp);
-                                } else {
-                                    split_store4(va, scale, a.q_hi + o, a.q_lo + o);
-                                    split_store4(vb, scale, a.q_hi + o + hp, a.q_lo + o + hp);
-                                }
+                        for (int x = 0; x < V; ++x) {
+                            const float ya = va[x] * rs, yb2 = vb[x] * rs;
+                            va[x] = rot ? ya * c[2 * x] - yb2 * c[2 * x + 1] : ya;
+                            vb[x] = rot ? yb2 * c[2 * x] + ya * c[2 * x + 1] : yb2;
+                        }
+                        if (hg < a.Hq) {
+                            // attention operands: q * log2(e) / sqrt(hd) as bf16 hi + lo
+                            const size_t o = ((size_t)tt * a.Hq + hg) * HD + jj;
+                            if (V == 1) {
+                                split_store(va[0] * scale, a.q_hi + o, a.q_lo + o);
+                                split_store(vb[0] * scale, a.q_hi + o + hp, a.q_lo + o + hp);
                             } else {
-                                const int sq = s.meta[s.rowb[tt]].seq, kv = rot ? 0 : 1;
-                                if (sl < a.cap && (unsigned)sq < (unsigned)a.max_batch) {   // never past the cache
-                                    __nv_bfloat16* d = a.cache + idx_cache(layer, a.max_batch, sq, kv, a.Hkv, hg - a.Hq - kv * a.Hkv,
-                                                                           a.cap, sl, HD) + jj;
-                                    if (V == 1) {
-                                        d[0] = __float2bfloat16_rn(va[0]);
-                                        d[hp] = __float2bfloat16_rn(vb[0]);
-                                    } else {
-                                        store_bf4(va, d);
-                                        store_bf4(vb, d + hp);
-                                    }
+                                split_store4(va, scale, a.q_hi + o, a.q_lo + o);
+                                split_store4(vb, scale, a.q_hi + o + hp, a.q_lo + o + hp);
+                            }
+                        } else {
+                            const int sq = s.meta[s.rowb[tt]].seq, kv = rot ? 0 : 1;
+                            if (sl < a.cap && (unsigned)sq < (unsigned)a.max_batch) {   // never past the cache
+                                __nv_bfloat16* d = a.cache + idx_cache(layer, a.max_batch, sq, kv, a.Hkv, hg - a.Hq - kv * a.Hkv,
+                                                                       a.cap, sl, HD) + jj;
+                                if (V == 1) {
+                                    d[0] = __float2bfloat16_rn(va[0]);
+                                    d[hp] = __float2bfloat16_rn(vb[0]);
+                                } else {
+                                    store_bf4(va, d);
+                                    store_bf4(vb, d + hp);
                                 }
                             }
                         }
-                        t = tn; j = jn;
                     }
+                    t = tn; j = jn;
                 }
             } else if (KIND == FW_GATEUP) {
                 int t = it0, j = ij0;
@@ -1927,7 +1908,7 @@ bool fw_plan(FwArgs& a, const mtad_model_desc& d, int B, int R, int n_cta) {
                 break;
             }
         }
-        const int per = a.terms == 3 ? 5 : 16;             // rows of one drain load
+        const int per = a.terms == 3 ? 5 : 16;             // rows of one drain load (gate / up with one slice has no use for blk)
         const int fit = FW_UNION / (per * (f.nbox * f.S * f.hr + 4) * 4);
         if (fit < 1) return false;
         f.blk = std::min(up_div(T, per), fit) * per;
