@@ -30,7 +30,7 @@ TAU = 0.1
 SEED = 0
 # (DRAM read + write) / (weights + committed K / V) of the forward launch, ncu on the 4-layer workloads (profiles/forward_7b_4l.md):
 # chain and tree of the 7B shape; no figure for other shapes
-NCU_TRAFFIC_RATIO = {"7b_chain": 1.005, "7b_chain_4l": 1.005, "7b_chain_l512": 1.005, "7b_tree": 1.025, "7b_tree_4l": 1.025}
+NCU_TRAFFIC_RATIO = {"7b_chain": 1.005, "7b_chain_4l": 1.005, "7b_chain_l512": 1.005, "7b_tree": 1.024, "7b_tree_4l": 1.024}
 
 
 def measured_peaks():

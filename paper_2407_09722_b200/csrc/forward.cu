@@ -9,14 +9,14 @@
 // stays busy across the barrier for as long as the ring is deep.  Two more things keep the boundary short: every block
 // owns whole output features (the features are cut into one tile per SM, not into 128-row tiles), so no partial sum leaves
 // an SM while rows are few; and only the call's terms x rows operand rows are multiplied (16 columns for five rows).
-// Measured (chain of launches -> one launch, a whole verification step): 7B, 5 rows 3.55 -> 2.91 ms (weights and K / V in
-// 2.2 ms at copy speed), 33 rows 4.37 -> 3.57, 65 rows 5.90 -> 4.79; 13B, 8 x 7 rows 9.41 -> 8.80; two-layer auxiliary
-// model of width 768, four draft steps 520 -> 378 us.  A phase of a large model costs its bytes plus about 3 us (barrier 1.1,
-// first operand rows 0.6, last MMA to last store 1.2 and up); the phases of the auxiliary model, which move next to nothing,
-// take about 6, and the attention of a chain 7 more than its bytes.  Much of that is waiting for instructions: what an epilogue
-// executes runs once a phase, and a layer's worth of it does not fit an SM's instruction cache (four layers of 7B, 5 rows: 6.2k
-// misses of 23.8k lookups an SM, 8.1k of 26.6k before the code of few rows was made smaller).  Code here should be short before
-// it is clever: unrolled groups of loads that saved round trips made a step slower.
+// Measured (chain of launches -> one launch, both ways in turn on one GPU, a whole verification step): 7B, 5 rows 3.36 ->
+// 2.94 ms (weights and K / V in 2.2 ms at copy speed), 33 rows 4.30 -> 3.53, 65 rows 6.03 -> 4.56; 13B, 8 x 7 rows 9.98 -> 8.58;
+// two-layer auxiliary model of width 768, four draft steps 506 -> 380 us.  A phase of a large model costs its bytes plus about
+// 3 us (barrier 1.1, first operand rows 0.6, last MMA to last store 1.2 and up); the phases of the auxiliary model, which move next to
+// nothing, take about 6, and the attention of a chain 7 more than its bytes.  Part of that is waiting for instructions: what an
+// epilogue executes runs once a phase, and a layer's worth of it does not fit an SM's instruction cache (four layers of 7B, 5 rows:
+// 6.3k misses of 23.8k lookups an SM; 8.1k of 26.6k, and 0.3 us more a phase, before the code of few rows was made smaller).  Code here
+// should be short before it is clever: unrolled groups of loads that saved round trips made a step slower.
 //
 // Contraction.  Weights are the 128-row MMA operand A, the operand rows (two or three bf16 terms per activation, see
 // store_terms) operand B.  Where a block owns at most 64 features, the MMA takes S k-blocks at once: their weights lie
@@ -24,7 +24,8 @@
 // the k-blocks' contributions, summed by the epilogue.  One MMA of 128 x 64 costs what one of 128 x 16 does, so this is S
 // times fewer MMAs (an MMA takes 65 cycles whatever N <= 128 is: 32 rows at a time would cap an SM at 30 GB/s).
 //
-// Attention: keys as the M dimension.  The (sequence, KV head, 128-key tile) items are dealt out evenly, in order.
+// Attention: keys as the M dimension.  The (sequence, KV head, 128-key tile) items are dealt out in pieces of one (sequence, KV head)
+// each, or evenly, in order.
 //   S^T = K Q^T   A = K tile as it lies in the cache, B = query rows (bf16 hi rows, then lo rows)
 //   P = exp2(S - m), a thread per key and half of the query rows, written to shared memory as three bf16 terms
 //   O^T += V^T P  A = V tile (MN-major), B = P; a thread per head dimension and half of the rows adds it to its registers
@@ -1064,7 +1065,9 @@ __device__ __forceinline__ void merge_rows(const FwArgs& a, const FwTail& s, con
         }
     }
 }
-// Wide items have many rows in few pieces: a thread's rows are fetched side by side.
+// Wide items have many rows in few pieces: of two, a thread's rows are fetched side by side.  Pieces six at a time -> two of three rows,
+// us of eight layers: two pieces 675 -> 669, 852 -> 833, 742 -> 732, 937 -> 925 (7B, 65 rows 4755 -> 4705); four to eight pieces 451 -> 459,
+// 505 -> 516, 701 -> 714.
 template <int HD, int NQP>
 __device__ __forceinline__ void merge_pieces(const FwArgs& a, const FwTail& s, const AttnPos& q, int n_piece, int G, int e, int kp) {
     if (NQP > FW_QROWS && n_piece <= 2) merge_rows<HD, NQP, 2, 3>(a, s, q, n_piece, G, e, kp);
@@ -1168,9 +1171,11 @@ __global__ void __launch_bounds__(FW_THREADS, 1) forward_kernel(const __grid_con
     const AttnPos &a_zero = s.apos[0], &a_last = s.apos[1], &a_first = s.apos[2];
     if (warp == 1) {
         // Dealt out evenly, a block's tiles may be of two (sequence, KV head)s or more, and the end of each (sums over the keys,
-        // output to global memory, the next one's first scores) costs as much as two tiles and a half: pieces that keep to one are
-        // taken where they are at most two tiles longer, a lane per length tried.  7B chain, 32 heads of 17 tiles: pieces of
-        // five instead of runs of four, a step 3069 -> 3009 us.
+        // output to global memory, the next one's first scores) costs as much as a few tiles: pieces that keep to one are
+        // taken where they are at most two tiles longer, a lane per length tried.  7B chain, 32 heads of 17 tiles, one tile longer:
+        // a step 2954 -> 2894 us; 65-row tree 4794 -> 4705.  Eight layers of width 1024, runs -> pieces one tile longer: heads of 64
+        // 315 -> 304 us, wide items 526 -> 505, heads of 128 442 -> 433, wide 762 -> 732; two longer 485 -> 484, 854 -> 833, 557 -> 558,
+        // 953 -> 925; four longer (with a bound of five) 560 -> 570, 994 -> 1003, 659 -> 669, 1103 -> 1117.
         int per = max(1, (a_tot + n_cta - 1) / n_cta), lo = min(cta * per, a_tot), n = min(lo + per, a_tot) - lo, lo2 = 0, n2 = 0;
         const bool fits = lane < 3 && a_tot > 0 && attn_cut(s.meta, a.B, heads, per + lane, cta, lo2, n2) <= n_cta;
         const uint32_t can = __ballot_sync(0xffffffffu, fits);
